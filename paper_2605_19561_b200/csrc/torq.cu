@@ -34,6 +34,7 @@ struct DeviceState {
   int sm_count = 0;
   int rot_pairs = 0;    // CTA pairs of the pair kernels that can be resident at once
   int gemm_pairs = 0;
+  int few_fit[9] = {};  // clusters of S CTAs resident at once, one CTA per SM
   int* err_word = nullptr;
 };
 static DeviceState g_dev[kMaxDevices];
@@ -52,23 +53,31 @@ static bool opt_in_smem(K kernel, int bytes) {
          cudaSuccess;
 }
 
-// How many 2-CTA clusters of `kernel` fit on the device at once (GPC boundaries can leave a few
-// SMs unpaired, so this may be below sm_count / 2).
+// How many clusters of `size` CTAs of `kernel` fit on the device at once (GPC boundaries can leave SMs unused).
 template <typename K>
-static int max_active_pairs(K kernel, int threads, int smem, int sm_count) {
+static int max_active_clusters(K kernel, int size, int threads, int smem, int sm_count) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(sm_count / 2 * 2), 1, 1);
+  cfg.gridDim = dim3((unsigned)(4 * sm_count / size * size), 1, 1);     // the answer never exceeds the grid
   cfg.blockDim = dim3((unsigned)threads, 1, 1);
   cfg.dynamicSmemBytes = (size_t)smem;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.x = (unsigned)size;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+// CTA pairs of a kernel that fills its SMs.
+template <typename K>
+static int max_active_pairs(K kernel, int threads, int smem, int sm_count) {
+  const int n = max_active_clusters(kernel, 2, threads, smem, sm_count);
   return n < sm_count / 2 ? n : sm_count / 2;
 }
 
@@ -137,6 +146,8 @@ static DeviceState* device_state() {
     st.gemm_pairs = max_active_pairs(mxfp4_gemm_pair_kernel<FMT_NVFP4>, GemmPairCfg::THREADS,
                                      GemmPairCfgT<FMT_NVFP4>::SMEM_BYTES, st.sm_count);
     if (st.rot_pairs < 1 || st.gemm_pairs < 1) return nullptr;
+    for (int s = 1; s <= RotFewCfg::MAX_CLUSTER; ++s)
+      st.few_fit[s] = max_active_clusters(rotate_fewtok_kernel<FMT_MXFP4, 2>, s, 320, RotFewCfg::smem_bytes(256), st.sm_count);
     cudaGetLastError();
   }
   st.ready = true;
@@ -219,19 +230,27 @@ static int rotation_splits(int64_t M, int64_t d, int sm_count) {
 constexpr int kRotFewMaxTokens = 256;    // up to here the rotation streams R_inter through the few-token kernel
 constexpr int kGemmFewMaxTokens = 128;   // and the GEMM the weights
 static_assert(kRotFewMaxTokens <= RotFewCfg::MAX_TOK && kGemmFewMaxTokens <= GemmFewCfg<FMT_MXFP4>::MAX_TOK, "few-token limits");
-// Few-token kernels: tokens per instruction and the cluster size = number of K splits of
-// one 128-feature tile.  Two of these CTAs fit on an SM, and a grid of about 1.4 CTAs per SM measured
-// fastest (more loads in flight; beyond that the clusters no longer all become resident at once):
-// the largest S <= 8 with tiles * S <= 1.4 SMs, each split at least `min_k` K steps.  7 is skipped:
-// clusters of 7 did not all become resident at sizes where 6 and 8 did.
+// Few-token kernels: tokens per instruction, and the cluster size S = number of K splits of one 128-feature
+// tile: the largest S up to 8 within these bounds, each with both sides measured (us, cold operands):
+//  * all clusters are resident at once.  `fit[S]` is what the runtime answers for one CTA per SM (148, 74, 45, 33,
+//    26, 22, 15, 15: clusters do not cross GPCs); where two CTAs fit on an SM, twice that.  More in flight pays up
+//    to there -- rotation d = 14336, M = 50: S = 2 (112 clusters) 63.6, S = 1 80.8; d = 7168: S = 4 (56) 20.3, S = 2
+//    24.7; GEMM K = 14336, N = 6144: S = 4 (48) 11.5, S = 2 13.8 -- and a second wave costs more than it brings:
+//    d = 5120, S = 7 (40, 30 fit) 20.7 against 13.5 at S = 6; d = 2048, M = 100: S = 8 (16, 15 fit) 14.1, S = 4 7.7;
+//  * above S = 4, at most 1.4 CTAs per SM, so that CTAs of the next kernel in the stream find room and send their
+//    weight loads early (decode layer at d = N = 5120, M = 1: S = 5 17.86, S = 6 17.97, though the rotation by
+//    itself is the faster one with S = 6), and `long_k` K steps per CTA: a longer reduction has to be paid for by a shorter stream (rotation
+//    d = 2048, M = 50: S = 8 7.1, S = 4 6.5; GEMM K = 2048, N = 5120: S = 5 5.5, S = 4 5.1).  With 256 tokens
+//    the reduction itself is shared out (16 token groups), so there is no such bound (d = 1536: S = 8 9.9, S = 4 11.3);
+//  * no S above the smallest one with the same longest K range (GEMM K = 4096: S = 5 has ranges of 4 steps like S = 4).
 static inline int fewtok_ntok(int64_t M) { return M <= 16 ? 16 : (M <= 32 ? 32 : (M <= 64 ? 64 : (M <= 128 ? 128 : 256))); }
-static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int min_k, int sm_count, int ctas_per_sm) {
-  // two CTAs fit on an SM: 1.4 per SM on average keeps the most bytes in flight; one: one wave
-  int64_t s = (int64_t)sm_count * (ctas_per_sm >= 2 ? 14 : 10) / 10 / (tiles > 0 ? tiles : 1);
-  if (s > 8) s = 8;
-  if (s > k_steps / min_k) s = k_steps / min_k;
-  if (s == 7) s = 6;
-  return s < 1 ? 1 : (int)s;
+static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int long_k, int ctas_per_sm, int sm_count, const int* fit) {
+  int64_t most = k_steps / long_k;
+  most = most < 4 ? 4 : (most > 8 ? 8 : most);
+  int s = (int)(most < k_steps ? most : k_steps);
+  while (s > 1 && (tiles > (int64_t)ctas_per_sm * fit[s] || (s > 4 && 10 * tiles * s > 14 * (int64_t)sm_count))) --s;
+  while (s > 1 && (k_steps + s - 2) / (s - 1) == (k_steps + s - 1) / s) --s;      // fewer clusters' CTAs: they fit as well
+  return s < 1 ? 1 : s;
 }
 constexpr double kNarrowTileCost = 0.88;   // a 192-column tile against a 256-column one: 0.75 of the math, 0.875 of the operand bytes
 
@@ -411,7 +430,7 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
     // distributed shared memory; one launch, no scratch.
     const int ntok = fewtok_ntok(M);
     const int tiles = (int)(d / 128);
-    const int S = fewtok_cluster(tiles, d / 64, 2, st->sm_count, RotFewCfg::ctas_per_sm(ntok));
+    const int S = fewtok_cluster(tiles, d / 64, ntok == 256 ? 1 : 10, RotFewCfg::ctas_per_sm(ntok), st->sm_count, st->few_fit);
     if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d, (uint32_t)ntok, 64) ||
         !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 64))
       return TORQ_ERR_LAUNCH;
@@ -604,7 +623,7 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
     using FC = GemmFewCfg<FMT>;
     const int ntok = fewtok_ntok(M);
     const int tiles = (int)((N + 127) / 128);
-    const int S = fewtok_cluster(tiles, (K + FC::BK - 1) / FC::BK, 1, st->sm_count, FC::ctas_per_sm(ntok));
+    const int S = fewtok_cluster(tiles, (K + FC::BK - 1) / FC::BK, 3, FC::ctas_per_sm(ntok), st->sm_count, st->few_fit);
     if (!encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, 128, 128) ||
         !encode_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Aq, (uint64_t)M, krow, (uint32_t)ntok, 128))
       return TORQ_ERR_LAUNCH;

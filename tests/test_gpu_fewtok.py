@@ -56,6 +56,13 @@ def test_rotation_alone_without_any_workspace(M, d):
         assert not raw.any()
 
 
+# the ends of the cluster rule: one K step per CTA (d = 256: four CTAs), more CTAs than SMs (d = 7168: 224),
+# 16 feature tiles with one CTA per SM (clusters of 8 would not all fit)
+@pytest.mark.parametrize("M,d", [(1, 256), (50, 256), (256, 256), (50, 7168), (100, 2048), (200, 2048)])
+def test_rotation_cluster_sizes(M, d):
+    test_rotation_alone_without_any_workspace(M, d)
+
+
 def test_rotation_exact_cases_are_bit_exact():
     """Permutation and identity rotations with integer activations: every partial sum is exact in any
     order, so codes and scales must equal the oracle's bit for bit through the split and the reduction."""
@@ -111,6 +118,12 @@ def test_gemm_random_operands(M, N, K):
     assert np.array_equal(gotb, O.round_to_bf16(got))
     refb = O.round_to_bf16(ref)
     assert np.linalg.norm(gotb - refb) / np.linalg.norm(refb) <= 1e-3
+
+
+# the ends of the cluster rule: 96 tiles x 2 CTAs, ranges of one and of seven K steps, clusters of eight
+@pytest.mark.parametrize("M,N,K", [(33, 12288, 1024), (3, 264, 256), (64, 1024, 14336), (100, 1024, 14336), (100, 2048, 4096)])
+def test_gemm_cluster_sizes(M, N, K):
+    test_gemm_random_operands(M, N, K)
 
 
 def test_gemm_exact_integer_regime_and_one_hot_rows():
