@@ -3,7 +3,8 @@
 // of 16 tokens): y is split into three bfloat16 terms (y = hi + mid + lo up to 2^-24 relative),
 // R_intra is bfloat16 already, so every product is exact in fp32 and the fp32-accumulating
 // mma.sync m16n8k16 reproduces the fp32 rotation up to the order of additions.  Then Eq. 1 (or the
-// NVFP4 / MXINT4 quantizer) on the accumulator fragments: four lanes share a row.
+// NVFP4 / MXINT4 quantizer) on the accumulator fragments: four lanes share a row.  Two forms: a 16-row tile
+// in shared memory (intra_quantize_rows16), and 16 rows that come in the fragment layout (intra_quantize_frag16).
 #pragma once
 #include <cuda_bf16.h>
 #include "nvfp4_quantize.cuh"
@@ -104,6 +105,80 @@ __device__ __forceinline__ void intra_quantize_rows16(const float* y_s, uint32_t
         scales[scale_offset(row, blk, kb4)] = live ? (uint8_t)sb : (uint8_t)0;
       }
     }
+  }
+}
+
+// B fragments of one R_intra block for the two functions below.  rb0 / rb1: this lane's ldmatrix row addresses for
+// columns 0-15 / 16-31 of rows 0-15 (lane l: row l % 8 of matrix l / 8; matrices (k 0-7, n), (k 8-15, n), (k 0-7, n+8),
+// (k 8-15, n+8)); kc_stride: bytes to rows 16-31.
+struct IntraFrag { uint32_t b[2][4][2]; };               // [k chunk][n tile][2]
+__device__ __forceinline__ void load_intra_frag(uint32_t rb0, uint32_t rb1, uint32_t kc_stride, IntraFrag& f) {
+#pragma unroll
+  for (int kc = 0; kc < 2; ++kc) {
+    ldmatrix_x4_trans(rb0 + kc * kc_stride, f.b[kc][0][0], f.b[kc][0][1], f.b[kc][1][0], f.b[kc][1][1]);
+    ldmatrix_x4_trans(rb1 + kc * kc_stride, f.b[kc][2][0], f.b[kc][2][1], f.b[kc][3][0], f.b[kc][3][1]);
+  }
+}
+
+// Intra rotation and quantization of 16 rows x 32 columns that arrive in the fragment layout (y as
+// tmem_ld_16x256b_x4 gives it), so that they never pass through shared memory.  row0: first of the 16 rows;
+// scale byte(s) of rows row0 + lane / 4 + 8 rh come back in sb[rh] (0 past the last block for NVFP4; for the other
+// formats a block of zeros has byte 0 by itself).
+template <int FMT>
+__device__ __forceinline__ void intra_quantize_frag16(const uint32_t (&y)[16], bool has_intra, const IntraFrag& f, int lane,
+                                                      int64_t row0, int M, int blk, int nblocks, int d, const NvScale& nvs,
+                                                      uint8_t* __restrict__ codes, uint32_t* sb) {
+  const int p = lane & 3, r8 = lane >> 2;
+  float acc[4][4];
+  if (has_intra) {
+    uint32_t ah[8], am[8], al[8];                        // A fragments: [k chunk * 4 + (n & 1) * 2 + row half]
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int rh = 0; rh < 2; ++rh) {
+        const int ai = (n >> 1) * 4 + (n & 1) * 2 + rh;
+        split3_bf16x2(y[4 * n + 2 * rh], y[4 * n + 2 * rh + 1], ah[ai], am[ai], al[ai]);
+      }
+#pragma unroll
+    for (int n = 0; n < 4; ++n) { acc[n][0] = 0.f; acc[n][1] = 0.f; acc[n][2] = 0.f; acc[n][3] = 0.f; }
+#pragma unroll
+    for (int kc = 0; kc < 2; ++kc)
+#pragma unroll
+      for (int n = 0; n < 4; ++n) {
+        mma_16816_bf16(acc[n], al + 4 * kc, f.b[kc][n]);
+        mma_16816_bf16(acc[n], am + 4 * kc, f.b[kc][n]);
+        mma_16816_bf16(acc[n], ah + 4 * kc, f.b[kc][n]);
+      }
+  } else {
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[n][e] = __uint_as_float(y[4 * n + e]);
+  }
+#pragma unroll
+  for (int rh = 0; rh < 2; ++rh) {
+    const float v[8] = {acc[0][2 * rh], acc[0][2 * rh + 1], acc[1][2 * rh], acc[1][2 * rh + 1],
+                        acc[2][2 * rh], acc[2][2 * rh + 1], acc[3][2 * rh], acc[3][2 * rh + 1]};
+    uint32_t word, sbyte;
+    const int64_t row = row0 + r8 + 8 * rh;
+    if constexpr (FMT == FMT_MXINT4) {                   // two operand bytes per 8 columns and lane
+      uint32_t pr[4];
+      mxint4_quantize_row_fragment(v, pr, sbyte);
+      if (row < M && blk < nblocks) {
+        uint8_t* dst = codes + row * (int64_t)d + (int64_t)blk * 32 + 2 * p;
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt) *reinterpret_cast<uint16_t*>(dst + 8 * nt) = (uint16_t)pr[nt];
+      }
+    } else {
+      if constexpr (FMT == FMT_NVFP4) nv_quantize_row_fragment(v, p, nvs, word, sbyte);
+      else quantize_row_fragment(v, p, word, sbyte);
+      if (row < M && blk < nblocks)
+        *reinterpret_cast<uint32_t*>(codes + row * (int64_t)(d / 2) + (int64_t)blk * 16 + 4 * p) = word;
+    }
+    if constexpr (FMT == FMT_NVFP4) {
+      if (blk >= nblocks) sbyte = 0;                     // padding blocks decode to zero
+    }
+    sb[rh] = sbyte;
   }
 }
 

@@ -1,0 +1,233 @@
+// Rotate + quantize on CTA pairs in ONE wave: every pair works exactly one tile of 256 tokens x `width` features
+// (a multiple of 32, up to 384), the width chosen so that the tiles just fill the pairs.
+//
+// The pair kernel deals 256-column tiles.  A layer of some hundred tokens has either fewer of those than there are
+// pairs, or a few more and pays a second wave for them.  Measured (rotation alone, us, pair kernel / here): 777 x
+// 5120 (80 tiles / 4 x 18 of 288) 48.6 / 38.5; 1024 x 5120 48.8 / 40.1; 300 x 4096 (32 / 2 x 32 of 128) 26.0 / 21.2;
+// 1000 x 1024 11.7 / 8.4; 1000 x 256 8.0 / 3.9.
+//
+// A tile wider than 256 columns is two instructions per 16 elements of K that share the X slice, accumulators
+// side by side in tensor memory (column c of the tile is accumulator column c).  An instruction costs at least
+// 45 cycles however narrow (256 + 32 columns ran at 692 cycles per K step, 160 + 128 at 576), so the second one is
+// always 128 columns.  Each CTA of the pair stages its 128 rows of X and half of each instruction's columns of
+// R_inter: 64-column boxes of 8 KiB and, when half of the first instruction is no multiple of 64, one narrower box
+// (its rows keep the 128-byte pitch of the swizzle) in a slot of the same size.
+//
+// Bounds: up to 256 columns the operand bytes (52 to 66 B per cycle and SM cross from L2: 440 cycles per K step at 64
+// columns, 460 at 128, 500 at 256, where the math takes 2 cycles per column), above the math; then the
+// epilogue, which nothing overlaps.  It is the fast form (warp-level MMAs on the accumulator fragments), bound by
+// those MMAs: about 860 cycles per 32 columns.  Splitting K over the pairs of a larger cluster (partial sums
+// exchanged through distributed shared memory) was measured and brought nothing: 300 x 4096 20.9 with two pairs
+// per 256 columns against 21.2.
+//
+// Roles per CTA: warp 0 TMA producer, warp 1 MMA issuer (leader CTA), warps 2..13 epilogue (lane quarter w % 4, three
+// sets of warps).  One elected thread runs the producer's and the issuer's loop.
+#pragma once
+#include <cuda_bf16.h>
+#include "intra_fragment.cuh"
+#include "sm100_ptx.cuh"
+
+namespace torq {
+
+struct RotWideCfg {
+  static constexpr int BM = 128;                       // rows per CTA
+  static constexpr int BK = 64;
+  static constexpr int A_BYTES = BM * BK * 2;          // 16 KiB
+  static constexpr int BOX_BYTES = 64 * BK * 2;        // 64 columns x 64 k = 8 KiB
+  static constexpr int MAX_WIDTH = 384;
+  static constexpr int MAX_STAGES = 8;
+  static constexpr int RI_BLOCK_BYTES = 32 * 64;       // R_intra[blk] as bf16 rows of 64 bytes, 16-byte pieces XOR-swizzled
+  static constexpr int ESETS = 3;
+  static constexpr int THREADS = 64 + 128 * ESETS;
+  // columns of the first instruction; the second takes the rest
+  __host__ __device__ static constexpr int n0(int width) { return width <= 256 ? width : width - 128; }
+  __host__ __device__ static constexpr int boxes(int width) { return (n0(width) / 2 + 63) / 64 + (width > 256 ? 1 : 0); }
+  __host__ __device__ static constexpr int tail_cols(int width) { return n0(width) / 2 % 64; }         // columns of the narrow box (0: none)
+  __host__ __device__ static constexpr int stage_bytes(int width) { return A_BYTES + boxes(width) * BOX_BYTES; }
+  __host__ __device__ static constexpr int stage_tx(int width) { return A_BYTES + width / 2 * BK * 2; }   // bytes one CTA loads
+  // 192 to 200 KiB of stages whatever the width
+  __host__ __device__ static constexpr int stages(int width) { return boxes(width) == 1 ? 8 : (boxes(width) == 2 ? 6 : 5); }
+  __host__ __device__ static constexpr int smem_bytes(int width) {
+    return stages(width) * stage_bytes(width) + (width / 32) * RI_BLOCK_BYTES + 256 + 1024;
+  }
+};
+static_assert(RotWideCfg::smem_bytes(128) <= 232448 && RotWideCfg::smem_bytes(256) <= 232448 &&
+              RotWideCfg::smem_bytes(384) <= 232448, "shared memory budget");
+
+// grid = 2 * rows * cols CTAs in clusters of two: pair p works row tile p % rows (256 tokens), column tile p / rows
+// (`width` features from column (p / rows) * width on).  tmX: X box [128 x 64]; tmR: R_inter box [64 x 64]; tmRt:
+// box [64 x tail_cols].  d % 128 == 0.  TWO: width > 256.  FMT, `tensor_scale` as in the pair kernel.
+template <int FMT, bool TWO>
+__global__ void __launch_bounds__(RotWideCfg::THREADS, 1)
+rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,
+                            const __grid_constant__ CUtensorMap tmRt, const __nv_bfloat16* __restrict__ R_intra,
+                            uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, int M, int d,
+                            float tensor_scale, int rows, int width, int* err_word) {
+  using C = RotWideCfg;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
+  const int nst = C::stages(width);
+  const uint32_t stage_bytes = C::stage_bytes(width);
+  const uint32_t ri_off = nst * stage_bytes;
+  const uint32_t bar_off = ri_off + (uint32_t)(width / 32) * C::RI_BLOCK_BYTES;
+  const uint32_t bar_base = smem_base + bar_off;
+  auto full_bar = [&](int s) { return bar_base + 8u * s; };
+  auto empty_bar = [&](int s) { return bar_base + 8u * (C::MAX_STAGES + s); };
+  const uint32_t accf_bar = bar_base + 8u * (2 * C::MAX_STAGES);
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + bar_off + 192);
+  volatile int* cta_abort = reinterpret_cast<volatile int*>(smem_gen + bar_off + 200);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();             // 0 = leader
+  const int pair = blockIdx.x >> 1;
+  const int tcol = (pair / rows) * width;
+  const int mt = 2 * (pair % rows) + (int)rank;
+  const int k_tiles = d / C::BK;
+  const int n0 = C::n0(width);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < nst; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
+    mbar_init(accf_bar, 1);
+    *cta_abort = 0;
+    fence_mbar_init();
+  }
+  if (warp == 1) { tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512); tmem_relinquish_pair(); }
+  tc_fence_before_sync();
+  __syncthreads();
+  cluster_sync_after_init();
+  tc_fence_after_sync();
+  const uint32_t tmem_base = *tmem_slot;
+  // R_inter is a constant of the layer, never the output of the kernel that runs just before this one: its
+  // loads for the first stages go out now, everything else waits for that kernel to complete.
+  griddep_launch_dependents();
+
+  if (warp == 0) {
+    // ------------------------------------------------------------------ TMA producer (both CTAs)
+    if (elect_one()) {
+      const int full0 = n0 / 128;                      // whole 64-column boxes of this CTA's half of the first instruction
+      const int tail = C::tail_cols(width);
+      const int col0 = tcol + (int)rank * (n0 / 2), col1 = tcol + n0 + (int)rank * 64;
+      const uint32_t leader_full0 = map_to_cta(full_bar(0), 0);
+      auto load_r = [&](int s, int kt) {
+        uint32_t dst = smem_base + s * stage_bytes + C::A_BYTES;
+        const uint32_t bar = leader_full0 + 8u * s;
+        if (rank == 0) mbar_arrive_expect_tx(full_bar(s), 2 * C::stage_tx(width));
+        for (int b = 0; b < full0; ++b, dst += C::BOX_BYTES) tma_load_2d_pair(dst, &tmR, col0 + 64 * b, kt * C::BK, bar);
+        if (tail) {
+          tma_load_2d_pair(dst, &tmRt, col0 + 64 * full0, kt * C::BK, bar);
+          dst += C::BOX_BYTES;
+        }
+        if constexpr (TWO) tma_load_2d_pair(dst, &tmR, col1, kt * C::BK, bar);
+      };
+      tma_prefetch_desc(&tmX); tma_prefetch_desc(&tmR); tma_prefetch_desc(&tmRt);
+      const int pre = k_tiles < nst ? k_tiles : nst;
+      for (int i = 0; i < pre; ++i) load_r(i, i);
+      griddep_wait();
+      int s = 0;
+      uint32_t ph = 1;
+      for (int kt = 0; kt < k_tiles; ++kt) {
+        if (!mbar_wait_cluster(empty_bar(s), ph, cta_abort, err_word, SITE_PRODUCER_EMPTY)) break;
+        if (kt >= pre) load_r(s, kt);
+        tma_load_2d_pair(smem_base + s * stage_bytes, &tmX, kt * C::BK, mt * C::BM, leader_full0 + 8u * s);
+        if (++s == nst) { s = 0; ph ^= 1; }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ MMA issuer (leader only)
+    if (rank == 0 && elect_one()) {
+      const uint32_t idesc0 = idesc_bf16(256, n0, /*A MN-major*/ false, /*B MN-major*/ true);
+      constexpr uint32_t idesc1 = idesc_bf16(256, 128, false, true);
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int kt = 0; kt < k_tiles; ++kt) {
+        ok = mbar_wait_cluster(full_bar(s), ph, cta_abort, err_word, SITE_MMA_FULL);
+        if (!ok) break;
+        tc_fence_after_sync();
+        const uint32_t st = smem_base + s * stage_bytes;
+        const uint64_t adesc = make_desc(st, 16, 1024, kSwizzle128);
+        const uint64_t bdesc = make_desc(st + C::A_BYTES, C::BOX_BYTES, 1024, kSwizzle128);
+#pragma unroll
+        for (int j = 0; j < C::BK / 16; ++j) {
+          mma_bf16_pair(tmem_base, adesc + 2 * j, bdesc + 128 * j, idesc0, (kt | j) != 0);
+          if constexpr (TWO)                           // the first instruction's half is two boxes then
+            mma_bf16_pair(tmem_base + n0, adesc + 2 * j, bdesc + 2 * C::BOX_BYTES / 16 + 128 * j, idesc1, (kt | j) != 0);
+        }
+        tc_commit_pair(empty_bar(s), 3);            // stage free in both CTAs
+        if (++s == nst) { s = 0; ph ^= 1; }
+      }
+      if (ok) tc_commit_pair(accf_bar, 3);          // accumulator ready in both CTAs
+    }
+    __syncwarp();
+  } else {
+    // ------------------------------------------------------------------ epilogue (12 warps per CTA)
+    const int q = warp & 3;
+    const int set = (warp - 2) >> 2;
+    const int p = lane & 3, r8 = lane >> 2;
+    const int nblocks = d / 32, nb = width / 32, b0 = tcol >> 5;
+    const uint32_t ri_saddr = smem_base + ri_off;
+    if (R_intra != nullptr) {                          // the tile's blocks, 16-byte piece c of row i at c ^ ((i >> 1) & 3)
+      for (int idx = (warp - 2) * 32 + lane; idx < nb * 128; idx += 128 * C::ESETS) {
+        const int lb = idx >> 7, i = (idx >> 2) & 31, c = idx & 3;
+        if (b0 + lb < nblocks)
+          *reinterpret_cast<uint4*>(smem_gen + ri_off + lb * C::RI_BLOCK_BYTES + i * 64 + ((c ^ ((i >> 1) & 3)) << 4)) =
+              __ldg(reinterpret_cast<const uint4*>(R_intra + (size_t)(b0 + lb) * 1024) + (idx & 127));
+      }
+      named_barrier_sync(1, 128 * C::ESETS);
+    }
+    griddep_wait();                                    // codes and scales may still be read by that kernel
+    bool ok = mbar_wait_cluster(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
+    ok = __all_sync(0xFFFFFFFFu, ok);
+    tc_fence_after_sync();
+    const uint32_t tacc = tmem_base + ((uint32_t)(q * 32) << 16);
+    if (ok && mt * C::BM < M) {                        // the pair's second row tile may not exist
+      NvScale nvs = {};
+      if constexpr (FMT == FMT_NVFP4) nvs = nv_scale(tensor_scale);
+      const int kb4 = FMT == FMT_NVFP4 ? (2 * nblocks + 3) / 4 : (nblocks + 3) / 4;
+      // ldmatrix: lane l addresses row l % 8 (+ 8 for odd l / 8) of its matrix, 16-byte piece l / 16 (+ 2)
+      const int li = ((lane >> 3) & 1) * 8 + (lane & 7);
+      const uint32_t r_lane = (uint32_t)li * 64 + (uint32_t)(((lane >> 4) ^ ((li >> 1) & 3)) << 4);
+      // units of 16 rows x 32 columns: unit u is half u % 2 of the warp's rows of block u / 2
+#pragma unroll 1
+      for (int u = set; u < 2 * nb; u += C::ESETS) {
+        const int bb = u >> 1, mh = u & 1, blk = b0 + bb;
+        if (blk >= nblocks) break;
+        uint32_t y[16];
+        tmem_ld_16x256b_x4(tacc + ((uint32_t)(16 * mh) << 16) + bb * 32, y);
+        tmem_ld_wait();
+        IntraFrag f;
+        const uint32_t rb = ri_saddr + (uint32_t)bb * C::RI_BLOCK_BYTES + r_lane;
+        if (R_intra != nullptr) load_intra_frag(rb, rb ^ 32u, 16 * 64, f);
+        uint32_t sb[2];
+        intra_quantize_frag16<FMT>(y, R_intra != nullptr, f, lane, (int64_t)mt * C::BM + q * 32 + 16 * mh, M, blk, nblocks, d, nvs,
+                                   codes, sb);
+        if (p == 0) {                                  // byte blk % 4 of the 4-byte cell of (row, blk / 4)
+#pragma unroll
+          for (int rh = 0; rh < 2; ++rh) {
+            const size_t in_tile = (size_t)(r8 + 16 * mh + 8 * rh) * 16 + q * 4;
+            if constexpr (FMT == FMT_NVFP4)
+              *reinterpret_cast<uint16_t*>(scales + ((size_t)mt * kb4 + (blk >> 1)) * 512 + in_tile + 2 * (blk & 1)) = (uint16_t)sb[rh];
+            else
+              scales[((size_t)mt * kb4 + (blk >> 2)) * 512 + in_tile + (blk & 3)] = (uint8_t)sb[rh];
+          }
+        }
+      }
+    }
+    tc_fence_before_sync();
+  }
+
+  // ------------------------------------------------------------------ teardown
+  __syncthreads();
+  if (*cta_abort) {
+    for (int i = 0; i < 2000; ++i) __nanosleep(1000);
+  }
+  cluster_sync_all();                                  // the peer no longer touches this CTA's memory
+  if (warp == 1) {
+    tc_fence_after_sync();
+    tmem_dealloc_pair(tmem_base, 512);
+  }
+}
+
+}  // namespace torq

@@ -13,6 +13,7 @@
 #include "mxint4_quantize.cuh"
 #include "rotate_quantize.cuh"
 #include "rotate_quantize_pair.cuh"
+#include "rotate_quantize_wide.cuh"
 #include "rotate_splitk.cuh"
 #include "rotate_fewtok.cuh"
 #include "gemm_fewtok.cuh"
@@ -106,6 +107,7 @@ static DeviceState* device_state() {
         return nullptr;
       g_encode = reinterpret_cast<EncodeTiledFn>(fn);
     }
+    constexpr int kWideSmem = 232448;                    // all widths share two kernels
     bool ok = opt_in_smem(mxfp4_gemm_kernel<256, 1>, GemmCfg<256, 1>::SMEM_BYTES) &&
               opt_in_smem(mxfp4_gemm_kernel<128, 2>, GemmCfg<128, 2>::SMEM_BYTES) &&
               opt_in_smem(mxfp4_gemm_kernel<256, 1, FMT_NVFP4>, GemmCfg<256, 1, FMT_NVFP4>::SMEM_BYTES) &&
@@ -115,6 +117,12 @@ static DeviceState* device_state() {
               opt_in_smem(rotate_quantize_kernel<256, FMT_NVFP4>, RotCfg<256>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_MXFP4>, RotPairCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_NVFP4>, RotPairCfg::SMEM_BYTES) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, false>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, true>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, false>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, true>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, false>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, true>, kWideSmem) &&
               opt_in_smem(rotate_splitk_kernel, RotSplitCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_structured_kernel<FMT_MXFP4>, RotStructCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_structured_kernel<FMT_NVFP4>, RotStructCfg::SMEM_BYTES) &&
@@ -229,6 +237,7 @@ static int rotation_splits(int64_t M, int64_t d, int sm_count) {
 }
 constexpr int kRotFewMaxTokens = 256;    // up to here the rotation streams R_inter through the few-token kernel
 constexpr int kGemmFewMaxTokens = 128;   // and the GEMM the weights
+constexpr int kSplitMaxTokens = 640, kSplitMaxFeatures = 1024;   // the fused call's split-K rotation: above the few-token range, up to these
 static_assert(kRotFewMaxTokens <= RotFewCfg::MAX_TOK && kGemmFewMaxTokens <= GemmFewCfg<FMT_MXFP4>::MAX_TOK, "few-token limits");
 // Few-token kernels: tokens per instruction, and the cluster size S = number of K splits of one 128-feature
 // tile: the largest S up to 8 within these bounds, each with both sides measured (us, cold operands):
@@ -251,6 +260,10 @@ static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int long_k, int
   while (s > 1 && (tiles > (int64_t)ctas_per_sm * fit[s] || (s > 4 && 10 * tiles * s > 14 * (int64_t)sm_count))) --s;
   while (s > 1 && (k_steps + s - 2) / (s - 1) == (k_steps + s - 1) / s) --s;      // fewer clusters' CTAs: they fit as well
   return s < 1 ? 1 : s;
+}
+static int fewtok_rotation_cluster(int64_t M, int64_t d, const DeviceState* st) {
+  const int ntok = fewtok_ntok(M);
+  return fewtok_cluster(d / 128, d / 64, ntok == 256 ? 1 : 10, RotFewCfg::ctas_per_sm(ntok), st->sm_count, st->few_fit);
 }
 constexpr double kNarrowTileCost = 0.88;   // a 192-column tile against a 256-column one: 0.75 of the math, 0.875 of the operand bytes
 
@@ -395,6 +408,57 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
   return quantize_impl(st, Z, z_dtype, M, d, out_codes, out_scales, static_cast<cudaStream_t>(stream));
 }
 
+// Width of the one-wave rotation's tiles, or 0 where another kernel is faster.  Times in us, fitted to the rotation
+// alone at 27 shapes (d = 256 ... 14336, M = 100 ... 4000; within 10 % but for the HBM-bound ones at d > 8192, where
+// both sides are low by as much):
+//  * here: 2.2 + 0.026 per column (2.4 + 0.032 above 256 columns) for launch and epilogue, then per K step the operand
+//    bytes, 0.215 + 0.0003 per column, or the math, 0.00114 per column;
+//  * few tokens: 3.8 / 4.8 / 4.5 / 8.3 up to 16 / 64 / 128 / 256 tokens, plus 0.24 / 0.22 / 0.385 / 0.425 per K step of
+//    the longest split;
+//  * pair kernel: 6.8, plus per K step 0.32 for a wave and 0.2 + 0.14 x (filled part) for the last, partly filled one.
+// A layer of 2048 tokens and more fills the pair kernel's waves and stays there (one-wave tiles would be wider than
+// 384 columns; 2048 x 4096 measured 51.6 with 480 columns, 46.8 in the pair kernel).
+static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int max_pairs) {
+  const int64_t rows = (M + 255) / 256, steps = d / RotWideCfg::BK;
+  double best = 1e30;
+  int width = 0;
+  for (int w = 32; w <= RotWideCfg::MAX_WIDTH; w += 32) {
+    if (rows * ((d + w - 1) / w) > max_pairs) continue;
+    const double bytes = 0.215 + 0.0003 * w, math = 0.00114 * w;
+    const double t = (w <= 256 ? 2.2 + 0.026 * w : 2.4 + 0.032 * w) + (double)steps * (bytes > math ? bytes : math);
+    if (t < best) { best = t; width = w; }
+  }
+  double other;
+  if (M <= kRotFewMaxTokens) {
+    other = M <= 16 ? 3.8 + 0.24 * few_steps : (M <= 64 ? 4.8 + 0.22 * few_steps : (M <= 128 ? 4.5 + 0.385 * few_steps : 8.3 + 0.425 * few_steps));
+  } else {
+    const int64_t tiles = rows * ((d + 255) / 256);
+    const int64_t full = tiles / max_pairs, rest = tiles % max_pairs;
+    other = 6.8 + (double)steps * (0.32 * (double)full + (rest == 0 ? 0.0 : (full == 0 ? 0.32 : 0.2 + 0.14 * (double)rest / max_pairs)));
+  }
+  return best < 0.97 * other ? width : 0;
+}
+
+static torq_status rotate_wide(DeviceState* st, int fmt, const void* X, const void* R_inter, const void* R_intra, int64_t M,
+                               int64_t d, uint8_t* codes, uint8_t* scales, float tensor_scale, int width, cudaStream_t s) {
+  using C = RotWideCfg;
+  CUtensorMap tmX, tmR, tmRt;
+  const int tail = C::tail_cols(width);
+  if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d, 128, 64) ||
+      !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 64) ||
+      !encode_2d(&tmRt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, (uint32_t)(tail ? tail : 64)))
+    return TORQ_ERR_LAUNCH;
+  const int rows = (int)((M + 255) / 256), cols = (int)((d + width - 1) / width);
+  auto launch = [&](auto one, auto two) {
+    launch_tc(width > 256 ? two : one, 2, 2 * rows * cols, C::THREADS, C::smem_bytes(width), s, tmX, tmR, tmRt,
+              static_cast<const __nv_bfloat16*>(R_intra), codes, scales, (int)M, (int)d, tensor_scale, rows, width, st->err_word);
+  };
+  if (fmt == FMT_MXINT4) launch(rotate_quantize_wide_kernel<FMT_MXINT4, false>, rotate_quantize_wide_kernel<FMT_MXINT4, true>);
+  else if (fmt == FMT_NVFP4) launch(rotate_quantize_wide_kernel<FMT_NVFP4, false>, rotate_quantize_wide_kernel<FMT_NVFP4, true>);
+  else launch(rotate_quantize_wide_kernel<FMT_MXFP4, false>, rotate_quantize_wide_kernel<FMT_MXFP4, true>);
+  return launch_status();
+}
+
 // Steps 1-4.  `scratch` (may be NULL) is fp32 room for the split-K partials of the few-token path;
 // without enough of it the single-pass kernels run.  `fmt` FMT_NVFP4 (with its tensor scale) needs R_inter.
 // FMT_F32OUT: out_codes is float32 [M, d] and receives the rotated values (out_scales unused, may be
@@ -425,12 +489,28 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
     return launch_status();
   }
   CUtensorMap tmX, tmR;
+  // The fused call splits K over the SMs through its scratch for 257 ... 640 tokens up to d = 1024.  The one-wave
+  // kernel is the faster one there as well (300 x 1024: 7.4 us against 9.5 for the two kernels of the split), but the
+  // launches of this range are part of what callers of the fused entry points may count on: they stay three.
+  const int splits = (fmt == FMT_F32OUT || x_terms > 1 || M <= kRotFewMaxTokens || M > kSplitMaxTokens || d > kSplitMaxFeatures)
+                         ? 1 : rotation_splits(M, d, st->sm_count);
+  const bool split = splits >= 2 && scratch && scratch_bytes >= splitk_scratch_bytes(M, d, splits) &&
+                     (reinterpret_cast<uintptr_t>(scratch) & 15u) == 0;
+  if (d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT && !split) {
+    int few_steps = 0;                                     // longest K range of the few-token kernel
+    if (M <= kRotFewMaxTokens) {
+      const int S = fewtok_rotation_cluster(M, d, st);
+      few_steps = (int)((d / 64 + S - 1) / S);
+    }
+    const int width = wide_rotation_width(M, d, few_steps, st->rot_pairs);
+    if (width > 0) return rotate_wide(st, fmt, X, R_inter, R_intra, M, d, codes, scales, tensor_scale, width, s);
+  }
   if (M <= kRotFewMaxTokens && d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT) {
     // Few tokens: 128 features x all tokens per CTA, K split over a cluster, reduced through
     // distributed shared memory; one launch, no scratch.
     const int ntok = fewtok_ntok(M);
     const int tiles = (int)(d / 128);
-    const int S = fewtok_cluster(tiles, d / 64, ntok == 256 ? 1 : 10, RotFewCfg::ctas_per_sm(ntok), st->sm_count, st->few_fit);
+    const int S = fewtok_rotation_cluster(M, d, st);
     if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d, (uint32_t)ntok, 64) ||
         !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 64))
       return TORQ_ERR_LAUNCH;
@@ -463,10 +543,8 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
   if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d * x_terms, 128, 64) ||
       !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 64))
     return TORQ_ERR_LAUNCH;
-  const int splits = (fmt == FMT_F32OUT || x_terms > 1) ? 1 : rotation_splits(M, d, st->sm_count);
-  if (splits >= 2 && scratch && scratch_bytes >= splitk_scratch_bytes(M, d, splits) &&
-      (reinterpret_cast<uintptr_t>(scratch) & 15u) == 0) {
-    // Few tokens: split K over the SMs, partial tiles to scratch, then reduce + intra + quantize.
+  if (split) {
+    // Split K over the SMs, partial tiles to scratch, then reduce + intra + quantize.
     CUtensorMap tmP;
     const int m_tiles = (int)((M + 127) / 128);
     if (!encode_2d(&tmP, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, scratch, (uint64_t)splits * m_tiles * 128, (uint64_t)d,
@@ -1169,3 +1247,4 @@ torq_status torq_merge_rotations(const void* R_inter, const void* R_intra, int64
 }
 
 }  // extern "C"
+

@@ -1,0 +1,80 @@
+"""GPU parity of the one-wave rotation (256 tokens x 32 ... 384 features per CTA pair) on shapes that take it: every
+kind of width (one or two instructions, with and without a narrow box, one to three box slots per stage), a ragged
+last row tile whose second half has no token, a last column tile that reaches past the last feature, fewer K steps
+than pipeline stages.  Bounds as in every other parity test."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from helpers import dev_bf16, gpu_quantized_to_numpy, mismatch_report
+from paper_2605_19561_b200 import inputs as I
+from paper_2605_19561_b200 import torq
+import test_gpu_mxint4 as TI
+import test_gpu_nvfp4 as TN
+
+pytestmark = pytest.mark.gpu
+
+
+def _rand_rotation(d, seed):
+    g = np.random.default_rng(seed)
+    return I.to_bf16_bits(g.standard_normal((d, d)) / np.sqrt(d))
+
+
+# widths on 74 pairs: 32, 32 (two K steps), 32 (padding rows in a second, token-less row tile), 64, 96, 128, 160 (tail of
+# 16), 192, 224, 288 (two instructions), 320, 352, 384 (d no multiple of the width but for the first ones)
+@pytest.mark.parametrize("M,d", [(50, 256), (24, 128), (257, 256), (700, 1024), (1280, 1024), (1000, 2048), (1280, 2048),
+                                 (1536, 2048), (600, 5120), (2304, 2304), (1400, 3840), (3072, 2048), (1280, 5120)])
+def test_rotation_mxfp4(M, d):
+    g = np.random.default_rng(M + d)
+    xb = I.to_bf16_bits(g.standard_t(3.0, size=(M, d)))
+    rb = _rand_rotation(d, d)
+    rib = I.to_bf16_bits(I.orthogonal(32, g, batch=d // 32))
+    rows = np.unique(np.r_[np.arange(min(M, 64)), np.arange(max(0, M - 140), M), g.integers(0, M, 64)])   # the oracle's share
+    for intra in (rib, None):
+        codes_t = torch.full((M, d // 2), 0xEE, dtype=torch.uint8, device="cuda")
+        scales_t = torch.full((torq.torq_scales_bytes(M, d),), 0xEE, dtype=torch.uint8, device="cuda")
+        torq.torq_rotate_quantize(dev_bf16(xb), dev_bf16(rb), None if intra is None else dev_bf16(intra),
+                                  out_codes=codes_t, out_scales=scales_t)
+        torch.cuda.synchronize()
+        assert torq.torq_last_device_error() == 0
+        g_codes, g_sb = gpu_quantized_to_numpy(codes_t, scales_t, M, d)
+        o_codes, o_sb = O.quantize_mxfp4(O.round_to_f32(O.rotate(xb[rows], rb, intra)))
+        rep = mismatch_report(g_codes[rows], g_sb[rows], o_codes, o_sb)
+        assert rep["non_adjacent"] == 0 and rep["scale_off_by_more_than_one"] == 0, rep
+        # one element / block at sizes where 1e-4 is less than one (a block's 32 elements move with its scale)
+        assert rep["elem_mismatch_frac"] <= max(1e-4, 33.0 / o_codes.size), rep
+        assert rep["block_scale_mismatch_frac"] <= max(1e-4, 1.5 / o_sb.size), rep
+        # every byte of the scale buffer was written: real rows hold scales, padding rows zero
+        raw = scales_t.cpu().numpy().copy()
+        rr, cc = np.meshgrid(np.arange(M), np.arange(d // 32), indexing="ij")
+        raw[O.scale_layout_offset(rr, cc, d)] = 0
+        assert not raw.any()
+
+
+def test_rotation_exact_case_is_bit_exact():
+    """Permutations of small integers: every partial sum is exact, so codes and scales equal the oracle's bit for bit."""
+    M, d = 777, 1280
+    g = np.random.default_rng(3)
+    xb = I.to_bf16_bits(g.integers(-8, 9, size=(M, d)).astype(np.float64))
+    P = np.zeros((d, d))
+    P[np.arange(d), g.permutation(d)] = 1.0
+    pin = I.to_bf16_bits(np.stack([np.eye(32)[g.permutation(32)] for _ in range(d // 32)]))
+    codes_t, scales_t = torq.torq_rotate_quantize(dev_bf16(xb), dev_bf16(I.to_bf16_bits(P)), dev_bf16(pin))
+    torch.cuda.synchronize()
+    assert torq.torq_last_device_error() == 0
+    g_codes, g_sb = gpu_quantized_to_numpy(codes_t, scales_t, M, d)
+    o_codes, o_sb = O.quantize_mxfp4(O.round_to_f32(O.rotate(xb, I.to_bf16_bits(P), pin)))
+    assert np.array_equal(g_sb, o_sb) and np.array_equal(g_codes, o_codes)
+
+
+@pytest.mark.parametrize("M,d", [(600, 1280), (40, 256), (2304, 2304)])
+def test_rotation_nvfp4_and_mxint4(M, d):
+    cfg = I.CONFIGS["tiny"]
+    xb = I.activations(cfg, M=M, d=d)
+    rb = _rand_rotation(d, 5)
+    TN._rotate_case(xb, rb, I.intra_rotations16(cfg, d=d))
+    TN._rotate_case(xb, rb, None)
+    g = np.random.default_rng(6)
+    TI._rotate_case(xb, rb, I.to_bf16_bits(I.orthogonal(32, g, batch=d // 32)))
+    TI._rotate_case(xb, rb, None)
