@@ -8,6 +8,7 @@
 #include "../../include/torq.h"
 #include "mxfp4_gemm.cuh"
 #include "mxfp4_gemm_pair.cuh"
+#include "mxfp4_gemm_wide.cuh"
 #include "quantize.cuh"
 #include "nvfp4_quantize.cuh"
 #include "mxint4_quantize.cuh"
@@ -107,7 +108,7 @@ static DeviceState* device_state() {
         return nullptr;
       g_encode = reinterpret_cast<EncodeTiledFn>(fn);
     }
-    constexpr int kWideSmem = 232448;                    // all widths share two kernels
+    constexpr int kWideSmem = 232448;                    // the widths share the kernels
     bool ok = opt_in_smem(mxfp4_gemm_kernel<256, 1>, GemmCfg<256, 1>::SMEM_BYTES) &&
               opt_in_smem(mxfp4_gemm_kernel<128, 2>, GemmCfg<128, 2>::SMEM_BYTES) &&
               opt_in_smem(mxfp4_gemm_kernel<256, 1, FMT_NVFP4>, GemmCfg<256, 1, FMT_NVFP4>::SMEM_BYTES) &&
@@ -123,6 +124,12 @@ static DeviceState* device_state() {
               opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, true>, kWideSmem) &&
               opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, false>, kWideSmem) &&
               opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, true>, kWideSmem) &&
+              opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXFP4, false>, kWideSmem) &&
+              opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXFP4, true>, kWideSmem) &&
+              opt_in_smem(mxfp4_gemm_wide_kernel<FMT_NVFP4, false>, kWideSmem) &&
+              opt_in_smem(mxfp4_gemm_wide_kernel<FMT_NVFP4, true>, kWideSmem) &&
+              opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXINT4, false>, kWideSmem) &&
+              opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXINT4, true>, kWideSmem) &&
               opt_in_smem(rotate_splitk_kernel, RotSplitCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_structured_kernel<FMT_MXFP4>, RotStructCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_structured_kernel<FMT_NVFP4>, RotStructCfg::SMEM_BYTES) &&
@@ -677,6 +684,60 @@ torq_status torq_rotate_quantize_structured_nvfp4(const void* X, const void* R_B
 
 }  // extern "C"
 
+// Width of the one-wave GEMM's tiles, or 0 where another kernel is faster.  Times in us, fitted to MXFP4 with bf16 output
+// at K = 256 ... 14336, N = 256 ... 12288, M = 200 ... 8000 (within 8 %); f = filled part of a wave:
+//  * here: 2.3 + 0.0062 per column + f for launch and epilogue, then per K step 0.265 or the math, 0.0011 per
+//    column, + 0.025 f;
+//  * pair kernel: one wave 4.1 + 0.9 f + (0.285 + 0.04 f) per K step, more (the last one as narrower tiles) 5.2 + per K step
+//    0.325 for a full wave and 0.21 + 0.14 f for the last;
+//  * single CTAs (129 to 256 tokens, few column tiles): 3.2 + 1.3 f + 0.285 per K step.
+// Where it pays: 777 x 5120, K = 14336 (80 pair tiles) 35.1 -> 28.5, K = 4096 13.8 -> 12.3; 1280 x 4096, K = 14336 35.2 ->
+// 29.1; few and narrow outputs, 2000 x 256, K = 1024 5.2 -> 3.9.
+static int wide_gemm_width(int64_t M, int64_t N, int64_t steps, bool pairs, int max_pairs) {
+  const int64_t rows = (M + 255) / 256;
+  double best = 1e30;
+  int width = 0;
+  for (int w = 64; w <= GemmWideCfg<>::MAX_WIDTH; w += 64) {
+    const int64_t tiles = rows * ((N + w - 1) / w);
+    if (tiles > max_pairs) continue;
+    const double f = (double)tiles / max_pairs, math = 0.0011 * w;
+    const double t = 2.3 + 0.0062 * w + f + (double)steps * ((math > 0.265 ? math : 0.265) + 0.025 * f);
+    if (t < best) { best = t; width = w; }
+  }
+  const int64_t tiles = rows * ((N + 255) / 256), full = tiles / max_pairs, rest = tiles % max_pairs;
+  const double f = (double)rest / max_pairs;
+  double other;
+  if (!pairs) other = 3.2 + 1.3 * (double)((M + 127) / 128 * ((N + 127) / 128)) / (2 * max_pairs) + 0.285 * (double)steps;
+  else if (full == 0) other = 4.1 + 0.9 * f + (double)steps * (0.285 + 0.04 * f);
+  else other = 5.2 + (double)steps * (0.325 * (double)full + (rest ? 0.21 + 0.14 * f : 0.0));
+  return best < 0.97 * other ? width : 0;
+}
+
+template <int FMT>
+static torq_status gemm_wide(DeviceState* st, const void* Aq, const void* As, const void* Wq, const void* Ws, int64_t M, int64_t N,
+                             int64_t K, void* Y, torq_dtype y_dtype, float alpha, int width, cudaStream_t s) {
+  using C = GemmWideCfg<FMT>;
+  const uint64_t krow = (uint64_t)(FMT == FMT_MXINT4 ? K : K / 2);
+  const uint64_t sf_words = (uint64_t)(K / (FMT == FMT_NVFP4 ? 64 : 128)) * 128;   // scale words per 128 rows
+  const bool ybf = y_dtype == TORQ_BF16;
+  CUtensorMap tmA, tmB, tmB1, tmSFA, tmSFB, tmY;
+  if (!encode_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Aq, (uint64_t)M, krow, 128, 128) ||
+      !encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, (uint32_t)C::n0(width) / 2, 128) ||
+      !encode_2d(&tmB1, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, 64, 128) ||
+      !encode_2d(&tmSFA, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, As, (uint64_t)((M + 127) / 128), sf_words, 1, C::SF_BOX_WORDS,
+                 CU_TENSOR_MAP_SWIZZLE_NONE) ||
+      !encode_2d(&tmSFB, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, Ws, (uint64_t)((N + 127) / 128), sf_words, (uint32_t)C::chunks(width),
+                 C::SF_BOX_WORDS, CU_TENSOR_MAP_SWIZZLE_NONE) ||
+      !encode_2d(&tmY, ybf ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, ybf ? 2 : 4, Y, (uint64_t)M,
+                 (uint64_t)N, 32, ybf ? 64 : 32))
+    return TORQ_ERR_LAUNCH;
+  const int rows = (int)((M + 255) / 256), cols = (int)((N + width - 1) / width);
+  launch_tc(width > 256 ? mxfp4_gemm_wide_kernel<FMT, true> : mxfp4_gemm_wide_kernel<FMT, false>, 2, 2 * rows * cols, C::THREADS,
+            C::smem_bytes(width), s, tmA, tmB, tmB1, tmSFA, tmSFB, tmY, ybf ? 1 : 0, (int)M, (int)N, (int)K, rows, width, alpha,
+            st->err_word);
+  return launch_status();
+}
+
 // Step 5 for either format; `alpha` multiplies the NVFP4 result (product of the tensor scales).
 template <int FMT>
 static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, const void* Ws, int64_t M,
@@ -719,7 +780,9 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
   // that the pairs would leave more than half of the SMs idle: 128 x 128 tiles on single CTAs then
   // put four times as many SMs to work on streaming W.
   const int64_t pair_tiles = ((M + 255) / 256) * ((N + BN - 1) / BN);
-  const bool use_pairs = M > 128 && !(M <= 256 && 4 * pair_tiles <= st->sm_count);
+  const bool use_pairs = !(M <= 256 && 4 * pair_tiles <= st->sm_count);
+  const int width = wide_gemm_width(M, N, (K + GemmWideCfg<FMT>::BK - 1) / GemmWideCfg<FMT>::BK, use_pairs, st->gemm_pairs);
+  if (width > 0) return gemm_wide<FMT>(st, Aq, As, Wq, Ws, M, N, K, Y, y_dtype, alpha, width, s);
   if (use_pairs) {
     CUtensorMap tmSFA, tmSFB;
     const uint64_t kb4 = (uint64_t)(K / (FMT == FMT_NVFP4 ? 64 : 128));   // 512-byte scale chunks per row

@@ -1,13 +1,13 @@
-"""GPU parity of the one-wave rotation (256 tokens x 32 ... 384 features per CTA pair) on shapes that take it: every
+"""GPU parity of the one-wave kernels: the rotation (256 tokens x 32 ... 384 features per CTA pair) on shapes that take it: every
 kind of width (one or two instructions, with and without a narrow box, one to three box slots per stage), a ragged
 last row tile whose second half has no token, a last column tile that reaches past the last feature, fewer K steps
-than pipeline stages.  Bounds as in every other parity test."""
+than pipeline stages; and the GEMM built the same way.  Bounds as in every other parity test."""
 import numpy as np
 import pytest
 import torch
 
 import oracle as O
-from helpers import dev_bf16, gpu_quantized_to_numpy, mismatch_report
+from helpers import dev_bf16, dev_u8, gpu_quantized_to_numpy, mismatch_report
 from paper_2605_19561_b200 import inputs as I
 from paper_2605_19561_b200 import torq
 import test_gpu_mxint4 as TI
@@ -78,3 +78,52 @@ def test_rotation_nvfp4_and_mxint4(M, d):
     g = np.random.default_rng(6)
     TI._rotate_case(xb, rb, I.to_bf16_bits(I.orthogonal(32, g, batch=d // 32)))
     TI._rotate_case(xb, rb, None)
+
+
+# ------------------------------------------------------------------------------------- GEMM
+def _rand_operand(rows, k, seed):
+    g = np.random.default_rng(seed)
+    return g.integers(0, 16, size=(rows, k), dtype=np.uint8), g.integers(118, 134, size=(rows, k // 32), dtype=np.uint8)
+
+
+# one-wave GEMM: widths 64 and 128 (few output tiles), 192, 320 and 384 (two instructions, W tiles that start 64 rows
+# into a scale chunk); ragged rows and columns, a half last K stage (K % 256 == 128)
+@pytest.mark.parametrize("M,N,K", [(1300, 200, 384), (300, 136, 128), (1000, 1000, 256), (2000, 1096, 256), (777, 5120, 2176),
+                                   (1000, 6136, 4096)])
+def test_gemm_mxfp4(M, N, K):
+    ac, asb = _rand_operand(M, K, 1)
+    wc, wsb = _rand_operand(N, K, 2)
+    ops = (dev_u8(O.pack_codes(ac)), dev_u8(O.swizzle_scales(asb, K, fill=0)), dev_u8(O.pack_codes(wc)),
+           dev_u8(O.swizzle_scales(wsb, K, fill=0)))
+    rows = np.unique(np.r_[np.arange(96), np.arange(M - 140, M)])        # the oracle's share
+    ref = O.gemm_dequant(ac[rows], asb[rows], wc, wsb)
+    out = {}
+    for dt in (torch.float32, torch.bfloat16):
+        Y = torch.full((M + 2, N), 777.0, dtype=dt, device="cuda")
+        torq.torq_mxfp4_gemm(*ops, Y=Y[1:M + 1])
+        torch.cuda.synchronize()
+        assert torq.torq_last_device_error() == 0
+        assert bool((Y[0] == 777).all()) and bool((Y[M + 1] == 777).all())
+        out[dt] = Y[1:M + 1].float().cpu().numpy().astype(np.float64)
+    got = out[torch.float32][rows]
+    assert np.linalg.norm(got - ref) / np.linalg.norm(ref) <= 1e-5
+    assert np.array_equal(out[torch.bfloat16], O.round_to_bf16(out[torch.float32]))     # the same fp32 sums, rounded once
+
+
+@pytest.mark.parametrize("M,N,K", [(300, 136, 384), (777, 5120, 256)])
+def test_gemm_nvfp4_and_mxint4(M, N, K):
+    g = np.random.default_rng(3)
+    ac, wc = (g.integers(0, 16, (r, K), dtype=np.uint8) for r in (M, N))
+    a16, w16 = (g.integers(0x30, 0x40, (r, K // 16), dtype=np.uint8) for r in (M, N))
+    y = torq.torq_nvfp4_gemm(dev_u8(O.pack_codes(ac)), dev_u8(O.nv_swizzle_scales(a16, K)), 0.02, dev_u8(O.pack_codes(wc)),
+                             dev_u8(O.nv_swizzle_scales(w16, K)), 0.01, out_dtype=torch.float32)
+    ref = O.gemm_nvfp4(ac, a16, np.float32(0.02), wc, w16, np.float32(0.01))
+    assert np.linalg.norm(y.cpu().numpy() - ref) / np.linalg.norm(ref) <= 1e-5
+    aq, wq = (g.integers(-7, 8, (r, K)).astype(np.int8) for r in (M, N))
+    asb, wsb = (g.integers(120, 134, (r, K // 32), dtype=np.uint8) for r in (M, N))
+    y = torq.torq_mxint4_gemm(dev_u8(O.int4_to_e4m3(aq)), dev_u8(O.swizzle_scales(asb, K, fill=0)), dev_u8(O.int4_to_e4m3(wq)),
+                              dev_u8(O.swizzle_scales(wsb, K, fill=0)), out_dtype=torch.float32)
+    ref = O.gemm_mxint4(aq, asb, wq, wsb)
+    assert np.linalg.norm(y.cpu().numpy() - ref) / np.linalg.norm(ref) <= 1e-5
+    torch.cuda.synchronize()
+    assert torq.torq_last_device_error() == 0
