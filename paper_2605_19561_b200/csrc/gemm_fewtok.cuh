@@ -2,21 +2,24 @@
 // weights from HBM once.  One kernel, no scratch in global memory.
 //
 // Swapped operands: the tensor-core instruction's 128 rows are 128 output FEATURES (rows of the
-// stored weight W' [N, K]) and its N columns are the tokens (16, 32, 64 or 128):
+// stored weight W' [N, K]) and its N columns are the tokens (16 ... 128, in steps of 16):
 //   D[n, m] = sum_k w^[n, k] a^[m, k]
 //   A = W tile [128 rows x 128 B of K], scale chunks of W;  B = activation tile [tokens x 128 B],
 //   scale chunks of the activations (their single 128-row scale tile).
 // A layer has only N / 128 such tiles (40 at N = 5120), so K is split as well: a CLUSTER of S CTAs
-// shares one tile, CTA r contracts k range r; the fp32 partial tiles stay on the SMs -- each CTA
-// writes its partial [token][feature] into its own shared memory, a cluster barrier publishes them,
-// and CTA r then adds, for the tokens m = r (mod S), the S partials in rank order through
-// distributed shared memory (plain ld.shared::cluster; fixed order) and stores that token's 128
-// outputs as one 256- or 512-byte piece of a row of Y.
+// shares one tile, CTA r contracts k range r; the fp32 partial tiles stay on the SMs and are added in rank order (fixed).
+// As in the few-token rotation they reach the adding CTA in one of two ways:
+//  * PUSH (up to 16 tokens): tokens are dealt in pieces of four, piece c belongs to CTA c % S, and every CTA stores its
+//    partial sums of a piece straight from registers into that CTA's shared memory (st.async, 16 bytes per lane =
+//    four tokens of one feature).  K = N = 5120, M = 1: 4.0 us (4.7 before, pulling); 64 tokens: 7.2 against 6.1.
+//  * pull (more tokens): each CTA writes its partial [token][feature] into its own shared memory, a cluster barrier
+//    publishes them, and CTA r adds, for the tokens m = r (mod S), the S partials read with 16-byte ld.shared::cluster.
+// With S = 1 (an ordinary launch without clusters) the accumulator goes to Y directly.
 //
 // Roles per CTA: warp 0 TMA producer, warp 1 MMA issuer (scale chunks shared -> tensor memory, then the
 // instructions), warps 2..5 epilogue / reduction.  Shared memory: 4 stages of (16 KiB of W + tokens x
-// 128 B + the scale chunks), reused for the partial tile after the mainloop; at most 113 KiB, so these
-// CTAs become resident beside those of the few-token rotation that precedes them in the stream and
+// 128 B + the scale chunks), reused for the partials after the mainloop; at most 113 KiB up to 64 tokens, so
+// these CTAs become resident beside those of the few-token rotation that precedes them in the stream and
 // fetch their first weight stages while it still runs (the weights are constants of the layer).
 #pragma once
 #include <cuda_bf16.h>
@@ -45,9 +48,11 @@ struct GemmFewCfg {
   }
   __host__ __device__ static constexpr int smem_bytes(int ntok) { return stages(ntok) * stage_bytes(ntok) + BAR_BYTES + 1024; }
   __host__ __device__ static constexpr int ctas_per_sm(int ntok) { return smem_bytes(ntok) <= 113 * 1024 ? 2 : 1; }
-  __host__ __device__ static constexpr int max_smem_bytes() {                  // over the token counts in use
-    return smem_bytes(64) > smem_bytes(128) ? smem_bytes(64) : smem_bytes(128);
-  }
+  __host__ __device__ static constexpr int max_smem_bytes() { return smem_bytes(MAX_TOK); }
+  static constexpr int PIECE_BYTES = BF * 16;          // partial sums of four tokens from one CTA: [feature][4 tokens]
+  static constexpr int MAX_PUSH_TOK = 16;
+  // what lies in the stages after the mainloop: the pushed partials of up to four pieces, or the partial tile
+  static_assert(4 * MAX_CLUSTER * PIECE_BYTES <= STAGES * A_BYTES && BF * 4 <= STAGES * 128, "reduction buffers");
   __host__ __device__ static constexpr uint32_t tmem_cols(int ntok) {
     return ntok + 8 * CH <= 32 ? 32u : (ntok + 8 * CH <= 64 ? 64u : (ntok + 8 * CH <= 128 ? 128u : 256u));
   }
@@ -56,8 +61,8 @@ struct GemmFewCfg {
 // grid = ceil(N / 128) * S CTAs in clusters of S along x: CTA b works feature tile b / S, k split b % S.
 // tmW: Wq [N, K bytes] box [128 x 128]; tmA: Aq [M, K bytes] box [ntok x 128]; As / Ws: tiled scales.
 // ESETS: sets of four epilogue warps (threads = 64 + 128 ESETS): one set and two CTAs per SM up to 64 tokens;
-// two sets at 128 tokens, where a CTA fills an SM by itself and has some forty tokens to add up and store.
-template <int FMT = FMT_MXFP4, int ESETS = 1>
+// two sets above, where a CTA fills an SM by itself and has some forty tokens to add up and store.
+template <int FMT = FMT_MXFP4, int ESETS = 1, bool PUSH = false>
 __global__ void __launch_bounds__(64 + 128 * ESETS, ESETS == 1 ? 2 : 1)
 gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmA,
                    const uint8_t* __restrict__ As, const uint8_t* __restrict__ Ws, void* __restrict__ Y,
@@ -75,9 +80,10 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (C::STAGES + s); };
   const uint32_t accf_bar = bar_base + 8u * (2 * C::STAGES);
+  const uint32_t ready_bar = accf_bar + 8;               // PUSH: the owners' stages are free to be written
+  const uint32_t recv_bar = accf_bar + 16;               // PUSH: all partials of this CTA's pieces are here
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + bar_off + 192);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(smem_gen + bar_off + 200);
-  float* P = reinterpret_cast<float*>(smem_gen);         // after the mainloop: partial tile [token][feature]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = blockIdx.x % S, nt = blockIdx.x / S;
@@ -85,6 +91,8 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   const int kb4 = K / (C::BK / CH);                      // scale chunks per row
   const int kt0 = (int)((long long)k_tiles * rank / S), kt1 = (int)((long long)k_tiles * (rank + 1) / S);
   const uint32_t tmem_cols = C::tmem_cols(ntok);
+  const int pieces = (M + 3) / 4;                        // of four tokens; piece c belongs to CTA c % S
+  const int owners = pieces < S ? pieces : S;
 
   // The weights and their scales are constants of the layer, never the output of the kernel that runs
   // just before this one: the thread that initialises the barriers sends their loads for the first
@@ -95,6 +103,7 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   if (threadIdx.x == 0) {
     for (int s = 0; s < nst; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     mbar_init(accf_bar, 1);
+    if constexpr (PUSH) { mbar_init(ready_bar, (uint32_t)owners); mbar_init(recv_bar, 1); }
     *cta_abort = 0;
     fence_mbar_init();
     fence_proxy_async_smem();                            // the copy engine sees the initialised barriers
@@ -107,10 +116,12 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
                    512u * (uint32_t)min(CH, kb4 - CH * kt), full_bar(it));
     }
     tma_prefetch_desc(&tmA);
+    if (PUSH && S > 1 && rank < owners) mbar_arrive_expect_tx(recv_bar, (uint32_t)((pieces - rank + S - 1) / S * S * C::PIECE_BYTES));
   }
   if (warp == 1) { tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), tmem_cols); tmem_relinquish(); }
   tc_fence_before_sync();
   __syncthreads();
+  if (PUSH && S > 1) cluster_arrive_relaxed();           // the wait stands before the first access to another CTA
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   griddep_launch_dependents();
@@ -193,92 +204,167 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     // ------------------------------------------------------------------ epilogue (warps 2..5)
     // Two passes over the SAME instructions, as in the few-token rotation: pass 0 is a dry run while the
     // mainloop streams (reads this CTA's own shared memory, stores nothing) so that the reduction's code is
-    // in the instruction cache when it is needed; pass 1: accumulator -> own shared memory, cluster
-    // barrier, then the tokens of this CTA.
-    // A warp takes one token per pass: lane l adds features 4 l .. 4 l + 3 (16-byte loads, 512 contiguous
-    // bytes per warp and partial) and stores 8 or 16 bytes of the token's row of Y.  Two tokens per
-    // iteration, all their loads issued before the first add: few round trips through the cluster.
+    // in the instruction cache when it is needed; pass 1: accumulator -> partials, then the tokens of this CTA.
     const int q = warp & 3;
     const int ew = warp - 2;                             // 0 .. 4 ESETS - 1
-    constexpr int NW = 4 * ESETS;
-    const int64_t n = (int64_t)nt * C::BF + 4 * lane;
-    const uint32_t p_saddr = smem_u32(P);
-#pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-      const bool live = pass == 1;
-      if (live) {
-        // ---- epilogue 1: partial tile -> own shared memory
-        acc_ok = mbar_wait(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
-        acc_ok = __all_sync(0xFFFFFFFFu, acc_ok);
-        if (acc_ok) {
-          tc_fence_after_sync();
-          const uint32_t tacc = tmem_base + ((uint32_t)(q * 32) << 16);
-          float* prow = P + q * 32 + lane;               // feature 32 q + lane of token 0
-          for (int c0 = 16 * (ew >> 2); c0 < ntok; c0 += 16 * ESETS) {
-            uint32_t v[16];
-            tmem_ld_32x32_x16(tacc + c0, v);
-            tmem_ld_wait();
+    const int feature = q * 32 + lane;                   // of this lane in tensor memory
+    const uint32_t tacc = tmem_base + ((uint32_t)(q * 32) << 16);
+    if (S == 1) {                                        // nothing to add: accumulator -> Y
+      acc_ok = mbar_wait(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
+      acc_ok = __all_sync(0xFFFFFFFFu, acc_ok);
+      tc_fence_after_sync();
+      const int64_t n = (int64_t)nt * C::BF + feature;
+      for (int c0 = 16 * (ew >> 2); acc_ok && c0 < M; c0 += 16 * ESETS) {
+        uint32_t v[16];
+        tmem_ld_32x32_x16(tacc + c0, v);
+        tmem_ld_wait();
 #pragma unroll
-            for (int j = 0; j < 16; ++j) prow[(c0 + j) * C::BF] = __uint_as_float(v[j]);
+        for (int j = 0; j < 16; ++j) {
+          float y = __uint_as_float(v[j]);
+          if constexpr (FMT == FMT_NVFP4) y *= alpha;
+          if (c0 + j < M && n < N) {
+            if (y_is_bf16) reinterpret_cast<__nv_bfloat16*>(Y)[(int64_t)(c0 + j) * N + n] = __float2bfloat16_rn(y);
+            else reinterpret_cast<float*>(Y)[(int64_t)(c0 + j) * N + n] = y;
           }
         }
-        tc_fence_before_sync();
-        cluster_sync_all();                              // every CTA's partial tile is visible cluster-wide
       }
-      // ---- epilogue 2: add the partials, store Y
-      uint32_t p_rank[C::MAX_CLUSTER];
+    } else if constexpr (PUSH) {
+      // Lane l of warp q has feature 32 q + l of the tile: one 16-byte load per partial gives its four tokens.
+      const int64_t n = (int64_t)nt * C::BF + feature;
+#pragma unroll 1
+      for (int pass = 0; pass < 2; ++pass) {
+        const bool live = pass == 1;
+        if (live) {
+          acc_ok = mbar_wait(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
+          // every load into the stages has landed and every instruction that read them has completed
+          acc_ok = __all_sync(0xFFFFFFFFu, acc_ok);
+          cluster_wait();
+          if (!acc_ok) break;
+          if (rank < owners && warp == 2 && lane < S) mbar_arrive_cluster(map_to_cta(ready_bar, (uint32_t)lane));
+          bool ok = mbar_wait_cluster(ready_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
+          if (!__all_sync(0xFFFFFFFFu, ok)) break;
+          tc_fence_after_sync();
+          uint32_t v[16];
+          tmem_ld_32x32_x16(tacc, v);
+          tmem_ld_wait();
 #pragma unroll
-      for (int s = 0; s < C::MAX_CLUSTER; ++s)
-        p_rank[s] = s < S ? map_to_cta(p_saddr, live ? (uint32_t)s : (uint32_t)rank) : 0u;
-      for (int m0 = rank + S * ew; m0 < M; m0 += 2 * NW * S) {
-        float4 part[2][C::MAX_CLUSTER];
+          for (int c = 0; c < 4; ++c)
+            if (c < pieces)
+              st_async_v4(map_to_cta(smem_base, (uint32_t)(c % S)) + (uint32_t)(((c / S) * S + rank) * C::PIECE_BYTES + feature * 16),
+                          v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3], map_to_cta(recv_bar, (uint32_t)(c % S)));
+          if (rank >= owners) break;                     // nothing to receive
+          ok = mbar_wait_cluster(recv_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
+          if (!__all_sync(0xFFFFFFFFu, ok)) break;
+        }
+        for (int ci = 0; rank + ci * S < pieces; ++ci) {
+          const int m0 = 4 * (rank + ci * S);
+          float4 part[C::MAX_CLUSTER];
+          const uint32_t src = smem_base + (uint32_t)(ci * S * C::PIECE_BYTES + feature * 16);
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int m = m0 + NW * S * j;
-          if (m < M) {
-            const uint32_t off = (uint32_t)((m * C::BF + 4 * lane) * 4);
+          for (int s = 0; s < C::MAX_CLUSTER; ++s)
+            if (s < S)
+              asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                           : "=f"(part[s].x), "=f"(part[s].y), "=f"(part[s].z), "=f"(part[s].w) : "r"(src + (uint32_t)(s * C::PIECE_BYTES)));
+          float y[4] = {0.f, 0.f, 0.f, 0.f};             // rank order: the result does not depend on timing
 #pragma unroll
-            for (int s = 0; s < C::MAX_CLUSTER; ++s)
-              if (s < S)
-                asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                             : "=f"(part[j][s].x), "=f"(part[j][s].y), "=f"(part[j][s].z), "=f"(part[j][s].w)
-                             : "r"(p_rank[s] + off));
+          for (int s = 0; s < C::MAX_CLUSTER; ++s)
+            if (s < S) { y[0] += part[s].x; y[1] += part[s].y; y[2] += part[s].z; y[3] += part[s].w; }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if constexpr (FMT == FMT_NVFP4) y[j] *= alpha;
+            if (live && m0 + j < M && n < N) {
+              if (y_is_bf16) reinterpret_cast<__nv_bfloat16*>(Y)[(int64_t)(m0 + j) * N + n] = __float2bfloat16_rn(y[j]);
+              else reinterpret_cast<float*>(Y)[(int64_t)(m0 + j) * N + n] = y[j];
+            }
           }
         }
+      }
+    } else {
+      // A warp takes one token per pass: lane l adds features 4 l .. 4 l + 3 (16-byte loads, 512 contiguous
+      // bytes per warp and partial) and stores 8 or 16 bytes of the token's row of Y.  Two tokens per
+      // iteration, all their loads issued before the first add: few round trips through the cluster.
+      constexpr int NW = 4 * ESETS;
+      const int64_t n = (int64_t)nt * C::BF + 4 * lane;
+      const uint32_t p_saddr = smem_base;
+#pragma unroll 1
+      for (int pass = 0; pass < 2; ++pass) {
+        const bool live = pass == 1;
+        if (live) {
+          // ---- epilogue 1: partial tile -> own shared memory
+          acc_ok = mbar_wait(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
+          acc_ok = __all_sync(0xFFFFFFFFu, acc_ok);
+          if (acc_ok) {
+            tc_fence_after_sync();
+            float* prow = reinterpret_cast<float*>(smem_gen) + feature;     // partial tile [token][feature]
+            for (int c0 = 16 * (ew >> 2); c0 < ntok; c0 += 16 * ESETS) {
+              uint32_t v[16];
+              tmem_ld_32x32_x16(tacc + c0, v);
+              tmem_ld_wait();
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int m = m0 + NW * S * j;
-          if (m < M) {
-            float4 y = make_float4(0.f, 0.f, 0.f, 0.f);  // rank order: the result does not depend on timing
+              for (int j = 0; j < 16; ++j) prow[(c0 + j) * C::BF] = __uint_as_float(v[j]);
+            }
+          }
+          tc_fence_before_sync();
+          cluster_sync_all();                              // every CTA's partial tile is visible cluster-wide
+        }
+        // ---- epilogue 2: add the partials, store Y
+        uint32_t p_rank[C::MAX_CLUSTER];
 #pragma unroll
-            for (int s = 0; s < C::MAX_CLUSTER; ++s)
-              if (s < S) { y.x += part[j][s].x; y.y += part[j][s].y; y.z += part[j][s].z; y.w += part[j][s].w; }
-            if constexpr (FMT == FMT_NVFP4) { y.x *= alpha; y.y *= alpha; y.z *= alpha; y.w *= alpha; }
-            if (live && n < N) {                         // N % 8 == 0: four features are inside or outside together
-              if (y_is_bf16) {
-                __nv_bfloat162 h0 = __floats2bfloat162_rn(y.x, y.y), h1 = __floats2bfloat162_rn(y.z, y.w);
-                *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(Y) + (int64_t)m * N + n) =
-                    make_uint2(*reinterpret_cast<uint32_t*>(&h0), *reinterpret_cast<uint32_t*>(&h1));
-              } else {
-                *reinterpret_cast<float4*>(reinterpret_cast<float*>(Y) + (int64_t)m * N + n) = y;
+        for (int s = 0; s < C::MAX_CLUSTER; ++s)
+          p_rank[s] = s < S ? map_to_cta(p_saddr, live ? (uint32_t)s : (uint32_t)rank) : 0u;
+        for (int m0 = rank + S * ew; m0 < M; m0 += 2 * NW * S) {
+          float4 part[2][C::MAX_CLUSTER];
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const int m = m0 + NW * S * j;
+            if (m < M) {
+              const uint32_t off = (uint32_t)((m * C::BF + 4 * lane) * 4);
+#pragma unroll
+              for (int s = 0; s < C::MAX_CLUSTER; ++s)
+                if (s < S)
+                  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                               : "=f"(part[j][s].x), "=f"(part[j][s].y), "=f"(part[j][s].z), "=f"(part[j][s].w)
+                               : "r"(p_rank[s] + off));
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const int m = m0 + NW * S * j;
+            if (m < M) {
+              float4 y = make_float4(0.f, 0.f, 0.f, 0.f);  // rank order: the result does not depend on timing
+#pragma unroll
+              for (int s = 0; s < C::MAX_CLUSTER; ++s)
+                if (s < S) { y.x += part[j][s].x; y.y += part[j][s].y; y.z += part[j][s].z; y.w += part[j][s].w; }
+              if constexpr (FMT == FMT_NVFP4) { y.x *= alpha; y.y *= alpha; y.z *= alpha; y.w *= alpha; }
+              if (live && n < N) {                         // N % 8 == 0: four features are inside or outside together
+                if (y_is_bf16) {
+                  __nv_bfloat162 h0 = __floats2bfloat162_rn(y.x, y.y), h1 = __floats2bfloat162_rn(y.z, y.w);
+                  *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(Y) + (int64_t)m * N + n) =
+                      make_uint2(*reinterpret_cast<uint32_t*>(&h0), *reinterpret_cast<uint32_t*>(&h1));
+                } else {
+                  *reinterpret_cast<float4*>(reinterpret_cast<float*>(Y) + (int64_t)m * N + n) = y;
+                }
               }
             }
           }
         }
       }
     }
-  }
-  if (warp < 2) {                                        // the epilogue warps passed this barrier inside their pass 1
     tc_fence_before_sync();
-    cluster_sync_all();
+  }
+  if (S > 1) {
+    if (PUSH) {
+      if (warp < 2) cluster_wait();                      // the epilogue warps have waited above
+    } else {
+      if (warp < 2) { tc_fence_before_sync(); cluster_sync_all(); }        // as the epilogue warps in their pass 1
+      cluster_arrive_relaxed();                          // every partial that this warp asked for has come: its sums are out
+      cluster_wait();                                    // no CTA of the cluster reads this one's partial tile any more
+    }
   }
 
   // ------------------------------------------------------------------ teardown
   __syncthreads();
-  if (*cta_abort) {
-    for (int i = 0; i < 2000; ++i) __nanosleep(1000);
-  }
-  cluster_sync_all();                                    // no CTA of the cluster reads this one's partial tile any more
+  if (PUSH && S > 1 && *cta_abort) cluster_sync_all();   // others may still push to this CTA, see the few-token rotation
   if (warp == 1) {
     tc_fence_after_sync();
     tmem_dealloc(tmem_base, tmem_cols);

@@ -2,28 +2,38 @@
 // (Algorithm 3 steps 2-4).  One kernel, no scratch in global memory.
 //
 // Swapped operands: the tensor-core instruction's 128 rows are 128 output FEATURES (four 32-blocks)
-// and its N columns are the tokens (16 ... 256), so no row of the instruction is padding and the
+// and its N columns are the tokens (16 ... 256, in steps of 16), so no row of the instruction is padding and the
 // accumulator is small:  D[j, m] = sum_i R_inter[i, j] X[m, i].
 //   A = R_inter tile [64 (i) x 128 (j)], features contiguous = MN-major, two 64 x 64 boxes (128-B swizzle)
 //   B = X tile [tokens x 64 (i)], K-major
 // A layer has only d / 128 feature tiles (40 at d = 5120), too few CTAs to pull R_inter at HBM rate,
 // so the contraction is also split: a CLUSTER of S CTAs shares one feature tile, CTA r of the cluster
-// contracts k range r.  The fp32 partial tiles never leave the SMs: every CTA writes its partial
-// [token][feature] into its own shared memory, a cluster barrier publishes them, and each warp of
-// the cluster then owns some (16 tokens x one 32-block) units: it adds the S partials of its unit in
-// rank order through distributed shared memory (plain ld.shared::cluster; fixed order, so the result
-// does not depend on timing), applies the intra-block rotation on the warp-level tensor cores (y split
-// into three bf16 terms, fp32 accumulation) and quantizes (Eq. 1).
+// contracts k range r.  The fp32 partial tiles never leave the SMs: token group g (16 tokens) belongs to CTA g % S
+// (its owner), which adds the S partials in rank order (fixed order, so the result does not depend on timing), applies
+// the intra-block rotation on the warp-level tensor cores (y split into three bf16 terms, fp32 accumulation) and
+// quantizes (Eq. 1).  The partials reach the owner in one of two ways:
+//  * PUSH (up to 16 tokens, one group): every CTA stores its partial straight from registers into the owner's shared
+//    memory (st.async, 16 bytes per lane, counted on a barrier of the owner).  They go where the owner's stages
+//    were, so the owner first says, on a barrier of each CTA, that its own mainloop has left them.  No
+//    cluster-wide barrier stands on the path, nor at the end: the owner has waited for all that it receives, and the
+//    other CTAs leave right after their stores, which lets the CTAs of the next kernel in.  Bound by the one owner's
+//    chain of latencies (d = 5120, M = 1: stores 0.5 us, unit 1 us where pulling took 0.8 + 1.8 + 0.7 us for barrier, unit
+//    and second barrier; rotation 12.1 -> 10.9 us).  The stores arrive at about 11 B per cycle: with 64 tokens
+//    the same way took 15.3 us, pulling 13.7.
+//  * pull (more tokens): every CTA writes its partial [token][feature] into its own shared memory, a cluster barrier
+//    publishes them, and the owner reads them with 16-byte ld.shared::cluster.  A second barrier, at which a warp arrives
+//    as soon as its last such load is back and for which it waits only before it exits, keeps the partials in place
+//    (one full barrier at the end: d = 5120, M = 64 14.0 -> 13.7 us, GEMM 6.7 -> 6.1).
+// With S = 1 (an ordinary launch without clusters) a warp writes its features into its own shared memory and goes on.
 //
-// Units: epilogue warp w of every CTA owns 32-block w of the tile (its R_intra block is fetched into
+// Units: the epilogue warps of lane quarter q of every CTA own 32-block q of the tile (its R_intra block is fetched into
 // shared memory when the kernel starts, long before it is needed: a first touch of that array from a
-// cold TLB costs microseconds); CTA r of the cluster takes the token groups r, r + S, ...
+// cold TLB costs microseconds).
 //
 // Roles per CTA: warp 0 TMA producer, warp 1 MMA issuer, warps 2..5 epilogue / reduction.
 // Shared memory: 4 stages of (16 KiB of R_inter + tokens x 128 B of X); after the mainloop the same
-// memory holds the partial tile and the per-warp staging of the reduction.  Up to 64 tokens that is small
-// enough (<= 107 KiB) for two CTAs per SM: the grid may exceed the SM count, which keeps more loads in
-// flight; with 128 or 256 tokens one CTA fills an SM and the grid stays within the SM count.
+// memory holds the partials.  Up to 64 tokens that is small enough (<= 107 KiB) for two CTAs per SM: the
+// grid may exceed the SM count, which keeps more loads in flight; above, one CTA fills an SM.
 #pragma once
 #include <cuda_bf16.h>
 #include "intra_fragment.cuh"
@@ -40,8 +50,10 @@ struct RotFewCfg {
   // the same for every token count: three stages at 128 tokens would let two CTAs share an SM (clusters of 5
   // instead of 3), which measured 4 - 10 % slower than four stages and one CTA per SM
   __host__ __device__ static constexpr int stages(int) { return STAGES; }
-  static constexpr int MAX_TOK = 256;                  // N of the instruction; 16, 32, 64, 128 or 256 are used
-  static constexpr int Y_BYTES = 16 * 33 * 4;          // per epilogue warp: 16 tokens x 32 features, row stride 33
+  static constexpr int MAX_TOK = 256;                  // N of the instruction: a multiple of 16
+  static constexpr int MAX_PUSH_TOK = 16;              // one token group
+  static constexpr int PART_BYTES = BF * 16 * 4;       // pushed partial of the group from one CTA: [4][feature][4 tokens]
+  static constexpr int Y_BYTES = 16 * 33 * 4;          // pull, per epilogue warp: 16 tokens x 32 features, row stride 33
   static constexpr int RI_BYTES = 32 * 80;             // per epilogue warp: R_intra[block] as bf16 rows of 80 bytes
   static constexpr int BAR_BYTES = 256;
   static constexpr int THREADS = 192;
@@ -50,25 +62,20 @@ struct RotFewCfg {
   __host__ __device__ static constexpr int smem_bytes(int ntok) {
     return stages(ntok) * stage_bytes(ntok) + BAR_BYTES + 4 * RI_BYTES + 1024;
   }
-  // the partial tile (ntok x 512 B) and the warps' y tiles must fit inside the stages they reuse
-  __host__ __device__ static constexpr bool reduction_fits(int ntok) {
-    return ntok * BF * 4 + 8 * Y_BYTES <= stages(ntok) * stage_bytes(ntok);   // up to eight epilogue warps
-  }
   __host__ __device__ static constexpr int ctas_per_sm(int ntok) { return smem_bytes(ntok) <= 113 * 1024 ? 2 : 1; }
-  __host__ __device__ static constexpr int max_smem_bytes() {                  // over the token counts in use
-    return smem_bytes(256) > smem_bytes(64) ? smem_bytes(256) : smem_bytes(64);
-  }
+  __host__ __device__ static constexpr int max_smem_bytes() { return smem_bytes(MAX_TOK); }
 };
-static_assert(RotFewCfg::reduction_fits(16) && RotFewCfg::reduction_fits(32) && RotFewCfg::reduction_fits(64) &&
-              RotFewCfg::reduction_fits(128) && RotFewCfg::reduction_fits(256), "reduction buffers");
+// what lies in the stages after the mainloop: S pushed partials, or the partial tile (ntok x 512 B) and the y tiles
+static_assert(RotFewCfg::MAX_CLUSTER * RotFewCfg::PART_BYTES <= RotFewCfg::STAGES * RotFewCfg::stage_bytes(16) &&
+              8 * RotFewCfg::Y_BYTES <= 4 * RotFewCfg::A_BYTES && RotFewCfg::BF * 4 <= RotFewCfg::STAGES * RotFewCfg::BK * 2, "reduction buffers");
 
 // grid = (d / 128) * S CTAs in clusters of S along x: CTA b works feature tile b / S, k split b % S.
-// tmX: X [M, d] bf16, box [ntok rows x 64]; tmR: R_inter [d, d] bf16, box [64 x 64].  ntok = 16, 32, 64, 128 or 256
-// >= M.  d % 128 == 0.  `codes` / `scales` / `tensor_scale` as in rotate_quantize_kernel for FMT.
+// tmX: X [M, d] bf16, box [ntok rows x 64]; tmR: R_inter [d, d] bf16, box [64 x 64].  ntok = M rounded up to
+// a multiple of 16.  d % 128 == 0.  `codes` / `scales` / `tensor_scale` as in rotate_quantize_kernel for FMT.
 // ESETS: sets of four epilogue warps (threads = 64 + 128 ESETS).  One set and two CTAs per SM up to 64
-// tokens; with 128 or 256 tokens a CTA fills an SM by itself and has several token groups to reduce, rotate
+// tokens; with more a CTA fills an SM by itself and has several token groups to reduce, rotate
 // and quantize, each a dependent chain of about a microsecond for one warp: two sets take them in turn.
-template <int FMT = FMT_MXFP4, int ESETS = 1>
+template <int FMT = FMT_MXFP4, int ESETS = 1, bool PUSH = false>
 __global__ void __launch_bounds__(64 + 128 * ESETS, ESETS == 1 ? 2 : 1)
 rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,
                      const __nv_bfloat16* __restrict__ R_intra, uint8_t* __restrict__ codes,
@@ -85,18 +92,18 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (C::STAGES + s); };
   const uint32_t accf_bar = bar_base + 8u * (2 * C::STAGES);
+  const uint32_t ready_bar = accf_bar + 8;               // PUSH: the owner's stages are free to be written
+  const uint32_t recv_bar = accf_bar + 16;               // PUSH, in the owner: all partials are here
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + bar_off + 192);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(smem_gen + bar_off + 200);
-  // after the mainloop: partial tile P[token][feature] fp32 at offset 0, then the warps' y tiles
-  float* P = reinterpret_cast<float*>(smem_gen);
-  uint8_t* y_tiles = smem_gen + ntok * C::BF * 4;
   uint8_t* ri_tiles = smem_gen + bar_off + C::BAR_BYTES;    // not part of the stages: filled at kernel start
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = blockIdx.x % S, ft = blockIdx.x / S;
   const int k_tiles = d / C::BK;
   const int kt0 = (int)((long long)k_tiles * rank / S), kt1 = (int)((long long)k_tiles * (rank + 1) / S);
-  const uint32_t tmem_cols = ntok < 32 ? 32u : (uint32_t)ntok;
+  const uint32_t tmem_cols = ntok <= 32 ? 32u : (ntok <= 64 ? 64u : (ntok <= 128 ? 128u : 256u));
+  const int groups = (M + 15) / 16;                      // token groups; group g belongs to CTA g % S
 
   // R_inter is a constant of the layer, never the output of the kernel that runs just before this
   // one: the thread that initialises the barriers sends the loads of the first stages' R_inter tiles
@@ -106,6 +113,7 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   if (threadIdx.x == 0) {
     for (int s = 0; s < nst; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     mbar_init(accf_bar, 1);
+    if constexpr (PUSH) { mbar_init(ready_bar, 1); mbar_init(recv_bar, 1); }
     *cta_abort = 0;
     fence_mbar_init();
     fence_proxy_async_smem();                            // the copy engine sees the initialised barriers
@@ -116,18 +124,19 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
       tma_load_2d(st + C::A_BOX_BYTES, &tmR, ft * C::BF + 64, (kt0 + it) * C::BK, full_bar(it));
     }
     tma_prefetch_desc(&tmX);
+    if (PUSH && S > 1 && rank == 0) mbar_arrive_expect_tx(recv_bar, (uint32_t)((M + 3) / 4 * S * C::BF * 16));
   }
   if (warp == 1) { tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), tmem_cols); tmem_relinquish(); }
   tc_fence_before_sync();
   __syncthreads();
+  if (PUSH && S > 1) cluster_arrive_relaxed();           // the wait stands before the first access to another CTA
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   griddep_launch_dependents();
-  const int groups = ntok / 16;                          // token groups of 16; group g belongs to CTA g % S
   if (warp >= 2 && warp < 6 && R_intra != nullptr && rank < groups) {
     // this warp's R_intra block (a constant of the layer as well), 128 pieces of 16 B: row piece / 4
-    uint8_t* r_s = ri_tiles + (warp - 2) * C::RI_BYTES;
-    const uint4* src = reinterpret_cast<const uint4*>(R_intra + (size_t)(ft * 4 + (warp - 2)) * 1024);
+    uint8_t* r_s = ri_tiles + (warp & 3) * C::RI_BYTES;
+    const uint4* src = reinterpret_cast<const uint4*>(R_intra + (size_t)(ft * 4 + (warp & 3)) * 1024);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int piece = lane + 32 * i;
@@ -189,104 +198,191 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
     // this CTA's own shared memory (whatever it holds), computes, and stores nothing.  Its only purpose
     // is to have the reduction's code in the instruction cache: executed cold, after the mainloop,
     // that code cost about 2.5 us of instruction fetches -- a fifth of the kernel.  Pass 1 is the
-    // real one: accumulator -> own shared memory, cluster barrier, then the units of this warp.
-    const int q = warp & 3;
-    const int ew = (warp - 2) & 3;                       // 0..3 = 32-block of the tile
+    // real one: accumulator -> partials, then the units of this warp.
+    const int q = warp & 3;                              // lane quarter = 32-block of the tile
     const int es = (warp - 2) >> 2;                      // set of epilogue warps
+    const int p = lane & 3, r8 = lane >> 2;
     const int nblocks = d / 32;
-    const int blk = ft * 4 + ew;
-    float* y_s = reinterpret_cast<float*>(y_tiles + (es * 4 + ew) * C::Y_BYTES);
-    const uint32_t r_saddr = smem_u32(ri_tiles + ew * C::RI_BYTES);
-    const uint32_t p_saddr = smem_u32(P);
-    // lane l adds tokens (l / 8) + 4 j, j = 0..3, features 4 (l % 8) .. + 3 of the block, two tokens at a
-    // time: their 2 S loads of 16 bytes go out before the first add, so a unit costs two round trips
-    // through the cluster
-    const int tr = lane >> 3, fc = (lane & 7) * 4;
-#pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-      const bool live = pass == 1;
-      if (live) {
-        // ---- epilogue 1: partial tile -> own shared memory
-        acc_ok = mbar_wait(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
-        acc_ok = __all_sync(0xFFFFFFFFu, acc_ok);
-        if (acc_ok) {
-          tc_fence_after_sync();
-          // every load into the stages has landed and every instruction that read them has completed
-          const uint32_t tacc = tmem_base + ((uint32_t)(q * 32) << 16);
-          float* prow = P + q * 32 + lane;               // feature 32 q + lane of token 0
-          for (int c0 = 16 * es; c0 < ntok; c0 += 16 * ESETS) {
-            uint32_t v[16];
-            tmem_ld_32x32_x16(tacc + c0, v);
-            tmem_ld_wait();
+    const int blk = ft * 4 + q;
+    const int kb4 = FMT == FMT_NVFP4 ? (2 * nblocks + 3) / 4 : (nblocks + 3) / 4;
+    const uint32_t r_saddr = smem_u32(ri_tiles + q * C::RI_BYTES);
+    const uint32_t r_lane = r_saddr + (uint32_t)(((lane >> 3) & 1) * 8 + (lane & 7)) * 80 + (uint32_t)(lane >> 4) * 16;
+    const int feature = q * 32 + lane;                   // of this lane in tensor memory
+    NvScale nvs = {};
+    if constexpr (FMT == FMT_NVFP4) nvs = nv_scale(tensor_scale);
+    // rotate inside the block, quantize, store: y in the fragment layout (rows = tokens of group g, columns = features)
+    auto finish = [&](const uint32_t (&y)[16], int g, bool live) {
+      IntraFrag f;
+      if (R_intra != nullptr) load_intra_frag(r_lane, r_lane + 32, 16 * 80, f);
+      uint32_t sb[2];
+      intra_quantize_frag16<FMT, true>(y, R_intra != nullptr, f, lane, 16 * g, live ? M : 0, blk, nblocks, d, nvs, codes, sb);
+      if (p == 0 && live) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) prow[(c0 + j) * C::BF] = __uint_as_float(v[j]);
-          }
+        for (int rh = 0; rh < 2; ++rh) {                 // rows of the group past the last token: zero
+          const int row = 16 * g + r8 + 8 * rh;
+          const uint32_t b = row < M ? sb[rh] : 0u;
+          if constexpr (FMT == FMT_NVFP4) *reinterpret_cast<uint16_t*>(scales + scale_offset(row, 2 * blk, kb4)) = (uint16_t)b;
+          else scales[scale_offset(row, blk, kb4)] = (uint8_t)b;
         }
-        tc_fence_before_sync();
-        cluster_sync_all();                              // every CTA's partial tile is visible cluster-wide
       }
-      // ---- epilogue 2: reduce, intra-rotate, quantize
-      uint32_t p_rank[C::MAX_CLUSTER];
-#pragma unroll
-      for (int s = 0; s < C::MAX_CLUSTER; ++s)
-        p_rank[s] = s < S ? map_to_cta(p_saddr, live ? (uint32_t)s : (uint32_t)rank) : 0u;
-      for (int g = rank + es * S; g < groups; g += S * ESETS) {
-#pragma unroll
-        for (int jh = 0; jh < 2; ++jh) {
-          if (16 * g + 8 * jh >= M) break;               // rows 8 jh .. 8 jh + 7 of the group hold no token
-          float4 part[2][C::MAX_CLUSTER];
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const uint32_t off = (uint32_t)(((16 * g + tr + 4 * (2 * jh + j)) * C::BF + ew * 32 + fc) * 4);
-#pragma unroll
-            for (int s = 0; s < C::MAX_CLUSTER; ++s)
-              if (s < S)
-                asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                             : "=f"(part[j][s].x), "=f"(part[j][s].y), "=f"(part[j][s].z), "=f"(part[j][s].w)
-                             : "r"(p_rank[s] + off));
+    };
+    const uint32_t tacc = tmem_base + ((uint32_t)(q * 32) << 16);
+    if constexpr (PUSH) {
+      const uint32_t my_part = (uint32_t)rank * C::PART_BYTES + (uint32_t)feature * 16;
+#pragma unroll 1
+      for (int pass = rank == 0 ? 0 : 1; pass < 2; ++pass) {
+        const bool live = pass == 1;
+        if (live) {
+          acc_ok = mbar_wait(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
+          // every load into the stages has landed and every instruction that read them has completed
+          acc_ok = __all_sync(0xFFFFFFFFu, acc_ok);
+          bool ok = acc_ok;
+          if (S > 1) {
+            cluster_wait();
+            if (rank == 0 && ok && warp == 2 && lane < S) mbar_arrive_cluster(map_to_cta(ready_bar, (uint32_t)lane));
+            if (ok) ok = mbar_wait_cluster(ready_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
+            ok = __all_sync(0xFFFFFFFFu, ok);
           }
+          if (!ok) break;
+          tc_fence_after_sync();
+          uint32_t v[16];
+          tmem_ld_32x32_x16(tacc, v);
+          tmem_ld_wait();
+          const uint32_t dst = map_to_cta(smem_base, 0) + my_part, bar = map_to_cta(recv_bar, 0);
 #pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            float4 y = make_float4(0.f, 0.f, 0.f, 0.f);  // rank order: the result does not depend on timing
+          for (int c = 0; c < 4; ++c)                    // piece c: four tokens
+            if (S == 1)
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(smem_base + my_part + (uint32_t)(c * C::BF * 16)),
+                           "r"(v[4 * c]), "r"(v[4 * c + 1]), "r"(v[4 * c + 2]), "r"(v[4 * c + 3]) : "memory");
+            else if (4 * c < M)
+              st_async_v4(dst + (uint32_t)(c * C::BF * 16), v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3], bar);
+          if (rank != 0) break;                          // not the owner
+          if (S > 1) ok = __all_sync(0xFFFFFFFFu, mbar_wait_cluster(recv_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL));
+          if (!ok) break;
+          __syncwarp();
+        }
+        float sum[16];
 #pragma unroll
-            for (int s = 0; s < C::MAX_CLUSTER; ++s)
-              if (s < S) { y.x += part[j][s].x; y.y += part[j][s].y; y.z += part[j][s].z; y.w += part[j][s].w; }
-            if (live) {                                  // the y tile lies inside the stages: untouched while they are in use
-              float* dst = y_s + (tr + 4 * (2 * jh + j)) * 33 + fc;
-              dst[0] = y.x; dst[1] = y.y; dst[2] = y.z; dst[3] = y.w;
+        for (int i = 0; i < 16; ++i) sum[i] = 0.f;
+        const uint32_t part0 = smem_base + (uint32_t)(r8 & 3) * 4;
+        for (int s = 0; s < S; ++s) {                    // rank order: the result does not depend on timing
+#pragma unroll
+          for (int n = 0; n < 4; ++n)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int col = q * 32 + 8 * n + 2 * p + (i & 1);
+              float v;
+              asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v)
+                           : "r"(part0 + (uint32_t)(s * C::PART_BYTES + (((r8 >> 2) + 2 * (i >> 1)) * C::BF + col) * 16)));
+              sum[4 * n + i] += v;
+            }
+        }
+        uint32_t y[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) y[i] = __float_as_uint(sum[i]);
+        finish(y, 0, live);
+      }
+    } else {
+      float* y_s = reinterpret_cast<float*>(smem_gen + ntok * C::BF * 4 + (es * 4 + q) * C::Y_BYTES);
+      const uint32_t p_saddr = smem_base;
+      // lane l adds tokens (l / 8) + 4 j, j = 0..3, features 4 (l % 8) .. + 3 of the block, two tokens at a
+      // time: their 2 S loads of 16 bytes go out before the first add, so a unit costs two round trips
+      // through the cluster
+      const int tr = lane >> 3, fc = (lane & 7) * 4;
+#pragma unroll 1
+      for (int pass = 0; pass < 2; ++pass) {
+        const bool live = pass == 1;
+        if (live) {
+          acc_ok = mbar_wait(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
+          acc_ok = __all_sync(0xFFFFFFFFu, acc_ok);
+          if (acc_ok) {
+            tc_fence_after_sync();
+            float* prow = reinterpret_cast<float*>(smem_gen) + feature;     // partial tile [token][feature]
+            for (int c0 = 16 * es; c0 < ntok; c0 += 16 * ESETS) {
+              uint32_t v[16];
+              tmem_ld_32x32_x16(tacc + c0, v);
+              tmem_ld_wait();
+#pragma unroll
+              for (int j = 0; j < 16; ++j) prow[(c0 + j) * C::BF] = __uint_as_float(v[j]);
             }
           }
+          tc_fence_before_sync();
+          cluster_sync_all();                            // every CTA's partial tile is visible cluster-wide
         }
-        __syncwarp();
-        intra_quantize_rows16<FMT>(y_s, r_saddr, R_intra != nullptr, lane, 16 * g, M, blk, d, nblocks, tensor_scale,
-                                   codes, scales, live);
-        __syncwarp();
+        uint32_t p_rank[C::MAX_CLUSTER];
+#pragma unroll
+        for (int s = 0; s < C::MAX_CLUSTER; ++s)
+          p_rank[s] = s < S ? map_to_cta(p_saddr, live ? (uint32_t)s : (uint32_t)rank) : 0u;
+        int g = rank + es * S;
+        if (live && g >= groups) cluster_arrive_relaxed();      // nothing to read
+        for (; g < groups; g += S * ESETS) {
+#pragma unroll
+          for (int jh = 0; jh < 2; ++jh) {
+            if (16 * g + 8 * jh >= M) break;             // rows 8 jh .. 8 jh + 7 of the group hold no token
+            float4 part[2][C::MAX_CLUSTER];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+              const uint32_t off = (uint32_t)(((16 * g + tr + 4 * (2 * jh + j)) * C::BF + q * 32 + fc) * 4);
+#pragma unroll
+              for (int s = 0; s < C::MAX_CLUSTER; ++s)
+                if (s < S)
+                  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                               : "=f"(part[j][s].x), "=f"(part[j][s].y), "=f"(part[j][s].z), "=f"(part[j][s].w)
+                               : "r"(p_rank[s] + off));
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+              float4 y = make_float4(0.f, 0.f, 0.f, 0.f);  // rank order: the result does not depend on timing
+#pragma unroll
+              for (int s = 0; s < C::MAX_CLUSTER; ++s)
+                if (s < S) { y.x += part[j][s].x; y.y += part[j][s].y; y.z += part[j][s].z; y.w += part[j][s].w; }
+              if (live) {                                // the y tile lies inside the stages: untouched while they are in use
+                float* dst = y_s + (tr + 4 * (2 * jh + j)) * 33 + fc;
+                dst[0] = y.x; dst[1] = y.y; dst[2] = y.z; dst[3] = y.w;
+              }
+            }
+          }
+          __syncwarp();
+          if (live && g + S * ESETS >= groups) cluster_arrive_relaxed();   // the last unit's partials are read
+          uint32_t y[16];
+#pragma unroll
+          for (int n = 0; n < 4; ++n)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              y[4 * n + i] = __float_as_uint(y_s[(r8 + 8 * (i >> 1)) * 33 + 8 * n + 2 * p + (i & 1)]);
+          finish(y, g, live);
+          __syncwarp();
+        }
       }
     }
-    // scale bytes of the rows no unit covers (ntok .. 127 of the single 128-row scale tile): zero
+    // scale bytes of the rows no group covers, up to the last row of the 128-row scale tiles: zero
     if (rank == 0 && es == 0) {
-      const int row = ew * 32 + lane;
-      if (row >= ntok) {
-        if constexpr (FMT == FMT_NVFP4) {
-          *reinterpret_cast<uint32_t*>(scales + (size_t)(2 * ft) * 512 + (row & 31) * 16 + (row >> 5) * 4) = 0u;
-          *reinterpret_cast<uint32_t*>(scales + (size_t)(2 * ft + 1) * 512 + (row & 31) * 16 + (row >> 5) * 4) = 0u;
-        } else {
-          *reinterpret_cast<uint32_t*>(scales + (size_t)ft * 512 + (row & 31) * 16 + (row >> 5) * 4) = 0u;
+      for (int row = q * 32 + lane; row < (M > 128 ? 256 : 128); row += 128) {
+        if (row >= 16 * groups) {
+          uint8_t* cell = scales + (size_t)(row >> 7) * kb4 * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4;
+          if constexpr (FMT == FMT_NVFP4) {
+            *reinterpret_cast<uint32_t*>(cell + (size_t)(2 * ft) * 512) = 0u;
+            *reinterpret_cast<uint32_t*>(cell + (size_t)(2 * ft + 1) * 512) = 0u;
+          } else {
+            *reinterpret_cast<uint32_t*>(cell + (size_t)ft * 512) = 0u;
+          }
         }
       }
     }
-  }
-  if (warp < 2) {                                        // the epilogue warps passed this barrier inside their pass 1
     tc_fence_before_sync();
-    cluster_sync_all();
+  }
+  if (PUSH) {
+    if (warp < 2 && S > 1) cluster_wait();               // the epilogue warps have waited above
+  } else {
+    if (warp < 2) { tc_fence_before_sync(); cluster_sync_all(); cluster_arrive_relaxed(); }    // as the epilogue warps in their pass 1
+    cluster_wait();                                      // no CTA of the cluster reads this one's partial tile any more
   }
 
   // ------------------------------------------------------------------ teardown
   __syncthreads();
-  if (*cta_abort) {
-    for (int i = 0; i < 2000; ++i) __nanosleep(1000);
-  }
-  cluster_sync_all();                                    // no CTA of the cluster reads this one's partial tile any more
+  // After a wait has given up, others may still push to this CTA: stay until they have left or given up as well (the
+  // barrier does not count threads that have exited).
+  if (PUSH && S > 1 && *cta_abort) cluster_sync_all();
   if (warp == 1) {
     tc_fence_after_sync();
     tmem_dealloc(tmem_base, tmem_cols);

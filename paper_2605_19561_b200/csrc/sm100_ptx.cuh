@@ -357,6 +357,21 @@ __device__ __forceinline__ void cluster_sync_after_init() {
   asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
                ::: "memory");
 }
+// A cluster barrier in two halves, for work in between.  Every thread of the CTA executes both.  The arrive is relaxed: it
+// orders no data -- after the barriers' initialisation (published by its own fence), or after remote loads whose
+// values this thread has used.  (Asking for .release makes each warp wait for all its global stores: 0.3 - 0.5 us.)
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Four words from registers into the shared memory of a CTA of the cluster; their 16 bytes are counted on `bar`,
+// a barrier of that same CTA (both addresses from map_to_cta).
+__device__ __forceinline__ void st_async_v4(uint32_t dst, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(dst), "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar) : "memory");
+}
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(

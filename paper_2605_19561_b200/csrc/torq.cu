@@ -141,17 +141,17 @@ static DeviceState* device_state() {
               opt_in_smem(rotate_quantize_kernel<256, FMT_MXINT4>, RotCfg<256>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_MXINT4>, RotPairCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_structured_kernel<FMT_MXINT4>, RotStructCfg::SMEM_BYTES) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 2>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 2>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 2>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 1>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) &&
+              opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 1, true>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) && opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 1>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) &&
               opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 2>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) &&
-              opt_in_smem(gemm_fewtok_kernel<FMT_NVFP4, 1>, GemmFewCfg<FMT_NVFP4>::max_smem_bytes()) &&
+              opt_in_smem(gemm_fewtok_kernel<FMT_NVFP4, 1, true>, GemmFewCfg<FMT_NVFP4>::max_smem_bytes()) && opt_in_smem(gemm_fewtok_kernel<FMT_NVFP4, 1>, GemmFewCfg<FMT_NVFP4>::max_smem_bytes()) &&
               opt_in_smem(gemm_fewtok_kernel<FMT_NVFP4, 2>, GemmFewCfg<FMT_NVFP4>::max_smem_bytes()) &&
-              opt_in_smem(gemm_fewtok_kernel<FMT_MXINT4, 1>, GemmFewCfg<FMT_MXINT4>::max_smem_bytes()) &&
+              opt_in_smem(gemm_fewtok_kernel<FMT_MXINT4, 1, true>, GemmFewCfg<FMT_MXINT4>::max_smem_bytes()) && opt_in_smem(gemm_fewtok_kernel<FMT_MXINT4, 1>, GemmFewCfg<FMT_MXINT4>::max_smem_bytes()) &&
               opt_in_smem(gemm_fewtok_kernel<FMT_MXINT4, 2>, GemmFewCfg<FMT_MXINT4>::max_smem_bytes()) &&
               opt_in_smem(rotate_quantize_kernel<256, FMT_F32OUT>, RotCfg<256>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_F32OUT>, RotPairCfg::SMEM_BYTES);
@@ -256,10 +256,10 @@ static_assert(kRotFewMaxTokens <= RotFewCfg::MAX_TOK && kGemmFewMaxTokens <= Gem
 //  * above S = 4, at most 1.4 CTAs per SM, so that CTAs of the next kernel in the stream find room and send their
 //    weight loads early (decode layer at d = N = 5120, M = 1: S = 5 17.86, S = 6 17.97, though the rotation by
 //    itself is the faster one with S = 6), and `long_k` K steps per CTA: a longer reduction has to be paid for by a shorter stream (rotation
-//    d = 2048, M = 50: S = 8 7.1, S = 4 6.5; GEMM K = 2048, N = 5120: S = 5 5.5, S = 4 5.1).  With 256 tokens
-//    the reduction itself is shared out (16 token groups), so there is no such bound (d = 1536: S = 8 9.9, S = 4 11.3);
+//    d = 2048, M = 50: S = 8 7.1, S = 4 6.5; GEMM K = 2048, N = 5120: S = 5 5.5, S = 4 5.1).  Above 128
+//    tokens the reduction itself is shared out (up to 16 token groups), so there is no such bound (d = 1536: S = 8 9.9, S = 4 11.3);
 //  * no S above the smallest one with the same longest K range (GEMM K = 4096: S = 5 has ranges of 4 steps like S = 4).
-static inline int fewtok_ntok(int64_t M) { return M <= 16 ? 16 : (M <= 32 ? 32 : (M <= 64 ? 64 : (M <= 128 ? 128 : 256))); }
+static inline int fewtok_ntok(int64_t M) { return (int)((M + 15) / 16 * 16); }
 static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int long_k, int ctas_per_sm, int sm_count, const int* fit) {
   int64_t most = k_steps / long_k;
   most = most < 4 ? 4 : (most > 8 ? 8 : most);
@@ -270,7 +270,7 @@ static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int long_k, int
 }
 static int fewtok_rotation_cluster(int64_t M, int64_t d, const DeviceState* st) {
   const int ntok = fewtok_ntok(M);
-  return fewtok_cluster(d / 128, d / 64, ntok == 256 ? 1 : 10, RotFewCfg::ctas_per_sm(ntok), st->sm_count, st->few_fit);
+  return fewtok_cluster(d / 128, d / 64, ntok > 128 ? 1 : 10, RotFewCfg::ctas_per_sm(ntok), st->sm_count, st->few_fit);
 }
 constexpr double kNarrowTileCost = 0.88;   // a 192-column tile against a 256-column one: 0.75 of the math, 0.875 of the operand bytes
 
@@ -524,27 +524,18 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
     const int smem = RotFewCfg::smem_bytes(ntok);
     const float ts = fmt == FMT_NVFP4 ? tensor_scale : 0.0f;
     const __nv_bfloat16* ri = static_cast<const __nv_bfloat16*>(R_intra);
-    if (RotFewCfg::ctas_per_sm(ntok) >= 2) {             // up to 64 tokens: one set of epilogue warps, two CTAs per SM
-      if (fmt == FMT_MXINT4)
-        launch_tc(rotate_fewtok_kernel<FMT_MXINT4, 1>, S, tiles * S, 192, smem, s, tmX, tmR, ri, codes, scales, (int)M,
-                  (int)d, ntok, S, ts, st->err_word);
-      else if (fmt == FMT_NVFP4)
-        launch_tc(rotate_fewtok_kernel<FMT_NVFP4, 1>, S, tiles * S, 192, smem, s, tmX, tmR, ri, codes, scales, (int)M,
-                  (int)d, ntok, S, ts, st->err_word);
-      else
-        launch_tc(rotate_fewtok_kernel<FMT_MXFP4, 1>, S, tiles * S, 192, smem, s, tmX, tmR, ri, codes, scales, (int)M,
-                  (int)d, ntok, S, ts, st->err_word);
-    } else {                                             // 128 or 256 tokens: two sets
-      if (fmt == FMT_MXINT4)
-        launch_tc(rotate_fewtok_kernel<FMT_MXINT4, 2>, S, tiles * S, 320, smem, s, tmX, tmR, ri, codes, scales, (int)M,
-                  (int)d, ntok, S, ts, st->err_word);
-      else if (fmt == FMT_NVFP4)
-        launch_tc(rotate_fewtok_kernel<FMT_NVFP4, 2>, S, tiles * S, 320, smem, s, tmX, tmR, ri, codes, scales, (int)M,
-                  (int)d, ntok, S, ts, st->err_word);
-      else
-        launch_tc(rotate_fewtok_kernel<FMT_MXFP4, 2>, S, tiles * S, 320, smem, s, tmX, tmR, ri, codes, scales, (int)M,
-                  (int)d, ntok, S, ts, st->err_word);
-    }
+    // up to 16 tokens: partials pushed to one CTA; up to 64: one set of epilogue warps, two CTAs per SM; more: two sets
+    auto launch = [&](auto push, auto one, auto two) {
+      const bool small = RotFewCfg::ctas_per_sm(ntok) >= 2;
+      launch_tc(ntok <= RotFewCfg::MAX_PUSH_TOK ? push : (small ? one : two), S, tiles * S, small ? 192 : 320, smem, s, tmX, tmR, ri,
+                codes, scales, (int)M, (int)d, ntok, S, ts, st->err_word);
+    };
+    if (fmt == FMT_MXINT4)
+      launch(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, rotate_fewtok_kernel<FMT_MXINT4, 1>, rotate_fewtok_kernel<FMT_MXINT4, 2>);
+    else if (fmt == FMT_NVFP4)
+      launch(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, rotate_fewtok_kernel<FMT_NVFP4, 1>, rotate_fewtok_kernel<FMT_NVFP4, 2>);
+    else
+      launch(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, rotate_fewtok_kernel<FMT_MXFP4, 1>, rotate_fewtok_kernel<FMT_MXFP4, 2>);
     return launch_status();
   }
   if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d * x_terms, 128, 64) ||
@@ -766,14 +757,11 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
     if (!encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, 128, 128) ||
         !encode_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Aq, (uint64_t)M, krow, (uint32_t)ntok, 128))
       return TORQ_ERR_LAUNCH;
-    if (FC::ctas_per_sm(ntok) >= 2)                      // up to 64 tokens: one set of epilogue warps, two CTAs per SM
-      launch_tc(gemm_fewtok_kernel<FMT, 1>, S, tiles * S, 192, FC::smem_bytes(ntok), s, tmB, tmA,
-                static_cast<const uint8_t*>(As), static_cast<const uint8_t*>(Ws), Y, y_dtype == TORQ_BF16 ? 1 : 0, (int)M,
-                (int)N, (int)K, ntok, S, alpha, st->err_word);
-    else                                                 // 128 tokens: two sets
-      launch_tc(gemm_fewtok_kernel<FMT, 2>, S, tiles * S, 320, FC::smem_bytes(ntok), s, tmB, tmA,
-                static_cast<const uint8_t*>(As), static_cast<const uint8_t*>(Ws), Y, y_dtype == TORQ_BF16 ? 1 : 0, (int)M,
-                (int)N, (int)K, ntok, S, alpha, st->err_word);
+    // up to 16 tokens: partials pushed; up to 64: one set of epilogue warps, two CTAs per SM; more: two sets
+    const bool small = FC::ctas_per_sm(ntok) >= 2;
+    launch_tc(ntok <= FC::MAX_PUSH_TOK ? gemm_fewtok_kernel<FMT, 1, true> : (small ? gemm_fewtok_kernel<FMT, 1> : gemm_fewtok_kernel<FMT, 2>),
+              S, tiles * S, small ? 192 : 320, FC::smem_bytes(ntok), s, tmB, tmA, static_cast<const uint8_t*>(As),
+              static_cast<const uint8_t*>(Ws), Y, y_dtype == TORQ_BF16 ? 1 : 0, (int)M, (int)N, (int)K, ntok, S, alpha, st->err_word);
     return launch_status();
   }
   // CTA pairs from two row tiles on -- except for exactly two row tiles with so few 256-column tiles

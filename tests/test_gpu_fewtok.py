@@ -63,6 +63,14 @@ def test_rotation_cluster_sizes(M, d):
     test_rotation_alone_without_any_workspace(M, d)
 
 
+# tokens per instruction go in steps of 16: first and last count of some steps, on both sides of the one-group (pushed)
+# form, of one CTA per SM (65) and of the second scale tile (129); one, several and eight CTAs per cluster
+@pytest.mark.parametrize("M,d", [(7, 640), (15, 1536), (16, 2560), (17, 896), (48, 896), (49, 1536), (80, 2560), (81, 3072),
+                                 (112, 4096), (144, 2176), (145, 4096), (208, 3072), (241, 2176), (12, 12288)])
+def test_rotation_token_steps(M, d):
+    test_rotation_alone_without_any_workspace(M, d)
+
+
 def test_rotation_exact_cases_are_bit_exact():
     """Permutation and identity rotations with integer activations: every partial sum is exact in any
     order, so codes and scales must equal the oracle's bit for bit through the split and the reduction."""
@@ -123,6 +131,13 @@ def test_gemm_random_operands(M, N, K):
 # the ends of the cluster rule: 96 tiles x 2 CTAs, ranges of one and of seven K steps, clusters of eight
 @pytest.mark.parametrize("M,N,K", [(33, 12288, 1024), (3, 264, 256), (64, 1024, 14336), (100, 1024, 14336), (100, 2048, 4096)])
 def test_gemm_cluster_sizes(M, N, K):
+    test_gemm_random_operands(M, N, K)
+
+
+# the same for the GEMM; K = 256 and 128: a cluster of one CTA, whose accumulator goes to Y directly
+@pytest.mark.parametrize("M,N,K", [(3, 1000, 2048), (13, 520, 4096), (16, 264, 384), (48, 1000, 2048), (49, 264, 4096),
+                                   (81, 520, 2048), (112, 264, 640), (40, 264, 256), (128, 72, 128), (5, 72, 256)])
+def test_gemm_token_steps(M, N, K):
     test_gemm_random_operands(M, N, K)
 
 
