@@ -1,5 +1,5 @@
-"""Thin ctypes binding over the C-ABI library (include/torq.h).  Argument marshalling only:
-every step of the path runs in the CUDA kernels; PyTorch provides device memory and streams.
+"""Thin binding over the C-ABI library (include/torq.h): ctypes, and for the whole-layer calls a native extension.
+Argument marshalling only: every step of the path runs in the CUDA kernels; PyTorch provides device memory and streams.
 There is no fallback: a missing library or a non-zero status raises."""
 from __future__ import annotations
 
@@ -115,8 +115,30 @@ def lib() -> ctypes.CDLL:
     L.torq_pair_tile_list.restype = i64
     L.torq_launch_count.argtypes = []
     L.torq_launch_count.restype = i64
+    if _build.needs_binding():
+        _build.build_binding()
+    from . import _torq_binding
+    for kind, fn in enumerate((L.torq_rotated_linear, L.torq_rotated_linear_mxint4, L.torq_rotated_linear_structured,
+                               L.torq_rotated_linear_nvfp4)):
+        _torq_binding.set_entry(kind, ctypes.cast(fn, vp).value)
+    global _layer
+    _layer = _torq_binding.layer
     _lib_handle = L
     return L
+
+
+# The whole-layer calls go through the native binding (csrc/binding.cpp), which returns the library's status, or -1 for
+# operands that it does not take: those go on to the checks below it, which say what is wrong with them.
+def _layer(*args):                               # until lib() has put the native function here
+    lib()
+    return _layer(*args)
+
+
+_MXFP4, _MXINT4, _STRUCTURED, _NVFP4 = range(4)
+
+
+def _handle(stream):
+    return None if stream is None else stream.cuda_stream
 
 
 # The marshalling below is paid on every call, and a layer of a few tokens takes the GPU 13 us: addresses and
@@ -233,16 +255,22 @@ def torq_mxfp4_gemm(Aq, As, Wq, Ws, out_dtype=torch.bfloat16, Y=None, stream=Non
 def torq_rotated_linear(X, R_inter, R_intra, Wq, Ws, out_dtype=torch.bfloat16, Y=None, workspace=None,
                         dbg_codes=None, dbg_scales=None, stream=None):
     """Rotate, quantize and multiply in one call.  Returns Y [M,N]."""
+    if Y is None:
+        Y = torch.empty((X.shape[0], Wq.shape[0]), dtype=out_dtype, device=X.device)
+    if workspace is None:
+        M, d = X.shape
+        workspace = torch.empty(torq_workspace_bytes(M, d, Wq.shape[0]), dtype=torch.uint8, device=X.device)
+    rc = _layer(_MXFP4, X, R_inter, R_intra, Wq, Ws, Y, workspace, dbg_codes, dbg_scales, _handle(stream))
+    if rc == 0:
+        return Y
+    if rc > 0:
+        raise TorqError(rc, "torq_rotated_linear")
     M, d = X.shape
     N = Wq.shape[0]
     for t, n in ((X, "X"), (R_inter, "R_inter"), (R_intra, "R_intra")):
         _check(t, torch.bfloat16, n)
     for t, n in ((Wq, "Wq"), (Ws, "Ws"), (dbg_codes, "dbg_codes"), (dbg_scales, "dbg_scales")):
         _check(t, torch.uint8, n)
-    if Y is None:
-        Y = torch.empty((M, N), dtype=out_dtype, device=X.device)
-    if workspace is None:
-        workspace = torch.empty(torq_workspace_bytes(M, d, N), dtype=torch.uint8, device=X.device)
     dt = TORQ_F32 if Y.dtype == torch.float32 else TORQ_BF16
     _raise(lib().torq_rotated_linear(_ptr(X), _ptr(R_inter), _ptr(R_intra), _ptr(Wq), _ptr(Ws), M, d, N,
                                      _ptr(Y), dt, _ptr(workspace), workspace.numel(), _ptr(dbg_codes),
@@ -253,16 +281,22 @@ def torq_rotated_linear(X, R_inter, R_intra, Wq, Ws, out_dtype=torch.bfloat16, Y
 def torq_rotated_linear_structured(X, R_B, R_intra, Wq, Ws, out_dtype=torch.bfloat16, Y=None, workspace=None,
                                    dbg_codes=None, dbg_scales=None, stream=None):
     """The whole layer with the rotation in the paper's structure (R_B [d/32,d/32], shared R_intra [32,32])."""
+    if Y is None:
+        Y = torch.empty((X.shape[0], Wq.shape[0]), dtype=out_dtype, device=X.device)
+    if workspace is None:
+        M, d = X.shape
+        workspace = torch.empty(torq_workspace_bytes(M, d, Wq.shape[0]), dtype=torch.uint8, device=X.device)
+    rc = _layer(_STRUCTURED, X, R_B, R_intra, Wq, Ws, Y, workspace, dbg_codes, dbg_scales, _handle(stream))
+    if rc == 0:
+        return Y
+    if rc > 0:
+        raise TorqError(rc, "torq_rotated_linear_structured")
     M, d = X.shape
     N = Wq.shape[0]
     for t, n in ((X, "X"), (R_B, "R_B"), (R_intra, "R_intra")):
         _check(t, torch.bfloat16, n)
     for t, n in ((Wq, "Wq"), (Ws, "Ws"), (dbg_codes, "dbg_codes"), (dbg_scales, "dbg_scales")):
         _check(t, torch.uint8, n)
-    if Y is None:
-        Y = torch.empty((M, N), dtype=out_dtype, device=X.device)
-    if workspace is None:
-        workspace = torch.empty(torq_workspace_bytes(M, d, N), dtype=torch.uint8, device=X.device)
     dt = TORQ_F32 if Y.dtype == torch.float32 else TORQ_BF16
     _raise(lib().torq_rotated_linear_structured(_ptr(X), _ptr(R_B), _ptr(R_intra), _ptr(Wq), _ptr(Ws), M, d, N,
                                                 _ptr(Y), dt, _ptr(workspace), workspace.numel(), _ptr(dbg_codes),
@@ -439,16 +473,22 @@ def torq_rotated_linear_nvfp4(X, R_inter, R_intra32, x_tensor_scale: float, Wq, 
                               out_dtype=torch.bfloat16, Y=None, workspace=None, dbg_codes=None, dbg_scales=None,
                               stream=None):
     """Rotate, quantize to NVFP4 and multiply in one call.  Returns Y [M,N]."""
+    if Y is None:
+        Y = torch.empty((X.shape[0], Wq.shape[0]), dtype=out_dtype, device=X.device)
+    if workspace is None:
+        M, d = X.shape
+        workspace = torch.empty(torq_nvfp4_workspace_bytes(M, d, Wq.shape[0]), dtype=torch.uint8, device=X.device)
+    rc = _layer(_NVFP4, X, R_inter, R_intra32, Wq, Ws, Y, workspace, dbg_codes, dbg_scales, _handle(stream), x_tensor_scale, w_tensor_scale)
+    if rc == 0:
+        return Y
+    if rc > 0:
+        raise TorqError(rc, "torq_rotated_linear_nvfp4")
     M, d = X.shape
     N = Wq.shape[0]
     for t, n in ((X, "X"), (R_inter, "R_inter"), (R_intra32, "R_intra32")):
         _check(t, torch.bfloat16, n)
     for t, n in ((Wq, "Wq"), (Ws, "Ws"), (dbg_codes, "dbg_codes"), (dbg_scales, "dbg_scales")):
         _check(t, torch.uint8, n)
-    if Y is None:
-        Y = torch.empty((M, N), dtype=out_dtype, device=X.device)
-    if workspace is None:
-        workspace = torch.empty(torq_nvfp4_workspace_bytes(M, d, N), dtype=torch.uint8, device=X.device)
     dt = TORQ_F32 if Y.dtype == torch.float32 else TORQ_BF16
     _raise(lib().torq_rotated_linear_nvfp4(_ptr(X), _ptr(R_inter), _ptr(R_intra32), x_tensor_scale, _ptr(Wq),
                                            _ptr(Ws), w_tensor_scale, M, d, N, _ptr(Y), dt, _ptr(workspace),
@@ -553,16 +593,22 @@ def torq_mxint4_gemm(A8, As, W8, Ws, out_dtype=torch.bfloat16, Y=None, stream=No
 def torq_rotated_linear_mxint4(X, R_inter, R_intra, W8, Ws, out_dtype=torch.bfloat16, Y=None, workspace=None,
                                dbg_bytes=None, dbg_scales=None, stream=None):
     """Rotate, quantize to MXINT4 and multiply in one call.  Returns Y [M,N]."""
+    if Y is None:
+        Y = torch.empty((X.shape[0], W8.shape[0]), dtype=out_dtype, device=X.device)
+    if workspace is None:
+        M, d = X.shape
+        workspace = torch.empty(torq_mxint4_workspace_bytes(M, d, W8.shape[0]), dtype=torch.uint8, device=X.device)
+    rc = _layer(_MXINT4, X, R_inter, R_intra, W8, Ws, Y, workspace, dbg_bytes, dbg_scales, _handle(stream))
+    if rc == 0:
+        return Y
+    if rc > 0:
+        raise TorqError(rc, "torq_rotated_linear_mxint4")
     M, d = X.shape
     N = W8.shape[0]
     for t, n in ((X, "X"), (R_inter, "R_inter"), (R_intra, "R_intra")):
         _check(t, torch.bfloat16, n)
     for t, n in ((W8, "W8"), (Ws, "Ws"), (dbg_bytes, "dbg_bytes"), (dbg_scales, "dbg_scales")):
         _check(t, torch.uint8, n)
-    if Y is None:
-        Y = torch.empty((M, N), dtype=out_dtype, device=X.device)
-    if workspace is None:
-        workspace = torch.empty(torq_mxint4_workspace_bytes(M, d, N), dtype=torch.uint8, device=X.device)
     dt = TORQ_F32 if Y.dtype == torch.float32 else TORQ_BF16
     _raise(lib().torq_rotated_linear_mxint4(_ptr(X), _ptr(R_inter), _ptr(R_intra), _ptr(W8), _ptr(Ws), M, d, N,
                                             _ptr(Y), dt, _ptr(workspace), workspace.numel(), _ptr(dbg_bytes),
