@@ -278,7 +278,7 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       tmem_ld_wait();
       tc_fence_before_sync();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(map_to_cta(acce_bar, 0));   // accumulator is free again
+      if (lane == 0 && tile + npairs < total_tiles) mbar_arrive_cluster(map_to_cta(acce_bar, 0));   // accumulator is free again
       if constexpr (FMT == FMT_NVFP4) {                    // product of the two tensor scales
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
@@ -355,7 +355,8 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
   if (*cta_abort) {
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
-  cluster_sync_all();
+  cluster_arrive_relaxed();                            // every arrival this CTA sent has been waited for: no data to order
+  cluster_wait();
   if (warp == 1) {
     tc_fence_after_sync();
     tmem_dealloc_pair(tmem_base, C::TMEM_COLS);

@@ -260,7 +260,8 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
   if (*cta_abort) {
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
-  cluster_sync_all();
+  cluster_arrive_relaxed();                            // the peer no longer touches this CTA's memory; no data to order
+  cluster_wait();
   if (warp == 1) {
     tc_fence_after_sync();
     tmem_dealloc_pair(tmem_base, 512);

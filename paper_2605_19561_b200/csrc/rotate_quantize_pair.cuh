@@ -17,7 +17,8 @@
 // acc_empty[a] lives in the leader and takes one arrival per epilogue warp of both CTAs (16).
 #pragma once
 #include <cuda_bf16.h>
-#include "intra_fragment.cuh"
+#include "nvfp4_quantize.cuh"
+#include "mxint4_quantize.cuh"
 #include "sm100_ptx.cuh"
 
 namespace torq {
@@ -288,10 +289,10 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
           uint32_t yv[32];
           tmem_ld_32x32(tacc + bb * 32, yv);
           tmem_ld_wait();
-          if (bb == nbb - 1) {                           // this warp's share is read: tell the leader
+          if (bb == nbb - 1) {                           // this warp's share is read: tell the leader (of another tile to come)
             tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_to_cta(acce_bar(a), 0));
+            if (lane == 0 && tile + npairs < total_tiles) mbar_arrive_cluster(map_to_cta(acce_bar(a), 0));
           }
           float z[32];
           if (R_intra != nullptr) {
@@ -345,18 +346,27 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       }
       // ---- accumulator fragment layout (16 rows at a time): thread t holds rows t/4 and t/4 + 8,
       //      eight columns of each per block
+      const int64_t row_base = (int64_t)mt * C::BM + q * 32 + r8;     // + 16 mh + 8 rh
       uint32_t sc_word[4] = {0u, 0u, 0u, 0u};            // rows r8 + 16 mh + 8 rh -> index 2 mh + rh
       uint32_t sc_hi[4] = {0u, 0u, 0u, 0u};              // NVFP4: second group of four 16-blocks
       NvScale nvs = {};
       if constexpr (FMT == FMT_NVFP4) nvs = nv_scale(tensor_scale);
 #pragma unroll 1
       for (int bb = 0; bb < nbb; ++bb) {
-        // lane l: row l % 8 of matrix l / 8
-        const uint32_t rb = ri_saddr + (uint32_t)(h * nbb + bb) * C::RI_BLOCK_BYTES +
-                            (uint32_t)(((lane >> 3) & 1) * 8 + (lane & 7)) * C::RI_ROW_BYTES + (uint32_t)(lane >> 4) * 16;
-        IntraFrag f;
-        if (R_intra != nullptr) load_intra_frag(rb, rb + 32, 16 * C::RI_ROW_BYTES, f);
-        uint32_t sb[4];
+        const int blk = fb + bb;
+        uint32_t bfrag[2][4][2];                         // [k chunk][n tile][2]
+        if (R_intra != nullptr) {
+          // lane l: row l % 8 of matrix l / 8; matrices (k 0-7, n), (k 8-15, n), (k 0-7, n+8), (k 8-15, n+8)
+          const uint32_t rb = ri_saddr + (uint32_t)(h * nbb + bb) * C::RI_BLOCK_BYTES +
+                              (uint32_t)(((lane >> 3) & 1) * 8 + (lane & 7)) * C::RI_ROW_BYTES +
+                              (uint32_t)(lane >> 4) * 16;
+#pragma unroll
+          for (int kc = 0; kc < 2; ++kc)
+#pragma unroll
+            for (int np = 0; np < 2; ++np)
+              ldmatrix_x4_trans(rb + kc * 16 * C::RI_ROW_BYTES + np * 32, bfrag[kc][2 * np][0], bfrag[kc][2 * np][1],
+                                bfrag[kc][2 * np + 1][0], bfrag[kc][2 * np + 1][1]);
+        }
 #pragma unroll
         for (int mh = 0; mh < 2; ++mh) {
           uint32_t y[16];
@@ -365,18 +375,61 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
           if (bb == nbb - 1 && mh == 1) {                // this warp's share is read: tell the leader
             tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_to_cta(acce_bar(a), 0));
+            if (lane == 0 && tile + npairs < total_tiles) mbar_arrive_cluster(map_to_cta(acce_bar(a), 0));
           }
-          intra_quantize_frag16<FMT>(y, R_intra != nullptr, f, lane, (int64_t)mt * C::BM + q * 32 + 16 * mh, M, fb + bb,
-                                     nblocks, d, nvs, codes, sb + 2 * mh);
-        }
+          float acc[4][4];
+          if (R_intra != nullptr) {
+            uint32_t ah[8], am[8], al[8];                // A fragments: [k chunk * 4 + (n & 1) * 2 + row half]
 #pragma unroll
-        for (int rs = 0; rs < 4; ++rs) {
-          if constexpr (FMT == FMT_NVFP4) {
-            if (bb < 2) sc_word[rs] |= sb[rs] << (16 * bb);
-            else sc_hi[rs] |= sb[rs] << (16 * (bb - 2));
+            for (int n = 0; n < 4; ++n)
+#pragma unroll
+              for (int rh = 0; rh < 2; ++rh) {
+                const int ai = (n >> 1) * 4 + (n & 1) * 2 + rh;
+                split3_bf16x2(y[4 * n + 2 * rh], y[4 * n + 2 * rh + 1], ah[ai], am[ai], al[ai]);
+              }
+#pragma unroll
+            for (int n = 0; n < 4; ++n) { acc[n][0] = 0.f; acc[n][1] = 0.f; acc[n][2] = 0.f; acc[n][3] = 0.f; }
+#pragma unroll
+            for (int kc = 0; kc < 2; ++kc)
+#pragma unroll
+              for (int n = 0; n < 4; ++n) {
+                mma_16816_bf16(acc[n], al + 4 * kc, bfrag[kc][n]);
+                mma_16816_bf16(acc[n], am + 4 * kc, bfrag[kc][n]);
+                mma_16816_bf16(acc[n], ah + 4 * kc, bfrag[kc][n]);
+              }
           } else {
-            sc_word[rs] |= sb[rs] << (8 * bb);
+#pragma unroll
+            for (int n = 0; n < 4; ++n)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) acc[n][e] = __uint_as_float(y[4 * n + e]);
+          }
+#pragma unroll
+          for (int rh = 0; rh < 2; ++rh) {
+            const float v[8] = {acc[0][2 * rh], acc[0][2 * rh + 1], acc[1][2 * rh], acc[1][2 * rh + 1],
+                                acc[2][2 * rh], acc[2][2 * rh + 1], acc[3][2 * rh], acc[3][2 * rh + 1]};
+            uint32_t word, sbyte;
+            const int64_t row = row_base + 16 * mh + 8 * rh;
+            if constexpr (FMT == FMT_MXINT4) {             // two operand bytes per 8 columns and lane
+              uint32_t pr[4];
+              mxint4_quantize_row_fragment(v, pr, sbyte);
+              if (row < M && blk < nblocks) {
+                uint8_t* dst = codes + row * (int64_t)d + (int64_t)blk * 32 + 2 * p;
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) *reinterpret_cast<uint16_t*>(dst + 8 * nt) = (uint16_t)pr[nt];
+              }
+            } else {
+              if constexpr (FMT == FMT_NVFP4) nv_quantize_row_fragment(v, p, nvs, word, sbyte);
+              else quantize_row_fragment(v, p, word, sbyte);
+              if (row < M && blk < nblocks)
+                *reinterpret_cast<uint32_t*>(codes + row * (int64_t)(d / 2) + (int64_t)blk * 16 + 4 * p) = word;
+            }
+            if constexpr (FMT == FMT_NVFP4) {
+              if (blk >= nblocks) sbyte = 0;
+              if (bb < 2) sc_word[2 * mh + rh] |= sbyte << (16 * bb);
+              else sc_hi[2 * mh + rh] |= sbyte << (16 * (bb - 2));
+            } else {
+              sc_word[2 * mh + rh] |= sbyte << (8 * bb);
+            }
           }
         }
       }
@@ -402,7 +455,10 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   if (*cta_abort) {
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
-  cluster_sync_all();                                  // the peer no longer touches this CTA's memory
+  // The peer no longer touches this CTA's memory after this.  Relaxed: every arrival this CTA sent has been waited for (its
+  // last tile sends none), and a release would make each warp wait for its global stores (0.3 - 0.5 us).
+  cluster_arrive_relaxed();
+  cluster_wait();
   if (warp == 1) {
     tc_fence_after_sync();
     tmem_dealloc_pair(tmem_base, C::TMEM_COLS);

@@ -223,7 +223,8 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   if (*cta_abort) {
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
-  cluster_sync_all();                                  // the peer no longer touches this CTA's memory
+  cluster_arrive_relaxed();                            // the peer no longer touches this CTA's memory; no data to order
+  cluster_wait();
   if (warp == 1) {
     tc_fence_after_sync();
     tmem_dealloc_pair(tmem_base, 512);

@@ -416,13 +416,13 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 }
 
 // Width of the one-wave rotation's tiles, or 0 where another kernel is faster.  Times in us, fitted to the rotation
-// alone at 27 shapes (d = 256 ... 14336, M = 100 ... 4000; within 10 % but for the HBM-bound ones at d > 8192, where
-// both sides are low by as much):
-//  * here: 2.2 + 0.026 per column (2.4 + 0.032 above 256 columns) for launch and epilogue, then per K step the operand
-//    bytes, 0.215 + 0.0003 per column, or the math, 0.00114 per column;
-//  * few tokens: 3.8 / 4.8 / 4.5 / 8.3 up to 16 / 64 / 128 / 256 tokens, plus 0.24 / 0.22 / 0.385 / 0.425 per K step of
+// alone at 60 shapes (d = 128 ... 14336, M = 1 ... 4000; within 10 % but for the HBM-bound ones at d > 8192, where both
+// sides are low by as much); f = filled part of a wave:
+//  * here: 1.6 + 0.022 per column (2 + 0.032 above 256 columns) for launch and epilogue, then per K step the operand
+//    bytes, 0.17 + 0.0003 per column + 0.03 f, or the math, 0.00114 per column;
+//  * few tokens: 3.1 / 4.4 / 5.6 / 8.3 up to 16 / 64 / 128 / 256 tokens, plus 0.22 / 0.2 / 0.36 / 0.42 per K step of
 //    the longest split;
-//  * pair kernel: 6.8, plus per K step 0.32 for a wave and 0.2 + 0.14 x (filled part) for the last, partly filled one.
+//  * pair kernel: 6.8, plus per K step 0.32 for a wave and 0.2 + 0.14 f for the last, partly filled one.
 // A layer of 2048 tokens and more fills the pair kernel's waves and stays there (one-wave tiles would be wider than
 // 384 columns; 2048 x 4096 measured 51.6 with 480 columns, 46.8 in the pair kernel).
 static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int max_pairs) {
@@ -431,13 +431,14 @@ static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int max_pair
   int width = 0;
   for (int w = 32; w <= RotWideCfg::MAX_WIDTH; w += 32) {
     if (rows * ((d + w - 1) / w) > max_pairs) continue;
-    const double bytes = 0.215 + 0.0003 * w, math = 0.00114 * w;
-    const double t = (w <= 256 ? 2.2 + 0.026 * w : 2.4 + 0.032 * w) + (double)steps * (bytes > math ? bytes : math);
+    const double f = (double)(rows * ((d + w - 1) / w)) / max_pairs;
+    const double bytes = 0.17 + 0.0003 * w + 0.03 * f, math = 0.00114 * w;
+    const double t = (w <= 256 ? 1.6 + 0.022 * w : 2.0 + 0.032 * w) + (double)steps * (bytes > math ? bytes : math);
     if (t < best) { best = t; width = w; }
   }
   double other;
   if (M <= kRotFewMaxTokens) {
-    other = M <= 16 ? 3.8 + 0.24 * few_steps : (M <= 64 ? 4.8 + 0.22 * few_steps : (M <= 128 ? 4.5 + 0.385 * few_steps : 8.3 + 0.425 * few_steps));
+    other = M <= 16 ? 3.1 + 0.22 * few_steps : (M <= 64 ? 4.4 + 0.2 * few_steps : (M <= 128 ? 5.6 + 0.36 * few_steps : 8.3 + 0.42 * few_steps));
   } else {
     const int64_t tiles = rows * ((d + 255) / 256);
     const int64_t full = tiles / max_pairs, rest = tiles % max_pairs;
@@ -676,15 +677,17 @@ torq_status torq_rotate_quantize_structured_nvfp4(const void* X, const void* R_B
 }  // extern "C"
 
 // Width of the one-wave GEMM's tiles, or 0 where another kernel is faster.  Times in us, fitted to MXFP4 with bf16 output
-// at K = 256 ... 14336, N = 256 ... 12288, M = 200 ... 8000 (within 8 %); f = filled part of a wave:
-//  * here: 2.3 + 0.0062 per column + f for launch and epilogue, then per K step 0.265 or the math, 0.0011 per
+// at K = 128 ... 14336, N = 256 ... 12288, M = 17 ... 8000 (within 10 %); f = filled part of a wave:
+//  * here: 2 + 0.0062 per column + f for launch and epilogue, then per K step 0.265 or the math, 0.0011 per
 //    column, + 0.025 f;
+//  * few tokens (17 to 128, S CTAs per tile): 2.3 + 0.2 per K step of the longest split + per token 0.025 with S = 1 (the
+//    accumulator goes to Y), else 0.012 + 0.035 / S;
 //  * pair kernel: one wave 4.1 + 0.9 f + (0.285 + 0.04 f) per K step, more (the last one as narrower tiles) 5.2 + per K step
 //    0.325 for a full wave and 0.21 + 0.14 f for the last;
 //  * single CTAs (129 to 256 tokens, few column tiles): 3.2 + 1.3 f + 0.285 per K step.
 // Where it pays: 777 x 5120, K = 14336 (80 pair tiles) 35.1 -> 28.5, K = 4096 13.8 -> 12.3; 1280 x 4096, K = 14336 35.2 ->
-// 29.1; few and narrow outputs, 2000 x 256, K = 1024 5.2 -> 3.9.
-static int wide_gemm_width(int64_t M, int64_t N, int64_t steps, bool pairs, int max_pairs) {
+// 29.1; short contractions: 64 x 256, K = 256 3.9 -> 2.4; 100 x 4096, K = 512 5.0 -> 3.4; 2000 x 256, K = 1024 5.2 -> 3.9.
+static int wide_gemm_width(int64_t M, int64_t N, int64_t steps, bool pairs, int few_S, int max_pairs) {
   const int64_t rows = (M + 255) / 256;
   double best = 1e30;
   int width = 0;
@@ -692,13 +695,15 @@ static int wide_gemm_width(int64_t M, int64_t N, int64_t steps, bool pairs, int 
     const int64_t tiles = rows * ((N + w - 1) / w);
     if (tiles > max_pairs) continue;
     const double f = (double)tiles / max_pairs, math = 0.0011 * w;
-    const double t = 2.3 + 0.0062 * w + f + (double)steps * ((math > 0.265 ? math : 0.265) + 0.025 * f);
+    const double t = 2.0 + 0.0062 * w + f + (double)steps * ((math > 0.265 ? math : 0.265) + 0.025 * f);
     if (t < best) { best = t; width = w; }
   }
   const int64_t tiles = rows * ((N + 255) / 256), full = tiles / max_pairs, rest = tiles % max_pairs;
   const double f = (double)rest / max_pairs;
   double other;
-  if (!pairs) other = 3.2 + 1.3 * (double)((M + 127) / 128 * ((N + 127) / 128)) / (2 * max_pairs) + 0.285 * (double)steps;
+  if (few_S > 0)
+    other = 2.3 + 0.2 * (double)((steps + few_S - 1) / few_S) + (double)M * (few_S == 1 ? 0.025 : 0.012 + 0.035 / few_S);
+  else if (!pairs) other = 3.2 + 1.3 * (double)((M + 127) / 128 * ((N + 127) / 128)) / (2 * max_pairs) + 0.285 * (double)steps;
   else if (full == 0) other = 4.1 + 0.9 * f + (double)steps * (0.285 + 0.04 * f);
   else other = 5.2 + (double)steps * (0.325 * (double)full + (rest ? 0.21 + 0.14 * f : 0.0));
   return best < 0.97 * other ? width : 0;
@@ -753,7 +758,10 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
     using FC = GemmFewCfg<FMT>;
     const int ntok = fewtok_ntok(M);
     const int tiles = (int)((N + 127) / 128);
-    const int S = fewtok_cluster(tiles, (K + FC::BK - 1) / FC::BK, 3, FC::ctas_per_sm(ntok), st->sm_count, st->few_fit);
+    const int64_t steps = (K + FC::BK - 1) / FC::BK;
+    const int S = fewtok_cluster(tiles, steps, 3, FC::ctas_per_sm(ntok), st->sm_count, st->few_fit);
+    const int width = M > FC::MAX_PUSH_TOK ? wide_gemm_width(M, N, steps, false, S, st->gemm_pairs) : 0;
+    if (width > 0) return gemm_wide<FMT>(st, Aq, As, Wq, Ws, M, N, K, Y, y_dtype, alpha, width, s);
     if (!encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, 128, 128) ||
         !encode_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Aq, (uint64_t)M, krow, (uint32_t)ntok, 128))
       return TORQ_ERR_LAUNCH;
@@ -769,7 +777,7 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
   // put four times as many SMs to work on streaming W.
   const int64_t pair_tiles = ((M + 255) / 256) * ((N + BN - 1) / BN);
   const bool use_pairs = !(M <= 256 && 4 * pair_tiles <= st->sm_count);
-  const int width = wide_gemm_width(M, N, (K + GemmWideCfg<FMT>::BK - 1) / GemmWideCfg<FMT>::BK, use_pairs, st->gemm_pairs);
+  const int width = wide_gemm_width(M, N, (K + GemmWideCfg<FMT>::BK - 1) / GemmWideCfg<FMT>::BK, use_pairs, 0, st->gemm_pairs);
   if (width > 0) return gemm_wide<FMT>(st, Aq, As, Wq, Ws, M, N, K, Y, y_dtype, alpha, width, s);
   if (use_pairs) {
     CUtensorMap tmSFA, tmSFB;

@@ -23,7 +23,7 @@ def _rand_rotation(d, seed):
 
 # widths on 74 pairs: 32, 32 (two K steps), 32 (padding rows in a second, token-less row tile), 64, 96, 128, 160 (tail of
 # 16), 192, 224, 288 (two instructions), 320, 352, 384 (d no multiple of the width but for the first ones)
-@pytest.mark.parametrize("M,d", [(50, 256), (24, 128), (257, 256), (700, 1024), (1280, 1024), (1000, 2048), (1280, 2048),
+@pytest.mark.parametrize("M,d", [(50, 256), (24, 128), (16, 256), (1, 128), (257, 256), (700, 1024), (1280, 1024), (1000, 2048), (1280, 2048),
                                  (1536, 2048), (600, 5120), (2304, 2304), (1400, 3840), (3072, 2048), (1280, 5120)])
 def test_rotation_mxfp4(M, d):
     g = np.random.default_rng(M + d)
@@ -86,16 +86,16 @@ def _rand_operand(rows, k, seed):
     return g.integers(0, 16, size=(rows, k), dtype=np.uint8), g.integers(118, 134, size=(rows, k // 32), dtype=np.uint8)
 
 
-# one-wave GEMM: widths 64 and 128 (few output tiles), 192, 320 and 384 (two instructions, W tiles that start 64 rows
+# one-wave GEMM: few tokens with a short contraction; widths 64 and 128 (few output tiles), 192, 320 and 384 (two instructions, W tiles that start 64 rows
 # into a scale chunk); ragged rows and columns, a half last K stage (K % 256 == 128)
-@pytest.mark.parametrize("M,N,K", [(1300, 200, 384), (300, 136, 128), (1000, 1000, 256), (2000, 1096, 256), (777, 5120, 2176),
+@pytest.mark.parametrize("M,N,K", [(64, 256, 256), (17, 72, 128), (128, 1032, 512), (1300, 200, 384), (300, 136, 128), (1000, 1000, 256), (2000, 1096, 256), (777, 5120, 2176),
                                    (1000, 6136, 4096)])
 def test_gemm_mxfp4(M, N, K):
     ac, asb = _rand_operand(M, K, 1)
     wc, wsb = _rand_operand(N, K, 2)
     ops = (dev_u8(O.pack_codes(ac)), dev_u8(O.swizzle_scales(asb, K, fill=0)), dev_u8(O.pack_codes(wc)),
            dev_u8(O.swizzle_scales(wsb, K, fill=0)))
-    rows = np.unique(np.r_[np.arange(96), np.arange(M - 140, M)])        # the oracle's share
+    rows = np.unique(np.r_[np.arange(min(M, 96)), np.arange(max(0, M - 140), M)])        # the oracle's share
     ref = O.gemm_dequant(ac[rows], asb[rows], wc, wsb)
     out = {}
     for dt in (torch.float32, torch.bfloat16):
