@@ -651,15 +651,7 @@ static torq_status rotate_structured_impl(const void* X, const void* R_B, const 
     launch_tc(rotate_structured_kernel<FMT_MXFP4>, 1, grid, RotStructCfg::THREADS, RotStructCfg::SMEM_BYTES, s, tmRB,
               tmX3, static_cast<const __nv_bfloat16*>(R_intra), static_cast<uint8_t*>(out_codes),
               static_cast<uint8_t*>(out_scales), (int)M, (int)d, 0.0f, st->err_word);
-  if (launch_status() != TORQ_OK) return TORQ_ERR_LAUNCH;
-  const int64_t ns = fmt == FMT_NVFP4 ? 2 * nb : nb;     // scale bytes per row
-  const int64_t kc = (ns + 3) / 4 * 4, mpad = (M + 127) / 128 * 128;
-  const int64_t pad = (mpad - M) * kc + M * (kc - ns);
-  if (pad > 0) {
-    scale_padding_kernel<<<ew_grid(pad, 256, st->sm_count), 256, 0, s>>>(static_cast<uint8_t*>(out_scales), M, ns);
-    return launch_status();
-  }
-  return TORQ_OK;
+  return launch_status();
 }
 
 torq_status torq_rotate_quantize_structured(const void* X, const void* R_B, const void* R_intra, int64_t M,

@@ -133,3 +133,18 @@ def test_whole_layer_with_the_structured_rotation():
     # and the rotated-quantized layer approximates the unrotated full-precision one (identity chain)
     exact = O.decode_bf16(xb) @ w.astype(np.float64)
     assert np.linalg.norm(got - exact) / np.linalg.norm(exact) <= 0.25
+
+
+@pytest.mark.parametrize("M,d", [(593, 256), (1303, 256), (2, 4352), (301, 4352)])
+def test_one_two_and_several_tiles_per_block_of_threads(M, d):
+    """A tile is 4 tokens x 128 blocks, and the grid also zeroes the scale rows past the last token: one tile on every SM
+    and two on one, two and three on each, and a second block tile with only 8 of its 128 rows in use."""
+    g = np.random.default_rng(M + d)
+    nb = d // 32
+    xb = I.to_bf16_bits(g.integers(-8, 9, size=(M, d)).astype(np.float32))
+    PB = np.zeros((nb, nb), np.float32); PB[np.arange(nb), g.permutation(nb)] = 1
+    PK = np.zeros((32, 32), np.float32); PK[g.permutation(32), np.arange(32)] = 1
+    _run(xb, I.to_bf16_bits(PB), I.to_bf16_bits(PK), exact=True)      # every element, exactly
+    _run(xb, I.to_bf16_bits(PB), None, exact=True)
+    xr = I.activations(I.CONFIGS["tiny"], M=M, d=d)
+    _run(xr, I.to_bf16_bits(I.orthogonal(nb, g)), I.to_bf16_bits(I.orthogonal(32, g)))
