@@ -19,6 +19,13 @@
 //   R_intra (bf16, exact) as the N-major B tile.  Six small MMAs (M 128, N 32, K 16) per token.
 //   D2 has lanes = b', 32 columns per token: one thread reads one (token, block) row and runs Eq. 1.
 //
+// R_B stays in shared memory: the grid is a multiple of the number of 128-row block tiles, so all tiles of a CTA have the
+// same output blocks, and for d <= 14336 their 128 rows of R_B (at most 112 KiB) are loaded on the first tile only and X
+// alone goes through the ring.  Loaded again for every tile, the same lines were asked of the L2 by every SM at the same
+// time: 53.5 -> 41.7 us at 3000 tokens x 11008, 18.0 -> 16.4 us at 2000 x 8192; no difference at 4096 (14.0 us at 4096
+// tokens), where the epilogue and the tensor pipe's instruction minima (55 cycles for each of the 24 small MMAs of step 3)
+// bound a tile.
+//
 // Persistent, warp-specialised: warp 0 TMA producer, warp 1 issues the step-2 MMAs, warp 18 the step-3
 // MMAs, warps 2..17 epilogue in four groups of four (lane quarter w % 4; group (w - 2) / 4 owns that
 // token of the tile's four): read y from tensor memory, split it, write the terms back to tensor
@@ -41,8 +48,9 @@ struct RotStructCfg {
   static constexpr int B_BYTES = TOK * B_BOX_BYTES;    // 16 KiB
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;   // 32 KiB
   static constexpr int STAGES = 6;
+  static constexpr int RB_SLABS = 7;                   // 64-block column slabs of R_B that fit beside the ring: d <= 14336
   static constexpr int RI_BYTES = 32 * 64;             // R_intra, 64-byte swizzle
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + RI_BYTES + 256 + 1024;
+  static constexpr int SMEM_BYTES = RB_SLABS * A_BYTES + STAGES * B_BYTES + RI_BYTES + 256 + 1024;
   static constexpr int ACC2_COL = 2 * BN;              // D1 double-buffered in columns [0, 256); D2 in [256, 384)
   static constexpr int LO_COL = ACC2_COL + BN;         // third split term: 16 columns per token, [384, 448)
   static constexpr int TMEM_COLS = 512;
@@ -66,8 +74,9 @@ rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-  const uint32_t ri_base = smem_base + C::STAGES * C::STAGE_BYTES;
-  const uint32_t bar_off = C::STAGES * C::STAGE_BYTES + C::RI_BYTES;
+  const uint32_t x_base = smem_base + C::RB_SLABS * C::A_BYTES;      // ring of X; R_B lies before it
+  const uint32_t ri_base = x_base + C::STAGES * C::B_BYTES;
+  const uint32_t bar_off = C::RB_SLABS * C::A_BYTES + C::STAGES * C::B_BYTES + C::RI_BYTES;
   const uint32_t bar_base = smem_base + bar_off;
   // barrier map (8 bytes each)
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
@@ -86,6 +95,8 @@ rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_
   const int t_tiles = (M + C::TOK - 1) / C::TOK;
   const int total_tiles = b_tiles * t_tiles;
   const int k_tiles = (nblocks + C::BK - 1) / C::BK;
+  // A CTA whose tiles all have the same output blocks (the grid is a multiple of b_tiles then) keeps its rows of R_B.
+  const bool resident = k_tiles <= C::RB_SLABS && gridDim.x % b_tiles == 0;
   const int kb4 = (nblocks + 3) / 4;
   const bool intra = R_intra != nullptr;
 
@@ -116,13 +127,14 @@ rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_
         const int s = it % C::STAGES;
         if (!mbar_wait_warp(empty_bar(s), ((it / C::STAGES) & 1) ^ 1, cta_abort, err_word,
                             SITE_PRODUCER_EMPTY)) { ok = false; break; }
-        const uint32_t st = smem_base + s * C::STAGE_BYTES;
+        const uint32_t st = x_base + s * C::B_BYTES;
+        const bool load_rb = !resident || it < (uint32_t)k_tiles;      // resident: on the first tile only
         if (elect_one()) {
-          mbar_arrive_expect_tx(full_bar(s), C::STAGE_BYTES);
-          tma_load_2d(st, &tmRB, kt * C::BK, bt * C::BM, full_bar(s));
+          mbar_arrive_expect_tx(full_bar(s), C::B_BYTES + (load_rb ? C::A_BYTES : 0));
+          if (load_rb) tma_load_2d(smem_base + (resident ? kt : s) * C::A_BYTES, &tmRB, kt * C::BK, bt * C::BM, full_bar(s));
 #pragma unroll
           for (int j = 0; j < C::TOK; ++j)              // one token per box
-            tma_load_3d(st + C::A_BYTES + j * C::B_BOX_BYTES, &tmX3, 0, tg * C::TOK + j, kt * C::BK,
+            tma_load_3d(st + j * C::B_BOX_BYTES, &tmX3, 0, tg * C::TOK + j, kt * C::BK,
                         full_bar(s));
         }
         __syncwarp();
@@ -152,11 +164,10 @@ rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_
           ok = false; return;
         }
         tc_fence_after_sync();
-        const uint32_t st = smem_base + s * C::STAGE_BYTES;
-        const uint64_t adesc = make_desc(st, 16, 1024, kSwizzle128);
+        const uint64_t adesc = make_desc(smem_base + (resident ? kt : s) * C::A_BYTES, 16, 1024, kSwizzle128);
         // B: N-major, 64-byte swizzle: 32 n-elements (64 B) contiguous, k rows 64 B apart, 8-row
         // groups 512 B apart (stride offset), next 32 n-elements = next token's sub-tile (leading offset)
-        const uint64_t bdesc = make_desc(st + C::A_BYTES, C::B_BOX_BYTES, 512, kSwizzle64);
+        const uint64_t bdesc = make_desc(x_base + s * C::B_BYTES, C::B_BOX_BYTES, 512, kSwizzle64);
         if (elect_one()) {
 #pragma unroll
           for (int j = 0; j < C::BK / 16; ++j)          // 16 k-rows = 1 KiB; steps past the last block are skipped

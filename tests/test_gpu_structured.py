@@ -135,10 +135,11 @@ def test_whole_layer_with_the_structured_rotation():
     assert np.linalg.norm(got - exact) / np.linalg.norm(exact) <= 0.25
 
 
-@pytest.mark.parametrize("M,d", [(593, 256), (1303, 256), (2, 4352), (301, 4352)])
+@pytest.mark.parametrize("M,d", [(593, 256), (1303, 256), (2, 4352), (301, 4352), (9, 14336), (5, 14592)])
 def test_one_two_and_several_tiles_per_block_of_threads(M, d):
     """A tile is 4 tokens x 128 blocks, and the grid also zeroes the scale rows past the last token: one tile on every SM
-    and two on one, two and three on each, and a second block tile with only 8 of its 128 rows in use."""
+    and two on one, two and three on each, a second block tile with only 8 of its 128 rows in use,
+    and the last width whose rows of R_B stay in shared memory and the first whose rows do not."""
     g = np.random.default_rng(M + d)
     nb = d // 32
     xb = I.to_bf16_bits(g.integers(-8, 9, size=(M, d)).astype(np.float32))
