@@ -30,6 +30,7 @@
 // the chunk's 4-byte cells.
 #pragma once
 #include <cuda_bf16.h>
+#include <type_traits>
 #include "sm100_ptx.cuh"
 
 namespace torq {
@@ -88,6 +89,9 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
   const int total_tiles = tiles.total;
   const int k_tiles = (K + C::BK - 1) / C::BK;
   const int kb4 = K / (C::BK / CH);                    // scale chunks per row
+  // From 8 stages on a tile's output boxes are spread over the next tile and its first scale chunks go out before the
+  // accumulator is free.  8192 tokens x 14336 features, K = 4096: 181.7 -> 172.5 us, K = 2048 107.5 -> 103.8; K = 1024 lost 3 %.
+  const bool long_k = k_tiles >= 8;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
@@ -197,15 +201,12 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         // The W scales of rows 32 j .. 32 j + 31 of a 128-row chunk sit in column j of the chunk's four
         // columns: a tile that starts 64 rows into its first chunk reads them from two columns further on.
         const uint32_t sfb_m = sfb_t + ((tcol & 127) ? 2u : 0u);
-        if (!mbar_wait_cluster_warp(acce_bar, (tcount & 1) ^ 1, cta_abort, err_word, SITE_MMA_ACC_EMPTY)) {
-          ok = false; break;
-        }
-        tc_fence_after_sync();
-        for (int kt = 0; kt < k_tiles; ++kt, ++it) {
+        // One stage: the scale chunks go to tensor memory, then the instructions.  The first stage of every tile but the
+        // CTA pair's first waits between the two until the epilogue has read the accumulator.
+        auto stage = [&](int kt, auto waits) -> bool {
+          constexpr bool WAITS = decltype(waits)::value;
           const int s = it % C::STAGES;
-          if (!mbar_wait_cluster_warp(full_bar(s), (it / C::STAGES) & 1, cta_abort, err_word, SITE_MMA_FULL)) {
-            ok = false; break;
-          }
+          if (!mbar_wait_cluster_warp(full_bar(s), (it / C::STAGES) & 1, cta_abort, err_word, SITE_MMA_FULL)) return false;
           tc_fence_after_sync();
           const bool two = (kb4 - CH * kt) >= CH;          // K % 256 == 128: the last stage is half
           const uint32_t st = smem_base + s * C::STAGE_BYTES;
@@ -213,7 +214,7 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
           const uint64_t bdesc = make_desc(st + C::A_BYTES, 16, 1024, kSwizzle128);
           const uint64_t sfa_d = make_desc(st + C::A_BYTES + C::B_BYTES, 0, 128, 0);
           const uint64_t sfb_d = make_desc(st + C::A_BYTES + C::B_BYTES + C::SFA_BYTES, 0, 128, 0);
-          if (elect_one()) {
+          auto copy_scales = [&]() {
             // scale chunks shared -> tensor memory (descriptor address unit = 16 B: +32 = next
             // chunk, + SFA_BYTES / 16 = second 128-row tile of W), then 64 elements of K per instruction
 #pragma unroll
@@ -224,6 +225,15 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                 tmem_cp_32x128b_warpx4_pair(sfb_t + 8 * c + 4, sfb_d + 32 * c + C::SFA_BYTES / 16);
               }
             }
+          };
+          if constexpr (WAITS) {
+            if (elect_one()) copy_scales();
+            __syncwarp();
+            if (!mbar_wait_cluster_warp(acce_bar, (tcount - 1) & 1, cta_abort, err_word, SITE_MMA_ACC_EMPTY)) return false;
+            tc_fence_after_sync();
+          }
+          if (elect_one()) {
+            if constexpr (!WAITS) copy_scales();
             if constexpr (FMT == FMT_MXINT4) {             // a quarter chunk (one scale byte) per instruction
               mma_mxf8_pair(tmem_base, adesc, bdesc, idesc_mxf8(256, BN, 0) - nsub, sfa_t, sfb_m, kt != 0);
               mma_mxf8_pair(tmem_base, adesc + 2, bdesc + 2, idesc_mxf8(256, BN, 1) - nsub, sfa_t, sfb_m, 1);
@@ -246,7 +256,18 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             tc_commit_pair(empty_bar(s), 3);
           }
           __syncwarp();
+          ++it;
+          return true;
+        };
+        int kt = 0;
+        if (tcount > 0 && long_k) {
+          ok = stage(0, std::true_type{});
+          kt = 1;
+        } else if (tcount > 0) {
+          ok = mbar_wait_cluster_warp(acce_bar, (tcount - 1) & 1, cta_abort, err_word, SITE_MMA_ACC_EMPTY);
+          tc_fence_after_sync();
         }
+        for (; kt < k_tiles && ok; ++kt) ok = stage(kt, std::false_type{});
         if (ok && elect_one()) tc_commit_pair(accf_bar, 3);
         __syncwarp();
       }
@@ -304,7 +325,13 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(lo), __uint_as_float(hi));
         return *reinterpret_cast<uint32_t*>(&hh);
       };
+      // With another tile behind this one the 16 or 32 boxes of a CTA go out one by one over three quarters of that tile's
+      // instructions (512 cycles per stage): all at once they hold up its loads.
+      const int box_gap = long_k && tile + npairs < total_tiles ? k_tiles * (y_is_bf16 ? 24 : 12) : 0;
+      long long box_time = clock64() + (warp - 2) * box_gap;
       auto flush = [&](int col) {                        // whole warp
+        while (clock64() < box_time) __nanosleep(40);
+        box_time += 8 * box_gap;
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0 && row0 < M && col < N) {

@@ -172,3 +172,25 @@ def test_gemm_nvfp4_and_mxint4():
     ref = O.gemm_mxint4(aq, asb, wq, wsb)
     got = TI._gpu_gemm(aq, asb, wq, wsb, torch.float32)
     assert np.linalg.norm(got - ref) / np.linalg.norm(ref) <= 1e-5
+
+
+@pytest.mark.parametrize("fmt,M,N,K", [("mxfp4", 2500, 2048, 1792), ("mxfp4", 2500, 2048, 1920), ("mxfp4", 2500, 6152, 2048),
+                                       ("nvfp4", 2500, 2048, 1920), ("mxint4", 2500, 2048, 896), ("mxint4", 2500, 2048, 1024)])
+def test_gemm_from_eight_stages_on_paces_the_output_and_starts_the_scales_early(fmt, M, N, K):
+    """Seven and eight stages of 256 (MXINT4: 128) elements, the eighth a half one, with two to four tiles per CTA pair."""
+    if fmt == "mxfp4":
+        ac, asb = _rand_operand(M, K, 1)
+        wc, wsb = _rand_operand(N, K, 2)
+        run, ref = lambda dt: _gpu_gemm(ac, asb, wc, wsb, dt), O.gemm_dequant(ac, asb, wc, wsb)
+    elif fmt == "nvfp4":
+        ac, asb = TN._rand_operand(M, K, 1)
+        wc, wsb = TN._rand_operand(N, K, 2)
+        ats, wts = np.float32(0.013), np.float32(2.5e-4)
+        run, ref = lambda dt: TN._gpu_gemm(ac, asb, ats, wc, wsb, wts, dt), O.gemm_nvfp4(ac, asb, ats, wc, wsb, wts)
+    else:
+        ac, asb = TI._rand_operand(M, K, 3)
+        wc, wsb = TI._rand_operand(N, K, 4)
+        run, ref = lambda dt: TI._gpu_gemm(ac, asb, wc, wsb, dt), O.gemm_mxint4(ac, asb, wc, wsb)
+    got = run(torch.float32)
+    assert np.linalg.norm(got - ref) / np.linalg.norm(ref) <= 1e-5      # the bound of the shorter contractions above
+    assert np.array_equal(run(torch.bfloat16), O.round_to_bf16(got))
