@@ -8,7 +8,7 @@
 //   B = X tile [tokens x 64 (i)], K-major
 // A layer has only d / 128 feature tiles (40 at d = 5120), too few CTAs to pull R_inter at HBM rate,
 // so the contraction is also split: a CLUSTER of S CTAs shares one feature tile, CTA r of the cluster
-// contracts k range r.  The fp32 partial tiles never leave the SMs: token group g (16 tokens) belongs to CTA g % S
+// contracts k range r.  The fp32 partial tiles never leave the SMs: token group g (8 or 16 tokens) belongs to CTA g % S
 // (its owner), which adds the S partials in rank order (fixed order, so the result does not depend on timing), applies
 // the intra-block rotation on the warp-level tensor cores (y split into three bf16 terms, fp32 accumulation) and
 // quantizes (Eq. 1).  The partials reach the owner in one of two ways:
@@ -103,7 +103,11 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   const int k_tiles = d / C::BK;
   const int kt0 = (int)((long long)k_tiles * rank / S), kt1 = (int)((long long)k_tiles * (rank + 1) / S);
   const uint32_t tmem_cols = ntok <= 32 ? 32u : (ntok <= 64 ? 64u : (ntok <= 128 ? 128u : 256u));
-  const int groups = (M + 15) / 16;                      // token groups; group g belongs to CTA g % S
+  // Token groups; group g belongs to CTA g % S.  Groups of 8 up to 32 tokens, where that leaves no CTA more than one: a
+  // group of 16 takes its partials in two round trips through the cluster (24 tokens: d = 4096 10.0 -> 9.5 us, d = 2048
+  // 5.95 -> 5.7).  At 40 tokens the whole layer gains at d = 4096 (1 %) and loses at 2048 (1 %), at 48 it loses.
+  const int gtok = !PUSH && M <= 32 && (M + 7) / 8 <= S ? 8 : 16;
+  const int groups = (M + gtok - 1) / gtok;
 
   // R_inter is a constant of the layer, never the output of the kernel that runs just before this
   // one: the thread that initialises the barriers sends the loads of the first stages' R_inter tiles
@@ -215,11 +219,12 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
       IntraFrag f;
       if (R_intra != nullptr) load_intra_frag(r_lane, r_lane + 32, 16 * 80, f);
       uint32_t sb[2];
-      intra_quantize_frag16<FMT, true>(y, R_intra != nullptr, f, lane, 16 * g, live ? M : 0, blk, nblocks, d, nvs, codes, sb);
+      intra_quantize_frag16<FMT, true>(y, R_intra != nullptr, f, lane, gtok * g, live ? min(M, gtok * (g + 1)) : 0, blk, nblocks, d, nvs, codes, sb);
       if (p == 0 && live) {
 #pragma unroll
         for (int rh = 0; rh < 2; ++rh) {                 // rows of the group past the last token: zero
-          const int row = 16 * g + r8 + 8 * rh;
+          if (8 * rh >= gtok) break;
+          const int row = gtok * g + r8 + 8 * rh;
           const uint32_t b = row < M ? sb[rh] : 0u;
           if constexpr (FMT == FMT_NVFP4) *reinterpret_cast<uint16_t*>(scales + scale_offset(row, 2 * blk, kb4)) = (uint16_t)b;
           else scales[scale_offset(row, blk, kb4)] = (uint8_t)b;
@@ -318,11 +323,11 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
         for (; g < groups; g += S * ESETS) {
 #pragma unroll
           for (int jh = 0; jh < 2; ++jh) {
-            if (16 * g + 8 * jh >= M) break;             // rows 8 jh .. 8 jh + 7 of the group hold no token
+            if (8 * jh >= gtok || gtok * g + 8 * jh >= M) break;      // rows 8 jh .. 8 jh + 7 of the group hold no token
             float4 part[2][C::MAX_CLUSTER];
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-              const uint32_t off = (uint32_t)(((16 * g + tr + 4 * (2 * jh + j)) * C::BF + q * 32 + fc) * 4);
+              const uint32_t off = (uint32_t)(((gtok * g + tr + 4 * (2 * jh + j)) * C::BF + q * 32 + fc) * 4);
 #pragma unroll
               for (int s = 0; s < C::MAX_CLUSTER; ++s)
                 if (s < S)
@@ -358,7 +363,7 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
     // scale bytes of the rows no group covers, up to the last row of the 128-row scale tiles: zero
     if (rank == 0 && es == 0) {
       for (int row = q * 32 + lane; row < (M > 128 ? 256 : 128); row += 128) {
-        if (row >= 16 * groups) {
+        if (row >= gtok * groups) {
           uint8_t* cell = scales + (size_t)(row >> 7) * kb4 * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4;
           if constexpr (FMT == FMT_NVFP4) {
             *reinterpret_cast<uint32_t*>(cell + (size_t)(2 * ft) * 512) = 0u;

@@ -12,6 +12,8 @@ import oracle as O
 from helpers import dev_bf16, dev_u8, gpu_quantized_to_numpy, lattice, mismatch_report
 from paper_2605_19561_b200 import inputs as I
 from paper_2605_19561_b200 import torq
+import test_gpu_mxint4 as TI
+import test_gpu_nvfp4 as TN
 
 pytestmark = pytest.mark.gpu
 
@@ -69,6 +71,19 @@ def test_rotation_cluster_sizes(M, d):
                                  (112, 4096), (144, 2176), (145, 4096), (208, 3072), (241, 2176), (12, 12288)])
 def test_rotation_token_steps(M, d):
     test_rotation_alone_without_any_workspace(M, d)
+
+
+# 17 to 32 tokens on clusters that give every group of 8 a CTA of its own, and sizes on the other side of that rule
+@pytest.mark.parametrize("M,d", [(17, 1536), (24, 4096), (25, 4096), (33, 2560), (40, 1536), (41, 1536), (18, 256)])
+def test_rotation_token_groups_of_eight(M, d):
+    test_rotation_alone_without_any_workspace(M, d)
+    g = np.random.default_rng(M + d)
+    xb = I.to_bf16_bits(g.integers(-8, 9, size=(M, d)).astype(np.float64))
+    P = np.zeros((d, d))
+    P[np.arange(d), g.permutation(d)] = 1.0
+    pb = I.to_bf16_bits(P)
+    TN._rotate_case(xb, pb, None, exact=True)
+    TI._rotate_case(xb, pb, None, exact=True)
 
 
 def test_rotation_exact_cases_are_bit_exact():
