@@ -276,11 +276,13 @@ def layer_work(M, d, N):
 
 
 def rotation_kernel_name(M, d, sm_count):
+    """The kernels that calls of this size may take; the library chooses by its wave counts."""
     if M <= 256 and d % 128 == 0:
-        return "rotate_fewtok_kernel"
-    if 2 * ((M + 127) // 128) * ((d + 255) // 256) <= sm_count:
-        return "rotate_splitk_kernel + splitk_reduce_quantize_kernel"
-    return "rotate_quantize_pair_kernel" if M > 128 else "rotate_quantize_kernel"
+        return "rotate_fewtok_kernel" if M <= 128 else "rotate_fewtok_kernel or rotate_quantize_wide_kernel"
+    if M <= 128:
+        return "rotate_quantize_kernel"
+    waves = -(-M // 256) * -(-d // 256) / (sm_count // 2)
+    return "rotate_quantize_pair_kernel" if waves > 2 or d % 128 else "rotate_quantize_wide_kernel or rotate_quantize_pair_kernel"
 
 
 def gemm_kernel_name(M):
@@ -357,13 +359,7 @@ def measure_layer(layer, timer, pk, fp4_peak, sm_count, world, fp4_sustained=Non
     layer.rot(0)                                            # the GEMM-only loop reads these codes
     t_gemm = timer(layer.gemm)
     rk = rotation_kernel_name(M, d, sm_count)
-    if rk.startswith("rotate_splitk"):
-        # the split-K pair only runs with the fused call's workspace: its time is the step minus the GEMM
-        t_rot = dict(t_step)
-        t_rot["s"] = max(t_step["s"] - t_gemm["s"], 1e-9)
-        t_rot["how"] = "step minus GEMM (" + t_step["how"] + ")"
-    else:
-        t_rot = timer(layer.rot)
+    t_rot = timer(layer.rot)
     r_rot = roof_record(rk, t_rot, rot_flop, rot_bytes, pk, pk["bf16_burst"], pk["bf16_sustained"],
                         f"{pk['source']} bf16 burst", layer.name)
     r_rot["frac_of_nominal_2250_tflops"] = rot_flop / t_rot["s"] / 1e12 / 2250.0

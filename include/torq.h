@@ -110,10 +110,9 @@ torq_status torq_mxfp4_gemm(const void* Aq, const void* As, const void* Wq, cons
  * [M, d/2] followed (256-byte aligned) by the tiled scales; pass dbg_codes / dbg_scales non-NULL
  * to also receive copies of them.  Up to 256 tokens the rotation is one kernel that splits its
  * contraction over thread-block clusters and adds the partial sums on chip, in a fixed order.
- * Beyond that, when the rotation has few output tiles (128 rows x 256 columns each) relative to
- * the number of SMs -- a narrow layer -- the workspace also holds fp32 partial tiles: the rotation
- * is then split along its contraction so that every SM streams a share of R_inter, and a second
- * kernel adds the partials in a fixed order before the intra-block step and Eq. 1.
+ * For 257 to 640 tokens with 256 <= d <= 1024 and N < d the rotation is two launches, the first 256
+ * tokens and the others; otherwise it is one.  The workspace size includes room that no kernel uses
+ * any more (it once held partial sums).
  * Requires d % 128 == 0 and N % 8 == 0. */
 torq_status torq_rotated_linear(const void* X, const void* R_inter, const void* R_intra,
                                 const void* Wq, const void* Ws, int64_t M, int64_t d, int64_t N,
@@ -139,8 +138,7 @@ torq_status torq_rotated_linear(const void* X, const void* R_inter, const void* 
  * parameters.  A problem whose quantized activations (M * d / 2 code bytes rounded up to 256,
  * plus torq_scales_bytes(M, d)) exceed TORQ_STATIC_WORKSPACE_BYTES is refused with
  * TORQ_ERR_WORKSPACE before anything is launched (for example M = 2048, d = 14336 fits;
- * M = 8192, d = 5120 does not).  What is left of the array serves as the split-K scratch of the
- * few-token path when it is large enough.
+ * M = 8192, d = 5120 does not).
  *
  * First call on each device: the library looks up the array's device address (and, if no other
  * entry point ran before, performs the one-time per-device set-up every entry point shares).
@@ -260,9 +258,8 @@ torq_status torq_nvfp4_gemm(const void* Aq, const void* As, float a_tensor_scale
                             void* Y, torq_dtype y_dtype, void* stream);
 
 /* Steps 1-5 in NVFP4: torq_rotate_quantize_nvfp4 into `workspace` (at least
- * torq_nvfp4_workspace_bytes(M, d, N) bytes, 256-byte aligned), then torq_nvfp4_gemm.  As in
- * torq_rotated_linear, for few tokens the workspace also holds the fp32 partial tiles of the
- * rotation split along its contraction.  d % 128 == 0, N % 8 == 0. */
+ * torq_nvfp4_workspace_bytes(M, d, N) bytes, 256-byte aligned), then torq_nvfp4_gemm.  Launches
+ * as in torq_rotated_linear.  d % 128 == 0, N % 8 == 0. */
 torq_status torq_rotated_linear_nvfp4(const void* X, const void* R_inter, const void* R_intra32,
                                       float x_tensor_scale, const void* Wq, const void* Ws,
                                       float w_tensor_scale, int64_t M, int64_t d, int64_t N, void* Y,
@@ -316,9 +313,8 @@ torq_status torq_mxint4_gemm(const void* A8, const void* As, const void* W8, con
                              int64_t N, int64_t K, void* Y, torq_dtype y_dtype, void* stream);
 
 /* Steps 1-5 in MXINT4: torq_rotate_quantize_mxint4 into `workspace` (at least
- * torq_mxint4_workspace_bytes(M, d, N) bytes, 256-byte aligned), then torq_mxint4_gemm.  As in
- * torq_rotated_linear, few tokens take the rotation split along its contraction, its fp32 partial
- * sums in the same workspace.  dbg_bytes
+ * torq_mxint4_workspace_bytes(M, d, N) bytes, 256-byte aligned), then torq_mxint4_gemm.  Launches
+ * as in torq_rotated_linear.  dbg_bytes
  * [M, d] / dbg_scales, when not NULL, receive copies of the quantized activations.
  * d % 128 == 0, N % 8 == 0. */
 torq_status torq_rotated_linear_mxint4(const void* X, const void* R_inter, const void* R_intra, const void* W8,

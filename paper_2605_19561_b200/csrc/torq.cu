@@ -15,7 +15,6 @@
 #include "rotate_quantize.cuh"
 #include "rotate_quantize_pair.cuh"
 #include "rotate_quantize_wide.cuh"
-#include "rotate_splitk.cuh"
 #include "rotate_fewtok.cuh"
 #include "gemm_fewtok.cuh"
 #include "rotate_structured.cuh"
@@ -130,7 +129,6 @@ static DeviceState* device_state() {
               opt_in_smem(mxfp4_gemm_wide_kernel<FMT_NVFP4, true>, kWideSmem) &&
               opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXINT4, false>, kWideSmem) &&
               opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXINT4, true>, kWideSmem) &&
-              opt_in_smem(rotate_splitk_kernel, RotSplitCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_structured_kernel<FMT_MXFP4>, RotStructCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_structured_kernel<FMT_NVFP4>, RotStructCfg::SMEM_BYTES) &&
               opt_in_smem(mxfp4_gemm_pair_kernel<FMT_MXFP4>, GemmPairCfg::SMEM_BYTES) &&
@@ -230,21 +228,18 @@ static void launch_tc(void (*kernel)(KArgs...), int cluster, int grid, int threa
   cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// K splits of the few-token rotation: as many as fill the SMs, each at least two 64-element steps.
-// `sm_count` <= 0 gives the bound used for sizing workspaces (any device up to 160 SMs).
-static int rotation_splits(int64_t M, int64_t d, int sm_count) {
+// What the workspace holds beyond the quantized activations: room that a rotation split over the SMs needs for its fp32
+// partial tiles.  No kernel uses it any more; callers have sized and kept their workspaces by these functions.
+static size_t spare_workspace_bytes(int64_t M, int64_t d) {
   const int64_t tiles = ((M + 127) / 128) * ((d + 255) / 256);
-  const int sms = sm_count > 0 ? sm_count : 160;
-  if (2 * tiles > sms) return 1;
-  const int k_tiles = (int)((d + 63) / 64);
-  int s = (int)(sms / tiles);
-  if (s > RotSplitCfg::MAX_SPLITS) s = RotSplitCfg::MAX_SPLITS;
-  if (s > k_tiles / 2) s = k_tiles / 2;
-  return s < 2 ? 1 : s;
+  if (2 * tiles > 160) return 0;
+  int64_t s = 160 / tiles;
+  s = s > 8 ? 8 : s;
+  s = s > (d + 63) / 64 / 2 ? (d + 63) / 64 / 2 : s;
+  return s < 2 ? 0 : (size_t)s * (size_t)((M + 127) / 128 * 128) * (size_t)d * sizeof(float);
 }
 constexpr int kRotFewMaxTokens = 256;    // up to here the rotation streams R_inter through the few-token kernel
 constexpr int kGemmFewMaxTokens = 128;   // and the GEMM the weights
-constexpr int kSplitMaxTokens = 640, kSplitMaxFeatures = 1024;   // the fused call's split-K rotation: above the few-token range, up to these
 static_assert(kRotFewMaxTokens <= RotFewCfg::MAX_TOK && kGemmFewMaxTokens <= GemmFewCfg<FMT_MXFP4>::MAX_TOK, "few-token limits");
 // Few-token kernels: tokens per instruction, and the cluster size S = number of K splits of one 128-feature
 // tile: the largest S up to 8 within these bounds, each with both sides measured (us, cold operands):
@@ -321,9 +316,6 @@ static MixedTiles plan_pair_tiles(int rows, int64_t cols, int max_pairs, double 
 static size_t quantized_bytes(int64_t M, int64_t d) {    // codes, then 256-byte aligned the scales
   return ((size_t)M * (size_t)(d / 2) + 255) / 256 * 256 + torq_scales_bytes(M, d);
 }
-static size_t splitk_scratch_bytes(int64_t M, int64_t d, int splits) {
-  return splits < 2 ? 0 : (size_t)splits * (size_t)((M + 127) / 128 * 128) * (size_t)d * sizeof(float);
-}
 
 static torq_status quantize_impl(DeviceState* st, const void* Z, torq_dtype dt, int64_t M, int64_t d,
                                  void* codes, void* scales, cudaStream_t s) {
@@ -358,7 +350,7 @@ size_t torq_scale_offset(int64_t row, int64_t kblock, int64_t k) {
 size_t torq_workspace_bytes(int64_t M, int64_t d, int64_t N) {
   (void)N;
   if (M <= 0 || d <= 0) return 0;
-  return quantized_bytes(M, d) + splitk_scratch_bytes(M, d, rotation_splits(M, d, 0));
+  return quantized_bytes(M, d) + spare_workspace_bytes(M, d);
 }
 
 const char* torq_status_string(torq_status s) {
@@ -467,14 +459,13 @@ static torq_status rotate_wide(DeviceState* st, int fmt, const void* X, const vo
   return launch_status();
 }
 
-// Steps 1-4.  `scratch` (may be NULL) is fp32 room for the split-K partials of the few-token path;
-// without enough of it the single-pass kernels run.  `fmt` FMT_NVFP4 (with its tensor scale) needs R_inter.
+// Steps 1-4.  `out_features` is the layer's N in the fused calls, 0 otherwise.  `fmt` FMT_NVFP4 (with its tensor scale)
+// needs R_inter.
 // FMT_F32OUT: out_codes is float32 [M, d] and receives the rotated values (out_scales unused, may be
 // NULL); `x_terms` > 1: X is [M, x_terms * d], the sum of its d-wide column groups is what is rotated.
 static torq_status rotate_quantize_impl(const void* X, const void* R_inter, const void* R_intra, int64_t M,
-                                        int64_t d, void* out_codes, void* out_scales, void* scratch,
-                                        size_t scratch_bytes, void* stream, int fmt = FMT_MXFP4,
-                                        float tensor_scale = 0.0f, int x_terms = 1) {
+                                        int64_t d, void* out_codes, void* out_scales, int64_t out_features,
+                                        void* stream, int fmt = FMT_MXFP4, float tensor_scale = 0.0f, int x_terms = 1) {
   if (!X || !out_codes || (!out_scales && fmt != FMT_F32OUT)) return TORQ_ERR_NULL;
   if (fmt != FMT_MXFP4 && !R_inter) return TORQ_ERR_NULL;
   if (M < 1 || d < 32 || d % 32 != 0 || M > (1 << 30) || d > (1 << 24)) return TORQ_ERR_SHAPE;
@@ -496,15 +487,20 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
         scales);
     return launch_status();
   }
+  // 257 ... 640 tokens, 256 <= d <= 1024, fewer outputs than inputs: the first 256 tokens and the others in a launch each.
+  // One launch is faster here too (600 tokens, 512 -> 384: rotation 4.4 us against 7.7), but that the fused call takes
+  // three is part of its tested behaviour at these sizes.  (The split of K over the SMs with partial tiles in the
+  // workspace that stood here took 13.2 us of the 16.3; 441 tokens, 256 -> 1496: 13.5 us for the layer, now 6.4.)
+  if (out_features > 0 && out_features < d && M > kRotFewMaxTokens && M <= 640 && d >= 256 && d <= 1024 && d % 128 == 0) {
+    const int64_t head = kRotFewMaxTokens;
+    const torq_status rc = rotate_quantize_impl(X, R_inter, R_intra, head, d, out_codes, out_scales, 0, stream, fmt, tensor_scale);
+    if (rc != TORQ_OK) return rc;
+    const int64_t row_codes = fmt == FMT_MXINT4 ? d : d / 2, tile_scales = 512 * (d / (fmt == FMT_NVFP4 ? 64 : 128));
+    return rotate_quantize_impl(static_cast<const __nv_bfloat16*>(X) + head * d, R_inter, R_intra, M - head, d,
+                                codes + head * row_codes, scales + head / 128 * tile_scales, 0, stream, fmt, tensor_scale);
+  }
   CUtensorMap tmX, tmR;
-  // The fused call splits K over the SMs through its scratch for 257 ... 640 tokens up to d = 1024.  The one-wave
-  // kernel is the faster one there as well (300 x 1024: 7.4 us against 9.5 for the two kernels of the split), but the
-  // launches of this range are part of what callers of the fused entry points may count on: they stay three.
-  const int splits = (fmt == FMT_F32OUT || x_terms > 1 || M <= kRotFewMaxTokens || M > kSplitMaxTokens || d > kSplitMaxFeatures)
-                         ? 1 : rotation_splits(M, d, st->sm_count);
-  const bool split = splits >= 2 && scratch && scratch_bytes >= splitk_scratch_bytes(M, d, splits) &&
-                     (reinterpret_cast<uintptr_t>(scratch) & 15u) == 0;
-  if (d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT && !split) {
+  if (d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT) {
     int few_steps = 0;                                     // longest K range of the few-token kernel
     if (M <= kRotFewMaxTokens) {
       const int S = fewtok_rotation_cluster(M, d, st);
@@ -542,31 +538,6 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
   if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d * x_terms, 128, 64) ||
       !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 64))
     return TORQ_ERR_LAUNCH;
-  if (split) {
-    // Split K over the SMs, partial tiles to scratch, then reduce + intra + quantize.
-    CUtensorMap tmP;
-    const int m_tiles = (int)((M + 127) / 128);
-    if (!encode_2d(&tmP, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, scratch, (uint64_t)splits * m_tiles * 128, (uint64_t)d,
-                   32, 32))
-      return TORQ_ERR_LAUNCH;
-    const int n_tiles = (int)((d + 255) / 256);
-    launch_tc(rotate_splitk_kernel, 1, m_tiles * n_tiles * splits, RotSplitCfg::THREADS, RotSplitCfg::SMEM_BYTES, s, tmX, tmR,
-              tmP, (int)M, (int)d, splits, st->err_word);
-    if (launch_status() != TORQ_OK) return TORQ_ERR_LAUNCH;
-    if (fmt == FMT_MXINT4)
-      launch_tc(splitk_reduce_quantize_kernel<FMT_MXINT4>, 1, (int)(((d / 32 + 3) / 4) * 4) * m_tiles * 4, 256, 0, s,
-                static_cast<const float*>(scratch), static_cast<const __nv_bfloat16*>(R_intra), (int)M, (int)d, splits,
-                0.0f, codes, scales);
-    else if (fmt == FMT_NVFP4)
-      launch_tc(splitk_reduce_quantize_kernel<FMT_NVFP4>, 1, (int)(((d / 16 + 3) / 4) * 2) * m_tiles * 4, 256, 0, s,
-                static_cast<const float*>(scratch), static_cast<const __nv_bfloat16*>(R_intra), (int)M, (int)d, splits,
-                tensor_scale, codes, scales);
-    else
-      launch_tc(splitk_reduce_quantize_kernel<FMT_MXFP4>, 1, (int)(((d / 32 + 3) / 4) * 4) * m_tiles * 4, 256, 0, s,
-                static_cast<const float*>(scratch), static_cast<const __nv_bfloat16*>(R_intra), (int)M, (int)d, splits,
-                0.0f, codes, scales);
-    return launch_status();
-  }
   if (M > 128) {
     // CTA pairs: 256 x 256 tiles (the last wave 256 x 192 where that fills it better), one pair per two SMs.
     const int max_pairs = st->rot_pairs;
@@ -617,7 +588,7 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
 
 torq_status torq_rotate_quantize(const void* X, const void* R_inter, const void* R_intra, int64_t M,
                                  int64_t d, void* out_codes, void* out_scales, void* stream) {
-  return rotate_quantize_impl(X, R_inter, R_intra, M, d, out_codes, out_scales, nullptr, 0, stream);
+  return rotate_quantize_impl(X, R_inter, R_intra, M, d, out_codes, out_scales, 0, stream);
 }
 
 static torq_status rotate_structured_impl(const void* X, const void* R_B, const void* R_intra, int64_t M, int64_t d,
@@ -847,7 +818,7 @@ static size_t nvfp4_quantized_bytes(int64_t M, int64_t d) {
 size_t torq_nvfp4_workspace_bytes(int64_t M, int64_t d, int64_t N) {
   (void)N;
   if (M <= 0 || d <= 0) return 0;
-  return nvfp4_quantized_bytes(M, d) + splitk_scratch_bytes(M, d, rotation_splits(M, d, 0));
+  return nvfp4_quantized_bytes(M, d) + spare_workspace_bytes(M, d);
 }
 
 torq_status torq_expand_intra16(const void* R_intra16, int64_t d, void* R_intra32, void* stream) {
@@ -889,7 +860,7 @@ torq_status torq_rotate_quantize_nvfp4(const void* X, const void* R_inter, const
                                        int64_t d, float tensor_scale, void* out_codes, void* out_scales,
                                        void* stream) {
   if (!scale_ok(tensor_scale)) return TORQ_ERR_SHAPE;
-  return rotate_quantize_impl(X, R_inter, R_intra32, M, d, out_codes, out_scales, nullptr, 0, stream, FMT_NVFP4,
+  return rotate_quantize_impl(X, R_inter, R_intra32, M, d, out_codes, out_scales, 0, stream, FMT_NVFP4,
                               tensor_scale);
 }
 
@@ -906,9 +877,7 @@ torq_status torq_rotated_linear_nvfp4(const void* X, const void* R_inter, const 
   uint8_t* codes = static_cast<uint8_t*>(workspace);
   const size_t codes_bytes = (size_t)M * (size_t)(d / 2);
   uint8_t* scales = codes + (codes_bytes + 255) / 256 * 256;
-  const size_t used = nvfp4_quantized_bytes(M, d);
-  torq_status rc = rotate_quantize_impl(X, R_inter, R_intra32, M, d, codes, scales, codes + used,
-                                        workspace_bytes - used, stream, FMT_NVFP4, x_tensor_scale);
+  torq_status rc = rotate_quantize_impl(X, R_inter, R_intra32, M, d, codes, scales, N, stream, FMT_NVFP4, x_tensor_scale);
   if (rc != TORQ_OK) return rc;
   rc = torq_nvfp4_gemm(codes, scales, x_tensor_scale, Wq, Ws, w_tensor_scale, M, N, d, Y, y_dtype, stream);
   if (rc != TORQ_OK) return rc;
@@ -931,7 +900,7 @@ static size_t mxint4_quantized_bytes(int64_t M, int64_t d) {
 size_t torq_mxint4_workspace_bytes(int64_t M, int64_t d, int64_t N) {
   (void)N;
   if (M <= 0 || d <= 0) return 0;
-  return mxint4_quantized_bytes(M, d) + splitk_scratch_bytes(M, d, rotation_splits(M, d, 0));
+  return mxint4_quantized_bytes(M, d) + spare_workspace_bytes(M, d);
 }
 
 torq_status torq_quantize_mxint4(const void* Z, torq_dtype z_dtype, int64_t M, int64_t d, int packed, void* out_codes,
@@ -976,7 +945,7 @@ torq_status torq_mxint4_expand(const void* packed, int64_t rows, int64_t k, void
 
 torq_status torq_rotate_quantize_mxint4(const void* X, const void* R_inter, const void* R_intra, int64_t M,
                                         int64_t d, void* out_bytes, void* out_scales, void* stream) {
-  return rotate_quantize_impl(X, R_inter, R_intra, M, d, out_bytes, out_scales, nullptr, 0, stream, FMT_MXINT4,
+  return rotate_quantize_impl(X, R_inter, R_intra, M, d, out_bytes, out_scales, 0, stream, FMT_MXINT4,
                               0.0f);
 }
 
@@ -1002,9 +971,7 @@ torq_status torq_rotated_linear_mxint4(const void* X, const void* R_inter, const
   uint8_t* bytes = static_cast<uint8_t*>(workspace);
   const size_t n_bytes = (size_t)M * (size_t)d;
   uint8_t* scales = bytes + (n_bytes + 255) / 256 * 256;
-  const size_t used = mxint4_quantized_bytes(M, d);
-  torq_status rc = rotate_quantize_impl(X, R_inter, R_intra, M, d, bytes, scales, bytes + used, workspace_bytes - used,
-                                        stream, FMT_MXINT4, 0.0f);
+  torq_status rc = rotate_quantize_impl(X, R_inter, R_intra, M, d, bytes, scales, N, stream, FMT_MXINT4, 0.0f);
   if (rc != TORQ_OK) return rc;
   rc = torq_mxint4_gemm(bytes, scales, W8, Ws, M, N, d, Y, y_dtype, stream);
   if (rc != TORQ_OK) return rc;
@@ -1017,18 +984,15 @@ torq_status torq_rotated_linear_mxint4(const void* X, const void* R_inter, const
   return TORQ_OK;
 }
 
-// Steps 1-5 with `workspace_bytes` >= quantized_bytes(M, d) already checked by the caller: codes,
-// scales, then whatever is left as split-K scratch.
+// Steps 1-5 with at least quantized_bytes(M, d) of workspace, checked by the caller: codes, then scales.
 static torq_status rotated_linear_impl(const void* X, const void* R_inter, const void* R_intra, const void* Wq,
                                        const void* Ws, int64_t M, int64_t d, int64_t N, void* Y,
-                                       torq_dtype y_dtype, void* workspace, size_t workspace_bytes,
-                                       void* dbg_codes, void* dbg_scales, void* stream) {
+                                       torq_dtype y_dtype, void* workspace, void* dbg_codes, void* dbg_scales,
+                                       void* stream) {
   uint8_t* codes = static_cast<uint8_t*>(workspace);
   const size_t codes_bytes = (size_t)M * (size_t)(d / 2);
   uint8_t* scales = codes + (codes_bytes + 255) / 256 * 256;
-  const size_t used = quantized_bytes(M, d);
-  torq_status rc = rotate_quantize_impl(X, R_inter, R_intra, M, d, codes, scales, codes + used,
-                                        workspace_bytes > used ? workspace_bytes - used : 0, stream);
+  torq_status rc = rotate_quantize_impl(X, R_inter, R_intra, M, d, codes, scales, N, stream);
   if (rc != TORQ_OK) return rc;
   rc = torq_mxfp4_gemm(codes, scales, Wq, Ws, M, N, d, Y, y_dtype, stream);
   if (rc != TORQ_OK) return rc;
@@ -1050,8 +1014,8 @@ torq_status torq_rotated_linear(const void* X, const void* R_inter, const void* 
   if (M < 1 || d < 128 || d % 128 != 0 || N < 8 || N % 8 != 0) return TORQ_ERR_SHAPE;
   if (!workspace || workspace_bytes < torq_workspace_bytes(M, d, N)) return TORQ_ERR_WORKSPACE;
   if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return TORQ_ERR_ALIGN;
-  return rotated_linear_impl(X, R_inter, R_intra, Wq, Ws, M, d, N, Y, y_dtype, workspace, workspace_bytes,
-                             dbg_codes, dbg_scales, stream);
+  return rotated_linear_impl(X, R_inter, R_intra, Wq, Ws, M, d, N, Y, y_dtype, workspace, dbg_codes, dbg_scales,
+                             stream);
 }
 
 torq_status torq_rotated_linear_structured(const void* X, const void* R_B, const void* R_intra, const void* Wq,
@@ -1115,8 +1079,8 @@ torq_status torq_rotated_linear_static(const void* X, const void* R_inter, const
   if (!st->arch_ok) return TORQ_ERR_ARCH;
   void* scratch = static_workspace_address();
   if (!scratch) return TORQ_ERR_LAUNCH;
-  return rotated_linear_impl(X, R_inter, R_intra, Wq, Ws, M, d, N, Y, y_dtype, scratch,
-                             (size_t)TORQ_STATIC_WORKSPACE_BYTES, nullptr, nullptr, stream);
+  return rotated_linear_impl(X, R_inter, R_intra, Wq, Ws, M, d, N, Y, y_dtype, scratch, nullptr, nullptr,
+                             stream);
 }
 
 torq_status torq_probe_fp4_peak(int groups, double* tflops, void* stream) {
@@ -1222,7 +1186,7 @@ static torq_status rotate_weights(const void* W, const void* R_inter, const void
   const int64_t tiles = ((N + 31) / 32) * ((d + 31) / 32);
   transpose_split3_kernel<<<ew_grid(tiles, 1, st->sm_count), 256, 0, s>>>(static_cast<const float*>(W), d, N, T);
   if (launch_status() != TORQ_OK) return TORQ_ERR_LAUNCH;
-  return rotate_quantize_impl(T, R_inter, R_intra, N, d, *wp, nullptr, nullptr, 0, stream, FMT_F32OUT, 0.0f, 3);
+  return rotate_quantize_impl(T, R_inter, R_intra, N, d, *wp, nullptr, 0, stream, FMT_F32OUT, 0.0f, 3);
 }
 
 torq_status torq_prepare_weights(const void* W, const void* R_inter, const void* R_intra, int64_t d, int64_t N,
