@@ -717,12 +717,17 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
   constexpr int BN = 256;
   const uint64_t krow = (uint64_t)(FMT == FMT_MXINT4 ? K : K / 2);   // operand bytes per row
   CUtensorMap tmA, tmB;
-  if (M <= kGemmFewMaxTokens) {
+  using FC = GemmFewCfg<FMT>;
+  const int ntok = M <= kGemmFewMaxTokens ? fewtok_ntok(M) : 0;
+  const int tiles = (int)((N + 127) / 128);
+  // More tiles than CTAs that fit: every further wave of few-token CTAs starts with empty stages.  From 49 tokens on the
+  // persistent pair kernels do better, half empty as their rows are (us, few-token against pairs: 100 tokens K = 4096,
+  // N = 20480 20.4 / 12.9, N = 28672 21.4 / 16.3, N = 14336 10.9 / 11.1; 64 tokens, two CTAs per SM: K = 2048, N = 40960
+  // 15.3 / 12.9, K = 4096, N = 28672 14.4 / 16.0; 40 tokens K = 5120, N = 51200 29.7 / 30.1).
+  const bool many_waves = ntok > 48 && (int64_t)tiles > (int64_t)FC::ctas_per_sm(ntok) * st->sm_count;
+  if (ntok > 0 && !many_waves) {
     // Few tokens: 128 output features x all tokens per CTA, K split over a cluster, reduced through
     // distributed shared memory.
-    using FC = GemmFewCfg<FMT>;
-    const int ntok = fewtok_ntok(M);
-    const int tiles = (int)((N + 127) / 128);
     const int64_t steps = (K + FC::BK - 1) / FC::BK;
     const int S = fewtok_cluster(tiles, steps, 3, FC::ctas_per_sm(ntok), st->sm_count, st->few_fit);
     const int width = M > FC::MAX_PUSH_TOK ? wide_gemm_width(M, N, steps, false, S, st->gemm_pairs) : 0;
@@ -777,8 +782,8 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
   if (!encode_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Aq, (uint64_t)M, krow, 128, 128) ||
       !encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, bn, 128))
     return TORQ_ERR_LAUNCH;
-  const int tiles = (int)((M + 127) / 128) * (int)((N + bn - 1) / bn);
-  const int grid = tiles < st->sm_count ? tiles : st->sm_count;
+  const int out_tiles = (int)((M + 127) / 128) * (int)((N + bn - 1) / bn);
+  const int grid = out_tiles < st->sm_count ? out_tiles : st->sm_count;
   if (narrow)
     launch_tc(mxfp4_gemm_kernel<128, 2, FMT>, 1, grid, GemmCfg<128, 2, FMT>::THREADS, GemmCfg<128, 2, FMT>::SMEM_BYTES,
               s, tmA, tmB, static_cast<const uint8_t*>(As), static_cast<const uint8_t*>(Ws), Y,

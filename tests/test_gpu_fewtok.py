@@ -156,6 +156,13 @@ def test_gemm_token_steps(M, N, K):
     test_gemm_random_operands(M, N, K)
 
 
+# more 128-feature tiles than CTAs that fit (one per SM above 64 tokens, two up to there), and the last sizes that fit
+@pytest.mark.parametrize("M,N,K", [(65, 18952, 384), (65, 18944, 384), (128, 20480, 256), (100, 28424, 640), (64, 37896, 256),
+                                   (49, 37896, 384), (48, 37896, 256)])
+def test_gemm_more_tiles_than_fit_at_once(M, N, K):
+    test_gemm_random_operands(M, N, K)
+
+
 def test_gemm_exact_integer_regime_and_one_hot_rows():
     """Equal scales: fp32 accumulation is exact in any order and through the split, so the result is the
     oracle's bit for bit.  One-hot activation rows return single dequantized weight columns: a mix-up of
