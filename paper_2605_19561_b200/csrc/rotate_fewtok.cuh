@@ -47,9 +47,9 @@ struct RotFewCfg {
   static constexpr int A_BYTES = BK * BF * 2;          // 16 KiB: two boxes of 64 (k) x 64 (j)
   static constexpr int A_BOX_BYTES = 64 * 64 * 2;
   static constexpr int STAGES = 4;
-  // the same for every token count: three stages at 128 tokens would let two CTAs share an SM (clusters of 5
-  // instead of 3), which measured 4 - 10 % slower than four stages and one CTA per SM
-  __host__ __device__ static constexpr int stages(int) { return STAGES; }
+  // With three stages two CTAs of 65 to 128 tokens share an SM: for long K ranges, where one CTA per SM leaves SMs without
+  // a CTA and too few loads in flight (the rule stands where the kernel is launched).
+  static constexpr int SHARED_STAGES = 3, MAX_SHARED_TOK = 128;
   static constexpr int MAX_TOK = 256;                  // N of the instruction: a multiple of 16
   static constexpr int MAX_PUSH_TOK = 16;              // one token group
   static constexpr int PART_BYTES = BF * 16 * 4;       // pushed partial of the group from one CTA: [4][feature][4 tokens]
@@ -59,23 +59,28 @@ struct RotFewCfg {
   static constexpr int THREADS = 192;
   static constexpr int MAX_CLUSTER = 8;
   __host__ __device__ static constexpr int stage_bytes(int ntok) { return A_BYTES + ntok * BK * 2; }
-  __host__ __device__ static constexpr int smem_bytes(int ntok) {
-    return stages(ntok) * stage_bytes(ntok) + BAR_BYTES + 4 * RI_BYTES + 1024;
+  __host__ __device__ static constexpr int smem_bytes(int ntok, int stages = STAGES) {
+    return stages * stage_bytes(ntok) + BAR_BYTES + 4 * RI_BYTES + 1024;
   }
-  __host__ __device__ static constexpr int ctas_per_sm(int ntok) { return smem_bytes(ntok) <= 113 * 1024 ? 2 : 1; }
+  __host__ __device__ static constexpr int ctas_per_sm(int ntok, int stages = STAGES) {
+    return smem_bytes(ntok, stages) <= 113 * 1024 ? 2 : 1;
+  }
   __host__ __device__ static constexpr int max_smem_bytes() { return smem_bytes(MAX_TOK); }
 };
 // what lies in the stages after the mainloop: S pushed partials, or the partial tile (ntok x 512 B) and the y tiles
 static_assert(RotFewCfg::MAX_CLUSTER * RotFewCfg::PART_BYTES <= RotFewCfg::STAGES * RotFewCfg::stage_bytes(16) &&
               8 * RotFewCfg::Y_BYTES <= 4 * RotFewCfg::A_BYTES && RotFewCfg::BF * 4 <= RotFewCfg::STAGES * RotFewCfg::BK * 2, "reduction buffers");
+static_assert(RotFewCfg::ctas_per_sm(RotFewCfg::MAX_SHARED_TOK, RotFewCfg::SHARED_STAGES) == 2 &&
+              4 * RotFewCfg::Y_BYTES + 80 * RotFewCfg::BF * 4 <= RotFewCfg::SHARED_STAGES * RotFewCfg::stage_bytes(80) &&
+              4 * RotFewCfg::Y_BYTES + 128 * RotFewCfg::BF * 4 <= RotFewCfg::SHARED_STAGES * RotFewCfg::stage_bytes(128), "three stages");
 
 // grid = (d / 128) * S CTAs in clusters of S along x: CTA b works feature tile b / S, k split b % S.
 // tmX: X [M, d] bf16, box [ntok rows x 64]; tmR: R_inter [d, d] bf16, box [64 x 64].  ntok = M rounded up to
 // a multiple of 16.  d % 128 == 0.  `codes` / `scales` / `tensor_scale` as in rotate_quantize_kernel for FMT.
-// ESETS: sets of four epilogue warps (threads = 64 + 128 ESETS).  One set and two CTAs per SM up to 64
-// tokens; with more a CTA fills an SM by itself and has several token groups to reduce, rotate
-// and quantize, each a dependent chain of about a microsecond for one warp: two sets take them in turn.
-template <int FMT = FMT_MXFP4, int ESETS = 1, bool PUSH = false>
+// ESETS: sets of four epilogue warps (threads = 64 + 128 ESETS).  One set where two CTAs share an SM; a CTA that fills an SM
+// by itself has several token groups to reduce, rotate and quantize, each a dependent chain of about a microsecond for
+// one warp: two sets take them in turn.  NST: stages.
+template <int FMT = FMT_MXFP4, int ESETS = 1, bool PUSH = false, int NST = RotFewCfg::STAGES>
 __global__ void __launch_bounds__(64 + 128 * ESETS, ESETS == 1 ? 2 : 1)
 rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,
                      const __nv_bfloat16* __restrict__ R_intra, uint8_t* __restrict__ codes,
@@ -86,7 +91,7 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
   const int stage_bytes = C::stage_bytes(ntok);
-  const int nst = C::stages(ntok);
+  constexpr int nst = NST;
   const uint32_t bar_off = nst * stage_bytes;
   const uint32_t bar_base = smem_base + bar_off;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };

@@ -139,11 +139,14 @@ static DeviceState* device_state() {
               opt_in_smem(rotate_quantize_kernel<256, FMT_MXINT4>, RotCfg<256>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_MXINT4>, RotPairCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_structured_kernel<FMT_MXINT4>, RotStructCfg::SMEM_BYTES) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 2>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 2>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 2>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 1, true>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) && opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 1>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) &&
               opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 2>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) &&
@@ -263,9 +266,19 @@ static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int long_k, int
   while (s > 1 && (k_steps + s - 2) / (s - 1) == (k_steps + s - 1) / s) --s;      // fewer clusters' CTAs: they fit as well
   return s < 1 ? 1 : s;
 }
-static int fewtok_rotation_cluster(int64_t M, int64_t d, const DeviceState* st) {
+// Cluster size and stages of the few-token rotation.  65 to 128 tokens have an SM to themselves with four stages and share
+// it with three.  Sharing wins where the K range of a CTA would be longer than 32 steps, that is where 148 CTAs are few for
+// the tiles (us, alone / shared, 72 and 128 tokens: d = 5120, 27 steps 14.2 / 14.7 and 16.2 / 17.7; d = 6400, 50 steps 21.7 /
+// 19.9 and 23.4 / 22.0; d = 8192 28.0 / 26.4 and 30.3 / 28.0; d = 11008, one CTA for each of 86 tiles 52.0 / 41.1 and 53.6 /
+// 44.4; d = 14336 78 / 68 and 79 / 73).
+struct FewRotation { int cluster, stages; };
+static FewRotation fewtok_rotation(int64_t M, int64_t d, const DeviceState* st) {
   const int ntok = fewtok_ntok(M);
-  return fewtok_cluster(d / 128, d / 64, ntok > 128 ? 1 : 10, RotFewCfg::ctas_per_sm(ntok), st->sm_count, st->few_fit);
+  const int64_t tiles = d / 128, steps = d / 64;
+  const int long_k = ntok > 128 ? 1 : 10, ctas = RotFewCfg::ctas_per_sm(ntok);
+  const int S = fewtok_cluster(tiles, steps, long_k, ctas, st->sm_count, st->few_fit);
+  if (ctas > 1 || ntok > RotFewCfg::MAX_SHARED_TOK || steps <= 32 * S) return {S, RotFewCfg::STAGES};
+  return {fewtok_cluster(tiles, steps, long_k, 2, st->sm_count, st->few_fit), RotFewCfg::SHARED_STAGES};
 }
 constexpr double kNarrowTileCost = 0.88;   // a 192-column tile against a 256-column one: 0.75 of the math, 0.875 of the operand bytes
 
@@ -412,8 +425,9 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 // sides are low by as much); f = filled part of a wave:
 //  * here: 1.6 + 0.022 per column (2 + 0.032 above 256 columns) for launch and epilogue, then per K step the operand
 //    bytes, 0.17 + 0.0003 per column + 0.03 f, or the math, 0.00114 per column;
-//  * few tokens: 3.1 / 4.4 / 5.6 / 8.3 up to 16 / 64 / 128 / 256 tokens, plus 0.22 / 0.2 / 0.36 / 0.42 per K step of
-//    the longest split;
+//  * few tokens: 3.1 / 4.4 / 5.6 / 7.6 / 10.5 up to 16 / 64 / 128 / 192 / 256 tokens, plus 0.22 / 0.2 / 0.36 / 0.42 / 0.42
+//    per K step of the longest split (192 and 256 tokens measured: d = 2560 10.9 and 13.6, here 11.5; d = 3072 13.1 and 15.4,
+//    here 13.4; d = 8192 33.5 and 37.4, here 35.1 and 35.8);
 //  * pair kernel: 6.8, plus per K step 0.32 for a wave and 0.2 + 0.14 f for the last, partly filled one.
 // A layer of 2048 tokens and more fills the pair kernel's waves and stays there (one-wave tiles would be wider than
 // 384 columns; 2048 x 4096 measured 51.6 with 480 columns, 46.8 in the pair kernel).
@@ -430,7 +444,7 @@ static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int max_pair
   }
   double other;
   if (M <= kRotFewMaxTokens) {
-    other = M <= 16 ? 3.1 + 0.22 * few_steps : (M <= 64 ? 4.4 + 0.2 * few_steps : (M <= 128 ? 5.6 + 0.36 * few_steps : 8.3 + 0.42 * few_steps));
+    other = M <= 16 ? 3.1 + 0.22 * few_steps : (M <= 64 ? 4.4 + 0.2 * few_steps : (M <= 128 ? 5.6 + 0.36 * few_steps : (M <= 192 ? 7.6 : 10.5) + 0.42 * few_steps));
   } else {
     const int64_t tiles = rows * ((d + 255) / 256);
     const int64_t full = tiles / max_pairs, rest = tiles % max_pairs;
@@ -503,7 +517,7 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
   if (d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT) {
     int few_steps = 0;                                     // longest K range of the few-token kernel
     if (M <= kRotFewMaxTokens) {
-      const int S = fewtok_rotation_cluster(M, d, st);
+      const int S = fewtok_rotation(M, d, st).cluster;
       few_steps = (int)((d / 64 + S - 1) / S);
     }
     const int width = wide_rotation_width(M, d, few_steps, st->rot_pairs);
@@ -514,25 +528,30 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
     // distributed shared memory; one launch, no scratch.
     const int ntok = fewtok_ntok(M);
     const int tiles = (int)(d / 128);
-    const int S = fewtok_rotation_cluster(M, d, st);
+    const FewRotation few = fewtok_rotation(M, d, st);
+    const int S = few.cluster;
     if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d, (uint32_t)ntok, 64) ||
         !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 64))
       return TORQ_ERR_LAUNCH;
-    const int smem = RotFewCfg::smem_bytes(ntok);
+    const int smem = RotFewCfg::smem_bytes(ntok, few.stages);
     const float ts = fmt == FMT_NVFP4 ? tensor_scale : 0.0f;
     const __nv_bfloat16* ri = static_cast<const __nv_bfloat16*>(R_intra);
-    // up to 16 tokens: partials pushed to one CTA; up to 64: one set of epilogue warps, two CTAs per SM; more: two sets
-    auto launch = [&](auto push, auto one, auto two) {
-      const bool small = RotFewCfg::ctas_per_sm(ntok) >= 2;
-      launch_tc(ntok <= RotFewCfg::MAX_PUSH_TOK ? push : (small ? one : two), S, tiles * S, small ? 192 : 320, smem, s, tmX, tmR, ri,
-                codes, scales, (int)M, (int)d, ntok, S, ts, st->err_word);
+    // up to 16 tokens: partials pushed to one CTA; two CTAs per SM: one set of epilogue warps; one CTA: two sets
+    auto launch = [&](auto push, auto one, auto shared, auto two) {
+      const bool share = few.stages != RotFewCfg::STAGES, small = share || RotFewCfg::ctas_per_sm(ntok) >= 2;
+      launch_tc(ntok <= RotFewCfg::MAX_PUSH_TOK ? push : (share ? shared : (small ? one : two)), S, tiles * S, small ? 192 : 320, smem, s,
+                tmX, tmR, ri, codes, scales, (int)M, (int)d, ntok, S, ts, st->err_word);
     };
+    constexpr int NS = RotFewCfg::SHARED_STAGES;
     if (fmt == FMT_MXINT4)
-      launch(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, rotate_fewtok_kernel<FMT_MXINT4, 1>, rotate_fewtok_kernel<FMT_MXINT4, 2>);
+      launch(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, rotate_fewtok_kernel<FMT_MXINT4, 1>, rotate_fewtok_kernel<FMT_MXINT4, 1, false, NS>,
+             rotate_fewtok_kernel<FMT_MXINT4, 2>);
     else if (fmt == FMT_NVFP4)
-      launch(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, rotate_fewtok_kernel<FMT_NVFP4, 1>, rotate_fewtok_kernel<FMT_NVFP4, 2>);
+      launch(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, rotate_fewtok_kernel<FMT_NVFP4, 1>, rotate_fewtok_kernel<FMT_NVFP4, 1, false, NS>,
+             rotate_fewtok_kernel<FMT_NVFP4, 2>);
     else
-      launch(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, rotate_fewtok_kernel<FMT_MXFP4, 1>, rotate_fewtok_kernel<FMT_MXFP4, 2>);
+      launch(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, rotate_fewtok_kernel<FMT_MXFP4, 1>, rotate_fewtok_kernel<FMT_MXFP4, 1, false, NS>,
+             rotate_fewtok_kernel<FMT_MXFP4, 2>);
     return launch_status();
   }
   if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d * x_terms, 128, 64) ||

@@ -86,6 +86,36 @@ def test_rotation_token_groups_of_eight(M, d):
     TI._rotate_case(xb, pb, None, exact=True)
 
 
+# 65 to 128 tokens on long K ranges: three stages and two CTAs per SM; d = 5120 and 64 tokens stay as they were
+@pytest.mark.parametrize("M,d", [(65, 6400), (128, 6272), (100, 9600)])
+def test_rotation_two_ctas_share_an_sm(M, d):
+    g = np.random.default_rng(M + d)
+    xb = I.to_bf16_bits(g.standard_t(3.0, size=(M, d)))
+    perm = g.permutation(d)                                  # a rotation by one element of each row: sums of one product
+    R = torch.zeros((d, d), dtype=torch.bfloat16, device="cuda")
+    R[torch.arange(d), torch.from_numpy(perm)] = 1.0
+    ri = I.to_bf16_bits(I.orthogonal(32, g, batch=d // 32))
+    x = dev_bf16(xb)
+    for intra in (None, dev_bf16(ri)):
+        codes, scales = torq.torq_rotate_quantize(x, R, intra)
+        xp = torch.empty_like(x)
+        xp[:, torch.from_numpy(perm)] = x
+        y = xp.float() if intra is None else torch.einsum("mbk,bkj->mbj", xp.double().view(M, d // 32, 32), intra.double()).reshape(M, d).float()
+        torch.cuda.synchronize()
+        assert torq.torq_last_device_error() == 0
+        g_codes, g_sb = gpu_quantized_to_numpy(codes, scales, M, d)
+        o_codes, o_sb = O.quantize_mxfp4(y.cpu().numpy())
+        rep = mismatch_report(g_codes, g_sb, o_codes, o_sb)
+        assert rep["non_adjacent"] == 0 and rep["elem_mismatch_frac"] <= (0 if intra is None else 1e-4), rep
+    # dense: the sum over K, against double precision
+    R = (torch.randn(d, d, generator=torch.Generator(device="cuda").manual_seed(d), device="cuda") / d ** 0.5).to(torch.bfloat16)
+    y = (x.double() @ R.double()).float()
+    codes, scales = torq.torq_rotate_quantize(x, R, None)
+    torch.cuda.synchronize()
+    rep = mismatch_report(*gpu_quantized_to_numpy(codes, scales, M, d), *O.quantize_mxfp4(y.cpu().numpy()))
+    assert rep["non_adjacent"] == 0 and rep["elem_mismatch_frac"] <= 1e-4 and rep["block_scale_mismatch_frac"] <= 1e-4, rep
+
+
 def test_rotation_exact_cases_are_bit_exact():
     """Permutation and identity rotations with integer activations: every partial sum is exact in any
     order, so codes and scales must equal the oracle's bit for bit through the split and the reduction."""
