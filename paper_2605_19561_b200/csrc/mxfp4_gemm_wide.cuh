@@ -44,7 +44,7 @@ struct GemmWideCfg {
     return (232448 - 2048) / stage_bytes(width) < MAX_STAGES ? (232448 - 2048) / stage_bytes(width) : MAX_STAGES;
   }
   __host__ __device__ static constexpr int smem_bytes(int width) { return stages(width) * stage_bytes(width) + 256 + 1024; }
-  static_assert(SF_COL + 4 * CH + 4 * CH * 4 <= 512, "tensor memory");       // up to four chunks of W scales
+  static_assert(SF_COL + 4 * CH + 4 * CH * 3 <= 512 && chunks(MAX_WIDTH) <= 3 && chunks(MAX_WIDTH - 64) <= 3, "up to three chunks of W scales");
 };
 
 // grid = 2 * rows * cols CTAs in clusters of two: pair p works row tile p % rows (256 tokens), column tile p / rows.
@@ -132,7 +132,10 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader only)
-    if (rank == 0 && elect_one()) {
+    // The whole warp runs the loop and an elected lane issues.  As a loop of one lane, with a loop over the scale chunks inside,
+    // issuing took longer than the instructions of a narrow tile: M = 512, N = 4096, K = 14336 23.4 -> 18.8 us, M = 200
+    // 19.1 -> 17.0, M = 200, N = 6144, K = 4096 8.45 -> 7.75.
+    if (rank == 0) {
       // instruction descriptors of the two widths differ only in the N field ([17,23) = N >> 3)
       const uint32_t less = (uint32_t)((256 - n0) >> 3) << 17;
       constexpr uint32_t less1 = (uint32_t)((256 - 128) >> 3) << 17;
@@ -146,7 +149,7 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       uint32_t ph = 0;
       bool ok = true;
       for (int kt = 0; kt < k_tiles; ++kt) {
-        ok = mbar_wait_cluster(full_bar(s), ph, cta_abort, err_word, SITE_MMA_FULL);
+        ok = mbar_wait_cluster_warp(full_bar(s), ph, cta_abort, err_word, SITE_MMA_FULL);
         if (!ok) break;
         tc_fence_after_sync();
         const bool two = FMT == FMT_MXINT4 || K - kt * C::BK > C::BK / 2;      // K % 256 == 128: the last stage is half
@@ -156,40 +159,45 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         const uint64_t b1desc = make_desc(st + C::A_BYTES + n0 / 2 * 128, 16, 1024, kSwizzle128);
         const uint64_t sfa_d = make_desc(st + sfa_off, 0, 128, 0);
         const uint64_t sfb_d = make_desc(st + sfb_off, 0, 128, 0);
-        // scale chunks shared -> tensor memory (descriptor address unit = 16 B)
+        if (elect_one()) {
+          // scale chunks shared -> tensor memory (descriptor address unit = 16 B)
 #pragma unroll
-        for (int c = 0; c < CH; ++c) {
-          if (CH == 1 || c < CH / 2 || two) {
-            tmem_cp_32x128b_warpx4_pair(sfa_t + 4 * c, sfa_d + 32 * c);
-            for (int t = 0; t < nchk; ++t)
-              tmem_cp_32x128b_warpx4_pair(sfb_t + c * sfb_c + 4 * t,
-                                          sfb_d + ((c >> 1) * nchk + t) * (C::SF_BOX_BYTES / 16) + 32 * (c & 1));
-          }
-        }
+          for (int c = 0; c < CH; ++c) {
+            if (CH == 1 || c < CH / 2 || two) {
+              tmem_cp_32x128b_warpx4_pair(sfa_t + 4 * c, sfa_d + 32 * c);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (j < 2 || two) {
-            const uint32_t accumulate = (kt | j) != 0;
-            if constexpr (FMT == FMT_MXINT4) {         // a quarter chunk (one scale byte) per instruction
-              mma_mxf8_pair(tmem_base, adesc + 2 * j, bdesc + 2 * j, idesc_mxf8(256, 256, j) - less, sfa_t, sfb_m, accumulate);
-              if constexpr (TWO)
-                mma_mxf8_pair(acc1, adesc + 2 * j, b1desc + 2 * j, idesc_mxf8(256, 256, j) - less1, sfa_t, sfb_m1, accumulate);
-            } else if constexpr (FMT == FMT_NVFP4) {   // one chunk per instruction
-              mma_nvf4_pair(tmem_base, adesc + 2 * j, bdesc + 2 * j, full_a - less, sfa_t + 4 * j, sfb_m + j * sfb_c, accumulate);
-              if constexpr (TWO)
-                mma_nvf4_pair(acc1, adesc + 2 * j, b1desc + 2 * j, full_a - less1, sfa_t + 4 * j, sfb_m1 + j * sfb_c, accumulate);
-            } else {                                   // half a chunk (two scale bytes) per instruction
-              const uint32_t id = (j & 1) ? full_b : full_a;
-              mma_mxf4_pair(tmem_base, adesc + 2 * j, bdesc + 2 * j, id - less, sfa_t + 4 * (j >> 1), sfb_m + (j >> 1) * sfb_c, accumulate);
-              if constexpr (TWO)
-                mma_mxf4_pair(acc1, adesc + 2 * j, b1desc + 2 * j, id - less1, sfa_t + 4 * (j >> 1), sfb_m1 + (j >> 1) * sfb_c, accumulate);
+              for (int t = 0; t < 3; ++t)
+                if (t < nchk)
+                  tmem_cp_32x128b_warpx4_pair(sfb_t + c * sfb_c + 4 * t,
+                                              sfb_d + ((c >> 1) * nchk + t) * (C::SF_BOX_BYTES / 16) + 32 * (c & 1));
             }
           }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (j < 2 || two) {
+              const uint32_t accumulate = (kt | j) != 0;
+              if constexpr (FMT == FMT_MXINT4) {         // a quarter chunk (one scale byte) per instruction
+                mma_mxf8_pair(tmem_base, adesc + 2 * j, bdesc + 2 * j, idesc_mxf8(256, 256, j) - less, sfa_t, sfb_m, accumulate);
+                if constexpr (TWO)
+                  mma_mxf8_pair(acc1, adesc + 2 * j, b1desc + 2 * j, idesc_mxf8(256, 256, j) - less1, sfa_t, sfb_m1, accumulate);
+              } else if constexpr (FMT == FMT_NVFP4) {   // one chunk per instruction
+                mma_nvf4_pair(tmem_base, adesc + 2 * j, bdesc + 2 * j, full_a - less, sfa_t + 4 * j, sfb_m + j * sfb_c, accumulate);
+                if constexpr (TWO)
+                  mma_nvf4_pair(acc1, adesc + 2 * j, b1desc + 2 * j, full_a - less1, sfa_t + 4 * j, sfb_m1 + j * sfb_c, accumulate);
+              } else {                                   // half a chunk (two scale bytes) per instruction
+                const uint32_t id = (j & 1) ? full_b : full_a;
+                mma_mxf4_pair(tmem_base, adesc + 2 * j, bdesc + 2 * j, id - less, sfa_t + 4 * (j >> 1), sfb_m + (j >> 1) * sfb_c, accumulate);
+                if constexpr (TWO)
+                  mma_mxf4_pair(acc1, adesc + 2 * j, b1desc + 2 * j, id - less1, sfa_t + 4 * (j >> 1), sfb_m1 + (j >> 1) * sfb_c, accumulate);
+              }
+            }
+          }
+          tc_commit_pair(empty_bar(s), 3);
         }
-        tc_commit_pair(empty_bar(s), 3);
+        __syncwarp();
         if (++s == nst) { s = 0; ph ^= 1; }
       }
-      if (ok) tc_commit_pair(accf_bar, 3);
+      if (ok && elect_one()) tc_commit_pair(accf_bar, 3);
     }
     __syncwarp();
   } else {

@@ -662,24 +662,25 @@ torq_status torq_rotate_quantize_structured_nvfp4(const void* X, const void* R_B
 
 // Width of the one-wave GEMM's tiles, or 0 where another kernel is faster.  Times in us, fitted to MXFP4 with bf16 output
 // at K = 128 ... 14336, N = 256 ... 12288, M = 17 ... 8000 (within 10 %); f = filled part of a wave:
-//  * here: 2 + 0.0062 per column + f for launch and epilogue, then per K step 0.265 or the math, 0.0011 per
-//    column, + 0.025 f;
+//  * here: 2 (1.8 / 1.5 up to 128 / 64 tokens) + 0.0062 per column + f for launch and epilogue, then per K step 0.24 or the
+//    math, 0.0011 per column, + 0.025 f;
 //  * few tokens (17 to 128, S CTAs per tile): 2.3 + 0.2 per K step of the longest split + per token 0.025 with S = 1 (the
 //    accumulator goes to Y), else 0.012 + 0.035 / S;
 //  * pair kernel: one wave 4.1 + 0.9 f + (0.285 + 0.04 f) per K step, more (the last one as narrower tiles) 5.2 + per K step
 //    0.325 for a full wave and 0.21 + 0.14 f for the last;
 //  * single CTAs (129 to 256 tokens, few column tiles): 3.2 + 1.3 f + 0.285 per K step.
-// Where it pays: 777 x 5120, K = 14336 (80 pair tiles) 35.1 -> 28.5, K = 4096 13.8 -> 12.3; 1280 x 4096, K = 14336 35.2 ->
-// 29.1; short contractions: 64 x 256, K = 256 3.9 -> 2.4; 100 x 4096, K = 512 5.0 -> 3.4; 2000 x 256, K = 1024 5.2 -> 3.9.
+// Where it pays: 777 x 5120, K = 14336 (80 pair tiles) 34.7 -> 27.3, K = 4096 13.1 -> 11.2; 1280 x 4096, K = 14336 34.6 ->
+// 27.8; short contractions: 40 x 4096, K = 512 4.0 -> 3.0; 100 x 4096, K = 512 5.1 -> 3.3; 3000 x 1024, K = 2048 7.1 -> 6.4.
 static int wide_gemm_width(int64_t M, int64_t N, int64_t steps, bool pairs, int few_S, int max_pairs) {
   const int64_t rows = (M + 255) / 256;
+  const double base = M <= 64 ? 1.5 : (M <= 128 ? 1.8 : 2.0);
   double best = 1e30;
   int width = 0;
   for (int w = 64; w <= GemmWideCfg<>::MAX_WIDTH; w += 64) {
     const int64_t tiles = rows * ((N + w - 1) / w);
     if (tiles > max_pairs) continue;
     const double f = (double)tiles / max_pairs, math = 0.0011 * w;
-    const double t = 2.0 + 0.0062 * w + f + (double)steps * ((math > 0.265 ? math : 0.265) + 0.025 * f);
+    const double t = base + 0.0062 * w + f + (double)steps * ((math > 0.24 ? math : 0.24) + 0.025 * f);
     if (t < best) { best = t; width = w; }
   }
   const int64_t tiles = rows * ((N + 255) / 256), full = tiles / max_pairs, rest = tiles % max_pairs;
