@@ -74,7 +74,7 @@ static_assert(RotFewCfg::ctas_per_sm(RotFewCfg::MAX_SHARED_TOK, RotFewCfg::SHARE
               4 * RotFewCfg::Y_BYTES + 80 * RotFewCfg::BF * 4 <= RotFewCfg::SHARED_STAGES * RotFewCfg::stage_bytes(80) &&
               4 * RotFewCfg::Y_BYTES + 128 * RotFewCfg::BF * 4 <= RotFewCfg::SHARED_STAGES * RotFewCfg::stage_bytes(128), "three stages");
 
-// grid = (d / 128) * S CTAs in clusters of S along x: CTA b works feature tile b / S, k split b % S.
+// grid = (d / 128 or fewer feature tiles) * S CTAs in clusters of S along x: CTA b works feature tile ft0 + b / S, k split b % S.
 // tmX: X [M, d] bf16, box [ntok rows x 64]; tmR: R_inter [d, d] bf16, box [64 x 64].  ntok = M rounded up to
 // a multiple of 16.  d % 128 == 0.  `codes` / `scales` / `tensor_scale` as in rotate_quantize_kernel for FMT.
 // ESETS: sets of four epilogue warps (threads = 64 + 128 ESETS).  One set where two CTAs share an SM; a CTA that fills an SM
@@ -84,8 +84,8 @@ template <int FMT = FMT_MXFP4, int ESETS = 1, bool PUSH = false, int NST = RotFe
 __global__ void __launch_bounds__(64 + 128 * ESETS, ESETS == 1 ? 2 : 1)
 rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,
                      const __nv_bfloat16* __restrict__ R_intra, uint8_t* __restrict__ codes,
-                     uint8_t* __restrict__ scales, int M, int d, int ntok, int S, float tensor_scale,
-                     int* err_word) {
+                     uint8_t* __restrict__ scales, int M, int d, int ntok, int S, int ft0,
+                     float tensor_scale, int* err_word) {
   using C = RotFewCfg;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -104,7 +104,7 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   uint8_t* ri_tiles = smem_gen + bar_off + C::BAR_BYTES;    // not part of the stages: filled at kernel start
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rank = blockIdx.x % S, ft = blockIdx.x / S;
+  const int rank = blockIdx.x % S, ft = ft0 + blockIdx.x / S;
   const int k_tiles = d / C::BK;
   const int kt0 = (int)((long long)k_tiles * rank / S), kt1 = (int)((long long)k_tiles * (rank + 1) / S);
   const uint32_t tmem_cols = ntok <= 32 ? 32u : (ntok <= 64 ? 64u : (ntok <= 128 ? 128u : 256u));

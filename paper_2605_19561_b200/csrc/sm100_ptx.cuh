@@ -504,7 +504,8 @@ __host__ __device__ __forceinline__ void pair_tile_coords(int tile, int mp_tiles
 // pair_tile_coords.  With narrow_b == 0 and rows_a == 0 this is pair_tile_coords itself.
 struct MixedTiles {
   int rows;        // 256-row tiles
-  int rows_a;      // row tiles [0, rows_a) have wide_b - 3 wide and narrow_b + 4 narrow tiles
+  int rows_a;      // row tiles [0, rows_a) have wide_b - less wide and narrow_b + 4 narrow tiles
+  int less;        // 3; or rows_a = 1 and the number of wide tiles that another kernel computes (no narrow ones then)
   int wide_b;      // 256-column tiles of the other row tiles
   int narrow_b;    // 192-column tiles of the other row tiles
   int total;       // tiles in all
@@ -515,6 +516,7 @@ __host__ __device__ __forceinline__ MixedTiles mixed_tiles_make(int rows, int wi
   MixedTiles t;
   t.rows = rows;
   t.rows_a = units % rows;
+  t.less = 3;
   t.wide_b = wide_cols - 3 * (units / rows);
   t.narrow_b = 4 * (units / rows);
   t.total = rows * wide_cols + units;
@@ -522,7 +524,7 @@ __host__ __device__ __forceinline__ MixedTiles mixed_tiles_make(int rows, int wi
 }
 
 __host__ __device__ __forceinline__ void mixed_tile_coords(int tile, const MixedTiles& t, int& mp, int& col0, bool& narrow) {
-  const int wide_common = t.rows_a > 0 ? t.wide_b - 3 : t.wide_b;
+  const int wide_common = t.rows_a > 0 ? t.wide_b - t.less : t.wide_b;
   int nt;
   const int n1 = t.rows * wide_common;
   if (tile < n1) {
@@ -533,7 +535,7 @@ __host__ __device__ __forceinline__ void mixed_tile_coords(int tile, const Mixed
   }
   tile -= n1;
   const int rows_b = t.rows - t.rows_a;
-  const int n2 = t.rows_a > 0 ? rows_b * 3 : 0;
+  const int n2 = t.rows_a > 0 ? rows_b * t.less : 0;
   if (tile < n2) {
     mp = t.rows_a + tile % rows_b;
     col0 = (wide_common + tile / rows_b) * 256;
@@ -550,7 +552,7 @@ __host__ __device__ __forceinline__ void mixed_tile_coords(int tile, const Mixed
     mp = tile % t.rows_a;
     nt = t.narrow_b + tile / t.rows_a;
   }
-  col0 = (mp < t.rows_a ? t.wide_b - 3 : t.wide_b) * 256 + nt * kNarrowCols;
+  col0 = (mp < t.rows_a ? t.wide_b - t.less : t.wide_b) * 256 + nt * kNarrowCols;
 }
 
 // Instruction descriptors (32-bit).  Common fields: [17,23) N>>3, [24,29) M>>4, bit 15 / 16 =

@@ -280,6 +280,7 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, const DeviceState* st) 
   if (ctas > 1 || ntok > RotFewCfg::MAX_SHARED_TOK || steps <= 32 * S) return {S, RotFewCfg::STAGES};
   return {fewtok_cluster(tiles, steps, long_k, 2, st->sm_count, st->few_fit), RotFewCfg::SHARED_STAGES};
 }
+constexpr int kTailTiles = 8;              // a last wave of up to so many tiles leaves the pair rotation (below)
 constexpr double kNarrowTileCost = 0.88;   // a 192-column tile against a 256-column one: 0.75 of the math, 0.875 of the operand bytes
 
 // Tile list of a pair kernel: `rows` 256-row tiles by `cols` columns on `max_pairs` CTA pairs, tiles dealt
@@ -473,6 +474,38 @@ static torq_status rotate_wide(DeviceState* st, int fmt, const void* X, const vo
   return launch_status();
 }
 
+// Few tokens: 128 features x all tokens per CTA, K split over a cluster, reduced through distributed shared memory; one
+// launch, no scratch.  Feature tiles [ft0, ft0 + tiles) of all d / 128.
+static torq_status rotate_fewtok(DeviceState* st, int fmt, const void* X, const void* R_inter, const void* R_intra, int64_t M,
+                                 int64_t d, int ft0, int tiles, FewRotation few, uint8_t* codes, uint8_t* scales,
+                                 float tensor_scale, cudaStream_t s) {
+  CUtensorMap tmX, tmR;
+  const int ntok = fewtok_ntok(M), S = few.cluster;
+  if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d, (uint32_t)ntok, 64) ||
+      !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 64))
+    return TORQ_ERR_LAUNCH;
+  const int smem = RotFewCfg::smem_bytes(ntok, few.stages);
+  const float ts = fmt == FMT_NVFP4 ? tensor_scale : 0.0f;
+  const __nv_bfloat16* ri = static_cast<const __nv_bfloat16*>(R_intra);
+  // up to 16 tokens: partials pushed to one CTA; two CTAs per SM: one set of epilogue warps; one CTA: two sets
+  auto launch = [&](auto push, auto one, auto shared, auto two) {
+    const bool share = few.stages != RotFewCfg::STAGES, small = share || RotFewCfg::ctas_per_sm(ntok) >= 2;
+    launch_tc(ntok <= RotFewCfg::MAX_PUSH_TOK ? push : (share ? shared : (small ? one : two)), S, tiles * S, small ? 192 : 320, smem, s,
+              tmX, tmR, ri, codes, scales, (int)M, (int)d, ntok, S, ft0, ts, st->err_word);
+  };
+  constexpr int NS = RotFewCfg::SHARED_STAGES;
+  if (fmt == FMT_MXINT4)
+    launch(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, rotate_fewtok_kernel<FMT_MXINT4, 1>, rotate_fewtok_kernel<FMT_MXINT4, 1, false, NS>,
+           rotate_fewtok_kernel<FMT_MXINT4, 2>);
+  else if (fmt == FMT_NVFP4)
+    launch(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, rotate_fewtok_kernel<FMT_NVFP4, 1>, rotate_fewtok_kernel<FMT_NVFP4, 1, false, NS>,
+           rotate_fewtok_kernel<FMT_NVFP4, 2>);
+  else
+    launch(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, rotate_fewtok_kernel<FMT_MXFP4, 1>, rotate_fewtok_kernel<FMT_MXFP4, 1, false, NS>,
+           rotate_fewtok_kernel<FMT_MXFP4, 2>);
+  return launch_status();
+}
+
 // Steps 1-4.  `out_features` is the layer's N in the fused calls, 0 otherwise.  `fmt` FMT_NVFP4 (with its tensor scale)
 // needs R_inter.
 // FMT_F32OUT: out_codes is float32 [M, d] and receives the rotated values (out_scales unused, may be
@@ -523,37 +556,8 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
     const int width = wide_rotation_width(M, d, few_steps, st->rot_pairs);
     if (width > 0) return rotate_wide(st, fmt, X, R_inter, R_intra, M, d, codes, scales, tensor_scale, width, s);
   }
-  if (M <= kRotFewMaxTokens && d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT) {
-    // Few tokens: 128 features x all tokens per CTA, K split over a cluster, reduced through
-    // distributed shared memory; one launch, no scratch.
-    const int ntok = fewtok_ntok(M);
-    const int tiles = (int)(d / 128);
-    const FewRotation few = fewtok_rotation(M, d, st);
-    const int S = few.cluster;
-    if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d, (uint32_t)ntok, 64) ||
-        !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 64))
-      return TORQ_ERR_LAUNCH;
-    const int smem = RotFewCfg::smem_bytes(ntok, few.stages);
-    const float ts = fmt == FMT_NVFP4 ? tensor_scale : 0.0f;
-    const __nv_bfloat16* ri = static_cast<const __nv_bfloat16*>(R_intra);
-    // up to 16 tokens: partials pushed to one CTA; two CTAs per SM: one set of epilogue warps; one CTA: two sets
-    auto launch = [&](auto push, auto one, auto shared, auto two) {
-      const bool share = few.stages != RotFewCfg::STAGES, small = share || RotFewCfg::ctas_per_sm(ntok) >= 2;
-      launch_tc(ntok <= RotFewCfg::MAX_PUSH_TOK ? push : (share ? shared : (small ? one : two)), S, tiles * S, small ? 192 : 320, smem, s,
-                tmX, tmR, ri, codes, scales, (int)M, (int)d, ntok, S, ts, st->err_word);
-    };
-    constexpr int NS = RotFewCfg::SHARED_STAGES;
-    if (fmt == FMT_MXINT4)
-      launch(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, rotate_fewtok_kernel<FMT_MXINT4, 1>, rotate_fewtok_kernel<FMT_MXINT4, 1, false, NS>,
-             rotate_fewtok_kernel<FMT_MXINT4, 2>);
-    else if (fmt == FMT_NVFP4)
-      launch(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, rotate_fewtok_kernel<FMT_NVFP4, 1>, rotate_fewtok_kernel<FMT_NVFP4, 1, false, NS>,
-             rotate_fewtok_kernel<FMT_NVFP4, 2>);
-    else
-      launch(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, rotate_fewtok_kernel<FMT_MXFP4, 1>, rotate_fewtok_kernel<FMT_MXFP4, 1, false, NS>,
-             rotate_fewtok_kernel<FMT_MXFP4, 2>);
-    return launch_status();
-  }
+  if (M <= kRotFewMaxTokens && d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT)
+    return rotate_fewtok(st, fmt, X, R_inter, R_intra, M, d, 0, (int)(d / 128), fewtok_rotation(M, d, st), codes, scales, tensor_scale, s);
   if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d * x_terms, 128, 64) ||
       !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 64))
     return TORQ_ERR_LAUNCH;
@@ -563,7 +567,22 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
     CUtensorMap tmRn;                                      // second half of a narrow tile's 96 columns per CTA
     if (!encode_2d(&tmRn, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 32))
       return TORQ_ERR_LAUNCH;
-    const MixedTiles tiles = plan_pair_tiles((int)((M + 255) / 256), d, max_pairs, kNarrowTileCost);
+    MixedTiles tiles = plan_pair_tiles((int)((M + 255) / 256), d, max_pairs, kNarrowTileCost);
+    // A last wave of a few tiles: the last `rest` column tiles of the first 256 tokens go to the few-token kernel instead, whose
+    // K split puts up to 8 CTAs on each 128 features.  That is worth its launch where a wave is long (us, one list of tiles /
+    // with this: 2048 x 14336 558 / 542 (the layer 724 / 703), 2048 x 4864 73.1 / 71.5, 2304 x 4352 66.2 / 65.5, 3584 x 4096
+    // 85.9 / 86.0, 3328 x 3072 51.7 / 52.6).
+    const int rest = (int)((M + 255) / 256 * (d / 256) % max_pairs), full = (int)((M + 255) / 256 * (d / 256) / max_pairs);
+    if (full >= 2 && rest > 0 && rest <= kTailTiles && rest <= d / 256 - 1 && d > 4096 && d % 256 == 0 && x_terms == 1 && fmt != FMT_F32OUT) {
+      tiles = mixed_tiles_make((int)((M + 255) / 256), (int)(d / 256), 0);
+      tiles.rows_a = 1;
+      tiles.less = rest;
+      tiles.total -= rest;
+      const int S = fewtok_cluster(2 * rest, d / 64, 1, 1, st->sm_count, st->few_fit);
+      const torq_status rc = rotate_fewtok(st, fmt, X, R_inter, R_intra, 256, d, (int)(d / 128) - 2 * rest, 2 * rest,
+                                           {S, RotFewCfg::STAGES}, codes, scales, tensor_scale, s);
+      if (rc != TORQ_OK) return rc;
+    }
     const int pairs = tiles.total < max_pairs ? tiles.total : max_pairs;
     if (fmt == FMT_MXINT4)
       launch_tc(rotate_quantize_pair_kernel<FMT_MXINT4>, 2, 2 * pairs, RotPairCfg::THREADS, RotPairCfg::SMEM_BYTES,

@@ -194,3 +194,37 @@ def test_gemm_from_eight_stages_on_paces_the_output_and_starts_the_scales_early(
     got = run(torch.float32)
     assert np.linalg.norm(got - ref) / np.linalg.norm(ref) <= 1e-5      # the bound of the shorter contractions above
     assert np.array_equal(run(torch.bfloat16), O.round_to_bf16(got))
+
+
+@pytest.mark.parametrize("M,d", [(2300, 4352), (2000, 4864), (4096, 4864)])
+def test_rotation_gives_a_short_last_wave_to_the_few_token_kernel(M, d):
+    """2 x 74 + 5, 2 x 74 + 4 and 4 x 74 + 8 tiles of 256 x 256: the last columns of the first 256 tokens come from the other
+    kernel.  Permutations: every element, scale byte and padding byte exactly."""
+    if _pairs() == 74:
+        assert (M + 255) // 256 * (d // 256) % 74 in (4, 5, 8)
+    g = np.random.default_rng(M)
+    xb = I.to_bf16_bits(g.integers(-8, 9, size=(M, d)).astype(np.float64))
+    P = np.zeros((d, d), np.float32)
+    perm = g.permutation(d)
+    P[np.arange(d), perm] = 1.0
+    pin = np.stack([np.eye(32, dtype=np.float32)[g.permutation(32)] for _ in range(d // 32)])
+    x = O.decode_bf16(xb)
+    y = np.empty_like(x)
+    y[:, perm] = x
+    z = np.einsum("mbk,bkj->mbj", y.reshape(M, d // 32, 32), pin.astype(np.float64)).reshape(M, d)
+    R, Ri = dev_bf16(I.to_bf16_bits(P)), dev_bf16(I.to_bf16_bits(pin))
+    codes_t = torch.full((M, d // 2), 0xEE, dtype=torch.uint8, device="cuda")
+    scales_t = torch.full((torq.torq_scales_bytes(M, d),), 0xEE, dtype=torch.uint8, device="cuda")
+    before = torq.torq_launch_count()
+    torq.torq_rotate_quantize(dev_bf16(xb), R, Ri, out_codes=codes_t, out_scales=scales_t)
+    torch.cuda.synchronize()
+    assert torq.torq_last_device_error() == 0
+    if _pairs() == 74:
+        assert torq.torq_launch_count() - before == 2
+    g_codes, g_sb = gpu_quantized_to_numpy(codes_t, scales_t, M, d)
+    o_codes, o_sb = O.quantize_mxfp4(O.round_to_f32(z))
+    assert np.array_equal(g_sb, o_sb) and np.array_equal(g_codes, o_codes)
+    raw = scales_t.cpu().numpy().copy()
+    rr, cc = np.meshgrid(np.arange(M), np.arange(d // 32), indexing="ij")
+    raw[O.scale_layout_offset(rr, cc, d)] = 0
+    assert not raw.any()
