@@ -31,6 +31,7 @@
 #pragma once
 #include <cuda_bf16.h>
 #include <type_traits>
+#include "pair_handshake.cuh"
 #include "sm100_ptx.cuh"
 
 namespace torq {
@@ -299,7 +300,7 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       tmem_ld_wait();
       tc_fence_before_sync();
       __syncwarp();
-      if (lane == 0 && tile + npairs < total_tiles) mbar_arrive_cluster(map_to_cta(acce_bar, 0));   // accumulator is free again
+      if (lane == 0 && accumulator_is_waited_for(tile, npairs, 1, total_tiles)) mbar_arrive_cluster(map_to_cta(acce_bar, 0));   // free again
       if constexpr (FMT == FMT_NVFP4) {                    // product of the two tensor scales
 #pragma unroll
         for (int j = 0; j < 32; ++j) {

@@ -19,6 +19,7 @@
 #include <cuda_bf16.h>
 #include "nvfp4_quantize.cuh"
 #include "mxint4_quantize.cuh"
+#include "pair_handshake.cuh"
 #include "sm100_ptx.cuh"
 
 namespace torq {
@@ -289,10 +290,11 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
           uint32_t yv[32];
           tmem_ld_32x32(tacc + bb * 32, yv);
           tmem_ld_wait();
-          if (bb == nbb - 1) {                           // this warp's share is read: tell the leader (of another tile to come)
+          if (bb == nbb - 1) {                           // this warp's share is read: tell the leader if it waits for that
             tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0 && tile + npairs < total_tiles) mbar_arrive_cluster(map_to_cta(acce_bar(a), 0));
+            if (lane == 0 && accumulator_is_waited_for(tile, npairs, C::NACC, total_tiles))
+              mbar_arrive_cluster(map_to_cta(acce_bar(a), 0));
           }
           float z[32];
           if (R_intra != nullptr) {
@@ -372,11 +374,6 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
           uint32_t y[16];
           tmem_ld_16x256b_x4(tacc + ((uint32_t)(16 * mh) << 16) + bb * 32, y);
           tmem_ld_wait();
-          if (bb == nbb - 1 && mh == 1) {                // this warp's share is read: tell the leader
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0 && tile + npairs < total_tiles) mbar_arrive_cluster(map_to_cta(acce_bar(a), 0));
-          }
           float acc[4][4];
           if (R_intra != nullptr) {
             uint32_t ah[8], am[8], al[8];                // A fragments: [k chunk * 4 + (n & 1) * 2 + row half]
@@ -455,8 +452,8 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   if (*cta_abort) {
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
-  // The peer no longer touches this CTA's memory after this.  Relaxed: every arrival this CTA sent has been waited for (its
-  // last tile sends none), and a release would make each warp wait for its global stores (0.3 - 0.5 us).
+  // The peer no longer touches this CTA's memory after this.  Relaxed: every arrival this CTA sent has been waited for (the
+  // last tile of each accumulator sends none), and a release would make each warp wait for its global stores (0.3 - 0.5 us).
   cluster_arrive_relaxed();
   cluster_wait();
   if (warp == 1) {
