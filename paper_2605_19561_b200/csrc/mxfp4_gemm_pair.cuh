@@ -331,7 +331,8 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       const int box_gap = long_k && tile + npairs < total_tiles ? k_tiles * (y_is_bf16 ? 24 : 12) : 0;
       long long box_time = clock64() + (warp - 2) * box_gap;
       auto flush = [&](int col) {                        // whole warp
-        while (clock64() < box_time) __nanosleep(40);
+        // a turn lasts 16 cycles at least, a box waits 8 gaps at most; were the limit met, the boxes would go out early
+        paced_wait(box_time, box_gap / 2 + 16, [] { return clock64(); }, [] { __nanosleep(40); });
         box_time += 8 * box_gap;
         fence_proxy_async_smem();
         __syncwarp();

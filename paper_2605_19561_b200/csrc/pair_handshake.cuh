@@ -16,4 +16,11 @@ TORQ_HD bool accumulator_is_waited_for(int tile, int npairs, int accs, int total
   return tile < total_tiles - accs * npairs;
 }
 
+// Sleeps until `clock` has reached `until`, at most `tries` times: a wait for a time has a limit of its own, like one for a
+// barrier, so that it ends whatever the counter does (a CTA that is moved to another SM reads another one).
+template <typename Clock, typename Sleep>
+TORQ_HD void paced_wait(long long until, int tries, Clock clock, Sleep sleep) {
+  for (; tries > 0 && clock() < until; --tries) sleep();
+}
+
 }  // namespace torq

@@ -36,3 +36,19 @@ def test_every_accumulator_arrival_is_waited_for(tmp_path):
             }
         }
 """)
+
+
+def test_paced_wait_ends_whatever_the_clock_does(tmp_path):
+    _run(tmp_path, r"""
+  long long now = 0;
+  int slept = 0;
+  auto frozen = [&] { return now; };
+  torq::paced_wait(1000, 7, frozen, [&] { ++slept; });
+  if (slept != 7) { std::printf("frozen clock: %d\n", slept); return 1; }
+  slept = 0;
+  torq::paced_wait(1000, 7, frozen, [&] { ++slept; now += 400; });
+  if (slept != 3) { std::printf("running clock: %d\n", slept); return 1; }
+  slept = 0;
+  torq::paced_wait(1000, 7, frozen, [&] { ++slept; });
+  if (slept != 0) { std::printf("time already past: %d\n", slept); return 1; }
+""")
