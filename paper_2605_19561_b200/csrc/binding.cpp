@@ -32,6 +32,16 @@ bool operand(PyObject* o, at::ScalarType dtype, bool optional, void** out) {
   return true;
 }
 
+// Scratch: any dtype; the caller counts a byte for each element.
+bool scratch(PyObject* o, void** out, size_t* bytes) {
+  if (!THPVariable_Check(o)) return false;
+  const at::Tensor& t = THPVariable_Unpack(o);
+  if (!t.is_cuda() || !t.is_contiguous()) return false;
+  *out = t.data_ptr();
+  *bytes = (size_t)t.numel();
+  return true;
+}
+
 PyObject* set_entry(PyObject*, PyObject* const* a, Py_ssize_t n) {
   const long kind = n == 2 ? PyLong_AsLong(a[0]) : -1;
   if (kind < 0 || kind >= kKinds) {
@@ -51,20 +61,21 @@ PyObject* layer(PyObject*, PyObject* const* a, Py_ssize_t n) try {
     return nullptr;
   }
   void *X, *R, *Ri, *Wq, *Ws, *ws, *dc, *ds;
+  size_t ws_bytes;
   if (!operand(a[1], at::kBFloat16, false, &X) || !operand(a[2], at::kBFloat16, true, &R) ||
       !operand(a[3], at::kBFloat16, true, &Ri) || !operand(a[4], at::kByte, false, &Wq) || !operand(a[5], at::kByte, false, &Ws) ||
-      !operand(a[7], at::kByte, false, &ws) || !operand(a[8], at::kByte, true, &dc) || !operand(a[9], at::kByte, true, &ds) ||
+      !scratch(a[7], &ws, &ws_bytes) || !operand(a[8], at::kByte, true, &dc) || !operand(a[9], at::kByte, true, &ds) ||
       !THPVariable_Check(a[6]))
     return PyLong_FromLong(-1);
   const at::Tensor &x = THPVariable_Unpack(a[1]), &w = THPVariable_Unpack(a[4]), &y = THPVariable_Unpack(a[6]);
   const bool f32 = y.scalar_type() == at::kFloat;
-  if (x.dim() != 2 || w.dim() != 2 || !y.is_cuda() || !y.is_contiguous() || (!f32 && y.scalar_type() != at::kBFloat16))
+  if (x.dim() != 2 || w.dim() < 1 || !y.is_cuda() || !y.is_contiguous() || (!f32 && y.scalar_type() != at::kBFloat16) ||
+      y.numel() < x.size(0) * w.size(0))
     return PyLong_FromLong(-1);
   void* stream = a[10] == Py_None ? (void*)c10::cuda::getCurrentCUDAStream().stream() : PyLong_AsVoidPtr(a[10]);
   if (PyErr_Occurred()) return nullptr;
   const int64_t M = x.size(0), d = x.size(1), N = w.size(0);
   const torq_dtype dt = f32 ? TORQ_F32 : TORQ_BF16;
-  const size_t ws_bytes = (size_t)THPVariable_Unpack(a[7]).numel();
   void* yp = y.data_ptr();
   torq_status rc;
   if (kind == kNv) {

@@ -128,7 +128,7 @@ def lib() -> ctypes.CDLL:
 
 
 # The whole-layer calls go through the native binding (csrc/binding.cpp), which returns the library's status, or -1 for
-# operands that it does not take: those go on to the checks below it, which say what is wrong with them.
+# operands that it does not take: _refuse then says what is wrong with them.
 def _layer(*args):                               # until lib() has put the native function here
     lib()
     return _layer(*args)
@@ -157,6 +157,27 @@ def _stream(stream=None):
 def _check(t, dtype, name):
     if t is not None and not (t.dtype is dtype and t.is_cuda and t.is_contiguous()):
         raise ValueError(f"{name}: expected a contiguous CUDA tensor of {dtype}, got {t.dtype} on {t.device}")
+
+
+def _check_result(Y, M, N):
+    """Y is written densely as float32 or bfloat16: anything else would get other bytes than its own, or bytes beside it."""
+    if not (Y.dtype in (torch.float32, torch.bfloat16) and Y.is_cuda and Y.is_contiguous()):
+        raise ValueError(f"Y: expected a contiguous CUDA tensor of float32 or bfloat16, got {Y.dtype} on {Y.device}")
+    if Y.numel() < M * N:
+        raise ValueError(f"Y: expected room for {M} x {N} values, got {tuple(Y.shape)}")
+
+
+def _refuse(where, bf16, u8, Y, workspace):
+    """Says what is wrong with the operands that the native binding did not take; nothing was launched."""
+    X, Wq = bf16[0][1], u8[0][1]
+    M, d = X.shape
+    for n, t in bf16:
+        _check(t, torch.bfloat16, n)
+    for n, t in u8:
+        _check(t, torch.uint8, n)
+    _check_result(Y, M, Wq.shape[0])
+    _check(workspace, workspace.dtype, "workspace")
+    raise ValueError(f"{where}: an operand is not a plain CUDA tensor")
 
 
 def _raise(code, where):
@@ -245,7 +266,7 @@ def torq_mxfp4_gemm(Aq, As, Wq, Ws, out_dtype=torch.bfloat16, Y=None, stream=Non
         _check(t, torch.uint8, n)
     if Y is None:
         Y = torch.empty((M, N), dtype=out_dtype, device=Aq.device)
-    _check(Y, Y.dtype, "Y")
+    _check_result(Y, M, N)
     dt = TORQ_F32 if Y.dtype == torch.float32 else TORQ_BF16
     _raise(lib().torq_mxfp4_gemm(_ptr(Aq), _ptr(As), _ptr(Wq), _ptr(Ws), M, N, 2 * K2, _ptr(Y), dt,
                                  _stream(stream)), "torq_mxfp4_gemm")
@@ -265,17 +286,8 @@ def torq_rotated_linear(X, R_inter, R_intra, Wq, Ws, out_dtype=torch.bfloat16, Y
         return Y
     if rc > 0:
         raise TorqError(rc, "torq_rotated_linear")
-    M, d = X.shape
-    N = Wq.shape[0]
-    for t, n in ((X, "X"), (R_inter, "R_inter"), (R_intra, "R_intra")):
-        _check(t, torch.bfloat16, n)
-    for t, n in ((Wq, "Wq"), (Ws, "Ws"), (dbg_codes, "dbg_codes"), (dbg_scales, "dbg_scales")):
-        _check(t, torch.uint8, n)
-    dt = TORQ_F32 if Y.dtype == torch.float32 else TORQ_BF16
-    _raise(lib().torq_rotated_linear(_ptr(X), _ptr(R_inter), _ptr(R_intra), _ptr(Wq), _ptr(Ws), M, d, N,
-                                     _ptr(Y), dt, _ptr(workspace), workspace.numel(), _ptr(dbg_codes),
-                                     _ptr(dbg_scales), _stream(stream)), "torq_rotated_linear")
-    return Y
+    _refuse("torq_rotated_linear", (("X", X), ("R_inter", R_inter), ("R_intra", R_intra)),
+            (("Wq", Wq), ("Ws", Ws), ("dbg_codes", dbg_codes), ("dbg_scales", dbg_scales)), Y, workspace)
 
 
 def torq_rotated_linear_structured(X, R_B, R_intra, Wq, Ws, out_dtype=torch.bfloat16, Y=None, workspace=None,
@@ -291,17 +303,8 @@ def torq_rotated_linear_structured(X, R_B, R_intra, Wq, Ws, out_dtype=torch.bflo
         return Y
     if rc > 0:
         raise TorqError(rc, "torq_rotated_linear_structured")
-    M, d = X.shape
-    N = Wq.shape[0]
-    for t, n in ((X, "X"), (R_B, "R_B"), (R_intra, "R_intra")):
-        _check(t, torch.bfloat16, n)
-    for t, n in ((Wq, "Wq"), (Ws, "Ws"), (dbg_codes, "dbg_codes"), (dbg_scales, "dbg_scales")):
-        _check(t, torch.uint8, n)
-    dt = TORQ_F32 if Y.dtype == torch.float32 else TORQ_BF16
-    _raise(lib().torq_rotated_linear_structured(_ptr(X), _ptr(R_B), _ptr(R_intra), _ptr(Wq), _ptr(Ws), M, d, N,
-                                                _ptr(Y), dt, _ptr(workspace), workspace.numel(), _ptr(dbg_codes),
-                                                _ptr(dbg_scales), _stream(stream)), "torq_rotated_linear_structured")
-    return Y
+    _refuse("torq_rotated_linear_structured", (("X", X), ("R_B", R_B), ("R_intra", R_intra)),
+            (("Wq", Wq), ("Ws", Ws), ("dbg_codes", dbg_codes), ("dbg_scales", dbg_scales)), Y, workspace)
 
 
 TORQ_STATIC_WORKSPACE_BYTES = 16 << 20
@@ -322,7 +325,7 @@ def torq_rotated_linear_static(X, R_inter, R_intra, Wq, Ws, Y, stream=None):
         _check(t, torch.bfloat16, n)
     for t, n in ((Wq, "Wq"), (Ws, "Ws")):
         _check(t, torch.uint8, n)
-    _check(Y, Y.dtype, "Y")
+    _check_result(Y, M, N)
     dt = TORQ_F32 if Y.dtype == torch.float32 else TORQ_BF16
     _raise(lib().torq_rotated_linear_static(_ptr(X), _ptr(R_inter), _ptr(R_intra), _ptr(Wq), _ptr(Ws), M, d, N,
                                             _ptr(Y), dt, _stream(stream)), "torq_rotated_linear_static")
@@ -462,7 +465,7 @@ def torq_nvfp4_gemm(Aq, As, a_tensor_scale: float, Wq, Ws, w_tensor_scale: float
         _check(t, torch.uint8, n)
     if Y is None:
         Y = torch.empty((M, N), dtype=out_dtype, device=Aq.device)
-    _check(Y, Y.dtype, "Y")
+    _check_result(Y, M, N)
     dt = TORQ_F32 if Y.dtype == torch.float32 else TORQ_BF16
     _raise(lib().torq_nvfp4_gemm(_ptr(Aq), _ptr(As), a_tensor_scale, _ptr(Wq), _ptr(Ws), w_tensor_scale, M, N,
                                  2 * K2, _ptr(Y), dt, _stream(stream)), "torq_nvfp4_gemm")
@@ -483,18 +486,8 @@ def torq_rotated_linear_nvfp4(X, R_inter, R_intra32, x_tensor_scale: float, Wq, 
         return Y
     if rc > 0:
         raise TorqError(rc, "torq_rotated_linear_nvfp4")
-    M, d = X.shape
-    N = Wq.shape[0]
-    for t, n in ((X, "X"), (R_inter, "R_inter"), (R_intra32, "R_intra32")):
-        _check(t, torch.bfloat16, n)
-    for t, n in ((Wq, "Wq"), (Ws, "Ws"), (dbg_codes, "dbg_codes"), (dbg_scales, "dbg_scales")):
-        _check(t, torch.uint8, n)
-    dt = TORQ_F32 if Y.dtype == torch.float32 else TORQ_BF16
-    _raise(lib().torq_rotated_linear_nvfp4(_ptr(X), _ptr(R_inter), _ptr(R_intra32), x_tensor_scale, _ptr(Wq),
-                                           _ptr(Ws), w_tensor_scale, M, d, N, _ptr(Y), dt, _ptr(workspace),
-                                           workspace.numel(), _ptr(dbg_codes), _ptr(dbg_scales), _stream(stream)),
-           "torq_rotated_linear_nvfp4")
-    return Y
+    _refuse("torq_rotated_linear_nvfp4", (("X", X), ("R_inter", R_inter), ("R_intra32", R_intra32)),
+            (("Wq", Wq), ("Ws", Ws), ("dbg_codes", dbg_codes), ("dbg_scales", dbg_scales)), Y, workspace)
 
 
 def torq_prepare_weights_nvfp4(R_inter, R_intra32, W, workspace=None, stream=None):
@@ -583,7 +576,7 @@ def torq_mxint4_gemm(A8, As, W8, Ws, out_dtype=torch.bfloat16, Y=None, stream=No
         _check(t, torch.uint8, n)
     if Y is None:
         Y = torch.empty((M, N), dtype=out_dtype, device=A8.device)
-    _check(Y, Y.dtype, "Y")
+    _check_result(Y, M, N)
     dt = TORQ_F32 if Y.dtype == torch.float32 else TORQ_BF16
     _raise(lib().torq_mxint4_gemm(_ptr(A8), _ptr(As), _ptr(W8), _ptr(Ws), M, N, K, _ptr(Y), dt, _stream(stream)),
            "torq_mxint4_gemm")
@@ -603,17 +596,8 @@ def torq_rotated_linear_mxint4(X, R_inter, R_intra, W8, Ws, out_dtype=torch.bflo
         return Y
     if rc > 0:
         raise TorqError(rc, "torq_rotated_linear_mxint4")
-    M, d = X.shape
-    N = W8.shape[0]
-    for t, n in ((X, "X"), (R_inter, "R_inter"), (R_intra, "R_intra")):
-        _check(t, torch.bfloat16, n)
-    for t, n in ((W8, "W8"), (Ws, "Ws"), (dbg_bytes, "dbg_bytes"), (dbg_scales, "dbg_scales")):
-        _check(t, torch.uint8, n)
-    dt = TORQ_F32 if Y.dtype == torch.float32 else TORQ_BF16
-    _raise(lib().torq_rotated_linear_mxint4(_ptr(X), _ptr(R_inter), _ptr(R_intra), _ptr(W8), _ptr(Ws), M, d, N,
-                                            _ptr(Y), dt, _ptr(workspace), workspace.numel(), _ptr(dbg_bytes),
-                                            _ptr(dbg_scales), _stream(stream)), "torq_rotated_linear_mxint4")
-    return Y
+    _refuse("torq_rotated_linear_mxint4", (("X", X), ("R_inter", R_inter), ("R_intra", R_intra)),
+            (("W8", W8), ("Ws", Ws), ("dbg_bytes", dbg_bytes), ("dbg_scales", dbg_scales)), Y, workspace)
 
 
 def torq_prepare_weights_mxint4(R_inter, R_intra, W, workspace=None, stream=None):

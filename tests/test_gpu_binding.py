@@ -58,3 +58,69 @@ def test_refusals():
         torq.torq_rotated_linear(X, R, Ri, Wq.cpu(), Ws)
     with pytest.raises(torq.TorqError):                            # from the library: the workspace is too small
         torq.torq_rotated_linear(X, R, Ri, Wq, Ws, workspace=torch.empty(16, dtype=torch.uint8, device="cuda"))
+
+
+def _layer_calls():
+    """Every whole-layer entry point as f(X, Y=..., workspace=...), with the operands it takes."""
+    X, R, Ri, Wq, Ws = _layer(4, 256, 64, 1)
+    Rb, Rs = R[:8, :8].contiguous(), Ri[0].contiguous()
+    Ws16 = torch.full((torq.torq_nvfp4_scales_bytes(64, 256),), 0x38, dtype=torch.uint8, device="cuda")
+    W8 = torch.zeros(64, 256, dtype=torch.uint8, device="cuda")
+    return X, {
+        "mxfp4": lambda **k: torq.torq_rotated_linear(X, R, Ri, Wq, Ws, **k),
+        "structured": lambda **k: torq.torq_rotated_linear_structured(X, Rb, Rs, Wq, Ws, **k),
+        "nvfp4": lambda **k: torq.torq_rotated_linear_nvfp4(X, R, Ri, 0.01, Wq, Ws16, 0.01, **k),
+        "mxint4": lambda **k: torq.torq_rotated_linear_mxint4(X, R, Ri, W8, Ws, **k),
+    }
+
+
+@pytest.mark.parametrize("kind", ["mxfp4", "structured", "nvfp4", "mxint4"])
+def test_results_and_scratch_that_are_refused(kind):
+    """A result that could not hold what the kernels write, or scratch that they could not use: ValueError, nothing launched,
+    nothing written."""
+    X, calls = _layer_calls()
+    call = calls[kind]
+    torch.cuda.synchronize()
+    before = torq.torq_launch_count()
+    wide = torch.full((4, 80), 7.0, dtype=torch.bfloat16, device="cuda")
+    half = torch.full((4, 64), 7.0, dtype=torch.float16, device="cuda")
+    small = torch.full((3, 64), 7.0, dtype=torch.bfloat16, device="cuda")
+    for Y in (wide[:, :64], half, small, torch.empty(4, 64, dtype=torch.bfloat16), torch.empty(4, 64, dtype=torch.int16, device="cuda")):
+        with pytest.raises(ValueError, match="Y"):
+            call(Y=Y)
+    size = 1 << 20
+    for ws in (torch.empty(size, dtype=torch.uint8), torch.empty(2 * size, dtype=torch.uint8, device="cuda")[::2]):
+        with pytest.raises(ValueError, match="workspace"):
+            call(workspace=ws)
+    with pytest.raises(ValueError):
+        call(out_dtype=torch.float16)
+    torch.cuda.synchronize()
+    assert torq.torq_launch_count() == before
+    assert bool((wide == 7).all()) and bool((half == 7).all()) and bool((small == 7).all())
+
+
+@pytest.mark.parametrize("kind", ["mxfp4", "structured", "nvfp4", "mxint4"])
+def test_results_and_scratch_that_are_taken(kind):
+    """As before: a larger or differently shaped contiguous result, scratch of any type (one byte counted per element)."""
+    X, calls = _layer_calls()
+    call = calls[kind]
+    ref = call()
+    big = torch.full((6, 64), 7.0, dtype=torch.bfloat16, device="cuda")
+    call(Y=big)
+    flat = call(Y=torch.empty(4 * 64, dtype=torch.bfloat16, device="cuda"), workspace=torch.empty(1 << 20, dtype=torch.float32, device="cuda"))
+    torch.cuda.synchronize()
+    assert torch.equal(big[:4], ref) and bool((big[4:] == 7).all()) and torch.equal(flat.view(4, 64), ref)
+
+
+def test_the_separate_gemms_refuse_the_same_results():
+    g = torch.Generator(device="cuda").manual_seed(3)
+    A = torch.randint(0, 256, (4, 128), dtype=torch.uint8, device="cuda", generator=g)
+    W = torch.randint(0, 256, (64, 128), dtype=torch.uint8, device="cuda", generator=g)
+    s = torch.full((torq.torq_nvfp4_scales_bytes(64, 256),), 0x38, dtype=torch.uint8, device="cuda")
+    before = torq.torq_launch_count()
+    for Y in (torch.empty(4, 64, dtype=torch.float16, device="cuda"), torch.empty(3, 64, dtype=torch.bfloat16, device="cuda")):
+        for f in (lambda: torq.torq_mxfp4_gemm(A, s, W, s, Y=Y), lambda: torq.torq_nvfp4_gemm(A, s, 1.0, W, s, 1.0, Y=Y),
+                  lambda: torq.torq_mxint4_gemm(A, s, W, s, Y=Y)):
+            with pytest.raises(ValueError, match="Y"):
+                f()
+    assert torq.torq_launch_count() == before
