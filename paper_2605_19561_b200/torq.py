@@ -4,7 +4,9 @@ There is no fallback: a missing library or a non-zero status raises."""
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
+import warnings
 
 import torch
 
@@ -115,26 +117,55 @@ def lib() -> ctypes.CDLL:
     L.torq_pair_tile_list.restype = i64
     L.torq_launch_count.argtypes = []
     L.torq_launch_count.restype = i64
-    if _build.needs_binding():
-        _build.build_binding()
-    from . import _torq_binding
-    for kind, fn in enumerate((L.torq_rotated_linear, L.torq_rotated_linear_mxint4, L.torq_rotated_linear_structured,
-                               L.torq_rotated_linear_nvfp4)):
-        _torq_binding.set_entry(kind, ctypes.cast(fn, vp).value)
-    global _layer
-    _layer = _torq_binding.layer
     _lib_handle = L
     return L
 
 
 # The whole-layer calls go through the native binding (csrc/binding.cpp), which returns the library's status, or -1 for
-# operands that it does not take: _refuse then says what is wrong with them.
-def _layer(*args):                               # until lib() has put the native function here
-    lib()
+# operands that it does not take: _refuse then says what is wrong with them.  It is built and loaded by the first such call;
+# the library itself needs no compiler beside its own.  Where the binding cannot be had, the same call goes through ctypes.
+_MXFP4, _MXINT4, _STRUCTURED, _NVFP4 = range(4)
+_LAYER_ENTRIES = ("torq_rotated_linear", "torq_rotated_linear_mxint4", "torq_rotated_linear_structured",
+                  "torq_rotated_linear_nvfp4")
+
+
+def _layer(*args):                               # until the first call has put the native function here
+    global _layer
+    _layer = _layer_native() or _layer_ctypes
     return _layer(*args)
 
 
-_MXFP4, _MXINT4, _STRUCTURED, _NVFP4 = range(4)
+def _layer_native():
+    L = lib()
+    try:
+        spec = importlib.util.spec_from_file_location(__package__ + "._torq_binding", _build.build_binding())
+        binding = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(binding)
+    except (ImportError, OSError, RuntimeError) as e:
+        warnings.warn(f"the native binding of the layer calls is missing, they cost 5 us more on the host: {e}")
+        return None
+    for kind, name in enumerate(_LAYER_ENTRIES):
+        binding.set_entry(kind, ctypes.cast(getattr(L, name), ctypes.c_void_p).value)
+    return binding.layer
+
+
+def _layer_ctypes(kind, X, R, R_intra, Wq, Ws, Y, workspace, dbg_codes, dbg_scales, stream, x_scale=None, w_scale=None):
+    for t, dtype, optional in ((X, torch.bfloat16, False), (R, torch.bfloat16, True), (R_intra, torch.bfloat16, True),
+                               (Wq, torch.uint8, False), (Ws, torch.uint8, False), (Y, None, False), (workspace, None, False),
+                               (dbg_codes, torch.uint8, True), (dbg_scales, torch.uint8, True)):
+        if t is None and optional:
+            continue
+        if not (isinstance(t, torch.Tensor) and (dtype is None or t.dtype is dtype) and t.is_cuda and t.is_contiguous()):
+            return -1
+    if X.dim() != 2 or Wq.dim() < 1 or Y.dtype not in (torch.float32, torch.bfloat16) or Y.numel() < X.shape[0] * Wq.shape[0]:
+        return -1
+    M, d = X.shape
+    rest = (M, d, Wq.shape[0], _ptr(Y), TORQ_F32 if Y.dtype == torch.float32 else TORQ_BF16, _ptr(workspace), workspace.numel(),
+            _ptr(dbg_codes), _ptr(dbg_scales), _stream() if stream is None else stream)
+    f = getattr(lib(), _LAYER_ENTRIES[kind])
+    if kind == _NVFP4:
+        return f(_ptr(X), _ptr(R), _ptr(R_intra), x_scale, _ptr(Wq), _ptr(Ws), w_scale, *rest)
+    return f(_ptr(X), _ptr(R), _ptr(R_intra), _ptr(Wq), _ptr(Ws), *rest)
 
 
 def _handle(stream):

@@ -48,7 +48,7 @@ def test_streams_and_threads():
     assert torq.torq_last_device_error() == 0
 
 
-def test_refusals():
+def test_refusals(binding):
     X, R, Ri, Wq, Ws = _layer(4, 256, 64, 1)
     with pytest.raises(ValueError, match="R_inter"):
         torq.torq_rotated_linear(X, R.float(), Ri, Wq, Ws)
@@ -58,6 +58,16 @@ def test_refusals():
         torq.torq_rotated_linear(X, R, Ri, Wq.cpu(), Ws)
     with pytest.raises(torq.TorqError):                            # from the library: the workspace is too small
         torq.torq_rotated_linear(X, R, Ri, Wq, Ws, workspace=torch.empty(16, dtype=torch.uint8, device="cuda"))
+
+
+@pytest.fixture(params=["native", "ctypes"])
+def binding(request, monkeypatch):
+    """Both ways a layer call can take: the native binding, and ctypes where that is missing."""
+    if request.param == "ctypes":
+        monkeypatch.setattr(torq, "_layer", torq._layer_ctypes)
+    else:
+        monkeypatch.setattr(torq, "_layer", torq._layer_native())
+        assert torq._layer is not None
 
 
 def _layer_calls():
@@ -75,7 +85,7 @@ def _layer_calls():
 
 
 @pytest.mark.parametrize("kind", ["mxfp4", "structured", "nvfp4", "mxint4"])
-def test_results_and_scratch_that_are_refused(kind):
+def test_results_and_scratch_that_are_refused(binding, kind):
     """A result that could not hold what the kernels write, or scratch that they could not use: ValueError, nothing launched,
     nothing written."""
     X, calls = _layer_calls()
@@ -100,7 +110,7 @@ def test_results_and_scratch_that_are_refused(kind):
 
 
 @pytest.mark.parametrize("kind", ["mxfp4", "structured", "nvfp4", "mxint4"])
-def test_results_and_scratch_that_are_taken(kind):
+def test_results_and_scratch_that_are_taken(binding, kind):
     """As before: a larger or differently shaped contiguous result, scratch of any type (one byte counted per element)."""
     X, calls = _layer_calls()
     call = calls[kind]
