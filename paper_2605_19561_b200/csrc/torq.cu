@@ -647,8 +647,10 @@ static torq_status rotate_structured_impl(const void* X, const void* R_B, const 
       !encode_x_blocks_3d(&tmX3, X, (uint64_t)M, (uint64_t)d))
     return TORQ_ERR_LAUNCH;
   const int64_t tiles = ((nb + 127) / 128) * ((M + RotStructCfg::TOK - 1) / RotStructCfg::TOK);
-  const int64_t b_tiles = (nb + 127) / 128;             // a multiple of these, so that a CTA keeps its rows of R_B
-  const int64_t most = b_tiles <= st->sm_count ? st->sm_count / b_tiles * b_tiles : st->sm_count;
+  // Where a CTA can keep its rows of R_B, the grid is a multiple of the tiles that have others; where they do not fit (d >
+  // 14336) they are loaded for every tile anyway and every SM works (d = 24576: 148 CTAs, as a multiple 144).
+  const int64_t b_tiles = (nb + 127) / 128, k_slabs = (nb + RotStructCfg::BK - 1) / RotStructCfg::BK;
+  const int64_t most = k_slabs <= RotStructCfg::RB_SLABS ? st->sm_count / b_tiles * b_tiles : st->sm_count;
   const int grid = (int)(tiles < most ? tiles : most);
   if (fmt == FMT_MXINT4)
     launch_tc(rotate_structured_kernel<FMT_MXINT4>, 1, grid, RotStructCfg::THREADS, RotStructCfg::SMEM_BYTES, s, tmRB,

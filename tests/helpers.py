@@ -58,3 +58,28 @@ def mismatch_report(g_codes, g_sb, o_codes, o_sb):
         "non_adjacent": bad_elems,
         "scale_off_by_more_than_one": bad_blocks,
     }
+
+
+def captured_launches(fn):
+    """[(kernel name, CTAs), ...] of the kernels that fn() launches on the current stream: the calls are captured, not run.
+    (fn must have run once before, so that the library's per-device set-up lies behind it.)"""
+    from cuda.bindings import driver as cu
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        fn()
+
+    def ok(res):
+        assert res[0] == cu.CUresult.CUDA_SUCCESS, res[0]
+        return res[1] if len(res) == 2 else res[1:]
+
+    g = cu.CUgraph(graph.raw_cuda_graph())
+    n = ok(cu.cuGraphGetNodes(g, 0))[1]
+    out = []
+    for node in ok(cu.cuGraphGetNodes(g, n))[0]:
+        if ok(cu.cuGraphNodeGetType(node)) != cu.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            continue
+        p = ok(cu.cuGraphKernelNodeGetParams(node))
+        name = ok(cu.cuKernelGetName(p.kern) if int(p.kern) else cu.cuFuncGetName(p.func))
+        out.append((name.decode(), p.gridDimX * p.gridDimY * p.gridDimZ))
+    return out

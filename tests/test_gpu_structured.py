@@ -8,7 +8,7 @@ import pytest
 import torch
 
 import oracle as O
-from helpers import dev_bf16, gpu_quantized_to_numpy, mismatch_report
+from helpers import captured_launches, dev_bf16, gpu_quantized_to_numpy, mismatch_report
 from paper_2605_19561_b200 import inputs as I
 from paper_2605_19561_b200 import torq
 
@@ -149,3 +149,27 @@ def test_one_two_and_several_tiles_per_block_of_threads(M, d):
     _run(xb, I.to_bf16_bits(PB), None, exact=True)
     xr = I.activations(I.CONFIGS["tiny"], M=M, d=d)
     _run(xr, I.to_bf16_bits(I.orthogonal(nb, g)), I.to_bf16_bits(I.orthogonal(32, g)))
+
+
+@pytest.mark.parametrize("d,M,ctas", [(4096, 2000, 148), (14336, 400, 148), (12288, 400, 147), (24576, 100, 148), (24576, 8, 12)])
+def test_grid_of_the_structured_rotation(d, M, ctas):
+    """A multiple of the tiles with different rows of R_B only where those rows stay in shared memory (d <= 14336); beyond, every SM."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    X = torch.zeros((M, d), dtype=torch.bfloat16, device="cuda")
+    R = torch.zeros((d // 32, d // 32), dtype=torch.bfloat16, device="cuda")
+    call = lambda: torq.torq_rotate_quantize_structured(X, R, None)
+    call()
+    launches = captured_launches(call)
+    assert len(launches) == 1 and "rotate_structured_kernel" in launches[0][0]
+    assert launches[0][1] == (ctas if sms == 148 else launches[0][1])
+
+
+def test_rows_of_the_matrix_that_change_between_a_block_of_threads_tiles():
+    """Six block tiles and 150 tiles on 148 CTAs: the second tile of the first CTAs has other rows of R_B than their first."""
+    g = np.random.default_rng(8)
+    M, nb = 100, 768
+    x = g.integers(-8, 9, size=(M, nb * 32)).astype(np.float32)
+    PB = np.zeros((nb, nb), np.float32); PB[np.arange(nb), g.permutation(nb)] = 1
+    PK = np.zeros((32, 32), np.float32); PK[g.permutation(32), np.arange(32)] = 1
+    _run(I.to_bf16_bits(x), I.to_bf16_bits(PB), I.to_bf16_bits(PK), exact=True)
+    _run(I.to_bf16_bits(x), I.to_bf16_bits(PB), None, exact=True)
