@@ -235,14 +235,21 @@ rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_
       named_barrier_sync(1, 512);
     }
     // Scale bytes of the rows past the last token, up to the end of the last 128-row scale tile: zero.  (d % 256 == 0, so
-    // there is no padding along K.)  One 4-byte cell per thread and step, dealt over the whole grid: as a second launch
-    // these zeros took 2.0 to 2.7 us of a 1000- or 300-token call at d = 4096 (9.6 -> 7.0 and 7.0 -> 4.8 us).
-    {
-      const int ns4 = FMT == FMT_NVFP4 ? nblocks / 2 : nblocks / 4;            // cells per row
-      const int pad_rows = (M + 127) / 128 * 128 - M;
-      for (int64_t c = (int64_t)blockIdx.x * 512 + et; c < (int64_t)pad_rows * ns4; c += (int64_t)gridDim.x * 512) {
-        const int64_t r = M + c / ns4;
-        *reinterpret_cast<uint32_t*>(scales + scale_offset(r, 4 * (c % ns4), ns4)) = 0u;
+    // there is no padding along K.)  A thread takes 16 bytes, rows r, r + 32, r + 64, r + 96 of one chunk, the tokens' rows
+    // first, dealt over the whole grid: as a second launch these zeros took 2.0 to 2.7 us of a 1000- or 300-token call at
+    // d = 4096 (9.6 -> 7.0 and 7.0 -> 4.8 us); one row at a time, with 64-bit divisions, they held up the single tile of a CTA with
+    // few tokens (one token, NVFP4, d = 8192: 10.2 us against 7.2 with the second launch).
+    if (M & 127) {
+      const int chunks = FMT == FMT_NVFP4 ? nblocks / 2 : nblocks / 4;         // of 512 bytes per 128 rows
+      const int tokens = M & 127;                                              // in the last 128 rows
+      uint8_t* tile = scales + (size_t)(M >> 7) * chunks * 512;
+      for (int c = blockIdx.x * 512 + et; c < 32 * chunks; c += gridDim.x * 512) {
+        const int r = c & 31, used = (tokens - r + 31) >> 5;                   // rows of this thread's four that hold a token
+        uint32_t* cell = reinterpret_cast<uint32_t*>(tile + (size_t)c * 16);
+        if (used <= 0) *reinterpret_cast<uint4*>(cell) = make_uint4(0u, 0u, 0u, 0u);
+        else if (used <= 1) { cell[1] = 0u; *reinterpret_cast<uint2*>(cell + 2) = make_uint2(0u, 0u); }
+        else if (used <= 2) *reinterpret_cast<uint2*>(cell + 2) = make_uint2(0u, 0u);
+        else if (used <= 3) cell[3] = 0u;
       }
     }
     const int row = q * 32 + lane;                       // b' within the tile = tensor-memory lane

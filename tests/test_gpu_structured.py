@@ -173,3 +173,20 @@ def test_rows_of_the_matrix_that_change_between_a_block_of_threads_tiles():
     PK = np.zeros((32, 32), np.float32); PK[g.permutation(32), np.arange(32)] = 1
     _run(I.to_bf16_bits(x), I.to_bf16_bits(PB), I.to_bf16_bits(PK), exact=True)
     _run(I.to_bf16_bits(x), I.to_bf16_bits(PB), None, exact=True)
+
+
+@pytest.mark.parametrize("M", [1, 31, 32, 33, 64, 65, 95, 96, 97, 127, 128, 129, 256 + 40])
+@pytest.mark.parametrize("d", [256, 8192])
+def test_every_scale_byte_past_the_last_token_is_zero_and_no_other(M, d):
+    """The bytes are zeroed in pieces of four rows 32 apart, some of which may be tokens; a token's scale is never zero here."""
+    X = torch.ones((M, d), dtype=torch.bfloat16, device="cuda")
+    R = torch.eye(d // 32, dtype=torch.bfloat16, device="cuda")
+    for fn, args, group, size in ((torq.torq_rotate_quantize_structured, (), 32, torq.torq_scales_bytes),
+                                  (torq.torq_rotate_quantize_structured_mxint4, (), 32, torq.torq_scales_bytes),
+                                  (torq.torq_rotate_quantize_structured_nvfp4, (0.01,), 16, torq.torq_nvfp4_scales_bytes)):
+        S = torch.full((size(M, d),), 0xEE, dtype=torch.uint8, device="cuda")
+        fn(X, R, None, *args, out_scales=S)
+        torch.cuda.synchronize()
+        got = S.view(-1, d // group // 4, 32, 4, 4).permute(0, 3, 2, 1, 4).reshape(-1, d // group)      # rows in order
+        assert torq.torq_last_device_error() == 0
+        assert bool((got[M:] == 0).all()) and bool((got[:M] != 0).all()) and bool((got[:M] != 0xEE).all())
