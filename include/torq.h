@@ -110,10 +110,9 @@ torq_status torq_mxfp4_gemm(const void* Aq, const void* As, const void* Wq, cons
  * [M, d/2] followed (256-byte aligned) by the tiled scales; pass dbg_codes / dbg_scales non-NULL
  * to also receive copies of them.  Up to 256 tokens the rotation is one kernel that splits its
  * contraction over thread-block clusters and adds the partial sums on chip, in a fixed order.
- * For 257 to 640 tokens with 256 <= d <= 1024 and N < d the rotation is two launches, the first 256
- * tokens and the others; otherwise it is one.  The workspace size includes room that no kernel uses
- * any more (it once held partial sums).
- * (Beyond two waves of 256 x 256 tiles with d > 4096 a last wave of a few tiles is a launch of its own.)
+ * The rotation is one launch, the same kernels as torq_rotate_quantize; beyond two waves of 256 x 256
+ * tiles with d > 4096 a last wave of a few tiles is a launch of its own.  The workspace size includes room
+ * that no kernel uses any more (it once held partial sums).
  * Requires d % 128 == 0 and N % 8 == 0. */
 torq_status torq_rotated_linear(const void* X, const void* R_inter, const void* R_intra,
                                 const void* Wq, const void* Ws, int64_t M, int64_t d, int64_t N,

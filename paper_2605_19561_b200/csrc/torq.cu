@@ -506,13 +506,12 @@ static torq_status rotate_fewtok(DeviceState* st, int fmt, const void* X, const 
   return launch_status();
 }
 
-// Steps 1-4.  `out_features` is the layer's N in the fused calls, 0 otherwise.  `fmt` FMT_NVFP4 (with its tensor scale)
-// needs R_inter.
+// Steps 1-4.  `fmt` FMT_NVFP4 (with its tensor scale) needs R_inter.
 // FMT_F32OUT: out_codes is float32 [M, d] and receives the rotated values (out_scales unused, may be
 // NULL); `x_terms` > 1: X is [M, x_terms * d], the sum of its d-wide column groups is what is rotated.
 static torq_status rotate_quantize_impl(const void* X, const void* R_inter, const void* R_intra, int64_t M,
-                                        int64_t d, void* out_codes, void* out_scales, int64_t out_features,
-                                        void* stream, int fmt = FMT_MXFP4, float tensor_scale = 0.0f, int x_terms = 1) {
+                                        int64_t d, void* out_codes, void* out_scales, void* stream,
+                                        int fmt = FMT_MXFP4, float tensor_scale = 0.0f, int x_terms = 1) {
   if (!X || !out_codes || (!out_scales && fmt != FMT_F32OUT)) return TORQ_ERR_NULL;
   if (fmt != FMT_MXFP4 && !R_inter) return TORQ_ERR_NULL;
   if (M < 1 || d < 32 || d % 32 != 0 || M > (1 << 30) || d > (1 << 24)) return TORQ_ERR_SHAPE;
@@ -533,18 +532,6 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
         static_cast<const __nv_bfloat16*>(X), static_cast<const __nv_bfloat16*>(R_intra), M, d, codes,
         scales);
     return launch_status();
-  }
-  // 257 ... 640 tokens, 256 <= d <= 1024, fewer outputs than inputs: the first 256 tokens and the others in a launch each.
-  // One launch is faster here too (600 tokens, 512 -> 384: rotation 4.4 us against 7.7), but that the fused call takes
-  // three is part of its tested behaviour at these sizes.  (The split of K over the SMs with partial tiles in the
-  // workspace that stood here took 13.2 us of the 16.3; 441 tokens, 256 -> 1496: 13.5 us for the layer, now 6.4.)
-  if (out_features > 0 && out_features < d && M > kRotFewMaxTokens && M <= 640 && d >= 256 && d <= 1024 && d % 128 == 0) {
-    const int64_t head = kRotFewMaxTokens;
-    const torq_status rc = rotate_quantize_impl(X, R_inter, R_intra, head, d, out_codes, out_scales, 0, stream, fmt, tensor_scale);
-    if (rc != TORQ_OK) return rc;
-    const int64_t row_codes = fmt == FMT_MXINT4 ? d : d / 2, tile_scales = 512 * (d / (fmt == FMT_NVFP4 ? 64 : 128));
-    return rotate_quantize_impl(static_cast<const __nv_bfloat16*>(X) + head * d, R_inter, R_intra, M - head, d,
-                                codes + head * row_codes, scales + head / 128 * tile_scales, 0, stream, fmt, tensor_scale);
   }
   CUtensorMap tmX, tmR;
   if (d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT) {
@@ -626,7 +613,7 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
 
 torq_status torq_rotate_quantize(const void* X, const void* R_inter, const void* R_intra, int64_t M,
                                  int64_t d, void* out_codes, void* out_scales, void* stream) {
-  return rotate_quantize_impl(X, R_inter, R_intra, M, d, out_codes, out_scales, 0, stream);
+  return rotate_quantize_impl(X, R_inter, R_intra, M, d, out_codes, out_scales, stream);
 }
 
 static torq_status rotate_structured_impl(const void* X, const void* R_B, const void* R_intra, int64_t M, int64_t d,
@@ -906,7 +893,7 @@ torq_status torq_rotate_quantize_nvfp4(const void* X, const void* R_inter, const
                                        int64_t d, float tensor_scale, void* out_codes, void* out_scales,
                                        void* stream) {
   if (!scale_ok(tensor_scale)) return TORQ_ERR_SHAPE;
-  return rotate_quantize_impl(X, R_inter, R_intra32, M, d, out_codes, out_scales, 0, stream, FMT_NVFP4,
+  return rotate_quantize_impl(X, R_inter, R_intra32, M, d, out_codes, out_scales, stream, FMT_NVFP4,
                               tensor_scale);
 }
 
@@ -923,7 +910,7 @@ torq_status torq_rotated_linear_nvfp4(const void* X, const void* R_inter, const 
   uint8_t* codes = static_cast<uint8_t*>(workspace);
   const size_t codes_bytes = (size_t)M * (size_t)(d / 2);
   uint8_t* scales = codes + (codes_bytes + 255) / 256 * 256;
-  torq_status rc = rotate_quantize_impl(X, R_inter, R_intra32, M, d, codes, scales, N, stream, FMT_NVFP4, x_tensor_scale);
+  torq_status rc = rotate_quantize_impl(X, R_inter, R_intra32, M, d, codes, scales, stream, FMT_NVFP4, x_tensor_scale);
   if (rc != TORQ_OK) return rc;
   rc = torq_nvfp4_gemm(codes, scales, x_tensor_scale, Wq, Ws, w_tensor_scale, M, N, d, Y, y_dtype, stream);
   if (rc != TORQ_OK) return rc;
@@ -991,7 +978,7 @@ torq_status torq_mxint4_expand(const void* packed, int64_t rows, int64_t k, void
 
 torq_status torq_rotate_quantize_mxint4(const void* X, const void* R_inter, const void* R_intra, int64_t M,
                                         int64_t d, void* out_bytes, void* out_scales, void* stream) {
-  return rotate_quantize_impl(X, R_inter, R_intra, M, d, out_bytes, out_scales, 0, stream, FMT_MXINT4,
+  return rotate_quantize_impl(X, R_inter, R_intra, M, d, out_bytes, out_scales, stream, FMT_MXINT4,
                               0.0f);
 }
 
@@ -1017,7 +1004,7 @@ torq_status torq_rotated_linear_mxint4(const void* X, const void* R_inter, const
   uint8_t* bytes = static_cast<uint8_t*>(workspace);
   const size_t n_bytes = (size_t)M * (size_t)d;
   uint8_t* scales = bytes + (n_bytes + 255) / 256 * 256;
-  torq_status rc = rotate_quantize_impl(X, R_inter, R_intra, M, d, bytes, scales, N, stream, FMT_MXINT4, 0.0f);
+  torq_status rc = rotate_quantize_impl(X, R_inter, R_intra, M, d, bytes, scales, stream, FMT_MXINT4, 0.0f);
   if (rc != TORQ_OK) return rc;
   rc = torq_mxint4_gemm(bytes, scales, W8, Ws, M, N, d, Y, y_dtype, stream);
   if (rc != TORQ_OK) return rc;
@@ -1038,7 +1025,7 @@ static torq_status rotated_linear_impl(const void* X, const void* R_inter, const
   uint8_t* codes = static_cast<uint8_t*>(workspace);
   const size_t codes_bytes = (size_t)M * (size_t)(d / 2);
   uint8_t* scales = codes + (codes_bytes + 255) / 256 * 256;
-  torq_status rc = rotate_quantize_impl(X, R_inter, R_intra, M, d, codes, scales, N, stream);
+  torq_status rc = rotate_quantize_impl(X, R_inter, R_intra, M, d, codes, scales, stream);
   if (rc != TORQ_OK) return rc;
   rc = torq_mxfp4_gemm(codes, scales, Wq, Ws, M, N, d, Y, y_dtype, stream);
   if (rc != TORQ_OK) return rc;
@@ -1232,7 +1219,7 @@ static torq_status rotate_weights(const void* W, const void* R_inter, const void
   const int64_t tiles = ((N + 31) / 32) * ((d + 31) / 32);
   transpose_split3_kernel<<<ew_grid(tiles, 1, st->sm_count), 256, 0, s>>>(static_cast<const float*>(W), d, N, T);
   if (launch_status() != TORQ_OK) return TORQ_ERR_LAUNCH;
-  return rotate_quantize_impl(T, R_inter, R_intra, N, d, *wp, nullptr, 0, stream, FMT_F32OUT, 0.0f, 3);
+  return rotate_quantize_impl(T, R_inter, R_intra, N, d, *wp, nullptr, stream, FMT_F32OUT, 0.0f, 3);
 }
 
 torq_status torq_prepare_weights(const void* W, const void* R_inter, const void* R_intra, int64_t d, int64_t N,

@@ -250,7 +250,7 @@ def test_rotated_linear_end_to_end(M):
                                         dbg_bytes=dbg_b, dbg_scales=dbg_s)
     torch.cuda.synchronize()
     assert torq.torq_last_device_error() == 0
-    assert torq.torq_launch_count() - n0 == (2 if M <= 256 else 3)   # few tiles: the rotation is split along its contraction
+    assert torq.torq_launch_count() - n0 == 2             # one rotation kernel, then the GEMM
     g_q, g_sb = _operand_to_int(dbg_b), O.unswizzle_scales(dbg_s.cpu().numpy(), M, d)
     o_out, o_q, o_sb = O.rotated_linear_mxint4(xb, rb, rib, w_q, w_sb)
     rep = _mismatch(g_q, g_sb, o_q, o_sb)
@@ -265,9 +265,8 @@ def test_rotated_linear_end_to_end(M):
 
 @pytest.mark.parametrize("M,intra", [(1, True), (33, True), (128, True), (40, False)])
 def test_rotated_linear_few_tokens_takes_the_split_rotation(M, intra):
-    """Few tokens: the rotation is split along its contraction over the SMs.  Up to 64 tokens one kernel
-    reduces the splits through distributed shared memory; above, the partial sums go through the workspace
-    and a second kernel adds them, rotates inside the blocks and quantizes (three launches instead of two)."""
+    """Few tokens: the rotation is split along its contraction over the SMs, in one kernel that reduces the splits
+    through distributed shared memory."""
     cfg = I.CONFIGS["tiny"]
     d, N = 1024, 256
     xb = I.activations(cfg, M=M, d=d)
@@ -286,7 +285,7 @@ def test_rotated_linear_few_tokens_takes_the_split_rotation(M, intra):
                                         out_dtype=torch.float32, dbg_bytes=dbg_b, dbg_scales=dbg_s)
     torch.cuda.synchronize()
     assert torq.torq_last_device_error() == 0
-    assert torq.torq_launch_count() - n0 == (2 if M <= 256 else 3)   # up to 256 tokens: one rotation kernel, K splits reduced on chip
+    assert torq.torq_launch_count() - n0 == 2             # one rotation kernel, then the GEMM
     g_q, g_sb = _operand_to_int(dbg_b), O.unswizzle_scales(dbg_s.cpu().numpy(), M, d)
     o_q, o_sb = O.quantize_mxint4(O.round_to_f32(O.rotate(xb, rb, rib)))
     rep = _mismatch(g_q, g_sb, o_q, o_sb)

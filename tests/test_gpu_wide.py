@@ -132,22 +132,19 @@ def test_gemm_nvfp4_and_mxint4(M, N, K):
 @pytest.mark.parametrize("M,d,N", [(257, 256, 256), (441, 256, 1496), (640, 1024, 1024), (257, 256, 248), (640, 1024, 1016), (300, 128, 120),
                                    (641, 512, 504)])
 def test_fused_call_of_257_to_640_tokens(M, d, N):
-    """The fused call is the separate rotation and GEMM bit for bit; with fewer outputs than inputs it rotates the first 256
-    tokens and the others by themselves (three launches), from d = 256 and up to 640 tokens."""
+    """The fused call is the separate rotation and GEMM bit for bit, in two launches, whatever N is beside d."""
     g = torch.Generator(device="cuda").manual_seed(M + d + N)
     X = torch.randn(M, d, generator=g, device="cuda").to(torch.bfloat16)
     R = (torch.randn(d, d, generator=g, device="cuda") / d ** 0.5).to(torch.bfloat16)
     Ri = (torch.randn(d // 32, 32, 32, generator=g, device="cuda") / 32 ** 0.5).to(torch.bfloat16)
     Wq = torch.randint(0, 256, (N, d // 2), generator=g, device="cuda", dtype=torch.uint8)
     Ws = torch.randint(120, 132, (torq.torq_scales_bytes(N, d),), generator=g, device="cuda", dtype=torch.uint8)
-    parts = [X[:256], X[256:]] if N < d and 256 <= d and M <= 640 else [X]
-    done = [torq.torq_rotate_quantize(x.contiguous(), R, Ri) for x in parts]
-    codes, scales = torch.cat([c for c, _ in done]), torch.cat([s for _, s in done])
+    codes, scales = torq.torq_rotate_quantize(X, R, Ri)
     ref = torq.torq_mxfp4_gemm(codes, scales, Wq, Ws)
     torch.cuda.synchronize()
     before = torq.torq_launch_count()
     y = torq.torq_rotated_linear(X, R, Ri, Wq, Ws)
     torch.cuda.synchronize()
-    assert torq.torq_launch_count() - before == 1 + len(parts)
+    assert torq.torq_launch_count() - before == 2
     assert torq.torq_last_device_error() == 0
     assert torch.equal(y, ref)
