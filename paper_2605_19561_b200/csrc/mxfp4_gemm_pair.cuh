@@ -327,13 +327,17 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         return *reinterpret_cast<uint32_t*>(&hh);
       };
       // With another tile behind this one the 16 or 32 boxes of a CTA go out one by one over three quarters of that tile's
-      // instructions (512 cycles per stage): all at once they hold up its loads.
-      const int box_gap = long_k && tile + npairs < total_tiles ? k_tiles * (y_is_bf16 ? 24 : 12) : 0;
-      long long box_time = clock64() + (warp - 2) * box_gap;
+      // instructions (512 cycles per stage): all at once they hold up its loads.  bf16 from 8 stages on; float32 boxes, twice as
+      // many, from 16 (us, all at once / spread: 1280 x 14336, K = 2048 MXFP4 24.9 / 26.3, NVFP4 26.9 / 28.4, 8192 x 14336,
+      // K = 2048 154 / 160; 2048 x 14336, K = 4096 65.6 / 64.5, MXINT4 114.5 / 102.8).
+      const int box_gap = k_tiles >= (y_is_bf16 ? 8 : 16) && tile + npairs < total_tiles ? k_tiles * (y_is_bf16 ? 24 : 12) : 0;
+      long long box_time = box_gap ? clock64() + (warp - 2) * box_gap : 0;
       auto flush = [&](int col) {                        // whole warp
-        // a turn lasts 16 cycles at least, a box waits 8 gaps at most; were the limit met, the boxes would go out early
-        paced_wait(box_time, box_gap / 2 + 16, [] { return clock64(); }, [] { __nanosleep(40); });
-        box_time += 8 * box_gap;
+        if (box_gap) {
+          // a turn lasts more than a cycle and a box waits 8 gaps at most, so the limit is not met while the counter runs
+          paced_wait(box_time, 8 * box_gap + 16, [] { return clock64(); }, [] { __nanosleep(40); });
+          box_time += 8 * box_gap;
+        }
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0 && row0 < M && col < N) {

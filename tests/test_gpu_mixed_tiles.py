@@ -196,6 +196,13 @@ def test_gemm_from_eight_stages_on_paces_the_output_and_starts_the_scales_early(
     assert np.array_equal(run(torch.bfloat16), O.round_to_bf16(got))
 
 
+@pytest.mark.parametrize("fmt,M,N,K", [("mxfp4", 2500, 2048, 3840), ("mxfp4", 2500, 2048, 4096), ("mxint4", 2500, 2048, 1920),
+                                       ("mxint4", 2500, 2048, 2048)])
+def test_gemm_from_sixteen_stages_on_paces_float32_output_too(fmt, M, N, K):
+    """Fifteen and sixteen stages: the last length at which float32 boxes go out at once and the first at which they are spread."""
+    test_gemm_from_eight_stages_on_paces_the_output_and_starts_the_scales_early(fmt, M, N, K)
+
+
 @pytest.mark.parametrize("M,d", [(2300, 4352), (2000, 4864), (4096, 4864)])
 def test_rotation_gives_a_short_last_wave_to_the_few_token_kernel(M, d):
     """2 x 74 + 5, 2 x 74 + 4 and 4 x 74 + 8 tiles of 256 x 256: the last columns of the first 256 tokens come from the other
