@@ -58,6 +58,27 @@ struct RotStructCfg {
   static_assert(SMEM_BYTES <= 232448, "shared memory budget");
 };
 
+// Scale bytes of the rows past the last token, up to the end of the last 128-row scale tile: zero.  (d % 256 == 0, so there
+// is no padding along K.)  Thread et of the 512 epilogue threads takes 16 bytes, rows r, r + 32, r + 64, r + 96 of one chunk,
+// the tokens' rows first, dealt over the whole grid: as a second launch these zeros took 2.0 to 2.7 us of a 1000- or
+// 300-token call at d = 4096 (9.6 -> 7.0 and 7.0 -> 4.8 us); one row at a time, with 64-bit divisions, they held up the single
+// tile of a CTA with few tokens (one token, NVFP4, d = 8192: 10.2 us against 7.2 with the second launch, now 5.0).  Not inlined:
+// in the epilogue's own code it cost the calls that have no such row up to 4 % (MXINT4 512 x 256 5.35 -> 5.59 us, so 5.49).
+template <int FMT>
+__device__ __noinline__ void zero_scale_rows(uint8_t* __restrict__ scales, int M, int nblocks, int et) {
+  const int chunks = FMT == FMT_NVFP4 ? nblocks / 2 : nblocks / 4;             // of 512 bytes per 128 rows
+  const int tokens = M & 127;                                                  // in the last 128 rows
+  uint8_t* tile = scales + (size_t)(M >> 7) * chunks * 512;
+  for (int c = blockIdx.x * 512 + et; c < 32 * chunks; c += gridDim.x * 512) {
+    const int r = c & 31, used = (tokens - r + 31) >> 5;                       // rows of this thread's four that hold a token
+    uint32_t* cell = reinterpret_cast<uint32_t*>(tile + (size_t)c * 16);
+    if (used <= 0) *reinterpret_cast<uint4*>(cell) = make_uint4(0u, 0u, 0u, 0u);
+    else if (used <= 1) { cell[1] = 0u; *reinterpret_cast<uint2*>(cell + 2) = make_uint2(0u, 0u); }
+    else if (used <= 2) *reinterpret_cast<uint2*>(cell + 2) = make_uint2(0u, 0u);
+    else if (used <= 3) cell[3] = 0u;
+  }
+}
+
 // tmRB: R_B [B, B] bf16, box [128 x 64], 128-byte swizzle.  tmX3: X as (k, token, block), box (32, 1, 64),
 // 64-byte swizzle.
 // FMT_NVFP4: the NVFP4 quantizer at the end (two 16-element blocks per row of 32, E4M3 scales,
@@ -234,24 +255,7 @@ rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_
       fence_proxy_async_smem();                          // visible to the tensor core's reads
       named_barrier_sync(1, 512);
     }
-    // Scale bytes of the rows past the last token, up to the end of the last 128-row scale tile: zero.  (d % 256 == 0, so
-    // there is no padding along K.)  A thread takes 16 bytes, rows r, r + 32, r + 64, r + 96 of one chunk, the tokens' rows
-    // first, dealt over the whole grid: as a second launch these zeros took 2.0 to 2.7 us of a 1000- or 300-token call at
-    // d = 4096 (9.6 -> 7.0 and 7.0 -> 4.8 us); one row at a time, with 64-bit divisions, they held up the single tile of a CTA with
-    // few tokens (one token, NVFP4, d = 8192: 10.2 us against 7.2 with the second launch).
-    if (M & 127) {
-      const int chunks = FMT == FMT_NVFP4 ? nblocks / 2 : nblocks / 4;         // of 512 bytes per 128 rows
-      const int tokens = M & 127;                                              // in the last 128 rows
-      uint8_t* tile = scales + (size_t)(M >> 7) * chunks * 512;
-      for (int c = blockIdx.x * 512 + et; c < 32 * chunks; c += gridDim.x * 512) {
-        const int r = c & 31, used = (tokens - r + 31) >> 5;                   // rows of this thread's four that hold a token
-        uint32_t* cell = reinterpret_cast<uint32_t*>(tile + (size_t)c * 16);
-        if (used <= 0) *reinterpret_cast<uint4*>(cell) = make_uint4(0u, 0u, 0u, 0u);
-        else if (used <= 1) { cell[1] = 0u; *reinterpret_cast<uint2*>(cell + 2) = make_uint2(0u, 0u); }
-        else if (used <= 2) *reinterpret_cast<uint2*>(cell + 2) = make_uint2(0u, 0u);
-        else if (used <= 3) cell[3] = 0u;
-      }
-    }
+    if (M & 127) zero_scale_rows<FMT>(scales, M, nblocks, et);
     const int row = q * 32 + lane;                       // b' within the tile = tensor-memory lane
     const uint32_t tlane = tmem_base + ((uint32_t)(q * 32) << 16);
     uint32_t tcount = 0;
