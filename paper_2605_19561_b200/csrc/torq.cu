@@ -280,6 +280,17 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, const DeviceState* st) 
   if (ctas > 1 || ntok > RotFewCfg::MAX_SHARED_TOK || steps <= 32 * S) return {S, RotFewCfg::STAGES};
   return {fewtok_cluster(tiles, steps, long_k, 2, st->sm_count, st->few_fit), RotFewCfg::SHARED_STAGES};
 }
+// Cluster size of the few-token GEMM: above S = 4 three K steps per CTA, or two while the partial sums of all CTAs are few, 32
+// tokens per SM (us, S = 4 / 8, 17 and 64 tokens: N = 256, K = 4096 3.44 / 2.99 and 4.33 / 3.92, N = 1024 3.58 / 3.20 and 4.60 /
+// 4.34; S = 4 / 6: 17 tokens N = 2048 3.75 / 3.47; beyond the line 64 tokens N = 2048 NVFP4 4.53 / 4.70).  Up to 16 tokens, where the
+// sums are pushed, three.
+static int fewtok_gemm_cluster(int ntok, int64_t tiles, int64_t steps, int ctas, const DeviceState* st) {
+  if (ntok > 16) {
+    const int S = fewtok_cluster(tiles, steps, 2, ctas, st->sm_count, st->few_fit);
+    if (tiles * S * ntok <= 32 * (int64_t)st->sm_count) return S;
+  }
+  return fewtok_cluster(tiles, steps, 3, ctas, st->sm_count, st->few_fit);
+}
 constexpr int kTailTiles = 8;              // a last wave of up to so many tiles leaves the pair rotation (below)
 constexpr double kNarrowTileCost = 0.88;   // a 192-column tile against a 256-column one: 0.75 of the math, 0.875 of the operand bytes
 
@@ -757,7 +768,7 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
     // Few tokens: 128 output features x all tokens per CTA, K split over a cluster, reduced through
     // distributed shared memory.
     const int64_t steps = (K + FC::BK - 1) / FC::BK;
-    const int S = fewtok_cluster(tiles, steps, 3, FC::ctas_per_sm(ntok), st->sm_count, st->few_fit);
+    const int S = fewtok_gemm_cluster(ntok, tiles, steps, FC::ctas_per_sm(ntok), st);
     const int width = M > FC::MAX_PUSH_TOK ? wide_gemm_width(M, N, steps, false, S, st->gemm_pairs) : 0;
     if (width > 0) return gemm_wide<FMT>(st, Aq, As, Wq, Ws, M, N, K, Y, y_dtype, alpha, width, s);
     if (!encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, 128, 128) ||

@@ -9,7 +9,7 @@ import pytest
 import torch
 
 import oracle as O
-from helpers import dev_bf16, dev_u8, gpu_quantized_to_numpy, lattice, mismatch_report
+from helpers import captured_launches, dev_bf16, dev_u8, gpu_quantized_to_numpy, lattice, mismatch_report
 from paper_2605_19561_b200 import inputs as I
 from paper_2605_19561_b200 import torq
 import test_gpu_mxint4 as TI
@@ -225,3 +225,18 @@ def test_gemm_leaves_the_neighbours_of_its_output_alone():
     assert bool((buf[0] == 777.0).all()) and bool((buf[M + 1] == 777.0).all())
     ref = O.gemm_dequant(ac, asb, wc, wsb)
     assert np.linalg.norm(Y.cpu().numpy() - ref) / np.linalg.norm(ref) <= 1e-5
+
+
+# K ranges of two steps: the first and last token counts, and sizes on both sides of the line (32 tokens of partial sums per SM)
+@pytest.mark.parametrize("M,N,K,ctas", [(17, 256, 4096, 16), (128, 256, 4096, 16), (40, 512, 4096, 32), (64, 1024, 4096, 64), (32, 2048, 4096, 128),
+                                        (48, 2048, 4096, 64), (16, 512, 4096, 16), (24, 520, 3968, 40)])
+def test_gemm_few_tiles_split_a_short_contraction_further(M, N, K, ctas):
+    ac, asb = _rand_operand(M, K, 1)
+    wc, wsb = _rand_operand(N, K, 2)
+    ops = (dev_u8(O.pack_codes(ac)), dev_u8(O.swizzle_scales(asb, K, fill=0)), dev_u8(O.pack_codes(wc)), dev_u8(O.swizzle_scales(wsb, K, fill=0)))
+    got = torq.torq_mxfp4_gemm(*ops, out_dtype=torch.float32).cpu().numpy()
+    ref = O.gemm_dequant(ac, asb, wc, wsb)
+    assert np.linalg.norm(got - ref) / np.linalg.norm(ref) <= 1e-5
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        (name, grid), = captured_launches(lambda: torq.torq_mxfp4_gemm(*ops, out_dtype=torch.float32))
+        assert "gemm_fewtok_kernel" in name and grid == ctas
