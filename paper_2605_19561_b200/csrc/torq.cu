@@ -253,13 +253,12 @@ static_assert(kRotFewMaxTokens <= RotFewCfg::MAX_TOK && kGemmFewMaxTokens <= Gem
 //    d = 5120, S = 7 (40, 30 fit) 20.7 against 13.5 at S = 6; d = 2048, M = 100: S = 8 (16, 15 fit) 14.1, S = 4 7.7;
 //  * above S = 4, at most 1.4 CTAs per SM, so that CTAs of the next kernel in the stream find room and send their
 //    weight loads early (decode layer at d = N = 5120, M = 1: S = 5 17.86, S = 6 17.97, though the rotation by
-//    itself is the faster one with S = 6), and `long_k` K steps per CTA: a longer reduction has to be paid for by a shorter stream (rotation
-//    d = 2048, M = 50: S = 8 7.1, S = 4 6.5; GEMM K = 2048, N = 5120: S = 5 5.5, S = 4 5.1).  Above 128
+//    itself is the faster one with S = 6), and `most`, so that a CTA has some K steps (the callers say how many): a longer
+//    reduction has to be paid for by a shorter stream (rotation d = 2048, M = 50: S = 8 7.1, S = 4 6.5; GEMM K = 2048, N = 5120: S = 5 5.5, S = 4 5.1).  Above 128
 //    tokens the reduction itself is shared out (up to 16 token groups), so there is no such bound (d = 1536: S = 8 9.9, S = 4 11.3);
 //  * no S above the smallest one with the same longest K range (GEMM K = 4096: S = 5 has ranges of 4 steps like S = 4).
 static inline int fewtok_ntok(int64_t M) { return (int)((M + 15) / 16 * 16); }
-static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int long_k, int ctas_per_sm, int sm_count, const int* fit) {
-  int64_t most = k_steps / long_k;
+static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int64_t most, int ctas_per_sm, int sm_count, const int* fit) {
   most = most < 4 ? 4 : (most > 8 ? 8 : most);
   int s = (int)(most < k_steps ? most : k_steps);
   while (s > 1 && (tiles > (int64_t)ctas_per_sm * fit[s] || (s > 4 && 10 * tiles * s > 14 * (int64_t)sm_count))) --s;
@@ -276,9 +275,12 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, const DeviceState* st) 
   const int ntok = fewtok_ntok(M);
   const int64_t tiles = d / 128, steps = d / 64;
   const int long_k = ntok > 128 ? 1 : 10, ctas = RotFewCfg::ctas_per_sm(ntok);
-  const int S = fewtok_cluster(tiles, steps, long_k, ctas, st->sm_count, st->few_fit);
+  // 17 to 64 tokens: two steps less are enough for one more CTA (us, S = 4 / 5 at 48 steps, d = 3072, 24 and 64 tokens: 8.4 /
+  // 7.7 and 9.8 / 9.0, the layer with N = 3072 12.7 / 11.2 and 15.1 / 14.6; S = 5 / 6 at 58, d = 3712: 9.6 / 8.9 and 11.0 / 10.6)
+  const int64_t most = (steps + (ntok > RotFewCfg::MAX_PUSH_TOK && ntok <= 64 ? 2 : 0)) / long_k;
+  const int S = fewtok_cluster(tiles, steps, most, ctas, st->sm_count, st->few_fit);
   if (ctas > 1 || ntok > RotFewCfg::MAX_SHARED_TOK || steps <= 32 * S) return {S, RotFewCfg::STAGES};
-  return {fewtok_cluster(tiles, steps, long_k, 2, st->sm_count, st->few_fit), RotFewCfg::SHARED_STAGES};
+  return {fewtok_cluster(tiles, steps, most, 2, st->sm_count, st->few_fit), RotFewCfg::SHARED_STAGES};
 }
 // Cluster size of the few-token GEMM: above S = 4 three K steps per CTA, or two while the partial sums of all CTAs are few, 32
 // tokens per SM (us, S = 4 / 8, 17 and 64 tokens: N = 256, K = 4096 3.44 / 2.99 and 4.33 / 3.92, N = 1024 3.58 / 3.20 and 4.60 /
@@ -286,10 +288,10 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, const DeviceState* st) 
 // sums are pushed, three.
 static int fewtok_gemm_cluster(int ntok, int64_t tiles, int64_t steps, int ctas, const DeviceState* st) {
   if (ntok > 16) {
-    const int S = fewtok_cluster(tiles, steps, 2, ctas, st->sm_count, st->few_fit);
+    const int S = fewtok_cluster(tiles, steps, steps / 2, ctas, st->sm_count, st->few_fit);
     if (tiles * S * ntok <= 32 * (int64_t)st->sm_count) return S;
   }
-  return fewtok_cluster(tiles, steps, 3, ctas, st->sm_count, st->few_fit);
+  return fewtok_cluster(tiles, steps, steps / 3, ctas, st->sm_count, st->few_fit);
 }
 constexpr int kTailTiles = 8;              // a last wave of up to so many tiles leaves the pair rotation (below)
 constexpr double kNarrowTileCost = 0.88;   // a 192-column tile against a 256-column one: 0.75 of the math, 0.875 of the operand bytes
@@ -576,7 +578,7 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
       tiles.rows_a = 1;
       tiles.less = rest;
       tiles.total -= rest;
-      const int S = fewtok_cluster(2 * rest, d / 64, 1, 1, st->sm_count, st->few_fit);
+      const int S = fewtok_cluster(2 * rest, d / 64, d / 64, 1, st->sm_count, st->few_fit);
       const torq_status rc = rotate_fewtok(st, fmt, X, R_inter, R_intra, 256, d, (int)(d / 128) - 2 * rest, 2 * rest,
                                            {S, RotFewCfg::STAGES}, codes, scales, tensor_scale, s);
       if (rc != TORQ_OK) return rc;

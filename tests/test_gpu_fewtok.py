@@ -240,3 +240,13 @@ def test_gemm_few_tiles_split_a_short_contraction_further(M, N, K, ctas):
     if torch.cuda.get_device_properties(0).multi_processor_count == 148:
         (name, grid), = captured_launches(lambda: torq.torq_mxfp4_gemm(*ops, out_dtype=torch.float32))
         assert "gemm_fewtok_kernel" in name and grid == ctas
+
+
+# 48 and 58 K steps: clusters of 5 and 6 from 17 to 64 tokens, 4 (5) below and above
+@pytest.mark.parametrize("M,d,ctas", [(16, 3072, 96), (17, 3072, 120), (64, 3072, 120), (65, 3072, 96), (33, 3712, 174), (64, 2944, 92)])
+def test_rotation_cluster_of_a_contraction_that_just_misses_a_split(M, d, ctas):
+    test_rotation_alone_without_any_workspace(M, d)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        X, R = torch.zeros((M, d), dtype=torch.bfloat16, device="cuda"), torch.zeros((d, d), dtype=torch.bfloat16, device="cuda")
+        (name, grid), = captured_launches(lambda: torq.torq_rotate_quantize(X, R, None))
+        assert "rotate_fewtok_kernel" in name and grid == ctas
