@@ -23,7 +23,8 @@
 //  * pull (more tokens): every CTA writes its partial [token][feature] into its own shared memory, a cluster barrier
 //    publishes them, and the owner reads them with 16-byte ld.shared::cluster.  A second barrier, at which a warp arrives
 //    as soon as its last such load is back and for which it waits only before it exits, keeps the partials in place
-//    (one full barrier at the end: d = 5120, M = 64 14.0 -> 13.7 us, GEMM 6.7 -> 6.1).
+//    (one full barrier at the end: d = 5120, M = 64 14.0 -> 13.7 us, GEMM 6.7 -> 6.1).  CTAs without a unit then leave earlier
+//    than the others; where that harms (`together`, see the launch) the second barrier is a full one at the end after all.
 // With S = 1 (an ordinary launch without clusters) a warp writes its features into its own shared memory and goes on.
 //
 // Units: the epilogue warps of lane quarter q of every CTA own 32-block q of the tile (its R_intra block is fetched into
@@ -79,12 +80,12 @@ static_assert(RotFewCfg::ctas_per_sm(RotFewCfg::MAX_SHARED_TOK, RotFewCfg::SHARE
 // a multiple of 16.  d % 128 == 0.  `codes` / `scales` / `tensor_scale` as in rotate_quantize_kernel for FMT.
 // ESETS: sets of four epilogue warps (threads = 64 + 128 ESETS).  One set where two CTAs share an SM; a CTA that fills an SM
 // by itself has several token groups to reduce, rotate and quantize, each a dependent chain of about a microsecond for
-// one warp: two sets take them in turn.  NST: stages.
+// one warp: two sets take them in turn.  NST: stages.  `together`: the CTAs of a cluster leave together (S > 1 only).
 template <int FMT = FMT_MXFP4, int ESETS = 1, bool PUSH = false, int NST = RotFewCfg::STAGES>
 __global__ void __launch_bounds__(64 + 128 * ESETS, ESETS == 1 ? 2 : 1)
 rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,
                      const __nv_bfloat16* __restrict__ R_intra, uint8_t* __restrict__ codes,
-                     uint8_t* __restrict__ scales, int M, int d, int ntok, int S, int ft0,
+                     uint8_t* __restrict__ scales, int M, int d, int ntok, int S, int ft0, int together,
                      float tensor_scale, int* err_word) {
   using C = RotFewCfg;
   extern __shared__ uint8_t smem_raw[];
@@ -324,7 +325,7 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
         for (int s = 0; s < C::MAX_CLUSTER; ++s)
           p_rank[s] = s < S ? map_to_cta(p_saddr, live ? (uint32_t)s : (uint32_t)rank) : 0u;
         int g = rank + es * S;
-        if (live && g >= groups) cluster_arrive_relaxed();      // nothing to read
+        if (live && g >= groups && !together) cluster_arrive_relaxed();      // nothing to read
         for (; g < groups; g += S * ESETS) {
 #pragma unroll
           for (int jh = 0; jh < 2; ++jh) {
@@ -353,7 +354,7 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
             }
           }
           __syncwarp();
-          if (live && g + S * ESETS >= groups) cluster_arrive_relaxed();   // the last unit's partials are read
+          if (live && g + S * ESETS >= groups && !together) cluster_arrive_relaxed();   // the last unit's partials are read
           uint32_t y[16];
 #pragma unroll
           for (int n = 0; n < 4; ++n)
@@ -384,8 +385,13 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   if (PUSH) {
     if (warp < 2 && S > 1) cluster_wait();               // the epilogue warps have waited above
   } else {
-    if (warp < 2) { tc_fence_before_sync(); cluster_sync_all(); cluster_arrive_relaxed(); }    // as the epilogue warps in their pass 1
-    cluster_wait();                                      // no CTA of the cluster reads this one's partial tile any more
+    if (warp < 2) {                                      // as the epilogue warps in their pass 1
+      tc_fence_before_sync();
+      cluster_sync_all();
+      if (!together) cluster_arrive_relaxed();
+    }
+    if (together) cluster_sync_all();                    // no CTA of the cluster reads this one's partial tile any more
+    else cluster_wait();
   }
 
   // ------------------------------------------------------------------ teardown

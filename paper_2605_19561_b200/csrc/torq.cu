@@ -251,6 +251,9 @@ static_assert(kRotFewMaxTokens <= RotFewCfg::MAX_TOK && kGemmFewMaxTokens <= Gem
 //    to there -- rotation d = 14336, M = 50: S = 2 (112 clusters) 63.6, S = 1 80.8; d = 7168: S = 4 (56) 20.3, S = 2
 //    24.7; GEMM K = 14336, N = 6144: S = 4 (48) 11.5, S = 2 13.8 -- and a second wave costs more than it brings:
 //    d = 5120, S = 7 (40, 30 fit) 20.7 against 13.5 at S = 6; d = 2048, M = 100: S = 8 (16, 15 fit) 14.1, S = 4 7.7;
+//    With one CTA per SM, clusters of 5 that nearly fill the GPCs hinder the next kernel's: at 25 and 26 tiles (fit[5] = 26) S = 4
+//    (d = 3328, 96 and 128 tokens: S = 5 13.7 and 12.8, S = 4 9.7 and 10.5; layer N = 3328, MXINT4, 96 tokens 22.0, GEMM K = 8192
+//    N = 3200 7.7 and 7.4); clusters of 4, 6 and 8 fill them without harm.  Of 3 see fewtok_leave_together;
 //  * above S = 4, at most 1.4 CTAs per SM, so that CTAs of the next kernel in the stream find room and send their
 //    weight loads early (decode layer at d = N = 5120, M = 1: S = 5 17.86, S = 6 17.97, though the rotation by
 //    itself is the faster one with S = 6), and `most`, so that a CTA has some K steps (the callers say how many): a longer
@@ -261,7 +264,8 @@ static inline int fewtok_ntok(int64_t M) { return (int)((M + 15) / 16 * 16); }
 static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int64_t most, int ctas_per_sm, int sm_count, const int* fit) {
   most = most < 4 ? 4 : (most > 8 ? 8 : most);
   int s = (int)(most < k_steps ? most : k_steps);
-  while (s > 1 && (tiles > (int64_t)ctas_per_sm * fit[s] || (s > 4 && 10 * tiles * s > 14 * (int64_t)sm_count))) --s;
+  while (s > 1 && (tiles > (int64_t)ctas_per_sm * fit[s] || (s > 4 && 10 * tiles * s > 14 * (int64_t)sm_count) ||
+                   (s == 5 && ctas_per_sm == 1 && tiles > fit[5] - 2))) --s;
   while (s > 1 && (k_steps + s - 2) / (s - 1) == (k_steps + s - 1) / s) --s;      // fewer clusters' CTAs: they fit as well
   return s < 1 ? 1 : s;
 }
@@ -281,6 +285,14 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, const DeviceState* st) 
   const int S = fewtok_cluster(tiles, steps, most, ctas, st->sm_count, st->few_fit);
   if (ctas > 1 || ntok > RotFewCfg::MAX_SHARED_TOK || steps <= 32 * S) return {S, RotFewCfg::STAGES};
   return {fewtok_cluster(tiles, steps, most, 2, st->sm_count, st->few_fit), RotFewCfg::SHARED_STAGES};
+}
+// Whether the CTAs of a cluster leave together instead of each when it has no more to do.  Alone on their SMs (65 tokens and
+// more), clusters of 3 that nearly fill the GPCs (44 and 45 tiles, fit[3] = 45) hinder the clusters of the next kernel when
+// they leave one by one (us, one by one / together: d = 5632, 96 and 128 tokens 18.5 / 16.3 and 19.1 / 18.0, layer N = 5632 25.1 /
+// 24.3 and 26.8 / 26.6; d = 5760 MXINT4 layer 32.7 / 29.5 and 35.1 / 31.9); elsewhere leaving early is the better (d = 4096, 96
+// tokens 11.1 / 11.8).  Above 128 tokens the rotation alone gains as well (200 tokens 24.2 / 20.5), the layer loses (29.6 / 30.4).
+static bool fewtok_leave_together(int64_t M, int64_t tiles, FewRotation few, const DeviceState* st) {
+  return M > 64 && M <= 128 && few.stages == RotFewCfg::STAGES && few.cluster == 3 && tiles > st->few_fit[3] - 2;
 }
 // Cluster size of the few-token GEMM: above S = 4 three K steps per CTA, or two while the partial sums of all CTAs are few, 32
 // tokens per SM (us, S = 4 / 8, 17 and 64 tokens: N = 256, K = 4096 3.44 / 2.99 and 4.33 / 3.92, N = 1024 3.58 / 3.20 and 4.60 /
@@ -504,7 +516,7 @@ static torq_status rotate_fewtok(DeviceState* st, int fmt, const void* X, const 
   auto launch = [&](auto push, auto one, auto shared, auto two) {
     const bool share = few.stages != RotFewCfg::STAGES, small = share || RotFewCfg::ctas_per_sm(ntok) >= 2;
     launch_tc(ntok <= RotFewCfg::MAX_PUSH_TOK ? push : (share ? shared : (small ? one : two)), S, tiles * S, small ? 192 : 320, smem, s,
-              tmX, tmR, ri, codes, scales, (int)M, (int)d, ntok, S, ft0, ts, st->err_word);
+              tmX, tmR, ri, codes, scales, (int)M, (int)d, ntok, S, ft0, fewtok_leave_together(M, tiles, few, st) ? 1 : 0, ts, st->err_word);
   };
   constexpr int NS = RotFewCfg::SHARED_STAGES;
   if (fmt == FMT_MXINT4)

@@ -250,3 +250,32 @@ def test_rotation_cluster_of_a_contraction_that_just_misses_a_split(M, d, ctas):
         X, R = torch.zeros((M, d), dtype=torch.bfloat16, device="cuda"), torch.zeros((d, d), dtype=torch.bfloat16, device="cuda")
         (name, grid), = captured_launches(lambda: torq.torq_rotate_quantize(X, R, None))
         assert "rotate_fewtok_kernel" in name and grid == ctas
+
+
+# tiles that nearly fill the device with clusters of 5 (taken as clusters of 4) and of 3 (whose CTAs leave together up to 128 tokens)
+@pytest.mark.parametrize("M,d", [(65, 3200), (128, 3328), (160, 3328), (96, 3072), (65, 5632), (128, 5760), (100, 5760), (160, 5632), (96, 5504)])
+def test_rotation_with_clusters_that_nearly_fill_the_device(M, d):
+    """Permutations of small integers: every code and scale exactly, three calls in a row on the same buffers."""
+    g = np.random.default_rng(M + d)
+    xb = I.to_bf16_bits(g.integers(-8, 9, size=(M, d)).astype(np.float64))
+    perm = g.permutation(d)
+    P = torch.zeros((d, d), dtype=torch.bfloat16, device="cuda")
+    P[torch.arange(d, device="cuda"), torch.from_numpy(perm).cuda()] = 1
+    pin = np.stack([np.eye(32)[g.permutation(32)] for _ in range(d // 32)])
+    y = np.empty((M, d))
+    y[:, perm] = O.decode_bf16(xb)
+    z = np.einsum("mbk,bkj->mbj", y.reshape(M, d // 32, 32), pin).reshape(M, d)
+    X, Ri = dev_bf16(xb), dev_bf16(I.to_bf16_bits(pin))
+    codes_t = torch.full((M, d // 2), 0xEE, dtype=torch.uint8, device="cuda")
+    scales_t = torch.full((torq.torq_scales_bytes(M, d),), 0xEE, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(3):
+        torq.torq_rotate_quantize(X, P, Ri, out_codes=codes_t, out_scales=scales_t)
+    torch.cuda.synchronize()
+    assert torq.torq_last_device_error() == 0
+    g_codes, g_sb = gpu_quantized_to_numpy(codes_t, scales_t, M, d)
+    o_codes, o_sb = O.quantize_mxfp4(O.round_to_f32(z))
+    assert np.array_equal(g_sb, o_sb) and np.array_equal(g_codes, o_codes)
+    if d in (3200, 3328):
+        (name, grid), = captured_launches(lambda: torq.torq_rotate_quantize(X, P, Ri))
+        assert "fewtok" not in name or grid == 4 * (d // 128)
