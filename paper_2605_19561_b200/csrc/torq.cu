@@ -788,8 +788,10 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
     if (!encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, 128, 128) ||
         !encode_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Aq, (uint64_t)M, krow, (uint32_t)ntok, 128))
       return TORQ_ERR_LAUNCH;
-    // up to 16 tokens: partials pushed; up to 64: one set of epilogue warps, two CTAs per SM; more: two sets
-    const bool small = FC::ctas_per_sm(ntok) >= 2;
+    // up to 16 tokens: partials pushed; up to 64: one set of epilogue warps, two CTAs per SM; more: two sets.  65 to 80 tokens in
+    // MXINT4 fit twice on an SM as well, and share it only where that gives them more K splits (us, shared / alone, 72 tokens:
+    // N = 768, K = 3072 4.9 / 4.4, N = 1536 6.0 / 5.1, S = 8 either way; N = 6144, K = 4096, S = 4 and 1: 9.1 / 9.9).
+    const bool small = FC::ctas_per_sm(ntok) >= 2 && (ntok <= 64 || S > fewtok_gemm_cluster(ntok, tiles, steps, 1, st));
     launch_tc(ntok <= FC::MAX_PUSH_TOK ? gemm_fewtok_kernel<FMT, 1, true> : (small ? gemm_fewtok_kernel<FMT, 1> : gemm_fewtok_kernel<FMT, 2>),
               S, tiles * S, small ? 192 : 320, FC::smem_bytes(ntok), s, tmB, tmA, static_cast<const uint8_t*>(As),
               static_cast<const uint8_t*>(Ws), Y, y_dtype == TORQ_BF16 ? 1 : 0, (int)M, (int)N, (int)K, ntok, S, alpha, st->err_word);

@@ -279,3 +279,18 @@ def test_rotation_with_clusters_that_nearly_fill_the_device(M, d):
     if d in (3200, 3328):
         (name, grid), = captured_launches(lambda: torq.torq_rotate_quantize(X, P, Ri))
         assert "fewtok" not in name or grid == 4 * (d // 128)
+
+
+# 65 to 80 tokens of byte operands: two sets of epilogue warps where one CTA per SM splits K as far as two would, one set beyond
+@pytest.mark.parametrize("M,N,K,sets", [(65, 768, 3072, 2), (80, 1536, 3072, 2), (72, 264, 640, 2), (80, 2560, 3072, 1), (65, 6144, 512, 1), (81, 2560, 3072, 2)])
+def test_gemm_mxint4_shares_an_sm_only_for_more_splits(M, N, K, sets):
+    aq, asb = TI._rand_operand(M, K, 3)
+    wq, wsb = TI._rand_operand(N, K, 4)
+    got = TI._gpu_gemm(aq, asb, wq, wsb, torch.float32)
+    ref = O.gemm_mxint4(aq, asb, wq, wsb)
+    assert np.linalg.norm(got - ref) / np.linalg.norm(ref) <= 1e-5
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        A, W = torch.zeros((M, K), dtype=torch.uint8, device="cuda"), torch.zeros((N, K), dtype=torch.uint8, device="cuda")
+        As, Ws = (torch.zeros(torq.torq_scales_bytes(r, K), dtype=torch.uint8, device="cuda") for r in (M, N))
+        (name, _), = captured_launches(lambda: torq.torq_mxint4_gemm(A, As, W, Ws))
+        assert "wide" in name or f"gemm_fewtok_kernelILi2ELi{sets}E" in name, name
