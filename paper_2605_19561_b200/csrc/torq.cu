@@ -6,7 +6,6 @@
 #include <mutex>
 
 #include "../../include/torq.h"
-#include "mxfp4_gemm.cuh"
 #include "mxfp4_gemm_pair.cuh"
 #include "mxfp4_gemm_wide.cuh"
 #include "quantize.cuh"
@@ -108,12 +107,7 @@ static DeviceState* device_state() {
       g_encode = reinterpret_cast<EncodeTiledFn>(fn);
     }
     constexpr int kWideSmem = 232448;                    // the widths share the kernels
-    bool ok = opt_in_smem(mxfp4_gemm_kernel<256, 1>, GemmCfg<256, 1>::SMEM_BYTES) &&
-              opt_in_smem(mxfp4_gemm_kernel<128, 2>, GemmCfg<128, 2>::SMEM_BYTES) &&
-              opt_in_smem(mxfp4_gemm_kernel<256, 1, FMT_NVFP4>, GemmCfg<256, 1, FMT_NVFP4>::SMEM_BYTES) &&
-              opt_in_smem(mxfp4_gemm_kernel<128, 2, FMT_NVFP4>, GemmCfg<128, 2, FMT_NVFP4>::SMEM_BYTES) &&
-              opt_in_smem(rotate_quantize_kernel<256>, RotCfg<256>::SMEM_BYTES) &&
-              opt_in_smem(rotate_quantize_kernel<128>, RotCfg<128>::SMEM_BYTES) &&
+    bool ok = opt_in_smem(rotate_quantize_kernel<256>, RotCfg<256>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_kernel<256, FMT_NVFP4>, RotCfg<256>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_MXFP4>, RotPairCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_NVFP4>, RotPairCfg::SMEM_BYTES) &&
@@ -133,8 +127,6 @@ static DeviceState* device_state() {
               opt_in_smem(rotate_structured_kernel<FMT_NVFP4>, RotStructCfg::SMEM_BYTES) &&
               opt_in_smem(mxfp4_gemm_pair_kernel<FMT_MXFP4>, GemmPairCfg::SMEM_BYTES) &&
               opt_in_smem(mxfp4_gemm_pair_kernel<FMT_NVFP4>, GemmPairCfgT<FMT_NVFP4>::SMEM_BYTES) &&
-              opt_in_smem(mxfp4_gemm_kernel<256, 1, FMT_MXINT4>, GemmCfg<256, 1, FMT_MXINT4>::SMEM_BYTES) &&
-              opt_in_smem(mxfp4_gemm_kernel<128, 2, FMT_MXINT4>, GemmCfg<128, 2, FMT_MXINT4>::SMEM_BYTES) &&
               opt_in_smem(mxfp4_gemm_pair_kernel<FMT_MXINT4>, GemmPairCfgT<FMT_MXINT4>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_kernel<256, FMT_MXINT4>, RotCfg<256>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_MXINT4>, RotPairCfg::SMEM_BYTES) &&
@@ -700,11 +692,10 @@ torq_status torq_rotate_quantize_structured_nvfp4(const void* X, const void* R_B
 //  * few tokens (17 to 128, S CTAs per tile): 2.3 + 0.2 per K step of the longest split + per token 0.025 with S = 1 (the
 //    accumulator goes to Y), else 0.012 + 0.035 / S;
 //  * pair kernel: one wave 4.1 + 0.9 f + (0.285 + 0.04 f) per K step, more (the last one as narrower tiles) 5.2 + per K step
-//    0.325 for a full wave and 0.21 + 0.14 f for the last;
-//  * single CTAs (129 to 256 tokens, few column tiles): 3.2 + 1.3 f + 0.285 per K step.
+//    0.325 for a full wave and 0.21 + 0.14 f for the last.
 // Where it pays: 777 x 5120, K = 14336 (80 pair tiles) 34.7 -> 27.3, K = 4096 13.1 -> 11.2; 1280 x 4096, K = 14336 34.6 ->
 // 27.8; short contractions: 40 x 4096, K = 512 4.0 -> 3.0; 100 x 4096, K = 512 5.1 -> 3.3; 3000 x 1024, K = 2048 7.1 -> 6.4.
-static int wide_gemm_width(int64_t M, int64_t N, int64_t steps, bool pairs, int few_S, int max_pairs) {
+static int wide_gemm_width(int64_t M, int64_t N, int64_t steps, int few_S, int max_pairs) {
   const int64_t rows = (M + 255) / 256;
   const double base = M <= 64 ? 1.5 : (M <= 128 ? 1.8 : 2.0);
   double best = 1e30;
@@ -721,7 +712,6 @@ static int wide_gemm_width(int64_t M, int64_t N, int64_t steps, bool pairs, int 
   double other;
   if (few_S > 0)
     other = 2.3 + 0.2 * (double)((steps + few_S - 1) / few_S) + (double)M * (few_S == 1 ? 0.025 : 0.012 + 0.035 / few_S);
-  else if (!pairs) other = 3.2 + 1.3 * (double)((M + 127) / 128 * ((N + 127) / 128)) / (2 * max_pairs) + 0.285 * (double)steps;
   else if (full == 0) other = 4.1 + 0.9 * f + (double)steps * (0.285 + 0.04 * f);
   else other = 5.2 + (double)steps * (0.325 * (double)full + (rest ? 0.21 + 0.14 * f : 0.0));
   return best < 0.97 * other ? width : 0;
@@ -783,7 +773,7 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
     // distributed shared memory.
     const int64_t steps = (K + FC::BK - 1) / FC::BK;
     const int S = fewtok_gemm_cluster(ntok, tiles, steps, FC::ctas_per_sm(ntok), st);
-    const int width = M > FC::MAX_PUSH_TOK ? wide_gemm_width(M, N, steps, false, S, st->gemm_pairs) : 0;
+    const int width = M > FC::MAX_PUSH_TOK ? wide_gemm_width(M, N, steps, S, st->gemm_pairs) : 0;
     if (width > 0) return gemm_wide<FMT>(st, Aq, As, Wq, Ws, M, N, K, Y, y_dtype, alpha, width, s);
     if (!encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, 128, 128) ||
         !encode_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Aq, (uint64_t)M, krow, (uint32_t)ntok, 128))
@@ -797,56 +787,31 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
               static_cast<const uint8_t*>(Ws), Y, y_dtype == TORQ_BF16 ? 1 : 0, (int)M, (int)N, (int)K, ntok, S, alpha, st->err_word);
     return launch_status();
   }
-  // CTA pairs from two row tiles on -- except for exactly two row tiles with so few 256-column tiles
-  // that the pairs would leave more than half of the SMs idle: 128 x 128 tiles on single CTAs then
-  // put four times as many SMs to work on streaming W.
-  const int64_t pair_tiles = ((M + 255) / 256) * ((N + BN - 1) / BN);
-  const bool use_pairs = !(M <= 256 && 4 * pair_tiles <= st->sm_count);
-  const int width = wide_gemm_width(M, N, (K + GemmWideCfg<FMT>::BK - 1) / GemmWideCfg<FMT>::BK, use_pairs, 0, st->gemm_pairs);
+  const int width = wide_gemm_width(M, N, (K + GemmWideCfg<FMT>::BK - 1) / GemmWideCfg<FMT>::BK, 0, st->gemm_pairs);
   if (width > 0) return gemm_wide<FMT>(st, Aq, As, Wq, Ws, M, N, K, Y, y_dtype, alpha, width, s);
-  if (use_pairs) {
-    CUtensorMap tmSFA, tmSFB;
-    const uint64_t kb4 = (uint64_t)(K / (FMT == FMT_NVFP4 ? 64 : 128));   // 512-byte scale chunks per row
-    constexpr uint32_t sf_box = GemmPairCfgT<FMT>::SF_BOX_WORDS;
-    if (!encode_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Aq, (uint64_t)M, krow, 128, 128) ||
-        !encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, BN / 2, 128) ||
-        !encode_2d(&tmSFA, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, As, (uint64_t)((M + 127) / 128), kb4 * 128, 1, sf_box,
-                   CU_TENSOR_MAP_SWIZZLE_NONE) ||
-        !encode_2d(&tmSFB, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, Ws, (uint64_t)((N + 127) / 128), kb4 * 128, 1, sf_box,
-                   CU_TENSOR_MAP_SWIZZLE_NONE))
-      return TORQ_ERR_LAUNCH;
-    CUtensorMap tmY;
-    const bool ybf = y_dtype == TORQ_BF16;
-    if (!encode_2d(&tmY, ybf ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, ybf ? 2 : 4,
-                   Y, (uint64_t)M, (uint64_t)N, 32, ybf ? 64 : 32))
-      return TORQ_ERR_LAUNCH;
-    CUtensorMap tmBn;                                      // half of a 192-column tile: 96 rows of W
-    if (!encode_2d(&tmBn, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, kNarrowCols / 2, 128))
-      return TORQ_ERR_LAUNCH;
-    const int max_pairs = st->gemm_pairs;
-    const MixedTiles tiles = plan_pair_tiles((int)((M + 255) / 256), N, max_pairs, kNarrowTileCost);
-    const int pairs = tiles.total < max_pairs ? tiles.total : max_pairs;
-    launch_tc(mxfp4_gemm_pair_kernel<FMT>, 2, 2 * pairs, GemmPairCfgT<FMT>::THREADS, GemmPairCfgT<FMT>::SMEM_BYTES, s,
-              tmA, tmB, tmSFA, tmSFB, tmY, tmBn, tiles, ybf ? 1 : 0, (int)M, (int)N, (int)K, alpha, st->err_word);
-    return launch_status();
-  }
-  // One or two row tiles: the work is streaming W once, so prefer the narrower tile while it still leaves
-  // SMs idle (128-column tiles double the number of CTAs pulling on memory).
-  const bool narrow = 2 * (int)((M + 127) / 128) * (int)((N + BN - 1) / BN) <= st->sm_count;
-  const uint32_t bn = narrow ? 128 : BN;
+  CUtensorMap tmSFA, tmSFB;
+  const uint64_t kb4 = (uint64_t)(K / (FMT == FMT_NVFP4 ? 64 : 128));   // 512-byte scale chunks per row
+  constexpr uint32_t sf_box = GemmPairCfgT<FMT>::SF_BOX_WORDS;
   if (!encode_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Aq, (uint64_t)M, krow, 128, 128) ||
-      !encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, bn, 128))
+      !encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, BN / 2, 128) ||
+      !encode_2d(&tmSFA, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, As, (uint64_t)((M + 127) / 128), kb4 * 128, 1, sf_box,
+                 CU_TENSOR_MAP_SWIZZLE_NONE) ||
+      !encode_2d(&tmSFB, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, Ws, (uint64_t)((N + 127) / 128), kb4 * 128, 1, sf_box,
+                 CU_TENSOR_MAP_SWIZZLE_NONE))
     return TORQ_ERR_LAUNCH;
-  const int out_tiles = (int)((M + 127) / 128) * (int)((N + bn - 1) / bn);
-  const int grid = out_tiles < st->sm_count ? out_tiles : st->sm_count;
-  if (narrow)
-    launch_tc(mxfp4_gemm_kernel<128, 2, FMT>, 1, grid, GemmCfg<128, 2, FMT>::THREADS, GemmCfg<128, 2, FMT>::SMEM_BYTES,
-              s, tmA, tmB, static_cast<const uint8_t*>(As), static_cast<const uint8_t*>(Ws), Y,
-              y_dtype == TORQ_BF16 ? 1 : 0, (int)M, (int)N, (int)K, alpha, st->err_word);
-  else
-    launch_tc(mxfp4_gemm_kernel<BN, 1, FMT>, 1, grid, GemmCfg<BN, 1, FMT>::THREADS, GemmCfg<BN, 1, FMT>::SMEM_BYTES, s,
-              tmA, tmB, static_cast<const uint8_t*>(As), static_cast<const uint8_t*>(Ws), Y,
-              y_dtype == TORQ_BF16 ? 1 : 0, (int)M, (int)N, (int)K, alpha, st->err_word);
+  CUtensorMap tmY;
+  const bool ybf = y_dtype == TORQ_BF16;
+  if (!encode_2d(&tmY, ybf ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, ybf ? 2 : 4,
+                 Y, (uint64_t)M, (uint64_t)N, 32, ybf ? 64 : 32))
+    return TORQ_ERR_LAUNCH;
+  CUtensorMap tmBn;                                      // half of a 192-column tile: 96 rows of W
+  if (!encode_2d(&tmBn, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, kNarrowCols / 2, 128))
+    return TORQ_ERR_LAUNCH;
+  const int max_pairs = st->gemm_pairs;
+  const MixedTiles list = plan_pair_tiles((int)((M + 255) / 256), N, max_pairs, kNarrowTileCost);
+  const int pairs = list.total < max_pairs ? list.total : max_pairs;
+  launch_tc(mxfp4_gemm_pair_kernel<FMT>, 2, 2 * pairs, GemmPairCfgT<FMT>::THREADS, GemmPairCfgT<FMT>::SMEM_BYTES, s,
+            tmA, tmB, tmSFA, tmSFB, tmY, tmBn, list, ybf ? 1 : 0, (int)M, (int)N, (int)K, alpha, st->err_word);
   return launch_status();
 }
 

@@ -7,7 +7,7 @@ import pytest
 import torch
 
 import oracle as O
-from helpers import dev_bf16, dev_u8, gpu_quantized_to_numpy, mismatch_report
+from helpers import captured_launches, dev_bf16, dev_u8, gpu_quantized_to_numpy, mismatch_report
 from paper_2605_19561_b200 import inputs as I
 from paper_2605_19561_b200 import torq
 import test_gpu_mxint4 as TI
@@ -148,3 +148,16 @@ def test_fused_call_of_257_to_640_tokens(M, d, N):
     assert torq.torq_launch_count() - before == 2
     assert torq.torq_last_device_error() == 0
     assert torch.equal(y, ref)
+
+
+@pytest.mark.parametrize("M,N,K,kernel", [(129, 8, 128, "wide"), (200, 6144, 4096, "wide"), (256, 9472, 256, "wide"), (256, 128, 14336, "wide"),
+                                          (2048, 6144, 4096, "pair"), (100, 28672, 512, "pair")])
+def test_gemm_kernel_of_more_than_the_few_tokens(M, N, K, kernel):
+    """129 to 256 tokens run on the one-wave kernel however few columns there are; nothing else serves them."""
+    A, W = (torch.zeros((r, K // 2), dtype=torch.uint8, device="cuda") for r in (M, N))
+    As, Ws = (torch.zeros(torq.torq_scales_bytes(r, K), dtype=torch.uint8, device="cuda") for r in (M, N))
+    call = lambda: torq.torq_mxfp4_gemm(A, As, W, Ws)
+    y = call()
+    (name, _), = captured_launches(call)
+    assert f"mxfp4_gemm_{kernel}_kernel" in name and not bool(y.any())
+    assert torq.torq_last_device_error() == 0
