@@ -280,11 +280,12 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, const DeviceState* st) 
 }
 // Whether the CTAs of a cluster leave together instead of each when it has no more to do.  Alone on their SMs (65 tokens and
 // more), clusters of 3 that nearly fill the GPCs (44 and 45 tiles, fit[3] = 45) hinder the clusters of the next kernel when
-// they leave one by one (us, one by one / together: d = 5632, 96 and 128 tokens 18.5 / 16.3 and 19.1 / 18.0, layer N = 5632 25.1 /
-// 24.3 and 26.8 / 26.6; d = 5760 MXINT4 layer 32.7 / 29.5 and 35.1 / 31.9); elsewhere leaving early is the better (d = 4096, 96
-// tokens 11.1 / 11.8).  Above 128 tokens the rotation alone gains as well (200 tokens 24.2 / 20.5), the layer loses (29.6 / 30.4).
+// they leave one by one (us, one by one / together: d = 5632, 96, 128 and 256 tokens 18.5 / 16.3, 19.1 / 18.0 and 28.1 / 22.9, layer
+// with N = 256 and 256 tokens 36.0 / 29.9, with N = 5632 and 96 tokens 25.1 / 24.3; d = 5760 MXINT4, N = 5760, 128 tokens 35.1 /
+// 31.9; only 129 tokens and more with many outputs lose, 31.1 / 31.8); elsewhere leaving early is the better (d = 4096, 96 tokens
+// 11.1 / 11.8).
 static bool fewtok_leave_together(int64_t M, int64_t tiles, FewRotation few, const DeviceState* st) {
-  return M > 64 && M <= 128 && few.stages == RotFewCfg::STAGES && few.cluster == 3 && tiles > st->few_fit[3] - 2;
+  return M > 64 && few.stages == RotFewCfg::STAGES && few.cluster == 3 && tiles > st->few_fit[3] - 2;
 }
 // Cluster size of the few-token GEMM: above S = 4 three K steps per CTA, or two while the partial sums of all CTAs are few, 32
 // tokens per SM (us, S = 4 / 8, 17 and 64 tokens: N = 256, K = 4096 3.44 / 2.99 and 4.33 / 3.92, N = 1024 3.58 / 3.20 and 4.60 /
