@@ -273,7 +273,12 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, const DeviceState* st) 
   const int long_k = ntok > 128 ? 1 : 10, ctas = RotFewCfg::ctas_per_sm(ntok);
   // 17 to 64 tokens: two steps less are enough for one more CTA (us, S = 4 / 5 at 48 steps, d = 3072, 24 and 64 tokens: 8.4 /
   // 7.7 and 9.8 / 9.0, the layer with N = 3072 12.7 / 11.2 and 15.1 / 14.6; S = 5 / 6 at 58, d = 3712: 9.6 / 8.9 and 11.0 / 10.6)
-  const int64_t most = (steps + (ntok > RotFewCfg::MAX_PUSH_TOK && ntok <= 64 ? 2 : 0)) / long_k;
+  int64_t most = (steps + (ntok > RotFewCfg::MAX_PUSH_TOK && ntok <= 64 ? 2 : 0)) / long_k;
+  // 65 to 96 tokens are five or six groups: a cluster of six, where it fits, has one unit per CTA, which pays from ranges of
+  // four steps on (us, S = 4 or the one-wave kernel / S = 6, 65 and 96 tokens: d = 1536 7.4 / 6.1 and 7.4 / 6.5, MXINT4 7.6 / 6.2 and
+  // 7.7 / 6.6, layer with N = 256 11.6 / 10.0 and 12.0 / 10.9; d = 2560 8.1 / 7.5 and 8.7 / 8.2).  At 23 and 24 tiles, where only five
+  // fit, 96 tokens lose (d = 3072 9.3 / 9.6).
+  if (ntok > 64 && ntok <= 96 && steps >= 24 && tiles <= st->few_fit[6] && most < 6) most = 6;
   const int S = fewtok_cluster(tiles, steps, most, ctas, st->sm_count, st->few_fit);
   if (ctas > 1 || ntok > RotFewCfg::MAX_SHARED_TOK || steps <= 32 * S) return {S, RotFewCfg::STAGES};
   return {fewtok_cluster(tiles, steps, most, 2, st->sm_count, st->few_fit), RotFewCfg::SHARED_STAGES};

@@ -294,3 +294,13 @@ def test_gemm_mxint4_shares_an_sm_only_for_more_splits(M, N, K, sets):
         As, Ws = (torch.zeros(torq.torq_scales_bytes(r, K), dtype=torch.uint8, device="cuda") for r in (M, N))
         (name, _), = captured_launches(lambda: torq.torq_mxint4_gemm(A, As, W, Ws))
         assert "wide" in name or f"gemm_fewtok_kernelILi2ELi{sets}E" in name, name
+
+
+# 65 to 96 tokens: clusters of six from 24 K steps on and up to the tiles that fit; 64 and 97 tokens and 23 tiles as before
+@pytest.mark.parametrize("M,d,ctas", [(65, 1536, 72), (96, 1536, 72), (80, 2816, 132), (96, 2304, 108), (64, 1536, 48), (97, 2560, 80), (96, 2944, 92)])
+def test_rotation_cluster_with_one_unit_per_cta(M, d, ctas):
+    test_rotation_alone_without_any_workspace(M, d)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        X, R = torch.zeros((M, d), dtype=torch.bfloat16, device="cuda"), torch.zeros((d, d), dtype=torch.bfloat16, device="cuda")
+        (name, grid), = captured_launches(lambda: torq.torq_rotate_quantize(X, R, None))
+        assert "rotate_fewtok_kernel" in name and grid == ctas
