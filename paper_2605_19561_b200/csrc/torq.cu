@@ -292,15 +292,14 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, const DeviceState* st) 
 static bool fewtok_leave_together(int64_t M, int64_t tiles, FewRotation few, const DeviceState* st) {
   return M > 64 && few.stages == RotFewCfg::STAGES && few.cluster == 3 && tiles > st->few_fit[3] - 2;
 }
-// Cluster size of the few-token GEMM: above S = 4 three K steps per CTA, or two while the partial sums of all CTAs are few, 32
+// Cluster size of the few-token GEMM: above S = 4 three K steps per CTA, or two while the partial sums of all CTAs are few: 32
 // tokens per SM (us, S = 4 / 8, 17 and 64 tokens: N = 256, K = 4096 3.44 / 2.99 and 4.33 / 3.92, N = 1024 3.58 / 3.20 and 4.60 /
-// 4.34; S = 4 / 6: 17 tokens N = 2048 3.75 / 3.47; beyond the line 64 tokens N = 2048 NVFP4 4.53 / 4.70).  Up to 16 tokens, where the
-// sums are pushed, three.
+// 4.34; S = 4 / 6: 17 tokens N = 2048 3.75 / 3.47; beyond the line 64 tokens N = 2048 NVFP4 4.53 / 4.70), and 8 up to 16 tokens,
+// where the sums are pushed (1 token N = 256 2.96 / 2.58, N = 1024 3.10 / 2.82, the layer 11.2 / 10.9; beyond: N = 2048 the GEMM 3.62 /
+// 3.51, the layer of 16 tokens 13.2 / 13.5; S = 4 / 5 at K = 2560, N = 5120 the layer 11.0 / 11.5).
 static int fewtok_gemm_cluster(int ntok, int64_t tiles, int64_t steps, int ctas, const DeviceState* st) {
-  if (ntok > 16) {
-    const int S = fewtok_cluster(tiles, steps, steps / 2, ctas, st->sm_count, st->few_fit);
-    if (tiles * S * ntok <= 32 * (int64_t)st->sm_count) return S;
-  }
+  const int S = fewtok_cluster(tiles, steps, steps / 2, ctas, st->sm_count, st->few_fit);
+  if (tiles * S * ntok <= (ntok > 16 ? 32 : 8) * (int64_t)st->sm_count) return S;
   return fewtok_cluster(tiles, steps, steps / 3, ctas, st->sm_count, st->few_fit);
 }
 constexpr int kTailTiles = 8;              // a last wave of up to so many tiles leaves the pair rotation (below)

@@ -229,7 +229,8 @@ def test_gemm_leaves_the_neighbours_of_its_output_alone():
 
 # K ranges of two steps: the first and last token counts, and sizes on both sides of the line (32 tokens of partial sums per SM)
 @pytest.mark.parametrize("M,N,K,ctas", [(17, 256, 4096, 16), (128, 256, 4096, 16), (40, 512, 4096, 32), (64, 1024, 4096, 64), (32, 2048, 4096, 128),
-                                        (48, 2048, 4096, 64), (16, 512, 4096, 16), (24, 520, 3968, 40)])
+                                        (48, 2048, 4096, 64), (1, 256, 4096, 16), (16, 1024, 4096, 64), (16, 1032, 4096, 72), (16, 2048, 4096, 64),
+                                        (24, 520, 3968, 40)])
 def test_gemm_few_tiles_split_a_short_contraction_further(M, N, K, ctas):
     ac, asb = _rand_operand(M, K, 1)
     wc, wsb = _rand_operand(N, K, 2)
