@@ -116,6 +116,41 @@ def test_rotation_two_ctas_share_an_sm(M, d):
     assert rep["non_adjacent"] == 0 and rep["elem_mismatch_frac"] <= 1e-4 and rep["block_scale_mismatch_frac"] <= 1e-4, rep
 
 
+@pytest.mark.parametrize("M,d", [(65, 6400), (128, 6272)])
+def test_rotation_two_ctas_share_an_sm_in_the_other_formats(M, d):
+    """The three-stage instances of NVFP4 and MXINT4: permutations of small integers, every code and scale byte exactly."""
+    g = np.random.default_rng(M + d)
+    xb = I.to_bf16_bits(g.integers(-8, 9, size=(M, d)).astype(np.float64))
+    perm = g.permutation(d)
+    R = torch.zeros((d, d), dtype=torch.bfloat16, device="cuda")
+    R[torch.arange(d), torch.from_numpy(perm)] = 1.0
+    y = np.empty((M, d))
+    y[:, perm] = O.decode_bf16(xb)
+    X = dev_bf16(xb)
+    for width in (None, 16, 32):                             # no rotation inside the blocks, a permutation of each
+        z, Ri = y, None
+        if width is not None:
+            pin = np.stack([np.eye(width)[g.permutation(width)] for _ in range(d // width)])
+            z = np.einsum("mbk,bkj->mbj", y.reshape(M, d // width, width), pin).reshape(M, d)
+            Ri = dev_bf16(I.to_bf16_bits(pin))
+            Ri = torq.torq_expand_intra16(Ri) if width == 16 else Ri
+        if width != 32:
+            ts = O.tensor_scale_from_amax(np.abs(z).max())
+            call = lambda: torq.torq_rotate_quantize_nvfp4(X, R, Ri, float(ts))
+            g_codes, g_sb = TN._to_numpy(*call(), M, d)
+            o_codes, o_sb = O.quantize_nvfp4(z.astype(np.float32), ts)
+            assert np.array_equal(g_sb, o_sb) and np.array_equal(g_codes, o_codes)
+            assert "ILi1ELi1ELb0ELi3E" in captured_launches(call)[0][0]
+        if width != 16:
+            call = lambda: torq.torq_rotate_quantize_mxint4(X, R, Ri)
+            byt, s = call()
+            torch.cuda.synchronize()
+            o_q, o_sb = O.quantize_mxint4(z.astype(np.float32))
+            assert np.array_equal(TI._operand_to_int(byt), o_q) and np.array_equal(O.unswizzle_scales(s.cpu().numpy(), M, d), o_sb)
+            assert "ILi2ELi1ELb0ELi3E" in captured_launches(call)[0][0]
+    assert torq.torq_last_device_error() == 0
+
+
 def test_rotation_exact_cases_are_bit_exact():
     """Permutation and identity rotations with integer activations: every partial sum is exact in any
     order, so codes and scales must equal the oracle's bit for bit through the split and the reduction."""
