@@ -13,6 +13,7 @@ from __future__ import annotations
 import argparse
 import json
 import os
+import re
 import subprocess
 import sys
 import threading
@@ -29,15 +30,44 @@ METRIC = "rotate+MXFP4-quant GB/s and MXFP4 GEMM TFLOP/s, % of roofline (8B shap
 WORKLOAD = "llama3_8b_qkv"
 
 
-def profiled_traffic(kernel: str, workload: str):
-    """DRAM bytes (read + written) per launch of `kernel` on `workload`, from the committed ncu
-    summary under profiles/ (a line `dram_bytes_per_launch: N`); None when there is none."""
-    import re
+def profiled_traffic(kernel: str, workload: str, tokens: int):
+    """DRAM bytes (read + written) per launch of `kernel` on `workload` with that many tokens, from the committed
+    ncu summary under profiles/ (lines `dram_bytes_per_launch: N` and `tokens: M`); None when there is none."""
     path = os.path.join(ROOT, "profiles", f"{kernel}_{workload}.md")
     if not os.path.exists(path):
         return None
-    m = re.search(r"dram_bytes_per_launch:\s*([0-9.eE+]+)", open(path).read())
-    return float(m.group(1)) if m else None
+    text = open(path).read()
+    m, t = re.search(r"dram_bytes_per_launch:\s*([0-9.eE+]+)", text), re.search(r"^tokens:\s*([0-9]+)", text, re.M)
+    return float(m.group(1)) if m and t and int(t.group(1)) == tokens else None
+
+
+def launched_kernels(call):
+    """The kernels that call() launches, "a + b" where it launches several.  The call is captured in a graph and its
+    nodes are read: nothing runs, and the library's choice is not repeated here."""
+    from cuda.bindings import driver as cu
+
+    def ok(res):
+        if res[0] != cu.CUresult.CUDA_SUCCESS:
+            raise RuntimeError(str(res[0]))
+        return res[1] if len(res) == 2 else res[1:]
+
+    try:
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph(keep_graph=True)
+        with torch.cuda.graph(graph):
+            call()
+        g = cu.CUgraph(graph.raw_cuda_graph())
+        names = []
+        for node in ok(cu.cuGraphGetNodes(g, ok(cu.cuGraphGetNodes(g, 0))[1]))[0]:
+            if ok(cu.cuGraphNodeGetType(node)) == cu.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+                p = ok(cu.cuGraphKernelNodeGetParams(node))
+                mangled = ok(cu.cuKernelGetName(p.kern) if int(p.kern) else cu.cuFuncGetName(p.func)).decode()
+                m = re.match(r"_ZN4torq(\d+)", mangled)                 # a name in the namespace, its length first
+                names.append(mangled[m.end():m.end() + int(m.group(1))] if m else mangled)
+        return " + ".join(names)
+    except Exception as exc:
+        sys.stderr.write(f"[bench] kernel names unknown ({type(exc).__name__}: {exc})\n")
+        return "unknown"
 
 
 def hold_gpu(stream, ms: float = 5.0):
@@ -244,7 +274,7 @@ class KernelTimer:
                 "reasons": clk["reasons"], "how": "cuda graph replay" if graph is not None else "direct launches"}
 
 
-def roof_record(kernel, tm, flop, nbytes, pk, tensor_burst, tensor_sustained, tensor_name, workload):
+def roof_record(kernel, tm, flop, nbytes, pk, tensor_burst, tensor_sustained, tensor_name, workload, tokens):
     """Roofline record of one kernel: the binding bound is the slower of its HBM floor and its tensor
     floor (at the burst peak).  `frac` is quoted against the burst peak; the fraction of the
     sustained peak is printed beside it, never substituted for it."""
@@ -252,7 +282,7 @@ def roof_record(kernel, tm, flop, nbytes, pk, tensor_burst, tensor_sustained, te
     t_hbm, t_tc = nbytes / (pk["hbm_gbs"] * 1e9), flop / (tensor_burst * 1e12)
     rec = {"kernel": kernel, "ms_per_launch": t * 1e3, "launches_timed": tm["launches"], "loop_ms": tm["loop_ms"],
            "sm_mhz_in_loop": tm["sm_mhz"], "throttle_reasons_in_loop": tm["reasons"], "timing": tm["how"],
-           "algorithmic_flop": flop, "algorithmic_bytes": nbytes, "traffic": profiled_traffic(kernel, workload)}
+           "algorithmic_flop": flop, "algorithmic_bytes": nbytes, "traffic": profiled_traffic(kernel, workload, tokens)}
     if t_tc >= t_hbm:
         ach = flop / t / 1e12
         rec.update({"bound": "tensor", "achieved": ach, "peak": tensor_burst, "unit": "TFLOP/s", "frac": ach / tensor_burst,
@@ -273,20 +303,6 @@ def layer_work(M, d, N):
     gemm_flop = 2.0 * M * N * d
     gemm_bytes = M * d / 2 + M * d / 32 + N * d / 2 + N * d / 32 + 2.0 * M * N
     return rot_flop, rot_bytes, gemm_flop, gemm_bytes
-
-
-def rotation_kernel_name(M, d, sm_count):
-    """The kernels that calls of this size may take; the library chooses by its wave counts."""
-    if M <= 256 and d % 128 == 0:
-        return "rotate_fewtok_kernel" if M <= 128 else "rotate_fewtok_kernel or rotate_quantize_wide_kernel"
-    if M <= 128:
-        return "rotate_quantize_kernel"
-    waves = -(-M // 256) * -(-d // 256) / (sm_count // 2)
-    return "rotate_quantize_pair_kernel" if waves > 2 or d % 128 else "rotate_quantize_wide_kernel or rotate_quantize_pair_kernel"
-
-
-def gemm_kernel_name(M):
-    return "gemm_fewtok_kernel" if M <= 128 else ("mxfp4_gemm_pair_kernel" if M > 128 else "mxfp4_gemm_kernel")
 
 
 class Layer:
@@ -351,21 +367,20 @@ class Layer:
         self.torq.torq_mxfp4_gemm(c, sc, b["Wq"], b["Ws"], Y=b["Y"])
 
 
-def measure_layer(layer, timer, pk, fp4_peak, sm_count, world, fp4_sustained=None):
+def measure_layer(layer, timer, pk, fp4_peak, world, fp4_sustained=None):
     """Step, rotate+quantize and GEMM of one workload, each in its own loop with its own clock sample."""
     M, d, N = layer.M, layer.d, layer.N
     rot_flop, rot_bytes, gemm_flop, gemm_bytes = layer_work(M, d, N)
     t_step = timer(layer.step)
     layer.rot(0)                                            # the GEMM-only loop reads these codes
     t_gemm = timer(layer.gemm)
-    rk = rotation_kernel_name(M, d, sm_count)
     t_rot = timer(layer.rot)
-    r_rot = roof_record(rk, t_rot, rot_flop, rot_bytes, pk, pk["bf16_burst"], pk["bf16_sustained"],
-                        f"{pk['source']} bf16 burst", layer.name)
+    r_rot = roof_record(launched_kernels(lambda: layer.rot(0)), t_rot, rot_flop, rot_bytes, pk, pk["bf16_burst"], pk["bf16_sustained"],
+                        f"{pk['source']} bf16 burst", layer.name, M)
     r_rot["frac_of_nominal_2250_tflops"] = rot_flop / t_rot["s"] / 1e12 / 2250.0
     r_rot["GBps"] = rot_bytes / t_rot["s"] / 1e9
-    r_gemm = roof_record(gemm_kernel_name(M), t_gemm, gemm_flop, gemm_bytes, pk, fp4_peak, fp4_sustained,
-                         "self-measured: torq_probe_fp4_peak (FP4 block-scaled MMA issue loop, no loads)", layer.name)
+    r_gemm = roof_record(launched_kernels(lambda: layer.gemm(0)), t_gemm, gemm_flop, gemm_bytes, pk, fp4_peak, fp4_sustained,
+                         "self-measured: torq_probe_fp4_peak (FP4 block-scaled MMA issue loop, no loads)", layer.name, M)
     r_gemm["frac_of_nominal_9000_tflops"] = gemm_flop / t_gemm["s"] / 1e12 / 9000.0
     r_gemm["frac_of_4x_measured_bf16_burst"] = gemm_flop / t_gemm["s"] / 1e12 / (4.0 * pk["bf16_burst"])
     r_gemm["TFLOPs"] = gemm_flop / t_gemm["s"] / 1e12
@@ -408,7 +423,7 @@ def measure_variants(torq, I, layer, timer, pk, fp4_peak, t_rot, world):
             "R_intra (the paper's structure, 2d(B+32) flop per token) on the same activations", "bound": "hbm",
             "ms_per_launch": ts["s"] * 1e3, "sm_mhz_in_loop": ts["sm_mhz"], "achieved": nbytes / ts["s"] / 1e9,
             "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": nbytes / ts["s"] / 1e9 / pk["hbm_gbs"],
-            "algorithmic_bytes": nbytes, "traffic": profiled_traffic("rotate_structured_kernel", layer.name),
+            "algorithmic_bytes": nbytes, "traffic": profiled_traffic("rotate_structured_kernel", layer.name, M),
             "speedup_over_dense_rotation": t_rot["s"] / ts["s"],
             "whole_layer_ms_per_step": tl["s"] * 1e3, "whole_layer_tokens_per_s": world * M / tl["s"]}
 
@@ -580,7 +595,6 @@ def main():
     cfg = I.CONFIGS[args.workload]
     M, d, N = (args.M or cfg.M), cfg.d, cfg.N
     pk = peaks()
-    sm_count = torch.cuda.get_device_properties(local_rank).multi_processor_count
     stream = torch.cuda.current_stream()
     loop_stream = torch.cuda.Stream()                      # graph capture needs a stream of its own
     sampler = ClockSampler(local_rank)
@@ -625,7 +639,7 @@ def main():
         clocks = sampler.summary(t_host0 - 0.05, t_host1 + 0.05)
 
     # ---- per-kernel loops of the main workload, each >= MIN_LOOP_MS with its own clock sample
-    main_rec, t_step, t_rot, t_gemm = measure_layer(layer, timer, pk, fp4_probe, sm_count, world, fp4_sustained)
+    main_rec, t_step, t_rot, t_gemm = measure_layer(layer, timer, pk, fp4_probe, world, fp4_sustained)
     extras = {}
     if not args.only_main:
         extras = measure_variants(torq, I, layer, timer, pk, fp4_probe, t_rot, world)
@@ -639,7 +653,7 @@ def main():
         del layer.sets[1:]
         torch.cuda.empty_cache()
         down = Layer(torq, I, "llama3_8b_down", I.CONFIGS["llama3_8b_down"].M)
-        rec, _, _, _ = measure_layer(down, KernelTimer(loop_stream, sampler, down.n_sets), pk, fp4_probe, sm_count, 1, fp4_sustained)
+        rec, _, _, _ = measure_layer(down, KernelTimer(loop_stream, sampler, down.n_sets), pk, fp4_probe, 1, fp4_sustained)
         others["llama3_8b_down"] = rec
         del down
         torch.cuda.empty_cache()
@@ -648,7 +662,7 @@ def main():
         for m in SWEEP_M:
             lay = Layer(torq, I, "qwen3_32b_sweep", m) if base is None else base.with_tokens(I, m)
             base = base or lay
-            rec, _, _, _ = measure_layer(lay, KernelTimer(loop_stream, sampler, lay.n_sets), pk, fp4_probe, sm_count, 1, fp4_sustained)
+            rec, _, _, _ = measure_layer(lay, KernelTimer(loop_stream, sampler, lay.n_sets), pk, fp4_probe, 1, fp4_sustained)
             sweep.append({"M": m, "us_per_step": rec["ms_per_step"] * 1e3, "tokens_per_s": rec["tokens_per_s"],
                           "sm_mhz": rec["sm_mhz_in_step_loop"],
                           "rotate_quantize": {k: rec["rotate_quantize"][k] for k in
