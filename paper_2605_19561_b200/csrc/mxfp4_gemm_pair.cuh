@@ -300,7 +300,8 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       tmem_ld_wait();
       tc_fence_before_sync();
       __syncwarp();
-      if (lane == 0 && accumulator_is_waited_for(tile, npairs, 1, total_tiles)) mbar_arrive_cluster(map_to_cta(acce_bar, 0));   // free again
+      const bool more = accumulator_is_waited_for(tile, npairs, 1, total_tiles);
+      if (lane == 0 && more) mbar_arrive_cluster(map_to_cta(acce_bar, 0));   // free again
       if constexpr (FMT == FMT_NVFP4) {                    // product of the two tensor scales
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
@@ -330,14 +331,12 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       // instructions (512 cycles per stage): all at once they hold up its loads.  bf16 from 8 stages on; float32 boxes, twice as
       // many, from 16 (us, all at once / spread: 1280 x 14336, K = 2048 MXFP4 24.9 / 26.3, NVFP4 26.9 / 28.4, 8192 x 14336,
       // K = 2048 154 / 160; 2048 x 14336, K = 4096 65.6 / 64.5, MXINT4 114.5 / 102.8).
-      const int box_gap = k_tiles >= (y_is_bf16 ? 8 : 16) && tile + npairs < total_tiles ? k_tiles * (y_is_bf16 ? 24 : 12) : 0;
-      long long box_time = box_gap ? clock64() + (warp - 2) * box_gap : 0;
+      const int box_gap = k_tiles >= (y_is_bf16 ? 8 : 16) && more ? k_tiles * (y_is_bf16 ? 24 : 12) : 0;
+      const unsigned since = (unsigned)clock();
+      unsigned box_wait = (unsigned)((warp - 2) * box_gap);
       auto flush = [&](int col) {                        // whole warp
-        if (box_gap) {
-          // a turn lasts more than a cycle and a box waits 8 gaps at most, so the limit is not met while the counter runs
-          paced_wait(box_time, 8 * box_gap + 16, [] { return clock64(); }, [] { __nanosleep(40); });
-          box_time += 8 * box_gap;
-        }
+        if (box_gap) paced_wait(since, box_wait, [] { return (unsigned)clock(); }, [] { __nanosleep(40); });
+        box_wait += 8u * box_gap;
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0 && row0 < M && col < N) {

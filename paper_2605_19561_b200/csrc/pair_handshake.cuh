@@ -13,14 +13,15 @@ namespace torq {
 // such a tile.  An arrival that nobody waits for would cross to the leader's shared memory with nothing to keep that CTA
 // there: the kernels' last cluster barrier is relaxed and orders no arrivals.
 TORQ_HD bool accumulator_is_waited_for(int tile, int npairs, int accs, int total_tiles) {
-  return tile < total_tiles - accs * npairs;
+  return tile + accs * npairs < total_tiles;
 }
 
-// Sleeps until `clock` has reached `until`, at most `tries` times: a wait for a time has a limit of its own, like one for a
-// barrier, so that it ends whatever the counter does (a CTA that is moved to another SM reads another one).
+// Sleeps until `cycles` have passed since `since`, by a counter that wraps around.  Whatever the counter does, the wait ends: it
+// goes on only while the counter shows a time within `cycles` after `since`, so a counter that jumps (a CTA that is moved to
+// another SM reads another one), back or ahead, ends it.
 template <typename Clock, typename Sleep>
-TORQ_HD void paced_wait(long long until, int tries, Clock clock, Sleep sleep) {
-  for (; tries > 0 && clock() < until; --tries) sleep();
+TORQ_HD void paced_wait(unsigned since, unsigned cycles, Clock clock, Sleep sleep) {
+  while (clock() - since < cycles) sleep();
 }
 
 }  // namespace torq

@@ -40,15 +40,14 @@ def test_every_accumulator_arrival_is_waited_for(tmp_path):
 
 def test_paced_wait_ends_whatever_the_clock_does(tmp_path):
     _run(tmp_path, r"""
-  long long now = 0;
-  int slept = 0;
-  auto frozen = [&] { return now; };
-  torq::paced_wait(1000, 7, frozen, [&] { ++slept; });
-  if (slept != 7) { std::printf("frozen clock: %d\n", slept); return 1; }
-  slept = 0;
-  torq::paced_wait(1000, 7, frozen, [&] { ++slept; now += 400; });
-  if (slept != 3) { std::printf("running clock: %d\n", slept); return 1; }
-  slept = 0;
-  torq::paced_wait(1000, 7, frozen, [&] { ++slept; });
-  if (slept != 0) { std::printf("time already past: %d\n", slept); return 1; }
+  // start of the wait, cycles, what a turn adds to the counter: 40 each, 40 over the wrap, a jump back, a jump ahead, no wait
+  struct { unsigned since, cycles; int step[4]; int turns; } cases[] = {
+      {1000u, 100u, {40, 40, 40, 40}, 3}, {0xFFFFFFF0u, 100u, {40, 40, 40, 40}, 3}, {1000u, 100u, {40, -500, 40, 40}, 2},
+      {1000u, 100u, {40, 1000000, 40, 40}, 2}, {1000u, 0u, {40, 40, 40, 40}, 0}};
+  for (auto& c : cases) {
+    unsigned now = c.since;
+    int turns = 0;
+    torq::paced_wait(c.since, c.cycles, [&] { return now; }, [&] { now += (unsigned)c.step[turns & 3]; ++turns; });
+    if (turns != c.turns) { std::printf("since %u cycles %u: %d turns\\n", c.since, c.cycles, turns); return 1; }
+  }
 """)
