@@ -58,27 +58,6 @@ struct RotStructCfg {
   static_assert(SMEM_BYTES <= 232448, "shared memory budget");
 };
 
-// Scale bytes of the rows past the last token, up to the end of the last 128-row scale tile: zero.  (d % 256 == 0, so there
-// is no padding along K.)  Thread et of the 512 epilogue threads takes 16 bytes, rows r, r + 32, r + 64, r + 96 of one chunk,
-// the tokens' rows first, dealt over the whole grid: as a second launch these zeros took 2.0 to 2.7 us of a 1000- or
-// 300-token call at d = 4096 (9.6 -> 7.0 and 7.0 -> 4.8 us); one row at a time, with 64-bit divisions, they held up the single
-// tile of a CTA with few tokens (one token, NVFP4, d = 8192: 10.2 us against 7.2 with the second launch, now 5.0).  Not inlined:
-// in the epilogue's own code it cost the calls that have no such row up to 4 % (MXINT4 512 x 256 5.35 -> 5.59 us, so 5.49).
-template <int FMT>
-__device__ __noinline__ void zero_scale_rows(uint8_t* __restrict__ scales, int M, int nblocks, int et) {
-  const int chunks = FMT == FMT_NVFP4 ? nblocks / 2 : nblocks / 4;             // of 512 bytes per 128 rows
-  const int tokens = M & 127;                                                  // in the last 128 rows
-  uint8_t* tile = scales + (size_t)(M >> 7) * chunks * 512;
-  for (int c = blockIdx.x * 512 + et; c < 32 * chunks; c += gridDim.x * 512) {
-    const int r = c & 31, used = (tokens - r + 31) >> 5;                       // rows of this thread's four that hold a token
-    uint32_t* cell = reinterpret_cast<uint32_t*>(tile + (size_t)c * 16);
-    if (used <= 0) *reinterpret_cast<uint4*>(cell) = make_uint4(0u, 0u, 0u, 0u);
-    else if (used <= 1) { cell[1] = 0u; *reinterpret_cast<uint2*>(cell + 2) = make_uint2(0u, 0u); }
-    else if (used <= 2) *reinterpret_cast<uint2*>(cell + 2) = make_uint2(0u, 0u);
-    else if (used <= 3) cell[3] = 0u;
-  }
-}
-
 // tmRB: R_B [B, B] bf16, box [128 x 64], 128-byte swizzle.  tmX3: X as (k, token, block), box (32, 1, 64),
 // 64-byte swizzle.
 // FMT_NVFP4: the NVFP4 quantizer at the end (two 16-element blocks per row of 32, E4M3 scales,
@@ -255,7 +234,24 @@ rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_
       fence_proxy_async_smem();                          // visible to the tensor core's reads
       named_barrier_sync(1, 512);
     }
-    if (M & 127) zero_scale_rows<FMT>(scales, M, nblocks, et);
+    // Scale bytes of the rows past the last token, up to the end of the last 128-row scale tile: zero.  (d % 256 == 0, so
+    // there is no padding along K.)  A thread takes 16 bytes, rows r, r + 32, r + 64, r + 96 of one 512-byte chunk, the tokens'
+    // rows first, dealt over the whole grid: as a second launch these zeros took 2.0 to 2.7 us of a 1000- or 300-token call at
+    // d = 4096 (9.6 -> 7.0 and 7.0 -> 4.8 us); one row at a time they held up the single tile of a CTA with few tokens (one token,
+    // NVFP4, d = 8192: 10.2 us against 7.2 with the second launch, now 5.8).  This form is the one beside which the compiler
+    // keeps the tile loop as it is: with 32-bit counters, or as a function of its own, one token was 0.1 to 0.7 us faster but the
+    // layer of 4096 tokens slower (d = 4096, N = 6144: 61.6 us here, 62.5 to 62.8 with those).
+    {
+      const int chunks = FMT == FMT_NVFP4 ? nblocks / 2 : nblocks / 4;
+      const int pad = (M + 127) / 128 * 128 - M;
+      for (int64_t c = (int64_t)blockIdx.x * 512 + et; c < (pad ? (int64_t)32 * chunks : 0); c += (int64_t)gridDim.x * 512) {
+        uint32_t* cell = reinterpret_cast<uint32_t*>(scales + ((size_t)(M >> 7) * chunks * 512 + c * 16));
+        const int used = (159 - pad - (int)(c & 31)) >> 5;   // rows of this thread's four that hold a token
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (k >= used) cell[k] = 0u;
+      }
+    }
     const int row = q * 32 + lane;                       // b' within the tile = tensor-memory lane
     const uint32_t tlane = tmem_base + ((uint32_t)(q * 32) << 16);
     uint32_t tcount = 0;
