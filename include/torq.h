@@ -378,7 +378,8 @@ int torq_last_device_error(void* stream);
  * some row tiles are covered by fewer 256-column tiles followed by 192-column ones (three wide
  * tiles traded for four narrow ones), chosen so that the longest pair finishes earliest.  Both
  * torq_rotate_quantize (cols = d) and torq_mxfp4_gemm (cols = N), and their format variants, use
- * this list.
+ * this list where these kernels serve a call, except that a rotation with d > 4096 whose last wave
+ * would hold a few 256-column tiles leaves those to another kernel (see torq_rotated_linear).
  *   out: host array of 3 * cap int32, or NULL; receives (row_tile, first_column, width) per tile.
  * Returns the number of tiles (also when it exceeds cap; only cap triples are written), or -1 for
  * rows < 1, cols < 1 or pairs < 1. */

@@ -60,7 +60,8 @@ struct GemmFewCfg {
 
 // grid = ceil(N / 128) * S CTAs in clusters of S along x: CTA b works feature tile b / S, k split b % S.
 // tmW: Wq [N, K bytes] box [128 x 128]; tmA: Aq [M, K bytes] box [ntok x 128]; As / Ws: tiled scales.
-// ESETS: sets of four epilogue warps (threads = 64 + 128 ESETS): one set and two CTAs per SM up to 64 tokens;
+// ESETS: sets of four epilogue warps (threads = 64 + 128 ESETS): one set and two CTAs per SM up to 64 tokens (MXINT4: 80, where
+// that splits K further);
 // two sets above, where a CTA fills an SM by itself and has some forty tokens to add up and store.
 template <int FMT = FMT_MXFP4, int ESETS = 1, bool PUSH = false>
 __global__ void __launch_bounds__(64 + 128 * ESETS, ESETS == 1 ? 2 : 1)

@@ -1,4 +1,4 @@
-// Block-scaled GEMM on CTA pairs in ONE wave (M > 128): every pair works exactly one tile of 256 tokens x `width`
+// Block-scaled GEMM on CTA pairs in ONE wave (17 tokens and more; which sizes, wide_gemm_width says): every pair works exactly one tile of 256 tokens x `width`
 // output features (a multiple of 64, up to 384), the width chosen so that the tiles just fill the pairs.  The pair
 // kernel deals 256-column tiles and pays a whole wave for a remainder, or leaves pairs idle where there are few.
 //
@@ -11,8 +11,8 @@
 // Nothing overlaps the epilogue here, so it runs on twelve warps and stages its rows in the operand stages, which are
 // free by then: accumulator -> registers -> swizzled shared memory -> TMA store of [32 rows x 128 B] boxes.
 //
-// Roles per CTA: warp 0 TMA producer, warp 1 MMA issuer (leader CTA), warps 2..13 epilogue (lane quarter w % 4, three
-// sets).  One elected thread runs the producer's and the issuer's loop.
+// Roles per CTA: warp 0 TMA producer (one elected thread runs its loop), warp 1 MMA issuer (leader CTA; the whole warp runs the
+// loop, an elected lane issues), warps 2..13 epilogue (lane quarter w % 4, three sets).
 #pragma once
 #include <cuda_bf16.h>
 #include "mxfp4_gemm_pair.cuh"

@@ -77,7 +77,7 @@ def test_nvfp4_and_calibration_argument_errors_and_sizes():
         assert torq.torq_nvfp4_scales_bytes(rows, k) == O.nv_scale_layout_bytes(rows, k)
     assert torq.torq_nvfp4_scales_bytes(128, 4096) == 2 * torq.torq_scales_bytes(128, 4096)
     assert torq.torq_nvfp4_workspace_bytes(2048, 4096, 6144) >= 2048 * 2048 + torq.torq_nvfp4_scales_bytes(2048, 4096)
-    # few tokens: room for the fp32 partials of the split rotation as well
+    # few tokens: the room that partial sums once took is still part of the size
     assert torq.torq_nvfp4_workspace_bytes(16, 4096, 6144) > 16 * 2048 + torq.torq_nvfp4_scales_bytes(16, 4096) + 4 * 128 * 4096
     assert L.torq_quantize_nvfp4(one, 0, 4, 64, 1.0, None, one, None) == 1
     assert L.torq_quantize_nvfp4(one, 0, 4, 24, 1.0, one, one, None) == 2            # d % 16 != 0

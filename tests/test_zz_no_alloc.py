@@ -12,8 +12,8 @@ every call on a device reuses it.  These tests go through the C ABI and check th
   * this holds on two calls in a row with different inputs and shapes, i.e. whatever the first
     call left in the shared array does not leak into the second,
   * the calls allocate nothing: free device memory is the same before and after,
-  * each regime of the rotation is reached: split along the contraction (few tokens), CTA pairs
-    (many tokens), and the single-pass kernel when the array has no room left for partial sums,
+  * each regime of the rotation is reached: split along the contraction on chip (few tokens) and CTA
+    pairs (many tokens),
   * a problem too large for the array is refused with TORQ_ERR_WORKSPACE and launches nothing.
 
 The file name sorts after every other test file on purpose: a run that stops at the first failure
@@ -83,9 +83,8 @@ def test_static_entry_point_matches_the_workspace_one_on_two_calls_in_a_row():
 
 
 def test_static_entry_point_in_every_regime_of_the_rotation():
-    """Many tokens (CTA pairs, single pass: exactly two launches), several waves of tiles whose quantized
-    activations nearly fill the array, and a 128-token problem whose partial sums do not fit behind the
-    quantized activations in the array, which must fall back to the single pass."""
+    """Many tokens (CTA pairs: exactly two launches), several waves of tiles whose quantized activations nearly
+    fill the array, and 128 tokens of a long contraction, whose split needs no room in the array."""
     # (M, d, N, dtype, seed, exact, launches)
     cases = [(2048, 4096, 512, torch.bfloat16, 21, True, 2),
              (4096, 5120, 5120, torch.bfloat16, 22, True, 2),
@@ -94,8 +93,7 @@ def test_static_entry_point_in_every_regime_of_the_rotation():
         ops = _layer(M, d, N, seed)
         Y = torch.zeros((M, N), dtype=dt, device="cuda")
         if exact is None:
-            # the workspace entry point splits this rotation (other summation order): compare with the
-            # single-pass kernels instead, which is what the static entry point must have run
+            # compare with the separate rotation and GEMM, which is what the static entry point must have run
             codes, scales = torq.torq_rotate_quantize(*ops[:3])
             ref = torq.torq_mxfp4_gemm(codes, scales, ops[3], ops[4], out_dtype=dt)
             exact = True
