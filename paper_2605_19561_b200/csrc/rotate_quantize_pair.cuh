@@ -222,7 +222,6 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       const int b0 = tcol >> 5;                          // first 32-block of the tile: even, 2 mod 4 for some narrow tiles
       const int nbb = narrow ? 3 : 4;                    // this warp's blocks: half of the tile's 8 or 6
       const bool last = FMT != FMT_F32OUT && tile + npairs >= total_tiles;
-      const bool waited = accumulator_is_waited_for(tile, npairs, C::NACC, total_tiles);   // by the issuer, two tiles later
       if (R_intra != nullptr) {
         // Executed by every epilogue thread for every tile, also after a wait has given up.
         named_barrier_sync(1, 256);
@@ -294,7 +293,8 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
           if (bb == nbb - 1) {                           // this warp's share is read: tell the leader if it waits for that
             tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0 && waited) mbar_arrive_cluster(map_to_cta(acce_bar(a), 0));
+            if (lane == 0 && accumulator_is_waited_for(tile, npairs, C::NACC, total_tiles))
+              mbar_arrive_cluster(map_to_cta(acce_bar(a), 0));
           }
           float z[32];
           if (R_intra != nullptr) {
