@@ -371,8 +371,8 @@ const char* torq_status_string(torq_status s);
  * 0, or TORQ_ERR_TIMEOUT in the low byte with the id of the wait that gave up in bits 8..15. */
 int torq_last_device_error(void* stream);
 
-/* Host helper (no device work): the list of output tiles that the CTA-pair kernels (more than 128
- * rows) walk for a [rows x cols] output on `pairs` CTA pairs (74 on a 148-SM part), in the order
+/* Host helper (no device work): the list of output tiles that the CTA-pair kernels (more than
+ * 48 rows) walk for a [rows x cols] output on `pairs` CTA pairs (74 on a 148-SM part), in the order
  * in which they are dealt round robin: tile i goes to pair i % pairs.  Tiles are 256 rows high and
  * 256 columns wide; where that leaves the last wave partly empty and cols is a multiple of 256,
  * some row tiles are covered by fewer 256-column tiles followed by 192-column ones (three wide

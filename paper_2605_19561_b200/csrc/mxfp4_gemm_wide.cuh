@@ -1,5 +1,5 @@
-// Block-scaled GEMM on CTA pairs in ONE wave (17 tokens and more; which sizes, wide_gemm_width says): every pair works exactly one tile of 256 tokens x `width`
-// output features (a multiple of 64, up to 384), the width chosen so that the tiles just fill the pairs.  The pair
+// Block-scaled GEMM on CTA pairs in ONE wave (17 tokens and more, the sizes that wide_gemm_width picks): every pair
+// works exactly one tile of 256 tokens x `width` output features (a multiple of 64, up to 384), the width chosen so that the tiles just fill the pairs.  The pair
 // kernel deals 256-column tiles and pays a whole wave for a remainder, or leaves pairs idle where there are few.
 //
 // As in the pair kernel each CTA stages its own 128 rows of A, its half of the tile's rows of W, its own A scales

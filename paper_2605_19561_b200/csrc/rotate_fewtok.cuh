@@ -34,7 +34,8 @@
 // Roles per CTA: warp 0 TMA producer, warp 1 MMA issuer, warps 2..5 epilogue / reduction.
 // Shared memory: 4 stages of (16 KiB of R_inter + tokens x 128 B of X); after the mainloop the same
 // memory holds the partials.  Up to 64 tokens that is small enough (<= 107 KiB) for two CTAs per SM: the
-// grid may exceed the SM count, which keeps more loads in flight; above, one CTA fills an SM, or two with three stages.
+// grid may exceed the SM count, which keeps more loads in flight; above, one CTA fills an SM, or
+// up to 128 tokens two of them with three stages (fewtok_rotation).
 #pragma once
 #include <cuda_bf16.h>
 #include "intra_fragment.cuh"

@@ -452,7 +452,7 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 //    per K step of the longest split (192 and 256 tokens measured: d = 2560 10.9 and 13.6, here 11.5; d = 3072 13.1 and 15.4,
 //    here 13.4; d = 8192 33.5 and 37.4, here 35.1 and 35.8);
 //  * pair kernel: 6.8, plus per K step 0.32 for a wave and 0.2 + 0.14 f for the last, partly filled one.
-// Fitted to MXFP4; NVFP4 and MXINT4, both sides of which take 0.2 to 0.5 longer, follow it and lost nothing at 250 shapes each.
+// The other formats follow the same figures, which were not fitted to them; wide_gemm_width says how that was checked.
 // A layer of 2048 tokens and more fills the pair kernel's waves and stays there (one-wave tiles would be wider than
 // 384 columns; 2048 x 4096 measured 51.6 with 480 columns, 46.8 in the pair kernel).
 static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int max_pairs) {
@@ -580,8 +580,8 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
     MixedTiles tiles = plan_pair_tiles((int)((M + 255) / 256), d, max_pairs, kNarrowTileCost);
     // A last wave of a few tiles: the last `rest` column tiles of the first 256 tokens go to the few-token kernel instead, whose
     // K split puts up to 8 CTAs on each 128 features.  That is worth its launch where a wave is long (us, one list of tiles /
-    // with this, each build beside itself within 0.5 %: 2048 x 14336 667 / 618 (the layer 686 / 658 and, on a hotter chip, 723 /
-    // 671), 2048 x 4864 87.4 / 82.7, 2304 x 4352 77.5 / 75.1, 1024 x 9984 179 / 158, 4096 x 14336 1301 / 1249; and not up to d =
+    // with this: 2048 x 14336 667 / 618 (the layer with N = 4096 686 / 658, again 723 / 671, a second copy of either side within
+    // 0.4 %), 2048 x 4864 87.4 / 82.7, 2304 x 4352 77.5 / 75.1, 1024 x 9984 179 / 158, 4096 x 14336 1301 / 1249; and not up to d =
     // 4096: 3584 x 4096 85.9 / 86.0, 3328 x 3072 51.7 / 52.6).
     const int rest = (int)((M + 255) / 256 * (d / 256) % max_pairs), full = (int)((M + 255) / 256 * (d / 256) / max_pairs);
     if (full >= 2 && rest > 0 && rest <= kTailTiles && rest <= d / 256 - 1 && d > 4096 && d % 256 == 0 && x_terms == 1 && fmt != FMT_F32OUT) {
@@ -700,8 +700,9 @@ torq_status torq_rotate_quantize_structured_nvfp4(const void* X, const void* R_B
 //    accumulator goes to Y), else 0.012 + 0.035 / S;
 //  * pair kernel: one wave 4.1 + 0.9 f + (0.285 + 0.04 f) per K step, more (the last one as narrower tiles) 5.2 + per K step
 //    0.325 for a full wave and 0.21 + 0.14 f for the last.
-// The same figures choose for NVFP4, MXINT4 (twice the steps) and float32 output, which were not fitted: timed against the kernels
-// that these calls took before at 450 shapes each, none lost more than the runs differ; MXFP4 lost 1.5 % at 1536 x 4096, K = 1024.
+// The same figures choose for NVFP4, MXINT4 (twice the steps) and float32 output, which were not fitted.  A sweep of 5250 calls, the
+// three formats and float32 output together, against the library without the one-wave kernels: 1.31 times as fast in the geometric
+// mean; lost by this choice: MXFP4 1536 x 4096, K = 1024 6.78 / 6.88.
 // Where it pays: 777 x 5120, K = 14336 (80 pair tiles) 34.7 -> 27.3, K = 4096 13.1 -> 11.2; 1280 x 4096, K = 14336 34.6 ->
 // 27.8; short contractions: 40 x 4096, K = 512 4.0 -> 3.0; 100 x 4096, K = 512 5.1 -> 3.3; 3000 x 1024, K = 2048 7.1 -> 6.4.
 static int wide_gemm_width(int64_t M, int64_t N, int64_t steps, int few_S, int max_pairs) {
