@@ -46,6 +46,7 @@ struct GemmPairCfgT {
   static constexpr int CH = FMT == FMT_NVFP4 ? 4 : (FMT == FMT_MXINT4 ? 1 : 2);   // scale chunks per stage and 128 rows
   static constexpr int SF_BOXES = CH == 1 ? 1 : CH / 2;       // scale loads per stage and 128 rows:
   static constexpr int SF_BOX_WORDS = CH == 1 ? 128 : 256;    // 1 KiB (two chunks), or the single chunk
+  static constexpr int SF_BOX_BYTES = SF_BOX_WORDS * 4;
   static constexpr int SFA_BYTES = CH * 512;
   static constexpr int SFB_BYTES = 2 * SFA_BYTES;      // both 128-row tiles of the W scales
   static constexpr int STAGE_TX = A_BYTES + B_BYTES + SFA_BYTES + SFB_BYTES;      // bytes one CTA loads per stage
@@ -81,6 +82,7 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
   auto empty_bar = [&](int s) { return bar_base + 8u * (C::STAGES + s); };
   const uint32_t accf_bar = bar_base + 8u * (2 * C::STAGES);
   const uint32_t acce_bar = bar_base + 8u * (2 * C::STAGES + 1);
+  const uint32_t alloc_bar = bar_base + 8u * (2 * C::STAGES + 2);   // in the leader: the other CTA's tensor memory is allocated
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + bar_off + 192);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(smem_gen + bar_off + 200);
 
@@ -94,91 +96,88 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
   // accumulator is free.  8192 tokens x 14336 features, K = 4096: 181.7 -> 172.5 us, K = 2048 107.5 -> 103.8; K = 1024 lost 3 %.
   const bool long_k = k_tiles >= 8;
 
+  // Set-up as in the pair rotation kernel: the producer waits for nothing but the barriers of both CTAs.
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     mbar_init(accf_bar, 1);
     mbar_init(acce_bar, 16);
+    mbar_init(alloc_bar, 1);
     *cta_abort = 0;
     fence_mbar_init();
   }
-  if (warp == 1) { tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(tmem_slot)), C::TMEM_COLS); tmem_relinquish_pair(); }
-  tc_fence_before_sync();
-  __syncthreads();
-  cluster_sync_after_init();
-  tc_fence_after_sync();
-  const uint32_t tmem_base = *tmem_slot;
+  if (warp == 2 && elect_one()) {
+    tma_prefetch_desc(&tmB); tma_prefetch_desc(&tmSFB); tma_prefetch_desc(&tmBn);
+    tma_prefetch_desc(&tmA); tma_prefetch_desc(&tmSFA);
+  }
+  __syncwarp();
+  cluster_arrive_relaxed();
+  int mp0, tcol0;                                      // this pair's first tile
+  bool narrow0;
+  mixed_tile_coords(pair, tiles, mp0, tcol0, narrow0);
+  const int pre = k_tiles < C::STAGES ? k_tiles : C::STAGES;
+  uint32_t tmem_base = 0;
+  if (warp == 0) {
+    named_barrier_arrive(2, C::THREADS);
+    cluster_wait();                                    // both CTAs' barriers exist before any remote arrive
+  } else {
+    if (warp == 1) { tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(tmem_slot)), C::TMEM_COLS); tmem_relinquish_pair(); }
+    tc_fence_before_sync();
+    named_barrier_sync(2, C::THREADS);
+    cluster_wait();
+    tc_fence_after_sync();
+    tmem_base = *tmem_slot;
+    if (warp == 1 && rank == 1 && lane == 0) mbar_arrive_cluster(map_to_cta(alloc_bar, 0));   // this CTA's tensor memory is there
+  }
   // Set-up above touched no global memory.  The weights and their scales are constants of the
   // layer, never the output of the kernel that runs just before this one, so the producer starts
   // the first stages' W loads right away; everything else waits until that kernel has completed
   // (its output, the activations' codes and scales, is what the A-side loads read).
   griddep_launch_dependents();
-  const int pre = pair < total_tiles ? (k_tiles < C::STAGES ? k_tiles : C::STAGES) : 0;
-  if (warp == 0) {
-    if (elect_one()) {
-      tma_prefetch_desc(&tmA); tma_prefetch_desc(&tmB);
-      tma_prefetch_desc(&tmSFA); tma_prefetch_desc(&tmSFB);
-      int mp0 = 0, col0 = 0;
-      bool narrow = false;
-      if (pre > 0) { mixed_tile_coords(pair, tiles, mp0, col0, narrow); tma_prefetch_desc(&tmBn); }
-      (void)mp0;
-      const int bn_half = narrow ? kNarrowCols / 2 : BN / 2;
-      for (int kt = 0; kt < pre; ++kt) {
-        const uint32_t st = smem_base + kt * C::STAGE_BYTES;
-        const uint32_t leader_full = map_to_cta(full_bar(kt), 0);
-        if (rank == 0) mbar_arrive_expect_tx(full_bar(kt), 2 * (C::STAGE_TX - (BN / 2 - bn_half) * 128));
-        tma_load_2d_pair(st + C::A_BYTES, narrow ? &tmBn : &tmB, kt * 128, col0 + (int)rank * bn_half, leader_full);
+
+  // Scale tiles: one row of the [row tile, chunk x 512 B] view per 128 rows, in boxes of 1 KiB (two chunks; both row tiles
+  // of W in one box); anything outside the buffer arrives as zeros (scale 2^-127 or 0, multiplying operand data that is zero
+  // there as well).
+  auto load_a = [&](int s, int kt, int mt) {
+    const uint32_t st = smem_base + s * C::STAGE_BYTES;
+    const uint32_t leader_full = map_to_cta(full_bar(s), 0);
+    tma_load_2d_pair(st, &tmA, kt * 128, mt * C::BM, leader_full);
 #pragma unroll
-        for (int t = 0; t < 2; ++t)                      // one 1 KiB box = two chunks
-#pragma unroll
-          for (int b = 0; b < C::SF_BOXES; ++b)
-            tma_load_2d_pair(st + C::A_BYTES + C::B_BYTES + C::SFA_BYTES + t * C::SFA_BYTES + b * 1024, &tmSFB,
-                             kt * CH * 128 + b * 256, (col0 >> 7) + t, leader_full);
-      }
-    }
-    __syncwarp();
-  }
-  griddep_wait();
+    for (int b = 0; b < C::SF_BOXES; ++b)
+      tma_load_2d_pair(st + C::A_BYTES + C::B_BYTES + b * C::SF_BOX_BYTES, &tmSFA, kt * CH * 128 + b * 256, mt, leader_full);
+  };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (both CTAs)
-    uint32_t it = 0;
-    bool ok = true;
-    for (int tile = pair; tile < total_tiles && ok; tile += npairs) {
-      int mp, tcol;
-      bool narrow;
-      mixed_tile_coords(tile, tiles, mp, tcol, narrow);
-      const int mt = 2 * mp + (int)rank;
-      // a 192-column tile takes 96 rows of W per CTA; its scale rows start at a multiple of 64, so the two
-      // 128-row scale chunks from (tcol / 128) on still cover it
+    // a 192-column tile takes 96 rows of W per CTA; its scale rows start at a multiple of 64, so the two
+    // 128-row scale chunks from (tcol / 128) on still cover it
+    auto load_w = [&](int s, int kt, int tcol, bool narrow) {
+      const uint32_t st = smem_base + s * C::STAGE_BYTES;
+      const uint32_t leader_full = map_to_cta(full_bar(s), 0);
       const int bn_half = narrow ? kNarrowCols / 2 : BN / 2;
-      const uint32_t stage_tx = 2 * (C::STAGE_TX - (BN / 2 - bn_half) * 128);
-      for (int kt = 0; kt < k_tiles; ++kt, ++it) {
+      if (rank == 0) mbar_arrive_expect_tx(full_bar(s), 2 * (C::STAGE_TX - (BN / 2 - bn_half) * 128));
+      tma_load_2d_pair(st + C::A_BYTES, narrow ? &tmBn : &tmB, kt * 128, tcol + (int)rank * bn_half, leader_full);
+#pragma unroll
+      for (int b = 0; b < C::SF_BOXES; ++b)
+        tma_load_2d_pair(st + C::A_BYTES + C::B_BYTES + C::SFA_BYTES + b * 2 * C::SF_BOX_BYTES, &tmSFB, kt * CH * 128 + b * 256,
+                         tcol >> 7, leader_full);
+    };
+    if (elect_one())
+      for (int kt = 0; kt < pre; ++kt) load_w(kt, kt, tcol0, narrow0);
+    __syncwarp();
+    griddep_wait();
+    uint32_t it = pre;                                 // warp 2 sends the A-side loads of the first stages
+    bool ok = true;
+    int mp = mp0, tcol = tcol0, kt = pre;
+    bool narrow = narrow0;
+    for (int tile = pair; tile < total_tiles && ok; tile += npairs) {
+      if (tile != pair) { mixed_tile_coords(tile, tiles, mp, tcol, narrow); kt = 0; }
+      for (; kt < k_tiles; ++kt, ++it) {
         const int s = it % C::STAGES;
         if (!mbar_wait_cluster_warp(empty_bar(s), ((it / C::STAGES) & 1) ^ 1, cta_abort, err_word,
                                SITE_PRODUCER_EMPTY)) { ok = false; break; }
-        const uint32_t st = smem_base + s * C::STAGE_BYTES;
-        const uint32_t leader_full = map_to_cta(full_bar(s), 0);
         if (elect_one()) {
-          const bool w_issued = it < (uint32_t)pre;      // W side of this stage went out before the wait above
-          if (rank == 0 && !w_issued) mbar_arrive_expect_tx(full_bar(s), stage_tx);
-          tma_load_2d_pair(st, &tmA, kt * 128, mt * C::BM, leader_full);
-          if (!w_issued)
-            tma_load_2d_pair(st + C::A_BYTES, narrow ? &tmBn : &tmB, kt * 128, tcol + (int)rank * bn_half, leader_full);
-          // scale tiles: one row of the [row tile, chunk x 512 B] view per 128 rows, in boxes of
-          // 1 KiB (two chunks); anything outside the buffer arrives as zeros (scale 2^-127 or 0,
-          // multiplying operand data that is zero there as well).
-#pragma unroll
-          for (int b = 0; b < C::SF_BOXES; ++b)
-            tma_load_2d_pair(st + C::A_BYTES + C::B_BYTES + b * 1024, &tmSFA, kt * CH * 128 + b * 256, mt,
-                             leader_full);
-          if (!w_issued) {
-#pragma unroll
-            for (int t = 0; t < 2; ++t)
-#pragma unroll
-              for (int b = 0; b < C::SF_BOXES; ++b)
-                tma_load_2d_pair(st + C::A_BYTES + C::B_BYTES + C::SFA_BYTES + t * C::SFA_BYTES + b * 1024, &tmSFB,
-                                 kt * CH * 128 + b * 256, (tcol >> 7) + t, leader_full);
-          }
+          load_w(s, kt, tcol, narrow);
+          load_a(s, kt, 2 * mp + (int)rank);
         }
         __syncwarp();
       }
@@ -187,7 +186,7 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     // ------------------------------------------------------------------ MMA issuer (leader only)
     if (rank == 0) {
       uint32_t it = 0, tcount = 0;
-      bool ok = true;
+      bool ok = mbar_wait_cluster_warp(alloc_bar, 0, cta_abort, err_word, SITE_MMA_ACC_EMPTY);
       // instruction descriptors differ between the two tile widths only in the N field ([17,23) = N >> 3)
       constexpr uint32_t n_less = (uint32_t)((BN - kNarrowCols) >> 3) << 17;
       const uint32_t sfa_t = tmem_base + C::SFA_COL, sfb_t = tmem_base + C::SFB_COL;
@@ -217,13 +216,14 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
           const uint64_t sfb_d = make_desc(st + C::A_BYTES + C::B_BYTES + C::SFA_BYTES, 0, 128, 0);
           auto copy_scales = [&]() {
             // scale chunks shared -> tensor memory (descriptor address unit = 16 B: +32 = next
-            // chunk, + SFA_BYTES / 16 = second 128-row tile of W), then 64 elements of K per instruction
+            // chunk of a box, + SF_BOX_BYTES / 16 = second 128-row tile of W), then 64 elements of K per instruction
 #pragma unroll
             for (int c = 0; c < CH; ++c) {
               if (c < CH / 2 || two) {
                 tmem_cp_32x128b_warpx4_pair(sfa_t + 4 * c, sfa_d + 32 * c);
-                tmem_cp_32x128b_warpx4_pair(sfb_t + 8 * c, sfb_d + 32 * c);
-                tmem_cp_32x128b_warpx4_pair(sfb_t + 8 * c + 4, sfb_d + 32 * c + C::SFA_BYTES / 16);
+                const uint64_t w = sfb_d + (c >> 1) * 2 * (C::SF_BOX_BYTES / 16) + 32 * (c & 1);
+                tmem_cp_32x128b_warpx4_pair(sfb_t + 8 * c, w);
+                tmem_cp_32x128b_warpx4_pair(sfb_t + 8 * c + 4, w + C::SF_BOX_BYTES / 16);
               }
             }
           };
@@ -274,6 +274,14 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       }
     }
   } else {
+    griddep_wait();
+    if (warp == 2) {
+      // The A-side loads of the first stages: from a warp of its own, so that they go out when the kernel before has completed
+      // and not behind the W loads of all these stages.
+      if (elect_one())
+        for (int kt = 0; kt < pre; ++kt) load_a(kt, kt, 2 * mp0 + (int)rank);
+      __syncwarp();
+    }
     // ------------------------------------------------------------------ epilogue (8 warps per CTA)
     const int q = warp & 3;
     const int h = (warp - 2) >> 2;                       // column half

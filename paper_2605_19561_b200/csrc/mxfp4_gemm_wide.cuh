@@ -87,6 +87,11 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     *cta_abort = 0;
     fence_mbar_init();
   }
+  if (warp == 2 && elect_one()) {
+    tma_prefetch_desc(&tmB); tma_prefetch_desc(&tmB1); tma_prefetch_desc(&tmSFB);
+    tma_prefetch_desc(&tmA); tma_prefetch_desc(&tmSFA); tma_prefetch_desc(&tmY);
+  }
+  __syncwarp();
   if (warp == 1) { tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512); tmem_relinquish_pair(); }
   tc_fence_before_sync();
   __syncthreads();
@@ -96,6 +101,16 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
   // The weights and their scales are constants of the layer, never the output of the kernel that runs just before
   // this one: their loads for the first stages go out now, everything else waits for that kernel to complete.
   griddep_launch_dependents();
+  const int pre = k_tiles < nst ? k_tiles : nst;
+
+  auto load_a = [&](int s, int kt) {
+    const uint32_t st = smem_base + s * stage_bytes, bar = map_to_cta(full_bar(s), 0);
+    tma_load_2d_pair(st, &tmA, kt * 128, mt * C::BM, bar);
+    // anything outside the buffer arrives as zeros (scale 2^-127 or 0, on operand data that is zero as well)
+#pragma unroll
+    for (int b = 0; b < C::SF_BOXES; ++b)
+      tma_load_2d_pair(st + sfa_off + b * C::SF_BOX_BYTES, &tmSFA, kt * CH * 128 + b * C::SF_BOX_WORDS, mt, bar);
+  };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (both CTAs)
@@ -110,22 +125,14 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         for (int b = 0; b < C::SF_BOXES; ++b)
           tma_load_2d_pair(st + sfb_off + b * nchk * C::SF_BOX_BYTES, &tmSFB, kt * CH * 128 + b * C::SF_BOX_WORDS, tcol >> 7, bar);
       };
-      tma_prefetch_desc(&tmA); tma_prefetch_desc(&tmB); tma_prefetch_desc(&tmB1);
-      tma_prefetch_desc(&tmSFA); tma_prefetch_desc(&tmSFB); tma_prefetch_desc(&tmY);
-      const int pre = k_tiles < nst ? k_tiles : nst;
       for (int i = 0; i < pre; ++i) load_w(i, i);
       griddep_wait();
-      int s = 0;
-      uint32_t ph = 1;
-      for (int kt = 0; kt < k_tiles; ++kt) {
+      int s = 0;                                       // warp 2 sends the A-side loads of the first stages
+      uint32_t ph = 0;
+      for (int kt = pre; kt < k_tiles; ++kt) {
         if (!mbar_wait_cluster(empty_bar(s), ph, cta_abort, err_word, SITE_PRODUCER_EMPTY)) break;
-        if (kt >= pre) load_w(s, kt);
-        const uint32_t st = smem_base + s * stage_bytes, bar = leader_full0 + 8u * s;
-        tma_load_2d_pair(st, &tmA, kt * 128, mt * C::BM, bar);
-        // anything outside the buffer arrives as zeros (scale 2^-127 or 0, on operand data that is zero as well)
-#pragma unroll
-        for (int b = 0; b < C::SF_BOXES; ++b)
-          tma_load_2d_pair(st + sfa_off + b * C::SF_BOX_BYTES, &tmSFA, kt * CH * 128 + b * C::SF_BOX_WORDS, mt, bar);
+        load_w(s, kt);
+        load_a(s, kt);
         if (++s == nst) { s = 0; ph ^= 1; }
       }
     }
@@ -205,6 +212,11 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     const int q = warp & 3;
     const int set = (warp - 2) >> 2;
     griddep_wait();                                    // Y may still be read by that kernel
+    if (warp == 2) {                                   // from a warp of its own: not behind the W loads of all these stages
+      if (elect_one())
+        for (int i = 0; i < pre; ++i) load_a(i, i);
+      __syncwarp();
+    }
     bool ok = mbar_wait_cluster(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
     ok = __all_sync(0xFFFFFFFFu, ok);
     const int row0 = mt * C::BM + q * 32;

@@ -70,6 +70,7 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   auto empty_bar = [&](int s) { return bar_base + 8u * (C::STAGES + s); };
   auto accf_bar = [&](int a) { return bar_base + 8u * (2 * C::STAGES + a); };
   auto acce_bar = [&](int a) { return bar_base + 8u * (2 * C::STAGES + C::NACC + a); };
+  const uint32_t alloc_bar = bar_base + 8u * (2 * C::STAGES + 2 * C::NACC);   // in the leader: the other CTA's tensor memory is allocated
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + bar_off + 192);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(smem_gen + bar_off + 200);
 
@@ -83,75 +84,77 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   const int nblocks = d / 32;
   const int kb4 = (nblocks + 3) / 4;
 
+  // Set-up.  The producer waits for nothing but the barriers of both CTAs, whose cluster barrier therefore comes before the
+  // tensor-memory allocation; the other warps meet behind both on a barrier that the producer only counts itself on.  A CTA whose
+  // SM the kernel before leaves last sets the time here: device timestamps, 2048 x 4096, from that kernel's completion to
+  // the last pair's first full stage 3.6 us, 2.3 with this set-up and the first X loads from a warp of their own (the layer
+  // with N = 6144 84.9 -> 83.9 us, at the power cap; rotation and GEMM have it).
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int a = 0; a < C::NACC; ++a) { mbar_init(accf_bar(a), 1); mbar_init(acce_bar(a), 16); }
+    mbar_init(alloc_bar, 1);
     *cta_abort = 0;
     fence_mbar_init();
   }
-  if (warp == 1) { tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(tmem_slot)), C::TMEM_COLS); tmem_relinquish_pair(); }
-  tc_fence_before_sync();
-  __syncthreads();
-  cluster_sync_after_init();                                  // both CTAs' barriers exist before any remote arrive
-  tc_fence_after_sync();
-  const uint32_t tmem_base = *tmem_slot;
+  if (warp == 2 && elect_one()) { tma_prefetch_desc(&tmX); tma_prefetch_desc(&tmR); tma_prefetch_desc(&tmRn); }
+  __syncwarp();
+  cluster_arrive_relaxed();
+  int mp0, tcol0;                                      // this pair's first tile
+  bool narrow0;
+  mixed_tile_coords(pair, tiles, mp0, tcol0, narrow0);
+  const int pre = k_tiles < C::STAGES ? k_tiles : C::STAGES;
+  uint32_t tmem_base = 0;
+  if (warp == 0) {
+    named_barrier_arrive(2, C::THREADS);
+    cluster_wait();                                    // both CTAs' barriers exist before any remote arrive
+  } else {
+    if (warp == 1) { tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(tmem_slot)), C::TMEM_COLS); tmem_relinquish_pair(); }
+    tc_fence_before_sync();
+    named_barrier_sync(2, C::THREADS);
+    cluster_wait();
+    tc_fence_after_sync();
+    tmem_base = *tmem_slot;
+    if (warp == 1 && rank == 1 && lane == 0) mbar_arrive_cluster(map_to_cta(alloc_bar, 0));   // this CTA's tensor memory is there
+  }
   // Set-up above touched no global memory; from here on the previous kernel's results are needed.
   // R_inter is a constant of the layer, never the output of the kernel that runs just before this
   // one: the producer starts the first stages' R_inter loads right away; the X loads and all
   // other global accesses wait until that kernel has completed.
   griddep_launch_dependents();
-  const int pre = pair < total_tiles ? (k_tiles < C::STAGES ? k_tiles : C::STAGES) : 0;
-  if (warp == 0) {
-    if (elect_one()) {
-      tma_prefetch_desc(&tmX);
-      tma_prefetch_desc(&tmR);
-      int mp0 = 0, col0 = 0;
-      bool narrow = false;
-      if (pre > 0) mixed_tile_coords(pair, tiles, mp0, col0, narrow);
-      (void)mp0;
-      const int my_col = col0 + (int)rank * (narrow ? kNarrowCols / 2 : BN / 2);
-      if (narrow) tma_prefetch_desc(&tmRn);
-      for (int kt = 0; kt < pre; ++kt) {
-        const uint32_t st = smem_base + kt * C::STAGE_BYTES;
-        const uint32_t leader_full = map_to_cta(full_bar(kt), 0);
-        if (rank == 0) mbar_arrive_expect_tx(full_bar(kt), 2 * (C::STAGE_BYTES - (narrow ? C::B_BOX_BYTES / 2 : 0)));
-        tma_load_2d_pair(st + C::A_BYTES, &tmR, my_col, (kt % kr_tiles) * C::BK, leader_full);
-        tma_load_2d_pair(st + C::A_BYTES + C::B_BOX_BYTES, narrow ? &tmRn : &tmR, my_col + 64, (kt % kr_tiles) * C::BK,
-                         leader_full);
-      }
-    }
-    __syncwarp();
-  }
-  griddep_wait();
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (both CTAs)
-    uint32_t it = 0;
+    // A 192-column tile takes 96 columns of R_inter per CTA: one 64-column box and one 32-column box.
+    // Under the 128-byte swizzle a box whose rows are 64 bytes long still lands on a 128-byte pitch, i.e.
+    // as the first half of the 64-column layout the instruction's descriptor describes.
+    auto load_r = [&](int s, int kr, int my_col, bool narrow) {
+      const uint32_t st = smem_base + s * C::STAGE_BYTES;
+      const uint32_t leader_full = map_to_cta(full_bar(s), 0);
+      if (rank == 0) mbar_arrive_expect_tx(full_bar(s), 2 * (C::STAGE_BYTES - (narrow ? C::B_BOX_BYTES / 2 : 0)));
+      tma_load_2d_pair(st + C::A_BYTES, &tmR, my_col, kr * C::BK, leader_full);
+      tma_load_2d_pair(st + C::A_BYTES + C::B_BOX_BYTES, narrow ? &tmRn : &tmR, my_col + 64, kr * C::BK, leader_full);
+    };
+    if (elect_one()) {
+      const int my_col = tcol0 + (int)rank * (narrow0 ? kNarrowCols / 2 : BN / 2);
+      for (int kt = 0; kt < pre; ++kt) load_r(kt, kt % kr_tiles, my_col, narrow0);
+    }
+    __syncwarp();
+    griddep_wait();
+    uint32_t it = pre;                                 // warp 2 sends the X loads of the first stages
     bool ok = true;
+    int mp = mp0, tcol = tcol0, kt = pre, kr = pre % kr_tiles;
+    bool narrow = narrow0;
     for (int tile = pair; tile < total_tiles && ok; tile += npairs) {
-      int mp, tcol;
-      bool narrow;
-      mixed_tile_coords(tile, tiles, mp, tcol, narrow);
+      if (tile != pair) { mixed_tile_coords(tile, tiles, mp, tcol, narrow); kt = 0; kr = 0; }
       const int mt = 2 * mp + (int)rank;
-      // A 192-column tile takes 96 columns of R_inter per CTA: one 64-column box and one 32-column box.
-      // Under the 128-byte swizzle a box whose rows are 64 bytes long still lands on a 128-byte pitch, i.e.
-      // as the first half of the 64-column layout the instruction's descriptor describes.
       const int my_col = tcol + (int)rank * (narrow ? kNarrowCols / 2 : BN / 2);
-      const uint32_t stage_tx = 2 * (C::STAGE_BYTES - (narrow ? C::B_BOX_BYTES / 2 : 0));
-      for (int kt = 0, kr = 0; kt < k_tiles; ++kt, ++it, kr = (kr + 1 == kr_tiles ? 0 : kr + 1)) {
+      for (; kt < k_tiles; ++kt, ++it, kr = (kr + 1 == kr_tiles ? 0 : kr + 1)) {
         const int s = it % C::STAGES;
         if (!mbar_wait_cluster_warp(empty_bar(s), ((it / C::STAGES) & 1) ^ 1, cta_abort, err_word,
                                SITE_PRODUCER_EMPTY)) { ok = false; break; }
-        const uint32_t st = smem_base + s * C::STAGE_BYTES;
-        const uint32_t leader_full = map_to_cta(full_bar(s), 0);
         if (elect_one()) {
-          const bool r_issued = it < (uint32_t)pre;      // R side of this stage went out before the wait above
-          if (rank == 0 && !r_issued) mbar_arrive_expect_tx(full_bar(s), stage_tx);
-          tma_load_2d_pair(st, &tmX, kt * C::BK, mt * C::BM, leader_full);
-          if (!r_issued) {
-            tma_load_2d_pair(st + C::A_BYTES, &tmR, my_col, kr * C::BK, leader_full);
-            tma_load_2d_pair(st + C::A_BYTES + C::B_BOX_BYTES, narrow ? &tmRn : &tmR, my_col + 64, kr * C::BK, leader_full);
-          }
+          load_r(s, kr, my_col, narrow);
+          tma_load_2d_pair(smem_base + s * C::STAGE_BYTES, &tmX, kt * C::BK, mt * C::BM, map_to_cta(full_bar(s), 0));
         }
         __syncwarp();
       }
@@ -162,7 +165,7 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       constexpr uint32_t idesc_wide = idesc_bf16(256, BN, /*A MN-major*/ false, /*B MN-major*/ true);
       constexpr uint32_t idesc_narrow = idesc_bf16(256, kNarrowCols, false, true);
       uint32_t it = 0, tcount = 0;
-      bool ok = true;
+      bool ok = mbar_wait_cluster_warp(alloc_bar, 0, cta_abort, err_word, SITE_MMA_ACC_EMPTY);
       for (int tile = pair; tile < total_tiles && ok; tile += npairs, ++tcount) {
         int mp, tcol;
         bool narrow;
@@ -196,6 +199,15 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       }
     }
   } else {
+    griddep_wait();
+    if (warp == 2) {
+      // The X loads of the first stages: from a warp of its own, so that they go out when the kernel before has completed and
+      // not behind the R_inter loads of all these stages (a CTA that finds its SM late is not through with those by then).
+      if (elect_one())
+        for (int kt = 0; kt < pre; ++kt)
+          tma_load_2d_pair(smem_base + kt * C::STAGE_BYTES, &tmX, kt * C::BK, (2 * mp0 + (int)rank) * C::BM, map_to_cta(full_bar(kt), 0));
+      __syncwarp();
+    }
     // ------------------------------------------------------------------ epilogue (8 warps per CTA)
     // warp w reads lane quarter w % 4 (32 rows) and column half (w - 2) / 4 (four 32-blocks = one
     // 4-byte group of scale bytes; three blocks in a 192-column tile).  Two forms of the intra-block rotation:

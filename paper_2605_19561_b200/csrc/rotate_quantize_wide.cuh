@@ -75,6 +75,7 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (C::MAX_STAGES + s); };
   const uint32_t accf_bar = bar_base + 8u * (2 * C::MAX_STAGES);
+  const uint32_t alloc_bar = accf_bar + 8;             // in the leader: the other CTA's tensor memory is allocated
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + bar_off + 192);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(smem_gen + bar_off + 200);
 
@@ -86,21 +87,35 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   const int k_tiles = d / C::BK;
   const int n0 = C::n0(width);
 
+  // Set-up as in the pair kernels: the producer waits for nothing but the barriers of both CTAs, and the first stages' X loads
+  // come from a warp of their own (us, before / after: 200 x 1024 5.25 / 4.87, 200 x 2048 9.35 / 8.42, 300 x 4096 19.2 / 18.5).
   if (threadIdx.x == 0) {
     for (int s = 0; s < nst; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     mbar_init(accf_bar, 1);
+    mbar_init(alloc_bar, 1);
     *cta_abort = 0;
     fence_mbar_init();
   }
-  if (warp == 1) { tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512); tmem_relinquish_pair(); }
-  tc_fence_before_sync();
-  __syncthreads();
-  cluster_sync_after_init();
-  tc_fence_after_sync();
-  const uint32_t tmem_base = *tmem_slot;
+  if (warp == 2 && elect_one()) { tma_prefetch_desc(&tmX); tma_prefetch_desc(&tmR); tma_prefetch_desc(&tmRt); }
+  __syncwarp();
+  cluster_arrive_relaxed();
+  uint32_t tmem_base = 0;
+  if (warp == 0) {
+    named_barrier_arrive(2, C::THREADS);
+    cluster_wait();                                    // both CTAs' barriers exist before any remote arrive
+  } else {
+    if (warp == 1) { tmem_alloc_pair(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512); tmem_relinquish_pair(); }
+    tc_fence_before_sync();
+    named_barrier_sync(2, C::THREADS);
+    cluster_wait();
+    tc_fence_after_sync();
+    tmem_base = *tmem_slot;
+    if (warp == 1 && rank == 1 && lane == 0) mbar_arrive_cluster(map_to_cta(alloc_bar, 0));   // this CTA's tensor memory is there
+  }
   // R_inter is a constant of the layer, never the output of the kernel that runs just before this one: its
   // loads for the first stages go out now, everything else waits for that kernel to complete.
   griddep_launch_dependents();
+  const int pre = k_tiles < nst ? k_tiles : nst;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (both CTAs)
@@ -120,15 +135,13 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
         }
         if constexpr (TWO) tma_load_2d_pair(dst, &tmR, col1, kt * C::BK, bar);
       };
-      tma_prefetch_desc(&tmX); tma_prefetch_desc(&tmR); tma_prefetch_desc(&tmRt);
-      const int pre = k_tiles < nst ? k_tiles : nst;
       for (int i = 0; i < pre; ++i) load_r(i, i);
       griddep_wait();
-      int s = 0;
-      uint32_t ph = 1;
-      for (int kt = 0; kt < k_tiles; ++kt) {
+      int s = 0;                                       // warp 2 sends the X loads of the first stages
+      uint32_t ph = 0;
+      for (int kt = pre; kt < k_tiles; ++kt) {
         if (!mbar_wait_cluster(empty_bar(s), ph, cta_abort, err_word, SITE_PRODUCER_EMPTY)) break;
-        if (kt >= pre) load_r(s, kt);
+        load_r(s, kt);
         tma_load_2d_pair(smem_base + s * stage_bytes, &tmX, kt * C::BK, mt * C::BM, leader_full0 + 8u * s);
         if (++s == nst) { s = 0; ph ^= 1; }
       }
@@ -136,7 +149,7 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader only)
-    if (rank == 0 && elect_one()) {
+    if (rank == 0 && mbar_wait_cluster_warp(alloc_bar, 0, cta_abort, err_word, SITE_MMA_ACC_EMPTY) && elect_one()) {
       const uint32_t idesc0 = idesc_bf16(256, n0, /*A MN-major*/ false, /*B MN-major*/ true);
       constexpr uint32_t idesc1 = idesc_bf16(256, 128, false, true);
       int s = 0;
@@ -168,6 +181,14 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
     const int p = lane & 3, r8 = lane >> 2;
     const int nblocks = d / 32, nb = width / 32, b0 = tcol >> 5;
     const uint32_t ri_saddr = smem_base + ri_off;
+    if (warp == 2) {
+      // X loads of the first stages, from a warp of its own: not behind the R_inter loads of all these stages
+      griddep_wait();
+      if (elect_one())
+        for (int i = 0; i < pre; ++i)
+          tma_load_2d_pair(smem_base + i * stage_bytes, &tmX, i * C::BK, mt * C::BM, map_to_cta(full_bar(i), 0));
+      __syncwarp();
+    }
     if (R_intra != nullptr) {                          // the tile's blocks, 16-byte piece c of row i at c ^ ((i >> 1) & 3)
       for (int idx = (warp - 2) * 32 + lane; idx < nb * 128; idx += 128 * C::ESETS) {
         const int lb = idx >> 7, i = (idx >> 2) & 31, c = idx & 3;

@@ -806,7 +806,7 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
       !encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, BN / 2, 128) ||
       !encode_2d(&tmSFA, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, As, (uint64_t)((M + 127) / 128), kb4 * 128, 1, sf_box,
                  CU_TENSOR_MAP_SWIZZLE_NONE) ||
-      !encode_2d(&tmSFB, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, Ws, (uint64_t)((N + 127) / 128), kb4 * 128, 1, sf_box,
+      !encode_2d(&tmSFB, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, Ws, (uint64_t)((N + 127) / 128), kb4 * 128, 2, sf_box,
                  CU_TENSOR_MAP_SWIZZLE_NONE))
     return TORQ_ERR_LAUNCH;
   CUtensorMap tmY;
