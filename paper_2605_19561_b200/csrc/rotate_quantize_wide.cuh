@@ -10,11 +10,12 @@
 // side by side in tensor memory (column c of the tile is accumulator column c).  An instruction costs at least
 // 45 cycles however narrow (256 + 32 columns ran at 692 cycles per K step, 160 + 128 at 576), so the second one is
 // always 128 columns.  Each CTA of the pair stages its 128 rows of X and half of each instruction's columns of
-// R_inter: 64-column boxes of 8 KiB and, when half of the first instruction is no multiple of 64, one narrower box
+// R_inter: 64-column boxes of 8 KiB (16 KiB up to 128 columns, where a stage is 128 of K) and, when half of the first instruction is no multiple of 64, one narrower box
 // (its rows keep the 128-byte pitch of the swizzle) in a slot of the same size.
 //
-// Bounds: up to 256 columns the operand bytes (52 to 66 B per cycle and SM cross from L2: 440 cycles per K step at 64
-// columns, 460 at 128, 500 at 256, where the math takes 2 cycles per column), above the math; then the
+// Bounds: up to 256 columns the latency of the loads and of the hand-overs between the roles (440 cycles per 64 of K at 64
+// columns, 460 at 128, 500 at 256 with stages of 64; the same loads alone, from L2, run at 22 TB/s; an instruction takes the
+// larger of 2 cycles per column and a quarter of that plus 64 for its X slice), above the math; then the
 // epilogue, which nothing overlaps.  It is the fast form (warp-level MMAs on the accumulator fragments), bound by
 // those MMAs: about 860 cycles per 32 columns.  Splitting K over the pairs of a larger cluster (partial sums
 // exchanged through distributed shared memory) was measured and brought nothing: 300 x 4096 20.9 with two pairs
@@ -31,9 +32,13 @@ namespace torq {
 
 struct RotWideCfg {
   static constexpr int BM = 128;                       // rows per CTA
-  static constexpr int BK = 64;
-  static constexpr int A_BYTES = BM * BK * 2;          // 16 KiB
-  static constexpr int BOX_BYTES = 64 * BK * 2;        // 64 columns x 64 k = 8 KiB
+  static constexpr int SLAB = 64;                      // K elements of one 128-byte row of X
+  // K per stage: two slabs up to 128 columns, where the waits and the issue of loads per step bound a step and not its math (us, one
+  // slab / two: 200 tokens d = 1024 4.87 / 4.48, d = 2048 8.42 / 7.57, 300 tokens d = 4096 18.4 / 17.1; loops of the whole warp
+  // instead of one thread 5.51 and 9.10); above, three stages of twice the size lose against six (600 x 4096, 192 columns, 22.5 / 25.9)
+  __host__ __device__ static constexpr int bk(int width) { return width <= 128 ? 2 * SLAB : SLAB; }
+  __host__ __device__ static constexpr int a_bytes(int width) { return BM * bk(width) * 2; }       // 32 or 16 KiB
+  __host__ __device__ static constexpr int box_bytes(int width) { return 64 * bk(width) * 2; }     // 64 columns of R_inter
   static constexpr int MAX_WIDTH = 384;
   static constexpr int MAX_STAGES = 8;
   static constexpr int RI_BLOCK_BYTES = 32 * 64;       // R_intra[blk] as bf16 rows of 64 bytes, 16-byte pieces XOR-swizzled
@@ -43,10 +48,10 @@ struct RotWideCfg {
   __host__ __device__ static constexpr int n0(int width) { return width <= 256 ? width : width - 128; }
   __host__ __device__ static constexpr int boxes(int width) { return (n0(width) / 2 + 63) / 64 + (width > 256 ? 1 : 0); }
   __host__ __device__ static constexpr int tail_cols(int width) { return n0(width) / 2 % 64; }         // columns of the narrow box (0: none)
-  __host__ __device__ static constexpr int stage_bytes(int width) { return A_BYTES + boxes(width) * BOX_BYTES; }
-  __host__ __device__ static constexpr int stage_tx(int width) { return A_BYTES + width / 2 * BK * 2; }   // bytes one CTA loads
+  __host__ __device__ static constexpr int stage_bytes(int width) { return a_bytes(width) + boxes(width) * box_bytes(width); }
+  __host__ __device__ static constexpr int stage_tx(int width) { return a_bytes(width) + width / 2 * bk(width) * 2; }   // bytes one CTA loads
   // 192 to 200 KiB of stages whatever the width
-  __host__ __device__ static constexpr int stages(int width) { return boxes(width) == 1 ? 8 : (boxes(width) == 2 ? 6 : 5); }
+  __host__ __device__ static constexpr int stages(int width) { return boxes(width) == 1 ? 4 : (boxes(width) == 2 ? 6 : 5); }
   __host__ __device__ static constexpr int smem_bytes(int width) {
     return stages(width) * stage_bytes(width) + (width / 32) * RI_BLOCK_BYTES + 256 + 1024;
   }
@@ -56,8 +61,9 @@ static_assert(RotWideCfg::smem_bytes(128) <= 232448 && RotWideCfg::smem_bytes(25
 
 // grid = 2 * rows * cols CTAs in clusters of two: pair p works row tile p % rows (256 tokens), column tile p / rows
 // (`width` features from column (p / rows) * width on).  tmX: X box [128 x 64]; tmR: R_inter box [64 x 64]; tmRt:
-// box [64 x tail_cols].  d % 128 == 0.  TWO: width > 256.  FMT, `tensor_scale` as in the pair kernel.
-template <int FMT, bool TWO>
+// box [64 x tail_cols].  d % 128 == 0.  RANGE: 128, 256 or
+// 384, the first that is not below the width (two slabs of K per stage; one; two instructions per slice).  FMT, `tensor_scale` as in the pair kernel.
+template <int FMT, int RANGE>
 __global__ void __launch_bounds__(RotWideCfg::THREADS, 1)
 rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,
                             const __grid_constant__ CUtensorMap tmRt, const __nv_bfloat16* __restrict__ R_intra,
@@ -84,7 +90,9 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   const int pair = blockIdx.x >> 1;
   const int tcol = (pair / rows) * width;
   const int mt = 2 * (pair % rows) + (int)rank;
-  const int k_tiles = d / C::BK;
+  constexpr int BK = C::bk(RANGE), A_BYTES = C::a_bytes(RANGE), BOX_BYTES = C::box_bytes(RANGE);
+  constexpr bool TWO = RANGE > 256;
+  const int k_tiles = d / BK;
   const int n0 = C::n0(width);
 
   // Set-up as in the pair kernels: the producer waits for nothing but the barriers of both CTAs, and the first stages' X loads
@@ -125,15 +133,15 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       const int col0 = tcol + (int)rank * (n0 / 2), col1 = tcol + n0 + (int)rank * 64;
       const uint32_t leader_full0 = map_to_cta(full_bar(0), 0);
       auto load_r = [&](int s, int kt) {
-        uint32_t dst = smem_base + s * stage_bytes + C::A_BYTES;
+        uint32_t dst = smem_base + s * stage_bytes + A_BYTES;
         const uint32_t bar = leader_full0 + 8u * s;
         if (rank == 0) mbar_arrive_expect_tx(full_bar(s), 2 * C::stage_tx(width));
-        for (int b = 0; b < full0; ++b, dst += C::BOX_BYTES) tma_load_2d_pair(dst, &tmR, col0 + 64 * b, kt * C::BK, bar);
+        for (int b = 0; b < full0; ++b, dst += BOX_BYTES) tma_load_2d_pair(dst, &tmR, col0 + 64 * b, kt * BK, bar);
         if (tail) {
-          tma_load_2d_pair(dst, &tmRt, col0 + 64 * full0, kt * C::BK, bar);
-          dst += C::BOX_BYTES;
+          tma_load_2d_pair(dst, &tmRt, col0 + 64 * full0, kt * BK, bar);
+          dst += BOX_BYTES;
         }
-        if constexpr (TWO) tma_load_2d_pair(dst, &tmR, col1, kt * C::BK, bar);
+        if constexpr (TWO) tma_load_2d_pair(dst, &tmR, col1, kt * BK, bar);
       };
       for (int i = 0; i < pre; ++i) load_r(i, i);
       griddep_wait();
@@ -142,7 +150,7 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       for (int kt = pre; kt < k_tiles; ++kt) {
         if (!mbar_wait_cluster(empty_bar(s), ph, cta_abort, err_word, SITE_PRODUCER_EMPTY)) break;
         load_r(s, kt);
-        tma_load_2d_pair(smem_base + s * stage_bytes, &tmX, kt * C::BK, mt * C::BM, leader_full0 + 8u * s);
+        tma_load_3d_pair(smem_base + s * stage_bytes, &tmX, 0, mt * C::BM, kt * (BK / C::SLAB), leader_full0 + 8u * s);
         if (++s == nst) { s = 0; ph ^= 1; }
       }
     }
@@ -161,12 +169,13 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
         tc_fence_after_sync();
         const uint32_t st = smem_base + s * stage_bytes;
         const uint64_t adesc = make_desc(st, 16, 1024, kSwizzle128);
-        const uint64_t bdesc = make_desc(st + C::A_BYTES, C::BOX_BYTES, 1024, kSwizzle128);
+        const uint64_t bdesc = make_desc(st + A_BYTES, BOX_BYTES, 1024, kSwizzle128);
 #pragma unroll
-        for (int j = 0; j < C::BK / 16; ++j) {
-          mma_bf16_pair(tmem_base, adesc + 2 * j, bdesc + 128 * j, idesc0, (kt | j) != 0);
+        for (int j = 0; j < BK / 16; ++j) {
+          const uint64_t aj = adesc + (j >> 2) * (C::BM * C::SLAB * 2 / 16) + 2 * (j & 3);
+          mma_bf16_pair(tmem_base, aj, bdesc + 128 * j, idesc0, (kt | j) != 0);
           if constexpr (TWO)                           // the first instruction's half is two boxes then
-            mma_bf16_pair(tmem_base + n0, adesc + 2 * j, bdesc + 2 * C::BOX_BYTES / 16 + 128 * j, idesc1, (kt | j) != 0);
+            mma_bf16_pair(tmem_base + n0, aj, bdesc + 2 * BOX_BYTES / 16 + 128 * j, idesc1, (kt | j) != 0);
         }
         tc_commit_pair(empty_bar(s), 3);            // stage free in both CTAs
         if (++s == nst) { s = 0; ph ^= 1; }
@@ -186,7 +195,7 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       griddep_wait();
       if (elect_one())
         for (int i = 0; i < pre; ++i)
-          tma_load_2d_pair(smem_base + i * stage_bytes, &tmX, i * C::BK, mt * C::BM, map_to_cta(full_bar(i), 0));
+          tma_load_3d_pair(smem_base + i * stage_bytes, &tmX, 0, mt * C::BM, i * (BK / C::SLAB), map_to_cta(full_bar(i), 0));
       __syncwarp();
     }
     if (R_intra != nullptr) {                          // the tile's blocks, 16-byte piece c of row i at c ^ ((i >> 1) & 3)

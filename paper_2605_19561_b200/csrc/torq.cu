@@ -111,12 +111,12 @@ static DeviceState* device_state() {
               opt_in_smem(rotate_quantize_kernel<256, FMT_NVFP4>, RotCfg<256>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_MXFP4>, RotPairCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_NVFP4>, RotPairCfg::SMEM_BYTES) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, false>, kWideSmem) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, true>, kWideSmem) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, false>, kWideSmem) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, true>, kWideSmem) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, false>, kWideSmem) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, true>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, 128>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, 256>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, 384>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, 128>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, 256>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, 384>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, 128>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, 256>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, 384>, kWideSmem) &&
               opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXFP4, false>, kWideSmem) &&
               opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXFP4, true>, kWideSmem) &&
               opt_in_smem(mxfp4_gemm_wide_kernel<FMT_NVFP4, false>, kWideSmem) &&
@@ -185,6 +185,18 @@ static bool encode_x_blocks_3d(CUtensorMap* map, const void* base, uint64_t M, u
   cuuint32_t estr[3] = {1, 1, 1};
   return g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// X [M, d] bf16 seen as (K within a slab of 64, token, slab) with box (64, 128, slabs): each slab lands as 128 rows of 128 bytes,
+// 128-byte swizzle, one slab behind the other.
+static bool encode_x_slabs_3d(CUtensorMap* map, const void* base, uint64_t M, uint64_t d, uint32_t slabs) {
+  cuuint64_t dims[3] = {64, M, d / 64};
+  cuuint64_t strides[2] = {d * 2, 128};
+  cuuint32_t box[3] = {64, 128, slabs};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -446,29 +458,35 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 // Width of the one-wave rotation's tiles, or 0 where another kernel is faster.  Times in us, fitted to the rotation
 // alone at 60 shapes (d = 128 ... 14336, M = 1 ... 4000; within 10 % but for the HBM-bound ones at d > 8192, where both
 // sides are low by as much); f = filled part of a wave:
-//  * here: 1.6 + 0.022 per column (2 + 0.032 above 256 columns) for launch and epilogue, then per K step the operand
-//    bytes, 0.17 + 0.0003 per column + 0.03 f, or the math, 0.00114 per column;
-//  * few tokens: 3.1 / 4.4 / 5.6 / 7.6 / 10.5 up to 16 / 64 / 128 / 192 / 256 tokens, plus 0.22 / 0.2 / 0.36 / 0.42 / 0.42
-//    per K step of the longest split (192 and 256 tokens measured: d = 2560 10.9 and 13.6, here 11.5; d = 3072 13.1 and 15.4,
-//    here 13.4; d = 8192 33.5 and 37.4, here 35.1 and 35.8);
+//  * here: 1.6 + 0.022 per column (2 + 0.032 above 256 columns, 1.4 + 0.022 up to 128) for launch and epilogue, then per K step
+//    of 64 the operand bytes, 0.17 + 0.0003 per column + 0.03 f (up to 128 columns, where a stage is two of these steps, 0.145 +
+//    0.0003 per column + 0.035 f, but from d = 6272 on, where R_inter's stream sets the pace), or the math, 0.00114 per column;
+//  * few tokens: 3.1 / 4.4 / 5.6 up to 16 / 64 / 128 tokens, plus 0.22 / 0.2 / 0.36 per K step of the longest split; above, 6.4 at
+//    144 tokens and 0.025 per token more, 0.5 per CTA of a cluster above four, 0.42 per K step (us, few tokens / here: 144
+//    tokens d = 2560 9.7 / 10.4, d = 4096 13.6 / 14.9; 208 d = 2560 12.6 / 10.4, d = 4096 15.0 / 15.0 (the layer with N = 6144
+//    22.7 / 23.2), d = 5120 19.5 / 20.1; 256 d = 4096 16.2 / 15.1, d = 5120 20.9 / 20.0; 128 d = 2048 8.1 / 7.6);
 //  * pair kernel: 6.8, plus per K step 0.32 for a wave and 0.2 + 0.14 f for the last, partly filled one.
 // The other formats follow the same figures, which were not fitted to them; wide_gemm_width says how that was checked.
 // A layer of 2048 tokens and more fills the pair kernel's waves and stays there (one-wave tiles would be wider than
 // 384 columns; 2048 x 4096 measured 51.6 with 480 columns, 46.8 in the pair kernel).
-static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int max_pairs) {
-  const int64_t rows = (M + 255) / 256, steps = d / RotWideCfg::BK;
+static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int few_S, int max_pairs) {
+  const int64_t rows = (M + 255) / 256, steps = d / 64;
+  // The line of 65 to 96 tokens, clusters of six, stays where it was, and so does that of an X below 128 KiB, which these tiles read
+  // more slowly (us, few tokens / here: d = 1024 63 tokens 5.7 / 5.8, 64 tokens 5.7 / 4.5; d = 1152 56 5.6 / 5.7, 60 5.7 / 4.7;
+  // d = 1536 40 5.9 / 9.3, 48 6.0 / 5.6).
+  const bool two_slabs = d <= 6144 && (M > 96 || (M <= 64 && M * d >= 65536));
   double best = 1e30;
   int width = 0;
   for (int w = 32; w <= RotWideCfg::MAX_WIDTH; w += 32) {
     if (rows * ((d + w - 1) / w) > max_pairs) continue;
     const double f = (double)(rows * ((d + w - 1) / w)) / max_pairs;
-    const double bytes = 0.17 + 0.0003 * w + 0.03 * f, math = 0.00114 * w;
-    const double t = (w <= 256 ? 1.6 + 0.022 * w : 2.0 + 0.032 * w) + (double)steps * (bytes > math ? bytes : math);
+    const double bytes = (w <= 128 && two_slabs ? 0.145 + 0.035 * f : 0.17 + 0.03 * f) + 0.0003 * w, math = 0.00114 * w;
+    const double t = (w <= 128 && two_slabs ? 1.4 + 0.022 * w : (w <= 256 ? 1.6 + 0.022 * w : 2.0 + 0.032 * w)) + (double)steps * (bytes > math ? bytes : math);
     if (t < best) { best = t; width = w; }
   }
   double other;
   if (M <= kRotFewMaxTokens) {
-    other = M <= 16 ? 3.1 + 0.22 * few_steps : (M <= 64 ? 4.4 + 0.2 * few_steps : (M <= 128 ? 5.6 + 0.36 * few_steps : (M <= 192 ? 7.6 : 10.5) + 0.42 * few_steps));
+    other = M <= 16 ? 3.1 + 0.22 * few_steps : (M <= 64 ? 4.4 + 0.2 * few_steps : (M <= 128 ? 5.6 + 0.36 * few_steps : 6.4 + 0.025 * (double)(M - 144) + (few_S > 4 ? 0.5 * (few_S - 4) : 0.0) + 0.42 * few_steps));
   } else {
     const int64_t tiles = rows * ((d + 255) / 256);
     const int64_t full = tiles / max_pairs, rest = tiles % max_pairs;
@@ -482,18 +500,20 @@ static torq_status rotate_wide(DeviceState* st, int fmt, const void* X, const vo
   using C = RotWideCfg;
   CUtensorMap tmX, tmR, tmRt;
   const int tail = C::tail_cols(width);
-  if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d, 128, 64) ||
-      !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 64) ||
-      !encode_2d(&tmRt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, (uint32_t)(tail ? tail : 64)))
+  const uint32_t bk = (uint32_t)C::bk(width);
+  if (!encode_x_slabs_3d(&tmX, X, (uint64_t)M, (uint64_t)d, bk / C::SLAB) ||
+      !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, bk, 64) ||
+      (tail && !encode_2d(&tmRt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, bk, (uint32_t)tail)))
     return TORQ_ERR_LAUNCH;
+  if (!tail) tmRt = tmR;
   const int rows = (int)((M + 255) / 256), cols = (int)((d + width - 1) / width);
-  auto launch = [&](auto one, auto two) {
-    launch_tc(width > 256 ? two : one, 2, 2 * rows * cols, C::THREADS, C::smem_bytes(width), s, tmX, tmR, tmRt,
+  auto launch = [&](auto r128, auto r256, auto r384) {
+    launch_tc(width > 256 ? r384 : (width > 128 ? r256 : r128), 2, 2 * rows * cols, C::THREADS, C::smem_bytes(width), s, tmX, tmR, tmRt,
               static_cast<const __nv_bfloat16*>(R_intra), codes, scales, (int)M, (int)d, tensor_scale, rows, width, st->err_word);
   };
-  if (fmt == FMT_MXINT4) launch(rotate_quantize_wide_kernel<FMT_MXINT4, false>, rotate_quantize_wide_kernel<FMT_MXINT4, true>);
-  else if (fmt == FMT_NVFP4) launch(rotate_quantize_wide_kernel<FMT_NVFP4, false>, rotate_quantize_wide_kernel<FMT_NVFP4, true>);
-  else launch(rotate_quantize_wide_kernel<FMT_MXFP4, false>, rotate_quantize_wide_kernel<FMT_MXFP4, true>);
+  if (fmt == FMT_MXINT4) launch(rotate_quantize_wide_kernel<FMT_MXINT4, 128>, rotate_quantize_wide_kernel<FMT_MXINT4, 256>, rotate_quantize_wide_kernel<FMT_MXINT4, 384>);
+  else if (fmt == FMT_NVFP4) launch(rotate_quantize_wide_kernel<FMT_NVFP4, 128>, rotate_quantize_wide_kernel<FMT_NVFP4, 256>, rotate_quantize_wide_kernel<FMT_NVFP4, 384>);
+  else launch(rotate_quantize_wide_kernel<FMT_MXFP4, 128>, rotate_quantize_wide_kernel<FMT_MXFP4, 256>, rotate_quantize_wide_kernel<FMT_MXFP4, 384>);
   return launch_status();
 }
 
@@ -558,12 +578,12 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
   }
   CUtensorMap tmX, tmR;
   if (d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT) {
-    int few_steps = 0;                                     // longest K range of the few-token kernel
+    int few_steps = 0, few_S = 0;                          // longest K range and cluster of the few-token kernel
     if (M <= kRotFewMaxTokens) {
-      const int S = fewtok_rotation(M, d, st).cluster;
-      few_steps = (int)((d / 64 + S - 1) / S);
+      few_S = fewtok_rotation(M, d, st).cluster;
+      few_steps = (int)((d / 64 + few_S - 1) / few_S);
     }
-    const int width = wide_rotation_width(M, d, few_steps, st->rot_pairs);
+    const int width = wide_rotation_width(M, d, few_steps, few_S, st->rot_pairs);
     if (width > 0) return rotate_wide(st, fmt, X, R_inter, R_intra, M, d, codes, scales, tensor_scale, width, s);
   }
   if (M <= kRotFewMaxTokens && d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT)
@@ -737,7 +757,7 @@ static torq_status gemm_wide(DeviceState* st, const void* Aq, const void* As, co
   CUtensorMap tmA, tmB, tmB1, tmSFA, tmSFB, tmY;
   if (!encode_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Aq, (uint64_t)M, krow, 128, 128) ||
       !encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, (uint32_t)C::n0(width) / 2, 128) ||
-      !encode_2d(&tmB1, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, 64, 128) ||
+      (width > 256 && !encode_2d(&tmB1, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, 64, 128)) ||
       !encode_2d(&tmSFA, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, As, (uint64_t)((M + 127) / 128), sf_words, 1, C::SF_BOX_WORDS,
                  CU_TENSOR_MAP_SWIZZLE_NONE) ||
       !encode_2d(&tmSFB, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, Ws, (uint64_t)((N + 127) / 128), sf_words, (uint32_t)C::chunks(width),
@@ -745,6 +765,7 @@ static torq_status gemm_wide(DeviceState* st, const void* Aq, const void* As, co
       !encode_2d(&tmY, ybf ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, ybf ? 2 : 4, Y, (uint64_t)M,
                  (uint64_t)N, 32, ybf ? 64 : 32))
     return TORQ_ERR_LAUNCH;
+  if (width <= 256) tmB1 = tmB;
   const int rows = (int)((M + 255) / 256), cols = (int)((N + width - 1) / width);
   launch_tc(width > 256 ? mxfp4_gemm_wide_kernel<FMT, true> : mxfp4_gemm_wide_kernel<FMT, false>, 2, 2 * rows * cols, C::THREADS,
             C::smem_bytes(width), s, tmA, tmB, tmB1, tmSFA, tmSFB, tmY, ybf ? 1 : 0, (int)M, (int)N, (int)K, rows, width, alpha,

@@ -161,3 +161,21 @@ def test_gemm_kernel_of_more_than_the_few_tokens(M, N, K, kernel):
     (name, _), = captured_launches(call)
     assert f"mxfp4_gemm_{kernel}_kernel" in name and not bool(y.any())
     assert torq.torq_last_device_error() == 0
+
+
+@pytest.mark.parametrize("M,d", [(40, 384), (128, 896), (130, 128), (300, 640), (300, 1664), (256, 4096)])
+def test_rotation_with_two_slabs_per_stage(M, d):
+    """Tiles of up to 128 columns, where a stage is 128 of K: one stage, odd numbers of them, more than the ring holds, both
+    widths of the last box.  Permutations of small integers: bit for bit the oracle's."""
+    g = np.random.default_rng(M + d)
+    xb = I.to_bf16_bits(g.integers(-8, 9, size=(M, d)).astype(np.float64))
+    P = np.zeros((d, d))
+    P[np.arange(d), g.permutation(d)] = 1.0
+    pin = I.to_bf16_bits(np.stack([np.eye(32)[g.permutation(32)] for _ in range(d // 32)]))
+    rows = np.unique(np.r_[0:min(M, 40), max(0, M - 40):M])
+    codes_t, scales_t = torq.torq_rotate_quantize(dev_bf16(xb), dev_bf16(I.to_bf16_bits(P)), dev_bf16(pin))
+    torch.cuda.synchronize()
+    assert torq.torq_last_device_error() == 0
+    g_codes, g_sb = gpu_quantized_to_numpy(codes_t, scales_t, M, d)
+    o_codes, o_sb = O.quantize_mxfp4(O.round_to_f32(O.rotate(xb[rows], I.to_bf16_bits(P), pin)))
+    assert np.array_equal(g_sb[rows], o_sb) and np.array_equal(g_codes[rows], o_codes)
