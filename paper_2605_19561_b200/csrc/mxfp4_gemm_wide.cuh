@@ -39,30 +39,39 @@ struct GemmWideCfg {
   // chunks of W scales a tile can touch: tiles start on multiples of `width`, i.e. 0 or 64 rows into a chunk
   __host__ __device__ static constexpr int chunks(int width) { return (width + (width % 128 ? 64 : 0) + 127) / 128; }
   __host__ __device__ static constexpr int stage_tx(int width) { return A_BYTES + width / 2 * 128 + SF_BOXES * SF_BOX_BYTES * (1 + chunks(width)); }
-  __host__ __device__ static constexpr int stage_bytes(int width) { return (stage_tx(width) + 1023) / 1024 * 1024; }
-  __host__ __device__ static constexpr int stages(int width) {
-    return (232448 - 2048) / stage_bytes(width) < MAX_STAGES ? (232448 - 2048) / stage_bytes(width) : MAX_STAGES;
+  __host__ __device__ static constexpr int slab_bytes(int width) { return (stage_tx(width) + 1023) / 1024 * 1024; }
+  // K slabs of 128 bytes per stage of the kernel for widths up to `range`
+  __host__ __device__ static constexpr int slabs(int range) { return range <= 128 ? 2 : 1; }
+  // Two slabs halve the waits and barriers per K, which bound a step of up to 128 columns (us, one slab / two: 200 x 4096, K = 14336
+  // 15.9 / 13.2, 300 x 4096, K = 4096 7.3 / 6.7, NVFP4 400 x 4096 8.4 / 7.7, 150 x 5120, K = 5120 7.8 / 6.9, 200 x 6144, K = 4096
+  // 7.53 / 7.26; 512 x 4096, K = 14336 17.7 / 17.8).  With a few slabs in all the first stage is waited for longer (40 x 4096,
+  // K = 512 2.90 / 3.02): from four on.
+  __host__ __device__ static constexpr int range(int width, int64_t k_slabs) { return width > 256 ? 384 : (width > 128 || k_slabs < 4 ? 256 : 128); }
+  __host__ __device__ static constexpr int stage_bytes(int width, int range) { return slabs(range) * slab_bytes(width); }
+  __host__ __device__ static constexpr int stages(int width, int range) {
+    return (232448 - 2048) / stage_bytes(width, range) < MAX_STAGES ? (232448 - 2048) / stage_bytes(width, range) : MAX_STAGES;
   }
-  __host__ __device__ static constexpr int smem_bytes(int width) { return stages(width) * stage_bytes(width) + 256 + 1024; }
+  __host__ __device__ static constexpr int smem_bytes(int width, int range) { return stages(width, range) * stage_bytes(width, range) + 256 + 1024; }
   static_assert(SF_COL + 4 * CH + 4 * CH * 3 <= 512 && chunks(MAX_WIDTH) <= 3 && chunks(MAX_WIDTH - 64) <= 3, "up to three chunks of W scales");
 };
 
 // grid = 2 * rows * cols CTAs in clusters of two: pair p works row tile p % rows (256 tokens), column tile p / rows.
 // tmA: [128 x 128 B]; tmB: [n0 / 2 x 128 B]; tmB1: [64 x 128 B] (second instruction); tmSFA / tmSFB: boxes of 1 / nchk
-// rows of the scale view; tmY as in the pair kernel.  TWO: width > 256.
-template <int FMT, bool TWO>
+// rows of the scale view; tmY as in the pair kernel.  RANGE: of the width and K (GemmWideCfg).
+template <int FMT, int RANGE>
 __global__ void __launch_bounds__(GemmWideCfg<FMT>::THREADS, 1)
 mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                        const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmSFA,
                        const __grid_constant__ CUtensorMap tmSFB, const __grid_constant__ CUtensorMap tmY, int y_is_bf16,
                        int M, int N, int K, int rows, int width, float alpha, int* err_word) {
   using C = GemmWideCfg<FMT>;
-  constexpr int CH = C::CH;
+  constexpr int CH = C::CH, SL = C::slabs(RANGE);
+  constexpr bool TWO = RANGE > 256;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-  const int nst = C::stages(width);
-  const uint32_t stage_bytes = C::stage_bytes(width);
+  const int nst = C::stages(width, RANGE);
+  const uint32_t stage_bytes = C::stage_bytes(width, RANGE);
   const uint32_t bar_off = nst * stage_bytes;
   const uint32_t bar_base = smem_base + bar_off;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
@@ -76,7 +85,8 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
   const int pair = blockIdx.x >> 1;
   const int tcol = (pair / rows) * width;
   const int mt = 2 * (pair % rows) + (int)rank;
-  const int k_tiles = (K + C::BK - 1) / C::BK;
+  const int k_slabs = (K + C::BK - 1) / C::BK, k_tiles = (k_slabs + SL - 1) / SL;   // slabs of K, stages of them (the last may hold one)
+  const uint32_t slab_bytes = C::slab_bytes(width);
   const int n0 = C::n0(width), nchk = C::chunks(width);
   const uint32_t b_bytes = (uint32_t)width / 2 * 128;
   const uint32_t sfa_off = C::A_BYTES + b_bytes, sfb_off = sfa_off + C::SF_BOXES * C::SF_BOX_BYTES;
@@ -104,12 +114,15 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
   const int pre = k_tiles < nst ? k_tiles : nst;
 
   auto load_a = [&](int s, int kt) {
-    const uint32_t st = smem_base + s * stage_bytes, bar = map_to_cta(full_bar(s), 0);
-    tma_load_2d_pair(st, &tmA, kt * 128, mt * C::BM, bar);
-    // anything outside the buffer arrives as zeros (scale 2^-127 or 0, on operand data that is zero as well)
+    const uint32_t bar = map_to_cta(full_bar(s), 0);
+    for (int k = kt * SL; k < (kt + 1) * SL && k < k_slabs; ++k) {
+      const uint32_t st = smem_base + s * stage_bytes + (k - kt * SL) * slab_bytes;
+      tma_load_2d_pair(st, &tmA, k * 128, mt * C::BM, bar);
+      // anything outside the buffer arrives as zeros (scale 2^-127 or 0, on operand data that is zero as well)
 #pragma unroll
-    for (int b = 0; b < C::SF_BOXES; ++b)
-      tma_load_2d_pair(st + sfa_off + b * C::SF_BOX_BYTES, &tmSFA, kt * CH * 128 + b * C::SF_BOX_WORDS, mt, bar);
+      for (int b = 0; b < C::SF_BOXES; ++b)
+        tma_load_2d_pair(st + sfa_off + b * C::SF_BOX_BYTES, &tmSFA, k * CH * 128 + b * C::SF_BOX_WORDS, mt, bar);
+    }
   };
 
   if (warp == 0) {
@@ -117,13 +130,18 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     if (elect_one()) {
       const uint32_t leader_full0 = map_to_cta(full_bar(0), 0);
       auto load_w = [&](int s, int kt) {
-        const uint32_t st = smem_base + s * stage_bytes, bar = leader_full0 + 8u * s;
-        if (rank == 0) mbar_arrive_expect_tx(full_bar(s), 2 * C::stage_tx(width));
-        tma_load_2d_pair(st + C::A_BYTES, &tmB, kt * 128, tcol + (int)rank * (n0 / 2), bar);
-        if constexpr (TWO) tma_load_2d_pair(st + C::A_BYTES + n0 / 2 * 128, &tmB1, kt * 128, tcol + n0 + (int)rank * 64, bar);
+        const uint32_t bar = leader_full0 + 8u * s;
+        const int here = k_slabs - kt * SL < SL ? k_slabs - kt * SL : SL;
+        if (rank == 0) mbar_arrive_expect_tx(full_bar(s), 2 * here * C::stage_tx(width));
+        for (int i = 0; i < here; ++i) {
+          const int k = kt * SL + i;
+          const uint32_t st = smem_base + s * stage_bytes + i * slab_bytes;
+          tma_load_2d_pair(st + C::A_BYTES, &tmB, k * 128, tcol + (int)rank * (n0 / 2), bar);
+          if constexpr (TWO) tma_load_2d_pair(st + C::A_BYTES + n0 / 2 * 128, &tmB1, k * 128, tcol + n0 + (int)rank * 64, bar);
 #pragma unroll
-        for (int b = 0; b < C::SF_BOXES; ++b)
-          tma_load_2d_pair(st + sfb_off + b * nchk * C::SF_BOX_BYTES, &tmSFB, kt * CH * 128 + b * C::SF_BOX_WORDS, tcol >> 7, bar);
+          for (int b = 0; b < C::SF_BOXES; ++b)
+            tma_load_2d_pair(st + sfb_off + b * nchk * C::SF_BOX_BYTES, &tmSFB, k * CH * 128 + b * C::SF_BOX_WORDS, tcol >> 7, bar);
+        }
       };
       for (int i = 0; i < pre; ++i) load_w(i, i);
       griddep_wait();
@@ -159,43 +177,48 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         ok = mbar_wait_cluster_warp(full_bar(s), ph, cta_abort, err_word, SITE_MMA_FULL);
         if (!ok) break;
         tc_fence_after_sync();
-        const bool two = FMT == FMT_MXINT4 || K - kt * C::BK > C::BK / 2;      // K % 256 == 128: the last stage is half
-        const uint32_t st = smem_base + s * stage_bytes;
-        const uint64_t adesc = make_desc(st, 16, 1024, kSwizzle128);
-        const uint64_t bdesc = make_desc(st + C::A_BYTES, 16, 1024, kSwizzle128);
-        const uint64_t b1desc = make_desc(st + C::A_BYTES + n0 / 2 * 128, 16, 1024, kSwizzle128);
-        const uint64_t sfa_d = make_desc(st + sfa_off, 0, 128, 0);
-        const uint64_t sfb_d = make_desc(st + sfb_off, 0, 128, 0);
         if (elect_one()) {
-          // scale chunks shared -> tensor memory (descriptor address unit = 16 B)
 #pragma unroll
-          for (int c = 0; c < CH; ++c) {
-            if (CH == 1 || c < CH / 2 || two) {
-              tmem_cp_32x128b_warpx4_pair(sfa_t + 4 * c, sfa_d + 32 * c);
+          for (int i = 0; i < SL; ++i) {
+            const int k = kt * SL + i;
+            if (SL > 1 && k >= k_slabs) break;
+            const bool two = FMT == FMT_MXINT4 || K - k * C::BK > C::BK / 2;       // K % 256 == 128: the last slab is half
+            const uint32_t st = smem_base + s * stage_bytes + i * slab_bytes;
+            const uint64_t adesc = make_desc(st, 16, 1024, kSwizzle128);
+            const uint64_t bdesc = make_desc(st + C::A_BYTES, 16, 1024, kSwizzle128);
+            const uint64_t b1desc = make_desc(st + C::A_BYTES + n0 / 2 * 128, 16, 1024, kSwizzle128);
+            const uint64_t sfa_d = make_desc(st + sfa_off, 0, 128, 0);
+            const uint64_t sfb_d = make_desc(st + sfb_off, 0, 128, 0);
+            // scale chunks shared -> tensor memory (descriptor address unit = 16 B)
 #pragma unroll
-              for (int t = 0; t < 3; ++t)
-                if (t < nchk)
-                  tmem_cp_32x128b_warpx4_pair(sfb_t + c * sfb_c + 4 * t,
-                                              sfb_d + ((c >> 1) * nchk + t) * (C::SF_BOX_BYTES / 16) + 32 * (c & 1));
+            for (int c = 0; c < CH; ++c) {
+              if (CH == 1 || c < CH / 2 || two) {
+                tmem_cp_32x128b_warpx4_pair(sfa_t + 4 * c, sfa_d + 32 * c);
+#pragma unroll
+                for (int t = 0; t < 3; ++t)
+                  if (t < nchk)
+                    tmem_cp_32x128b_warpx4_pair(sfb_t + c * sfb_c + 4 * t,
+                                                sfb_d + ((c >> 1) * nchk + t) * (C::SF_BOX_BYTES / 16) + 32 * (c & 1));
+              }
             }
-          }
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if (j < 2 || two) {
-              const uint32_t accumulate = (kt | j) != 0;
-              if constexpr (FMT == FMT_MXINT4) {         // a quarter chunk (one scale byte) per instruction
-                mma_mxf8_pair(tmem_base, adesc + 2 * j, bdesc + 2 * j, idesc_mxf8(256, 256, j) - less, sfa_t, sfb_m, accumulate);
-                if constexpr (TWO)
-                  mma_mxf8_pair(acc1, adesc + 2 * j, b1desc + 2 * j, idesc_mxf8(256, 256, j) - less1, sfa_t, sfb_m1, accumulate);
-              } else if constexpr (FMT == FMT_NVFP4) {   // one chunk per instruction
-                mma_nvf4_pair(tmem_base, adesc + 2 * j, bdesc + 2 * j, full_a - less, sfa_t + 4 * j, sfb_m + j * sfb_c, accumulate);
-                if constexpr (TWO)
-                  mma_nvf4_pair(acc1, adesc + 2 * j, b1desc + 2 * j, full_a - less1, sfa_t + 4 * j, sfb_m1 + j * sfb_c, accumulate);
-              } else {                                   // half a chunk (two scale bytes) per instruction
-                const uint32_t id = (j & 1) ? full_b : full_a;
-                mma_mxf4_pair(tmem_base, adesc + 2 * j, bdesc + 2 * j, id - less, sfa_t + 4 * (j >> 1), sfb_m + (j >> 1) * sfb_c, accumulate);
-                if constexpr (TWO)
-                  mma_mxf4_pair(acc1, adesc + 2 * j, b1desc + 2 * j, id - less1, sfa_t + 4 * (j >> 1), sfb_m1 + (j >> 1) * sfb_c, accumulate);
+            for (int j = 0; j < 4; ++j) {
+              if (j < 2 || two) {
+                const uint32_t accumulate = (k | j) != 0;
+                if constexpr (FMT == FMT_MXINT4) {         // a quarter chunk (one scale byte) per instruction
+                  mma_mxf8_pair(tmem_base, adesc + 2 * j, bdesc + 2 * j, idesc_mxf8(256, 256, j) - less, sfa_t, sfb_m, accumulate);
+                  if constexpr (TWO)
+                    mma_mxf8_pair(acc1, adesc + 2 * j, b1desc + 2 * j, idesc_mxf8(256, 256, j) - less1, sfa_t, sfb_m1, accumulate);
+                } else if constexpr (FMT == FMT_NVFP4) {   // one chunk per instruction
+                  mma_nvf4_pair(tmem_base, adesc + 2 * j, bdesc + 2 * j, full_a - less, sfa_t + 4 * j, sfb_m + j * sfb_c, accumulate);
+                  if constexpr (TWO)
+                    mma_nvf4_pair(acc1, adesc + 2 * j, b1desc + 2 * j, full_a - less1, sfa_t + 4 * j, sfb_m1 + j * sfb_c, accumulate);
+                } else {                                   // half a chunk (two scale bytes) per instruction
+                  const uint32_t id = (j & 1) ? full_b : full_a;
+                  mma_mxf4_pair(tmem_base, adesc + 2 * j, bdesc + 2 * j, id - less, sfa_t + 4 * (j >> 1), sfb_m + (j >> 1) * sfb_c, accumulate);
+                  if constexpr (TWO)
+                    mma_mxf4_pair(acc1, adesc + 2 * j, b1desc + 2 * j, id - less1, sfa_t + 4 * (j >> 1), sfb_m1 + (j >> 1) * sfb_c, accumulate);
+                }
               }
             }
           }

@@ -179,3 +179,26 @@ def test_rotation_with_two_slabs_per_stage(M, d):
     g_codes, g_sb = gpu_quantized_to_numpy(codes_t, scales_t, M, d)
     o_codes, o_sb = O.quantize_mxfp4(O.round_to_f32(O.rotate(xb[rows], I.to_bf16_bits(P), pin)))
     assert np.array_equal(g_sb[rows], o_sb) and np.array_equal(g_codes[rows], o_codes)
+
+
+# one to four CTA pairs per row tile, widths 64 and 128: as many slabs of K as fill one ring, an odd number, a half last one, several rounds
+@pytest.mark.parametrize("M,N,K", [(200, 72, 1024), (300, 520, 1152), (129, 2056, 1280), (513, 1000, 2944), (200, 6144, 5376)])
+def test_gemm_with_two_slabs_per_stage(M, N, K):
+    """Scales of one and small integers as codes, so that every sum is exact: the three formats equal the product bit for bit."""
+    g = np.random.default_rng(M + N + K)
+    rows = np.unique(np.r_[0:min(M, 24), max(0, M - 24):M])
+    grid = np.array([0, .5, 1, 1.5, 2, 3, 4, 6, 0, -.5, -1, -1.5, -2, -3, -4, -6])
+    ac, wc = g.integers(0, 16, (M, K), dtype=np.uint8), g.integers(0, 16, (N, K), dtype=np.uint8)
+    ref = (grid[ac[rows]] @ grid[wc].T)
+    one = lambda n, k: dev_u8(O.swizzle_scales(np.full((n, k // 32), 127, np.uint8), k, fill=0))
+    one16 = lambda n, k: dev_u8(O.nv_swizzle_scales(np.full((n, k // 16), 0x38, np.uint8), k))     # E4M3 1.0
+    a, w = dev_u8(O.pack_codes(ac)), dev_u8(O.pack_codes(wc))
+    y = torq.torq_mxfp4_gemm(a, one(M, K), w, one(N, K), out_dtype=torch.float32)
+    assert np.array_equal(y.cpu().numpy()[rows], ref)
+    y = torq.torq_nvfp4_gemm(a, one16(M, K), 1.0, w, one16(N, K), 1.0, out_dtype=torch.float32)
+    assert np.array_equal(y.cpu().numpy()[rows], ref)
+    ai, wi = g.integers(-7, 8, (M, K)).astype(np.int8), g.integers(-7, 8, (N, K)).astype(np.int8)
+    y = torq.torq_mxint4_gemm(dev_u8(O.int4_to_e4m3(ai)), one(M, K), dev_u8(O.int4_to_e4m3(wi)), one(N, K), out_dtype=torch.float32)
+    torch.cuda.synchronize()
+    assert torq.torq_last_device_error() == 0
+    assert np.array_equal(y.cpu().numpy()[rows], ai[rows].astype(np.int64) @ wi.astype(np.int64).T)
