@@ -3,7 +3,8 @@
 // tile through tcgen05.mma cta_group::2.  Each CTA stages only its own 128 rows of X and its own
 // 128 columns of R_inter per K step (32 KiB instead of 48 KiB per 128 x 256 x 64 of work), which
 // is what the single-CTA kernel is short of: it cannot keep enough bytes in flight from L2 to
-// feed the tensor pipe.  Every CTA loads only for itself; operand sharing happens inside the MMA, which
+// feed the tensor pipe.  A 256 x 256 tile's loop of loads and instructions by itself runs at 512 cycles per K step, the
+// instructions' own rate (the loads alone at 22 TB/s, 400 cycles): what a long call waits for is the power cap.  Every CTA loads only for itself; operand sharing happens inside the MMA, which
 // reads both CTAs' shared memory.
 //
 // Tiles are dealt round robin from the list MixedTiles describes: 256 x 256 tiles, and where those
