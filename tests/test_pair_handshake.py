@@ -1,6 +1,9 @@
-"""Host-side rules of the CTA-pair kernels, compiled with the host compiler."""
+"""Rules of the kernels that need no device: host-side ones, compiled with the host compiler, and what their sources must say."""
 import os
+import re
 import subprocess
+
+import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_19561_b200", "csrc")
 
@@ -51,3 +54,20 @@ def test_paced_wait_ends_whatever_the_clock_does(tmp_path):
     if (turns != c.turns) { std::printf("since %u cycles %u: %d turns\\n", c.since, c.cycles, turns); return 1; }
   }
 """)
+
+
+@pytest.mark.parametrize("name", sorted(f for f in os.listdir(CSRC) if f.endswith(".cuh")
+                                        and re.search(r"^  griddep_launch_dependents\(\);", open(os.path.join(CSRC, f)).read(), re.M)))
+def test_no_limit_of_a_wait_counts_the_kernel_before(name):
+    """A kernel starts while the one before it in the stream still runs, for as long as that takes.  So every role passes
+    griddepcontrol.wait, which has no limit, before its first wait that has one."""
+    body = re.sub(r"//.*", "", open(os.path.join(CSRC, name)).read())
+    body = body[re.search(r"^  griddep_launch_dependents\(\);", body, re.M).start():]
+    roles = re.split(r"^  (?:if \(warp == \d+\) \{|\} else if \(warp == \d+\) \{|\} else \{)$", body, flags=re.M)
+    before, roles = roles[0], roles[1:]
+    assert len(roles) >= 3 and sum("mbar_wait" in r for r in roles) >= 3
+    if "griddep_wait();" in before:
+        return
+    for role in roles:
+        wait = re.search(r"mbar_wait\w*\(", role)
+        assert wait is None or "griddep_wait();" in role[:wait.start()], role[:400]
