@@ -842,11 +842,7 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
   if (!encode_2d(&tmBn, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, kNarrowCols / 2, 128))
     return TORQ_ERR_LAUNCH;
   const int max_pairs = st->gemm_pairs;
-  MixedTiles list = plan_pair_tiles((int)((M + 255) / 256), N, max_pairs, kNarrowTileCost);
-  // Every group of row tiles reads all of W: where that does not stay in the L2 beside Y's stream, in groups of sixteen (us, eight /
-  // sixteen: 8192 x 51200, K = 5120 838 / 816 (thirty-two 818), 4096 x 14336, K = 4096 101.3 / 99.9, MXINT4 185.5 / 182.1; below the
-  // line 16384 x 5120, K = 5120 169.6 / 171.9).
-  if ((uint64_t)N * krow >= (16u << 20)) list.group = 16;
+  const MixedTiles list = plan_pair_tiles((int)((M + 255) / 256), N, max_pairs, kNarrowTileCost);
   const int pairs = list.total < max_pairs ? list.total : max_pairs;
   launch_tc(mxfp4_gemm_pair_kernel<FMT>, 2, 2 * pairs, GemmPairCfgT<FMT>::THREADS, GemmPairCfgT<FMT>::SMEM_BYTES, s,
             tmA, tmB, tmSFA, tmSFB, tmY, tmBn, list, ybf ? 1 : 0, (int)M, (int)N, (int)K, alpha, st->err_word);

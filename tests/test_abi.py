@@ -163,3 +163,11 @@ def test_pair_tile_list_covers_every_output_exactly_once():
     tl = torq.torq_pair_tile_list(2048, 4096, 74)
     assert [w for _, _, w in tl].count(256) == 74 and [w for _, _, w in tl].count(192) == 72
     assert torq.lib().torq_pair_tile_list(0, 4096, 74, None, 0) == -1
+
+
+def test_the_gemm_walks_the_pair_tile_list_as_it_is():
+    """torq_pair_tile_list answers from rows and columns alone, so nothing else may go into the list that a launch is given."""
+    src = open(os.path.join(ROOT, "paper_2605_19561_b200", "csrc", "torq.cu")).read()
+    gemm = src[src.index("static torq_status gemm_impl("):src.index("torq_status torq_mxfp4_gemm(")]
+    assert gemm.count("MixedTiles list = plan_pair_tiles((int)((M + 255) / 256), N, max_pairs, kNarrowTileCost);") == 1
+    assert not re.search(r"\blist\.\w+\s*=[^=]", gemm)
