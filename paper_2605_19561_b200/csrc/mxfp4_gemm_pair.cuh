@@ -189,7 +189,7 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       // tensor memory may not be had, before that kernel has completed.
       griddep_wait();
       uint32_t it = 0, tcount = 0;
-      bool ok = mbar_wait_cluster_warp(alloc_bar, 0, cta_abort, err_word, SITE_MMA_ACC_EMPTY);
+      bool ok = mbar_wait_cluster_warp(alloc_bar, 0, cta_abort, err_word, SITE_PEER_TMEM);
       // instruction descriptors differ between the two tile widths only in the N field ([17,23) = N >> 3)
       constexpr uint32_t n_less = (uint32_t)((BN - kNarrowCols) >> 3) << 17;
       const uint32_t sfa_t = tmem_base + C::SFA_COL, sfb_t = tmem_base + C::SFB_COL;

@@ -12,7 +12,7 @@ namespace torq {
 // Low byte: status (6 = a bounded wait ran out); bits 8..15: id of the wait site.
 enum WaitSite : int {
   SITE_PRODUCER_EMPTY = 1, SITE_MMA_FULL = 2, SITE_MMA_ACC_EMPTY = 3, SITE_EPI_ACC_FULL = 4,
-  SITE_TEARDOWN = 5, SITE_SELFTEST = 7
+  SITE_TEARDOWN = 5, SITE_PEER_TMEM = 6, SITE_SELFTEST = 7
 };
 constexpr int kErrTimeout = 6;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s per wait

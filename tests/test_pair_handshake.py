@@ -71,3 +71,19 @@ def test_no_limit_of_a_wait_counts_the_kernel_before(name):
     for role in roles:
         wait = re.search(r"mbar_wait\w*\(", role)
         assert wait is None or "griddep_wait();" in role[:wait.start()], role[:400]
+
+
+def test_a_wait_reports_what_it_waits_for():
+    """The site that a wait names when it gives up is that of its barrier: one site per kind of barrier, none shared."""
+    kinds = {"full_bar": "SITE_MMA_FULL", "empty_bar": "SITE_PRODUCER_EMPTY", "acce_bar": "SITE_MMA_ACC_EMPTY", "accf_bar": "SITE_EPI_ACC_FULL",
+             "alloc_bar": "SITE_PEER_TMEM"}
+    sites = re.search(r"enum WaitSite : int \{(.*?)\};", open(os.path.join(CSRC, "sm100_ptx.cuh")).read(), re.S).group(1)
+    ids = re.findall(r"(SITE_\w+) = (\d+)", sites)
+    assert len({i for _, i in ids}) == len(ids) and set(kinds.values()) <= {n for n, _ in ids}
+    seen = set()
+    for f in os.listdir(CSRC):
+        for bar, site in re.findall(r"mbar_wait\w*\((\w+_bar)\b[^;{]*?(SITE_\w+)\)", open(os.path.join(CSRC, f)).read()):
+            if bar in kinds:
+                assert site == kinds[bar], (f, bar, site)
+                seen.add(bar)
+    assert seen == set(kinds)
