@@ -202,3 +202,23 @@ def test_gemm_with_two_slabs_per_stage(M, N, K):
     torch.cuda.synchronize()
     assert torq.torq_last_device_error() == 0
     assert np.array_equal(y.cpu().numpy()[rows], ai[rows].astype(np.int64) @ wi.astype(np.int64).T)
+
+
+@pytest.mark.parametrize("fmt,M,d,kernel", [("mxfp4", 104, 2048, "wide"), ("mxfp4", 104, 2176, "fewtok"), ("mxfp4", 144, 2176, "wide"),
+                                            ("mxfp4", 160, 2304, "wide"), ("mxfp4", 136, 2432, "fewtok"), ("mxfp4", 192, 2432, "wide"),
+                                            ("mxfp4", 160, 2560, "fewtok"), ("mxfp4", 168, 2816, "fewtok"), ("mxfp4", 208, 2816, "wide"),
+                                            ("nvfp4", 152, 2560, "fewtok"), ("mxint4", 176, 2432, "fewtok"), ("mxint4", 144, 2176, "wide"),
+                                            ("mxint4", 192, 2688, "fewtok"), ("mxint4", 192, 3072, "wide"), ("mxfp4", 192, 4864, "fewtok"), ("nvfp4", 184, 2816, "fewtok"),
+                                            ("mxfp4", 216, 4864, "wide"), ("mxfp4", 144, 6912, "wide"), ("nvfp4", 193, 7296, "wide"),
+                                            ("mxfp4", 150, 7168, "fewtok"), ("mxint4", 256, 9344, "wide")])
+def test_rotation_kernel_of_97_to_256_tokens(fmt, M, d, kernel):
+    """The faster of the two kernels on either side of the line, by measurements of both."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the line is one of 148 SMs")
+    X, R = torch.zeros(M, d, dtype=torch.bfloat16, device="cuda"), torch.zeros(d, d, dtype=torch.bfloat16, device="cuda")
+    call = {"mxfp4": lambda: torq.torq_rotate_quantize(X, R, None), "nvfp4": lambda: torq.torq_rotate_quantize_nvfp4(X, R, None, 1.0),
+            "mxint4": lambda: torq.torq_rotate_quantize_mxint4(X, R, None)}[fmt]
+    call()
+    (name, _), = captured_launches(call)
+    assert {"wide": "rotate_quantize_wide_kernel", "fewtok": "rotate_fewtok_kernel"}[kernel] in name
+    assert torq.torq_last_device_error() == 0
