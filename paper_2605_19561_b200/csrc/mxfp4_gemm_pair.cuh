@@ -185,9 +185,6 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader only)
     if (rank == 0) {
-      // The limits of this warp's waits do not count what is left of the kernel before: no stage is full, and the other CTA's
-      // tensor memory may not be had, before that kernel has completed.
-      griddep_wait();
       uint32_t it = 0, tcount = 0;
       bool ok = mbar_wait_cluster_warp(alloc_bar, 0, cta_abort, err_word, SITE_PEER_TMEM);
       // instruction descriptors differ between the two tile widths only in the N field ([17,23) = N >> 3)

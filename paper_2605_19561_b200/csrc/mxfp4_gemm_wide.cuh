@@ -173,7 +173,6 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       int s = 0;
       uint32_t ph = 0;
       bool ok = true;
-      griddep_wait();                                  // the limits of this warp's waits do not count what is left of that kernel
       for (int kt = 0; kt < k_tiles; ++kt) {
         ok = mbar_wait_cluster_warp(full_bar(s), ph, cta_abort, err_word, SITE_MMA_FULL);
         if (!ok) break;

@@ -163,7 +163,6 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader only)
     if (rank == 0) {
-      griddep_wait();                                  // the limits of this warp's waits do not count what is left of that kernel
       constexpr uint32_t idesc_wide = idesc_bf16(256, BN, /*A MN-major*/ false, /*B MN-major*/ true);
       constexpr uint32_t idesc_narrow = idesc_bf16(256, kNarrowCols, false, true);
       uint32_t it = 0, tcount = 0;

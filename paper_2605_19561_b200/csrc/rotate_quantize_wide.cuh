@@ -157,7 +157,6 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader only)
-    if (rank == 0) griddep_wait();                     // the limits of this warp's waits do not count what is left of that kernel
     if (rank == 0 && mbar_wait_cluster_warp(alloc_bar, 0, cta_abort, err_word, SITE_PEER_TMEM) && elect_one()) {
       const uint32_t idesc0 = idesc_bf16(256, n0, /*A MN-major*/ false, /*B MN-major*/ true);
       constexpr uint32_t idesc1 = idesc_bf16(256, 128, false, true);

@@ -26,6 +26,19 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
   return t;
 }
 
+// ---- programmatic dependent launch ----------------------------------------------------------------
+// A kernel launched with the programmatic-stream-serialization attribute may start while the
+// kernel before it in the stream is still running; griddep_wait() blocks until that kernel has
+// completed and its writes are visible, so everything that touches global memory comes after it.
+// griddep_launch_dependents() tells the runtime that the NEXT kernel in the stream may begin its
+// own launch processing now (it still waits in its griddep_wait for this kernel to finish).
+__device__ __forceinline__ void griddep_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void griddep_launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---- mbarrier --------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
@@ -53,7 +66,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 }
 // Bounded wait.  Returns false when the CTA has been told to give up (another wait timed out) or
 // when this wait itself exceeds kWaitLimitNs; in the latter case it latches the error word and
-// raises the CTA's abort flag so that every other role leaves its loop too.
+// raises the CTA's abort flag so that every other role leaves its loop too.  The limit does not count what is left of the kernel
+// before, which may take any time: the clock starts behind griddep_wait().  (There and not ahead of the wait, where it would cost
+// every call: an issuer that passed it before its first wait made the one-wave rotations 0.5 % slower, 0.025 us in the mean of 58 shapes.)
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* cta_abort,
                                           int* err_word, int site,
                                           unsigned long long limit_ns = kWaitLimitNs) {
@@ -63,6 +78,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if (mbar_try_wait(bar, parity)) return true;
     if ((it & 0x3FFu) == 0) {
       if (*cta_abort) return false;
+      if (t0 == 0) griddep_wait();
       unsigned long long now = globaltimer_ns();
       if (t0 == 0) t0 = now;
       else if (now - t0 > limit_ns) {
@@ -72,19 +88,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
       }
     }
   }
-}
-
-// ---- programmatic dependent launch ----------------------------------------------------------------
-// A kernel launched with the programmatic-stream-serialization attribute may start while the
-// kernel before it in the stream is still running; griddep_wait() blocks until that kernel has
-// completed and its writes are visible, so everything that touches global memory comes after it.
-// griddep_launch_dependents() tells the runtime that the NEXT kernel in the stream may begin its
-// own launch processing now (it still waits in its griddep_wait for this kernel to finish).
-__device__ __forceinline__ void griddep_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-__device__ __forceinline__ void griddep_launch_dependents() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // ---- single-lane election -----------------------------------------------------------------------
@@ -396,6 +399,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     if (mbar_try_wait_cluster(bar, parity)) return true;
     if ((it & 0x3FFu) == 0) {
       if (*cta_abort) return false;
+      if (t0 == 0) griddep_wait();
       unsigned long long now = globaltimer_ns();
       if (t0 == 0) t0 = now;
       else if (now - t0 > kWaitLimitNs) {

@@ -3,8 +3,6 @@ import os
 import re
 import subprocess
 
-import pytest
-
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_19561_b200", "csrc")
 
 
@@ -56,21 +54,18 @@ def test_paced_wait_ends_whatever_the_clock_does(tmp_path):
 """)
 
 
-@pytest.mark.parametrize("name", sorted(f for f in os.listdir(CSRC) if f.endswith(".cuh")
-                                        and re.search(r"^  griddep_launch_dependents\(\);", open(os.path.join(CSRC, f)).read(), re.M)))
-def test_no_limit_of_a_wait_counts_the_kernel_before(name):
-    """A kernel starts while the one before it in the stream still runs, for as long as that takes.  So every role passes
-    griddepcontrol.wait, which has no limit, before its first wait that has one."""
-    body = re.sub(r"//.*", "", open(os.path.join(CSRC, name)).read())
-    body = body[re.search(r"^  griddep_launch_dependents\(\);", body, re.M).start():]
-    roles = re.split(r"^  (?:if \(warp == \d+\) \{|\} else if \(warp == \d+\) \{|\} else \{)$", body, flags=re.M)
-    before, roles = roles[0], roles[1:]
-    assert len(roles) >= 3 and sum("mbar_wait" in r for r in roles) >= 3
-    if "griddep_wait();" in before:
-        return
-    for role in roles:
-        wait = re.search(r"mbar_wait\w*\(", role)
-        assert wait is None or "griddep_wait();" in role[:wait.start()], role[:400]
+def test_no_limit_of_a_wait_counts_the_kernel_before():
+    """A kernel starts while the one before it in the stream still runs, for as long as that takes.  So the clock of every wait that
+    gives up starts behind griddepcontrol.wait, which does not."""
+    src = re.sub(r"//.*", "", open(os.path.join(CSRC, "sm100_ptx.cuh")).read())
+    waits = [f for f in re.split(r"^__device__ ", src, flags=re.M) if "kErrTimeout | (site << 8)" in f]
+    assert len(waits) == 2
+    for body in waits:
+        clock = re.search(r"if \(t0 == 0\) griddep_wait\(\);\s+unsigned long long now = globaltimer_ns\(\);\s+if \(t0 == 0\) t0 = now;", body)
+        assert clock and body.count("globaltimer_ns()") == 1 and body.count("t0 = ") == 2      # zero, then the clock
+    for f in os.listdir(CSRC):                                    # no other file has a wait of its own
+        if f != "sm100_ptx.cuh":
+            assert "kErrTimeout" not in open(os.path.join(CSRC, f)).read(), f
 
 
 def test_a_wait_reports_what_it_waits_for():
