@@ -44,9 +44,17 @@ struct GemmWideCfg {
   __host__ __device__ static constexpr int slabs(int range) { return range <= 128 ? 2 : 1; }
   // Two slabs halve the waits and barriers per K, which bound a step of up to 128 columns (us, one slab / two: 200 x 4096, K = 14336
   // 15.9 / 13.2, 300 x 4096, K = 4096 7.3 / 6.7, NVFP4 400 x 4096 8.4 / 7.7, 150 x 5120, K = 5120 7.8 / 6.9, 200 x 6144, K = 4096
-  // 7.53 / 7.26; 512 x 4096, K = 14336 17.7 / 17.8).  With a few slabs in all the first stage is waited for longer (40 x 4096,
-  // K = 512 2.90 / 3.02): from four on.
-  __host__ __device__ static constexpr int range(int width, int64_t k_slabs) { return width > 256 ? 384 : (width > 128 || k_slabs < 4 ? 256 : 128); }
+  // 7.53 / 7.26), from four slabs on.  With few slabs the first stage is waited for longer (40 x 4096, K = 512 2.90 / 3.02), and so
+  // it is with four or five where more than 24 pairs read up to 176 tokens and the last slab is a half one, in NVFP4 with more
+  // tokens as well, or the pairs are up to 32 (144 x 4096, K = 1152 4.00 / 4.10, 80 x 2048 3.59 / 3.71, 80 x 4096, K = 1024 3.60 /
+  // 3.72, NVFP4 192 x 6144, K = 1152 4.74 / 4.98; beyond the line 112 x 3072, K = 1280 3.77 / 3.70, MXINT4 144 x 6144, K = 640 4.22 / 4.09).
+  __host__ __device__ static constexpr bool two_slabs(int64_t M, int64_t K, int64_t pairs) {
+    const int64_t k_slabs = (K + BK - 1) / BK;
+    if (k_slabs < 4 || k_slabs > 5 || pairs <= 24) return k_slabs >= 4;
+    if (K % BK != 0) return M > 176 && FMT != FMT_NVFP4;
+    return M > 176 || pairs > 32 || (FMT == FMT_MXINT4 && k_slabs == 5);
+  }
+  __host__ __device__ static constexpr int range(int width, bool two) { return width > 256 ? 384 : (width > 128 || !two ? 256 : 128); }
   __host__ __device__ static constexpr int stage_bytes(int width, int range) { return slabs(range) * slab_bytes(width); }
   __host__ __device__ static constexpr int stages(int width, int range) {
     return (232448 - 2048) / stage_bytes(width, range) < MAX_STAGES ? (232448 - 2048) / stage_bytes(width, range) : MAX_STAGES;

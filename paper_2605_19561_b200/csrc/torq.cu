@@ -786,7 +786,7 @@ static torq_status gemm_wide(DeviceState* st, const void* Aq, const void* As, co
     return TORQ_ERR_LAUNCH;
   if (width <= 256) tmB1 = tmB;
   const int rows = (int)((M + 255) / 256), cols = (int)((N + width - 1) / width);
-  const int range = C::range(width, (K + C::BK - 1) / C::BK);
+  const int range = C::range(width, C::two_slabs(M, K, (int64_t)rows * cols));
   launch_tc(range == 384 ? mxfp4_gemm_wide_kernel<FMT, 384> : (range == 256 ? mxfp4_gemm_wide_kernel<FMT, 256> : mxfp4_gemm_wide_kernel<FMT, 128>),
             2, 2 * rows * cols, C::THREADS, C::smem_bytes(width, range), s, tmA, tmB, tmB1, tmSFA, tmSFB, tmY, ybf ? 1 : 0, (int)M, (int)N, (int)K, rows, width, alpha,
             st->err_word);

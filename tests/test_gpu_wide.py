@@ -222,3 +222,24 @@ def test_rotation_kernel_of_97_to_256_tokens(fmt, M, d, kernel):
     (name, _), = captured_launches(call)
     assert {"wide": "rotate_quantize_wide_kernel", "fewtok": "rotate_fewtok_kernel"}[kernel] in name
     assert torq.torq_last_device_error() == 0
+
+
+@pytest.mark.parametrize("fmt,M,N,K,span", [("mxfp4", 144, 4096, 1152, 256), ("mxfp4", 80, 2048, 1024, 256), ("mxfp4", 144, 512, 1024, 128),
+                                            ("mxfp4", 176, 2048, 1280, 256), ("mxfp4", 177, 2048, 1280, 128), ("mxfp4", 144, 4096, 1408, 128),
+                                            ("mxfp4", 300, 4096, 768, 256), ("nvfp4", 192, 6144, 1152, 256), ("nvfp4", 192, 6144, 1280, 128),
+                                            ("nvfp4", 128, 1536, 1152, 128), ("mxint4", 128, 4096, 512, 256), ("mxint4", 200, 4096, 512, 128),
+                                            ("mxint4", 128, 4096, 640, 128), ("mxfp4", 144, 3072, 1280, 128), ("mxfp4", 144, 6144, 1152, 256),
+                                            ("mxfp4", 1000, 6144, 4096, 384)])
+def test_gemm_takes_two_slabs_per_stage_where_they_are_the_faster(fmt, M, N, K, span):
+    """Which instance of the one-wave kernel a call takes, by its template arguments: 128 is the one with two slabs."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the line is one of 148 SMs")
+    A, W = (torch.zeros((r, K if fmt == "mxint4" else K // 2), dtype=torch.uint8, device="cuda") for r in (M, N))
+    As, Ws = (torch.zeros(torq.torq_nvfp4_scales_bytes(r, K) if fmt == "nvfp4" else torq.torq_scales_bytes(r, K), dtype=torch.uint8,
+                          device="cuda") for r in (M, N))
+    call = {"mxfp4": lambda: torq.torq_mxfp4_gemm(A, As, W, Ws), "mxint4": lambda: torq.torq_mxint4_gemm(A, As, W, Ws),
+            "nvfp4": lambda: torq.torq_nvfp4_gemm(A, As, 1.0, W, Ws, 1.0)}[fmt]
+    call()
+    (name, _), = captured_launches(call)
+    assert f"mxfp4_gemm_wide_kernelILi{['mxfp4', 'nvfp4', 'mxint4'].index(fmt)}ELi{span}E" in name
+    assert torq.torq_last_device_error() == 0
