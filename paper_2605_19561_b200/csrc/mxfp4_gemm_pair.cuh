@@ -186,7 +186,7 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     // ------------------------------------------------------------------ MMA issuer (leader only)
     if (rank == 0) {
       uint32_t it = 0, tcount = 0;
-      bool ok = mbar_wait_cluster_warp(alloc_bar, 0, cta_abort, err_word, SITE_PEER_TMEM);
+      bool ok = mbar_wait_cluster_warp<true>(alloc_bar, 0, cta_abort, err_word, SITE_PEER_TMEM);
       // instruction descriptors differ between the two tile widths only in the N field ([17,23) = N >> 3)
       constexpr uint32_t n_less = (uint32_t)((BN - kNarrowCols) >> 3) << 17;
       const uint32_t sfa_t = tmem_base + C::SFA_COL, sfb_t = tmem_base + C::SFB_COL;
@@ -206,7 +206,7 @@ mxfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         auto stage = [&](int kt, auto waits) -> bool {
           constexpr bool WAITS = decltype(waits)::value;
           const int s = it % C::STAGES;
-          if (!mbar_wait_cluster_warp(full_bar(s), (it / C::STAGES) & 1, cta_abort, err_word, SITE_MMA_FULL)) return false;
+          if (!mbar_wait_cluster_warp<true>(full_bar(s), (it / C::STAGES) & 1, cta_abort, err_word, SITE_MMA_FULL)) return false;
           tc_fence_after_sync();
           const bool two = (kb4 - CH * kt) >= CH;          // K % 256 == 128: the last stage is half
           const uint32_t st = smem_base + s * C::STAGE_BYTES;

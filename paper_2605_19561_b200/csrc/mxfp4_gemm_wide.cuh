@@ -182,7 +182,7 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       uint32_t ph = 0;
       bool ok = true;
       for (int kt = 0; kt < k_tiles; ++kt) {
-        ok = mbar_wait_cluster_warp(full_bar(s), ph, cta_abort, err_word, SITE_MMA_FULL);
+        ok = mbar_wait_cluster_warp<true>(full_bar(s), ph, cta_abort, err_word, SITE_MMA_FULL);
         if (!ok) break;
         tc_fence_after_sync();
         if (elect_one()) {

@@ -166,7 +166,7 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       constexpr uint32_t idesc_wide = idesc_bf16(256, BN, /*A MN-major*/ false, /*B MN-major*/ true);
       constexpr uint32_t idesc_narrow = idesc_bf16(256, kNarrowCols, false, true);
       uint32_t it = 0, tcount = 0;
-      bool ok = mbar_wait_cluster_warp(alloc_bar, 0, cta_abort, err_word, SITE_PEER_TMEM);
+      bool ok = mbar_wait_cluster_warp<true>(alloc_bar, 0, cta_abort, err_word, SITE_PEER_TMEM);
       for (int tile = pair; tile < total_tiles && ok; tile += npairs, ++tcount) {
         int mp, tcol;
         bool narrow;
@@ -180,7 +180,7 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
         const uint32_t acc = tmem_base + a * BN;
         for (int kt = 0; kt < k_tiles; ++kt, ++it) {
           const int s = it % C::STAGES;
-          if (!mbar_wait_cluster_warp(full_bar(s), (it / C::STAGES) & 1, cta_abort, err_word, SITE_MMA_FULL)) {
+          if (!mbar_wait_cluster_warp<true>(full_bar(s), (it / C::STAGES) & 1, cta_abort, err_word, SITE_MMA_FULL)) {
             ok = false; break;
           }
           tc_fence_after_sync();

@@ -157,14 +157,14 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader only)
-    if (rank == 0 && mbar_wait_cluster_warp(alloc_bar, 0, cta_abort, err_word, SITE_PEER_TMEM) && elect_one()) {
+    if (rank == 0 && mbar_wait_cluster_warp<true>(alloc_bar, 0, cta_abort, err_word, SITE_PEER_TMEM) && elect_one()) {
       const uint32_t idesc0 = idesc_bf16(256, n0, /*A MN-major*/ false, /*B MN-major*/ true);
       constexpr uint32_t idesc1 = idesc_bf16(256, 128, false, true);
       int s = 0;
       uint32_t ph = 0;
       bool ok = true;
       for (int kt = 0; kt < k_tiles; ++kt) {
-        ok = mbar_wait_cluster(full_bar(s), ph, cta_abort, err_word, SITE_MMA_FULL);
+        ok = mbar_wait_cluster<true>(full_bar(s), ph, cta_abort, err_word, SITE_MMA_FULL);
         if (!ok) break;
         tc_fence_after_sync();
         const uint32_t st = smem_base + s * stage_bytes;

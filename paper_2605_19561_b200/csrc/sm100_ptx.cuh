@@ -66,9 +66,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 }
 // Bounded wait.  Returns false when the CTA has been told to give up (another wait timed out) or
 // when this wait itself exceeds kWaitLimitNs; in the latter case it latches the error word and
-// raises the CTA's abort flag so that every other role leaves its loop too.  The limit does not count what is left of the kernel
-// before, which may take any time: the clock starts behind griddep_wait().  (There and not ahead of the wait, where it would cost
-// every call: an issuer that passed it before its first wait made the one-wave rotations 0.5 % slower, 0.025 us in the mean of 58 shapes.)
+// raises the CTA's abort flag so that every other role leaves its loop too.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* cta_abort,
                                           int* err_word, int site,
                                           unsigned long long limit_ns = kWaitLimitNs) {
@@ -78,7 +76,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if (mbar_try_wait(bar, parity)) return true;
     if ((it & 0x3FFu) == 0) {
       if (*cta_abort) return false;
-      if (t0 == 0) griddep_wait();
       unsigned long long now = globaltimer_ns();
       if (t0 == 0) t0 = now;
       else if (now - t0 > limit_ns) {
@@ -390,7 +387,11 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
       : "memory");
   return ok != 0;
 }
-// Bounded wait on a local barrier whose arrivals may come from the peer CTA.
+// Bounded wait on a local barrier whose arrivals may come from the peer CTA.  BEHIND_DEP: of a role that has not passed
+// griddep_wait().  Its limit does not count what is left of the kernel before, which may take any time: the clock starts behind
+// that.  (Not ahead of the wait: an issuer that passed it before its first wait made the one-wave rotations 0.5 % slower.  And not in
+// every wait: a layer of one token and d = N = 5120 on the few-token kernels, which pass it at their start, 15.69 -> 15.75 us.)
+template <bool BEHIND_DEP = false>
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
                                                   volatile int* cta_abort, int* err_word, int site) {
   if (mbar_try_wait_cluster(bar, parity)) return true;
@@ -399,7 +400,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     if (mbar_try_wait_cluster(bar, parity)) return true;
     if ((it & 0x3FFu) == 0) {
       if (*cta_abort) return false;
-      if (t0 == 0) griddep_wait();
+      if (BEHIND_DEP && t0 == 0) griddep_wait();
       unsigned long long now = globaltimer_ns();
       if (t0 == 0) t0 = now;
       else if (now - t0 > kWaitLimitNs) {
@@ -410,9 +411,10 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     }
   }
 }
+template <bool BEHIND_DEP = false>
 __device__ __forceinline__ bool mbar_wait_cluster_warp(uint32_t bar, uint32_t parity,
                                                        volatile int* cta_abort, int* err_word, int site) {
-  return __all_sync(0xFFFFFFFFu, mbar_wait_cluster(bar, parity, cta_abort, err_word, site));
+  return __all_sync(0xFFFFFFFFu, mbar_wait_cluster<BEHIND_DEP>(bar, parity, cta_abort, err_word, site));
 }
 // 2-D tiled load into THIS CTA's shared memory whose completion bytes are counted on a barrier
 // that may live in the other CTA of the pair (`bar_cluster_addr` from map_to_cta).  The data goes to this CTA alone.

@@ -3,6 +3,8 @@ import os
 import re
 import subprocess
 
+import pytest
+
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_19561_b200", "csrc")
 
 
@@ -54,18 +56,28 @@ def test_paced_wait_ends_whatever_the_clock_does(tmp_path):
 """)
 
 
-def test_no_limit_of_a_wait_counts_the_kernel_before():
-    """A kernel starts while the one before it in the stream still runs, for as long as that takes.  So the clock of every wait that
-    gives up starts behind griddepcontrol.wait, which does not."""
-    src = re.sub(r"//.*", "", open(os.path.join(CSRC, "sm100_ptx.cuh")).read())
-    waits = [f for f in re.split(r"^__device__ ", src, flags=re.M) if "kErrTimeout | (site << 8)" in f]
-    assert len(waits) == 2
-    for body in waits:
-        clock = re.search(r"if \(t0 == 0\) griddep_wait\(\);\s+unsigned long long now = globaltimer_ns\(\);\s+if \(t0 == 0\) t0 = now;", body)
-        assert clock and body.count("globaltimer_ns()") == 1 and body.count("t0 = ") == 2      # zero, then the clock
-    for f in os.listdir(CSRC):                                    # no other file has a wait of its own
-        if f != "sm100_ptx.cuh":
-            assert "kErrTimeout" not in open(os.path.join(CSRC, f)).read(), f
+@pytest.mark.parametrize("name", sorted(f for f in os.listdir(CSRC) if f.endswith(".cuh")
+                                        and re.search(r"^  griddep_launch_dependents\(\);", open(os.path.join(CSRC, f)).read(), re.M)))
+def test_no_limit_of_a_wait_counts_the_kernel_before(name):
+    """A kernel starts while the one before it in the stream still runs, for as long as that takes.  So a role either passes
+    griddepcontrol.wait, which has no limit, before its first wait that has one, or the clock of all its waits for what other roles
+    bring after that starts behind it."""
+    body = re.sub(r"//.*", "", open(os.path.join(CSRC, name)).read())
+    body = body[re.search(r"^  griddep_launch_dependents\(\);", body, re.M).start():]
+    roles = re.split(r"^  (?:if \(warp == \d+\) \{|\} else if \(warp == \d+\) \{|\} else \{)$", body, flags=re.M)
+    before, roles = roles[0], roles[1:]
+    assert len(roles) >= 3 and sum("mbar_wait" in r for r in roles) >= 3
+    if "griddep_wait();" in before:
+        return
+    for role in roles:
+        first = re.search(r"mbar_wait", role)
+        if first is None or "griddep_wait();" in role[:first.start()]:
+            continue
+        waits = re.findall(r"mbar_wait\w*(<true>)?\((\w+)", role)
+        # a wait for a free accumulator passes at once in the first tiles and comes behind their instructions in later ones
+        assert waits and all(dep == "<true>" or bar == "acce_bar" for dep, bar in waits), waits
+    ptx = open(os.path.join(CSRC, "sm100_ptx.cuh")).read()
+    assert re.search(r"if \(BEHIND_DEP && t0 == 0\) griddep_wait\(\);\s+unsigned long long now = globaltimer_ns\(\);\s+if \(t0 == 0\) t0 = now;", ptx)
 
 
 def test_a_wait_reports_what_it_waits_for():
@@ -77,7 +89,7 @@ def test_a_wait_reports_what_it_waits_for():
     assert len({i for _, i in ids}) == len(ids) and set(kinds.values()) <= {n for n, _ in ids}
     seen = set()
     for f in os.listdir(CSRC):
-        for bar, site in re.findall(r"mbar_wait\w*\((\w+_bar)\b[^;{]*?(SITE_\w+)\)", open(os.path.join(CSRC, f)).read()):
+        for bar, site in re.findall(r"mbar_wait\w*(?:<true>)?\((\w+_bar)\b[^;{]*?(SITE_\w+)\)", open(os.path.join(CSRC, f)).read()):
             if bar in kinds:
                 assert site == kinds[bar], (f, bar, site)
                 seen.add(bar)
