@@ -376,14 +376,21 @@ int torq_last_device_error(void* stream);
  * in which they are dealt round robin: tile i goes to pair i % pairs.  Tiles are 256 rows high and
  * 256 columns wide; where that leaves the last wave partly empty and cols is a multiple of 256,
  * some row tiles are covered by fewer 256-column tiles followed by 192-column ones (three wide
- * tiles traded for four narrow ones), chosen so that the longest pair finishes earliest.  Both
- * torq_rotate_quantize (cols = d) and torq_mxfp4_gemm (cols = N), and their format variants, use
- * this list where these kernels serve a call, except that a rotation with d > 4096 whose last wave
- * would hold a few 256-column tiles leaves those to another kernel (see torq_rotated_linear).
+ * tiles traded for four narrow ones), chosen so that the longest pair finishes earliest.
+ * torq_rotate_quantize (cols = d) and its format variants use this list where these kernels serve a
+ * call, except that a rotation with d > 4096 whose last wave would hold a few 256-column tiles
+ * leaves those to another kernel (see torq_rotated_linear).  Of a GEMM (cols = N) these are the
+ * tiles; torq_gemm_tile_list has them in its order.
  *   out: host array of 3 * cap int32, or NULL; receives (row_tile, first_column, width) per tile.
  * Returns the number of tiles (also when it exceeds cap; only cap triples are written), or -1 for
  * rows < 1, cols < 1 or pairs < 1. */
 int64_t torq_pair_tile_list(int64_t rows, int64_t cols, int32_t pairs, int32_t* out, int64_t cap);
+
+/* The same for torq_mxfp4_gemm and its format variants on an [M x N] output with weights whose rows
+ * are `w_row_bytes` long (K / 2; MXINT4: K): the tiles of torq_pair_tile_list(M, N), with the row
+ * tiles taken in groups of sixteen instead of eight where N is 10240 or more and the weights are 16
+ * MiB or more, or 8192 and 32 MiB.  Same results; -1 also for w_row_bytes < 1. */
+int64_t torq_gemm_tile_list(int64_t M, int64_t N, int64_t w_row_bytes, int32_t pairs, int32_t* out, int64_t cap);
 
 /* Number of kernels this library has launched since load (all devices, all streams). */
 int64_t torq_launch_count(void);

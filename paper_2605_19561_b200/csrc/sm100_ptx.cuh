@@ -500,18 +500,16 @@ __device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint16_t cta_mask) 
       ::"r"(bar), "h"(cta_mask) : "memory");
 }
 
-// Tile order of the persistent CTA-pair kernels.  Row tiles are taken in groups of eight; inside a
-// group the row tile is the fast index.  The ~74 tiles in flight at any time then cover about
-// 8 row tiles x 9 column tiles, whatever M is, so both operands of a wave stay in L2 (with the row
+// Tile order of the persistent CTA-pair kernels.  Row tiles are taken in groups (of eight, or sixteen in GEMMs with many columns); inside
+// a group the row tile is the fast index.  The ~74 tiles in flight at any time then cover about
+// 8 row tiles x 9 column tiles or 16 x 5, whatever M is, so both operands of a wave stay in L2 (with the row
 // tile as the fast index over ALL of M, a wave at M = 16384 touched 64 row tiles and one or two
-// column tiles, and the row operand was re-read from HBM for every column tile).  Groups of sixteen for weights of 16 MiB and more
-// are no faster: 138 GEMMs of 2500 to 16384 tokens timed in turn with this, 0.997 in the geometric mean.
-__host__ __device__ __forceinline__ void pair_tile_coords(int tile, int mp_tiles, int n_tiles, int& mp, int& nt) {
-  constexpr int G = 8;
-  const int per_group = G * n_tiles;
+// column tiles, and the row operand was re-read from HBM for every column tile).
+__host__ __device__ __forceinline__ void pair_tile_coords(int tile, int mp_tiles, int n_tiles, int group, int& mp, int& nt) {
+  const int per_group = group * n_tiles;
   const int g = tile / per_group, r = tile - g * per_group;
-  const int rows_in_group = mp_tiles - g * G < G ? mp_tiles - g * G : G;
-  mp = g * G + r % rows_in_group;
+  const int rows_in_group = mp_tiles - g * group < group ? mp_tiles - g * group : group;
+  mp = g * group + r % rows_in_group;
   nt = r / rows_in_group;
 }
 
@@ -529,6 +527,7 @@ struct MixedTiles {
   int wide_b;      // 256-column tiles of the other row tiles
   int narrow_b;    // 192-column tiles of the other row tiles
   int total;       // tiles in all
+  int group;       // row tiles taken together
 };
 constexpr int kNarrowCols = 192;
 
@@ -540,6 +539,7 @@ __host__ __device__ __forceinline__ MixedTiles mixed_tiles_make(int rows, int wi
   t.wide_b = wide_cols - 3 * (units / rows);
   t.narrow_b = 4 * (units / rows);
   t.total = rows * wide_cols + units;
+  t.group = 8;
   return t;
 }
 
@@ -548,7 +548,7 @@ __host__ __device__ __forceinline__ void mixed_tile_coords(int tile, const Mixed
   int nt;
   const int n1 = t.rows * wide_common;
   if (tile < n1) {
-    pair_tile_coords(tile, t.rows, wide_common, mp, nt);
+    pair_tile_coords(tile, t.rows, wide_common, t.group, mp, nt);
     col0 = nt * 256;
     narrow = false;
     return;
@@ -566,7 +566,7 @@ __host__ __device__ __forceinline__ void mixed_tile_coords(int tile, const Mixed
   narrow = true;
   const int n3 = t.rows * t.narrow_b;
   if (tile < n3) {
-    pair_tile_coords(tile, t.rows, t.narrow_b, mp, nt);
+    pair_tile_coords(tile, t.rows, t.narrow_b, t.group, mp, nt);
   } else {
     tile -= n3;
     mp = tile % t.rows_a;

@@ -363,6 +363,30 @@ static MixedTiles plan_pair_tiles(int rows, int64_t cols, int max_pairs, double 
   return mixed_tiles_make(rows, wide_cols, best_units);
 }
 
+// The list of a GEMM whose weights have rows of `w_row_bytes`.  Every group of row tiles reads all of W once: many columns in groups of
+// sixteen.  A long call runs at the power cap, where the traffic that this saves is clock, so loops of 0.9 s on each side in turn
+// (us, eight / sixteen): 8192 x 51200, K = 5120 838 / 819, x 28672, K = 4096 388 / 378, x 14336 196 / 192, MXINT4 361 / 355, NVFP4 211 /
+// 207, 4096 x 16384, K = 2048 69.1 / 68.6, 4096 x 10240, K = 8192 133 / 130, 8192 x 10240, K = 4096 139.3 / 139.0, x 8192, K = 8192 215.0 /
+// 213.4.  Fewer columns or smaller weights lose: x 9216, K = 4096 125.0 / 125.3, 4500 x 8448 66.7 / 67.3, 8192 x 4096, K = 14336 179 /
+// 181, x 28672, K = 256 102 / 103; the rotation loses too (d = 14336, 8192 tokens, the layer 2886 / 3062).
+static MixedTiles plan_gemm_tiles(int64_t M, int64_t N, uint64_t w_row_bytes, int max_pairs) {
+  MixedTiles t = plan_pair_tiles((int)((M + 255) / 256), N, max_pairs, kNarrowTileCost);
+  if (N >= 8192 && (uint64_t)N * w_row_bytes >= (N >= 10240 ? 16u << 20 : 32u << 20)) t.group = 16;
+  return t;
+}
+
+static int64_t write_tile_list(const MixedTiles& t, int32_t* out, int64_t cap) {
+  for (int i = 0; out && i < t.total && i < cap; ++i) {
+    int mp, col0;
+    bool narrow;
+    mixed_tile_coords(i, t, mp, col0, narrow);
+    out[3 * i] = mp;
+    out[3 * i + 1] = col0;
+    out[3 * i + 2] = narrow ? kNarrowCols : 256;
+  }
+  return t.total;
+}
+
 static size_t quantized_bytes(int64_t M, int64_t d) {    // codes, then 256-byte aligned the scales
   return ((size_t)M * (size_t)(d / 2) + 255) / 256 * 256 + torq_scales_bytes(M, d);
 }
@@ -419,16 +443,12 @@ const char* torq_status_string(torq_status s) {
 
 int64_t torq_pair_tile_list(int64_t rows, int64_t cols, int32_t pairs, int32_t* out, int64_t cap) {
   if (rows < 1 || cols < 1 || pairs < 1 || rows > INT32_MAX / 2 || cols > INT32_MAX / 2) return -1;
-  const torq::MixedTiles t = torq::plan_pair_tiles((int)((rows + 255) / 256), cols, pairs, torq::kNarrowTileCost);
-  for (int i = 0; out && i < t.total && i < cap; ++i) {
-    int mp, col0;
-    bool narrow;
-    torq::mixed_tile_coords(i, t, mp, col0, narrow);
-    out[3 * i] = mp;
-    out[3 * i + 1] = col0;
-    out[3 * i + 2] = narrow ? torq::kNarrowCols : 256;
-  }
-  return t.total;
+  return write_tile_list(plan_pair_tiles((int)((rows + 255) / 256), cols, pairs, kNarrowTileCost), out, cap);
+}
+
+int64_t torq_gemm_tile_list(int64_t M, int64_t N, int64_t w_row_bytes, int32_t pairs, int32_t* out, int64_t cap) {
+  if (M < 1 || N < 1 || w_row_bytes < 1 || pairs < 1 || M > INT32_MAX / 2 || N > INT32_MAX / 2 || w_row_bytes > INT32_MAX) return -1;
+  return write_tile_list(plan_gemm_tiles(M, N, (uint64_t)w_row_bytes, pairs), out, cap);
 }
 
 int64_t torq_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
@@ -859,7 +879,7 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
   if (!encode_2d(&tmBn, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, kNarrowCols / 2, 128))
     return TORQ_ERR_LAUNCH;
   const int max_pairs = st->gemm_pairs;
-  const MixedTiles list = plan_pair_tiles((int)((M + 255) / 256), N, max_pairs, kNarrowTileCost);
+  const MixedTiles list = plan_gemm_tiles(M, N, krow, max_pairs);
   const int pairs = list.total < max_pairs ? list.total : max_pairs;
   launch_tc(mxfp4_gemm_pair_kernel<FMT>, 2, 2 * pairs, GemmPairCfgT<FMT>::THREADS, GemmPairCfgT<FMT>::SMEM_BYTES, s,
             tmA, tmB, tmSFA, tmSFB, tmY, tmBn, list, ybf ? 1 : 0, (int)M, (int)N, (int)K, alpha, st->err_word);

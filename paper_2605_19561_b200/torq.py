@@ -115,6 +115,8 @@ def lib() -> ctypes.CDLL:
     L.torq_last_device_error.restype = ci
     L.torq_pair_tile_list.argtypes = [i64, i64, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32), i64]
     L.torq_pair_tile_list.restype = i64
+    L.torq_gemm_tile_list.argtypes = [i64, i64, i64, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32), i64]
+    L.torq_gemm_tile_list.restype = i64
     L.torq_launch_count.argtypes = []
     L.torq_launch_count.restype = i64
     _lib_handle = L
@@ -235,6 +237,16 @@ def torq_pair_tile_list(rows: int, cols: int, pairs: int = 74):
         raise ValueError("torq_pair_tile_list: rows, cols and pairs must be positive")
     buf = (ctypes.c_int32 * (3 * n))()
     lib().torq_pair_tile_list(rows, cols, pairs, buf, n)
+    return [(buf[3 * i], buf[3 * i + 1], buf[3 * i + 2]) for i in range(n)]
+
+
+def torq_gemm_tile_list(M: int, N: int, w_row_bytes: int, pairs: int = 74):
+    """The same for a GEMM, in its order (w_row_bytes: K / 2, MXINT4 K)."""
+    n = lib().torq_gemm_tile_list(M, N, w_row_bytes, pairs, None, 0)
+    if n < 0:
+        raise ValueError("torq_gemm_tile_list: M, N, w_row_bytes and pairs must be positive")
+    buf = (ctypes.c_int32 * (3 * n))()
+    lib().torq_gemm_tile_list(M, N, w_row_bytes, pairs, buf, n)
     return [(buf[3 * i], buf[3 * i + 1], buf[3 * i + 2]) for i in range(n)]
 
 

@@ -165,9 +165,31 @@ def test_pair_tile_list_covers_every_output_exactly_once():
     assert torq.lib().torq_pair_tile_list(0, 4096, 74, None, 0) == -1
 
 
-def test_the_gemm_walks_the_pair_tile_list_as_it_is():
-    """torq_pair_tile_list answers from rows and columns alone, so nothing else may go into the list that a launch is given."""
+def test_gemm_tile_list_is_what_the_gemm_walks():
+    """The GEMM's own order: that of torq_pair_tile_list, or groups of sixteen row tiles from 10240 columns and 16 MiB of weights
+    (8192 and 32 MiB) on; each output covered exactly once either way, whole groups and partial ones, with and without narrow tiles."""
+    for pairs in (74, 66, 8):
+        for M, N in [(17 * 256, 10240), (4500, 10496), (25 * 256, 12288), (33 * 256, 14336), (8192, 51200), (16 * 256, 14336), (2048, 16384),
+                     (19 * 256, 1024), (5000, 10248), (33 * 256, 10232), (21 * 256, 8192),
+                     (18 * 256, 8184)]:
+            tiles = torq.torq_pair_tile_list(M, N, pairs)
+            line = -(-((16 if N >= 10240 else 32) << 20) // N)    # bytes per row from which W is 16 or 32 MiB
+            assert torq.torq_gemm_tile_list(M, N, line - 1, pairs) == tiles
+            tl = torq.torq_gemm_tile_list(M, N, line, pairs)
+            rt = (M + 255) // 256
+            assert len(tl) == len(tiles) and sorted(tl) == sorted(tiles)
+            cover = np.zeros((rt, (N + 63) // 64), np.int32)
+            for mp, c0, w in tl:
+                cover[mp, c0 // 64:-(-min(N, c0 + w) // 64)] += 1
+            assert (cover == 1).all(), (pairs, M, N)
+            if rt <= 8 or N < 8192:
+                assert tl == tiles
+            else:
+                group = min(rt, 16)
+                assert [mp for mp, _, _ in tl[:group]] == list(range(group)) and len({c0 for _, c0, _ in tl[:group]}) == 1
+    assert torq.lib().torq_gemm_tile_list(256, 256, 0, 74, None, 0) == -1
+    assert torq.lib().torq_gemm_tile_list(0, 256, 128, 74, None, 0) == -1
+    # the launch takes the planner's list as it is
     src = open(os.path.join(ROOT, "paper_2605_19561_b200", "csrc", "torq.cu")).read()
     gemm = src[src.index("static torq_status gemm_impl("):src.index("torq_status torq_mxfp4_gemm(")]
-    assert gemm.count("MixedTiles list = plan_pair_tiles((int)((M + 255) / 256), N, max_pairs, kNarrowTileCost);") == 1
-    assert not re.search(r"\blist\.\w+\s*=[^=]", gemm)
+    assert gemm.count("const MixedTiles list = plan_gemm_tiles(M, N, krow, max_pairs);") == 1

@@ -16,6 +16,7 @@ import test_gpu_mxint4 as TI
 import test_gpu_nvfp4 as TN
 
 pytestmark = pytest.mark.gpu
+E2M1 = np.array([0, .5, 1, 1.5, 2, 3, 4, 6, 0, -.5, -1, -1.5, -2, -3, -4, -6], np.float32)
 
 
 def _pairs():
@@ -201,6 +202,40 @@ def test_gemm_from_eight_stages_on_paces_the_output_and_starts_the_scales_early(
 def test_gemm_from_sixteen_stages_on_paces_float32_output_too(fmt, M, N, K):
     """Fifteen and sixteen stages: the last length at which float32 boxes go out at once and the first at which they are spread."""
     test_gemm_from_eight_stages_on_paces_the_output_and_starts_the_scales_early(fmt, M, N, K)
+
+
+@pytest.mark.parametrize("fmt,M,N,K,narrow", [("mxfp4", 4300, 10240, 3456, True), ("mxfp4", 4500, 10248, 4096, False),
+                                              ("nvfp4", 4500, 10752, 3328, True), ("mxint4", 4300, 11264, 1536, True)])
+def test_gemm_with_many_columns_takes_row_tiles_in_sixteens(fmt, M, N, K, narrow):
+    """A whole and a partial group of sixteen row tiles, with and without narrow tiles.  Scales of 1/2, 1 and 2 by block: every sum
+    is exact in float32, so the whole output is the product of the dequantized operands bit for bit."""
+    tl = torq.torq_gemm_tile_list(M, N, K if fmt == "mxint4" else K // 2, _pairs())
+    assert [mp for mp, _, _ in tl[:16]] == list(range(16)) and len({mp for mp, _, _ in tl}) % 16 != 0
+    if _pairs() == 74:
+        assert any(w == 192 for _, _, w in tl) == narrow
+    g = np.random.default_rng(M + N)
+    blk = 16 if fmt == "nvfp4" else 32
+
+    def operand(rows):
+        sb = g.integers(0, 3, (rows, K // blk))
+        if fmt == "mxint4":
+            q = g.integers(-7, 8, (rows, K)).astype(np.int8)
+            val, dat = q.astype(np.float32), dev_u8(O.int4_to_e4m3(q))
+        else:
+            c = g.integers(0, 16, (rows, K), dtype=np.uint8)
+            val, dat = E2M1[c], dev_u8(O.pack_codes(c))
+        sc = dev_u8(O.nv_swizzle_scales((0x30 + 8 * sb).astype(np.uint8), K) if fmt == "nvfp4"
+                    else O.swizzle_scales((126 + sb).astype(np.uint8), K, fill=0))
+        return dat, sc, torch.from_numpy(val).cuda() * torch.from_numpy(np.float32(2.0) ** (sb - 1)).float().cuda().repeat_interleave(blk, 1)
+
+    (a, As, av), (w, Ws, wv) = operand(M), operand(N)
+    if fmt == "nvfp4":
+        y = torq.torq_nvfp4_gemm(a, As, 1.0, w, Ws, 1.0, out_dtype=torch.float32)
+    else:
+        y = (torq.torq_mxint4_gemm if fmt == "mxint4" else torq.torq_mxfp4_gemm)(a, As, w, Ws, out_dtype=torch.float32)
+    torch.cuda.synchronize()
+    assert torq.torq_last_device_error() == 0
+    assert torch.equal(y, av @ wv.T)                             # sums below 2^24 units of the smallest product, in any order
 
 
 @pytest.mark.parametrize("M,d", [(2300, 4352), (2000, 4864), (4096, 4864)])
