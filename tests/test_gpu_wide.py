@@ -181,27 +181,42 @@ def test_rotation_with_two_slabs_per_stage(M, d):
     assert np.array_equal(g_sb[rows], o_sb) and np.array_equal(g_codes[rows], o_codes)
 
 
-# one to four CTA pairs per row tile, widths 64 and 128: as many slabs of K as fill one ring, an odd number, a half last one, several rounds
-@pytest.mark.parametrize("M,N,K", [(200, 72, 1024), (300, 520, 1152), (129, 2056, 1280), (513, 1000, 2944), (200, 6144, 5376)])
-def test_gemm_with_two_slabs_per_stage(M, N, K):
-    """Scales of one and small integers as codes, so that every sum is exact: the three formats equal the product bit for bit."""
+# tiles of 64 columns on 2, 18 and 33 CTA pairs and of 128 on 24 and 48: four slabs of K, as many as fill one ring (ten), an odd number, a half last
+# one, several rounds.  K8: of MXINT4, whose slabs are half as long
+@pytest.mark.parametrize("M,N,K,K8", [(200, 72, 1024, 512), (200, 72, 2560, 1280), (300, 520, 1152, 640), (129, 2056, 1280, 640), (513, 1000, 2944, 1408),
+                                      (200, 6144, 5376, 2688)])
+def test_gemm_with_two_slabs_per_stage(M, N, K, K8):
+    """Scales of 1/2, 1 and 2 by row and block and small integers as codes, so that every sum is exact: the three formats equal the product
+    bit for bit, and a chunk of scales taken from the other slab of a stage would show.  Each call is of the instance with two slabs."""
     g = np.random.default_rng(M + N + K)
     rows = np.unique(np.r_[0:min(M, 24), max(0, M - 24):M])
     grid = np.array([0, .5, 1, 1.5, 2, 3, 4, 6, 0, -.5, -1, -1.5, -2, -3, -4, -6])
+
+    def check(fmt, k, call, av, wv, asb, wsb):
+        blk = k // asb.shape[1]
+        y = call()
+        (name, _), = captured_launches(call)
+        assert f"mxfp4_gemm_wide_kernelILi{['mxfp4', 'nvfp4', 'mxint4'].index(fmt)}ELi128E" in name, (fmt, name)
+        scaled = lambda v, sb: v * np.repeat(2.0 ** (sb.astype(np.int64) - 1), blk, axis=1)
+        assert np.array_equal(y.cpu().numpy()[rows], scaled(av[rows], asb[rows]) @ scaled(wv, wsb).T), fmt
+
+    s32 = lambda sb, k: dev_u8(O.swizzle_scales((126 + sb).astype(np.uint8), k, fill=0))
+    s16 = lambda sb, k: dev_u8(O.nv_swizzle_scales((0x30 + 8 * sb).astype(np.uint8), k))                 # E4M3 1/2, 1, 2
+    sc = lambda n, k, blk: g.integers(0, 3, (n, k // blk), dtype=np.uint8)
     ac, wc = g.integers(0, 16, (M, K), dtype=np.uint8), g.integers(0, 16, (N, K), dtype=np.uint8)
-    ref = (grid[ac[rows]] @ grid[wc].T)
-    one = lambda n, k: dev_u8(O.swizzle_scales(np.full((n, k // 32), 127, np.uint8), k, fill=0))
-    one16 = lambda n, k: dev_u8(O.nv_swizzle_scales(np.full((n, k // 16), 0x38, np.uint8), k))     # E4M3 1.0
     a, w = dev_u8(O.pack_codes(ac)), dev_u8(O.pack_codes(wc))
-    y = torq.torq_mxfp4_gemm(a, one(M, K), w, one(N, K), out_dtype=torch.float32)
-    assert np.array_equal(y.cpu().numpy()[rows], ref)
-    y = torq.torq_nvfp4_gemm(a, one16(M, K), 1.0, w, one16(N, K), 1.0, out_dtype=torch.float32)
-    assert np.array_equal(y.cpu().numpy()[rows], ref)
-    ai, wi = g.integers(-7, 8, (M, K)).astype(np.int8), g.integers(-7, 8, (N, K)).astype(np.int8)
-    y = torq.torq_mxint4_gemm(dev_u8(O.int4_to_e4m3(ai)), one(M, K), dev_u8(O.int4_to_e4m3(wi)), one(N, K), out_dtype=torch.float32)
+    asb, wsb = sc(M, K, 32), sc(N, K, 32)
+    ops = (a, s32(asb, K), w, s32(wsb, K))
+    check("mxfp4", K, lambda: torq.torq_mxfp4_gemm(*ops, out_dtype=torch.float32), grid[ac], grid[wc], asb, wsb)
+    asb, wsb = sc(M, K, 16), sc(N, K, 16)
+    opn = (a, s16(asb, K), 1.0, w, s16(wsb, K), 1.0)
+    check("nvfp4", K, lambda: torq.torq_nvfp4_gemm(*opn, out_dtype=torch.float32), grid[ac], grid[wc], asb, wsb)
+    ai, wi = g.integers(-7, 8, (M, K8)).astype(np.int8), g.integers(-7, 8, (N, K8)).astype(np.int8)
+    asb, wsb = sc(M, K8, 32), sc(N, K8, 32)
+    opi = (dev_u8(O.int4_to_e4m3(ai)), s32(asb, K8), dev_u8(O.int4_to_e4m3(wi)), s32(wsb, K8))
+    check("mxint4", K8, lambda: torq.torq_mxint4_gemm(*opi, out_dtype=torch.float32), ai.astype(np.float64), wi.astype(np.float64), asb, wsb)
     torch.cuda.synchronize()
     assert torq.torq_last_device_error() == 0
-    assert np.array_equal(y.cpu().numpy()[rows], ai[rows].astype(np.int64) @ wi.astype(np.int64).T)
 
 
 @pytest.mark.parametrize("fmt,M,d,kernel", [("mxfp4", 104, 2048, "wide"), ("mxfp4", 104, 2176, "fewtok"), ("mxfp4", 144, 2176, "wide"),
