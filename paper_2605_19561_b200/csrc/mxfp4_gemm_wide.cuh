@@ -23,8 +23,8 @@ namespace torq {
 template <int FMT = FMT_MXFP4>
 struct GemmWideCfg {
   static constexpr int BM = 128;                       // rows per CTA
-  static constexpr int BK = GemmPairCfgT<FMT>::BK;     // elements of K per stage (128 bytes per row)
-  static constexpr int CH = GemmPairCfgT<FMT>::CH;     // scale chunks per stage and 128 rows
+  static constexpr int BK = GemmPairCfgT<FMT>::BK;     // elements of K per slab (128 bytes per row)
+  static constexpr int CH = GemmPairCfgT<FMT>::CH;     // scale chunks per slab and 128 rows
   static constexpr int SF_BOXES = GemmPairCfgT<FMT>::SF_BOXES;
   static constexpr int SF_BOX_WORDS = GemmPairCfgT<FMT>::SF_BOX_WORDS;   // one or two chunks per box
   static constexpr int SF_BOX_BYTES = SF_BOX_WORDS * 4;
@@ -38,8 +38,8 @@ struct GemmWideCfg {
   __host__ __device__ static constexpr int n0(int width) { return width <= 256 ? width : width - 128; }
   // chunks of W scales a tile can touch: tiles start on multiples of `width`, i.e. 0 or 64 rows into a chunk
   __host__ __device__ static constexpr int chunks(int width) { return (width + (width % 128 ? 64 : 0) + 127) / 128; }
-  __host__ __device__ static constexpr int stage_tx(int width) { return A_BYTES + width / 2 * 128 + SF_BOXES * SF_BOX_BYTES * (1 + chunks(width)); }
-  __host__ __device__ static constexpr int slab_bytes(int width) { return (stage_tx(width) + 1023) / 1024 * 1024; }
+  __host__ __device__ static constexpr int slab_tx(int width) { return A_BYTES + width / 2 * 128 + SF_BOXES * SF_BOX_BYTES * (1 + chunks(width)); }
+  __host__ __device__ static constexpr int slab_bytes(int width) { return (slab_tx(width) + 1023) / 1024 * 1024; }
   // K slabs of 128 bytes per stage of the kernel for widths up to `range`
   __host__ __device__ static constexpr int slabs(int range) { return range <= 128 ? 2 : 1; }
   // Two slabs halve the waits and barriers per K, which bound a step of up to 128 columns (us, one slab / two: 200 x 4096, K = 14336
@@ -140,7 +140,7 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       auto load_w = [&](int s, int kt) {
         const uint32_t bar = leader_full0 + 8u * s;
         const int here = k_slabs - kt * SL < SL ? k_slabs - kt * SL : SL;
-        if (rank == 0) mbar_arrive_expect_tx(full_bar(s), 2 * here * C::stage_tx(width));
+        if (rank == 0) mbar_arrive_expect_tx(full_bar(s), 2 * here * C::slab_tx(width));
         for (int i = 0; i < here; ++i) {
           const int k = kt * SL + i;
           const uint32_t st = smem_base + s * stage_bytes + i * slab_bytes;

@@ -1,11 +1,11 @@
 // Rotate + quantize for M > 128 on CTA pairs: the same computation and epilogue as
 // rotate_quantize_kernel, but two CTAs (a cluster of 2, one per SM) share one 256 x 256 output
 // tile through tcgen05.mma cta_group::2.  Each CTA stages only its own 128 rows of X and its own
-// 128 columns of R_inter per K step (32 KiB instead of 48 KiB per 128 x 256 x 64 of work), which
-// is what the single-CTA kernel is short of: it cannot keep enough bytes in flight from L2 to
-// feed the tensor pipe.  A 256 x 256 tile's loop of loads and instructions by itself runs at 512 cycles per K step, the
-// instructions' own rate (the loads alone at 22 TB/s, 400 cycles): what a long call waits for is the power cap.  Every CTA loads only for itself; operand sharing happens inside the MMA, which
-// reads both CTAs' shared memory.
+// 128 columns of R_inter per K step: 32 KiB per 128 x 256 x 64 of work where the single-CTA kernel
+// stages 48, with which it cannot feed the tensor pipe from L2.  Here the loop of loads and
+// instructions of a 256 x 256 tile by itself runs at 512 cycles per K step, the instructions' own rate (the
+// loads alone take 400, at 22 TB/s): what a long call waits for is the power cap.  Every CTA loads only
+// for itself; operand sharing happens inside the MMA, which reads both CTAs' shared memory.
 //
 // Tiles are dealt round robin from the list MixedTiles describes: 256 x 256 tiles, and where those
 // would leave the last wave partly empty, 256 x 192 tiles in its place (N = 192 instructions, 96
@@ -89,7 +89,7 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   // tensor-memory allocation; the other warps meet behind both on a barrier that the producer only counts itself on.  A CTA whose
   // SM the kernel before leaves last sets the time here: device timestamps, 2048 x 4096, from that kernel's completion to
   // the last pair's first full stage 3.6 us, 2.3 with this set-up and the first X loads from a warp of their own (the layer
-  // with N = 6144 84.9 -> 83.9 us, at the power cap; rotation and GEMM have it).
+  // with N = 6144, where rotation and GEMM have it, 86.1 -> 85.2 us, at the power cap, loops of 0.7 s on each side in turn).
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int a = 0; a < C::NACC; ++a) { mbar_init(accf_bar(a), 1); mbar_init(acce_bar(a), 16); }

@@ -7,16 +7,17 @@
 // 1000 x 1024 11.7 / 8.4; 1000 x 256 8.0 / 3.9.
 //
 // A tile wider than 256 columns is two instructions per 16 elements of K that share the X slice, accumulators
-// side by side in tensor memory (column c of the tile is accumulator column c).  An instruction costs at least
-// 45 cycles however narrow (256 + 32 columns ran at 692 cycles per K step, 160 + 128 at 576), so the second one is
-// always 128 columns.  Each CTA of the pair stages its 128 rows of X and half of each instruction's columns of
-// R_inter: 64-column boxes of 8 KiB (16 KiB up to 128 columns, where a stage is 128 of K) and, when half of the first instruction is no multiple of 64, one narrower box
-// (its rows keep the 128-byte pitch of the swizzle) in a slot of the same size.
+// side by side in tensor memory (column c of the tile is accumulator column c).  An instruction of N columns takes the
+// larger of N / 2 and 64 + N / 4 cycles, the reading of its slices from shared memory; a second one on the same X
+// slice N / 2, but at least 45 however narrow (per 64 of K 256 + 32 columns ran at 692 cycles, 160 + 128 at 576, 256 + 128 at 770),
+// so the second one is always 128 columns.  Each CTA of the pair stages its 128 rows of X and half of each instruction's
+// columns of R_inter: 64-column boxes of 8 KiB (16 KiB up to 128 columns, where a stage is 128 of K) and, when half of the
+// first instruction is no multiple of 64, one narrower box (its rows keep the 128-byte pitch of the swizzle) in a slot of the
+// same size.
 //
-// Bounds: up to 256 columns the latency of the loads and of the hand-overs between the roles (440 cycles per 64 of K at 64
-// columns, 460 at 128, 500 at 256 with stages of 64; the same loads alone, from L2, run at 22 TB/s; an instruction takes the
-// larger of 2 cycles per column and a quarter of that plus 64 for its X slice), above the math; then the
-// epilogue, which nothing overlaps.  It is the fast form (warp-level MMAs on the accumulator fragments), bound by
+// Bounds: up to 128 columns the latency of the loads and of the hand-overs between the roles (440 cycles per 64 of K at 64
+// columns, 460 at 128 with stages of 64, where the instructions take 320 and 384; the same loads alone, from L2, run at 22
+// TB/s), above the instructions (500 at 256); then the epilogue, which nothing overlaps.  It is the fast form (warp-level MMAs on the accumulator fragments), bound by
 // those MMAs: about 860 cycles per 32 columns.  Splitting K over the pairs of a larger cluster (partial sums
 // exchanged through distributed shared memory) was measured and brought nothing: 300 x 4096 20.9 with two pairs
 // per 256 columns against 21.2.
@@ -35,12 +36,13 @@ struct RotWideCfg {
   static constexpr int SLAB = 64;                      // K elements of one 128-byte row of X
   // K per stage: two slabs up to 128 columns, where the waits and the issue of loads per step bound a step and not its math (us, one
   // slab / two: 200 tokens d = 1024 4.87 / 4.48, d = 2048 8.42 / 7.57, 300 tokens d = 4096 18.4 / 17.1; loops of the whole warp
-  // instead of one thread 5.51 and 9.10); above, three stages of twice the size lose against six (600 x 4096, 192 columns, 22.5 / 25.9)
+  // instead of one thread 5.51 and 9.10); above, three stages of twice the size lose against six (us, six / three: 600 x 4096 25.6 / 27.8,
+  // 300 x 6144 35.5 / 39.3, 400 x 8192 60.3 / 62.8, 160 columns: 1280 x 2048 14.3 / 15.3)
   __host__ __device__ static constexpr int bk(int width) { return width <= 128 ? 2 * SLAB : SLAB; }
   __host__ __device__ static constexpr int a_bytes(int width) { return BM * bk(width) * 2; }       // 32 or 16 KiB
   __host__ __device__ static constexpr int box_bytes(int width) { return 64 * bk(width) * 2; }     // 64 columns of R_inter
   static constexpr int MAX_WIDTH = 384;
-  static constexpr int MAX_STAGES = 8;
+  static constexpr int MAX_STAGES = 6;
   static constexpr int RI_BLOCK_BYTES = 32 * 64;       // R_intra[blk] as bf16 rows of 64 bytes, 16-byte pieces XOR-swizzled
   static constexpr int ESETS = 3;
   static constexpr int THREADS = 64 + 128 * ESETS;
@@ -58,11 +60,14 @@ struct RotWideCfg {
 };
 static_assert(RotWideCfg::smem_bytes(128) <= 232448 && RotWideCfg::smem_bytes(256) <= 232448 &&
               RotWideCfg::smem_bytes(384) <= 232448, "shared memory budget");
+static_assert(RotWideCfg::stages(128) <= RotWideCfg::MAX_STAGES && RotWideCfg::stages(256) <= RotWideCfg::MAX_STAGES &&
+              RotWideCfg::stages(384) <= RotWideCfg::MAX_STAGES, "barriers");
 
 // grid = 2 * rows * cols CTAs in clusters of two: pair p works row tile p % rows (256 tokens), column tile p / rows
-// (`width` features from column (p / rows) * width on).  tmX: X box [128 x 64]; tmR: R_inter box [64 x 64]; tmRt:
-// box [64 x tail_cols].  d % 128 == 0.  RANGE: 128, 256 or
-// 384, the first that is not below the width (two slabs of K per stage; one; two instructions per slice).  FMT, `tensor_scale` as in the pair kernel.
+// (`width` features from column (p / rows) * width on).  tmX: X as (64 of K, token, slab of K), box [64 x 128 x slabs of a
+// stage]; tmR: R_inter box [BK of K x 64 columns]; tmRt: box [BK x tail_cols].  d % 128 == 0.  RANGE: 128, 256 or 384, the first
+// that is not below the width (two slabs of K per stage; one; two instructions per slice).  FMT, `tensor_scale` as in the pair
+// kernel.
 template <int FMT, int RANGE>
 __global__ void __launch_bounds__(RotWideCfg::THREADS, 1)
 rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,

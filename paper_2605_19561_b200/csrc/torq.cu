@@ -478,8 +478,8 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 }
 
 // Width of the one-wave rotation's tiles, or 0 where another kernel is faster.  Times in us, fitted to the rotation
-// alone at 60 shapes (d = 128 ... 14336, M = 1 ... 4000; within 10 % but for the HBM-bound ones at d > 8192, where both
-// sides are low by as much); f = filled part of a wave:
+// alone at 60 shapes (d = 128 ... 14336, M = 1 ... 4000; within 10 % but above d = 6144, where these tiles are rated up to 3 us too
+// high, and at d > 8192, where HBM bounds both sides and both are rated low); f = filled part of a wave:
 //  * here: 1.6 + 0.022 per column (2 + 0.032 above 256 columns, 1.4 + 0.022 up to 128) for launch and epilogue, then per K step
 //    of 64 the operand bytes, 0.17 + 0.0003 per column + 0.03 f (up to 128 columns, where a stage is two of these steps, 0.145 +
 //    0.0003 per column + 0.035 f, but from d = 6272 on, where R_inter's stream sets the pace), or the math, 0.00114 per column;
@@ -502,8 +502,8 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 // 384 columns; 2048 x 4096 measured 51.6 with 480 columns, 46.8 in the pair kernel).
 static int wide_rotation_width(int fmt, int64_t M, int64_t d, int few_steps, int few_S, int max_pairs) {
   const int64_t rows = (M + 255) / 256, steps = d / 64;
-  // The line of 65 to 96 tokens, clusters of six, stays where it was, and so does that of an X below 128 KiB, which these tiles read
-  // more slowly (us, few tokens / here: d = 1024 63 tokens 5.7 / 5.8, 64 tokens 5.7 / 4.5; d = 1152 56 5.6 / 5.7, 60 5.7 / 4.7;
+  // The line of 65 to 96 tokens, clusters of six, stays where it was, and so does that of an X below 128 KiB (up to 64 tokens; with
+  // more, an X so small has a d that comes here by either figures), which these tiles read more slowly: the cause is not known (us, few tokens / here: d = 1024 63 tokens 5.7 / 5.8, 64 tokens 5.7 / 4.5; d = 1152 56 5.6 / 5.7, 60 5.7 / 4.7;
   // d = 1536 40 5.9 / 9.3, 48 6.0 / 5.6).
   const bool two_slabs = d <= 6144 && (M > 96 || (M <= 64 && M * d >= 65536));
   double best = 1e30;
@@ -752,9 +752,11 @@ torq_status torq_rotate_quantize_structured_nvfp4(const void* X, const void* R_B
 }  // extern "C"
 
 // Width of the one-wave GEMM's tiles, or 0 where another kernel is faster.  Times in us, fitted to MXFP4 with bf16 output
-// at K = 128 ... 14336, N = 256 ... 12288, M = 17 ... 8000 (within 10 %); f = filled part of a wave:
+// at K = 128 ... 14336, N = 256 ... 12288, M = 17 ... 8000 (within 10 % of the kernels with one slab); f = filled part of a wave:
 //  * here: 2 (1.8 / 1.5 up to 128 / 64 tokens) + 0.0062 per column + f for launch and epilogue, then per K step 0.24 or the
-//    math, 0.0011 per column, + 0.025 f (fitted with one slab of K per stage: up to 128 columns two take 0.15 to 0.19);
+//    math, 0.0011 per column, + 0.025 f: with one slab of K per stage.  Up to 128 columns two take 0.15 to 0.19, which the figures
+//    do not know: there they are high by up to a third (200 x 4096, K = 14336 17.3 modelled, 13.1 measured; 300 x 4096, K = 4096 7.8,
+//    6.7) and take 192 columns in one slab where 128 in two would fit the pairs too (512 x 4096, K = 14336; 700 x 3072, K = 4096);
 //  * few tokens (17 to 128, S CTAs per tile): 2.3 + 0.2 per K step of the longest split + per token 0.025 with S = 1 (the
 //    accumulator goes to Y), else 0.012 + 0.035 / S;
 //  * pair kernel: one wave 4.1 + 0.9 f + (0.285 + 0.04 f) per K step, more (the last one as narrower tiles) 5.2 + per K step
