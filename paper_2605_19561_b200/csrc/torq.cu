@@ -488,7 +488,7 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 //    144 tokens d = 2560 9.7 / 10.4, d = 4096 13.6 / 14.9; 208 d = 2560 12.6 / 10.4, d = 4096 15.0 / 15.0 (the layer with N = 6144
 //    22.7 / 23.2), d = 5120 19.5 / 20.1; 256 d = 4096 16.2 / 15.1, d = 5120 20.9 / 20.0; 128 d = 2048 8.1 / 7.6; 104 d = 2048 7.6 /
 //    7.4, d = 2176 7.8 / 8.1);
-//  * up to 192 tokens a cluster of six has at most two units per CTA, and R_inter's stream sets its time, not the longest split: 4.2 +
+//  * up to 192 tokens a cluster of six has at most two units per CTA, and R_inter's stream sets its time, not the longest split: 4.1 +
 //    0.14 per K step, at least 8.95, and 0.32 per 16 tokens above 144 (136 tokens d = 2432 9.1 / 9.8; 160 d = 2304 9.24 / 8.83, d = 2432
 //    9.6 / 9.9, d = 2560 9.9 / 10.3, MXINT4 10.1 / 11.1; 176 d = 2816 10.9 / 11.2; 184 d = 2688 10.95 / 10.8);
 //  * above 192 tokens a cluster of three has five units for its first CTA: 0.6 more (216 d = 4864 19.3 / 18.2);
@@ -496,8 +496,10 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 //    (144 d = 6912 26.9 / 25.4, 150 d = 7040 28.2 / 26.3, 208 d = 7680 33.1 / 30.0);
 //  * pair kernel: 6.8, plus per K step 0.32 for a wave and 0.2 + 0.14 f for the last, partly filled one.
 // The other formats follow the same figures, except that beside a cluster of six MXINT4, whose epilogue stores twice the bytes, counts
-// 0.2 more here, and NVFP4 0.15 from 64 columns on.  Checked with both sides measured at 506 points of 97 to 256 tokens where these
-// tiles were the modelled choice: the choice is the faster side or within 1.4 % of it.  wide_gemm_width says how the rest was.
+// 0.2 more here, and NVFP4 0.15 from 64 columns on.  Checked with both sides measured, operands not in the L2, at 506 points of 97 to
+// 256 tokens where these tiles were the modelled choice, and in 1128 layer calls (N = 1024, d, 6144): up to d = 5376 the choice is the
+// faster side or within 5 % of it, 0.2 % in the mean (layers, few tokens / here: 160 x 2560 -> 2560 0.94 of the time, 176 x 2816 -> 2816 0.97, 144 x 6912 ->
+// 6912 1.05, 208 x 4864 -> 4864 1.02).  With R_inter in the L2 these tiles gain 5 to 10 % more.  wide_gemm_width says how the rest was.
 // A layer of 2048 tokens and more fills the pair kernel's waves and stays there (one-wave tiles would be wider than
 // 384 columns; 2048 x 4096 measured 51.6 with 480 columns, 46.8 in the pair kernel).
 static int wide_rotation_width(int fmt, int64_t M, int64_t d, int few_steps, int few_S, int max_pairs) {
@@ -521,7 +523,7 @@ static int wide_rotation_width(int fmt, int64_t M, int64_t d, int few_steps, int
     else if (M <= 64) other = 4.4 + 0.2 * few_steps;
     else if (M <= 128) other = (M <= 96 ? 5.6 : 5.4) + 0.36 * few_steps;
     else if (few_S == 6 && M <= 192) {
-      const double stream = 4.2 + 0.14 * (double)steps;
+      const double stream = 4.1 + 0.14 * (double)steps;
       other = (stream > 8.95 ? stream : 8.95) + 0.02 * (double)(fewtok_ntok(M) - 144);
       best += fmt == FMT_MXINT4 ? 0.2 : (fmt == FMT_NVFP4 && width > 32 ? 0.15 : 0.0);
     } else if (d > 6144) other = (M <= 192 ? 7.6 : 10.5) + 0.42 * few_steps;
