@@ -389,8 +389,9 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
 }
 // Bounded wait on a local barrier whose arrivals may come from the peer CTA.  BEHIND_DEP: of a role that has not passed
 // griddep_wait().  Its limit does not count what is left of the kernel before, which may take any time: the clock starts behind
-// that.  (Not ahead of the wait: an issuer that passed it before its first wait made the one-wave rotations 0.5 % slower.  And not in
-// every wait: a layer of one token and d = N = 5120 on the few-token kernels, which pass it at their start, 15.69 -> 15.75 us.)
+// that.  (Not ahead of the wait: an issuer that passed it before its first wait made the one-wave rotations 0.5 % slower.  Not as one
+// more wait for the first stage ahead of the loop: 265 GEMMs of one wave and pairs 3 % slower.  And not in every wait: a layer of
+// one token and d = N = 5120 on the few-token kernels, which pass it at their start, 15.69 -> 15.75 us.)
 template <bool BEHIND_DEP = false>
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
                                                   volatile int* cta_abort, int* err_word, int site) {
