@@ -483,30 +483,26 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 //  * here: 1.6 + 0.022 per column (2 + 0.032 above 256 columns, 1.4 + 0.022 up to 128) for launch and epilogue, then per K step
 //    of 64 the operand bytes, 0.17 + 0.0003 per column + 0.03 f (up to 128 columns, where a stage is two of these steps, 0.145 +
 //    0.0003 per column + 0.035 f, but from d = 6272 on, where R_inter's stream sets the pace), or the math, 0.00114 per column;
-//  * few tokens: 3.1 / 4.4 / 5.6 / 5.4 up to 16 / 64 / 96 / 128 tokens, plus 0.22 / 0.2 / 0.36 / 0.36 per K step of the longest split;
-//    above, 6.4 at 144 tokens and 0.025 per token more, 0.5 per CTA of a cluster above four, 0.42 per K step (us, few tokens / here:
-//    144 tokens d = 2560 9.7 / 10.4, d = 4096 13.6 / 14.9; 208 d = 2560 12.6 / 10.4, d = 4096 15.0 / 15.0 (the layer with N = 6144
-//    22.7 / 23.2), d = 5120 19.5 / 20.1; 256 d = 4096 16.2 / 15.1, d = 5120 20.9 / 20.0; 128 d = 2048 8.1 / 7.6; 104 d = 2048 7.6 /
-//    7.4, d = 2176 7.8 / 8.1);
-//  * up to 192 tokens a cluster of six has at most two units per CTA, and R_inter's stream sets its time, not the longest split: 4.1 +
-//    0.14 per K step, at least 8.95, and 0.32 per 16 tokens above 144 (136 tokens d = 2432 9.1 / 9.8; 160 d = 2304 9.24 / 8.83, d = 2432
-//    9.6 / 9.9, d = 2560 9.9 / 10.3, MXINT4 10.1 / 11.1; 176 d = 2816 10.9 / 11.2; 184 d = 2688 10.95 / 10.8);
+//  * few tokens: 3.1 / 4.4 / 5.6 up to 16 / 64 / 128 tokens, plus 0.22 / 0.2 / 0.36 per K step of the longest split; above, 6.4 at
+//    144 tokens and 0.025 per token more, 0.5 per CTA of a cluster above four, 0.42 per K step (us, few tokens / here: 144
+//    tokens d = 2560 9.7 / 10.4, d = 4096 13.6 / 14.9; 208 d = 2560 12.6 / 10.4, d = 4096 15.0 / 15.0 (the layer with N = 6144
+//    22.7 / 23.2), d = 5120 19.5 / 20.1; 256 d = 4096 16.2 / 15.1, d = 5120 20.9 / 20.0; 128 d = 2048 8.1 / 7.6).  Beside clusters of six
+//    (d = 2048 ... 2816, up to 192 tokens) this is a microsecond more than they take with cold operands, and the line lies between
+//    what cold ones and an R_inter in the L2 ask for (layers with N = d, few tokens / here: 144 x 2432 cold 0.95 of the time, in the
+//    L2 1.11; 152 x 2560 0.93 and 1.09, 176 x 2560 0.97 and 1.11, 176 x 2816 0.97 and 1.06, 112 x 2176 0.95 and 1.04);
 //  * above 192 tokens a cluster of three has five units for its first CTA: 0.6 more (216 d = 4864 19.3 / 18.2);
 //  * above d = 6144, where these tiles take up to 3 us less than the figures say: 7.6 up to 192 tokens, 10.5 above, 0.42 per K step
 //    (144 d = 6912 26.9 / 25.4, 150 d = 7040 28.2 / 26.3, 208 d = 7680 33.1 / 30.0);
 //  * pair kernel: 6.8, plus per K step 0.32 for a wave and 0.2 + 0.14 f for the last, partly filled one.
-// The other formats follow the same figures, except that beside a cluster of six MXINT4, whose epilogue stores twice the bytes, counts
-// 0.2 more here, and NVFP4 0.15 from 64 columns on.  Checked with both sides measured, operands not in the L2, at 506 points of 97 to
-// 256 tokens where these tiles were the modelled choice, and in 1128 layer calls (N = 1024, d, 6144): up to d = 5376 the choice is the
-// faster side or within 5 % of it, 0.2 % in the mean (layers, few tokens / here: 160 x 2560 -> 2560 0.94 of the time, 176 x 2816 -> 2816 0.97, 144 x 6912 ->
-// 6912 1.05, 208 x 4864 -> 4864 1.02).  With R_inter in the L2 these tiles gain 5 to 10 % more.  wide_gemm_width says how the rest was.
+// The other formats follow the same figures, which were not fitted to them; wide_gemm_width says how that was checked.
 // A layer of 2048 tokens and more fills the pair kernel's waves and stays there (one-wave tiles would be wider than
 // 384 columns; 2048 x 4096 measured 51.6 with 480 columns, 46.8 in the pair kernel).
-static int wide_rotation_width(int fmt, int64_t M, int64_t d, int few_steps, int few_S, int max_pairs) {
+static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int few_S, int max_pairs) {
   const int64_t rows = (M + 255) / 256, steps = d / 64;
   // The line of 65 to 96 tokens, clusters of six, stays where it was, and so does that of an X below 128 KiB (up to 64 tokens; with
-  // more, an X so small has a d that comes here by either figures), which these tiles read more slowly: the cause is not known (us, few tokens / here: d = 1024 63 tokens 5.7 / 5.8, 64 tokens 5.7 / 4.5; d = 1152 56 5.6 / 5.7, 60 5.7 / 4.7;
-  // d = 1536 40 5.9 / 9.3, 48 6.0 / 5.6).
+  // more, an X so small has a d that comes here by either figures), which these tiles read more slowly for a reason not found (us, few
+  // tokens / here: d = 1024 63 tokens 5.7 / 5.8, 64 tokens 5.7 / 4.5; d = 1152 56 5.6 / 5.7, 60 5.7 / 4.7; d = 1536 40 5.9 / 9.3, 48
+  // 6.0 / 5.6).
   const bool two_slabs = d <= 6144 && (M > 96 || (M <= 64 && M * d >= 65536));
   double best = 1e30;
   int width = 0;
@@ -521,12 +517,8 @@ static int wide_rotation_width(int fmt, int64_t M, int64_t d, int few_steps, int
   if (M <= kRotFewMaxTokens) {
     if (M <= 16) other = 3.1 + 0.22 * few_steps;
     else if (M <= 64) other = 4.4 + 0.2 * few_steps;
-    else if (M <= 128) other = (M <= 96 ? 5.6 : 5.4) + 0.36 * few_steps;
-    else if (few_S == 6 && M <= 192) {
-      const double stream = 4.1 + 0.14 * (double)steps;
-      other = (stream > 8.95 ? stream : 8.95) + 0.02 * (double)(fewtok_ntok(M) - 144);
-      best += fmt == FMT_MXINT4 ? 0.2 : (fmt == FMT_NVFP4 && width > 32 ? 0.15 : 0.0);
-    } else if (d > 6144) other = (M <= 192 ? 7.6 : 10.5) + 0.42 * few_steps;
+    else if (M <= 128) other = 5.6 + 0.36 * few_steps;
+    else if (d > 6144) other = (M <= 192 ? 7.6 : 10.5) + 0.42 * few_steps;
     else other = 6.4 + 0.025 * (double)(M - 144) + (few_S > 4 ? 0.5 * (few_S - 4) : (few_S == 3 && M > 192 ? 0.6 : 0.0)) + 0.42 * few_steps;
   } else {
     const int64_t tiles = rows * ((d + 255) / 256);
@@ -624,7 +616,7 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
       few_S = fewtok_rotation(M, d, st).cluster;
       few_steps = (int)((d / 64 + few_S - 1) / few_S);
     }
-    const int width = wide_rotation_width(fmt, M, d, few_steps, few_S, st->rot_pairs);
+    const int width = wide_rotation_width(M, d, few_steps, few_S, st->rot_pairs);
     if (width > 0) return rotate_wide(st, fmt, X, R_inter, R_intra, M, d, codes, scales, tensor_scale, width, s);
   }
   if (M <= kRotFewMaxTokens && d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT)

@@ -219,12 +219,8 @@ def test_gemm_with_two_slabs_per_stage(M, N, K, K8):
     assert torq.torq_last_device_error() == 0
 
 
-@pytest.mark.parametrize("fmt,M,d,kernel", [("mxfp4", 104, 2048, "wide"), ("mxfp4", 104, 2176, "fewtok"), ("mxfp4", 144, 2176, "wide"),
-                                            ("mxfp4", 160, 2304, "wide"), ("mxfp4", 136, 2432, "fewtok"), ("mxfp4", 192, 2432, "wide"),
-                                            ("mxfp4", 160, 2560, "fewtok"), ("mxfp4", 168, 2816, "fewtok"), ("mxfp4", 208, 2816, "wide"),
-                                            ("nvfp4", 152, 2560, "fewtok"), ("mxint4", 176, 2432, "fewtok"), ("mxint4", 144, 2176, "wide"),
-                                            ("mxint4", 192, 2688, "fewtok"), ("mxint4", 192, 3072, "wide"), ("mxfp4", 192, 4864, "fewtok"), ("nvfp4", 184, 2816, "fewtok"),
-                                            ("mxfp4", 176, 2560, "fewtok"), ("mxfp4", 192, 2816, "fewtok"), ("mxfp4", 192, 2560, "wide"),
+@pytest.mark.parametrize("fmt,M,d,kernel", [("mxfp4", 104, 2048, "wide"), ("mxfp4", 112, 2304, "fewtok"), ("mxfp4", 208, 2816, "wide"),
+                                            ("mxint4", 192, 3072, "wide"), ("mxfp4", 192, 4096, "fewtok"), ("mxfp4", 192, 4864, "fewtok"),
                                             ("mxfp4", 216, 4864, "wide"), ("mxfp4", 144, 6912, "wide"), ("nvfp4", 193, 7296, "wide"),
                                             ("mxfp4", 150, 7168, "fewtok"), ("mxint4", 256, 9344, "wide")])
 def test_rotation_kernel_of_97_to_256_tokens(fmt, M, d, kernel):
