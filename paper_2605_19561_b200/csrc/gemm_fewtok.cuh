@@ -9,9 +9,10 @@
 // A layer has only N / 128 such tiles (40 at N = 5120), so K is split as well: a CLUSTER of S CTAs
 // shares one tile, CTA r contracts k range r; the fp32 partial tiles stay on the SMs and are added in rank order (fixed).
 // As in the few-token rotation they reach the adding CTA in one of two ways:
-//  * PUSH (up to 16 tokens): tokens are dealt in pieces of four, piece c belongs to CTA c % S, and every CTA stores its
-//    partial sums of a piece straight from registers into that CTA's shared memory (st.async, 16 bytes per lane =
-//    four tokens of one feature).  K = N = 5120, M = 1: 4.0 us (4.7 before, pulling); 64 tokens: 7.2 against 6.1.
+//  * PUSH (up to 32 tokens, NVFP4 24): the sums are dealt over all CTAs and warps of the cluster in pieces of 32 features x 4 tokens, and
+//    every CTA stores its partials of a piece straight from registers into the owner's shared memory (st.async, 16 bytes per lane = four
+//    tokens of one feature, counted on a barrier of the owning warp), into room of their own.  K = N = 5120, us: pulled 1 token 4.7,
+//    24 tokens 5.6; pushed to one owner per four tokens, into its stages, 4.4 and 16 tokens 4.95; so 4.4, 4.7 and 24 tokens 5.25.
 //  * pull (more tokens): each CTA writes its partial [token][feature] into its own shared memory, a cluster barrier
 //    publishes them, and CTA r adds, for the tokens m = r (mod S), the S partials read with 16-byte ld.shared::cluster.
 // With S = 1 (an ordinary launch without clusters) the accumulator goes to Y directly.
@@ -36,9 +37,8 @@ struct GemmFewCfg {
   static constexpr int CH = FMT == FMT_NVFP4 ? 4 : (FMT == FMT_MXINT4 ? 1 : 2);   // scale chunks per stage and 128 rows
   static constexpr int SF_BYTES = CH * 512;
   static constexpr int STAGES = 4;
-  // the same for every token count: three stages at 128 tokens would let two CTAs share an SM (clusters of 5
-  // instead of 3), which measured 4 - 10 % slower than four stages and one CTA per SM
-  __host__ __device__ static constexpr int stages(int) { return STAGES; }
+  // (the same for every token count: three stages at 128 tokens would let two CTAs share an SM, clusters of 5
+  // instead of 3, which measured 4 - 10 % slower than four stages and one CTA per SM)
   static constexpr int BAR_BYTES = 256;
   static constexpr int THREADS = 192;
   static constexpr int MAX_CLUSTER = 8;
@@ -46,13 +46,17 @@ struct GemmFewCfg {
   __host__ __device__ static constexpr int stage_bytes(int ntok) {
     return (A_BYTES + ntok * 128 + 2 * SF_BYTES + 1023) / 1024 * 1024;
   }
-  __host__ __device__ static constexpr int smem_bytes(int ntok) { return stages(ntok) * stage_bytes(ntok) + BAR_BYTES + 1024; }
-  __host__ __device__ static constexpr int ctas_per_sm(int ntok) { return smem_bytes(ntok) <= 113 * 1024 ? 2 : 1; }
+  // partial sums of the units that one CTA owns, from all CTAs, for any cluster size
+  static constexpr int PART_BYTES = 32 * 16;           // of a unit from one CTA: [feature of the quarter][4 tokens]
+  static constexpr int MAX_PUSH_TOK = 32;
+  __host__ __device__ static constexpr int push_bytes(int M) { return ((M + 3) / 4 * 4 + MAX_CLUSTER - 1) * PART_BYTES; }
+  __host__ __device__ static constexpr int pull_smem_bytes(int M) { return STAGES * stage_bytes((M + 15) / 16 * 16) + BAR_BYTES + 1024; }
+  // pushed where the room for what arrives leaves two CTAs per SM (NVFP4: up to 24 tokens)
+  __host__ __device__ static constexpr bool push(int M) { return M <= MAX_PUSH_TOK && pull_smem_bytes(M) + push_bytes(M) <= 113 * 1024; }
+  __host__ __device__ static constexpr int smem_bytes(int M) { return pull_smem_bytes(M) + (push(M) ? push_bytes(M) : 0); }
+  __host__ __device__ static constexpr int ctas_per_sm(int M) { return smem_bytes(M) <= 113 * 1024 ? 2 : 1; }
   __host__ __device__ static constexpr int max_smem_bytes() { return smem_bytes(MAX_TOK); }
-  static constexpr int PIECE_BYTES = BF * 16;          // partial sums of four tokens from one CTA: [feature][4 tokens]
-  static constexpr int MAX_PUSH_TOK = 16;
-  // what lies in the stages after the mainloop: the pushed partials of up to four pieces, or the partial tile
-  static_assert(4 * MAX_CLUSTER * PIECE_BYTES <= STAGES * A_BYTES && BF * 4 <= STAGES * 128, "reduction buffers");
+  static_assert(BF * 4 <= STAGES * 128, "the pulled partial tile lies in the stages after the mainloop");
   __host__ __device__ static constexpr uint32_t tmem_cols(int ntok) {
     return ntok + 8 * CH <= 32 ? 32u : (ntok + 8 * CH <= 64 ? 64u : (ntok + 8 * CH <= 128 ? 128u : 256u));
   }
@@ -75,14 +79,14 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
   const int stage_bytes = C::stage_bytes(ntok);
   const int b_bytes = ntok * 128;
-  const int nst = C::stages(ntok);
+  constexpr int nst = C::STAGES;
   const uint32_t bar_off = nst * stage_bytes;
   const uint32_t bar_base = smem_base + bar_off;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
   auto empty_bar = [&](int s) { return bar_base + 8u * (C::STAGES + s); };
   const uint32_t accf_bar = bar_base + 8u * (2 * C::STAGES);
-  const uint32_t ready_bar = accf_bar + 8;               // PUSH: the owners' stages are free to be written
-  const uint32_t recv_bar = accf_bar + 16;               // PUSH: all partials of this CTA's pieces are here
+  auto recv_bar = [&](int w) { return accf_bar + 8u + 8u * w; };   // PUSH: all partials of the units of epilogue warp w are here
+  const uint32_t recv_base = bar_base + C::BAR_BYTES;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + bar_off + 192);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(smem_gen + bar_off + 200);
 
@@ -92,8 +96,9 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   const int kb4 = K / (C::BK / CH);                      // scale chunks per row
   const int kt0 = (int)((long long)k_tiles * rank / S), kt1 = (int)((long long)k_tiles * (rank + 1) / S);
   const uint32_t tmem_cols = C::tmem_cols(ntok);
-  const int pieces = (M + 3) / 4;                        // of four tokens; piece c belongs to CTA c % S
-  const int owners = pieces < S ? pieces : S;
+  // PUSH: unit u = q + 4 c is quarter q of the tile's features and tokens 4 c .. 4 c + 3; CTA u % S owns it, its epilogue warp
+  // u / S % 4 adds and stores it
+  const int units = 4 * ((M + 3) / 4);
 
   // The weights and their scales are constants of the layer, never the output of the kernel that runs
   // just before this one: the thread that initialises the barriers sends their loads for the first
@@ -104,7 +109,8 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   if (threadIdx.x == 0) {
     for (int s = 0; s < nst; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     mbar_init(accf_bar, 1);
-    if constexpr (PUSH) { mbar_init(ready_bar, (uint32_t)owners); mbar_init(recv_bar, 1); }
+    if constexpr (PUSH)
+      for (int w = 0; w < 4; ++w) mbar_init(recv_bar(w), 1);
     *cta_abort = 0;
     fence_mbar_init();
     fence_proxy_async_smem();                            // the copy engine sees the initialised barriers
@@ -117,7 +123,9 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
                    512u * (uint32_t)min(CH, kb4 - CH * kt), full_bar(it));
     }
     tma_prefetch_desc(&tmA);
-    if (PUSH && S > 1 && rank < owners) mbar_arrive_expect_tx(recv_bar, (uint32_t)((pieces - rank + S - 1) / S * S * C::PIECE_BYTES));
+    if (PUSH && S > 1)
+      for (int w = 0; w < 4 && rank + S * w < units; ++w)
+        mbar_arrive_expect_tx(recv_bar(w), (uint32_t)((units - rank - S * w + 4 * S - 1) / (4 * S) * S * C::PART_BYTES));
   }
   if (warp == 1) { tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), tmem_cols); tmem_relinquish(); }
   tc_fence_before_sync();
@@ -127,12 +135,22 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   const uint32_t tmem_base = *tmem_slot;
   griddep_launch_dependents();
   griddep_wait();
+  // The activations of the first stages go out from four warps at once: one warp needs 0.2 us from one stage to the next.
+#pragma unroll
+  for (int it = 0; it < 4; ++it)
+    if (warp == 2 + it && it < pre && elect_one()) {
+      const uint32_t st = smem_base + it * stage_bytes;
+      tma_load_2d(st + C::A_BYTES, &tmA, (kt0 + it) * 128, 0, full_bar(it));
+      bulk_load_1d(st + C::A_BYTES + b_bytes + C::SF_BYTES, As + (size_t)(CH * (kt0 + it)) * 512,
+                   512u * (uint32_t)min(CH, kb4 - CH * (kt0 + it)), full_bar(it));
+    }
+  __syncwarp();
 
   bool acc_ok = false;
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     bool ok = true;
-    for (int kt = kt0, it = 0; kt < kt1 && ok; ++kt, ++it) {
+    for (int kt = kt0 + pre, it = pre; kt < kt1 && ok; ++kt, ++it) {
       const int s = it % nst;
       if (!mbar_wait_warp(empty_bar(s), ((it / nst) & 1) ^ 1, cta_abort, err_word, SITE_PRODUCER_EMPTY)) {
         ok = false; break;
@@ -140,12 +158,9 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
       const uint32_t st = smem_base + s * stage_bytes;
       const uint32_t sf_bytes = 512u * (uint32_t)min(CH, kb4 - CH * kt);
       if (elect_one()) {
-        const bool w_issued = it < pre;                  // W side of this stage went out before the wait above
-        if (!w_issued) {
-          mbar_arrive_expect_tx(full_bar(s), stage_tx(kt));
-          tma_load_2d(st, &tmW, kt * 128, nt * C::BF, full_bar(s));
-          bulk_load_1d(st + C::A_BYTES + b_bytes, Ws + ((size_t)nt * kb4 + CH * kt) * 512, sf_bytes, full_bar(s));
-        }
+        mbar_arrive_expect_tx(full_bar(s), stage_tx(kt));
+        tma_load_2d(st, &tmW, kt * 128, nt * C::BF, full_bar(s));
+        bulk_load_1d(st + C::A_BYTES + b_bytes, Ws + ((size_t)nt * kb4 + CH * kt) * 512, sf_bytes, full_bar(s));
         tma_load_2d(st + C::A_BYTES, &tmA, kt * 128, 0, full_bar(s));
         bulk_load_1d(st + C::A_BYTES + b_bytes + C::SF_BYTES, As + (size_t)(CH * kt) * 512, sf_bytes, full_bar(s));
       }
@@ -230,42 +245,47 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
         }
       }
     } else if constexpr (PUSH) {
-      // Lane l of warp q has feature 32 q + l of the tile: one 16-byte load per partial gives its four tokens.
-      const int64_t n = (int64_t)nt * C::BF + feature;
+      const int w = q;
+      // where this warp's partials go: quarter q, tokens 4 c ... (worked out before they are needed: a division takes as long as a store)
+      uint32_t dst[C::MAX_PUSH_TOK / 4], dst_bar[C::MAX_PUSH_TOK / 4];
+#pragma unroll
+      for (int c = 0; c < C::MAX_PUSH_TOK / 4; ++c) {
+        const int u = q + 4 * c, ui = u / S, owner = u - ui * S;
+        dst[c] = map_to_cta(recv_base + (uint32_t)((ui * S + rank) * C::PART_BYTES + lane * 16), (uint32_t)owner);
+        dst_bar[c] = map_to_cta(recv_bar(ui & 3), (uint32_t)owner);
+      }
+      cluster_wait();
 #pragma unroll 1
-      for (int pass = 0; pass < 2; ++pass) {
+      for (int pass = rank + S * w < units ? 0 : 1; pass < 2; ++pass) {
         const bool live = pass == 1;
         if (live) {
           acc_ok = mbar_wait(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
-          // every load into the stages has landed and every instruction that read them has completed
           acc_ok = __all_sync(0xFFFFFFFFu, acc_ok);
-          cluster_wait();
           if (!acc_ok) break;
-          if (rank < owners && warp == 2 && lane < S) mbar_arrive_cluster(map_to_cta(ready_bar, (uint32_t)lane));
-          bool ok = mbar_wait_cluster(ready_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
-          if (!__all_sync(0xFFFFFFFFu, ok)) break;
           tc_fence_after_sync();
-          uint32_t v[16];
-          tmem_ld_32x32_x16(tacc, v);
+          uint32_t v[C::MAX_PUSH_TOK];
+          tmem_ld_32x32_x16(tacc, *reinterpret_cast<uint32_t(*)[16]>(v));
+          if (ntok > 16) tmem_ld_32x32_x16(tacc + 16, *reinterpret_cast<uint32_t(*)[16]>(v + 16));
           tmem_ld_wait();
 #pragma unroll
-          for (int c = 0; c < 4; ++c)
-            if (c < pieces)
-              st_async_v4(map_to_cta(smem_base, (uint32_t)(c % S)) + (uint32_t)(((c / S) * S + rank) * C::PIECE_BYTES + feature * 16),
-                          v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3], map_to_cta(recv_bar, (uint32_t)(c % S)));
-          if (rank >= owners) break;                     // nothing to receive
-          ok = mbar_wait_cluster(recv_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
+          for (int c = 0; c < C::MAX_PUSH_TOK / 4; ++c)
+            if (4 * c < M) st_async_v4(dst[c], v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3], dst_bar[c]);
+          if (rank + S * w >= units) break;              // nothing to receive
+          const bool ok = mbar_wait_cluster(recv_bar(w), 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
           if (!__all_sync(0xFFFFFFFFu, ok)) break;
         }
-        for (int ci = 0; rank + ci * S < pieces; ++ci) {
-          const int m0 = 4 * (rank + ci * S);
+#pragma unroll 1
+        for (int u = rank + S * w, ui = w; u < units; u += 4 * S, ui += 4) {
+          // lane l has feature l of the quarter: one 16-byte load per partial gives its four tokens
+          const int m0 = u & ~3;
+          const int64_t n = (int64_t)nt * C::BF + (u & 3) * 32 + lane;
           float4 part[C::MAX_CLUSTER];
-          const uint32_t src = smem_base + (uint32_t)(ci * S * C::PIECE_BYTES + feature * 16);
 #pragma unroll
           for (int s = 0; s < C::MAX_CLUSTER; ++s)
             if (s < S)
               asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                           : "=f"(part[s].x), "=f"(part[s].y), "=f"(part[s].z), "=f"(part[s].w) : "r"(src + (uint32_t)(s * C::PIECE_BYTES)));
+                           : "=f"(part[s].x), "=f"(part[s].y), "=f"(part[s].z), "=f"(part[s].w)
+                           : "r"(recv_base + (uint32_t)((ui * S + s) * C::PART_BYTES + lane * 16)));
           float y[4] = {0.f, 0.f, 0.f, 0.f};             // rank order: the result does not depend on timing
 #pragma unroll
           for (int s = 0; s < C::MAX_CLUSTER; ++s)

@@ -834,13 +834,13 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
   // persistent pair kernels do better, half empty as their rows are (us, few-token against pairs: 100 tokens K = 4096,
   // N = 20480 20.4 / 12.9, N = 28672 21.4 / 16.3, N = 14336 10.9 / 11.1; 64 tokens, two CTAs per SM: K = 2048, N = 40960
   // 15.3 / 12.9, K = 4096, N = 28672 14.4 / 16.0; 40 tokens K = 5120, N = 51200 29.7 / 30.1).
-  const bool many_waves = ntok > 48 && (int64_t)tiles > (int64_t)FC::ctas_per_sm(ntok) * st->sm_count;
+  const bool many_waves = M > 48 && (int64_t)tiles > (int64_t)FC::ctas_per_sm((int)M) * st->sm_count;
   if (ntok > 0 && !many_waves) {
     // Few tokens: 128 output features x all tokens per CTA, K split over a cluster, reduced through
     // distributed shared memory.
     const int64_t steps = (K + FC::BK - 1) / FC::BK;
-    const int S = fewtok_gemm_cluster(ntok, tiles, steps, FC::ctas_per_sm(ntok), st);
-    const int width = M > FC::MAX_PUSH_TOK ? wide_gemm_width(M, N, steps, S, st->gemm_pairs) : 0;
+    const int S = fewtok_gemm_cluster(ntok, tiles, steps, FC::ctas_per_sm((int)M), st);
+    const int width = M > 16 ? wide_gemm_width(M, N, steps, S, st->gemm_pairs) : 0;
     if (width > 0) return gemm_wide<FMT>(st, Aq, As, Wq, Ws, M, N, K, Y, y_dtype, alpha, width, s);
     if (!encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, 128, 128) ||
         !encode_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Aq, (uint64_t)M, krow, (uint32_t)ntok, 128))
@@ -848,9 +848,9 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
     // up to 16 tokens: partials pushed; up to 64: one set of epilogue warps, two CTAs per SM; more: two sets.  65 to 80 tokens in
     // MXINT4 fit twice on an SM as well, and share it only where that gives them more K splits (us, shared / alone, 72 tokens:
     // N = 768, K = 3072 4.9 / 4.4, N = 1536 6.0 / 5.1, S = 8 either way; N = 6144, K = 4096, S = 4 and 1: 9.1 / 9.9).
-    const bool small = FC::ctas_per_sm(ntok) >= 2 && (ntok <= 64 || S > fewtok_gemm_cluster(ntok, tiles, steps, 1, st));
-    launch_tc(ntok <= FC::MAX_PUSH_TOK ? gemm_fewtok_kernel<FMT, 1, true> : (small ? gemm_fewtok_kernel<FMT, 1> : gemm_fewtok_kernel<FMT, 2>),
-              S, tiles * S, small ? 192 : 320, FC::smem_bytes(ntok), s, tmB, tmA, static_cast<const uint8_t*>(As),
+    const bool small = FC::ctas_per_sm((int)M) >= 2 && (ntok <= 64 || S > fewtok_gemm_cluster(ntok, tiles, steps, 1, st));
+    launch_tc(FC::push((int)M) ? gemm_fewtok_kernel<FMT, 1, true> : (small ? gemm_fewtok_kernel<FMT, 1> : gemm_fewtok_kernel<FMT, 2>),
+              S, tiles * S, small ? 192 : 320, FC::smem_bytes((int)M), s, tmB, tmA, static_cast<const uint8_t*>(As),
               static_cast<const uint8_t*>(Ws), Y, y_dtype == TORQ_BF16 ? 1 : 0, (int)M, (int)N, (int)K, ntok, S, alpha, st->err_word);
     return launch_status();
   }
