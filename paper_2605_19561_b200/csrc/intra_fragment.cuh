@@ -110,4 +110,66 @@ __device__ __forceinline__ void intra_quantize_frag16(const uint32_t (&y)[16], b
   }
 }
 
+// Few tokens, ONE FEATURE OF A 32-BLOCK PER LANE, four tokens in registers.
+// z[t] = sum_k y[k][t] R[k][lane], fp32, k in index order.  y: shared memory [32 features][4 tokens] fp32, read by broadcast;
+// r[i]: R_intra[2 i][lane] (low half) and R_intra[2 i + 1][lane], bf16.
+__device__ __forceinline__ void intra_rotate_lane4(uint32_t y_saddr, const uint32_t (&r)[16], float (&z)[4]) {
+#pragma unroll
+  for (int t = 0; t < 4; ++t) z[t] = 0.f;
+#pragma unroll
+  for (int k = 0; k < 32; ++k) {
+    float4 y;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w) : "r"(y_saddr + 16u * k));
+    const float w = __uint_as_float((k & 1) ? (r[k >> 1] & 0xFFFF0000u) : (r[k >> 1] << 16));
+    z[0] = fmaf(y.x, w, z[0]); z[1] = fmaf(y.y, w, z[1]); z[2] = fmaf(y.z, w, z[2]); z[3] = fmaf(y.w, w, z[3]);
+  }
+}
+// Quantizes the 32 features x 4 tokens and stores codes and scale bytes of tokens row0 .. row0 + 3 below M (the scale bytes of the
+// others: zero; M = 0: nothing at all).  The arithmetic is that of the row forms above, value by value.
+template <int FMT>
+__device__ __forceinline__ void quantize_lane4(const float (&z)[4], int lane, int row0, int M, int blk, int d, int kb4, const NvScale& nvs,
+                                               uint8_t* __restrict__ codes, uint8_t* __restrict__ scales) {
+  float a[4];
+  uint32_t sb = 0;                                       // of token row0 + lane % 4 (NVFP4: and this lane's half of the 32 features)
+  float f[4];                                            // multiplier of the elements
+#pragma unroll
+  for (int t = 0; t < 4; ++t) a[t] = fmaxf(0.f, fabsf(z[t]));       // a NaN does not count
+  if constexpr (FMT == FMT_NVFP4) {
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+      for (int t = 0; t < 4; ++t) a[t] = fmaxf(a[t], __shfl_xor_sync(0xFFFFFFFFu, a[t], o));
+    const int t = lane & 3;                              // one division per lane
+    float r;
+    nv_block_scale(t == 0 ? a[0] : (t == 1 ? a[1] : (t == 2 ? a[2] : a[3])), nvs, sb, r);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) f[t] = __shfl_sync(0xFFFFFFFFu, r, (lane & 16) + t);
+  } else {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      uint32_t b;
+      block_scale(__uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(a[t]))), b, f[t]);
+      if (lane == t) sb = b;
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const int row = row0 + t;
+    if constexpr (FMT == FMT_MXINT4) {
+      const uint32_t w = pack4_e4m3(int4_round(z[t] * f[t]), 0.f, 0.f, 0.f);
+      if (row < M) codes[(int64_t)row * d + blk * 32 + lane] = (uint8_t)w;
+    } else {
+      const float v = __fmul_rn(z[t], f[t]), v1 = __shfl_down_sync(0xFFFFFFFFu, v, 1);
+      const uint32_t w = pack8_e2m1(v, v1, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f);
+      if (row < M && !(lane & 1)) codes[(int64_t)row * (d / 2) + blk * 16 + (lane >> 1)] = (uint8_t)w;
+    }
+  }
+  if (M > 0 && (lane & 15) < 4 && (FMT == FMT_NVFP4 || lane < 4)) {
+    const int row = row0 + (lane & 3);
+    const int kb = FMT == FMT_NVFP4 ? 2 * blk + (lane >> 4) : blk;
+    scales[scale_offset(row, kb, kb4)] = row < M ? (uint8_t)sb : (uint8_t)0;
+  }
+}
+
 }  // namespace torq

@@ -8,32 +8,35 @@
 //   B = X tile [tokens x 64 (i)], K-major
 // A layer has only d / 128 feature tiles (40 at d = 5120), too few CTAs to pull R_inter at HBM rate,
 // so the contraction is also split: a CLUSTER of S CTAs shares one feature tile, CTA r of the cluster
-// contracts k range r.  The fp32 partial tiles never leave the SMs: token group g (8 or 16 tokens) belongs to CTA g % S
-// (its owner), which adds the S partials in rank order (fixed order, so the result does not depend on timing), applies
-// the intra-block rotation on the warp-level tensor cores (y split into three bf16 terms, fp32 accumulation) and
-// quantizes (Eq. 1).  The partials reach the owner in one of two ways:
-//  * PUSH (up to 16 tokens, one group): every CTA stores its partial straight from registers into the owner's shared
-//    memory (st.async, 16 bytes per lane, counted on a barrier of the owner).  They go where the owner's stages
-//    were, so the owner first says, on a barrier of each CTA, that its own mainloop has left them.  No
-//    cluster-wide barrier stands on the path, nor at the end: the owner has waited for all that it receives, and the
-//    other CTAs leave right after their stores, which lets the CTAs of the next kernel in.  Bound by the one owner's
-//    chain of latencies (d = 5120, M = 1: stores 0.5 us, unit 1 us where pulling took 0.8 + 1.8 + 0.7 us for barrier, unit
-//    and second barrier; rotation 12.1 -> 10.9 us).  The stores arrive at about 11 B per cycle: with 64 tokens
-//    the same way took 15.3 us, pulling 13.7.
-//  * pull (more tokens): every CTA writes its partial [token][feature] into its own shared memory, a cluster barrier
-//    publishes them, and the owner reads them with 16-byte ld.shared::cluster.  A second barrier, at which a warp arrives
+// contracts k range r.  The fp32 partial tiles never leave the SMs: every output has one CTA of the cluster that owns it, adds the S
+// partials in rank order (fixed order, so the result does not depend on timing), rotates inside the block and quantizes (Eq. 1).
+// The partials reach the owner in one of two ways:
+//  * PUSH (up to 32 tokens): the pieces of work are small, 32 features x 4 tokens, and dealt over all CTAs and warps of the cluster, so that
+//    nearly every warp has one and no CTA takes in more than its share (what arrives at one SM comes at about 9 B per cycle).  A CTA
+//    stores its partials straight from registers into the owners' shared memory (st.async, 16 bytes per lane = four tokens of one
+//    feature, counted on a barrier of the owning warp), into room of their own: nobody has to say first that the stages there are free, and
+//    no cluster-wide barrier stands on the path.  The owning warp keeps one feature per lane: the intra rotation is 32 x 4 FMAs per lane
+//    on R_intra's column in registers, y read by broadcast.  The other CTAs leave right after their stores, which lets the CTAs of the next
+//    kernel in.  Against one owner for a tile (40 KiB to take in at 16 tokens, 80 loads per lane to add them, warp-level MMAs), us:
+//    rotation of 16 tokens, d = 4096 9.6 -> 8.8, 24 tokens NVFP4 (pulled before) 10.3 -> 9.4.
+//  * pull (more tokens): token group g (16 tokens) belongs to CTA g % S.  Every CTA writes its partial [token][feature] into its own shared
+//    memory, a cluster barrier publishes them, and the owner reads them with 16-byte ld.shared::cluster and rotates on the warp-level
+//    tensor cores (y split into three bf16 terms, fp32 accumulation).  A second barrier, at which a warp arrives
 //    as soon as its last such load is back and for which it waits only before it exits, keeps the partials in place
 //    (one full barrier at the end: d = 5120, M = 64 14.0 -> 13.7 us, GEMM 6.7 -> 6.1).  CTAs without a unit then leave earlier
 //    than the others; where that harms (`together`, see the launch) the second barrier is a full one at the end after all.
-// With S = 1 (an ordinary launch without clusters) a warp writes its features into its own shared memory and goes on.
+//    The epilogue warps of lane quarter q of every CTA own 32-block q of the tile (its R_intra block is fetched into
+//    shared memory when the kernel starts, long before it is needed: a first touch of that array from a
+//    cold TLB costs microseconds).
+// With S = 1 (an ordinary launch without clusters) a warp goes on with its own features.
 //
-// Units: the epilogue warps of lane quarter q of every CTA own 32-block q of the tile (its R_intra block is fetched into
-// shared memory when the kernel starts, long before it is needed: a first touch of that array from a
-// cold TLB costs microseconds).
+// What the kernel waits for at its start is X (the kernel before writes it): the stages are full of R_inter by then and HBM would idle.  So
+// the L2 is asked ahead of that wait for X, and for some R_inter beyond the stages (kAheadTiles): us, layer d = N = 5120, 1 token
+// 14.8 -> 14.3, d = 4096, N = 6144, 200 tokens 22.4 -> 21.7.
 //
 // Roles per CTA: warp 0 TMA producer, warp 1 MMA issuer, warps 2..5 epilogue / reduction.
-// Shared memory: 4 stages of (16 KiB of R_inter + tokens x 128 B of X); after the mainloop the same
-// memory holds the partials.  Up to 64 tokens that is small enough (<= 107 KiB) for two CTAs per SM: the
+// Shared memory: 4 stages (5 up to 16 tokens) of (16 KiB of R_inter + tokens x 128 B of X); pulled partials lie in
+// the same memory after the mainloop, pushed ones behind it.  Up to 64 tokens that is small enough (<= 107 KiB) for two CTAs per SM: the
 // grid may exceed the SM count, which keeps more loads in flight; above, one CTA fills an SM, or
 // up to 128 tokens two of them with three stages (fewtok_rotation).
 #pragma once
@@ -48,30 +51,31 @@ struct RotFewCfg {
   static constexpr int BK = 64;
   static constexpr int A_BYTES = BK * BF * 2;          // 16 KiB: two boxes of 64 (k) x 64 (j)
   static constexpr int A_BOX_BYTES = 64 * 64 * 2;
-  static constexpr int STAGES = 4;
+  static constexpr int STAGES = 4, PUSH_STAGES = 5, MAX_STAGES = 5;
   // With three stages two CTAs of 65 to 128 tokens share an SM: for long K ranges, where one CTA per SM leaves SMs without
   // a CTA and too few loads in flight (the rule stands where the kernel is launched).
   static constexpr int SHARED_STAGES = 3, MAX_SHARED_TOK = 128;
   static constexpr int MAX_TOK = 256;                  // N of the instruction: a multiple of 16
-  static constexpr int MAX_PUSH_TOK = 16;              // one token group
-  static constexpr int PART_BYTES = BF * 16 * 4;       // pushed partial of the group from one CTA: [4][feature][4 tokens]
+  static constexpr int MAX_PUSH_TOK = 32;
+  static constexpr int PART_BYTES = 32 * 16;           // pushed partial of a unit from one CTA: [feature of the block][4 tokens]
   static constexpr int Y_BYTES = 16 * 33 * 4;          // pull, per epilogue warp: 16 tokens x 32 features, row stride 33
   static constexpr int RI_BYTES = 32 * 80;             // per epilogue warp: R_intra[block] as bf16 rows of 80 bytes
   static constexpr int BAR_BYTES = 256;
   static constexpr int THREADS = 192;
   static constexpr int MAX_CLUSTER = 8;
   __host__ __device__ static constexpr int stage_bytes(int ntok) { return A_BYTES + ntok * BK * 2; }
+  // partials of the units that one CTA owns, from all CTAs, for any cluster size; then the y tile of each warp
+  __host__ __device__ static constexpr int push_bytes(int ntok) { return (ntok + MAX_CLUSTER - 1) * PART_BYTES + 4 * PART_BYTES; }
   __host__ __device__ static constexpr int smem_bytes(int ntok, int stages = STAGES) {
-    return stages * stage_bytes(ntok) + BAR_BYTES + 4 * RI_BYTES + 1024;
+    return stages * stage_bytes(ntok) + BAR_BYTES + (ntok <= MAX_PUSH_TOK ? push_bytes(ntok) : 4 * RI_BYTES) + 1024;
   }
   __host__ __device__ static constexpr int ctas_per_sm(int ntok, int stages = STAGES) {
     return smem_bytes(ntok, stages) <= 113 * 1024 ? 2 : 1;
   }
   __host__ __device__ static constexpr int max_smem_bytes() { return smem_bytes(MAX_TOK); }
 };
-// what lies in the stages after the mainloop: S pushed partials, or the partial tile (ntok x 512 B) and the y tiles
-static_assert(RotFewCfg::MAX_CLUSTER * RotFewCfg::PART_BYTES <= RotFewCfg::STAGES * RotFewCfg::stage_bytes(16) &&
-              8 * RotFewCfg::Y_BYTES <= 4 * RotFewCfg::A_BYTES && RotFewCfg::BF * 4 <= RotFewCfg::STAGES * RotFewCfg::BK * 2, "reduction buffers");
+// what lies in the stages after the mainloop where partials are pulled: the partial tile (ntok x 512 B) and the y tiles
+static_assert(8 * RotFewCfg::Y_BYTES <= 4 * RotFewCfg::A_BYTES && RotFewCfg::BF * 4 <= RotFewCfg::STAGES * RotFewCfg::BK * 2, "reduction buffers");
 static_assert(RotFewCfg::ctas_per_sm(RotFewCfg::MAX_SHARED_TOK, RotFewCfg::SHARED_STAGES) == 2 &&
               4 * RotFewCfg::Y_BYTES + 80 * RotFewCfg::BF * 4 <= RotFewCfg::SHARED_STAGES * RotFewCfg::stage_bytes(80) &&
               4 * RotFewCfg::Y_BYTES + 128 * RotFewCfg::BF * 4 <= RotFewCfg::SHARED_STAGES * RotFewCfg::stage_bytes(128), "three stages");
@@ -86,7 +90,7 @@ template <int FMT = FMT_MXFP4, int ESETS = 1, bool PUSH = false, int NST = RotFe
 __global__ void __launch_bounds__(64 + 128 * ESETS, ESETS == 1 ? 2 : 1)
 rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,
                      const __nv_bfloat16* __restrict__ R_intra, uint8_t* __restrict__ codes,
-                     uint8_t* __restrict__ scales, int M, int d, int ntok, int S, int ft0, int together,
+                     uint8_t* __restrict__ scales, int M, int d, int ntok, int S, int ft0, int together, int r_ahead,
                      float tensor_scale, int* err_word) {
   using C = RotFewCfg;
   extern __shared__ uint8_t smem_raw[];
@@ -97,24 +101,22 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   const uint32_t bar_off = nst * stage_bytes;
   const uint32_t bar_base = smem_base + bar_off;
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
-  auto empty_bar = [&](int s) { return bar_base + 8u * (C::STAGES + s); };
-  const uint32_t accf_bar = bar_base + 8u * (2 * C::STAGES);
-  const uint32_t ready_bar = accf_bar + 8;               // PUSH: the owner's stages are free to be written
-  const uint32_t recv_bar = accf_bar + 16;               // PUSH, in the owner: all partials are here
+  auto empty_bar = [&](int s) { return bar_base + 8u * (C::MAX_STAGES + s); };
+  const uint32_t accf_bar = bar_base + 8u * (2 * C::MAX_STAGES);
+  auto recv_bar = [&](int w) { return accf_bar + 8u + 8u * w; };   // PUSH: all partials of the units of epilogue warp w are here
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + bar_off + 192);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(smem_gen + bar_off + 200);
-  uint8_t* ri_tiles = smem_gen + bar_off + C::BAR_BYTES;    // not part of the stages: filled at kernel start
+  uint8_t* ri_tiles = smem_gen + bar_off + C::BAR_BYTES;    // not part of the stages: filled at kernel start (PUSH: the partials)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = blockIdx.x % S, ft = ft0 + blockIdx.x / S;
   const int k_tiles = d / C::BK;
   const int kt0 = (int)((long long)k_tiles * rank / S), kt1 = (int)((long long)k_tiles * (rank + 1) / S);
   const uint32_t tmem_cols = ntok <= 32 ? 32u : (ntok <= 64 ? 64u : (ntok <= 128 ? 128u : 256u));
-  // Token groups; group g belongs to CTA g % S.  Groups of 8 up to 32 tokens, where that leaves no CTA more than one: a
-  // group of 16 takes its partials in two round trips through the cluster (24 tokens: d = 4096 10.0 -> 9.5 us, d = 2048
-  // 5.95 -> 5.7).  At 40 tokens the whole layer gains at d = 4096 (1 %) and loses at 2048 (1 %), at 48 it loses.
-  const int gtok = !PUSH && M <= 32 && (M + 7) / 8 <= S ? 8 : 16;
-  const int groups = (M + gtok - 1) / gtok;
+  const int groups = (M + 15) / 16;                      // pull: token groups; group g belongs to CTA g % S
+  // PUSH: unit u = q + 4 c is block q of the tile and tokens 4 c .. 4 c + 3.  CTA u % S owns it, epilogue warp u / S % 4 of that
+  // CTA works it: the units of warp w are rank + S w, + 4 S, ..., all of the same block.
+  const int units = 4 * ((M + 3) / 4);
 
   // R_inter is a constant of the layer, never the output of the kernel that runs just before this
   // one: the thread that initialises the barriers sends the loads of the first stages' R_inter tiles
@@ -124,7 +126,8 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   if (threadIdx.x == 0) {
     for (int s = 0; s < nst; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     mbar_init(accf_bar, 1);
-    if constexpr (PUSH) { mbar_init(ready_bar, 1); mbar_init(recv_bar, 1); }
+    if constexpr (PUSH)
+      for (int w = 0; w < 4; ++w) mbar_init(recv_bar(w), 1);
     *cta_abort = 0;
     fence_mbar_init();
     fence_proxy_async_smem();                            // the copy engine sees the initialised barriers
@@ -135,7 +138,9 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
       tma_load_2d(st + C::A_BOX_BYTES, &tmR, ft * C::BF + 64, (kt0 + it) * C::BK, full_bar(it));
     }
     tma_prefetch_desc(&tmX);
-    if (PUSH && S > 1 && rank == 0) mbar_arrive_expect_tx(recv_bar, (uint32_t)((M + 3) / 4 * S * C::BF * 16));
+    if (PUSH && S > 1)
+      for (int w = 0; w < 4 && rank + S * w < units; ++w)
+        mbar_arrive_expect_tx(recv_bar(w), (uint32_t)((units - rank - S * w + 4 * S - 1) / (4 * S) * S * C::PART_BYTES));
   }
   if (warp == 1) { tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), tmem_cols); tmem_relinquish(); }
   tc_fence_before_sync();
@@ -144,7 +149,17 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   griddep_launch_dependents();
-  if (warp >= 2 && warp < 6 && R_intra != nullptr && rank < groups) {
+  uint32_t rr[16];                                       // PUSH: column `lane` of the unit's R_intra block, two rows per word
+  if constexpr (PUSH) {
+    const int u0 = rank + S * (warp & 3);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) rr[k] = 0u;
+    if (warp >= 2 && R_intra != nullptr && u0 < units) {
+      const uint16_t* src = reinterpret_cast<const uint16_t*>(R_intra) + (size_t)(ft * 4 + (u0 & 3)) * 1024 + lane;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) rr[k] = (uint32_t)__ldg(src + 64 * k) | ((uint32_t)__ldg(src + 64 * k + 32) << 16);
+    }
+  } else if (warp >= 2 && warp < 6 && R_intra != nullptr && rank < groups) {
     // this warp's R_intra block (a constant of the layer as well), 128 pieces of 16 B: row piece / 4
     uint8_t* r_s = ri_tiles + (warp & 3) * C::RI_BYTES;
     const uint4* src = reinterpret_cast<const uint4*>(R_intra + (size_t)(ft * 4 + (warp & 3)) * 1024);
@@ -154,13 +169,30 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
       *reinterpret_cast<uint4*>(r_s + (piece >> 2) * 80 + (piece & 3) * 16) = __ldg(src + piece);
     }
   }
+  // X is not a constant, but asking the L2 for it changes nothing that a later load sees: one box per CTA until the K range is out
+  // So does asking for R_inter beyond the stages: until X has come the stages stay full and HBM idle.
+  if (warp == 2 && elect_one())
+    for (int kt = kt0 + ft - ft0; kt < kt1; kt += gridDim.x / S) tma_prefetch_l2_2d(&tmX, kt * C::BK, 0);
+  if (warp == 3 && elect_one())
+    for (int kt = kt0 + pre; kt < min(kt1, kt0 + pre + r_ahead); ++kt) {
+      tma_prefetch_l2_2d(&tmR, ft * C::BF, kt * C::BK);
+      tma_prefetch_l2_2d(&tmR, ft * C::BF + 64, kt * C::BK);
+    }
   griddep_wait();
+  // The X tiles of the first stages go out from four warps at once: one warp needs 0.2 us from one stage to the next.  (PUSH only:
+  // elsewhere these warps may still wait for R_intra.  100 tokens, d = 8192: the layer 34.8 / 35.3.)
+  const int x_pre = !PUSH ? 0 : (pre < 4 ? pre : 4);
+#pragma unroll
+  for (int it = 0; it < 4; ++it)
+    if (PUSH && warp == 2 + it && it < x_pre && elect_one())
+      tma_load_2d(smem_base + it * stage_bytes + C::A_BYTES, &tmX, (kt0 + it) * C::BK, 0, full_bar(it));
+  __syncwarp();
 
   bool acc_ok = false;                                   // epilogue warps: the accumulator is complete
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     bool ok = true;
-    for (int kt = kt0, it = 0; kt < kt1 && ok; ++kt, ++it) {
+    for (int kt = kt0 + x_pre, it = x_pre; kt < kt1 && ok; ++kt, ++it) {
       const int s = it % nst;
       if (!mbar_wait_warp(empty_bar(s), ((it / nst) & 1) ^ 1, cta_abort, err_word, SITE_PRODUCER_EMPTY)) {
         ok = false; break;
@@ -226,12 +258,11 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
       IntraFrag f;
       if (R_intra != nullptr) load_intra_frag(r_lane, r_lane + 32, 16 * 80, f);
       uint32_t sb[2];
-      intra_quantize_frag16<FMT, true>(y, R_intra != nullptr, f, lane, gtok * g, live ? min(M, gtok * (g + 1)) : 0, blk, nblocks, d, nvs, codes, sb);
+      intra_quantize_frag16<FMT, true>(y, R_intra != nullptr, f, lane, 16 * g, live ? M : 0, blk, nblocks, d, nvs, codes, sb);
       if (p == 0 && live) {
 #pragma unroll
         for (int rh = 0; rh < 2; ++rh) {                 // rows of the group past the last token: zero
-          if (8 * rh >= gtok) break;
-          const int row = gtok * g + r8 + 8 * rh;
+          const int row = 16 * g + r8 + 8 * rh;
           const uint32_t b = row < M ? sb[rh] : 0u;
           if constexpr (FMT == FMT_NVFP4) *reinterpret_cast<uint16_t*>(scales + scale_offset(row, 2 * blk, kb4)) = (uint16_t)b;
           else scales[scale_offset(row, blk, kb4)] = (uint8_t)b;
@@ -240,59 +271,72 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
     };
     const uint32_t tacc = tmem_base + ((uint32_t)(q * 32) << 16);
     if constexpr (PUSH) {
-      const uint32_t my_part = (uint32_t)rank * C::PART_BYTES + (uint32_t)feature * 16;
+      const int w = q;                                   // its number among the four: with S = 1 its own features are its units
+      const uint32_t recv_base = smem_u32(ri_tiles);
+      const uint32_t y_tile = recv_base + (uint32_t)(C::push_bytes(ntok) - 4 * C::PART_BYTES + w * C::PART_BYTES);
+      // where this warp's partials go: block q, tokens 4 c ... (worked out before they are needed: a division takes as long as a store)
+      uint32_t dst[C::MAX_PUSH_TOK / 4], dst_bar[C::MAX_PUSH_TOK / 4];
+#pragma unroll
+      for (int c = 0; c < C::MAX_PUSH_TOK / 4; ++c) {
+        const int u = q + 4 * c, ui = u / S, owner = u - ui * S;
+        dst[c] = map_to_cta(recv_base + (uint32_t)((ui * S + rank) * C::PART_BYTES + lane * 16), (uint32_t)owner);
+        dst_bar[c] = map_to_cta(recv_bar(ui & 3), (uint32_t)owner);
+      }
+      if (S > 1) cluster_wait();
 #pragma unroll 1
-      for (int pass = rank == 0 ? 0 : 1; pass < 2; ++pass) {
+      for (int pass = rank + S * w < units ? 0 : 1; pass < 2; ++pass) {
         const bool live = pass == 1;
+        uint32_t v[C::MAX_PUSH_TOK];
         if (live) {
           acc_ok = mbar_wait(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
-          // every load into the stages has landed and every instruction that read them has completed
           acc_ok = __all_sync(0xFFFFFFFFu, acc_ok);
           bool ok = acc_ok;
-          if (S > 1) {
-            cluster_wait();
-            if (rank == 0 && ok && warp == 2 && lane < S) mbar_arrive_cluster(map_to_cta(ready_bar, (uint32_t)lane));
-            if (ok) ok = mbar_wait_cluster(ready_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
-            ok = __all_sync(0xFFFFFFFFu, ok);
-          }
           if (!ok) break;
           tc_fence_after_sync();
-          uint32_t v[16];
-          tmem_ld_32x32_x16(tacc, v);
+          tmem_ld_32x32_x16(tacc, *reinterpret_cast<uint32_t(*)[16]>(v));
+          if (ntok > 16) tmem_ld_32x32_x16(tacc + 16, *reinterpret_cast<uint32_t(*)[16]>(v + 16));
           tmem_ld_wait();
-          const uint32_t dst = map_to_cta(smem_base, 0) + my_part, bar = map_to_cta(recv_bar, 0);
+          if (S > 1) {
 #pragma unroll
-          for (int c = 0; c < 4; ++c)                    // piece c: four tokens
-            if (S == 1)
-              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(smem_base + my_part + (uint32_t)(c * C::BF * 16)),
-                           "r"(v[4 * c]), "r"(v[4 * c + 1]), "r"(v[4 * c + 2]), "r"(v[4 * c + 3]) : "memory");
-            else if (4 * c < M)
-              st_async_v4(dst + (uint32_t)(c * C::BF * 16), v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3], bar);
-          if (rank != 0) break;                          // not the owner
-          if (S > 1) ok = __all_sync(0xFFFFFFFFu, mbar_wait_cluster(recv_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL));
+            for (int c = 0; c < C::MAX_PUSH_TOK / 4; ++c)
+              if (4 * c < M) st_async_v4(dst[c], v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3], dst_bar[c]);
+            if (rank + S * w >= units) break;            // nothing to receive
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait_cluster(recv_bar(w), 0, cta_abort, err_word, SITE_EPI_ACC_FULL));
+          }
           if (!ok) break;
-          __syncwarp();
         }
-        float sum[16];
+#pragma unroll 1
+        for (int u = rank + S * w, ui = w; u < units; u += 4 * S, ui += 4) {
+          const int c = u >> 2, blk_u = ft * 4 + (u & 3);
+          float y[4] = {0.f, 0.f, 0.f, 0.f};             // of feature `lane` of the block, four tokens
+          if (S > 1) {
+            float4 part[C::MAX_CLUSTER];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) sum[i] = 0.f;
-        const uint32_t part0 = smem_base + (uint32_t)(r8 & 3) * 4;
-        for (int s = 0; s < S; ++s) {                    // rank order: the result does not depend on timing
+            for (int s = 0; s < C::MAX_CLUSTER; ++s)
+              if (s < S)
+                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                             : "=f"(part[s].x), "=f"(part[s].y), "=f"(part[s].z), "=f"(part[s].w)
+                             : "r"(recv_base + (uint32_t)((ui * S + s) * C::PART_BYTES + lane * 16)));
 #pragma unroll
-          for (int n = 0; n < 4; ++n)
+            for (int s = 0; s < C::MAX_CLUSTER; ++s)     // rank order: the result does not depend on timing
+              if (s < S) { y[0] += part[s].x; y[1] += part[s].y; y[2] += part[s].z; y[3] += part[s].w; }
+          } else if (live) {                             // S = 1: q = u % 4, the sums are this warp's own
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int col = q * 32 + 8 * n + 2 * p + (i & 1);
-              float v;
-              asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v)
-                           : "r"(part0 + (uint32_t)(s * C::PART_BYTES + (((r8 >> 2) + 2 * (i >> 1)) * C::BF + col) * 16)));
-              sum[4 * n + i] += v;
-            }
+            for (int cc = 0; cc < C::MAX_PUSH_TOK / 4; ++cc)
+              if (cc == c) {
+#pragma unroll
+                for (int t = 0; t < 4; ++t) y[t] = __uint_as_float(v[4 * cc + t]);
+              }
+          }
+          float z[4] = {y[0], y[1], y[2], y[3]};
+          if (R_intra != nullptr) {
+            __syncwarp();
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(y_tile + lane * 16), "f"(y[0]), "f"(y[1]), "f"(y[2]), "f"(y[3]) : "memory");
+            __syncwarp();
+            intra_rotate_lane4(y_tile, rr, z);
+          }
+          quantize_lane4<FMT>(z, lane, 4 * c, live ? M : 0, blk_u, d, kb4, nvs, codes, scales);
         }
-        uint32_t y[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) y[i] = __float_as_uint(sum[i]);
-        finish(y, 0, live);
       }
     } else {
       float* y_s = reinterpret_cast<float*>(smem_gen + ntok * C::BF * 4 + (es * 4 + q) * C::Y_BYTES);
@@ -330,11 +374,11 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
         for (; g < groups; g += S * ESETS) {
 #pragma unroll
           for (int jh = 0; jh < 2; ++jh) {
-            if (8 * jh >= gtok || gtok * g + 8 * jh >= M) break;      // rows 8 jh .. 8 jh + 7 of the group hold no token
+            if (16 * g + 8 * jh >= M) break;      // rows 8 jh .. 8 jh + 7 of the group hold no token
             float4 part[2][C::MAX_CLUSTER];
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-              const uint32_t off = (uint32_t)(((gtok * g + tr + 4 * (2 * jh + j)) * C::BF + q * 32 + fc) * 4);
+              const uint32_t off = (uint32_t)(((16 * g + tr + 4 * (2 * jh + j)) * C::BF + q * 32 + fc) * 4);
 #pragma unroll
               for (int s = 0; s < C::MAX_CLUSTER; ++s)
                 if (s < S)
@@ -370,7 +414,7 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
     // scale bytes of the rows no group covers, up to the last row of the 128-row scale tiles: zero
     if (rank == 0 && es == 0) {
       for (int row = q * 32 + lane; row < (M > 128 ? 256 : 128); row += 128) {
-        if (row >= gtok * groups) {
+        if (row >= (PUSH ? units : 16 * groups)) {
           uint8_t* cell = scales + (size_t)(row >> 7) * kb4 * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4;
           if constexpr (FMT == FMT_NVFP4) {
             *reinterpret_cast<uint32_t*>(cell + (size_t)(2 * ft) * 512) = 0u;

@@ -131,13 +131,13 @@ static DeviceState* device_state() {
               opt_in_smem(rotate_quantize_kernel<256, FMT_MXINT4>, RotCfg<256>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_MXINT4>, RotPairCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_structured_kernel<FMT_MXINT4>, RotStructCfg::SMEM_BYTES) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true, RotFewCfg::PUSH_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 2>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true, RotFewCfg::PUSH_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 2>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true, RotFewCfg::PUSH_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 2>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 1, true>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) && opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 1>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) &&
@@ -278,6 +278,10 @@ static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int64_t most, i
 // the tiles (us, alone / shared, 72 and 128 tokens: d = 5120, 27 steps 14.2 / 14.7 and 16.2 / 17.7; d = 6400, 50 steps 21.7 /
 // 19.9 and 23.4 / 22.0; d = 8192 28.0 / 26.4 and 30.3 / 28.0; d = 11008, one CTA for each of 86 tiles 52.0 / 41.1 and 53.6 /
 // 44.4; d = 14336 78 / 68 and 79 / 73).
+// R_inter tiles (16 KiB) that all CTAs together ask the L2 for beyond their stages: 10 MB (us, 0 / 3 / 4 / 6 / 16 per CTA of 200, d = N = 5120,
+// 1 token 14.8 / 14.3 / 14.25 / 14.4 / 15.7; of 192, 24 tokens d = 4096 NVFP4 3 / 4 / 6: 13.5 / 13.8 / 14.0; of 128, 100 tokens
+// d = 4096 0 / 3 / 5 / 8: 18.4 / 18.2 / 18.1 / 18.2).
+constexpr int kAheadTiles = 640;
 struct FewRotation { int cluster, stages; };
 static FewRotation fewtok_rotation(int64_t M, int64_t d, const DeviceState* st) {
   const int ntok = fewtok_ntok(M);
@@ -285,13 +289,16 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, const DeviceState* st) 
   const int long_k = ntok > 128 ? 1 : 10, ctas = RotFewCfg::ctas_per_sm(ntok);
   // 17 to 64 tokens: two steps less are enough for one more CTA (us, S = 4 / 5 at 48 steps, d = 3072, 24 and 64 tokens: 8.4 /
   // 7.7 and 9.8 / 9.0, the layer with N = 3072 12.7 / 11.2 and 15.1 / 14.6; S = 5 / 6 at 58, d = 3712: 9.6 / 8.9 and 11.0 / 10.6)
-  int64_t most = (steps + (ntok > RotFewCfg::MAX_PUSH_TOK && ntok <= 64 ? 2 : 0)) / long_k;
+  int64_t most = (steps + (ntok > 16 && ntok <= 64 ? 2 : 0)) / long_k;
   // 65 to 96 tokens are five or six groups: a cluster of six, where it fits, has one unit per CTA, which pays from ranges of
   // four steps on (us, S = 4 or the one-wave kernel / S = 6, 65 and 96 tokens: d = 1536 7.4 / 6.1 and 7.4 / 6.5, MXINT4 7.6 / 6.2 and
   // 7.7 / 6.6, layer with N = 256 11.6 / 10.0 and 12.0 / 10.9; d = 2560 8.1 / 7.5 and 8.7 / 8.2).  At 23 and 24 tiles, where only five
   // fit, 96 tokens lose (d = 3072 9.3 / 9.6).
   if (ntok > 64 && ntok <= 96 && steps >= 24 && tiles <= st->few_fit[6] && most < 6) most = 6;
   const int S = fewtok_cluster(tiles, steps, most, ctas, st->sm_count, st->few_fit);
+  // A fifth stage up to 16 tokens, but not on long K ranges (us, four / five stages, 1 token: layer d = N = 5120 14.5 / 14.3; rotation
+  // d = 14336 59.4 / 60.7).
+  if (ntok <= 16 && steps <= 32 * S) return {S, RotFewCfg::PUSH_STAGES};
   if (ctas > 1 || ntok > RotFewCfg::MAX_SHARED_TOK || steps <= 32 * S) return {S, RotFewCfg::STAGES};
   return {fewtok_cluster(tiles, steps, most, 2, st->sm_count, st->few_fit), RotFewCfg::SHARED_STAGES};
 }
@@ -564,20 +571,20 @@ static torq_status rotate_fewtok(DeviceState* st, int fmt, const void* X, const 
   const float ts = fmt == FMT_NVFP4 ? tensor_scale : 0.0f;
   const __nv_bfloat16* ri = static_cast<const __nv_bfloat16*>(R_intra);
   // up to 16 tokens: partials pushed to one CTA; two CTAs per SM: one set of epilogue warps; one CTA: two sets
-  auto launch = [&](auto push, auto one, auto shared, auto two) {
-    const bool share = few.stages != RotFewCfg::STAGES, small = share || RotFewCfg::ctas_per_sm(ntok) >= 2;
-    launch_tc(ntok <= RotFewCfg::MAX_PUSH_TOK ? push : (share ? shared : (small ? one : two)), S, tiles * S, small ? 192 : 320, smem, s,
-              tmX, tmR, ri, codes, scales, (int)M, (int)d, ntok, S, ft0, fewtok_leave_together(M, tiles, few, st) ? 1 : 0, ts, st->err_word);
+  auto launch = [&](auto push5, auto push, auto one, auto shared, auto two) {
+    const bool share = few.stages == RotFewCfg::SHARED_STAGES, small = share || RotFewCfg::ctas_per_sm(ntok) >= 2;
+    launch_tc(few.stages == RotFewCfg::PUSH_STAGES ? push5 : (ntok <= RotFewCfg::MAX_PUSH_TOK ? push : (share ? shared : (small ? one : two))), S, tiles * S, small ? 192 : 320, smem, s,
+              tmX, tmR, ri, codes, scales, (int)M, (int)d, ntok, S, ft0, fewtok_leave_together(M, tiles, few, st) ? 1 : 0, kAheadTiles / (tiles * S), ts, st->err_word);
   };
   constexpr int NS = RotFewCfg::SHARED_STAGES;
   if (fmt == FMT_MXINT4)
-    launch(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, rotate_fewtok_kernel<FMT_MXINT4, 1>, rotate_fewtok_kernel<FMT_MXINT4, 1, false, NS>,
+    launch(rotate_fewtok_kernel<FMT_MXINT4, 1, true, RotFewCfg::PUSH_STAGES>, rotate_fewtok_kernel<FMT_MXINT4, 1, true>, rotate_fewtok_kernel<FMT_MXINT4, 1>, rotate_fewtok_kernel<FMT_MXINT4, 1, false, NS>,
            rotate_fewtok_kernel<FMT_MXINT4, 2>);
   else if (fmt == FMT_NVFP4)
-    launch(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, rotate_fewtok_kernel<FMT_NVFP4, 1>, rotate_fewtok_kernel<FMT_NVFP4, 1, false, NS>,
+    launch(rotate_fewtok_kernel<FMT_NVFP4, 1, true, RotFewCfg::PUSH_STAGES>, rotate_fewtok_kernel<FMT_NVFP4, 1, true>, rotate_fewtok_kernel<FMT_NVFP4, 1>, rotate_fewtok_kernel<FMT_NVFP4, 1, false, NS>,
            rotate_fewtok_kernel<FMT_NVFP4, 2>);
   else
-    launch(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, rotate_fewtok_kernel<FMT_MXFP4, 1>, rotate_fewtok_kernel<FMT_MXFP4, 1, false, NS>,
+    launch(rotate_fewtok_kernel<FMT_MXFP4, 1, true, RotFewCfg::PUSH_STAGES>, rotate_fewtok_kernel<FMT_MXFP4, 1, true>, rotate_fewtok_kernel<FMT_MXFP4, 1>, rotate_fewtok_kernel<FMT_MXFP4, 1, false, NS>,
            rotate_fewtok_kernel<FMT_MXFP4, 2>);
   return launch_status();
 }

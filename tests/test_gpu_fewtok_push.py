@@ -1,0 +1,93 @@
+"""Few-token kernels whose partial sums are pushed in pieces of 32 features x 4 tokens (up to 32 tokens; the NVFP4 GEMM up to 24): token
+counts on both sides of every four, clusters of one CTA to eight, one and several pieces per warp.  Operands whose sums are exact in any
+order, so codes, scale bytes, padding and results must equal the oracle's bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from helpers import captured_launches, dev_bf16, gpu_quantized_to_numpy
+from paper_2605_19561_b200 import inputs as I
+from paper_2605_19561_b200 import torq
+import test_gpu_fewtok as TF
+import test_gpu_mxint4 as TI
+import test_gpu_nvfp4 as TN
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,d", [(1, 128), (2, 256), (3, 19072), (4, 640), (5, 1536), (7, 2560), (8, 5120), (9, 4096), (12, 7168), (13, 9600),
+                                 (16, 2048), (17, 128), (20, 14336), (21, 1536), (24, 4096), (28, 2560), (29, 896), (31, 640), (32, 5120),
+                                 (30, 19072)])
+def test_rotation_of_permutations_in_the_three_formats(M, d):
+    g = np.random.default_rng(M + d)
+    xb = I.to_bf16_bits(g.integers(-8, 9, size=(M, d)).astype(np.float64))
+    perm = g.permutation(d)
+    P = torch.zeros((d, d), dtype=torch.bfloat16, device="cuda")
+    P[torch.arange(d, device="cuda"), torch.from_numpy(perm).cuda()] = 1
+    y = np.empty((M, d))
+    y[:, perm] = O.decode_bf16(xb)
+    X = dev_bf16(xb)
+    for width in (None, 16, 32):                             # no rotation inside the blocks, a permutation of each
+        z, Ri = y, None
+        if width is not None:
+            pin = np.stack([np.eye(width)[g.permutation(width)] for _ in range(d // width)])
+            z = np.einsum("mbk,bkj->mbj", y.reshape(M, d // width, width), pin).reshape(M, d)
+            Ri = dev_bf16(I.to_bf16_bits(pin))
+        z = z.astype(np.float32)
+        if width != 16:
+            codes = torch.full((M, d // 2), 0xEE, dtype=torch.uint8, device="cuda")
+            scales = torch.full((torq.torq_scales_bytes(M, d),), 0xEE, dtype=torch.uint8, device="cuda")
+            call = lambda: torq.torq_rotate_quantize(X, P, Ri, out_codes=codes, out_scales=scales)
+            call()
+            torch.cuda.synchronize()
+            o_codes, o_sb = O.quantize_mxfp4(z)
+            g_codes, g_sb = gpu_quantized_to_numpy(codes, scales, M, d)
+            assert np.array_equal(g_codes, o_codes) and np.array_equal(g_sb, o_sb)
+            assert np.array_equal(scales.cpu().numpy(), O.swizzle_scales(o_sb, d, fill=0))       # padding rows hold zero
+            assert d < 1536 or "rotate_fewtok_kernelILi0ELi1ELb1E" in captured_launches(call)[0][0]
+            byt, s = torq.torq_rotate_quantize_mxint4(X, P, Ri)
+            torch.cuda.synchronize()
+            o_q, o_sb = O.quantize_mxint4(z)
+            assert np.array_equal(TI._operand_to_int(byt), o_q) and np.array_equal(O.unswizzle_scales(s.cpu().numpy(), M, d), o_sb)
+        if width != 32:
+            ts = O.tensor_scale_from_amax(np.abs(z).max())
+            Ri32 = None if Ri is None else torq.torq_expand_intra16(Ri)
+            n_codes, n_sb = TN._to_numpy(*torq.torq_rotate_quantize_nvfp4(X, P, Ri32, float(ts)), M, d)
+            o_codes, o_sb = O.quantize_nvfp4(z, ts)
+            assert np.array_equal(n_sb, o_sb) and np.array_equal(n_codes, o_codes)
+    assert torq.torq_last_device_error() == 0
+
+
+def test_rotation_keeps_what_is_not_a_number_in_its_token():
+    """One infinity and one NaN in X reach the outputs of their token only."""
+    M, d = 6, 256
+    x = np.ones((M, d))
+    X = dev_bf16(I.to_bf16_bits(x))
+    X[1, 5], X[4, 40] = float("inf"), float("nan")
+    E = torch.eye(d, dtype=torch.bfloat16, device="cuda")
+    clean, clean_s = torq.torq_rotate_quantize(dev_bf16(I.to_bf16_bits(x)), E, None)
+    codes, scales = torq.torq_rotate_quantize(X, E, None)
+    torch.cuda.synchronize()
+    same = [m for m in range(M) if m not in (1, 4)]
+    assert torch.equal(codes.view(M, -1)[same], clean.view(M, -1)[same])
+    a, b = (O.unswizzle_scales(t.cpu().numpy(), M, d) for t in (scales, clean_s))
+    assert np.array_equal(a[same], b[same])
+    assert torq.torq_last_device_error() == 0
+
+
+# N ragged in a 32-feature piece and in the tile, a half last stage of K, clusters of one to eight
+@pytest.mark.parametrize("M,N,K", [(1, 8, 128), (2, 72, 256), (3, 136, 640), (4, 264, 2048), (5, 1000, 2048), (8, 5120, 5120), (9, 520, 4096), (13, 1024, 4096),
+                                   (16, 6144, 896), (17, 264, 384), (20, 2560, 1024), (21, 1032, 4096), (24, 4096, 2048), (25, 264, 2048), (29, 72, 4096),
+                                   (32, 5120, 1152)])
+def test_gemm_of_exact_sums_in_the_three_formats(M, N, K):
+    g = np.random.default_rng(M + N + K)
+    ac, _ = TF._rand_operand(M, K, 3)
+    wc, _ = TF._rand_operand(N, K, 4)
+    one = lambda r: np.full((r, K // 32), 127, np.uint8)
+    assert (TF._gpu_gemm(ac, one(M), wc, one(N), torch.float32) == O.gemm_dequant(ac, one(M), wc, one(N))).all()
+    asb, wsb = (g.choice(np.array([0x30, 0x38, 0x40], np.uint8), size=(r, K // 16)) for r in (M, N))
+    got = TN._gpu_gemm(ac, asb, 0.25, wc, wsb, 2.0, torch.float32)
+    assert (got == O.gemm_nvfp4(ac, asb, 0.25, wc, wsb, 2.0)).all()      # multiples of 2^-4 up to 36 x 4 K: below 2^24 units
+    aq, wq = (g.integers(-7, 8, size=(r, K)).astype(np.int8) for r in (M, N))
+    assert (TI._gpu_gemm(aq, one(M), wq, one(N), torch.float32) == O.gemm_mxint4(aq, one(M), wq, one(N))).all()
