@@ -42,6 +42,7 @@ struct RotWideCfg {
   __host__ __device__ static constexpr int a_bytes(int width) { return BM * bk(width) * 2; }       // 32 or 16 KiB
   __host__ __device__ static constexpr int box_bytes(int width) { return 64 * bk(width) * 2; }     // 64 columns of R_inter
   static constexpr int MAX_WIDTH = 384;
+  static constexpr int AHEAD = 8;                      // K steps of R_inter that the L2 is asked for beyond the stages
   static constexpr int MAX_STAGES = 6;
   static constexpr int RI_BLOCK_BYTES = 32 * 64;       // R_intra[blk] as bf16 rows of 64 bytes, 16-byte pieces XOR-swizzled
   static constexpr int ESETS = 3;
@@ -195,6 +196,18 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
     const int p = lane & 3, r8 = lane >> 2;
     const int nblocks = d / 32, nb = width / 32, b0 = tcol >> 5;
     const uint32_t ri_saddr = smem_base + ri_off;
+    if (warp == 3 && elect_one()) {
+      // Until the kernel before has completed HBM idles.  In short calls the L2 is asked for the first K steps of X, one of each row tile
+      // per pair that shares it, and, for strips of 64 to 128 columns, for the next R_inter, a strip's steps dealt over its row tiles (us,
+      // without / X alone / both, layers: 300 x 2048 -> 2048 14.00 / 13.83 / 13.69, 600 x 2048 15.4 / 15.1 / 14.9, 400 x 4096 -> 4096 25.7 /
+      // 25.3 / 25.1, 1500 x 2048 22.0 / 21.6; narrower strips lose by R_inter, 220 x 2048 12.73 / 12.60 / 12.71).  Calls long enough to run
+      // at the power cap lose (loops of 0.6 s, 1024 x 4096 44.4 / 44.7 / 45.0, 777 x 5120 60.7 / 60.8).
+      if (width * d <= 128 * 4096 && pair / rows < k_tiles) tma_prefetch_l2_3d(&tmX, 0, mt * C::BM, pair / rows * (BK / C::SLAB));
+      if (RANGE == 128 && width >= 64)
+        for (int kt = pre + pair % rows; kt < min(k_tiles, pre + C::AHEAD); kt += rows)
+          for (int c = 0; c < width / 2; c += 64) tma_prefetch_l2_2d(&tmR, tcol + (int)rank * (width / 2) + c, kt * BK);
+    }
+    __syncwarp();
     if (warp == 2) {
       // X loads of the first stages, from a warp of its own: not behind the R_inter loads of all these stages
       griddep_wait();
