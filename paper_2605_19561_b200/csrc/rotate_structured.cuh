@@ -113,11 +113,11 @@ rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  griddep_launch_dependents();
-  griddep_wait();
+  griddep_launch_dependents();                           // each role passes griddep_wait first
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
+    griddep_wait();
     if (elect_one()) { tma_prefetch_desc(&tmRB); tma_prefetch_desc(&tmX3); }
     uint32_t it = 0;
     bool ok = true;
@@ -142,6 +142,7 @@ rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ step-2 issuer
+    griddep_wait();
     constexpr uint32_t idesc1 = idesc_bf16(128, BN, /*A MN-major*/ false, /*B MN-major*/ true);
     uint32_t it = 0;
     bool ok = true;
@@ -191,6 +192,14 @@ rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_
     // thread's loop the kernel's critical path.
     constexpr uint32_t idesc2 = idesc_bf16(128, 32, /*A MN-major*/ false, /*B MN-major*/ true);
     const uint64_t rdesc = make_desc(ri_base, 2048, 512, kSwizzle64);
+    // Until the kernel before has completed HBM idles: the L2 is asked for the first tile's X, one 4-KiB box per lane, and for R_B where
+    // it is one strip (with two or more the order in which they then run costs more: 4096 x 5120 -> 1024 37.1 / 38.6 us).  Here and
+    // not ahead of the roles, whose instructions would lie further apart (64 x 256 -> 256 6.54 / 6.62).  us, without / with, layers:
+    // 2048 x 4096 -> 6144 34.4 / 33.5, 300 x 4096 -> 4096 12.1 / 11.8, 8192 x 2048 -> 2048 40.3 / 39.9.
+    if ((lane >> 2) < k_tiles) tma_prefetch_l2_3d(&tmX3, 0, blockIdx.x / b_tiles * C::TOK + (lane & 3), (lane >> 2) * C::BK);
+    if (b_tiles == 1 && lane < k_tiles) tma_prefetch_l2_2d(&tmRB, lane * C::BK, 0);
+    __syncwarp();
+    griddep_wait();
     uint32_t tcount = 0;
     bool ok = true;
     for (int tile = blockIdx.x; intra && tile < total_tiles && ok; tile += gridDim.x, ++tcount) {
@@ -215,6 +224,7 @@ rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_
     }
   } else {
     // ------------------------------------------------------------------ epilogue (four groups of 4 warps)
+    griddep_wait();
     // Group g owns token g of every tile; inside a group warp q reads lane quarter q (32 output
     // blocks).  Sixteen warps = four per scheduler: while one group waits for its step-3 MMAs the
     // others split or quantize.  A warp whose 32 rows lie wholly beyond the last block (the second
