@@ -85,7 +85,8 @@ static_assert(RotFewCfg::ctas_per_sm(RotFewCfg::MAX_SHARED_TOK, RotFewCfg::SHARE
 // a multiple of 16.  d % 128 == 0.  `codes` / `scales` / `tensor_scale` as in rotate_quantize_kernel for FMT.
 // ESETS: sets of four epilogue warps (threads = 64 + 128 ESETS).  One set where two CTAs share an SM; a CTA that fills an SM
 // by itself has several token groups to reduce, rotate and quantize, each a dependent chain of about a microsecond for
-// one warp: two sets take them in turn.  NST: stages.  `together`: the CTAs of a cluster leave together (S > 1 only).
+// one warp: two sets take them in turn.  NST: stages.  `r_ahead`: R_inter tiles beyond
+// the stages that a CTA asks the L2 for.  `together`: the CTAs of a cluster leave together (S > 1 only).
 template <int FMT = FMT_MXFP4, int ESETS = 1, bool PUSH = false, int NST = RotFewCfg::STAGES>
 __global__ void __launch_bounds__(64 + 128 * ESETS, ESETS == 1 ? 2 : 1)
 rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,

@@ -278,7 +278,7 @@ static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int64_t most, i
 // the tiles (us, alone / shared, 72 and 128 tokens: d = 5120, 27 steps 14.2 / 14.7 and 16.2 / 17.7; d = 6400, 50 steps 21.7 /
 // 19.9 and 23.4 / 22.0; d = 8192 28.0 / 26.4 and 30.3 / 28.0; d = 11008, one CTA for each of 86 tiles 52.0 / 41.1 and 53.6 /
 // 44.4; d = 14336 78 / 68 and 79 / 73).
-// R_inter tiles (16 KiB) that all CTAs together ask the L2 for beyond their stages: 10 MB (us, 0 / 3 / 4 / 6 / 16 per CTA of 200, d = N = 5120,
+// R_inter or W tiles (16 KiB) that all CTAs together ask the L2 for beyond their stages: 10 MB (us, 0 / 3 / 4 / 6 / 16 per CTA of 200, d = N = 5120,
 // 1 token 14.8 / 14.3 / 14.25 / 14.4 / 15.7; of 192, 24 tokens d = 4096 NVFP4 3 / 4 / 6: 13.5 / 13.8 / 14.0; of 128, 100 tokens
 // d = 4096 0 / 3 / 5 / 8: 18.4 / 18.2 / 18.1 / 18.2).
 constexpr int kAheadTiles = 640;
@@ -858,7 +858,7 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
     const bool small = FC::ctas_per_sm((int)M) >= 2 && (ntok <= 64 || S > fewtok_gemm_cluster(ntok, tiles, steps, 1, st));
     launch_tc(FC::push((int)M) ? gemm_fewtok_kernel<FMT, 1, true> : (small ? gemm_fewtok_kernel<FMT, 1> : gemm_fewtok_kernel<FMT, 2>),
               S, tiles * S, small ? 192 : 320, FC::smem_bytes((int)M), s, tmB, tmA, static_cast<const uint8_t*>(As),
-              static_cast<const uint8_t*>(Ws), Y, y_dtype == TORQ_BF16 ? 1 : 0, (int)M, (int)N, (int)K, ntok, S, alpha, st->err_word);
+              static_cast<const uint8_t*>(Ws), Y, y_dtype == TORQ_BF16 ? 1 : 0, (int)M, (int)N, (int)K, ntok, S, kAheadTiles / (tiles * S), alpha, st->err_word);
     return launch_status();
   }
   const int width = wide_gemm_width(M, N, (K + GemmWideCfg<FMT>::BK - 1) / GemmWideCfg<FMT>::BK, 0, st->gemm_pairs);
