@@ -51,11 +51,15 @@ struct GemmFewCfg {
   static constexpr int MAX_PUSH_TOK = 32;
   __host__ __device__ static constexpr int push_bytes(int M) { return ((M + 3) / 4 * 4 + MAX_CLUSTER - 1) * PART_BYTES; }
   __host__ __device__ static constexpr int pull_smem_bytes(int M) { return STAGES * stage_bytes((M + 15) / 16 * 16) + BAR_BYTES + 1024; }
-  // pushed where the room for what arrives leaves two CTAs per SM (NVFP4: up to 24 tokens)
-  __host__ __device__ static constexpr bool push(int M) { return M <= MAX_PUSH_TOK && pull_smem_bytes(M) + push_bytes(M) <= 113 * 1024; }
-  __host__ __device__ static constexpr int smem_bytes(int M) { return pull_smem_bytes(M) + (push(M) ? push_bytes(M) : 0); }
-  __host__ __device__ static constexpr int ctas_per_sm(int M) { return smem_bytes(M) <= 113 * 1024 ? 2 : 1; }
-  __host__ __device__ static constexpr int max_smem_bytes() { return smem_bytes(MAX_TOK); }
+  // Pushed where the room for what arrives leaves two CTAs per SM (NVFP4: up to 24 tokens); from 17 tokens on for contractions long enough
+  // that a cluster of four has work for it (us, pulled / pushed, 32 tokens: N = 4096, K = 2048 3.72 / 4.01, K = 4096 4.47 / 4.49, K = 14336 8.82 /
+  // 7.93, layers 4096 x 4096 13.7 / 13.2, 2048 x 4096 9.1 / 9.3; 18 tokens N = K = 5120 5.31 / 4.83).
+  __host__ __device__ static constexpr bool push(int M, int K) {
+    return M <= 16 || (M <= MAX_PUSH_TOK && K > 2048 && pull_smem_bytes(M) + push_bytes(M) <= 113 * 1024);
+  }
+  __host__ __device__ static constexpr int smem_bytes(int M, int K) { return pull_smem_bytes(M) + (push(M, K) ? push_bytes(M) : 0); }
+  __host__ __device__ static constexpr int ctas_per_sm(int M, int K) { return smem_bytes(M, K) <= 113 * 1024 ? 2 : 1; }
+  __host__ __device__ static constexpr int max_smem_bytes() { return pull_smem_bytes(MAX_TOK); }
   static_assert(BF * 4 <= STAGES * 128, "the pulled partial tile lies in the stages after the mainloop");
   __host__ __device__ static constexpr uint32_t tmem_cols(int ntok) {
     return ntok + 8 * CH <= 32 ? 32u : (ntok + 8 * CH <= 64 ? 64u : (ntok + 8 * CH <= 128 ? 128u : 256u));
@@ -141,9 +145,10 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   __syncwarp();
   griddep_wait();
   // The activations of the first stages go out from four warps at once: one warp needs 0.2 us from one stage to the next.
+  const int a_pre = PUSH ? pre : 0;
 #pragma unroll
   for (int it = 0; it < 4; ++it)
-    if (warp == 2 + it && it < pre && elect_one()) {
+    if (PUSH && warp == 2 + it && it < pre && elect_one()) {
       const uint32_t st = smem_base + it * stage_bytes;
       tma_load_2d(st + C::A_BYTES, &tmA, (kt0 + it) * 128, 0, full_bar(it));
       bulk_load_1d(st + C::A_BYTES + b_bytes + C::SF_BYTES, As + (size_t)(CH * (kt0 + it)) * 512,
@@ -155,7 +160,7 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     bool ok = true;
-    for (int kt = kt0 + pre, it = pre; kt < kt1 && ok; ++kt, ++it) {
+    for (int kt = kt0 + a_pre, it = a_pre; kt < kt1 && ok; ++kt, ++it) {
       const int s = it % nst;
       if (!mbar_wait_warp(empty_bar(s), ((it / nst) & 1) ^ 1, cta_abort, err_word, SITE_PRODUCER_EMPTY)) {
         ok = false; break;
@@ -163,9 +168,11 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
       const uint32_t st = smem_base + s * stage_bytes;
       const uint32_t sf_bytes = 512u * (uint32_t)min(CH, kb4 - CH * kt);
       if (elect_one()) {
-        mbar_arrive_expect_tx(full_bar(s), stage_tx(kt));
-        tma_load_2d(st, &tmW, kt * 128, nt * C::BF, full_bar(s));
-        bulk_load_1d(st + C::A_BYTES + b_bytes, Ws + ((size_t)nt * kb4 + CH * kt) * 512, sf_bytes, full_bar(s));
+        if (it >= pre) {                                 // the W side of the first stages went out before the wait above
+          mbar_arrive_expect_tx(full_bar(s), stage_tx(kt));
+          tma_load_2d(st, &tmW, kt * 128, nt * C::BF, full_bar(s));
+          bulk_load_1d(st + C::A_BYTES + b_bytes, Ws + ((size_t)nt * kb4 + CH * kt) * 512, sf_bytes, full_bar(s));
+        }
         tma_load_2d(st + C::A_BYTES, &tmA, kt * 128, 0, full_bar(s));
         bulk_load_1d(st + C::A_BYTES + b_bytes + C::SF_BYTES, As + (size_t)(CH * kt) * 512, sf_bytes, full_bar(s));
       }

@@ -35,6 +35,7 @@ struct DeviceState {
   int rot_pairs = 0;    // CTA pairs of the pair kernels that can be resident at once
   int gemm_pairs = 0;
   int few_fit[9] = {};  // clusters of S CTAs resident at once, one CTA per SM
+  int push_fit[9] = {}; // the same of the few-token kernels that push, two CTAs per SM
   int* err_word = nullptr;
 };
 static DeviceState g_dev[kMaxDevices];
@@ -74,6 +75,10 @@ static int max_active_clusters(K kernel, int size, int threads, int smem, int sm
   }
   return n;
 }
+// Stands in for a few-token kernel in that question: of a kernel that allocates tensor memory the runtime counts one CTA per SM, whatever
+// its shared memory.  Never launched.
+__global__ void __launch_bounds__(RotFewCfg::THREADS, 2) fewtok_fit_kernel() {}
+
 // CTA pairs of a kernel that fills its SMs.
 template <typename K>
 static int max_active_pairs(K kernel, int threads, int smem, int sm_count) {
@@ -107,7 +112,7 @@ static DeviceState* device_state() {
       g_encode = reinterpret_cast<EncodeTiledFn>(fn);
     }
     constexpr int kWideSmem = 232448;                    // the widths share the kernels
-    bool ok = opt_in_smem(rotate_quantize_kernel<256>, RotCfg<256>::SMEM_BYTES) &&
+    bool ok = opt_in_smem(fewtok_fit_kernel, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_quantize_kernel<256>, RotCfg<256>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_kernel<256, FMT_NVFP4>, RotCfg<256>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_MXFP4>, RotPairCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_NVFP4>, RotPairCfg::SMEM_BYTES) &&
@@ -156,6 +161,9 @@ static DeviceState* device_state() {
     if (st.rot_pairs < 1 || st.gemm_pairs < 1) return nullptr;
     for (int s = 1; s <= RotFewCfg::MAX_CLUSTER; ++s)
       st.few_fit[s] = max_active_clusters(rotate_fewtok_kernel<FMT_MXFP4, 2>, s, 320, RotFewCfg::smem_bytes(256), st.sm_count);
+    for (int s = 1; s <= RotFewCfg::MAX_CLUSTER; ++s)
+      st.push_fit[s] = max_active_clusters(fewtok_fit_kernel, s, RotFewCfg::THREADS,
+                                           RotFewCfg::smem_bytes(RotFewCfg::MAX_PUSH_TOK), st.sm_count);
     cudaGetLastError();
   }
   st.ready = true;
@@ -283,9 +291,19 @@ static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int64_t most, i
 // d = 4096 0 / 3 / 5 / 8: 18.4 / 18.2 / 18.1 / 18.2).
 constexpr int kAheadTiles = 640;
 struct FewRotation { int cluster, stages; };
-static FewRotation fewtok_rotation(int64_t M, int64_t d, const DeviceState* st) {
+static FewRotation fewtok_rotation(int64_t M, int64_t d, bool intra, const DeviceState* st) {
   const int ntok = fewtok_ntok(M);
   const int64_t tiles = d / 128, steps = d / 64;
+  // Pushed partial sums make the reduction cheap: the largest cluster that leaves room for two more (push_fit: 148, 93, 71, 56, 45, 37, 33
+  // clusters of 2 ... 8).  us, layers d = N, S = 4 / 6 / 8, 1 and 32 tokens: d = 1536 6.46 / 6.17 / 6.27 and 9.55 / 8.87 / 8.13, d = 2560 8.29 /
+  // 7.57 / 7.23 and 10.7 / 10.35 / 9.49, d = 4096 11.2 / 10.5 / 10.6 and 14.5 / 13.6 / 12.7; without the room d = 4224 (33 tiles) S = 7 /
+  // 8 11.3 / 11.8, d = 7168 (56 tiles) S = 4 / 5 23.2 / 23.6.  A fifth stage up to 16 tokens, but not on long K ranges (four / five, 1 token:
+  // layer d = N = 5120 14.5 / 14.3; rotation d = 14336 59.4 / 60.7).  A rotation without R_intra keeps the clusters of the rule below.
+  if (ntok <= RotFewCfg::MAX_PUSH_TOK && intra) {
+    int S = (int)(steps < RotFewCfg::MAX_CLUSTER ? steps : RotFewCfg::MAX_CLUSTER);
+    while (S > 1 && tiles > st->push_fit[S] - 2) --S;
+    return {S, ntok <= 16 && steps <= 32 * S ? RotFewCfg::PUSH_STAGES : RotFewCfg::STAGES};
+  }
   const int long_k = ntok > 128 ? 1 : 10, ctas = RotFewCfg::ctas_per_sm(ntok);
   // 17 to 64 tokens: two steps less are enough for one more CTA (us, S = 4 / 5 at 48 steps, d = 3072, 24 and 64 tokens: 8.4 /
   // 7.7 and 9.8 / 9.0, the layer with N = 3072 12.7 / 11.2 and 15.1 / 14.6; S = 5 / 6 at 58, d = 3712: 9.6 / 8.9 and 11.0 / 10.6)
@@ -296,8 +314,6 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, const DeviceState* st) 
   // fit, 96 tokens lose (d = 3072 9.3 / 9.6).
   if (ntok > 64 && ntok <= 96 && steps >= 24 && tiles <= st->few_fit[6] && most < 6) most = 6;
   const int S = fewtok_cluster(tiles, steps, most, ctas, st->sm_count, st->few_fit);
-  // A fifth stage up to 16 tokens, but not on long K ranges (us, four / five stages, 1 token: layer d = N = 5120 14.5 / 14.3; rotation
-  // d = 14336 59.4 / 60.7).
   if (ntok <= 16 && steps <= 32 * S) return {S, RotFewCfg::PUSH_STAGES};
   if (ctas > 1 || ntok > RotFewCfg::MAX_SHARED_TOK || steps <= 32 * S) return {S, RotFewCfg::STAGES};
   return {fewtok_cluster(tiles, steps, most, 2, st->sm_count, st->few_fit), RotFewCfg::SHARED_STAGES};
@@ -316,6 +332,29 @@ static bool fewtok_leave_together(int64_t M, int64_t tiles, FewRotation few, con
 // 4.34; S = 4 / 6: 17 tokens N = 2048 3.75 / 3.47; beyond the line 64 tokens N = 2048 NVFP4 4.53 / 4.70), and 8 up to 16 tokens,
 // where the sums are pushed (1 token N = 256 2.96 / 2.58, N = 1024 3.10 / 2.82, the layer 11.2 / 10.9; beyond: N = 2048 the GEMM 3.62 /
 // 3.51, the layer of 16 tokens 13.2 / 13.5; S = 4 / 5 at K = 2560, N = 5120 the layer 11.0 / 11.5).
+// Where the sums are pushed (M tokens), from the largest cluster down: above four CTAs where each keeps four K steps and has its SM to itself
+// (a CTA's instructions wait for those of the other one on its SM), or with five and more steps; up to four where they have their SMs to
+// themselves (a tenth may share), or with more than five steps.  us, layers, S = 3 / 4 / 5 / 8: 8 x 5120 -> 5120 (20 steps) 15.35 / 14.5 /
+// 15.0 / 15.2, 16 x 4096 -> 1024 (16) 12.0 / 10.0 / 10.2 / 10.8, 16 x 2048 -> 6144 (8) 8.06 / 8.36, 8 x 8192 -> 2048 (32) 28.0 / 27.1 / 26.4 / 24.4,
+// 16 x 7168 -> 4096 (28), S = 4 / 6 23.25 / 22.3, 16 x 5120 -> 8192, S = 3 / 4 16.5 / 17.1; up to 4 tokens sharing costs less (1 x 5120 -> 5120
+// S = 4 / 5 14.4 / 14.3).  One or two steps are not split (16 tokens, N = 4096, K = 512 2.97 / 2.56), nor are four above 16 tokens (32 tokens
+// N = 8192, K = 1024 4.6 / 3.7).
+static int push_gemm_cluster(int64_t M, int64_t tiles, int64_t steps, const DeviceState* st) {
+  if (steps >= 8) {                          // few tiles: as many CTAs as have two steps, see fewtok_gemm_cluster
+    const int S = fewtok_cluster(tiles, steps, steps / 2, 2, st->sm_count, st->few_fit);
+    if (tiles * S * fewtok_ntok(M) <= (M > 16 ? 32 : 8) * (int64_t)st->sm_count) return S;
+  }
+  if (steps <= 2 || (M > 16 && steps <= 4 && tiles > 24)) return 1;
+  for (int S = GemmFewCfg<>::MAX_CLUSTER; S > 1; --S) {
+    if (S > steps || tiles > st->push_fit[S]) continue;
+    const bool alone = 10 * tiles * S <= 11 * (int64_t)st->sm_count;
+    if (S > 4 ? (steps >= 4 * S && (alone || M <= 4)) || 2 * steps >= 9 * S : alone || steps > 5 * S) {
+      while (S > 1 && (steps + S - 2) / (S - 1) == (steps + S - 1) / S) --S;
+      return S;
+    }
+  }
+  return 1;
+}
 static int fewtok_gemm_cluster(int ntok, int64_t tiles, int64_t steps, int ctas, const DeviceState* st) {
   const int S = fewtok_cluster(tiles, steps, steps / 2, ctas, st->sm_count, st->few_fit);
   if (tiles * S * ntok <= (ntok > 16 ? 32 : 8) * (int64_t)st->sm_count) return S;
@@ -620,14 +659,14 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
   if (d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT) {
     int few_steps = 0, few_S = 0;                          // longest K range and cluster of the few-token kernel
     if (M <= kRotFewMaxTokens) {
-      few_S = fewtok_rotation(M, d, st).cluster;
+      few_S = fewtok_rotation(M, d, R_intra != nullptr, st).cluster;
       few_steps = (int)((d / 64 + few_S - 1) / few_S);
     }
     const int width = wide_rotation_width(M, d, few_steps, few_S, st->rot_pairs);
     if (width > 0) return rotate_wide(st, fmt, X, R_inter, R_intra, M, d, codes, scales, tensor_scale, width, s);
   }
   if (M <= kRotFewMaxTokens && d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT)
-    return rotate_fewtok(st, fmt, X, R_inter, R_intra, M, d, 0, (int)(d / 128), fewtok_rotation(M, d, st), codes, scales, tensor_scale, s);
+    return rotate_fewtok(st, fmt, X, R_inter, R_intra, M, d, 0, (int)(d / 128), fewtok_rotation(M, d, R_intra != nullptr, st), codes, scales, tensor_scale, s);
   if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d * x_terms, 128, 64) ||
       !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 64))
     return TORQ_ERR_LAUNCH;
@@ -841,12 +880,12 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
   // persistent pair kernels do better, half empty as their rows are (us, few-token against pairs: 100 tokens K = 4096,
   // N = 20480 20.4 / 12.9, N = 28672 21.4 / 16.3, N = 14336 10.9 / 11.1; 64 tokens, two CTAs per SM: K = 2048, N = 40960
   // 15.3 / 12.9, K = 4096, N = 28672 14.4 / 16.0; 40 tokens K = 5120, N = 51200 29.7 / 30.1).
-  const bool many_waves = M > 48 && (int64_t)tiles > (int64_t)FC::ctas_per_sm((int)M) * st->sm_count;
+  const bool many_waves = M > 48 && (int64_t)tiles > (int64_t)FC::ctas_per_sm((int)M, (int)K) * st->sm_count;
   if (ntok > 0 && !many_waves) {
     // Few tokens: 128 output features x all tokens per CTA, K split over a cluster, reduced through
     // distributed shared memory.
     const int64_t steps = (K + FC::BK - 1) / FC::BK;
-    const int S = fewtok_gemm_cluster(ntok, tiles, steps, FC::ctas_per_sm((int)M), st);
+    const int S = FC::push((int)M, (int)K) ? push_gemm_cluster(M, tiles, steps, st) : fewtok_gemm_cluster(ntok, tiles, steps, FC::ctas_per_sm((int)M, (int)K), st);
     const int width = M > 16 ? wide_gemm_width(M, N, steps, S, st->gemm_pairs) : 0;
     if (width > 0) return gemm_wide<FMT>(st, Aq, As, Wq, Ws, M, N, K, Y, y_dtype, alpha, width, s);
     if (!encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, 128, 128) ||
@@ -855,9 +894,9 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
     // up to 16 tokens: partials pushed; up to 64: one set of epilogue warps, two CTAs per SM; more: two sets.  65 to 80 tokens in
     // MXINT4 fit twice on an SM as well, and share it only where that gives them more K splits (us, shared / alone, 72 tokens:
     // N = 768, K = 3072 4.9 / 4.4, N = 1536 6.0 / 5.1, S = 8 either way; N = 6144, K = 4096, S = 4 and 1: 9.1 / 9.9).
-    const bool small = FC::ctas_per_sm((int)M) >= 2 && (ntok <= 64 || S > fewtok_gemm_cluster(ntok, tiles, steps, 1, st));
-    launch_tc(FC::push((int)M) ? gemm_fewtok_kernel<FMT, 1, true> : (small ? gemm_fewtok_kernel<FMT, 1> : gemm_fewtok_kernel<FMT, 2>),
-              S, tiles * S, small ? 192 : 320, FC::smem_bytes((int)M), s, tmB, tmA, static_cast<const uint8_t*>(As),
+    const bool small = FC::ctas_per_sm((int)M, (int)K) >= 2 && (ntok <= 64 || S > fewtok_gemm_cluster(ntok, tiles, steps, 1, st));
+    launch_tc(FC::push((int)M, (int)K) ? gemm_fewtok_kernel<FMT, 1, true> : (small ? gemm_fewtok_kernel<FMT, 1> : gemm_fewtok_kernel<FMT, 2>),
+              S, tiles * S, small ? 192 : 320, FC::smem_bytes((int)M, (int)K), s, tmB, tmA, static_cast<const uint8_t*>(As),
               static_cast<const uint8_t*>(Ws), Y, y_dtype == TORQ_BF16 ? 1 : 0, (int)M, (int)N, (int)K, ntok, S, kAheadTiles / (tiles * S), alpha, st->err_word);
     return launch_status();
   }
