@@ -138,23 +138,11 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   griddep_launch_dependents();
-  // While the kernel before ends HBM idles: the L2 is asked for W beyond the stages, as in the rotation (us, without / with, layers: 128 x
-  // 4096 -> 6144 19.4 / 19.0, 100 x 4096 -> 12288 21.9 / 21.7, 16 x 8192 -> 8192 29.65 / 29.5).
-  if (warp == 3 && elect_one())
-    for (int kt = kt0 + pre; kt < min(kt1, kt0 + pre + w_ahead); ++kt) tma_prefetch_l2_2d(&tmW, kt * 128, nt * C::BF);
-  __syncwarp();
-  griddep_wait();
-  // The activations of the first stages go out from four warps at once: one warp needs 0.2 us from one stage to the next.
-  const int a_pre = PUSH ? pre : 0;
-#pragma unroll
-  for (int it = 0; it < 4; ++it)
-    if (PUSH && warp == 2 + it && it < pre && elect_one()) {
-      const uint32_t st = smem_base + it * stage_bytes;
-      tma_load_2d(st + C::A_BYTES, &tmA, (kt0 + it) * 128, 0, full_bar(it));
-      bulk_load_1d(st + C::A_BYTES + b_bytes + C::SF_BYTES, As + (size_t)(CH * (kt0 + it)) * 512,
-                   512u * (uint32_t)min(CH, kb4 - CH * (kt0 + it)), full_bar(it));
-    }
-  __syncwarp();
+  const int a_pre = PUSH ? pre : 0;                      // activation tiles that the epilogue warps send
+  // While the kernel before ends HBM idles: from an epilogue warp the L2 is asked for W beyond the stages.  Not for pulled sums up to 64
+  // tokens, where the instructions alone cost more (us, 18 tokens N = 4096, K = 2048 3.46 / 3.56).
+  constexpr bool kAsk = PUSH || ESETS == 2;
+  if (!kAsk || warp < 2) griddep_wait();
 
   bool acc_ok = false;
   if (warp == 0) {
@@ -230,6 +218,22 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     __syncwarp();
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..5)
+    // us, without / with, layers: 128 x 4096 -> 6144 19.05 / 18.8, 100 x 4096 -> 12288 21.9 / 21.6, 16 x 8192 -> 8192 29.65 / 29.5.
+    if constexpr (kAsk) {
+      if (warp == 3 && elect_one())
+        for (int kt = kt0 + pre; kt < min(kt1, kt0 + pre + w_ahead); ++kt) tma_prefetch_l2_2d(&tmW, kt * 128, nt * C::BF);
+      __syncwarp();
+      griddep_wait();
+    }
+    // The activations of the first stages go out from four warps at once: one warp needs 0.2 us from one stage to the next.
+    if (PUSH && warp - 2 < pre && elect_one()) {
+      const int it = warp - 2;
+      const uint32_t st = smem_base + it * stage_bytes;
+      tma_load_2d(st + C::A_BYTES, &tmA, (kt0 + it) * 128, 0, full_bar(it));
+      bulk_load_1d(st + C::A_BYTES + b_bytes + C::SF_BYTES, As + (size_t)(CH * (kt0 + it)) * 512,
+                   512u * (uint32_t)min(CH, kb4 - CH * (kt0 + it)), full_bar(it));
+    }
+    __syncwarp();
     // Two passes over the SAME instructions, as in the few-token rotation: pass 0 is a dry run while the
     // mainloop streams (reads this CTA's own shared memory, stores nothing) so that the reduction's code is
     // in the instruction cache when it is needed; pass 1: accumulator -> partials, then the tokens of this CTA.

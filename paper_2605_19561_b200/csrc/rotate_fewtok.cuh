@@ -170,24 +170,8 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
       *reinterpret_cast<uint4*>(r_s + (piece >> 2) * 80 + (piece & 3) * 16) = __ldg(src + piece);
     }
   }
-  // X is not a constant, but asking the L2 for it changes nothing that a later load sees: one box per CTA until the K range is out
-  // So does asking for R_inter beyond the stages: until X has come the stages stay full and HBM idle.
-  if (warp == 2 && elect_one())
-    for (int kt = kt0 + ft - ft0; kt < kt1; kt += gridDim.x / S) tma_prefetch_l2_2d(&tmX, kt * C::BK, 0);
-  if (warp == 3 && elect_one())
-    for (int kt = kt0 + pre; kt < min(kt1, kt0 + pre + r_ahead); ++kt) {
-      tma_prefetch_l2_2d(&tmR, ft * C::BF, kt * C::BK);
-      tma_prefetch_l2_2d(&tmR, ft * C::BF + 64, kt * C::BK);
-    }
-  griddep_wait();
-  // The X tiles of the first stages go out from four warps at once: one warp needs 0.2 us from one stage to the next.  (PUSH only:
-  // elsewhere these warps may still wait for R_intra.  100 tokens, d = 8192: the layer 34.8 / 35.3.)
-  const int x_pre = !PUSH ? 0 : (pre < 4 ? pre : 4);
-#pragma unroll
-  for (int it = 0; it < 4; ++it)
-    if (PUSH && warp == 2 + it && it < x_pre && elect_one())
-      tma_load_2d(smem_base + it * stage_bytes + C::A_BYTES, &tmX, (kt0 + it) * C::BK, 0, full_bar(it));
-  __syncwarp();
+  const int x_pre = !PUSH ? 0 : (pre < 4 ? pre : 4);     // X tiles that the epilogue warps send
+  if (warp < 2) griddep_wait();
 
   bool acc_ok = false;                                   // epilogue warps: the accumulator is complete
   if (warp == 0) {
@@ -238,6 +222,22 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
     __syncwarp();
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..5)
+    // X is not a constant, but asking the L2 for it changes nothing that a later load sees: one box per CTA until the K range is out.
+    // So does asking for R_inter beyond the stages: until X has come the stages stay full and HBM idle.
+    if (warp == 2 && elect_one())
+      for (int kt = kt0 + ft - ft0; kt < kt1; kt += gridDim.x / S) tma_prefetch_l2_2d(&tmX, kt * C::BK, 0);
+    if (warp == 3 && elect_one())
+      for (int kt = kt0 + pre; kt < min(kt1, kt0 + pre + r_ahead); ++kt) {
+        tma_prefetch_l2_2d(&tmR, ft * C::BF, kt * C::BK);
+        tma_prefetch_l2_2d(&tmR, ft * C::BF + 64, kt * C::BK);
+      }
+    __syncwarp();
+    griddep_wait();
+    // The X tiles of the first stages go out from four warps at once: one warp needs 0.2 us from one stage to the next.  (PUSH only:
+    // elsewhere these warps may still wait for R_intra.  100 tokens, d = 8192: the layer 34.8 / 35.3.)
+    if (PUSH && warp - 2 < x_pre && elect_one())
+      tma_load_2d(smem_base + (warp - 2) * stage_bytes + C::A_BYTES, &tmX, (kt0 + warp - 2) * C::BK, 0, full_bar(warp - 2));
+    __syncwarp();
     // Two passes over the SAME instructions.  Pass 0 is a dry run while the mainloop streams: it reads
     // this CTA's own shared memory (whatever it holds), computes, and stores nothing.  Its only purpose
     // is to have the reduction's code in the instruction cache: executed cold, after the mainloop,
