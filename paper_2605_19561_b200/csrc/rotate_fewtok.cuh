@@ -11,7 +11,7 @@
 // contracts k range r.  The fp32 partial tiles never leave the SMs: every output has one CTA of the cluster that owns it, adds the S
 // partials in rank order (fixed order, so the result does not depend on timing), rotates inside the block and quantizes (Eq. 1).
 // The partials reach the owner in one of two ways:
-//  * PUSH (up to 32 tokens): the pieces of work are small, 32 features x 4 tokens, and dealt over all CTAs and warps of the cluster, so that
+//  * PUSH (up to 32 tokens, with R_intra and clusters of eight up to 56): the pieces of work are small, 32 features x 4 tokens, and dealt over all CTAs and warps of the cluster, so that
 //    nearly every warp has one and no CTA takes in more than its share (what arrives at one SM comes at about 9 B per cycle).  A CTA
 //    stores its partials straight from registers into the owners' shared memory (st.async, 16 bytes per lane = four tokens of one
 //    feature, counted on a barrier of the owning warp), into room of their own: nobody has to say first that the stages there are free, and
@@ -35,7 +35,7 @@
 // 14.8 -> 14.3, d = 4096, N = 6144, 200 tokens 22.4 -> 21.7.
 //
 // Roles per CTA: warp 0 TMA producer, warp 1 MMA issuer, warps 2..5 epilogue / reduction.
-// Shared memory: 4 stages (5 up to 16 tokens) of (16 KiB of R_inter + tokens x 128 B of X); pulled partials lie in
+// Shared memory: 4 stages (5 up to 16 tokens, 3 where more than 32 push) of (16 KiB of R_inter + tokens x 128 B of X); pulled partials lie in
 // the same memory after the mainloop, pushed ones behind it.  Up to 64 tokens that is small enough (<= 107 KiB) for two CTAs per SM: the
 // grid may exceed the SM count, which keeps more loads in flight; above, one CTA fills an SM, or
 // up to 128 tokens two of them with three stages (fewtok_rotation).
@@ -56,7 +56,7 @@ struct RotFewCfg {
   // a CTA and too few loads in flight (the rule stands where the kernel is launched).
   static constexpr int SHARED_STAGES = 3, MAX_SHARED_TOK = 128;
   static constexpr int MAX_TOK = 256;                  // N of the instruction: a multiple of 16
-  static constexpr int MAX_PUSH_TOK = 32;
+  static constexpr int MAX_PUSH_TOK = 64;
   static constexpr int PART_BYTES = 32 * 16;           // pushed partial of a unit from one CTA: [feature of the block][4 tokens]
   static constexpr int Y_BYTES = 16 * 33 * 4;          // pull, per epilogue warp: 16 tokens x 32 features, row stride 33
   static constexpr int RI_BYTES = 32 * 80;             // per epilogue warp: R_intra[block] as bf16 rows of 80 bytes
@@ -66,17 +66,19 @@ struct RotFewCfg {
   __host__ __device__ static constexpr int stage_bytes(int ntok) { return A_BYTES + ntok * BK * 2; }
   // partials of the units that one CTA owns, from all CTAs, for any cluster size; then the y tile of each warp
   __host__ __device__ static constexpr int push_bytes(int ntok) { return (ntok + MAX_CLUSTER - 1) * PART_BYTES + 4 * PART_BYTES; }
-  __host__ __device__ static constexpr int smem_bytes(int ntok, int stages = STAGES) {
-    return stages * stage_bytes(ntok) + BAR_BYTES + (ntok <= MAX_PUSH_TOK ? push_bytes(ntok) : 4 * RI_BYTES) + 1024;
+  __host__ __device__ static constexpr int smem_bytes(int ntok, int stages, bool push) {
+    return stages * stage_bytes(ntok) + BAR_BYTES + (push ? push_bytes(ntok) : 4 * RI_BYTES) + 1024;
   }
-  __host__ __device__ static constexpr int ctas_per_sm(int ntok, int stages = STAGES) {
-    return smem_bytes(ntok, stages) <= 113 * 1024 ? 2 : 1;
+  __host__ __device__ static constexpr int ctas_per_sm(int ntok, int stages, bool push) {
+    return smem_bytes(ntok, stages, push) <= 113 * 1024 ? 2 : 1;
   }
-  __host__ __device__ static constexpr int max_smem_bytes() { return smem_bytes(MAX_TOK); }
+  __host__ __device__ static constexpr int max_smem_bytes() { return smem_bytes(MAX_TOK, STAGES, false); }
 };
 // what lies in the stages after the mainloop where partials are pulled: the partial tile (ntok x 512 B) and the y tiles
 static_assert(8 * RotFewCfg::Y_BYTES <= 4 * RotFewCfg::A_BYTES && RotFewCfg::BF * 4 <= RotFewCfg::STAGES * RotFewCfg::BK * 2, "reduction buffers");
-static_assert(RotFewCfg::ctas_per_sm(RotFewCfg::MAX_SHARED_TOK, RotFewCfg::SHARED_STAGES) == 2 &&
+static_assert(RotFewCfg::ctas_per_sm(16, RotFewCfg::PUSH_STAGES, true) == 2 && RotFewCfg::ctas_per_sm(32, RotFewCfg::STAGES, true) == 2 &&
+              RotFewCfg::ctas_per_sm(RotFewCfg::MAX_PUSH_TOK, RotFewCfg::SHARED_STAGES, true) == 2, "two CTAs per SM where sums are pushed");
+static_assert(RotFewCfg::ctas_per_sm(RotFewCfg::MAX_SHARED_TOK, RotFewCfg::SHARED_STAGES, false) == 2 &&
               4 * RotFewCfg::Y_BYTES + 80 * RotFewCfg::BF * 4 <= RotFewCfg::SHARED_STAGES * RotFewCfg::stage_bytes(80) &&
               4 * RotFewCfg::Y_BYTES + 128 * RotFewCfg::BF * 4 <= RotFewCfg::SHARED_STAGES * RotFewCfg::stage_bytes(128), "three stages");
 
@@ -275,32 +277,38 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
       const int w = q;                                   // its number among the four: with S = 1 its own features are its units
       const uint32_t recv_base = smem_u32(ri_tiles);
       const uint32_t y_tile = recv_base + (uint32_t)(C::push_bytes(ntok) - 4 * C::PART_BYTES + w * C::PART_BYTES);
-      // where this warp's partials go: block q, tokens 4 c ... (worked out before they are needed: a division takes as long as a store)
-      uint32_t dst[C::MAX_PUSH_TOK / 4], dst_bar[C::MAX_PUSH_TOK / 4];
-#pragma unroll
-      for (int c = 0; c < C::MAX_PUSH_TOK / 4; ++c) {
-        const int u = q + 4 * c, ui = u / S, owner = u - ui * S;
-        dst[c] = map_to_cta(recv_base + (uint32_t)((ui * S + rank) * C::PART_BYTES + lane * 16), (uint32_t)owner);
-        dst_bar[c] = map_to_cta(recv_bar(ui & 3), (uint32_t)owner);
-      }
+      const int ui0 = q / S, owner0 = q - ui0 * S;       // of piece 0 (a division takes as long as a store: not between the stores)
       if (S > 1) cluster_wait();
 #pragma unroll 1
       for (int pass = rank + S * w < units ? 0 : 1; pass < 2; ++pass) {
         const bool live = pass == 1;
-        uint32_t v[C::MAX_PUSH_TOK];
         if (live) {
           acc_ok = mbar_wait(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
           acc_ok = __all_sync(0xFFFFFFFFu, acc_ok);
           bool ok = acc_ok;
           if (!ok) break;
           tc_fence_after_sync();
-          tmem_ld_32x32_x16(tacc, *reinterpret_cast<uint32_t(*)[16]>(v));
-          if (ntok > 16) tmem_ld_32x32_x16(tacc + 16, *reinterpret_cast<uint32_t(*)[16]>(v + 16));
-          tmem_ld_wait();
-          if (S > 1) {
+          int ui = ui0, owner = owner0;
+#pragma unroll 1
+          for (int c0 = 0; c0 < M; c0 += 16) {
+            uint32_t v[16];
+            tmem_ld_32x32_x16(tacc + c0, v);
+            tmem_ld_wait();
 #pragma unroll
-            for (int c = 0; c < C::MAX_PUSH_TOK / 4; ++c)
-              if (4 * c < M) st_async_v4(dst[c], v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3], dst_bar[c]);
+            for (int c = 0; c < 4; ++c) {
+              const uint32_t slot = recv_base + (uint32_t)((ui * S + rank) * C::PART_BYTES + lane * 16);
+              if (c0 + 4 * c >= M) break;
+              if (S > 1)
+                st_async_v4(map_to_cta(slot, (uint32_t)owner), v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3],
+                            map_to_cta(recv_bar(ui & 3), (uint32_t)owner));
+              else                                       // S = 1: this warp's own units
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(slot), "r"(v[4 * c]), "r"(v[4 * c + 1]), "r"(v[4 * c + 2]),
+                             "r"(v[4 * c + 3]) : "memory");
+              owner += 4;                                // the unit four further on
+              while (owner >= S) { owner -= S; ++ui; }
+            }
+          }
+          if (S > 1) {
             if (rank + S * w >= units) break;            // nothing to receive
             ok = __all_sync(0xFFFFFFFFu, mbar_wait_cluster(recv_bar(w), 0, cta_abort, err_word, SITE_EPI_ACC_FULL));
           }
@@ -310,25 +318,16 @@ rotate_fewtok_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
         for (int u = rank + S * w, ui = w; u < units; u += 4 * S, ui += 4) {
           const int c = u >> 2, blk_u = ft * 4 + (u & 3);
           float y[4] = {0.f, 0.f, 0.f, 0.f};             // of feature `lane` of the block, four tokens
-          if (S > 1) {
-            float4 part[C::MAX_CLUSTER];
+          float4 part[C::MAX_CLUSTER];
 #pragma unroll
-            for (int s = 0; s < C::MAX_CLUSTER; ++s)
-              if (s < S)
-                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                             : "=f"(part[s].x), "=f"(part[s].y), "=f"(part[s].z), "=f"(part[s].w)
-                             : "r"(recv_base + (uint32_t)((ui * S + s) * C::PART_BYTES + lane * 16)));
+          for (int s = 0; s < C::MAX_CLUSTER; ++s)
+            if (s < S)
+              asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                           : "=f"(part[s].x), "=f"(part[s].y), "=f"(part[s].z), "=f"(part[s].w)
+                           : "r"(recv_base + (uint32_t)((ui * S + s) * C::PART_BYTES + lane * 16)));
 #pragma unroll
-            for (int s = 0; s < C::MAX_CLUSTER; ++s)     // rank order: the result does not depend on timing
-              if (s < S) { y[0] += part[s].x; y[1] += part[s].y; y[2] += part[s].z; y[3] += part[s].w; }
-          } else if (live) {                             // S = 1: q = u % 4, the sums are this warp's own
-#pragma unroll
-            for (int cc = 0; cc < C::MAX_PUSH_TOK / 4; ++cc)
-              if (cc == c) {
-#pragma unroll
-                for (int t = 0; t < 4; ++t) y[t] = __uint_as_float(v[4 * cc + t]);
-              }
-          }
+          for (int s = 0; s < C::MAX_CLUSTER; ++s)       // rank order: the result does not depend on timing
+            if (s < S) { y[0] += part[s].x; y[1] += part[s].y; y[2] += part[s].z; y[3] += part[s].w; }
           float z[4] = {y[0], y[1], y[2], y[3]};
           if (R_intra != nullptr) {
             __syncwarp();

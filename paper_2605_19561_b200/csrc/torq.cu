@@ -136,13 +136,13 @@ static DeviceState* device_state() {
               opt_in_smem(rotate_quantize_kernel<256, FMT_MXINT4>, RotCfg<256>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_MXINT4>, RotPairCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_structured_kernel<FMT_MXINT4>, RotStructCfg::SMEM_BYTES) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true, RotFewCfg::PUSH_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true, RotFewCfg::PUSH_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 2>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true, RotFewCfg::PUSH_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true, RotFewCfg::PUSH_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 2>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true, RotFewCfg::PUSH_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
+              opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true, RotFewCfg::PUSH_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 2>, RotFewCfg::max_smem_bytes()) &&
               opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 1, true>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) && opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 1>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) &&
@@ -160,10 +160,10 @@ static DeviceState* device_state() {
                                      GemmPairCfgT<FMT_NVFP4>::SMEM_BYTES, st.sm_count);
     if (st.rot_pairs < 1 || st.gemm_pairs < 1) return nullptr;
     for (int s = 1; s <= RotFewCfg::MAX_CLUSTER; ++s)
-      st.few_fit[s] = max_active_clusters(rotate_fewtok_kernel<FMT_MXFP4, 2>, s, 320, RotFewCfg::smem_bytes(256), st.sm_count);
+      st.few_fit[s] = max_active_clusters(rotate_fewtok_kernel<FMT_MXFP4, 2>, s, 320, RotFewCfg::smem_bytes(256, RotFewCfg::STAGES, false), st.sm_count);
     for (int s = 1; s <= RotFewCfg::MAX_CLUSTER; ++s)
       st.push_fit[s] = max_active_clusters(fewtok_fit_kernel, s, RotFewCfg::THREADS,
-                                           RotFewCfg::smem_bytes(RotFewCfg::MAX_PUSH_TOK), st.sm_count);
+                                           RotFewCfg::smem_bytes(RotFewCfg::MAX_PUSH_TOK, RotFewCfg::SHARED_STAGES, true), st.sm_count);
     cudaGetLastError();
   }
   st.ready = true;
@@ -290,7 +290,9 @@ static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int64_t most, i
 // 1 token 14.8 / 14.3 / 14.25 / 14.4 / 15.7; of 192, 24 tokens d = 4096 NVFP4 3 / 4 / 6: 13.5 / 13.8 / 14.0; of 128, 100 tokens
 // d = 4096 0 / 3 / 5 / 8: 18.4 / 18.2 / 18.1 / 18.2).
 constexpr int kAheadTiles = 640;
-struct FewRotation { int cluster, stages; };
+constexpr int kPushTokens = 56;
+static_assert(kPushTokens <= RotFewCfg::MAX_PUSH_TOK, "room for pushed sums");
+struct FewRotation { int cluster, stages; bool push; };
 static FewRotation fewtok_rotation(int64_t M, int64_t d, bool intra, const DeviceState* st) {
   const int ntok = fewtok_ntok(M);
   const int64_t tiles = d / 128, steps = d / 64;
@@ -299,12 +301,15 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, bool intra, const Devic
   // 7.57 / 7.23 and 10.7 / 10.35 / 9.49, d = 4096 11.2 / 10.5 / 10.6 and 14.5 / 13.6 / 12.7; without the room d = 4224 (33 tiles) S = 7 /
   // 8 11.3 / 11.8, d = 7168 (56 tiles) S = 4 / 5 23.2 / 23.6.  A fifth stage up to 16 tokens, but not on long K ranges (four / five, 1 token:
   // layer d = N = 5120 14.5 / 14.3; rotation d = 14336 59.4 / 60.7).  A rotation without R_intra keeps the clusters of the rule below.
-  if (ntok <= RotFewCfg::MAX_PUSH_TOK && intra) {
+  // Above 32 tokens (three stages then) where clusters of eight fit, up to 56: us, layers, pulled / pushed, 40 tokens: 2048 -> 2048 10.65 / 10.1, 4096 ->
+  // 4096 15.85 / 15.1, 56 tokens 2560 -> 2560 13.25 / 12.15, 64 tokens 11.3 / 11.8 and 16.9 / 16.9; d = 5120, S = 6, 50 tokens 19.4 / 19.8.  Above 48
+  // from 20 tiles on (56 tokens NVFP4 2048 -> 2048 10.96 / 11.6).
+  if (intra && (M <= 32 || (M <= (tiles < 20 ? 48 : kPushTokens) && tiles <= st->push_fit[RotFewCfg::MAX_CLUSTER] - 2))) {
     int S = (int)(steps < RotFewCfg::MAX_CLUSTER ? steps : RotFewCfg::MAX_CLUSTER);
     while (S > 1 && tiles > st->push_fit[S] - 2) --S;
-    return {S, ntok <= 16 && steps <= 32 * S ? RotFewCfg::PUSH_STAGES : RotFewCfg::STAGES};
+    return {S, ntok > 32 ? RotFewCfg::SHARED_STAGES : (ntok <= 16 && steps <= 32 * S ? RotFewCfg::PUSH_STAGES : RotFewCfg::STAGES), true};
   }
-  const int long_k = ntok > 128 ? 1 : 10, ctas = RotFewCfg::ctas_per_sm(ntok);
+  const int long_k = ntok > 128 ? 1 : 10, ctas = RotFewCfg::ctas_per_sm(ntok, RotFewCfg::STAGES, ntok <= 32);
   // 17 to 64 tokens: two steps less are enough for one more CTA (us, S = 4 / 5 at 48 steps, d = 3072, 24 and 64 tokens: 8.4 /
   // 7.7 and 9.8 / 9.0, the layer with N = 3072 12.7 / 11.2 and 15.1 / 14.6; S = 5 / 6 at 58, d = 3712: 9.6 / 8.9 and 11.0 / 10.6)
   int64_t most = (steps + (ntok > 16 && ntok <= 64 ? 2 : 0)) / long_k;
@@ -314,9 +319,9 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, bool intra, const Devic
   // fit, 96 tokens lose (d = 3072 9.3 / 9.6).
   if (ntok > 64 && ntok <= 96 && steps >= 24 && tiles <= st->few_fit[6] && most < 6) most = 6;
   const int S = fewtok_cluster(tiles, steps, most, ctas, st->sm_count, st->few_fit);
-  if (ntok <= 16 && steps <= 32 * S) return {S, RotFewCfg::PUSH_STAGES};
-  if (ctas > 1 || ntok > RotFewCfg::MAX_SHARED_TOK || steps <= 32 * S) return {S, RotFewCfg::STAGES};
-  return {fewtok_cluster(tiles, steps, most, 2, st->sm_count, st->few_fit), RotFewCfg::SHARED_STAGES};
+  if (ntok <= 16 && steps <= 32 * S) return {S, RotFewCfg::PUSH_STAGES, true};
+  if (ctas > 1 || ntok > RotFewCfg::MAX_SHARED_TOK || steps <= 32 * S) return {S, RotFewCfg::STAGES, ntok <= 32};
+  return {fewtok_cluster(tiles, steps, most, 2, st->sm_count, st->few_fit), RotFewCfg::SHARED_STAGES, false};
 }
 // Whether the CTAs of a cluster leave together instead of each when it has no more to do.  Alone on their SMs (65 tokens and
 // more), clusters of 3 that nearly fill the GPCs (44 and 45 tiles, fit[3] = 45) hinder the clusters of the next kernel when
@@ -536,6 +541,8 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 //    (d = 2048 ... 2816, up to 192 tokens) this is a microsecond more than they take with cold operands, and the line lies between
 //    what cold ones and an R_inter in the L2 ask for (layers with N = d, few tokens / here: 144 x 2432 cold 0.95 of the time, in the
 //    L2 1.11; 152 x 2560 0.93 and 1.09, 176 x 2560 0.97 and 1.11, 176 x 2816 0.97 and 1.06, 112 x 2176 0.95 and 1.04);
+//  * few tokens whose sums are pushed: 2.7 + 0.22 per K step + 0.025 per token, 0.04 above 32 tokens (us, here / few tokens, 1, 16 and 32 tokens: d = 256 2.95 / 2.96, 2.95 /
+//    3.21, 2.95 / 4.49; d = 512 3.97 / 3.08, 3.37 / 3.21, 3.46 / 3.60; d = 768 5.25 / 3.21, 4.24 / 3.37, 4.36 / 3.85);
 //  * above 192 tokens a cluster of three has five units for its first CTA: 0.6 more (216 d = 4864 19.3 / 18.2);
 //  * above d = 6144, where these tiles take up to 3 us less than the figures say: 7.6 up to 192 tokens, 10.5 above, 0.42 per K step
 //    (144 d = 6912 26.9 / 25.4, 150 d = 7040 28.2 / 26.3, 208 d = 7680 33.1 / 30.0);
@@ -543,7 +550,7 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 // The other formats follow the same figures, which were not fitted to them; wide_gemm_width says how that was checked.
 // A layer of 2048 tokens and more fills the pair kernel's waves and stays there (one-wave tiles would be wider than
 // 384 columns; 2048 x 4096 measured 51.6 with 480 columns, 46.8 in the pair kernel).
-static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int few_S, int max_pairs) {
+static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int few_S, bool push, int max_pairs) {
   const int64_t rows = (M + 255) / 256, steps = d / 64;
   // The line of 65 to 96 tokens, clusters of six, stays where it was, and so does that of an X below 128 KiB (up to 64 tokens; with
   // more, an X so small has a d that comes here by either figures), which these tiles read more slowly for a reason not found (us, few
@@ -561,7 +568,8 @@ static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int few_S, i
   }
   double other;
   if (M <= kRotFewMaxTokens) {
-    if (M <= 16) other = 3.1 + 0.22 * few_steps;
+    if (push) other = 2.7 + 0.22 * few_steps + (M <= 32 ? 0.025 : 0.04) * (double)M;
+    else if (M <= 16) other = 3.1 + 0.22 * few_steps;
     else if (M <= 64) other = 4.4 + 0.2 * few_steps;
     else if (M <= 128) other = 5.6 + 0.36 * few_steps;
     else if (d > 6144) other = (M <= 192 ? 7.6 : 10.5) + 0.42 * few_steps;
@@ -606,24 +614,25 @@ static torq_status rotate_fewtok(DeviceState* st, int fmt, const void* X, const 
   if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d, (uint32_t)ntok, 64) ||
       !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 64))
     return TORQ_ERR_LAUNCH;
-  const int smem = RotFewCfg::smem_bytes(ntok, few.stages);
+  const int smem = RotFewCfg::smem_bytes(ntok, few.stages, few.push);
   const float ts = fmt == FMT_NVFP4 ? tensor_scale : 0.0f;
   const __nv_bfloat16* ri = static_cast<const __nv_bfloat16*>(R_intra);
   // up to 16 tokens: partials pushed to one CTA; two CTAs per SM: one set of epilogue warps; one CTA: two sets
-  auto launch = [&](auto push5, auto push, auto one, auto shared, auto two) {
-    const bool share = few.stages == RotFewCfg::SHARED_STAGES, small = share || RotFewCfg::ctas_per_sm(ntok) >= 2;
-    launch_tc(few.stages == RotFewCfg::PUSH_STAGES ? push5 : (ntok <= RotFewCfg::MAX_PUSH_TOK ? push : (share ? shared : (small ? one : two))), S, tiles * S, small ? 192 : 320, smem, s,
-              tmX, tmR, ri, codes, scales, (int)M, (int)d, ntok, S, ft0, fewtok_leave_together(M, tiles, few, st) ? 1 : 0, kAheadTiles / (tiles * S), ts, st->err_word);
+  auto launch = [&](auto push5, auto push4, auto push3, auto one, auto shared, auto two) {
+    const bool share = few.stages == RotFewCfg::SHARED_STAGES, small = few.push || share || ntok <= 64;
+    launch_tc(few.push ? (few.stages == RotFewCfg::PUSH_STAGES ? push5 : (share ? push3 : push4)) : (share ? shared : (small ? one : two)), S,
+              tiles * S, small ? 192 : 320, smem, s, tmX, tmR, ri, codes, scales, (int)M, (int)d, ntok, S, ft0,
+              fewtok_leave_together(M, tiles, few, st) ? 1 : 0, kAheadTiles / (tiles * S), ts, st->err_word);
   };
   constexpr int NS = RotFewCfg::SHARED_STAGES;
   if (fmt == FMT_MXINT4)
-    launch(rotate_fewtok_kernel<FMT_MXINT4, 1, true, RotFewCfg::PUSH_STAGES>, rotate_fewtok_kernel<FMT_MXINT4, 1, true>, rotate_fewtok_kernel<FMT_MXINT4, 1>, rotate_fewtok_kernel<FMT_MXINT4, 1, false, NS>,
+    launch(rotate_fewtok_kernel<FMT_MXINT4, 1, true, RotFewCfg::PUSH_STAGES>, rotate_fewtok_kernel<FMT_MXINT4, 1, true>, rotate_fewtok_kernel<FMT_MXINT4, 1, true, NS>, rotate_fewtok_kernel<FMT_MXINT4, 1>, rotate_fewtok_kernel<FMT_MXINT4, 1, false, NS>,
            rotate_fewtok_kernel<FMT_MXINT4, 2>);
   else if (fmt == FMT_NVFP4)
-    launch(rotate_fewtok_kernel<FMT_NVFP4, 1, true, RotFewCfg::PUSH_STAGES>, rotate_fewtok_kernel<FMT_NVFP4, 1, true>, rotate_fewtok_kernel<FMT_NVFP4, 1>, rotate_fewtok_kernel<FMT_NVFP4, 1, false, NS>,
+    launch(rotate_fewtok_kernel<FMT_NVFP4, 1, true, RotFewCfg::PUSH_STAGES>, rotate_fewtok_kernel<FMT_NVFP4, 1, true>, rotate_fewtok_kernel<FMT_NVFP4, 1, true, NS>, rotate_fewtok_kernel<FMT_NVFP4, 1>, rotate_fewtok_kernel<FMT_NVFP4, 1, false, NS>,
            rotate_fewtok_kernel<FMT_NVFP4, 2>);
   else
-    launch(rotate_fewtok_kernel<FMT_MXFP4, 1, true, RotFewCfg::PUSH_STAGES>, rotate_fewtok_kernel<FMT_MXFP4, 1, true>, rotate_fewtok_kernel<FMT_MXFP4, 1>, rotate_fewtok_kernel<FMT_MXFP4, 1, false, NS>,
+    launch(rotate_fewtok_kernel<FMT_MXFP4, 1, true, RotFewCfg::PUSH_STAGES>, rotate_fewtok_kernel<FMT_MXFP4, 1, true>, rotate_fewtok_kernel<FMT_MXFP4, 1, true, NS>, rotate_fewtok_kernel<FMT_MXFP4, 1>, rotate_fewtok_kernel<FMT_MXFP4, 1, false, NS>,
            rotate_fewtok_kernel<FMT_MXFP4, 2>);
   return launch_status();
 }
@@ -657,12 +666,13 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
   }
   CUtensorMap tmX, tmR;
   if (d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT) {
-    int few_steps = 0, few_S = 0;                          // longest K range and cluster of the few-token kernel
+    int few_steps = 0;                                     // longest K range of the few-token kernel
+    FewRotation few = {0, 0, false};
     if (M <= kRotFewMaxTokens) {
-      few_S = fewtok_rotation(M, d, R_intra != nullptr, st).cluster;
-      few_steps = (int)((d / 64 + few_S - 1) / few_S);
+      few = fewtok_rotation(M, d, R_intra != nullptr, st);
+      few_steps = (int)((d / 64 + few.cluster - 1) / few.cluster);
     }
-    const int width = wide_rotation_width(M, d, few_steps, few_S, st->rot_pairs);
+    const int width = wide_rotation_width(M, d, few_steps, few.cluster, few.push && R_intra != nullptr, st->rot_pairs);
     if (width > 0) return rotate_wide(st, fmt, X, R_inter, R_intra, M, d, codes, scales, tensor_scale, width, s);
   }
   if (M <= kRotFewMaxTokens && d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT)
@@ -690,7 +700,7 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
       tiles.total -= rest;
       const int S = fewtok_cluster(2 * rest, d / 64, d / 64, 1, st->sm_count, st->few_fit);
       const torq_status rc = rotate_fewtok(st, fmt, X, R_inter, R_intra, 256, d, (int)(d / 128) - 2 * rest, 2 * rest,
-                                           {S, RotFewCfg::STAGES}, codes, scales, tensor_scale, s);
+                                           {S, RotFewCfg::STAGES, false}, codes, scales, tensor_scale, s);
       if (rc != TORQ_OK) return rc;
     }
     const int pairs = tiles.total < max_pairs ? tiles.total : max_pairs;

@@ -1,4 +1,4 @@
-"""Few-token kernels whose partial sums are pushed in pieces of 32 features x 4 tokens (up to 32 tokens; the NVFP4 GEMM up to 24): token
+"""Few-token kernels whose partial sums are pushed in pieces of 32 features x 4 tokens (up to 32 tokens, the rotation with R_intra up to 56; the NVFP4 GEMM up to 24): token
 counts on both sides of every four, clusters of one CTA to eight, one and several pieces per warp.  Operands whose sums are exact in any
 order, so codes, scale bytes, padding and results must equal the oracle's bit for bit."""
 import numpy as np
@@ -18,7 +18,9 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("M,d", [(1, 128), (2, 256), (3, 19072), (4, 640), (5, 1536), (7, 2560), (8, 5120), (9, 4096), (12, 7168), (13, 9600),
                                  (16, 2048), (17, 128), (20, 14336), (21, 1536), (24, 4096), (28, 2560), (29, 896), (31, 640), (32, 5120),
-                                 (30, 19072)])
+                                 (30, 19072),
+                                 # three stages: 33 to 56 tokens in clusters of eight
+                                 (33, 1024), (36, 2048), (37, 3968), (45, 1536), (48, 2432), (49, 2560), (53, 3712), (56, 3072)])
 def test_rotation_of_permutations_in_the_three_formats(M, d):
     g = np.random.default_rng(M + d)
     xb = I.to_bf16_bits(g.integers(-8, 9, size=(M, d)).astype(np.float64))
@@ -45,7 +47,7 @@ def test_rotation_of_permutations_in_the_three_formats(M, d):
             g_codes, g_sb = gpu_quantized_to_numpy(codes, scales, M, d)
             assert np.array_equal(g_codes, o_codes) and np.array_equal(g_sb, o_sb)
             assert np.array_equal(scales.cpu().numpy(), O.swizzle_scales(o_sb, d, fill=0))       # padding rows hold zero
-            assert d < 1536 or "rotate_fewtok_kernelILi0ELi1ELb1E" in captured_launches(call)[0][0]
+            assert d < 1536 or f"rotate_fewtok_kernelILi0ELi1ELb{int(M <= 32 or width is not None)}E" in captured_launches(call)[0][0]
             byt, s = torq.torq_rotate_quantize_mxint4(X, P, Ri)
             torch.cuda.synchronize()
             o_q, o_sb = O.quantize_mxint4(z)
