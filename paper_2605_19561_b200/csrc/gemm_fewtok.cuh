@@ -139,10 +139,15 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   const uint32_t tmem_base = *tmem_slot;
   griddep_launch_dependents();
   const int a_pre = PUSH ? pre : 0;                      // activation tiles that the epilogue warps send
-  // While the kernel before ends HBM idles: from an epilogue warp the L2 is asked for W beyond the stages.  Not for pulled sums up to 64
-  // tokens, where the instructions alone cost more (us, 18 tokens N = 4096, K = 2048 3.46 / 3.56).
-  constexpr bool kAsk = PUSH || ESETS == 2;
-  if (!kAsk || warp < 2) griddep_wait();
+  // While the kernel before ends HBM idles: the L2 is asked for W beyond the stages (us, without / with, layers: 128 x 4096 -> 6144 19.05 / 18.8,
+  // 100 x 4096 -> 12288 21.9 / 21.6, 16 x 8192 -> 8192 29.65 / 29.5).  By a warp that has time for it, in its own branch: in the way of the
+  // epilogue warps' dry pass the instructions alone cost up to 3 % (56 x 2048 -> 2048 NVFP4 10.76 / 11.1).
+  auto ask = [&]() {
+    if (elect_one())
+      for (int kt = kt0 + pre; kt < min(kt1, kt0 + pre + w_ahead); ++kt) tma_prefetch_l2_2d(&tmW, kt * 128, nt * C::BF);
+    __syncwarp();
+  };
+  if (PUSH ? warp < 2 : warp != 1) griddep_wait();
 
   bool acc_ok = false;
   if (warp == 0) {
@@ -168,6 +173,10 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
+    if constexpr (!PUSH) {
+      ask();
+      griddep_wait();
+    }
     bool ok = true;
     const uint32_t idesc0 = FMT == FMT_NVFP4 ? idesc_nvf4(128, ntok) : idesc_mxf4(128, ntok, 0, 0);
     const uint32_t idesc2 = FMT == FMT_NVFP4 ? idesc_nvf4(128, ntok) : idesc_mxf4(128, ntok, 2, 2);
@@ -218,11 +227,8 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     __syncwarp();
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..5)
-    // us, without / with, layers: 128 x 4096 -> 6144 19.05 / 18.8, 100 x 4096 -> 12288 21.9 / 21.6, 16 x 8192 -> 8192 29.65 / 29.5.
-    if constexpr (kAsk) {
-      if (warp == 3 && elect_one())
-        for (int kt = kt0 + pre; kt < min(kt1, kt0 + pre + w_ahead); ++kt) tma_prefetch_l2_2d(&tmW, kt * 128, nt * C::BF);
-      __syncwarp();
+    if constexpr (PUSH) {
+      if (warp == 3) ask();
       griddep_wait();
     }
     // The activations of the first stages go out from four warps at once: one warp needs 0.2 us from one stage to the next.
