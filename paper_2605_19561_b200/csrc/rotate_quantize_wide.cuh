@@ -47,6 +47,11 @@ struct RotWideCfg {
   static constexpr int RI_BLOCK_BYTES = 32 * 64;       // R_intra[blk] as bf16 rows of 64 bytes, 16-byte pieces XOR-swizzled
   static constexpr int ESETS = 3;
   static constexpr int THREADS = 64 + 128 * ESETS;
+  // Tensor memory behind the accumulator, for the intra rotation of one block per set of warps: the result, 32 columns, and the third split
+  // term, 16.  Beside 384 columns there is room for two sets.
+  __host__ __device__ static constexpr int sets(int width) { return width + 48 * ESETS <= 512 ? ESETS : 2; }
+  __host__ __device__ static constexpr int out_col(int width, int set) { return width + 32 * set; }
+  __host__ __device__ static constexpr int lo_col(int width, int set) { return width + 32 * sets(width) + 16 * set; }
   // columns of the first instruction; the second takes the rest
   __host__ __device__ static constexpr int n0(int width) { return width <= 256 ? width : width - 128; }
   __host__ __device__ static constexpr int boxes(int width) { return (n0(width) / 2 + 63) / 64 + (width > 256 ? 1 : 0); }
@@ -88,6 +93,9 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   auto empty_bar = [&](int s) { return bar_base + 8u * (C::MAX_STAGES + s); };
   const uint32_t accf_bar = bar_base + 8u * (2 * C::MAX_STAGES);
   const uint32_t alloc_bar = accf_bar + 8;             // in the leader: the other CTA's tensor memory is allocated
+  auto term_bar = [&](int set) { return accf_bar + 16u + 8u * set; };              // in the leader: both CTAs' split terms of a block
+  const uint32_t ri_bar = accf_bar + 16 + 16 * C::ESETS;                           // in the leader: R_intra is in both CTAs' shared memory
+  auto rot_bar = [&](int set) { return accf_bar + 16u + 8u * (C::ESETS + set); };  // the rotated block
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + bar_off + 192);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(smem_gen + bar_off + 200);
 
@@ -100,6 +108,8 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   constexpr bool TWO = RANGE > 256;
   const int k_tiles = d / BK;
   const int n0 = C::n0(width);
+  const int nb = min(width / 32, d / 32 - (tcol >> 5));            // 32-blocks of this tile that exist
+  const int sets = C::sets(width);
 
   // Set-up as in the pair kernels: the producer waits for nothing but the barriers of both CTAs, and the first stages' X loads
   // come from a warp of their own (us, before / after: 200 x 1024 5.25 / 4.87, 200 x 2048 9.35 / 8.42, 300 x 4096 19.2 / 18.5).
@@ -107,6 +117,8 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
     for (int s = 0; s < nst; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     mbar_init(accf_bar, 1);
     mbar_init(alloc_bar, 1);
+    for (int i = 0; i < C::ESETS; ++i) { mbar_init(term_bar(i), 8); mbar_init(rot_bar(i), 1); }
+    mbar_init(ri_bar, 2);
     *cta_abort = 0;
     fence_mbar_init();
   }
@@ -187,15 +199,31 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
         if (++s == nst) { s = 0; ph ^= 1; }
       }
       if (ok) tc_commit_pair(accf_bar, 3);          // accumulator ready in both CTAs
+      // Intra-block rotation: block bb by set bb % sets, three split terms x 32 of K, terms and result in tensor memory.
+      constexpr uint32_t idesc_r = idesc_bf16(256, 32, false, true);
+      if (R_intra != nullptr && ok) ok = mbar_wait_cluster(ri_bar, 0, cta_abort, err_word, SITE_MMA_FULL);
+      for (int bb = 0, set = 0, r = 0; R_intra != nullptr && ok && bb < nb; ++bb) {
+        ok = mbar_wait_cluster(term_bar(set), r & 1, cta_abort, err_word, SITE_MMA_FULL);
+        if (!ok) break;
+        tc_fence_after_sync();
+        const uint64_t rdesc = make_desc(smem_base + ri_off + bb * C::RI_BLOCK_BYTES, 2048, 512, kSwizzle64);
+        const uint32_t y = tmem_base + bb * 32, lo = tmem_base + C::lo_col(width, set), out = tmem_base + C::out_col(width, set);
+        mma_bf16_pair_tmem_a(out, lo, rdesc, idesc_r, 0);            // the smallest term first
+        mma_bf16_pair_tmem_a(out, lo + 8, rdesc + 64, idesc_r, 1);   // k 16 .. 31: +8 columns of terms, +16 rows of R_intra
+        mma_bf16_pair_tmem_a(out, y + 16, rdesc, idesc_r, 1);
+        mma_bf16_pair_tmem_a(out, y + 24, rdesc + 64, idesc_r, 1);
+        mma_bf16_pair_tmem_a(out, y, rdesc, idesc_r, 1);
+        mma_bf16_pair_tmem_a(out, y + 8, rdesc + 64, idesc_r, 1);
+        tc_commit_pair(rot_bar(set), 3);
+        if (++set == sets) { set = 0; ++r; }
+      }
     }
     __syncwarp();
   } else {
     // ------------------------------------------------------------------ epilogue (12 warps per CTA)
     const int q = warp & 3;
     const int set = (warp - 2) >> 2;
-    const int p = lane & 3, r8 = lane >> 2;
-    const int nblocks = d / 32, nb = width / 32, b0 = tcol >> 5;
-    const uint32_t ri_saddr = smem_base + ri_off;
+    const int nblocks = d / 32, b0 = tcol >> 5;
     if (warp == 3 && elect_one()) {
       // Until the kernel before has completed HBM idles.  In short calls the L2 is asked for the first K steps of X, one of each row tile
       // per pair that shares it, and, for strips of 64 to 128 columns, for the next R_inter, a strip's steps dealt over its row tiles (us,
@@ -216,51 +244,88 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
           tma_load_3d_pair(smem_base + i * stage_bytes, &tmX, 0, mt * C::BM, i * (BK / C::SLAB), map_to_cta(full_bar(i), 0));
       __syncwarp();
     }
-    if (R_intra != nullptr) {                          // the tile's blocks, 16-byte piece c of row i at c ^ ((i >> 1) & 3)
+    if (R_intra != nullptr) {
+      // The tile's blocks, rows of 64 bytes under the 64-byte swizzle: 16-byte piece c of row i at c ^ ((i >> 1) & 3).  This CTA's half of the
+      // instruction's 32 columns are the first 32 bytes of its rows: rank 1 holds its pieces two on.
       for (int idx = (warp - 2) * 32 + lane; idx < nb * 128; idx += 128 * C::ESETS) {
-        const int lb = idx >> 7, i = (idx >> 2) & 31, c = idx & 3;
-        if (b0 + lb < nblocks)
-          *reinterpret_cast<uint4*>(smem_gen + ri_off + lb * C::RI_BLOCK_BYTES + i * 64 + ((c ^ ((i >> 1) & 3)) << 4)) =
-              __ldg(reinterpret_cast<const uint4*>(R_intra + (size_t)(b0 + lb) * 1024) + (idx & 127));
+        const int lb = idx >> 7, i = (idx >> 2) & 31, c = (idx & 3) ^ (2 * (int)rank);
+        *reinterpret_cast<uint4*>(smem_gen + ri_off + lb * C::RI_BLOCK_BYTES + i * 64 + ((c ^ ((i >> 1) & 3)) << 4)) =
+            __ldg(reinterpret_cast<const uint4*>(R_intra + (size_t)(b0 + lb) * 1024) + (idx & 127));
       }
+      fence_proxy_async_smem();                        // visible to the tensor core's reads
       named_barrier_sync(1, 128 * C::ESETS);
+      if (warp == 2 && lane == 0) mbar_arrive_release_cluster(map_to_cta(ri_bar, 0));
     }
     griddep_wait();                                    // codes and scales may still be read by that kernel
     bool ok = mbar_wait_cluster(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);
     ok = __all_sync(0xFFFFFFFFu, ok);
     tc_fence_after_sync();
-    const uint32_t tacc = tmem_base + ((uint32_t)(q * 32) << 16);
-    if (ok && mt * C::BM < M) {                        // the pair's second row tile may not exist
-      NvScale nvs = {};
-      if constexpr (FMT == FMT_NVFP4) nvs = nv_scale(tensor_scale);
-      const int kb4 = FMT == FMT_NVFP4 ? (2 * nblocks + 3) / 4 : (nblocks + 3) / 4;
-      // ldmatrix: lane l addresses row l % 8 (+ 8 for odd l / 8) of its matrix, 16-byte piece l / 16 (+ 2)
-      const int li = ((lane >> 3) & 1) * 8 + (lane & 7);
-      const uint32_t r_lane = (uint32_t)li * 64 + (uint32_t)(((lane >> 4) ^ ((li >> 1) & 3)) << 4);
-      // units of 16 rows x 32 columns: unit u is half u % 2 of the warp's rows of block u / 2
+    const uint32_t tlane = tmem_base + ((uint32_t)(q * 32) << 16);
+    const int64_t row = (int64_t)mt * C::BM + q * 32 + lane;
+    const bool live = mt * C::BM + q * 32 < M;         // warp-uniform: else this warp only makes its arrivals
+    NvScale nvs = {};
+    if constexpr (FMT == FMT_NVFP4) nvs = nv_scale(tensor_scale);
+    const int kb4 = FMT == FMT_NVFP4 ? (2 * nblocks + 3) / 4 : (nblocks + 3) / 4;
+    const uint32_t term_leader = map_to_cta(term_bar(set), 0);
+    // A warp takes 32 rows of a block, one row per lane.  y goes back to tensor memory as hi + mid + lo (bf16, exact): hi and mid over y itself,
+    // lo in columns of the set's own, where the result comes as well.
+    uint32_t ph = 0;
 #pragma unroll 1
-      for (int u = set; u < 2 * nb; u += C::ESETS) {
-        const int bb = u >> 1, mh = u & 1, blk = b0 + bb;
-        if (blk >= nblocks) break;
-        uint32_t y[16];
-        tmem_ld_16x256b_x4(tacc + ((uint32_t)(16 * mh) << 16) + bb * 32, y);
+    for (int bb = set; ok && set < sets && bb < nb; bb += sets) {
+      const int blk = b0 + bb;
+      uint32_t y[32];
+      if (live) {
+        tmem_ld_32x32(tlane + bb * 32, y);
         tmem_ld_wait();
-        IntraFrag f;
-        const uint32_t rb = ri_saddr + (uint32_t)bb * C::RI_BLOCK_BYTES + r_lane;
-        if (R_intra != nullptr) load_intra_frag(rb, rb ^ 32u, 16 * 64, f);
-        uint32_t sb[2];
-        intra_quantize_frag16<FMT>(y, R_intra != nullptr, f, lane, (int64_t)mt * C::BM + q * 32 + 16 * mh, M, blk, nblocks, d, nvs,
-                                   codes, sb);
-        if (p == 0) {                                  // byte blk % 4 of the 4-byte cell of (row, blk / 4)
+      }
+      if (R_intra != nullptr) {
+        if (live) {
+          uint32_t hi[16], mid[16], lo[16];
 #pragma unroll
-          for (int rh = 0; rh < 2; ++rh) {
-            const size_t in_tile = (size_t)(r8 + 16 * mh + 8 * rh) * 16 + q * 4;
-            if constexpr (FMT == FMT_NVFP4)
-              *reinterpret_cast<uint16_t*>(scales + ((size_t)mt * kb4 + (blk >> 1)) * 512 + in_tile + 2 * (blk & 1)) = (uint16_t)sb[rh];
-            else
-              scales[((size_t)mt * kb4 + (blk >> 2)) * 512 + in_tile + (blk & 3)] = (uint8_t)sb[rh];
+          for (int e = 0; e < 16; ++e) split3_trunc_bf16x2(y[2 * e], y[2 * e + 1], hi[e], mid[e], lo[e]);
+          tmem_st_32x32_x16(tlane + bb * 32, hi);
+          tmem_st_32x32_x16(tlane + bb * 32 + 16, mid);
+          tmem_st_32x32_x16(tlane + C::lo_col(width, set), lo);
+          tmem_st_wait();
+        }
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(term_leader);
+        ok = mbar_wait_cluster(rot_bar(set), ph, cta_abort, err_word, SITE_EPI_ACC_FULL);
+        ok = __all_sync(0xFFFFFFFFu, ok);
+        if (!ok) break;
+        ph ^= 1;
+        tc_fence_after_sync();
+        if (live) {
+          tmem_ld_32x32(tlane + C::out_col(width, set), y);
+          tmem_ld_wait();
+        }
+        tc_fence_before_sync();
+      }
+      if (live) {
+        float z[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) z[i] = __uint_as_float(y[i]);
+        uint4 cw, cw2;
+        uint32_t sbyte;
+        if constexpr (FMT == FMT_MXINT4) mxint4_quantize_block32(z, cw, cw2, sbyte);
+        else if constexpr (FMT == FMT_NVFP4) nv_quantize_2x16(z, nvs, cw, sbyte);
+        else quantize_block32(z, cw, sbyte);
+        if (row < M) {
+          if constexpr (FMT == FMT_MXINT4) {           // one operand byte per element
+            uint4* dst = reinterpret_cast<uint4*>(codes + row * (int64_t)d + (int64_t)blk * 32);
+            dst[0] = cw;
+            dst[1] = cw2;
+          } else {
+            *reinterpret_cast<uint4*>(codes + row * (int64_t)(d / 2) + (int64_t)blk * 16) = cw;
           }
         }
+        // rows past the last token of the 128-row scale tile: their sums are zero, and so is their byte
+        if constexpr (FMT == FMT_NVFP4) *reinterpret_cast<uint16_t*>(scales + scale_offset(row, 2 * blk, kb4)) = (uint16_t)sbyte;
+        else scales[scale_offset(row, blk, kb4)] = (uint8_t)sbyte;
+      } else if (mt * C::BM < M) {                     // a quarter without a token
+        if constexpr (FMT == FMT_NVFP4) *reinterpret_cast<uint16_t*>(scales + scale_offset(row, 2 * blk, kb4)) = 0;
+        else scales[scale_offset(row, blk, kb4)] = 0;
       }
     }
     tc_fence_before_sync();
