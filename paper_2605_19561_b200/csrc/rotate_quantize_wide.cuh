@@ -17,8 +17,13 @@
 //
 // Bounds: up to 128 columns the latency of the loads and of the hand-overs between the roles (440 cycles per 64 of K at 64
 // columns, 460 at 128 with stages of 64, where the instructions take 320 and 384; the same loads alone, from L2, run at 22
-// TB/s), above the instructions (500 at 256); then the epilogue, which nothing overlaps.  It is the fast form (warp-level MMAs on the accumulator fragments), bound by
-// those MMAs: about 860 cycles per 32 columns.  Splitting K over the pairs of a larger cluster (partial sums
+// TB/s), above the instructions (500 at 256); then the epilogue, which nothing overlaps.  The intra rotation in it runs as tcgen05
+// instructions of both CTAs, y split into three bf16 terms in tensor memory; a lane then holds one row of a block and quantizes it.  As warp-level
+// MMAs on the accumulator fragments it was bound by those, about 860 cycles per 32 columns (us, these / here: rotation 777 x 5120 44.8 / 42.5, 300 x
+// 2048 8.72 / 8.45, layers 600 x 2048 -> 2048 15.7 / 14.95, loops of 0.5 s 1024 x 4096 -> 4096 44.3 / 43.0).  Tiles of 32 columns keep that form: a unit
+// of 16 rows for each of eight warps is done before the hand-over to the issuer and back (200 x 2048 7.68 / 7.88, 256 x 1024 4.48 / 4.64).  Measured
+// no faster: the terms of a set's next block sent before the result of this one is waited for (777 x 5120 42.4 / 41.9, but 300 x 2048 8.45 / 8.69:
+// what a short call waits for is this code's instructions), and a warp that runs it once ahead (8.45 / 8.58).  Splitting K over the pairs of a larger cluster (partial sums
 // exchanged through distributed shared memory) was measured and brought nothing: 300 x 4096 20.9 with two pairs
 // per 256 columns against 21.2.
 //
@@ -71,8 +76,8 @@ static_assert(RotWideCfg::stages(128) <= RotWideCfg::MAX_STAGES && RotWideCfg::s
 
 // grid = 2 * rows * cols CTAs in clusters of two: pair p works row tile p % rows (256 tokens), column tile p / rows
 // (`width` features from column (p / rows) * width on).  tmX: X as (64 of K, token, slab of K), box [64 x 128 x slabs of a
-// stage]; tmR: R_inter box [BK of K x 64 columns]; tmRt: box [BK x tail_cols].  d % 128 == 0.  RANGE: 128, 256 or 384, the first
-// that is not below the width (two slabs of K per stage; one; two instructions per slice).  FMT, `tensor_scale` as in the pair
+// stage]; tmR: R_inter box [BK of K x 64 columns]; tmRt: box [BK x tail_cols].  d % 128 == 0.  RANGE: 32, 128, 256 or 384, the first
+// that is not below the width (two slabs of K per stage, one block; two slabs; one; two instructions per slice).  FMT, `tensor_scale` as in the pair
 // kernel.
 template <int FMT, int RANGE>
 __global__ void __launch_bounds__(RotWideCfg::THREADS, 1)
@@ -105,7 +110,7 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   const int tcol = (pair / rows) * width;
   const int mt = 2 * (pair % rows) + (int)rank;
   constexpr int BK = C::bk(RANGE), A_BYTES = C::a_bytes(RANGE), BOX_BYTES = C::box_bytes(RANGE);
-  constexpr bool TWO = RANGE > 256;
+  constexpr bool TWO = RANGE > 256, kTerms = RANGE > 32;           // kTerms: the intra rotation as tcgen05 instructions
   const int k_tiles = d / BK;
   const int n0 = C::n0(width);
   const int nb = min(width / 32, d / 32 - (tcol >> 5));            // 32-blocks of this tile that exist
@@ -201,8 +206,8 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       if (ok) tc_commit_pair(accf_bar, 3);          // accumulator ready in both CTAs
       // Intra-block rotation: block bb by set bb % sets, three split terms x 32 of K, terms and result in tensor memory.
       constexpr uint32_t idesc_r = idesc_bf16(256, 32, false, true);
-      if (R_intra != nullptr && ok) ok = mbar_wait_cluster(ri_bar, 0, cta_abort, err_word, SITE_MMA_FULL);
-      for (int bb = 0, set = 0, r = 0; R_intra != nullptr && ok && bb < nb; ++bb) {
+      if (kTerms && R_intra != nullptr && ok) ok = mbar_wait_cluster(ri_bar, 0, cta_abort, err_word, SITE_MMA_FULL);
+      for (int bb = 0, set = 0, r = 0; kTerms && R_intra != nullptr && ok && bb < nb; ++bb) {
         ok = mbar_wait_cluster(term_bar(set), r & 1, cta_abort, err_word, SITE_MMA_FULL);
         if (!ok) break;
         tc_fence_after_sync();
@@ -246,9 +251,9 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
     }
     if (R_intra != nullptr) {
       // The tile's blocks, rows of 64 bytes under the 64-byte swizzle: 16-byte piece c of row i at c ^ ((i >> 1) & 3).  This CTA's half of the
-      // instruction's 32 columns are the first 32 bytes of its rows: rank 1 holds its pieces two on.
+      // instruction's 32 columns are the first 32 bytes of its rows: rank 1 holds its pieces two on (kTerms).
       for (int idx = (warp - 2) * 32 + lane; idx < nb * 128; idx += 128 * C::ESETS) {
-        const int lb = idx >> 7, i = (idx >> 2) & 31, c = (idx & 3) ^ (2 * (int)rank);
+        const int lb = idx >> 7, i = (idx >> 2) & 31, c = (idx & 3) ^ (kTerms ? 2 * (int)rank : 0);
         *reinterpret_cast<uint4*>(smem_gen + ri_off + lb * C::RI_BLOCK_BYTES + i * 64 + ((c ^ ((i >> 1) & 3)) << 4)) =
             __ldg(reinterpret_cast<const uint4*>(R_intra + (size_t)(b0 + lb) * 1024) + (idx & 127));
       }
@@ -266,66 +271,91 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
     NvScale nvs = {};
     if constexpr (FMT == FMT_NVFP4) nvs = nv_scale(tensor_scale);
     const int kb4 = FMT == FMT_NVFP4 ? (2 * nblocks + 3) / 4 : (nblocks + 3) / 4;
-    const uint32_t term_leader = map_to_cta(term_bar(set), 0);
-    // A warp takes 32 rows of a block, one row per lane.  y goes back to tensor memory as hi + mid + lo (bf16, exact): hi and mid over y itself,
-    // lo in columns of the set's own, where the result comes as well.
-    uint32_t ph = 0;
-#pragma unroll 1
-    for (int bb = set; ok && set < sets && bb < nb; bb += sets) {
-      const int blk = b0 + bb;
-      uint32_t y[32];
-      if (live) {
-        tmem_ld_32x32(tlane + bb * 32, y);
+    if constexpr (!kTerms) {
+      // One block: a unit of 16 rows per warp of the first two sets, on accumulator fragments (tmem_ld_16x256b_x4) and warp-level MMAs.
+      const int p = lane & 3, r8 = lane >> 2, mh = set;
+      if (ok && set < 2 && nb > 0 && mt * C::BM < M) {
+        uint32_t y[16];
+        tmem_ld_16x256b_x4(tlane + ((uint32_t)(16 * mh) << 16), y);
         tmem_ld_wait();
-      }
-      if (R_intra != nullptr) {
-        if (live) {
-          uint32_t hi[16], mid[16], lo[16];
+        // ldmatrix: lane l addresses row l % 8 (+ 8 for odd l / 8) of its matrix, 16-byte piece l / 16 (+ 2)
+        const int li = ((lane >> 3) & 1) * 8 + (lane & 7);
+        const uint32_t rb = smem_base + ri_off + (uint32_t)li * 64 + (uint32_t)(((lane >> 4) ^ ((li >> 1) & 3)) << 4);
+        IntraFrag f;
+        if (R_intra != nullptr) load_intra_frag(rb, rb ^ 32u, 16 * 64, f);
+        uint32_t sb[2];
+        intra_quantize_frag16<FMT>(y, R_intra != nullptr, f, lane, (int64_t)mt * C::BM + q * 32 + 16 * mh, M, b0, nblocks, d, nvs, codes, sb);
+        if (p == 0) {                                  // byte b0 % 4 of the 4-byte cell of (row, b0 / 4)
 #pragma unroll
-          for (int e = 0; e < 16; ++e) split3_trunc_bf16x2(y[2 * e], y[2 * e + 1], hi[e], mid[e], lo[e]);
-          tmem_st_32x32_x16(tlane + bb * 32, hi);
-          tmem_st_32x32_x16(tlane + bb * 32 + 16, mid);
-          tmem_st_32x32_x16(tlane + C::lo_col(width, set), lo);
-          tmem_st_wait();
-        }
-        tc_fence_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(term_leader);
-        ok = mbar_wait_cluster(rot_bar(set), ph, cta_abort, err_word, SITE_EPI_ACC_FULL);
-        ok = __all_sync(0xFFFFFFFFu, ok);
-        if (!ok) break;
-        ph ^= 1;
-        tc_fence_after_sync();
-        if (live) {
-          tmem_ld_32x32(tlane + C::out_col(width, set), y);
-          tmem_ld_wait();
-        }
-        tc_fence_before_sync();
-      }
-      if (live) {
-        float z[32];
-#pragma unroll
-        for (int i = 0; i < 32; ++i) z[i] = __uint_as_float(y[i]);
-        uint4 cw, cw2;
-        uint32_t sbyte;
-        if constexpr (FMT == FMT_MXINT4) mxint4_quantize_block32(z, cw, cw2, sbyte);
-        else if constexpr (FMT == FMT_NVFP4) nv_quantize_2x16(z, nvs, cw, sbyte);
-        else quantize_block32(z, cw, sbyte);
-        if (row < M) {
-          if constexpr (FMT == FMT_MXINT4) {           // one operand byte per element
-            uint4* dst = reinterpret_cast<uint4*>(codes + row * (int64_t)d + (int64_t)blk * 32);
-            dst[0] = cw;
-            dst[1] = cw2;
-          } else {
-            *reinterpret_cast<uint4*>(codes + row * (int64_t)(d / 2) + (int64_t)blk * 16) = cw;
+          for (int rh = 0; rh < 2; ++rh) {
+            const int64_t rr = (int64_t)mt * C::BM + q * 32 + r8 + 16 * mh + 8 * rh;
+            if constexpr (FMT == FMT_NVFP4) *reinterpret_cast<uint16_t*>(scales + scale_offset(rr, 2 * b0, kb4)) = (uint16_t)sb[rh];
+            else scales[scale_offset(rr, b0, kb4)] = (uint8_t)sb[rh];
           }
         }
-        // rows past the last token of the 128-row scale tile: their sums are zero, and so is their byte
-        if constexpr (FMT == FMT_NVFP4) *reinterpret_cast<uint16_t*>(scales + scale_offset(row, 2 * blk, kb4)) = (uint16_t)sbyte;
-        else scales[scale_offset(row, blk, kb4)] = (uint8_t)sbyte;
-      } else if (mt * C::BM < M) {                     // a quarter without a token
-        if constexpr (FMT == FMT_NVFP4) *reinterpret_cast<uint16_t*>(scales + scale_offset(row, 2 * blk, kb4)) = 0;
-        else scales[scale_offset(row, blk, kb4)] = 0;
+      }
+    } else {
+      const uint32_t term_leader = map_to_cta(term_bar(set), 0);
+      // A warp takes 32 rows of a block, one row per lane.  y goes back to tensor memory as hi + mid + lo (bf16, exact): hi and mid over y itself,
+      // lo in columns of the set's own, where the result comes as well.
+      uint32_t ph = 0;
+#pragma unroll 1
+      for (int bb = set; ok && set < sets && bb < nb; bb += sets) {
+        const int blk = b0 + bb;
+        uint32_t y[32];
+        if (live) {
+          tmem_ld_32x32(tlane + bb * 32, y);
+          tmem_ld_wait();
+        }
+        if (R_intra != nullptr) {
+          if (live) {
+            uint32_t hi[16], mid[16], lo[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) split3_trunc_bf16x2(y[2 * e], y[2 * e + 1], hi[e], mid[e], lo[e]);
+            tmem_st_32x32_x16(tlane + bb * 32, hi);
+            tmem_st_32x32_x16(tlane + bb * 32 + 16, mid);
+            tmem_st_32x32_x16(tlane + C::lo_col(width, set), lo);
+            tmem_st_wait();
+          }
+          tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(term_leader);
+          ok = mbar_wait_cluster(rot_bar(set), ph, cta_abort, err_word, SITE_EPI_ACC_FULL);
+          ok = __all_sync(0xFFFFFFFFu, ok);
+          if (!ok) break;
+          ph ^= 1;
+          tc_fence_after_sync();
+          if (live) {
+            tmem_ld_32x32(tlane + C::out_col(width, set), y);
+            tmem_ld_wait();
+          }
+          tc_fence_before_sync();
+        }
+        if (live) {
+          float z[32];
+#pragma unroll
+          for (int i = 0; i < 32; ++i) z[i] = __uint_as_float(y[i]);
+          uint4 cw, cw2;
+          uint32_t sbyte;
+          if constexpr (FMT == FMT_MXINT4) mxint4_quantize_block32(z, cw, cw2, sbyte);
+          else if constexpr (FMT == FMT_NVFP4) nv_quantize_2x16(z, nvs, cw, sbyte);
+          else quantize_block32(z, cw, sbyte);
+          if (row < M) {
+            if constexpr (FMT == FMT_MXINT4) {           // one operand byte per element
+              uint4* dst = reinterpret_cast<uint4*>(codes + row * (int64_t)d + (int64_t)blk * 32);
+              dst[0] = cw;
+              dst[1] = cw2;
+            } else {
+              *reinterpret_cast<uint4*>(codes + row * (int64_t)(d / 2) + (int64_t)blk * 16) = cw;
+            }
+          }
+          // rows past the last token of the 128-row scale tile: their sums are zero, and so is their byte
+          if constexpr (FMT == FMT_NVFP4) *reinterpret_cast<uint16_t*>(scales + scale_offset(row, 2 * blk, kb4)) = (uint16_t)sbyte;
+          else scales[scale_offset(row, blk, kb4)] = (uint8_t)sbyte;
+        } else if (mt * C::BM < M) {                     // a quarter without a token
+          if constexpr (FMT == FMT_NVFP4) *reinterpret_cast<uint16_t*>(scales + scale_offset(row, 2 * blk, kb4)) = 0;
+          else scales[scale_offset(row, blk, kb4)] = 0;
+        }
       }
     }
     tc_fence_before_sync();

@@ -116,11 +116,11 @@ static DeviceState* device_state() {
               opt_in_smem(rotate_quantize_kernel<256, FMT_NVFP4>, RotCfg<256>::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_MXFP4>, RotPairCfg::SMEM_BYTES) &&
               opt_in_smem(rotate_quantize_pair_kernel<FMT_NVFP4>, RotPairCfg::SMEM_BYTES) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, 128>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, 256>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, 32>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, 128>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, 256>, kWideSmem) &&
               opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, 384>, kWideSmem) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, 128>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, 256>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, 32>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, 128>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, 256>, kWideSmem) &&
               opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, 384>, kWideSmem) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, 128>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, 256>, kWideSmem) &&
+              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, 32>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, 128>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, 256>, kWideSmem) &&
               opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, 384>, kWideSmem) &&
               opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXFP4, 128>, kWideSmem) && opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXFP4, 256>, kWideSmem) &&
               opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXFP4, 384>, kWideSmem) &&
@@ -594,13 +594,13 @@ static torq_status rotate_wide(DeviceState* st, int fmt, const void* X, const vo
     return TORQ_ERR_LAUNCH;
   if (!tail) tmRt = tmR;
   const int rows = (int)((M + 255) / 256), cols = (int)((d + width - 1) / width);
-  auto launch = [&](auto r128, auto r256, auto r384) {
-    launch_tc(width > 256 ? r384 : (width > 128 ? r256 : r128), 2, 2 * rows * cols, C::THREADS, C::smem_bytes(width), s, tmX, tmR, tmRt,
+  auto launch = [&](auto r32, auto r128, auto r256, auto r384) {
+    launch_tc(width > 256 ? r384 : (width > 128 ? r256 : (width > 32 ? r128 : r32)), 2, 2 * rows * cols, C::THREADS, C::smem_bytes(width), s, tmX, tmR, tmRt,
               static_cast<const __nv_bfloat16*>(R_intra), codes, scales, (int)M, (int)d, tensor_scale, rows, width, st->err_word);
   };
-  if (fmt == FMT_MXINT4) launch(rotate_quantize_wide_kernel<FMT_MXINT4, 128>, rotate_quantize_wide_kernel<FMT_MXINT4, 256>, rotate_quantize_wide_kernel<FMT_MXINT4, 384>);
-  else if (fmt == FMT_NVFP4) launch(rotate_quantize_wide_kernel<FMT_NVFP4, 128>, rotate_quantize_wide_kernel<FMT_NVFP4, 256>, rotate_quantize_wide_kernel<FMT_NVFP4, 384>);
-  else launch(rotate_quantize_wide_kernel<FMT_MXFP4, 128>, rotate_quantize_wide_kernel<FMT_MXFP4, 256>, rotate_quantize_wide_kernel<FMT_MXFP4, 384>);
+  if (fmt == FMT_MXINT4) launch(rotate_quantize_wide_kernel<FMT_MXINT4, 32>, rotate_quantize_wide_kernel<FMT_MXINT4, 128>, rotate_quantize_wide_kernel<FMT_MXINT4, 256>, rotate_quantize_wide_kernel<FMT_MXINT4, 384>);
+  else if (fmt == FMT_NVFP4) launch(rotate_quantize_wide_kernel<FMT_NVFP4, 32>, rotate_quantize_wide_kernel<FMT_NVFP4, 128>, rotate_quantize_wide_kernel<FMT_NVFP4, 256>, rotate_quantize_wide_kernel<FMT_NVFP4, 384>);
+  else launch(rotate_quantize_wide_kernel<FMT_MXFP4, 32>, rotate_quantize_wide_kernel<FMT_MXFP4, 128>, rotate_quantize_wide_kernel<FMT_MXFP4, 256>, rotate_quantize_wide_kernel<FMT_MXFP4, 384>);
   return launch_status();
 }
 
