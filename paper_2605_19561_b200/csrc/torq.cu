@@ -531,7 +531,7 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 // Width of the one-wave rotation's tiles, or 0 where another kernel is faster.  Times in us, fitted to the rotation
 // alone at 60 shapes (d = 128 ... 14336, M = 1 ... 4000; within 10 % but above d = 6144, where these tiles are rated up to 3 us too
 // high, and at d > 8192, where HBM bounds both sides and both are rated low); f = filled part of a wave:
-//  * here: 1.6 + 0.022 per column (2 + 0.032 above 256 columns, 1.4 + 0.022 up to 128) for launch and epilogue, then per K step
+//  * here: 1.8 + 0.0155 per column (2 + 0.025 above 256 columns, 1.6 + 0.0155 up to 128) for launch and epilogue, then per K step
 //    of 64 the operand bytes, 0.17 + 0.0003 per column + 0.03 f (up to 128 columns, where a stage is two of these steps, 0.145 +
 //    0.0003 per column + 0.035 f, but from d = 6272 on, where R_inter's stream sets the pace), or the math, 0.00114 per column;
 //  * few tokens: 3.1 / 4.4 / 5.6 up to 16 / 64 / 128 tokens, plus 0.22 / 0.2 / 0.36 per K step of the longest split; above, 6.4 at
@@ -563,7 +563,7 @@ static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int few_S, b
     if (rows * ((d + w - 1) / w) > max_pairs) continue;
     const double f = (double)(rows * ((d + w - 1) / w)) / max_pairs;
     const double bytes = (w <= 128 && two_slabs ? 0.145 + 0.035 * f : 0.17 + 0.03 * f) + 0.0003 * w, math = 0.00114 * w;
-    const double t = (w <= 128 && two_slabs ? 1.4 + 0.022 * w : (w <= 256 ? 1.6 + 0.022 * w : 2.0 + 0.032 * w)) + (double)steps * (bytes > math ? bytes : math);
+    const double t = (w <= 128 && two_slabs ? 1.6 + 0.0155 * w : (w <= 256 ? 1.8 + 0.0155 * w : 2.0 + 0.025 * w)) + (double)steps * (bytes > math ? bytes : math);
     if (t < best) { best = t; width = w; }
   }
   double other;
