@@ -34,9 +34,8 @@ struct RotPairCfg {
   static constexpr int B_BYTES = (BN / 2 / 64) * B_BOX_BYTES;   // this CTA's 128 columns = 16 KiB
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;         // 32 KiB
   static constexpr int STAGES = 6;
-  static constexpr int RI_ROW_BYTES = 80;              // 32 bf16 + 16 B pad: conflict-free ldmatrix
-  static constexpr int RI_BLOCK_BYTES = 32 * RI_ROW_BYTES;
-  static constexpr int RI_BYTES = (BN / 32) * 32 * 32 * 4;     // the tile's R_intra blocks: fp32, or bf16 padded
+  static constexpr int RI_BLOCK_BYTES = 32 * 64;       // bf16, 64-byte swizzle: the last tile
+  static constexpr int RI_BYTES = (BN / 32) * 32 * 32 * 4;     // the tile's R_intra blocks: fp32, or bf16
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + RI_BYTES + 256 + 1024;
   static constexpr int NACC = 2;
   static constexpr int TMEM_COLS = 512;
@@ -72,6 +71,10 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   auto accf_bar = [&](int a) { return bar_base + 8u * (2 * C::STAGES + a); };
   auto acce_bar = [&](int a) { return bar_base + 8u * (2 * C::STAGES + C::NACC + a); };
   const uint32_t alloc_bar = bar_base + 8u * (2 * C::STAGES + 2 * C::NACC);   // in the leader: the other CTA's tensor memory is allocated
+  // last tile, per column half: in the leader, both CTAs' split terms of a block; the rotated block
+  auto term_bar = [&](int h) { return alloc_bar + 8u + 8u * h; };
+  auto rot_bar = [&](int h) { return alloc_bar + 24u + 8u * h; };
+  const uint32_t ri_bar = alloc_bar + 40;              // in the leader: the last tile's R_intra is in both CTAs' shared memory
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + bar_off + 192);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(smem_gen + bar_off + 200);
 
@@ -94,6 +97,8 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
     for (int s = 0; s < C::STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int a = 0; a < C::NACC; ++a) { mbar_init(accf_bar(a), 1); mbar_init(acce_bar(a), 16); }
     mbar_init(alloc_bar, 1);
+    for (int h = 0; h < 2; ++h) { mbar_init(term_bar(h), 8); mbar_init(rot_bar(h), 1); }
+    mbar_init(ri_bar, 2);
     *cta_abort = 0;
     fence_mbar_init();
   }
@@ -197,6 +202,29 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
         }
         if (ok && elect_one()) tc_commit_pair(accf_bar(a), 3);   // accumulator ready in both CTAs
         __syncwarp();
+        if (FMT != FMT_F32OUT && R_intra != nullptr && ok && tile + npairs >= total_tiles) {
+          // Intra-block rotation of the pair's last tile: three split terms x 32 of K per block, terms and result in tensor memory.
+          constexpr uint32_t idesc_r = idesc_bf16(256, 32, false, true);
+          const int nbb = narrow ? 3 : 4;
+          ok = mbar_wait_cluster_warp(ri_bar, 0, cta_abort, err_word, SITE_MMA_FULL);
+          for (int i = 0; i < 2 * nbb && ok; ++i) {
+            const int h = i & 1, bb = i >> 1;
+            if (!mbar_wait_cluster_warp(term_bar(h), bb & 1, cta_abort, err_word, SITE_MMA_FULL)) { ok = false; break; }
+            tc_fence_after_sync();
+            const uint64_t rdesc = make_desc(smem_u32(ri_smem) + (uint32_t)(h * nbb + bb) * C::RI_BLOCK_BYTES, 2048, 512, kSwizzle64);
+            const uint32_t y = acc + (h * nbb + bb) * 32, out = tmem_base + (a ^ 1) * BN + h * 128, lo = out + 32;
+            if (elect_one()) {
+              mma_bf16_pair_tmem_a(out, lo, rdesc, idesc_r, 0);            // the smallest term first
+              mma_bf16_pair_tmem_a(out, lo + 8, rdesc + 64, idesc_r, 1);   // k 16 .. 31: +8 columns of terms, +16 rows of R_intra
+              mma_bf16_pair_tmem_a(out, y + 16, rdesc, idesc_r, 1);
+              mma_bf16_pair_tmem_a(out, y + 24, rdesc + 64, idesc_r, 1);
+              mma_bf16_pair_tmem_a(out, y, rdesc, idesc_r, 1);
+              mma_bf16_pair_tmem_a(out, y + 8, rdesc + 64, idesc_r, 1);
+              tc_commit_pair(rot_bar(h), 3);
+            }
+            __syncwarp();
+          }
+        }
       }
     }
   } else {
@@ -222,14 +250,13 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
     //  * fp32 FMAs, one row per thread, R_intra broadcast from shared memory as fp32.  Bound by
     //    that broadcast (8 bytes per lane and cycle): about 3/4 of a mainloop per tile, which does
     //    not matter while the next tile's mainloop runs beside it on the tensor pipe.
-    //  * warp-level tensor-core MMAs on the accumulator fragment layout (y split into three bf16
-    //    terms, R_intra exact in bf16, fp32 accumulation): half the time when the tensor pipe is
-    //    otherwise idle, but it fights the mainloop when both run.  Used for the CTA's LAST tile,
-    //    whose epilogue nothing overlaps.
+    //  * tcgen05 instructions of both CTAs on three split bf16 terms of y in tensor memory (every product exact, fp32
+    //    accumulation), for the CTA's LAST tile, whose epilogue nothing overlaps and beside which half the tensor memory is free.  (As
+    //    warp-level MMAs on accumulator fragments that epilogue was bound by those: us, loops of 0.4 s, before / now, rotation
+    //    2048 x 4096 59.7 / 58.25, 1900 x 4096 NVFP4 60.0 / 58.6, 8192 x 1024 26.6 / 25.8; shorter loops 58.05 / 56.3, 59.6 / 55.7 and 26.5 / 25.3.)
     const int q = warp & 3;
     const int h = (warp - 2) >> 2;
     const int et = (warp - 2) * 32 + lane;               // 0..255 among the epilogue threads
-    const int p = lane & 3, r8 = lane >> 2;
     const uint32_t ri_saddr = smem_u32(ri_smem);
     uint32_t tcount = 0;
     bool ok = true;
@@ -247,11 +274,11 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
         named_barrier_sync(1, 256);
         for (int idx = et * 8; ok && idx < (BN / 32) * 1024; idx += 256 * 8) {
           const int lb = idx >> 10, blk = b0 + lb;
-          if (last) {                                    // bf16 rows of 80 bytes: conflict-free ldmatrix
-            const int i = (idx & 1023) >> 5, c = idx & 31;
+          if (last) {                                    // bf16, 16-byte piece c of row i at c ^ ((i >> 1) & 3); rank 1: two pieces on
+            const int i = (idx & 1023) >> 5, c = ((idx & 31) >> 3) ^ (2 * (int)rank);
             uint4 v = make_uint4(0u, 0u, 0u, 0u);
             if (blk < nblocks) v = __ldg(reinterpret_cast<const uint4*>(R_intra + (size_t)blk * 1024 + (idx & 1023)));
-            *reinterpret_cast<uint4*>(ri_smem + lb * C::RI_BLOCK_BYTES + i * C::RI_ROW_BYTES + c * 2) = v;
+            *reinterpret_cast<uint4*>(ri_smem + lb * C::RI_BLOCK_BYTES + i * 64 + ((c ^ ((i >> 1) & 3)) << 4)) = v;
           } else {                                       // fp32, dense
             float v[8];
             if (blk < nblocks) load8(R_intra + (size_t)blk * 1024 + (idx & 1023), v);
@@ -264,7 +291,9 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
             *reinterpret_cast<float4*>(dst + 4) = make_float4(v[4], v[5], v[6], v[7]);
           }
         }
+        if (last) fence_proxy_async_smem();              // visible to the tensor core's reads
         named_barrier_sync(1, 256);
+        if (last && et == 0) mbar_arrive_release_cluster(map_to_cta(ri_bar, 0));
       }
       if (ok) ok = mbar_wait_cluster(accf_bar(a), (tcount / C::NACC) & 1, cta_abort, err_word, SITE_EPI_ACC_FULL);
       ok = __all_sync(0xFFFFFFFFu, ok);
@@ -299,8 +328,8 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
           }
         }
       };
-      if (!last) {
-        // ---- one row per thread, fp32 FMAs
+      {
+        // ---- one row per thread
         const int64_t row = (int64_t)mt * C::BM + q * 32 + lane;
         uint32_t sc_word = 0, sc_word2 = 0;              // NVFP4: two groups of four 16-blocks
         NvScale nvs = {};
@@ -317,7 +346,29 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
               mbar_arrive_cluster(map_to_cta(acce_bar(a), 0));
           }
           float z[32];
-          if (R_intra != nullptr) {
+          if (FMT != FMT_F32OUT && last && R_intra != nullptr) {
+            // y goes back to tensor memory as hi + mid + lo (bf16, exact): hi and mid over y, lo where the other accumulator's columns of
+            // this half were, which these warps have read; the result comes beside it.
+            const uint32_t other = tmem_base + ((uint32_t)(q * 32) << 16) + (a ^ 1) * BN + h * 128;
+            uint32_t hi[16], mid[16], lo[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) split3_trunc_bf16x2(yv[2 * e], yv[2 * e + 1], hi[e], mid[e], lo[e]);
+            tmem_st_32x32_x16(tacc + bb * 32, hi);
+            tmem_st_32x32_x16(tacc + bb * 32 + 16, mid);
+            tmem_st_32x32_x16(other + 32, lo);
+            tmem_st_wait();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(map_to_cta(term_bar(h), 0));
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait_cluster(rot_bar(h), bb & 1, cta_abort, err_word, SITE_EPI_ACC_FULL));
+            if (!ok) break;
+            tc_fence_after_sync();
+            tmem_ld_32x32(other, yv);
+            tmem_ld_wait();
+            tc_fence_before_sync();
+#pragma unroll
+            for (int j = 0; j < 32; ++j) z[j] = __uint_as_float(yv[j]);
+          } else if (R_intra != nullptr) {
             intra_rotate32(yv, ri_saddr + (uint32_t)(h * nbb + bb) * 4096, z);
           } else {
 #pragma unroll
@@ -356,6 +407,7 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
             sc_word |= sbyte << (8 * bb);
           }
         }
+        if (!ok) continue;
         if constexpr (FMT == FMT_F32OUT) {
           continue;
         } else if constexpr (FMT == FMT_NVFP4) {
@@ -364,104 +416,6 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
         } else {
           if (mt < m_tiles) put_scales(sc_word, (size_t)lane * 16 + q * 4);   // the pair's second row tile may not exist
         }
-        continue;
-      }
-      // ---- accumulator fragment layout (16 rows at a time): thread t holds rows t/4 and t/4 + 8,
-      //      eight columns of each per block
-      const int64_t row_base = (int64_t)mt * C::BM + q * 32 + r8;     // + 16 mh + 8 rh
-      uint32_t sc_word[4] = {0u, 0u, 0u, 0u};            // rows r8 + 16 mh + 8 rh -> index 2 mh + rh
-      uint32_t sc_hi[4] = {0u, 0u, 0u, 0u};              // NVFP4: second group of four 16-blocks
-      NvScale nvs = {};
-      if constexpr (FMT == FMT_NVFP4) nvs = nv_scale(tensor_scale);
-#pragma unroll 1
-      for (int bb = 0; bb < nbb; ++bb) {
-        const int blk = fb + bb;
-        uint32_t bfrag[2][4][2];                         // [k chunk][n tile][2]
-        if (R_intra != nullptr) {
-          // lane l: row l % 8 of matrix l / 8; matrices (k 0-7, n), (k 8-15, n), (k 0-7, n+8), (k 8-15, n+8)
-          const uint32_t rb = ri_saddr + (uint32_t)(h * nbb + bb) * C::RI_BLOCK_BYTES +
-                              (uint32_t)(((lane >> 3) & 1) * 8 + (lane & 7)) * C::RI_ROW_BYTES +
-                              (uint32_t)(lane >> 4) * 16;
-#pragma unroll
-          for (int kc = 0; kc < 2; ++kc)
-#pragma unroll
-            for (int np = 0; np < 2; ++np)
-              ldmatrix_x4_trans(rb + kc * 16 * C::RI_ROW_BYTES + np * 32, bfrag[kc][2 * np][0], bfrag[kc][2 * np][1],
-                                bfrag[kc][2 * np + 1][0], bfrag[kc][2 * np + 1][1]);
-        }
-#pragma unroll
-        for (int mh = 0; mh < 2; ++mh) {
-          uint32_t y[16];
-          tmem_ld_16x256b_x4(tacc + ((uint32_t)(16 * mh) << 16) + bb * 32, y);
-          tmem_ld_wait();
-          float acc[4][4];
-          if (R_intra != nullptr) {
-            uint32_t ah[8], am[8], al[8];                // A fragments: [k chunk * 4 + (n & 1) * 2 + row half]
-#pragma unroll
-            for (int n = 0; n < 4; ++n)
-#pragma unroll
-              for (int rh = 0; rh < 2; ++rh) {
-                const int ai = (n >> 1) * 4 + (n & 1) * 2 + rh;
-                split3_bf16x2(y[4 * n + 2 * rh], y[4 * n + 2 * rh + 1], ah[ai], am[ai], al[ai]);
-              }
-#pragma unroll
-            for (int n = 0; n < 4; ++n) { acc[n][0] = 0.f; acc[n][1] = 0.f; acc[n][2] = 0.f; acc[n][3] = 0.f; }
-#pragma unroll
-            for (int kc = 0; kc < 2; ++kc)
-#pragma unroll
-              for (int n = 0; n < 4; ++n) {
-                mma_16816_bf16(acc[n], al + 4 * kc, bfrag[kc][n]);
-                mma_16816_bf16(acc[n], am + 4 * kc, bfrag[kc][n]);
-                mma_16816_bf16(acc[n], ah + 4 * kc, bfrag[kc][n]);
-              }
-          } else {
-#pragma unroll
-            for (int n = 0; n < 4; ++n)
-#pragma unroll
-              for (int e = 0; e < 4; ++e) acc[n][e] = __uint_as_float(y[4 * n + e]);
-          }
-#pragma unroll
-          for (int rh = 0; rh < 2; ++rh) {
-            const float v[8] = {acc[0][2 * rh], acc[0][2 * rh + 1], acc[1][2 * rh], acc[1][2 * rh + 1],
-                                acc[2][2 * rh], acc[2][2 * rh + 1], acc[3][2 * rh], acc[3][2 * rh + 1]};
-            uint32_t word, sbyte;
-            const int64_t row = row_base + 16 * mh + 8 * rh;
-            if constexpr (FMT == FMT_MXINT4) {             // two operand bytes per 8 columns and lane
-              uint32_t pr[4];
-              mxint4_quantize_row_fragment(v, pr, sbyte);
-              if (row < M && blk < nblocks) {
-                uint8_t* dst = codes + row * (int64_t)d + (int64_t)blk * 32 + 2 * p;
-#pragma unroll
-                for (int nt = 0; nt < 4; ++nt) *reinterpret_cast<uint16_t*>(dst + 8 * nt) = (uint16_t)pr[nt];
-              }
-            } else {
-              if constexpr (FMT == FMT_NVFP4) nv_quantize_row_fragment(v, p, nvs, word, sbyte);
-              else quantize_row_fragment(v, p, word, sbyte);
-              if (row < M && blk < nblocks)
-                *reinterpret_cast<uint32_t*>(codes + row * (int64_t)(d / 2) + (int64_t)blk * 16 + 4 * p) = word;
-            }
-            if constexpr (FMT == FMT_NVFP4) {
-              if (blk >= nblocks) sbyte = 0;
-              if (bb < 2) sc_word[2 * mh + rh] |= sbyte << (16 * bb);
-              else sc_hi[2 * mh + rh] |= sbyte << (16 * (bb - 2));
-            } else {
-              sc_word[2 * mh + rh] |= sbyte << (8 * bb);
-            }
-          }
-        }
-      }
-      if constexpr (FMT == FMT_NVFP4) {
-        const int kb4n = (2 * nblocks + 3) / 4;
-        if (p == 0 && mt < m_tiles) {
-#pragma unroll
-          for (int rs = 0; rs < 4; ++rs) {
-            put_scales16(sc_word[rs], sc_hi[rs], (size_t)(r8 + 16 * (rs >> 1) + 8 * (rs & 1)) * 16 + q * 4, kb4n);
-          }
-        }
-      } else if (p == 0 && mt < m_tiles) {               // the pair's second row tile may not exist
-#pragma unroll
-        for (int rs = 0; rs < 4; ++rs)
-          put_scales(sc_word[rs], (size_t)(r8 + 16 * (rs >> 1) + 8 * (rs & 1)) * 16 + q * 4);
       }
     }
   }

@@ -534,8 +534,8 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 //  * here: 1.8 + 0.0155 per column (2 + 0.025 above 256 columns, 1.6 + 0.0155 up to 128) for launch and epilogue, then per K step
 //    of 64 the operand bytes, 0.17 + 0.0003 per column + 0.03 f (up to 128 columns, where a stage is two of these steps, 0.145 +
 //    0.0003 per column + 0.035 f, but from d = 6272 on, where R_inter's stream sets the pace), or the math, 0.00114 per column;
-//  * few tokens: 3.1 / 4.4 / 5.6 up to 16 / 64 / 128 tokens, plus 0.22 / 0.2 / 0.36 per K step of the longest split; above, 6.4 at
-//    144 tokens and 0.025 per token more, 0.5 per CTA of a cluster above four, 0.42 per K step (us, few tokens / here: 144
+//  * few tokens: 3.1 / 4.4 / 5.6 up to 16 / 64 / 128 tokens, plus 0.22 / 0.2 / 0.36 per K step of the longest split; above, 6.4 (5.9 up
+//    to 176 tokens: 160 x 2816 15.2 / 16.05 as layers, but 180 x 3072 18.1 / 16.25) at 144 tokens and 0.025 per token more, 0.5 per CTA of a cluster above four, 0.42 per K step (us, few tokens / here: 144
 //    tokens d = 2560 9.7 / 10.4, d = 4096 13.6 / 14.9; 208 d = 2560 12.6 / 10.4, d = 4096 15.0 / 15.0 (the layer with N = 6144
 //    22.7 / 23.2), d = 5120 19.5 / 20.1; 256 d = 4096 16.2 / 15.1, d = 5120 20.9 / 20.0; 128 d = 2048 8.1 / 7.6).  Beside clusters of six
 //    (d = 2048 ... 2816, up to 192 tokens) this is a microsecond more than they take with cold operands, and the line lies between
@@ -544,7 +544,7 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 //  * few tokens whose sums are pushed: 2.7 + 0.22 per K step + 0.025 per token, 0.04 above 32 tokens (us, here / few tokens, 1, 16 and 32 tokens: d = 256 2.95 / 2.96, 2.95 /
 //    3.21, 2.95 / 4.49; d = 512 3.97 / 3.08, 3.37 / 3.21, 3.46 / 3.60; d = 768 5.25 / 3.21, 4.24 / 3.37, 4.36 / 3.85);
 //  * above 192 tokens a cluster of three has five units for its first CTA: 0.6 more (216 d = 4864 19.3 / 18.2);
-//  * above d = 6144, where these tiles take up to 3 us less than the figures say: 7.6 up to 192 tokens, 10.5 above, 0.42 per K step
+//  * above d = 6144, where these tiles take up to 3 us less than the figures say: 7.0 up to 192 tokens, 9.9 above, 0.42 per K step
 //    (144 d = 6912 26.9 / 25.4, 150 d = 7040 28.2 / 26.3, 208 d = 7680 33.1 / 30.0);
 //  * pair kernel: 6.8, plus per K step 0.32 for a wave and 0.2 + 0.14 f for the last, partly filled one.
 // The other formats follow the same figures, which were not fitted to them; wide_gemm_width says how that was checked.
@@ -572,8 +572,8 @@ static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int few_S, b
     else if (M <= 16) other = 3.1 + 0.22 * few_steps;
     else if (M <= 64) other = 4.4 + 0.2 * few_steps;
     else if (M <= 128) other = 5.6 + 0.36 * few_steps;
-    else if (d > 6144) other = (M <= 192 ? 7.6 : 10.5) + 0.42 * few_steps;
-    else other = 6.4 + 0.025 * (double)(M - 144) + (few_S > 4 ? 0.5 * (few_S - 4) : (few_S == 3 && M > 192 ? 0.6 : 0.0)) + 0.42 * few_steps;
+    else if (d > 6144) other = (M <= 192 ? 7.0 : 9.9) + 0.42 * few_steps;
+    else other = (M <= 176 ? 5.9 : 6.4) + 0.025 * (double)(M - 144) + (few_S > 4 ? 0.5 * (few_S - 4) : (few_S == 3 && M > 192 ? 0.6 : 0.0)) + 0.42 * few_steps;
   } else {
     const int64_t tiles = rows * ((d + 255) / 256);
     const int64_t full = tiles / max_pairs, rest = tiles % max_pairs;
