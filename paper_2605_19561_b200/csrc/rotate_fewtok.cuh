@@ -11,8 +11,8 @@
 // contracts k range r.  The fp32 partial tiles never leave the SMs: every output has one CTA of the cluster that owns it, adds the S
 // partials in rank order (fixed order, so the result does not depend on timing), rotates inside the block and quantizes (Eq. 1).
 // The partials reach the owner in one of two ways:
-//  * PUSH (up to 32 tokens, with R_intra and clusters of eight up to 56): the pieces of work are small, 32 features x 4 tokens, and dealt over all CTAs and warps of the cluster, so that
-//    nearly every warp has one and no CTA takes in more than its share (what arrives at one SM comes at about 9 B per cycle).  A CTA
+//  * PUSH (up to 32 tokens, with R_intra and clusters of eight up to 56): the pieces of work are small, 32 features x 4
+//    tokens, and dealt over all CTAs and warps of the cluster, so that nearly every warp has one and no CTA takes in more than its share (what arrives at one SM comes at about 9 B per cycle).  A CTA
 //    stores its partials straight from registers into the owners' shared memory (st.async, 16 bytes per lane = four tokens of one
 //    feature, counted on a barrier of the owning warp), into room of their own: nobody has to say first that the stages there are free, and
 //    no cluster-wide barrier stands on the path.  The owning warp keeps one feature per lane: the intra rotation is 32 x 4 FMAs per lane

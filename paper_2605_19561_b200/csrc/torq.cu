@@ -334,9 +334,14 @@ static bool fewtok_leave_together(int64_t M, int64_t tiles, FewRotation few, con
 }
 // Cluster size of the few-token GEMM: above S = 4 three K steps per CTA, or two while the partial sums of all CTAs are few: 32
 // tokens per SM (us, S = 4 / 8, 17 and 64 tokens: N = 256, K = 4096 3.44 / 2.99 and 4.33 / 3.92, N = 1024 3.58 / 3.20 and 4.60 /
-// 4.34; S = 4 / 6: 17 tokens N = 2048 3.75 / 3.47; beyond the line 64 tokens N = 2048 NVFP4 4.53 / 4.70), and 8 up to 16 tokens,
-// where the sums are pushed (1 token N = 256 2.96 / 2.58, N = 1024 3.10 / 2.82, the layer 11.2 / 10.9; beyond: N = 2048 the GEMM 3.62 /
+// 4.34; S = 4 / 6: 17 tokens N = 2048 3.75 / 3.47; beyond the line 64 tokens N = 2048 NVFP4 4.53 / 4.70), and 8 up to 16 tokens
+// (1 token N = 256 2.96 / 2.58, N = 1024 3.10 / 2.82, the layer 11.2 / 10.9; beyond: N = 2048 the GEMM 3.62 /
 // 3.51, the layer of 16 tokens 13.2 / 13.5; S = 4 / 5 at K = 2560, N = 5120 the layer 11.0 / 11.5).
+static int fewtok_gemm_cluster(int ntok, int64_t tiles, int64_t steps, int ctas, const DeviceState* st) {
+  const int S = fewtok_cluster(tiles, steps, steps / 2, ctas, st->sm_count, st->few_fit);
+  if (tiles * S * ntok <= (ntok > 16 ? 32 : 8) * (int64_t)st->sm_count) return S;
+  return fewtok_cluster(tiles, steps, steps / 3, ctas, st->sm_count, st->few_fit);
+}
 // Where the sums are pushed (M tokens), from the largest cluster down: above four CTAs where each keeps four K steps and has its SM to itself
 // (a CTA's instructions wait for those of the other one on its SM), or with five and more steps; up to four where they have their SMs to
 // themselves (a tenth may share), or with more than five steps.  us, layers, S = 3 / 4 / 5 / 8: 8 x 5120 -> 5120 (20 steps) 15.35 / 14.5 /
@@ -359,11 +364,6 @@ static int push_gemm_cluster(int64_t M, int64_t tiles, int64_t steps, const Devi
     }
   }
   return 1;
-}
-static int fewtok_gemm_cluster(int ntok, int64_t tiles, int64_t steps, int ctas, const DeviceState* st) {
-  const int S = fewtok_cluster(tiles, steps, steps / 2, ctas, st->sm_count, st->few_fit);
-  if (tiles * S * ntok <= (ntok > 16 ? 32 : 8) * (int64_t)st->sm_count) return S;
-  return fewtok_cluster(tiles, steps, steps / 3, ctas, st->sm_count, st->few_fit);
 }
 constexpr int kTailTiles = 8;              // a last wave of up to so many tiles leaves the pair rotation (below)
 // A 192-column tile against a 256-column one: an instruction takes the larger of N / 2 cycles and 64 + N / 4, the reading of its A and B
@@ -617,7 +617,7 @@ static torq_status rotate_fewtok(DeviceState* st, int fmt, const void* X, const 
   const int smem = RotFewCfg::smem_bytes(ntok, few.stages, few.push);
   const float ts = fmt == FMT_NVFP4 ? tensor_scale : 0.0f;
   const __nv_bfloat16* ri = static_cast<const __nv_bfloat16*>(R_intra);
-  // up to 16 tokens: partials pushed to one CTA; two CTAs per SM: one set of epilogue warps; one CTA: two sets
+  // sums pushed, with five, four or three stages; pulled, two CTAs per SM: one set of epilogue warps; one CTA: two sets
   auto launch = [&](auto push5, auto push4, auto push3, auto one, auto shared, auto two) {
     const bool share = few.stages == RotFewCfg::SHARED_STAGES, small = few.push || share || ntok <= 64;
     launch_tc(few.push ? (few.stages == RotFewCfg::PUSH_STAGES ? push5 : (share ? push3 : push4)) : (share ? shared : (small ? one : two)), S,
@@ -901,7 +901,7 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
     if (!encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, 128, 128) ||
         !encode_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Aq, (uint64_t)M, krow, (uint32_t)ntok, 128))
       return TORQ_ERR_LAUNCH;
-    // up to 16 tokens: partials pushed; up to 64: one set of epilogue warps, two CTAs per SM; more: two sets.  65 to 80 tokens in
+    // sums pushed (FC::push); up to 64 tokens: one set of epilogue warps, two CTAs per SM; more: two sets.  65 to 80 tokens in
     // MXINT4 fit twice on an SM as well, and share it only where that gives them more K splits (us, shared / alone, 72 tokens:
     // N = 768, K = 3072 4.9 / 4.4, N = 1536 6.0 / 5.1, S = 8 either way; N = 6144, K = 4096, S = 4 and 1: 9.1 / 9.9).
     const bool small = FC::ctas_per_sm((int)M, (int)K) >= 2 && (ntok <= 64 || S > fewtok_gemm_cluster(ntok, tiles, steps, 1, st));
