@@ -206,10 +206,10 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
           // Intra-block rotation of the pair's last tile: three split terms x 32 of K per block, terms and result in tensor memory.
           constexpr uint32_t idesc_r = idesc_bf16(256, 32, false, true);
           const int nbb = narrow ? 3 : 4;
-          ok = mbar_wait_cluster_warp(ri_bar, 0, cta_abort, err_word, SITE_MMA_FULL);
+          ok = mbar_wait_cluster_warp<true>(ri_bar, 0, cta_abort, err_word, SITE_MMA_FULL);
           for (int i = 0; i < 2 * nbb && ok; ++i) {
             const int h = i & 1, bb = i >> 1;
-            if (!mbar_wait_cluster_warp(term_bar(h), bb & 1, cta_abort, err_word, SITE_MMA_FULL)) { ok = false; break; }
+            if (!mbar_wait_cluster_warp<true>(term_bar(h), bb & 1, cta_abort, err_word, SITE_MMA_FULL)) { ok = false; break; }
             tc_fence_after_sync();
             const uint64_t rdesc = make_desc(smem_u32(ri_smem) + (uint32_t)(h * nbb + bb) * C::RI_BLOCK_BYTES, 2048, 512, kSwizzle64);
             const uint32_t y = acc + (h * nbb + bb) * 32, out = tmem_base + (a ^ 1) * BN + h * 128, lo = out + 32;

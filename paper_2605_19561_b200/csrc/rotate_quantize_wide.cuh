@@ -206,9 +206,9 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       if (ok) tc_commit_pair(accf_bar, 3);          // accumulator ready in both CTAs
       // Intra-block rotation: block bb by set bb % sets, three split terms x 32 of K, terms and result in tensor memory.
       constexpr uint32_t idesc_r = idesc_bf16(256, 32, false, true);
-      if (kTerms && R_intra != nullptr && ok) ok = mbar_wait_cluster(ri_bar, 0, cta_abort, err_word, SITE_MMA_FULL);
+      if (kTerms && R_intra != nullptr && ok) ok = mbar_wait_cluster<true>(ri_bar, 0, cta_abort, err_word, SITE_MMA_FULL);
       for (int bb = 0, set = 0, r = 0; kTerms && R_intra != nullptr && ok && bb < nb; ++bb) {
-        ok = mbar_wait_cluster(term_bar(set), r & 1, cta_abort, err_word, SITE_MMA_FULL);
+        ok = mbar_wait_cluster<true>(term_bar(set), r & 1, cta_abort, err_word, SITE_MMA_FULL);
         if (!ok) break;
         tc_fence_after_sync();
         const uint64_t rdesc = make_desc(smem_base + ri_off + bb * C::RI_BLOCK_BYTES, 2048, 512, kSwizzle64);
