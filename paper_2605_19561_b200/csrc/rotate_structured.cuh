@@ -195,9 +195,12 @@ rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_
     // Until the kernel before has completed HBM idles: the L2 is asked for the first tile's X, one 4-KiB box per lane, and for R_B where
     // it is one strip (with two or more the order in which they then run costs more: 4096 x 5120 -> 1024 37.1 / 38.6 us).  Here and
     // not ahead of the roles, whose instructions would lie further apart (64 x 256 -> 256 6.54 / 6.62).  us, without / with, layers:
-    // 2048 x 4096 -> 6144 34.4 / 33.5, 300 x 4096 -> 4096 12.1 / 11.8, 8192 x 2048 -> 2048 40.3 / 39.9.
-    if ((lane >> 2) < k_tiles) tma_prefetch_l2_3d(&tmX3, 0, blockIdx.x / b_tiles * C::TOK + (lane & 3), (lane >> 2) * C::BK);
-    if (b_tiles == 1 && lane < k_tiles) tma_prefetch_l2_2d(&tmRB, lane * C::BK, 0);
+    // 2048 x 4096 -> 6144 34.4 / 33.5, 300 x 4096 -> 4096 12.1 / 11.8.
+    // Whole boxes only: one that reaches beyond the tensor took the call 1 to 3 us (2025 x 256 -> 4096, 8 of a box's 64 blocks, 15.9 / 18.9;
+    // 9990 x 1280 -> 1424, 40 of 64, 41.0 / 41.8).
+    const int token = blockIdx.x / b_tiles * C::TOK + (lane & 3);
+    if (((lane >> 2) + 1) * C::BK <= nblocks && token < M) tma_prefetch_l2_3d(&tmX3, 0, token, (lane >> 2) * C::BK);
+    if (nblocks == C::BM && lane < k_tiles) tma_prefetch_l2_2d(&tmRB, lane * C::BK, 0);
     __syncwarp();
     griddep_wait();
     uint32_t tcount = 0;
