@@ -531,11 +531,13 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 // Width of the one-wave rotation's tiles, or 0 where another kernel is faster.  Times in us, fitted to the rotation
 // alone at 60 shapes (d = 128 ... 14336, M = 1 ... 4000; within 10 % but above d = 6144, where these tiles are rated up to 3 us too
 // high, and at d > 8192, where HBM bounds both sides and both are rated low); f = filled part of a wave:
-//  * here: 1.8 + 0.0155 per column (2 + 0.025 above 256 columns, 1.6 + 0.0155 up to 128) for launch and epilogue, then per K step
-//    of 64 the operand bytes, 0.17 + 0.0003 per column + 0.03 f (up to 128 columns, where a stage is two of these steps, 0.145 +
+//  * here: 1.8 + 0.0155 per column (2 + 0.025 above 256 columns, 1.6 + 0.0155 up to 128) for launch and epilogue, from 129 to 256
+//    tokens 1.6 + 0.022 (2 + 0.032, 1.4 + 0.022), what they were with warp-level instructions: the few-token kernel contracts K in
+//    parts, which these tiles do in one accumulator, and a line that follows the shorter epilogue gives up precision (codes that differ
+//    from those of 64-bit arithmetic, few tokens / here: 220 x 5504 6 / 51 of 1.2 M).  Then per K step of 64 the operand bytes, 0.17 + 0.0003 per column + 0.03 f (up to 128 columns, where a stage is two of these steps, 0.145 +
 //    0.0003 per column + 0.035 f, but from d = 6272 on, where R_inter's stream sets the pace), or the math, 0.00114 per column;
-//  * few tokens: 3.1 / 4.4 / 5.6 up to 16 / 64 / 128 tokens, plus 0.22 / 0.2 / 0.36 per K step of the longest split; above, 6.4 (5.9 up
-//    to 176 tokens: 160 x 2816 15.2 / 16.05 as layers, but 180 x 3072 18.1 / 16.25) at 144 tokens and 0.025 per token more, 0.5 per CTA of a cluster above four, 0.42 per K step (us, few tokens / here: 144
+//  * few tokens: 3.1 / 4.4 / 5.6 up to 16 / 64 / 128 tokens, plus 0.22 / 0.2 / 0.36 per K step of the longest split; above, 6.4 (6.1 up
+//    to 176 tokens: 160 x 2816 15.2 / 16.05 as layers) at 144 tokens and 0.025 per token more, 0.5 per CTA of a cluster above four, 0.42 per K step (us, few tokens / here: 144
 //    tokens d = 2560 9.7 / 10.4, d = 4096 13.6 / 14.9; 208 d = 2560 12.6 / 10.4, d = 4096 15.0 / 15.0 (the layer with N = 6144
 //    22.7 / 23.2), d = 5120 19.5 / 20.1; 256 d = 4096 16.2 / 15.1, d = 5120 20.9 / 20.0; 128 d = 2048 8.1 / 7.6).  Beside clusters of six
 //    (d = 2048 ... 2816, up to 192 tokens) this is a microsecond more than they take with cold operands, and the line lies between
@@ -544,7 +546,7 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 //  * few tokens whose sums are pushed: 2.7 + 0.22 per K step + 0.025 per token, 0.04 above 32 tokens (us, here / few tokens, 1, 16 and 32 tokens: d = 256 2.95 / 2.96, 2.95 /
 //    3.21, 2.95 / 4.49; d = 512 3.97 / 3.08, 3.37 / 3.21, 3.46 / 3.60; d = 768 5.25 / 3.21, 4.24 / 3.37, 4.36 / 3.85);
 //  * above 192 tokens a cluster of three has five units for its first CTA: 0.6 more (216 d = 4864 19.3 / 18.2);
-//  * above d = 6144, where these tiles take up to 3 us less than the figures say: 7.0 up to 192 tokens, 9.9 above, 0.42 per K step
+//  * above d = 6144, where these tiles take up to 3 us less than the figures say: 7.6 up to 192 tokens, 10.5 above, 0.42 per K step
 //    (144 d = 6912 26.9 / 25.4, 150 d = 7040 28.2 / 26.3, 208 d = 7680 33.1 / 30.0);
 //  * pair kernel: 6.8, plus per K step 0.32 for a wave and 0.2 + 0.14 f for the last, partly filled one.
 // The other formats follow the same figures, which were not fitted to them; wide_gemm_width says how that was checked.
@@ -557,13 +559,16 @@ static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int few_S, b
   // tokens / here: d = 1024 63 tokens 5.7 / 5.8, 64 tokens 5.7 / 4.5; d = 1152 56 5.6 / 5.7, 60 5.7 / 4.7; d = 1536 40 5.9 / 9.3, 48
   // 6.0 / 5.6).
   const bool two_slabs = d <= 6144 && (M > 96 || (M <= 64 && M * d >= 65536));
+  const bool against_parts = M > 128 && M <= kRotFewMaxTokens;
+  const double column = against_parts ? 0.022 : 0.0155, column_wide = against_parts ? 0.032 : 0.025, fixed = against_parts ? 1.6 : 1.8;
   double best = 1e30;
   int width = 0;
   for (int w = 32; w <= RotWideCfg::MAX_WIDTH; w += 32) {
     if (rows * ((d + w - 1) / w) > max_pairs) continue;
     const double f = (double)(rows * ((d + w - 1) / w)) / max_pairs;
     const double bytes = (w <= 128 && two_slabs ? 0.145 + 0.035 * f : 0.17 + 0.03 * f) + 0.0003 * w, math = 0.00114 * w;
-    const double t = (w <= 128 && two_slabs ? 1.6 + 0.0155 * w : (w <= 256 ? 1.8 + 0.0155 * w : 2.0 + 0.025 * w)) + (double)steps * (bytes > math ? bytes : math);
+    const double ends = w > 256 ? 2.0 + column_wide * w : fixed - (w <= 128 && two_slabs ? 0.2 : 0.0) + column * w;
+    const double t = ends + (double)steps * (bytes > math ? bytes : math);
     if (t < best) { best = t; width = w; }
   }
   double other;
@@ -572,8 +577,8 @@ static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int few_S, b
     else if (M <= 16) other = 3.1 + 0.22 * few_steps;
     else if (M <= 64) other = 4.4 + 0.2 * few_steps;
     else if (M <= 128) other = 5.6 + 0.36 * few_steps;
-    else if (d > 6144) other = (M <= 192 ? 7.0 : 9.9) + 0.42 * few_steps;
-    else other = (M <= 176 ? 5.9 : 6.4) + 0.025 * (double)(M - 144) + (few_S > 4 ? 0.5 * (few_S - 4) : (few_S == 3 && M > 192 ? 0.6 : 0.0)) + 0.42 * few_steps;
+    else if (d > 6144) other = (M <= 192 ? 7.6 : 10.5) + 0.42 * few_steps;
+    else other = (M <= 176 ? 6.1 : 6.4) + 0.025 * (double)(M - 144) + (few_S > 4 ? 0.5 * (few_S - 4) : (few_S == 3 && M > 192 ? 0.6 : 0.0)) + 0.42 * few_steps;
   } else {
     const int64_t tiles = rows * ((d + 255) / 256);
     const int64_t full = tiles / max_pairs, rest = tiles % max_pairs;
