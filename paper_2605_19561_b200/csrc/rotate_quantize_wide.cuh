@@ -257,9 +257,10 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
         *reinterpret_cast<uint4*>(smem_gen + ri_off + lb * C::RI_BLOCK_BYTES + i * 64 + ((c ^ ((i >> 1) & 3)) << 4)) =
             __ldg(reinterpret_cast<const uint4*>(R_intra + (size_t)(b0 + lb) * 1024) + (idx & 127));
       }
-      fence_proxy_async_smem();                        // visible to the tensor core's reads
+      if constexpr (kTerms) fence_proxy_async_smem();  // visible to the tensor core's reads
       named_barrier_sync(1, 128 * C::ESETS);
-      if (warp == 2 && lane == 0) mbar_arrive_release_cluster(map_to_cta(ri_bar, 0));
+      // kTerms only: without them nobody waits for it, and an arrival that is not waited for could reach a CTA that has exited
+      if (kTerms && warp == 2 && lane == 0) mbar_arrive_release_cluster(map_to_cta(ri_bar, 0));
     }
     griddep_wait();                                    // codes and scales may still be read by that kernel
     bool ok = mbar_wait_cluster(accf_bar, 0, cta_abort, err_word, SITE_EPI_ACC_FULL);

@@ -94,3 +94,36 @@ def test_a_wait_reports_what_it_waits_for():
                 assert site == kinds[bar], (f, bar, site)
                 seen.add(bar)
     assert seen == set(kinds)
+
+
+def _conditions(body, at):
+    """What has to hold for the statement at `at` to run: the conditions of the blocks around it and of its own if / for, their
+    && taken apart, flags that are declared once replaced by what they stand for."""
+    named = dict(re.findall(r"bool (?:\w+ = [^;]*?, )?(\w+) = ([^;?]*?);", body))
+    opens, depth = [], 0
+    for m in re.finditer(r"[{}]", body[:at]):
+        if m.group() == "{":
+            head = body[max(body.rfind(c, 0, m.start()) for c in "{}") + 1:m.start()]
+            opens.append(head[head.rfind(";\n") + 1:])
+        elif opens:
+            opens.pop()
+    own = body[max(body.rfind("{\n", 0, at), body.rfind("}\n", 0, at), body.rfind(";\n", 0, at)):at]
+    terms = set()
+    for text in opens + [own]:
+        for cond in re.findall(r"(?:if(?: constexpr)?|for) \((.*)\)", text + ")"):
+            for t in re.split(r"&&|;", cond.replace("(", " ").replace(")", " ")):
+                t = " ".join(t.split())
+                terms |= {" ".join(x.split()) for x in named.get(t, t).split("&&")}
+    return terms
+
+
+@pytest.mark.parametrize("name", ["rotate_quantize_wide.cuh", "rotate_quantize_pair.cuh"])
+def test_an_instance_that_does_not_wait_for_r_intra_sends_no_arrival(name):
+    """The arrival that tells the leader of the other CTA's R_intra stands behind every condition on the instance and on the arguments
+    that the leader's wait for it stands behind: one that nobody waits for could reach a CTA that has exited."""
+    body = re.sub(r"//.*", "", open(os.path.join(CSRC, name)).read())
+    wait = _conditions(body, re.search(r"mbar_wait\w*(?:<true>)?\(ri_bar", body).start())
+    arrive = _conditions(body, re.search(r"mbar_arrive\w*\(map_to_cta\(ri_bar", body).start())
+    wanted = {t for t in wait if re.search(r"FMT|RANGE|R_intra|total_tiles", t) and " = " not in t}
+    assert any("R_intra" in t for t in wanted) and any(re.search(r"FMT|RANGE", t) for t in wanted), wait
+    assert wanted <= arrive, (wanted, arrive)
