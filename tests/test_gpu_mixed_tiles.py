@@ -9,7 +9,7 @@ import pytest
 import torch
 
 import oracle as O
-from helpers import dev_bf16, dev_u8, gpu_quantized_to_numpy, mismatch_report
+from helpers import captured_launches, dev_bf16, dev_u8, gpu_quantized_to_numpy, mismatch_report
 from paper_2605_19561_b200 import inputs as I
 from paper_2605_19561_b200 import torq
 import test_gpu_mxint4 as TI
@@ -270,3 +270,53 @@ def test_rotation_gives_a_short_last_wave_to_the_few_token_kernel(M, d):
     rr, cc = np.meshgrid(np.arange(M), np.arange(d // 32), indexing="ij")
     raw[O.scale_layout_offset(rr, cc, d)] = 0
     assert not raw.any()
+
+
+# More 256-column tiles than one wave has pairs, so the pair kernel whatever the cost model says: narrow tiles of both kinds in a last row tile
+# whose second CTA has no token, a few, and nearly all; the last tile of a pair narrow behind a wide one.
+@pytest.mark.parametrize("M,d", [(3600, 2048), (3700, 2048), (4500, 1792), (2843, 2560)])
+def test_rotation_narrow_tiles_in_a_ragged_last_row_tile_of_the_pair_kernel(M, d):
+    """Permutations of small integers: codes, scales and padding equal the oracle's bit for bit in the three formats, and it is the pair
+    kernel that ran."""
+    if _pairs() == 74:
+        tl = torq.torq_pair_tile_list(M, d, _pairs())
+        last_row = [(c, w) for mp, c, w in tl if mp == (M + 255) // 256 - 1]
+        assert {c % 128 for c, w in last_row if w == 192} == {0, 64}
+    g = np.random.default_rng(M)
+    xb = I.to_bf16_bits(g.integers(-8, 9, size=(M, d)).astype(np.float64))
+    perm = g.permutation(d)
+    P = torch.zeros((d, d), dtype=torch.bfloat16, device="cuda")
+    P[torch.arange(d, device="cuda"), torch.from_numpy(perm).cuda()] = 1
+    y = np.empty((M, d))
+    y[:, perm] = O.decode_bf16(xb)
+    X = dev_bf16(xb)
+
+    def check(call, kernel, quantized, ref):
+        codes, scales = call()
+        torch.cuda.synchronize()
+        if _pairs() == 74:
+            assert kernel in captured_launches(call)[0][0]
+        got, got_sb = quantized(codes, scales)
+        assert np.array_equal(got, ref[0]) and np.array_equal(got_sb, ref[1])
+        return scales
+
+    for width in (None, 16, 32):                             # no rotation inside the blocks, a permutation of each
+        z, Ri = y, None
+        if width is not None:
+            pin = np.stack([np.eye(width)[g.permutation(width)] for _ in range(d // width)])
+            z = np.einsum("mbk,bkj->mbj", y.reshape(M, d // width, width), pin).reshape(M, d)
+            Ri = dev_bf16(I.to_bf16_bits(pin))
+        z = z.astype(np.float32)
+        if width != 16:
+            o = O.quantize_mxfp4(z)
+            s = check(lambda: torq.torq_rotate_quantize(X, P, Ri), "rotate_quantize_pair_kernelILi0E",
+                      lambda c, s: gpu_quantized_to_numpy(c, s, M, d), o)
+            assert np.array_equal(s.cpu().numpy(), O.swizzle_scales(o[1], d, fill=0))       # padding rows hold zero
+            check(lambda: torq.torq_rotate_quantize_mxint4(X, P, Ri), "rotate_quantize_pair_kernelILi2E",
+                  lambda c, s: (TI._operand_to_int(c), O.unswizzle_scales(s.cpu().numpy(), M, d)), O.quantize_mxint4(z))
+        if width != 32:
+            ts = O.tensor_scale_from_amax(np.abs(z).max())
+            Ri32 = None if Ri is None else torq.torq_expand_intra16(Ri)
+            check(lambda: torq.torq_rotate_quantize_nvfp4(X, P, Ri32, float(ts)), "rotate_quantize_pair_kernelILi1E",
+                  lambda c, s: TN._to_numpy(c, s, M, d), O.quantize_nvfp4(z, ts))
+    assert torq.torq_last_device_error() == 0
