@@ -93,3 +93,31 @@ def test_gemm_of_exact_sums_in_the_three_formats(M, N, K):
     assert (got == O.gemm_nvfp4(ac, asb, 0.25, wc, wsb, 2.0)).all()      # multiples of 2^-4 up to 36 x 4 K: below 2^24 units
     aq, wq = (g.integers(-7, 8, size=(r, K)).astype(np.int8) for r in (M, N))
     assert (TI._gpu_gemm(aq, one(M), wq, one(N), torch.float32) == O.gemm_mxint4(aq, one(M), wq, one(N))).all()
+
+
+@pytest.mark.parametrize("M,d,kernel", [(6, 2048, "rotate_fewtok_kernelILi0ELi1ELb1ELi5E"), (30, 2560, "rotate_fewtok_kernelILi0ELi1ELb1ELi4E"),
+                                        (50, 2560, "rotate_fewtok_kernelILi0ELi1ELb1ELi3E"), (100, 2304, "rotate_fewtok_kernelILi0ELi2ELb0ELi4E"),
+                                        (128, 1024, "rotate_quantize_wide_kernelILi0ELi32E"), (300, 2048, "rotate_quantize_wide_kernelILi0ELi128E"),
+                                        (1000, 4096, "rotate_quantize_wide_kernelILi0ELi256E"), (1100, 4096, "rotate_quantize_wide_kernelILi0ELi384E"),
+                                        (3600, 2048, "rotate_quantize_pair_kernelILi0E")])
+def test_every_rotation_keeps_what_is_not_a_number_in_its_token(M, d, kernel):
+    """The same with R_intra, through each kernel and each form of the intra rotation: the pieces of the pushed sums, the split terms in
+    tensor memory (the one-wave kernel, the pair kernel's last tiles), the warp-level instructions, the FMAs."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the rules are those of 148 SMs")
+    g = np.random.default_rng(M)
+    x = g.integers(-8, 9, size=(M, d)).astype(np.float64)
+    X = dev_bf16(I.to_bf16_bits(x))
+    bad = {1, M // 2, M - 2}
+    X[1, 5], X[M // 2, d - 40], X[M - 2, d // 2] = float("inf"), float("nan"), float("-inf")
+    E = torch.eye(d, dtype=torch.bfloat16, device="cuda")
+    Ri = dev_bf16(I.to_bf16_bits(np.stack([np.eye(32)[g.permutation(32)] for _ in range(d // 32)])))
+    clean, clean_s = torq.torq_rotate_quantize(dev_bf16(I.to_bf16_bits(x)), E, Ri)
+    codes, scales = torq.torq_rotate_quantize(X, E, Ri)
+    torch.cuda.synchronize()
+    assert kernel in captured_launches(lambda: torq.torq_rotate_quantize(X, E, Ri))[0][0]
+    same = torch.tensor([m for m in range(M) if m not in bad], device="cuda")
+    assert torch.equal(codes.view(M, -1)[same], clean.view(M, -1)[same])
+    a, b = (O.unswizzle_scales(t.cpu().numpy(), M, d)[same.cpu().numpy()] for t in (scales, clean_s))
+    assert np.array_equal(a, b)
+    assert torq.torq_last_device_error() == 0
