@@ -6,7 +6,7 @@ import pytest
 import torch
 
 import oracle as O
-from helpers import captured_launches, dev_bf16, gpu_quantized_to_numpy
+from helpers import captured_launches, dev_bf16, dev_u8, gpu_quantized_to_numpy
 from paper_2605_19561_b200 import inputs as I
 from paper_2605_19561_b200 import torq
 import test_gpu_fewtok as TF
@@ -14,6 +14,7 @@ import test_gpu_mxint4 as TI
 import test_gpu_nvfp4 as TN
 
 pytestmark = pytest.mark.gpu
+E2M1 = np.array([0, .5, 1, 1.5, 2, 3, 4, 6, 0, -.5, -1, -1.5, -2, -3, -4, -6])
 
 
 @pytest.mark.parametrize("M,d", [(1, 128), (2, 256), (3, 19072), (4, 640), (5, 1536), (7, 2560), (8, 5120), (9, 4096), (12, 7168), (13, 9600),
@@ -93,6 +94,37 @@ def test_gemm_of_exact_sums_in_the_three_formats(M, N, K):
     assert (got == O.gemm_nvfp4(ac, asb, 0.25, wc, wsb, 2.0)).all()      # multiples of 2^-4 up to 36 x 4 K: below 2^24 units
     aq, wq = (g.integers(-7, 8, size=(r, K)).astype(np.int8) for r in (M, N))
     assert (TI._gpu_gemm(aq, one(M), wq, one(N), torch.float32) == O.gemm_mxint4(aq, one(M), wq, one(N))).all()
+
+
+# Above 16 tokens sums are pushed from K > 2048 on, up to 32 tokens, NVFP4 24: both sides of each line, for a few tiles (clusters of eight)
+# and for many (one to four CTAs, so several pieces per warp and both reads of the accumulator).
+@pytest.mark.parametrize("M,N,K", [(17, 264, 4096), (20, 1032, 2176), (24, 264, 4096), (25, 520, 2176), (28, 264, 4096), (32, 264, 2176),
+                                   (17, 6144, 4096), (20, 6152, 2176), (24, 6144, 4096), (25, 6144, 4096), (28, 5128, 5120), (32, 6144, 4096),
+                                   (17, 20480, 2176), (24, 20480, 2176), (32, 20488, 2176), (32, 6144, 2048), (17, 264, 2048), (33, 6144, 4096)])
+def test_gemm_of_17_to_32_tokens_on_both_sides_of_the_line(M, N, K):
+    g = np.random.default_rng(M + N + K)
+    s32 = lambda r: dev_u8(O.swizzle_scales(np.full((r, K // 32), 127, np.uint8), K, fill=0))
+
+    def check(fmt, most, call, ref):
+        y = call()
+        (name, _), = captured_launches(call)
+        assert f"gemm_fewtok_kernelILi{fmt}ELi1ELb{int(M <= most and K > 2048)}E" in name, name
+        assert np.array_equal(y.cpu().numpy(), ref.astype(np.float32)), name
+
+    ac, wc = g.integers(0, 16, (M, K), dtype=np.uint8), g.integers(0, 16, (N, K), dtype=np.uint8)
+    a, w = dev_u8(O.pack_codes(ac)), dev_u8(O.pack_codes(wc))
+    av, wv = E2M1[ac], E2M1[wc]
+    ops = (a, s32(M), w, s32(N))
+    check(0, 32, lambda: torq.torq_mxfp4_gemm(*ops, out_dtype=torch.float32), av.astype(np.float64) @ wv.T)      # multiples of 1/4 up to 36 K
+    asb, wsb = (g.integers(0, 2, (r, K // 16), dtype=np.uint8) for r in (M, N))                                    # E4M3 1 and 2
+    opn = (a, dev_u8(O.nv_swizzle_scales((0x38 + 8 * asb).astype(np.uint8), K)), 1.0, w, dev_u8(O.nv_swizzle_scales((0x38 + 8 * wsb).astype(np.uint8), K)), 1.0)
+    scaled = lambda v, sb: v * np.repeat(1.0 + sb, 16, axis=1)
+    check(1, 24, lambda: torq.torq_nvfp4_gemm(*opn, out_dtype=torch.float32), scaled(av, asb) @ scaled(wv, wsb).T)  # up to 144 K
+    ai, wi = (g.integers(-7, 8, (r, K)).astype(np.int8) for r in (M, N))
+    opi = (dev_u8(O.int4_to_e4m3(ai)), s32(M), dev_u8(O.int4_to_e4m3(wi)), s32(N))
+    check(2, 32, lambda: torq.torq_mxint4_gemm(*opi, out_dtype=torch.float32), ai.astype(np.float64) @ wi.T.astype(np.float64))
+    torch.cuda.synchronize()
+    assert torq.torq_last_device_error() == 0
 
 
 @pytest.mark.parametrize("M,d,kernel", [(6, 2048, "rotate_fewtok_kernelILi0ELi1ELb1ELi5E"), (30, 2560, "rotate_fewtok_kernelILi0ELi1ELb1ELi4E"),
