@@ -32,6 +32,7 @@
 // memory as the A operand of step 3, wait for the token's six MMAs, read D2, quantize, store.
 #pragma once
 #include <cuda_bf16.h>
+#include "l2_requests.cuh"
 #include "nvfp4_quantize.cuh"
 #include "mxint4_quantize.cuh"
 #include "sm100_ptx.cuh"
@@ -59,7 +60,7 @@ struct RotStructCfg {
 };
 
 // tmRB: R_B [B, B] bf16, box [128 x 64], 128-byte swizzle.  tmX3: X as (k, token, block), box (32, 1, 64),
-// 64-byte swizzle.
+// 64-byte swizzle.  R_B: the matrix itself, which the L2 is asked for.
 // FMT_NVFP4: the NVFP4 quantizer at the end (two 16-element blocks per row of 32, E4M3 scales,
 // `tensor_scale` the tensor's float32 scale; unused for MXFP4); R_intra stays a 32 x 32 matrix (two
 // 16 x 16 blocks on its diagonal for a 16-wide intra rotation).  FMT_MXINT4: integer codes as one E4M3
@@ -67,8 +68,8 @@ struct RotStructCfg {
 template <int FMT = FMT_MXFP4>
 __global__ void __launch_bounds__(608, 1)
 rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_constant__ CUtensorMap tmX3,
-                         const __nv_bfloat16* __restrict__ R_intra, uint8_t* __restrict__ codes,
-                         uint8_t* __restrict__ scales, int M, int d, float tensor_scale, int* err_word) {
+                         const __nv_bfloat16* __restrict__ R_B, const __nv_bfloat16* __restrict__ R_intra,
+                         uint8_t* __restrict__ codes, uint8_t* __restrict__ scales, int M, int d, float tensor_scale, int* err_word) {
   using C = RotStructCfg;
   constexpr int BN = C::BN;
   extern __shared__ uint8_t smem_raw[];
@@ -193,14 +194,18 @@ rotate_structured_kernel(const __grid_constant__ CUtensorMap tmRB, const __grid_
     constexpr uint32_t idesc2 = idesc_bf16(128, 32, /*A MN-major*/ false, /*B MN-major*/ true);
     const uint64_t rdesc = make_desc(ri_base, 2048, 512, kSwizzle64);
     // Until the kernel before has completed HBM idles: the L2 is asked for the first tile's X, one 4-KiB box per lane, and for R_B where
-    // it is one strip (with two or more the order in which they then run costs more: 4096 x 5120 -> 1024 37.1 / 38.6 us).  Here and
-    // not ahead of the roles, whose instructions would lie further apart (64 x 256 -> 256 6.54 / 6.62).  us, without / with, layers:
-    // 2048 x 4096 -> 6144 34.4 / 33.5, 300 x 4096 -> 4096 12.1 / 11.8.
-    // Whole boxes only: one that reaches beyond the tensor took the call 1 to 3 us (2025 x 256 -> 4096, 8 of a box's 64 blocks, 15.9 / 18.9;
-    // 9990 x 1280 -> 1424, 40 of 64, 41.0 / 41.8).
+    // it is one strip, d <= 4096 (with two or more the order in which they then run costs more: 4096 x 5120 -> 1024 37.1 / 38.6 us).
+    // Here and not ahead of the roles, whose instructions would lie further apart (64 x 256 -> 256 6.54 / 6.62).  us, without / with,
+    // layers: 2048 x 4096 -> 6144 34.4 / 33.5, 300 x 4096 -> 4096 12.1 / 11.8.
+    // Whole boxes of X only: one that reaches beyond the tensor took the call 1 to 3 us (2025 x 256 -> 4096, 8 of a box's 64 blocks,
+    // 15.9 / 18.9; 9990 x 1280 -> 1424, 40 of 64, 41.0 / 41.8).  R_B therefore as the contiguous bytes that it is and not in the 128-row
+    // boxes of its loads, which fit d = 4096 alone (us, boxes there and nothing below it / bytes: 2048 x 4096 -> 6144 32.78 / 32.75,
+    // 4000 x 3840 -> 2048 31.33 / 31.22, 300 x 2048 -> 2048 9.41 / 9.37, 9990 x 1280 -> 1424 40.49 / 40.29, 2000 x 1536 -> 1536 14.19 / 14.22).
     const int token = blockIdx.x / b_tiles * C::TOK + (lane & 3);
     if (((lane >> 2) + 1) * C::BK <= nblocks && token < M) tma_prefetch_l2_3d(&tmX3, 0, token, (lane >> 2) * C::BK);
-    if (nblocks == C::BM && lane < k_tiles) tma_prefetch_l2_2d(&tmRB, lane * C::BK, 0);
+    if (b_tiles == 1 && lane_share_bytes(lane, 2 * nblocks * nblocks) > 0)      // at most 32 KiB
+      bulk_prefetch_l2(reinterpret_cast<const uint8_t*>(R_B) + lane_share_first(lane, 2 * nblocks * nblocks),
+                       (uint32_t)lane_share_bytes(lane, 2 * nblocks * nblocks));
     __syncwarp();
     griddep_wait();
     uint32_t tcount = 0;

@@ -145,6 +145,10 @@ __device__ __forceinline__ void tma_prefetch_l2_3d(const CUtensorMap* m, int32_t
   asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];"
                ::"l"(reinterpret_cast<uint64_t>(m)), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
+// The same for contiguous memory: address and size multiples of 16 bytes.
+__device__ __forceinline__ void bulk_prefetch_l2(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "r"(bytes) : "memory");
+}
 // 3-D tiled load (c0 innermost), same rules.
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* m, int32_t c0, int32_t c1,
                                             int32_t c2, uint32_t bar) {

@@ -779,15 +779,15 @@ static torq_status rotate_structured_impl(const void* X, const void* R_B, const 
   const int grid = (int)(tiles < most ? tiles : most);
   if (fmt == FMT_MXINT4)
     launch_tc(rotate_structured_kernel<FMT_MXINT4>, 1, grid, RotStructCfg::THREADS, RotStructCfg::SMEM_BYTES, s, tmRB,
-              tmX3, static_cast<const __nv_bfloat16*>(R_intra), static_cast<uint8_t*>(out_codes),
+              tmX3, static_cast<const __nv_bfloat16*>(R_B), static_cast<const __nv_bfloat16*>(R_intra), static_cast<uint8_t*>(out_codes),
               static_cast<uint8_t*>(out_scales), (int)M, (int)d, 0.0f, st->err_word);
   else if (fmt == FMT_NVFP4)
     launch_tc(rotate_structured_kernel<FMT_NVFP4>, 1, grid, RotStructCfg::THREADS, RotStructCfg::SMEM_BYTES, s, tmRB,
-              tmX3, static_cast<const __nv_bfloat16*>(R_intra), static_cast<uint8_t*>(out_codes),
+              tmX3, static_cast<const __nv_bfloat16*>(R_B), static_cast<const __nv_bfloat16*>(R_intra), static_cast<uint8_t*>(out_codes),
               static_cast<uint8_t*>(out_scales), (int)M, (int)d, tensor_scale, st->err_word);
   else
     launch_tc(rotate_structured_kernel<FMT_MXFP4>, 1, grid, RotStructCfg::THREADS, RotStructCfg::SMEM_BYTES, s, tmRB,
-              tmX3, static_cast<const __nv_bfloat16*>(R_intra), static_cast<uint8_t*>(out_codes),
+              tmX3, static_cast<const __nv_bfloat16*>(R_B), static_cast<const __nv_bfloat16*>(R_intra), static_cast<uint8_t*>(out_codes),
               static_cast<uint8_t*>(out_scales), (int)M, (int)d, 0.0f, st->err_word);
   return launch_status();
 }
