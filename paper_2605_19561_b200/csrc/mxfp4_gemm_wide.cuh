@@ -245,8 +245,9 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     const int set = (warp - 2) >> 2;
     // Up to 256 tokens HBM idles until the kernel before has completed: the L2 is asked for the next W (us, without / with, layers: 200 x 4096
     // -> 6144 21.5 / 21.2, 256 x 5120 -> 5120 27.9 / 27.5, 256 x 4096 -> 14336 25.9 / 25.8; with more row tiles 400 x 4096 -> 4096 25.8 / 26.1).
-    if (warp == 3 && rows == 1 && elect_one())
-      for (int k = pre * SL; k < min(k_slabs, pre * SL + C::AHEAD); ++k) tma_prefetch_l2_2d(&tmB, k * 128, tcol + (int)rank * (n0 / 2));
+    const int wrow = tcol + (int)rank * (n0 / 2);      // of W; a last tile narrower than half a tile has none for the second CTA
+    if (warp == 3 && rows == 1 && wrow < N && elect_one())
+      for (int k = pre * SL; k < min(k_slabs, pre * SL + C::AHEAD); ++k) tma_prefetch_l2_2d(&tmB, k * 128, wrow);
     __syncwarp();
     griddep_wait();                                    // Y may still be read by that kernel
     if (warp == 2) {                                   // from a warp of its own: not behind the W loads of all these stages

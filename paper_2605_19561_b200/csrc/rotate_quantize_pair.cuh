@@ -232,7 +232,8 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       // Until the kernel before has completed HBM idles: the L2 is asked for the first K steps of X, one per pair and row tile (us,
       // without / with: layer 1500 x 2048 -> 2048 21.2 / 20.9, 2048 x 4096 -> 6144 81.1 / 80.7).
       const int mp_tiles = (M + 255) / 256, kt = pair / (mp_tiles < 8 ? mp_tiles : 8);
-      if (kt < k_tiles) tma_prefetch_l2_2d(&tmX, kt * C::BK, (2 * mp0 + (int)rank) * C::BM);
+      const int row = (2 * mp0 + (int)rank) * C::BM;     // the pair's second row tile may not exist
+      if (kt < k_tiles && row < M) tma_prefetch_l2_2d(&tmX, kt * C::BK, row);
     }
     __syncwarp();
     griddep_wait();

@@ -234,7 +234,9 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       // per pair that shares it, and, for strips of 64 to 128 columns, for the next R_inter, a strip's steps dealt over its row tiles (us,
       // without / X alone / both, layers: 300 x 2048 -> 2048 14.00 / 13.83 / 13.69, 600 x 2048 15.4 / 15.1 / 14.9, 400 x 4096 -> 4096 25.7 /
       // 25.3 / 25.1, 1500 x 2048 22.0 / 21.6; narrower strips lose by R_inter, 220 x 2048 12.73 / 12.60 / 12.71).  Calls long enough to run
-      // at the power cap lose (loops of 0.6 s, 1024 x 4096 44.4 / 44.7 / 45.0, 777 x 5120 60.7 / 60.8).
+      // at the power cap lose (loops of 0.6 s, 1024 x 4096 44.4 / 44.7 / 45.0, 777 x 5120 60.7 / 60.8).  A box wholly beyond the last token or
+      // feature fetches nothing; to leave it out costs more (without / with that guard: 300 x 2048 -> 2048 12.77 / 12.81, 1000 x 2048
+      // -> 2048 15.48 / 15.53, 100 x 2048 -> 2048 12.00 / 12.02, three turns each that agree within 0.02).
       if (width * d <= 128 * 4096 && pair / rows < k_tiles) tma_prefetch_l2_3d(&tmX, 0, mt * C::BM, pair / rows * (BK / C::SLAB));
       if (RANGE == 128 && width >= 64)
         for (int kt = pre + pair % rows; kt < min(k_tiles, pre + C::AHEAD); kt += rows)

@@ -4,6 +4,8 @@ import os
 import re
 import subprocess
 
+import pytest
+
 from test_pair_handshake import CSRC, _conditions
 
 
@@ -39,3 +41,15 @@ def test_the_structured_rotation_asks_for_r_b_wherever_it_is_one_strip():
     assert len(asks) == 1
     sizes = {t for t in _conditions(body, asks[0]) if re.search(r"nblocks|b_tiles|k_tiles|\bd\b", t)}
     assert sizes == {"b_tiles == 1", "lane_share_bytes lane, 2 * nblocks * nblocks > 0"}, sizes
+
+
+@pytest.mark.parametrize("name,tensor,extent", [("rotate_quantize_pair.cuh", "tmX", "M"), ("mxfp4_gemm_wide.cuh", "tmB", "N"),
+                                                ("rotate_structured.cuh", "tmX3", "M")])
+def test_no_box_that_lies_wholly_outside_its_tensor_is_asked_for(name, tensor, extent):
+    """Tiles go on beyond the last token, feature or row of W: a CTA whose part of a tile begins there asks for nothing.  (The one-wave rotation
+    does ask, and the L2 then has nothing to fetch: the guard costs its short calls more than the request.)"""
+    body = re.sub(r"//.*", "", open(os.path.join(CSRC, name)).read())
+    asks = [m.start() for m in re.finditer(r"tma_prefetch_l2_\wd\(&%s," % tensor, body)]
+    assert asks
+    for at in asks:
+        assert any(t.endswith(" < " + extent) for t in _conditions(body, at)), _conditions(body, at)
