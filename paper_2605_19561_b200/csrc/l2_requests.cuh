@@ -17,4 +17,8 @@ TORQ_ASK_HD int lane_share_bytes(int lane, int bytes) {
   return first >= bytes ? 0 : (next < bytes ? next : bytes) - first;
 }
 
+// K step of X that the pair of CTAs with this first tile asks for.  The pairs of one row tile have its columns from the first on, so
+// each asks for another step and together for the first ones; a narrow tile lies behind the row's wide ones.
+TORQ_ASK_HD int x_step_of_tile(int first_column, bool narrow) { return first_column / (narrow ? 192 : 256); }
+
 }  // namespace torq

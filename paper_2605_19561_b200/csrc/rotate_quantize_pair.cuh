@@ -18,6 +18,7 @@
 // acc_empty[a] lives in the leader and takes one arrival per epilogue warp of both CTAs (16).
 #pragma once
 #include <cuda_bf16.h>
+#include "l2_requests.cuh"
 #include "nvfp4_quantize.cuh"
 #include "mxint4_quantize.cuh"
 #include "pair_handshake.cuh"
@@ -229,9 +230,10 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
     }
   } else {
     if (warp == 3 && elect_one()) {
-      // Until the kernel before has completed HBM idles: the L2 is asked for the first K steps of X, one per pair and row tile (us,
-      // without / with: layer 1500 x 2048 -> 2048 21.2 / 20.9, 2048 x 4096 -> 6144 81.1 / 80.7).
-      const int mp_tiles = (M + 255) / 256, kt = pair / (mp_tiles < 8 ? mp_tiles : 8);
+      // Until the kernel before has completed HBM idles: the L2 is asked for the first K steps of X, each pair of a row tile for one
+      // (us, without / with: layer 1500 x 2048 -> 2048 21.2 / 20.9, 2048 x 4096 -> 6144 81.1 / 80.7).  The step by the tile's column: by
+      // the pair's number, the pairs of the second eight row tiles asked for later ones (8192 x 1024 -> 1024 32.9 / 32.6).
+      const int kt = x_step_of_tile(tcol0, narrow0);
       const int row = (2 * mp0 + (int)rank) * C::BM;     // the pair's second row tile may not exist
       if (kt < k_tiles && row < M) tma_prefetch_l2_2d(&tmX, kt * C::BK, row);
     }

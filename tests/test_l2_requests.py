@@ -6,6 +6,7 @@ import subprocess
 
 import pytest
 
+from paper_2605_19561_b200 import torq
 from test_pair_handshake import CSRC, _conditions
 
 
@@ -53,3 +54,26 @@ def test_no_box_that_lies_wholly_outside_its_tensor_is_asked_for(name, tensor, e
     assert asks
     for at in asks:
         assert any(t.endswith(" < " + extent) for t in _conditions(body, at)), _conditions(body, at)
+
+
+@pytest.mark.parametrize("M,d", [(1500, 2048), (2048, 4096), (2300, 2048), (3600, 2048), (4096, 2304), (4500, 1792), (8192, 1024), (16384, 512), (2048, 14336)])
+def test_pairs_of_one_row_tile_ask_for_its_first_k_steps(M, d, tmp_path):
+    """The first wave's tiles: in every row tile each pair asks for another step, and those of wide tiles for the first ones without a gap."""
+    tiles = torq.torq_pair_tile_list(M, d, 74)[:74]
+    body = re.sub(r"//.*", "", open(os.path.join(CSRC, "rotate_quantize_pair.cuh")).read())
+    assert re.search(r"kt = x_step_of_tile\(tcol0, narrow0\);\s+[^}]*tma_prefetch_l2_2d\(&tmX, kt \* ", body)
+    rows = "".join("{%d, %d, %d}," % t for t in tiles)
+    _run(tmp_path, r"""
+  const struct { int mp, col, width; } t[] = {""" + rows + r"""};
+  for (const auto& a : t) {
+    const int step = torq::x_step_of_tile(a.col, a.width == 192);
+    int same = 0, before = 0, wide = 0;
+    for (const auto& b : t)
+      if (b.mp == a.mp) {
+        same += torq::x_step_of_tile(b.col, b.width == 192) == step;
+        before += torq::x_step_of_tile(b.col, b.width == 192) < step;
+        wide += b.width == 192;
+      }
+    if (same != 1 || (wide == 0 && before != step)) { std::printf("row tile %d column %d: step %d\n", a.mp, a.col, step); return 1; }
+  }
+""")
