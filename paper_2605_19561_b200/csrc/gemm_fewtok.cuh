@@ -9,7 +9,7 @@
 // A layer has only N / 128 such tiles (40 at N = 5120), so K is split as well: a CLUSTER of S CTAs
 // shares one tile, CTA r contracts k range r; the fp32 partial tiles stay on the SMs and are added in rank order (fixed).
 // As in the few-token rotation they reach the adding CTA in one of two ways:
-//  * PUSH (up to 32 tokens, NVFP4 24): the sums are dealt over all CTAs and warps of the cluster in pieces of 32 features x 4 tokens, and
+//  * PUSH (up to 16 tokens, for K > 2048 up to 32, NVFP4 24): the sums are dealt over all CTAs and warps of the cluster in pieces of 32 features x 4 tokens, and
 //    every CTA stores its partials of a piece straight from registers into the owner's shared memory (st.async, 16 bytes per lane = four
 //    tokens of one feature, counted on a barrier of the owning warp), into room of their own.  K = N = 5120, us: pulled 1 token 4.7,
 //    24 tokens 5.6; pushed to one owner per four tokens, into its stages, 4.4 and 16 tokens 4.95; so 4.4, 4.7 and 24 tokens 5.25.

@@ -332,14 +332,12 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, bool intra, const Devic
 static bool fewtok_leave_together(int64_t M, int64_t tiles, FewRotation few, const DeviceState* st) {
   return M > 64 && few.stages == RotFewCfg::STAGES && few.cluster == 3 && tiles > st->few_fit[3] - 2;
 }
-// Cluster size of the few-token GEMM: above S = 4 three K steps per CTA, or two while the partial sums of all CTAs are few: 32
-// tokens per SM (us, S = 4 / 8, 17 and 64 tokens: N = 256, K = 4096 3.44 / 2.99 and 4.33 / 3.92, N = 1024 3.58 / 3.20 and 4.60 /
-// 4.34; S = 4 / 6: 17 tokens N = 2048 3.75 / 3.47; beyond the line 64 tokens N = 2048 NVFP4 4.53 / 4.70), and 8 up to 16 tokens
-// (1 token N = 256 2.96 / 2.58, N = 1024 3.10 / 2.82, the layer 11.2 / 10.9; beyond: N = 2048 the GEMM 3.62 /
-// 3.51, the layer of 16 tokens 13.2 / 13.5; S = 4 / 5 at K = 2560, N = 5120 the layer 11.0 / 11.5).
+// Cluster size of the few-token GEMM whose sums are pulled (17 tokens and more): above S = 4 three K steps per CTA, or two while the
+// partial sums of all CTAs are few: 32 tokens per SM (us, S = 4 / 8, 17 and 64 tokens: N = 256, K = 4096 3.44 / 2.99 and 4.33 / 3.92,
+// N = 1024 3.58 / 3.20 and 4.60 / 4.34; S = 4 / 6: 17 tokens N = 2048 3.75 / 3.47; beyond the line 64 tokens N = 2048 NVFP4 4.53 / 4.70).
 static int fewtok_gemm_cluster(int ntok, int64_t tiles, int64_t steps, int ctas, const DeviceState* st) {
   const int S = fewtok_cluster(tiles, steps, steps / 2, ctas, st->sm_count, st->few_fit);
-  if (tiles * S * ntok <= (ntok > 16 ? 32 : 8) * (int64_t)st->sm_count) return S;
+  if (tiles * S * ntok <= 32 * (int64_t)st->sm_count) return S;
   return fewtok_cluster(tiles, steps, steps / 3, ctas, st->sm_count, st->few_fit);
 }
 // Where the sums are pushed (M tokens), from the largest cluster down: above four CTAs where each keeps four K steps and has its SM to itself
@@ -347,14 +345,16 @@ static int fewtok_gemm_cluster(int ntok, int64_t tiles, int64_t steps, int ctas,
 // themselves (a tenth may share), or with more than five steps.  us, layers, S = 3 / 4 / 5 / 8: 8 x 5120 -> 5120 (20 steps) 15.35 / 14.5 /
 // 15.0 / 15.2, 16 x 4096 -> 1024 (16) 12.0 / 10.0 / 10.2 / 10.8, 16 x 2048 -> 6144 (8) 8.06 / 8.36, 8 x 8192 -> 2048 (32) 28.0 / 27.1 / 26.4 / 24.4,
 // 16 x 7168 -> 4096 (28), S = 4 / 6 23.25 / 22.3, 16 x 5120 -> 8192, S = 3 / 4 16.5 / 17.1; up to 4 tokens sharing costs less (1 x 5120 -> 5120
-// S = 4 / 5 14.4 / 14.3).  One or two steps are not split (16 tokens, N = 4096, K = 512 2.97 / 2.56), nor are four above 16 tokens (32 tokens
-// N = 8192, K = 1024 4.6 / 3.7).
+// S = 4 / 5 14.4 / 14.3).  One or two steps are not split (16 tokens, N = 4096, K = 512 2.97 / 2.56; above 16 tokens there are nine and more).
+// Few tiles take as many CTAs as have two steps, while the sums are few as above, up to 16 tokens 8 tokens per SM (us, S = 4 / 8: 1 token
+// N = 256 2.96 / 2.58, N = 1024 3.10 / 2.82, the layer 11.2 / 10.9; beyond: N = 2048 the GEMM 3.62 / 3.51, the layer of 16 tokens
+// 13.2 / 13.5; S = 4 / 5 at K = 2560, N = 5120 the layer 11.0 / 11.5).
 static int push_gemm_cluster(int64_t M, int64_t tiles, int64_t steps, const DeviceState* st) {
-  if (steps >= 8) {                          // few tiles: as many CTAs as have two steps, see fewtok_gemm_cluster
+  if (steps >= 8) {
     const int S = fewtok_cluster(tiles, steps, steps / 2, 2, st->sm_count, st->few_fit);
     if (tiles * S * fewtok_ntok(M) <= (M > 16 ? 32 : 8) * (int64_t)st->sm_count) return S;
   }
-  if (steps <= 2 || (M > 16 && steps <= 4 && tiles > 24)) return 1;
+  if (steps <= 2) return 1;
   for (int S = GemmFewCfg<>::MAX_CLUSTER; S > 1; --S) {
     if (S > steps || tiles > st->push_fit[S]) continue;
     const bool alone = 10 * tiles * S <= 11 * (int64_t)st->sm_count;
@@ -813,7 +813,8 @@ torq_status torq_rotate_quantize_structured_nvfp4(const void* X, const void* R_B
 //    do not know: there they are high by up to a third (200 x 4096, K = 14336 17.3 modelled, 13.1 measured; 300 x 4096, K = 4096 7.8,
 //    6.7) and take 192 columns in one slab where 128 in two would fit the pairs too (512 x 4096, K = 14336; 700 x 3072, K = 4096);
 //  * few tokens (17 to 128, S CTAs per tile): 2.3 + 0.2 per K step of the longest split + per token 0.025 with S = 1 (the
-//    accumulator goes to Y), else 0.012 + 0.035 / S;
+//    accumulator goes to Y), else 0.012 + 0.035 / S.  With pulled sums; pushed ones (17 to 32 tokens, K > 2048) take less, and even by these
+//    figures the one-wave kernel is 1.11 times and more their time at every size;
 //  * pair kernel: one wave 4.1 + 0.9 f + (0.285 + 0.04 f) per K step, more (the last one as narrower tiles) 5.2 + per K step
 //    0.325 for a full wave and 0.21 + 0.14 f for the last.
 // The same figures choose for NVFP4, MXINT4 (twice the steps) and float32 output, which were not fitted.  A sweep of 5250 calls, the
