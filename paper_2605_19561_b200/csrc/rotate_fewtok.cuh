@@ -56,7 +56,8 @@ struct RotFewCfg {
   // a CTA and too few loads in flight (the rule stands where the kernel is launched).
   static constexpr int SHARED_STAGES = 3, MAX_SHARED_TOK = 128;
   static constexpr int MAX_TOK = 256;                  // N of the instruction: a multiple of 16
-  static constexpr int MAX_PUSH_TOK = 64;
+  static constexpr int PUSH_TOK = 56;                  // tokens up to which sums are pushed (the rule stands where the kernel is launched)
+  static constexpr int PUSH_NTOK = (PUSH_TOK + 15) / 16 * 16;
   static constexpr int PART_BYTES = 32 * 16;           // pushed partial of a unit from one CTA: [feature of the block][4 tokens]
   static constexpr int Y_BYTES = 16 * 33 * 4;          // pull, per epilogue warp: 16 tokens x 32 features, row stride 33
   static constexpr int RI_BYTES = 32 * 80;             // per epilogue warp: R_intra[block] as bf16 rows of 80 bytes
@@ -77,7 +78,7 @@ struct RotFewCfg {
 // what lies in the stages after the mainloop where partials are pulled: the partial tile (ntok x 512 B) and the y tiles
 static_assert(8 * RotFewCfg::Y_BYTES <= 4 * RotFewCfg::A_BYTES && RotFewCfg::BF * 4 <= RotFewCfg::STAGES * RotFewCfg::BK * 2, "reduction buffers");
 static_assert(RotFewCfg::ctas_per_sm(16, RotFewCfg::PUSH_STAGES, true) == 2 && RotFewCfg::ctas_per_sm(32, RotFewCfg::STAGES, true) == 2 &&
-              RotFewCfg::ctas_per_sm(RotFewCfg::MAX_PUSH_TOK, RotFewCfg::SHARED_STAGES, true) == 2, "two CTAs per SM where sums are pushed");
+              RotFewCfg::ctas_per_sm(RotFewCfg::PUSH_NTOK, RotFewCfg::SHARED_STAGES, true) == 2, "two CTAs per SM where sums are pushed");
 static_assert(RotFewCfg::ctas_per_sm(RotFewCfg::MAX_SHARED_TOK, RotFewCfg::SHARED_STAGES, false) == 2 &&
               4 * RotFewCfg::Y_BYTES + 80 * RotFewCfg::BF * 4 <= RotFewCfg::SHARED_STAGES * RotFewCfg::stage_bytes(80) &&
               4 * RotFewCfg::Y_BYTES + 128 * RotFewCfg::BF * 4 <= RotFewCfg::SHARED_STAGES * RotFewCfg::stage_bytes(128), "three stages");

@@ -163,7 +163,7 @@ static DeviceState* device_state() {
       st.few_fit[s] = max_active_clusters(rotate_fewtok_kernel<FMT_MXFP4, 2>, s, 320, RotFewCfg::smem_bytes(256, RotFewCfg::STAGES, false), st.sm_count);
     for (int s = 1; s <= RotFewCfg::MAX_CLUSTER; ++s)
       st.push_fit[s] = max_active_clusters(fewtok_fit_kernel, s, RotFewCfg::THREADS,
-                                           RotFewCfg::smem_bytes(RotFewCfg::MAX_PUSH_TOK, RotFewCfg::SHARED_STAGES, true), st.sm_count);
+                                           RotFewCfg::smem_bytes(RotFewCfg::PUSH_NTOK, RotFewCfg::SHARED_STAGES, true), st.sm_count);
     cudaGetLastError();
   }
   st.ready = true;
@@ -281,17 +281,15 @@ static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int64_t most, i
   while (s > 1 && (k_steps + s - 2) / (s - 1) == (k_steps + s - 1) / s) --s;      // fewer clusters' CTAs: they fit as well
   return s < 1 ? 1 : s;
 }
+// R_inter or W tiles (16 KiB) that all CTAs together ask the L2 for beyond their stages: 10 MB (us, 0 / 3 / 4 / 6 / 16 per CTA of 200,
+// d = N = 5120, 1 token 14.8 / 14.3 / 14.25 / 14.4 / 15.7; of 192, 24 tokens d = 4096 NVFP4 3 / 4 / 6: 13.5 / 13.8 / 14.0; of 128, 100
+// tokens d = 4096 0 / 3 / 5 / 8: 18.4 / 18.2 / 18.1 / 18.2).
+constexpr int kAheadTiles = 640;
 // Cluster size and stages of the few-token rotation.  65 to 128 tokens have an SM to themselves with four stages and share
 // it with three.  Sharing wins where the K range of a CTA would be longer than 32 steps, that is where 148 CTAs are few for
 // the tiles (us, alone / shared, 72 and 128 tokens: d = 5120, 27 steps 14.2 / 14.7 and 16.2 / 17.7; d = 6400, 50 steps 21.7 /
 // 19.9 and 23.4 / 22.0; d = 8192 28.0 / 26.4 and 30.3 / 28.0; d = 11008, one CTA for each of 86 tiles 52.0 / 41.1 and 53.6 /
 // 44.4; d = 14336 78 / 68 and 79 / 73).
-// R_inter or W tiles (16 KiB) that all CTAs together ask the L2 for beyond their stages: 10 MB (us, 0 / 3 / 4 / 6 / 16 per CTA of 200, d = N = 5120,
-// 1 token 14.8 / 14.3 / 14.25 / 14.4 / 15.7; of 192, 24 tokens d = 4096 NVFP4 3 / 4 / 6: 13.5 / 13.8 / 14.0; of 128, 100 tokens
-// d = 4096 0 / 3 / 5 / 8: 18.4 / 18.2 / 18.1 / 18.2).
-constexpr int kAheadTiles = 640;
-constexpr int kPushTokens = 56;
-static_assert(kPushTokens <= RotFewCfg::MAX_PUSH_TOK, "room for pushed sums");
 struct FewRotation { int cluster, stages; bool push; };
 static FewRotation fewtok_rotation(int64_t M, int64_t d, bool intra, const DeviceState* st) {
   const int ntok = fewtok_ntok(M);
@@ -304,7 +302,7 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, bool intra, const Devic
   // Above 32 tokens (three stages then) where clusters of eight fit, up to 56: us, layers, pulled / pushed, 40 tokens: 2048 -> 2048 10.65 / 10.1, 4096 ->
   // 4096 15.85 / 15.1, 56 tokens 2560 -> 2560 13.25 / 12.15, 64 tokens 11.3 / 11.8 and 16.9 / 16.9; d = 5120, S = 6, 50 tokens 19.4 / 19.8.  Above 48
   // from 20 tiles on (56 tokens NVFP4 2048 -> 2048 10.96 / 11.6).
-  if (intra && (M <= 32 || (M <= (tiles < 20 ? 48 : kPushTokens) && tiles <= st->push_fit[RotFewCfg::MAX_CLUSTER] - 2))) {
+  if (intra && (M <= 32 || (M <= (tiles < 20 ? 48 : RotFewCfg::PUSH_TOK) && tiles <= st->push_fit[RotFewCfg::MAX_CLUSTER] - 2))) {
     int S = (int)(steps < RotFewCfg::MAX_CLUSTER ? steps : RotFewCfg::MAX_CLUSTER);
     while (S > 1 && tiles > st->push_fit[S] - 2) --S;
     return {S, ntok > 32 ? RotFewCfg::SHARED_STAGES : (ntok <= 16 && steps <= 32 * S ? RotFewCfg::PUSH_STAGES : RotFewCfg::STAGES), true};
