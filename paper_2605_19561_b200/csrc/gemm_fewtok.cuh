@@ -9,10 +9,11 @@
 // A layer has only N / 128 such tiles (40 at N = 5120), so K is split as well: a CLUSTER of S CTAs
 // shares one tile, CTA r contracts k range r; the fp32 partial tiles stay on the SMs and are added in rank order (fixed).
 // As in the few-token rotation they reach the adding CTA in one of two ways:
-//  * PUSH (up to 16 tokens, for K > 2048 up to 32, NVFP4 24): the sums are dealt over all CTAs and warps of the cluster in pieces of 32 features x 4 tokens, and
-//    every CTA stores its partials of a piece straight from registers into the owner's shared memory (st.async, 16 bytes per lane = four
-//    tokens of one feature, counted on a barrier of the owning warp), into room of their own.  K = N = 5120, us: pulled 1 token 4.7,
-//    24 tokens 5.6; pushed to one owner per four tokens, into its stages, 4.4 and 16 tokens 4.95; so 4.4, 4.7 and 24 tokens 5.25.
+//  * PUSH (up to 16 tokens, for K > 2048 up to 32, NVFP4 24): the sums are dealt over all CTAs and warps of the cluster in pieces of 32
+//    features x 4 tokens, and every CTA stores its partials of a piece straight from registers into the owner's shared memory (st.async,
+//    16 bytes per lane = four tokens of one feature, counted on a barrier of the owning warp), into room of their own.  K = N = 5120, us:
+//    pulled 1 token 4.7, 24 tokens 5.6; pushed to one owner per four tokens, into its stages, 4.4 and 16 tokens 4.95; so 4.4, 4.7 and 24
+//    tokens 5.25.
 //  * pull (more tokens): each CTA writes its partial [token][feature] into its own shared memory, a cluster barrier
 //    publishes them, and CTA r adds, for the tokens m = r (mod S), the S partials read with 16-byte ld.shared::cluster.
 // With S = 1 (an ordinary launch without clusters) the accumulator goes to Y directly.
@@ -52,8 +53,8 @@ struct GemmFewCfg {
   __host__ __device__ static constexpr int push_bytes(int M) { return ((M + 3) / 4 * 4 + MAX_CLUSTER - 1) * PART_BYTES; }
   __host__ __device__ static constexpr int pull_smem_bytes(int M) { return STAGES * stage_bytes((M + 15) / 16 * 16) + BAR_BYTES + 1024; }
   // Pushed where the room for what arrives leaves two CTAs per SM (NVFP4: up to 24 tokens); from 17 tokens on for contractions long enough
-  // that a cluster of four has work for it (us, pulled / pushed, 32 tokens: N = 4096, K = 2048 3.72 / 4.01, K = 4096 4.47 / 4.49, K = 14336 8.82 /
-  // 7.93, layers 4096 x 4096 13.7 / 13.2, 2048 x 4096 9.1 / 9.3; 18 tokens N = K = 5120 5.31 / 4.83).
+  // that a cluster of four has work for it (us, pulled / pushed, 32 tokens: N = 4096, K = 2048 3.72 / 4.01, K = 4096 4.47 / 4.49, K =
+  // 14336 8.82 / 7.93, layers 4096 x 4096 13.7 / 13.2, 2048 x 4096 9.1 / 9.3; 18 tokens N = K = 5120 5.31 / 4.83).
   __host__ __device__ static constexpr bool push(int M, int K) {
     return M <= 16 || (M <= MAX_PUSH_TOK && K > 2048 && pull_smem_bytes(M) + push_bytes(M) <= 113 * 1024);
   }
@@ -67,10 +68,10 @@ struct GemmFewCfg {
 };
 
 // grid = ceil(N / 128) * S CTAs in clusters of S along x: CTA b works feature tile b / S, k split b % S.
-// w_ahead: W tiles beyond the stages that a CTA asks the L2 for.  tmW: Wq [N, K bytes] box [128 x 128]; tmA: Aq [M, K bytes] box [ntok x 128]; As / Ws: tiled scales.
+// w_ahead: W tiles beyond the stages that a CTA asks the L2 for.  tmW: Wq [N, K bytes] box [128 x 128]; tmA: Aq [M, K bytes] box [ntok x
+// 128]; As / Ws: tiled scales.
 // ESETS: sets of four epilogue warps (threads = 64 + 128 ESETS): one set and two CTAs per SM up to 64 tokens (MXINT4: 80, where
-// that splits K further);
-// two sets above, where a CTA fills an SM by itself and has some forty tokens to add up and store.
+// that splits K further); two sets above, where a CTA fills an SM by itself and has some forty tokens to add up and store.
 template <int FMT = FMT_MXFP4, int ESETS = 1, bool PUSH = false>
 __global__ void __launch_bounds__(64 + 128 * ESETS, ESETS == 1 ? 2 : 1)
 gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmA,
@@ -139,9 +140,9 @@ gemm_fewtok_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   const uint32_t tmem_base = *tmem_slot;
   griddep_launch_dependents();
   const int a_pre = PUSH ? pre : 0;                      // activation tiles that the epilogue warps send
-  // While the kernel before ends HBM idles: the L2 is asked for W beyond the stages (us, without / with, layers: 128 x 4096 -> 6144 19.05 / 18.8,
-  // 100 x 4096 -> 12288 21.9 / 21.6, 16 x 8192 -> 8192 29.65 / 29.5).  By a warp that has time for it, in its own branch: in the way of the
-  // epilogue warps' dry pass the instructions alone cost up to 3 % (56 x 2048 -> 2048 NVFP4 10.76 / 11.1).
+  // While the kernel before ends HBM idles: the L2 is asked for W beyond the stages (us, without / with, layers: 128 x 4096 -> 6144 19.05
+  // / 18.8, 100 x 4096 -> 12288 21.9 / 21.6, 16 x 8192 -> 8192 29.65 / 29.5).  By a warp that has time for it, in its own branch: in the
+  // way of the epilogue warps' dry pass the instructions alone cost up to 3 % (56 x 2048 -> 2048 NVFP4 10.76 / 11.1).
   auto ask = [&]() {
     if (elect_one())
       for (int kt = kt0 + pre; kt < min(kt1, kt0 + pre + w_ahead); ++kt) tma_prefetch_l2_2d(&tmW, kt * 128, nt * C::BF);

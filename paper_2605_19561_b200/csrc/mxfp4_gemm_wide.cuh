@@ -1,6 +1,7 @@
 // Block-scaled GEMM on CTA pairs in ONE wave (17 tokens and more, the sizes that wide_gemm_width picks): every pair
-// works exactly one tile of 256 tokens x `width` output features (a multiple of 64, up to 384), the width chosen so that the tiles just fill the pairs.  The pair
-// kernel deals 256-column tiles and pays a whole wave for a remainder, or leaves pairs idle where there are few.
+// works exactly one tile of 256 tokens x `width` output features (a multiple of 64, up to 384), the width chosen so that the tiles just
+// fill the pairs.  The pair kernel deals 256-column tiles and pays a whole wave for a remainder, or leaves pairs idle where there are
+// few.
 //
 // As in the pair kernel each CTA stages its own 128 rows of A, its half of the tile's rows of W, its own A scales
 // and the whole tile's W scales.  W scales come in chunks of 128 rows (four tensor-memory columns, rows 32 j ... 32 j +
@@ -48,7 +49,8 @@ struct GemmWideCfg {
   // 7.53 / 7.26), from four slabs on.  With few slabs the first stage is waited for longer (40 x 4096, K = 512 2.90 / 3.02), and so
   // it is with four or five where more than 24 pairs read up to 176 tokens and the last slab is a half one, in NVFP4 with more
   // tokens as well, or the pairs are up to 32 (144 x 4096, K = 1152 4.00 / 4.10, 80 x 2048 3.59 / 3.71, 80 x 4096, K = 1024 3.60 /
-  // 3.72, NVFP4 192 x 6144, K = 1152 4.74 / 4.98; beyond the line 112 x 3072, K = 1280 3.77 / 3.70, MXINT4 144 x 6144, K = 640 4.22 / 4.09).
+  // 3.72, NVFP4 192 x 6144, K = 1152 4.74 / 4.98; beyond the line 112 x 3072, K = 1280 3.77 / 3.70, MXINT4 144 x 6144, K = 640 4.22 /
+  // 4.09).
   __host__ __device__ static constexpr bool two_slabs(int64_t M, int64_t K, int64_t pairs) {
     const int64_t k_slabs = (K + BK - 1) / BK;
     if (k_slabs < 4 || k_slabs > 5 || pairs <= 24) return k_slabs >= 4;
@@ -243,8 +245,9 @@ mxfp4_gemm_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     // ------------------------------------------------------------------ epilogue (12 warps per CTA)
     const int q = warp & 3;
     const int set = (warp - 2) >> 2;
-    // Up to 256 tokens HBM idles until the kernel before has completed: the L2 is asked for the next W (us, without / with, layers: 200 x 4096
-    // -> 6144 21.5 / 21.2, 256 x 5120 -> 5120 27.9 / 27.5, 256 x 4096 -> 14336 25.9 / 25.8; with more row tiles 400 x 4096 -> 4096 25.8 / 26.1).
+    // Up to 256 tokens HBM idles until the kernel before has completed: the L2 is asked for the next W (us, without / with, layers: 200 x
+    // 4096 -> 6144 21.5 / 21.2, 256 x 5120 -> 5120 27.9 / 27.5, 256 x 4096 -> 14336 25.9 / 25.8; with more row tiles 400 x 4096 -> 4096
+    // 25.8 / 26.1).
     const int wrow = tcol + (int)rank * (n0 / 2);      // of W; a last tile narrower than half a tile has none for the second CTA
     if (warp == 3 && rows == 1 && wrow < N && elect_one())
       for (int k = pre * SL; k < min(k_slabs, pre * SL + C::AHEAD); ++k) tma_prefetch_l2_2d(&tmB, k * 128, wrow);

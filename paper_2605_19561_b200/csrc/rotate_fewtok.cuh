@@ -12,13 +12,14 @@
 // partials in rank order (fixed order, so the result does not depend on timing), rotates inside the block and quantizes (Eq. 1).
 // The partials reach the owner in one of two ways:
 //  * PUSH (up to 32 tokens, with R_intra and clusters of eight up to 56): the pieces of work are small, 32 features x 4
-//    tokens, and dealt over all CTAs and warps of the cluster, so that nearly every warp has one and no CTA takes in more than its share (what arrives at one SM comes at about 9 B per cycle).  A CTA
-//    stores its partials straight from registers into the owners' shared memory (st.async, 16 bytes per lane = four tokens of one
-//    feature, counted on a barrier of the owning warp), into room of their own: nobody has to say first that the stages there are free, and
-//    no cluster-wide barrier stands on the path.  The owning warp keeps one feature per lane: the intra rotation is 32 x 4 FMAs per lane
-//    on R_intra's column in registers, y read by broadcast.  The other CTAs leave right after their stores, which lets the CTAs of the next
-//    kernel in.  Against one owner for a tile (40 KiB to take in at 16 tokens, 80 loads per lane to add them, warp-level MMAs), us:
-//    rotation of 16 tokens, d = 4096 9.6 -> 8.8, 24 tokens NVFP4 (pulled before) 10.3 -> 9.4.
+//    tokens, and dealt over all CTAs and warps of the cluster, so that nearly every warp has one and no CTA takes in more than its share
+//    (what arrives at one SM comes at about 9 B per cycle).  A CTA stores its partials straight from registers into the owners' shared
+//    memory (st.async, 16 bytes per lane = four tokens of one feature, counted on a barrier of the owning warp), into room of their own:
+//    nobody has to say first that the stages there are free, and no cluster-wide barrier stands on the path.  The owning warp keeps one
+//    feature per lane: the intra rotation is 32 x 4 FMAs per lane on R_intra's column in registers, y read by broadcast.  The other CTAs
+//    leave right after their stores, which lets the CTAs of the next kernel in.  Against one owner for a tile (40 KiB to take in at 16
+//    tokens, 80 loads per lane to add them, warp-level MMAs), us: rotation of 16 tokens, d = 4096 9.6 -> 8.8, 24 tokens NVFP4 (pulled
+//    before) 10.3 -> 9.4.
 //  * pull (more tokens): token group g (16 tokens) belongs to CTA g % S.  Every CTA writes its partial [token][feature] into its own shared
 //    memory, a cluster barrier publishes them, and the owner reads them with 16-byte ld.shared::cluster and rotates on the warp-level
 //    tensor cores (y split into three bf16 terms, fp32 accumulation).  A second barrier, at which a warp arrives
@@ -35,9 +36,9 @@
 // 14.8 -> 14.3, d = 4096, N = 6144, 200 tokens 22.4 -> 21.7.
 //
 // Roles per CTA: warp 0 TMA producer, warp 1 MMA issuer, warps 2..5 epilogue / reduction.
-// Shared memory: 4 stages (5 up to 16 tokens, 3 where more than 32 push) of (16 KiB of R_inter + tokens x 128 B of X); pulled partials lie in
-// the same memory after the mainloop, pushed ones behind it.  Up to 64 tokens that is small enough (<= 107 KiB) for two CTAs per SM: the
-// grid may exceed the SM count, which keeps more loads in flight; above, one CTA fills an SM, or
+// Shared memory: 4 stages (5 up to 16 tokens, 3 where more than 32 push) of (16 KiB of R_inter + tokens x 128 B of X); pulled partials
+// lie in the same memory after the mainloop, pushed ones behind it.  Up to 64 tokens that is small enough (<= 107 KiB) for two CTAs per
+// SM: the grid may exceed the SM count, which keeps more loads in flight; above, one CTA fills an SM, or
 // up to 128 tokens two of them with three stages (fewtok_rotation).
 #pragma once
 #include <cuda_bf16.h>

@@ -256,7 +256,8 @@ rotate_quantize_pair_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
     //  * tcgen05 instructions of both CTAs on three split bf16 terms of y in tensor memory (every product exact, fp32
     //    accumulation), for the CTA's LAST tile, whose epilogue nothing overlaps and beside which half the tensor memory is free.  (As
     //    warp-level MMAs on accumulator fragments that epilogue was bound by those: us, loops of 0.4 s, before / now, rotation
-    //    2048 x 4096 59.7 / 58.25, 1900 x 4096 NVFP4 60.0 / 58.6, 8192 x 1024 26.6 / 25.8; shorter loops 58.05 / 56.3, 59.6 / 55.7 and 26.5 / 25.3.)
+    //    2048 x 4096 59.7 / 58.25, 1900 x 4096 NVFP4 60.0 / 58.6, 8192 x 1024 26.6 / 25.8; shorter loops 58.05 / 56.3, 59.6 / 55.7 and
+    //    26.5 / 25.3.)
     const int q = warp & 3;
     const int h = (warp - 2) >> 2;
     const int et = (warp - 2) * 32 + lane;               // 0..255 among the epilogue threads

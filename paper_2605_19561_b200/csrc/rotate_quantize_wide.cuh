@@ -18,14 +18,14 @@
 // Bounds: up to 128 columns the latency of the loads and of the hand-overs between the roles (440 cycles per 64 of K at 64
 // columns, 460 at 128 with stages of 64, where the instructions take 320 and 384; the same loads alone, from L2, run at 22
 // TB/s), above the instructions (500 at 256); then the epilogue, which nothing overlaps.  The intra rotation in it runs as tcgen05
-// instructions of both CTAs, y split into three bf16 terms in tensor memory; a lane then holds one row of a block and quantizes it.  As warp-level
-// MMAs on the accumulator fragments it was bound by those, about 860 cycles per 32 columns (us, these / here: rotation 777 x 5120 44.8 / 42.5, 300 x
-// 2048 8.72 / 8.45, layers 600 x 2048 -> 2048 15.7 / 14.95, loops of 0.5 s 1024 x 4096 -> 4096 44.3 / 43.0).  Tiles of 32 columns keep that form: a unit
-// of 16 rows for each of eight warps is done before the hand-over to the issuer and back (200 x 2048 7.68 / 7.88, 256 x 1024 4.48 / 4.64).  Measured
-// no faster: the terms of a set's next block sent before the result of this one is waited for (777 x 5120 42.4 / 41.9, but 300 x 2048 8.45 / 8.69:
-// what a short call waits for is this code's instructions), and a warp that runs it once ahead (8.45 / 8.58).  Splitting K over the pairs of a larger cluster (partial sums
-// exchanged through distributed shared memory) was measured and brought nothing: 300 x 4096 20.9 with two pairs
-// per 256 columns against 21.2.
+// instructions of both CTAs, y split into three bf16 terms in tensor memory; a lane then holds one row of a block and quantizes it.  As
+// warp-level MMAs on the accumulator fragments it was bound by those, about 860 cycles per 32 columns (us, these / here: rotation 777 x
+// 5120 44.8 / 42.5, 300 x 2048 8.72 / 8.45, layers 600 x 2048 -> 2048 15.7 / 14.95, loops of 0.5 s 1024 x 4096 -> 4096 44.3 / 43.0).
+// Tiles of 32 columns keep that form: a unit of 16 rows for each of eight warps is done before the hand-over to the issuer and back (200
+// x 2048 7.68 / 7.88, 256 x 1024 4.48 / 4.64).  Measured no faster: the terms of a set's next block sent before the result of this one is
+// waited for (777 x 5120 42.4 / 41.9, but 300 x 2048 8.45 / 8.69: what a short call waits for is this code's instructions), and a warp
+// that runs it once ahead (8.45 / 8.58).  Splitting K over the pairs of a larger cluster (partial sums exchanged through distributed
+// shared memory) was measured and brought nothing: 300 x 4096 20.9 with two pairs per 256 columns against 21.2.
 //
 // Roles per CTA: warp 0 TMA producer, warp 1 MMA issuer (leader CTA), warps 2..13 epilogue (lane quarter w % 4, three
 // sets of warps).  One elected thread runs the producer's and the issuer's loop.
@@ -77,8 +77,8 @@ static_assert(RotWideCfg::stages(128) <= RotWideCfg::MAX_STAGES && RotWideCfg::s
 // grid = 2 * rows * cols CTAs in clusters of two: pair p works row tile p % rows (256 tokens), column tile p / rows
 // (`width` features from column (p / rows) * width on).  tmX: X as (64 of K, token, slab of K), box [64 x 128 x slabs of a
 // stage]; tmR: R_inter box [BK of K x 64 columns]; tmRt: box [BK x tail_cols].  d % 128 == 0.  RANGE: 32, 128, 256 or 384, the first
-// that is not below the width (two slabs of K per stage, one block; two slabs; one; two instructions per slice).  FMT, `tensor_scale` as in the pair
-// kernel.
+// that is not below the width (two slabs of K per stage, one block; two slabs; one; two instructions per slice).  FMT, `tensor_scale` as
+// in the pair kernel.
 template <int FMT, int RANGE>
 __global__ void __launch_bounds__(RotWideCfg::THREADS, 1)
 rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmR,
@@ -232,11 +232,11 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
     if (warp == 3 && elect_one()) {
       // Until the kernel before has completed HBM idles.  In short calls the L2 is asked for the first K steps of X, one of each row tile
       // per pair that shares it, and, for strips of 64 to 128 columns, for the next R_inter, a strip's steps dealt over its row tiles (us,
-      // without / X alone / both, layers: 300 x 2048 -> 2048 14.00 / 13.83 / 13.69, 600 x 2048 15.4 / 15.1 / 14.9, 400 x 4096 -> 4096 25.7 /
-      // 25.3 / 25.1, 1500 x 2048 22.0 / 21.6; narrower strips lose by R_inter, 220 x 2048 12.73 / 12.60 / 12.71).  Calls long enough to run
-      // at the power cap lose (loops of 0.6 s, 1024 x 4096 44.4 / 44.7 / 45.0, 777 x 5120 60.7 / 60.8).  A box wholly beyond the last token or
-      // feature fetches nothing; to leave it out costs more (without / with that guard: 300 x 2048 -> 2048 12.77 / 12.81, 1000 x 2048
-      // -> 2048 15.48 / 15.53, 100 x 2048 -> 2048 12.00 / 12.02, three turns each that agree within 0.02).
+      // without / X alone / both, layers: 300 x 2048 -> 2048 14.00 / 13.83 / 13.69, 600 x 2048 15.4 / 15.1 / 14.9, 400 x 4096 -> 4096
+      // 25.7 / 25.3 / 25.1, 1500 x 2048 22.0 / 21.6; narrower strips lose by R_inter, 220 x 2048 12.73 / 12.60 / 12.71).  Calls long
+      // enough to run at the power cap lose (loops of 0.6 s, 1024 x 4096 44.4 / 44.7 / 45.0, 777 x 5120 60.7 / 60.8).  A box wholly
+      // beyond the last token or feature fetches nothing; to leave it out costs more (without / with that guard: 300 x 2048 -> 2048 12.77
+      // / 12.81, 1000 x 2048 -> 2048 15.48 / 15.53, 100 x 2048 -> 2048 12.00 / 12.02, three turns each that agree within 0.02).
       if (width * d <= 128 * 4096 && pair / rows < k_tiles) tma_prefetch_l2_3d(&tmX, 0, mt * C::BM, pair / rows * (BK / C::SLAB));
       if (RANGE == 128 && width >= 64)
         for (int kt = pre + pair % rows; kt < min(k_tiles, pre + C::AHEAD); kt += rows)
@@ -252,8 +252,8 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       __syncwarp();
     }
     if (R_intra != nullptr) {
-      // The tile's blocks, rows of 64 bytes under the 64-byte swizzle: 16-byte piece c of row i at c ^ ((i >> 1) & 3).  This CTA's half of the
-      // instruction's 32 columns are the first 32 bytes of its rows: rank 1 holds its pieces two on (kTerms).
+      // The tile's blocks, rows of 64 bytes under the 64-byte swizzle: 16-byte piece c of row i at c ^ ((i >> 1) & 3).  This CTA's half
+      // of the instruction's 32 columns are the first 32 bytes of its rows: rank 1 holds its pieces two on (kTerms).
       for (int idx = (warp - 2) * 32 + lane; idx < nb * 128; idx += 128 * C::ESETS) {
         const int lb = idx >> 7, i = (idx >> 2) & 31, c = (idx & 3) ^ (kTerms ? 2 * (int)rank : 0);
         *reinterpret_cast<uint4*>(smem_gen + ri_off + lb * C::RI_BLOCK_BYTES + i * 64 + ((c ^ ((i >> 1) & 3)) << 4)) =
@@ -299,8 +299,8 @@ rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       }
     } else {
       const uint32_t term_leader = map_to_cta(term_bar(set), 0);
-      // A warp takes 32 rows of a block, one row per lane.  y goes back to tensor memory as hi + mid + lo (bf16, exact): hi and mid over y itself,
-      // lo in columns of the set's own, where the result comes as well.
+      // A warp takes 32 rows of a block, one row per lane.  y goes back to tensor memory as hi + mid + lo (bf16, exact): hi and mid over
+      // y itself, lo in columns of the set's own, where the result comes as well.
       uint32_t ph = 0;
 #pragma unroll 1
       for (int bb = set; ok && set < sets && bb < nb; bb += sets) {

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 
 #include "../../include/torq.h"
 #include "mxfp4_gemm_pair.cuh"
@@ -79,6 +80,27 @@ static int max_active_clusters(K kernel, int size, int threads, int smem, int sm
 // its shared memory.  Never launched.
 __global__ void __launch_bounds__(RotFewCfg::THREADS, 2) fewtok_fit_kernel() {}
 
+// The kernels of one format.
+template <int FMT>
+static bool opt_in_format() {
+  constexpr int kWideSmem = 232448;                        // the widths share the kernels
+  constexpr int few_rot = RotFewCfg::max_smem_bytes(), few_gemm = GemmFewCfg<FMT>::max_smem_bytes();
+  return opt_in_smem(rotate_quantize_kernel<256, FMT>, RotCfg<256>::SMEM_BYTES) &&
+         opt_in_smem(rotate_quantize_pair_kernel<FMT>, RotPairCfg::SMEM_BYTES) &&
+         opt_in_smem(rotate_quantize_wide_kernel<FMT, 32>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT, 128>, kWideSmem) &&
+         opt_in_smem(rotate_quantize_wide_kernel<FMT, 256>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT, 384>, kWideSmem) &&
+         opt_in_smem(rotate_structured_kernel<FMT>, RotStructCfg::SMEM_BYTES) &&
+         opt_in_smem(rotate_fewtok_kernel<FMT, 1, true>, few_rot) &&
+         opt_in_smem(rotate_fewtok_kernel<FMT, 1, true, RotFewCfg::SHARED_STAGES>, few_rot) &&
+         opt_in_smem(rotate_fewtok_kernel<FMT, 1, true, RotFewCfg::PUSH_STAGES>, few_rot) &&
+         opt_in_smem(rotate_fewtok_kernel<FMT, 1, false, RotFewCfg::SHARED_STAGES>, few_rot) &&
+         opt_in_smem(rotate_fewtok_kernel<FMT, 1>, few_rot) && opt_in_smem(rotate_fewtok_kernel<FMT, 2>, few_rot) &&
+         opt_in_smem(mxfp4_gemm_pair_kernel<FMT>, GemmPairCfgT<FMT>::SMEM_BYTES) &&
+         opt_in_smem(mxfp4_gemm_wide_kernel<FMT, 128>, kWideSmem) && opt_in_smem(mxfp4_gemm_wide_kernel<FMT, 256>, kWideSmem) &&
+         opt_in_smem(mxfp4_gemm_wide_kernel<FMT, 384>, kWideSmem) && opt_in_smem(gemm_fewtok_kernel<FMT, 1, true>, few_gemm) &&
+         opt_in_smem(gemm_fewtok_kernel<FMT, 1>, few_gemm) && opt_in_smem(gemm_fewtok_kernel<FMT, 2>, few_gemm);
+}
+
 // CTA pairs of a kernel that fills its SMs.
 template <typename K>
 static int max_active_pairs(K kernel, int threads, int smem, int sm_count) {
@@ -111,48 +133,10 @@ static DeviceState* device_state() {
         return nullptr;
       g_encode = reinterpret_cast<EncodeTiledFn>(fn);
     }
-    constexpr int kWideSmem = 232448;                    // the widths share the kernels
-    bool ok = opt_in_smem(fewtok_fit_kernel, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_quantize_kernel<256>, RotCfg<256>::SMEM_BYTES) &&
-              opt_in_smem(rotate_quantize_kernel<256, FMT_NVFP4>, RotCfg<256>::SMEM_BYTES) &&
-              opt_in_smem(rotate_quantize_pair_kernel<FMT_MXFP4>, RotPairCfg::SMEM_BYTES) &&
-              opt_in_smem(rotate_quantize_pair_kernel<FMT_NVFP4>, RotPairCfg::SMEM_BYTES) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, 32>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, 128>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, 256>, kWideSmem) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXFP4, 384>, kWideSmem) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, 32>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, 128>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, 256>, kWideSmem) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_NVFP4, 384>, kWideSmem) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, 32>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, 128>, kWideSmem) && opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, 256>, kWideSmem) &&
-              opt_in_smem(rotate_quantize_wide_kernel<FMT_MXINT4, 384>, kWideSmem) &&
-              opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXFP4, 128>, kWideSmem) && opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXFP4, 256>, kWideSmem) &&
-              opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXFP4, 384>, kWideSmem) &&
-              opt_in_smem(mxfp4_gemm_wide_kernel<FMT_NVFP4, 128>, kWideSmem) && opt_in_smem(mxfp4_gemm_wide_kernel<FMT_NVFP4, 256>, kWideSmem) &&
-              opt_in_smem(mxfp4_gemm_wide_kernel<FMT_NVFP4, 384>, kWideSmem) &&
-              opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXINT4, 128>, kWideSmem) && opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXINT4, 256>, kWideSmem) &&
-              opt_in_smem(mxfp4_gemm_wide_kernel<FMT_MXINT4, 384>, kWideSmem) &&
-              opt_in_smem(rotate_structured_kernel<FMT_MXFP4>, RotStructCfg::SMEM_BYTES) &&
-              opt_in_smem(rotate_structured_kernel<FMT_NVFP4>, RotStructCfg::SMEM_BYTES) &&
-              opt_in_smem(mxfp4_gemm_pair_kernel<FMT_MXFP4>, GemmPairCfg::SMEM_BYTES) &&
-              opt_in_smem(mxfp4_gemm_pair_kernel<FMT_NVFP4>, GemmPairCfgT<FMT_NVFP4>::SMEM_BYTES) &&
-              opt_in_smem(mxfp4_gemm_pair_kernel<FMT_MXINT4>, GemmPairCfgT<FMT_MXINT4>::SMEM_BYTES) &&
-              opt_in_smem(rotate_quantize_kernel<256, FMT_MXINT4>, RotCfg<256>::SMEM_BYTES) &&
-              opt_in_smem(rotate_quantize_pair_kernel<FMT_MXINT4>, RotPairCfg::SMEM_BYTES) &&
-              opt_in_smem(rotate_structured_kernel<FMT_MXINT4>, RotStructCfg::SMEM_BYTES) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, true, RotFewCfg::PUSH_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 1>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXFP4, 2>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, true, RotFewCfg::PUSH_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 1>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_NVFP4, 2>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, true, RotFewCfg::PUSH_STAGES>, RotFewCfg::max_smem_bytes()) && opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1, false, RotFewCfg::SHARED_STAGES>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 1>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(rotate_fewtok_kernel<FMT_MXINT4, 2>, RotFewCfg::max_smem_bytes()) &&
-              opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 1, true>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) && opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 1>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) &&
-              opt_in_smem(gemm_fewtok_kernel<FMT_MXFP4, 2>, GemmFewCfg<FMT_MXFP4>::max_smem_bytes()) &&
-              opt_in_smem(gemm_fewtok_kernel<FMT_NVFP4, 1, true>, GemmFewCfg<FMT_NVFP4>::max_smem_bytes()) && opt_in_smem(gemm_fewtok_kernel<FMT_NVFP4, 1>, GemmFewCfg<FMT_NVFP4>::max_smem_bytes()) &&
-              opt_in_smem(gemm_fewtok_kernel<FMT_NVFP4, 2>, GemmFewCfg<FMT_NVFP4>::max_smem_bytes()) &&
-              opt_in_smem(gemm_fewtok_kernel<FMT_MXINT4, 1, true>, GemmFewCfg<FMT_MXINT4>::max_smem_bytes()) && opt_in_smem(gemm_fewtok_kernel<FMT_MXINT4, 1>, GemmFewCfg<FMT_MXINT4>::max_smem_bytes()) &&
-              opt_in_smem(gemm_fewtok_kernel<FMT_MXINT4, 2>, GemmFewCfg<FMT_MXINT4>::max_smem_bytes()) &&
-              opt_in_smem(rotate_quantize_kernel<256, FMT_F32OUT>, RotCfg<256>::SMEM_BYTES) &&
-              opt_in_smem(rotate_quantize_pair_kernel<FMT_F32OUT>, RotPairCfg::SMEM_BYTES);
+    const bool ok = opt_in_smem(fewtok_fit_kernel, RotFewCfg::max_smem_bytes()) && opt_in_format<FMT_MXFP4>() &&
+                    opt_in_format<FMT_NVFP4>() && opt_in_format<FMT_MXINT4>() &&
+                    opt_in_smem(rotate_quantize_kernel<256, FMT_F32OUT>, RotCfg<256>::SMEM_BYTES) &&
+                    opt_in_smem(rotate_quantize_pair_kernel<FMT_F32OUT>, RotPairCfg::SMEM_BYTES);
     if (!ok) return nullptr;
     st.rot_pairs = max_active_pairs(rotate_quantize_pair_kernel<FMT_MXFP4>, RotPairCfg::THREADS,
                                     RotPairCfg::SMEM_BYTES, st.sm_count);
@@ -269,8 +253,9 @@ static_assert(kRotFewMaxTokens <= RotFewCfg::MAX_TOK && kGemmFewMaxTokens <= Gem
 //  * above S = 4, at most 1.4 CTAs per SM, so that CTAs of the next kernel in the stream find room and send their
 //    weight loads early (decode layer at d = N = 5120, M = 1: S = 5 17.86, S = 6 17.97, though the rotation by
 //    itself is the faster one with S = 6), and `most`, so that a CTA has some K steps (the callers say how many): a longer
-//    reduction has to be paid for by a shorter stream (rotation d = 2048, M = 50: S = 8 7.1, S = 4 6.5; GEMM K = 2048, N = 5120: S = 5 5.5, S = 4 5.1).  Above 128
-//    tokens the reduction itself is shared out (up to 16 token groups), so there is no such bound (d = 1536: S = 8 9.9, S = 4 11.3);
+//    reduction has to be paid for by a shorter stream (rotation d = 2048, M = 50: S = 8 7.1, S = 4 6.5; GEMM K = 2048, N = 5120: S = 5
+//    5.5, S = 4 5.1).  Above 128 tokens the reduction itself is shared out (up to 16 token groups), so there is no such bound (d = 1536:
+//    S = 8 9.9, S = 4 11.3);
 //  * no S above the smallest one with the same longest K range (GEMM K = 4096: S = 5 has ranges of 4 steps like S = 4).
 static inline int fewtok_ntok(int64_t M) { return (int)((M + 15) / 16 * 16); }
 static inline int fewtok_cluster(int64_t tiles, int64_t k_steps, int64_t most, int ctas_per_sm, int sm_count, const int* fit) {
@@ -295,13 +280,13 @@ static FewRotation fewtok_rotation(int64_t M, int64_t d, bool intra, const Devic
   const int ntok = fewtok_ntok(M);
   const int64_t tiles = d / 128, steps = d / 64;
   // Pushed partial sums make the reduction cheap: the largest cluster that leaves room for two more (push_fit: 148, 93, 71, 56, 45, 37, 33
-  // clusters of 2 ... 8).  us, layers d = N, S = 4 / 6 / 8, 1 and 32 tokens: d = 1536 6.46 / 6.17 / 6.27 and 9.55 / 8.87 / 8.13, d = 2560 8.29 /
-  // 7.57 / 7.23 and 10.7 / 10.35 / 9.49, d = 4096 11.2 / 10.5 / 10.6 and 14.5 / 13.6 / 12.7; without the room d = 4224 (33 tiles) S = 7 /
-  // 8 11.3 / 11.8, d = 7168 (56 tiles) S = 4 / 5 23.2 / 23.6.  A fifth stage up to 16 tokens, but not on long K ranges (four / five, 1 token:
-  // layer d = N = 5120 14.5 / 14.3; rotation d = 14336 59.4 / 60.7).  A rotation without R_intra keeps the clusters of the rule below.
-  // Above 32 tokens (three stages then) where clusters of eight fit, up to 56: us, layers, pulled / pushed, 40 tokens: 2048 -> 2048 10.65 / 10.1, 4096 ->
-  // 4096 15.85 / 15.1, 56 tokens 2560 -> 2560 13.25 / 12.15, 64 tokens 11.3 / 11.8 and 16.9 / 16.9; d = 5120, S = 6, 50 tokens 19.4 / 19.8.  Above 48
-  // from 20 tiles on (56 tokens NVFP4 2048 -> 2048 10.96 / 11.6).
+  // clusters of 2 ... 8).  us, layers d = N, S = 4 / 6 / 8, 1 and 32 tokens: d = 1536 6.46 / 6.17 / 6.27 and 9.55 / 8.87 / 8.13, d = 2560
+  // 8.29 / 7.57 / 7.23 and 10.7 / 10.35 / 9.49, d = 4096 11.2 / 10.5 / 10.6 and 14.5 / 13.6 / 12.7; without the room d = 4224 (33 tiles)
+  // S = 7 / 8 11.3 / 11.8, d = 7168 (56 tiles) S = 4 / 5 23.2 / 23.6.  A fifth stage up to 16 tokens, but not on long K ranges (four /
+  // five, 1 token: layer d = N = 5120 14.5 / 14.3; rotation d = 14336 59.4 / 60.7).  A rotation without R_intra keeps the clusters of the
+  // rule below.  Above 32 tokens (three stages then) where clusters of eight fit, up to 56: us, layers, pulled / pushed, 40 tokens: 2048
+  // -> 2048 10.65 / 10.1, 4096 -> 4096 15.85 / 15.1, 56 tokens 2560 -> 2560 13.25 / 12.15, 64 tokens 11.3 / 11.8 and 16.9 / 16.9; d =
+  // 5120, S = 6, 50 tokens 19.4 / 19.8.  Above 48 from 20 tiles on (56 tokens NVFP4 2048 -> 2048 10.96 / 11.6).
   if (intra && (M <= 32 || (M <= (tiles < 20 ? 48 : RotFewCfg::PUSH_TOK) && tiles <= st->push_fit[RotFewCfg::MAX_CLUSTER] - 2))) {
     int S = (int)(steps < RotFewCfg::MAX_CLUSTER ? steps : RotFewCfg::MAX_CLUSTER);
     while (S > 1 && tiles > st->push_fit[S] - 2) --S;
@@ -338,15 +323,15 @@ static int fewtok_gemm_cluster(int ntok, int64_t tiles, int64_t steps, int ctas,
   if (tiles * S * ntok <= 32 * (int64_t)st->sm_count) return S;
   return fewtok_cluster(tiles, steps, steps / 3, ctas, st->sm_count, st->few_fit);
 }
-// Where the sums are pushed (M tokens), from the largest cluster down: above four CTAs where each keeps four K steps and has its SM to itself
-// (a CTA's instructions wait for those of the other one on its SM), or with five and more steps; up to four where they have their SMs to
-// themselves (a tenth may share), or with more than five steps.  us, layers, S = 3 / 4 / 5 / 8: 8 x 5120 -> 5120 (20 steps) 15.35 / 14.5 /
-// 15.0 / 15.2, 16 x 4096 -> 1024 (16) 12.0 / 10.0 / 10.2 / 10.8, 16 x 2048 -> 6144 (8) 8.06 / 8.36, 8 x 8192 -> 2048 (32) 28.0 / 27.1 / 26.4 / 24.4,
-// 16 x 7168 -> 4096 (28), S = 4 / 6 23.25 / 22.3, 16 x 5120 -> 8192, S = 3 / 4 16.5 / 17.1; up to 4 tokens sharing costs less (1 x 5120 -> 5120
-// S = 4 / 5 14.4 / 14.3).  One or two steps are not split (16 tokens, N = 4096, K = 512 2.97 / 2.56; above 16 tokens there are nine and more).
-// Few tiles take as many CTAs as have two steps, while the sums are few as above, up to 16 tokens 8 tokens per SM (us, S = 4 / 8: 1 token
-// N = 256 2.96 / 2.58, N = 1024 3.10 / 2.82, the layer 11.2 / 10.9; beyond: N = 2048 the GEMM 3.62 / 3.51, the layer of 16 tokens
-// 13.2 / 13.5; S = 4 / 5 at K = 2560, N = 5120 the layer 11.0 / 11.5).
+// Where the sums are pushed (M tokens), from the largest cluster down: above four CTAs where each keeps four K steps and has its SM to
+// itself (a CTA's instructions wait for those of the other one on its SM), or with five and more steps; up to four where they have their
+// SMs to themselves (a tenth may share), or with more than five steps.  us, layers, S = 3 / 4 / 5 / 8: 8 x 5120 -> 5120 (20 steps) 15.35
+// / 14.5 / 15.0 / 15.2, 16 x 4096 -> 1024 (16) 12.0 / 10.0 / 10.2 / 10.8, 16 x 2048 -> 6144 (8) 8.06 / 8.36, 8 x 8192 -> 2048 (32) 28.0 /
+// 27.1 / 26.4 / 24.4, 16 x 7168 -> 4096 (28), S = 4 / 6 23.25 / 22.3, 16 x 5120 -> 8192, S = 3 / 4 16.5 / 17.1; up to 4 tokens sharing
+// costs less (1 x 5120 -> 5120 S = 4 / 5 14.4 / 14.3).  One or two steps are not split (16 tokens, N = 4096, K = 512 2.97 / 2.56; above
+// 16 tokens there are nine and more).  Few tiles take as many CTAs as have two steps, while the sums are few as above, up to 16 tokens 8
+// tokens per SM (us, S = 4 / 8: 1 token N = 256 2.96 / 2.58, N = 1024 3.10 / 2.82, the layer 11.2 / 10.9; beyond: N = 2048 the GEMM 3.62
+// / 3.51, the layer of 16 tokens 13.2 / 13.5; S = 4 / 5 at K = 2560, N = 5120 the layer 11.0 / 11.5).
 static int push_gemm_cluster(int64_t M, int64_t tiles, int64_t steps, const DeviceState* st) {
   if (steps >= 8) {
     const int S = fewtok_cluster(tiles, steps, steps / 2, 2, st->sm_count, st->few_fit);
@@ -526,30 +511,38 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
   return quantize_impl(st, Z, z_dtype, M, d, out_codes, out_scales, static_cast<cudaStream_t>(stream));
 }
 
-// Width of the one-wave rotation's tiles, or 0 where another kernel is faster.  Times in us, fitted to the rotation
-// alone at 60 shapes (d = 128 ... 14336, M = 1 ... 4000; within 10 % but above d = 6144, where these tiles are rated up to 3 us too
-// high, and at d > 8192, where HBM bounds both sides and both are rated low); f = filled part of a wave:
+// Width of the one-wave rotation's tiles, or 0 where another kernel is faster.  Times in us: once a fit to the rotation alone, since
+// moved where both kernels were measured on either side of a line, so they say which kernel is the faster and not how long it takes.
+// Of 202 rotations (d = 128 ... 14336, 1 to 4000 tokens, operands from HBM) these tiles are rated 7 % off in the median, a quarter low
+// where a call runs at the power cap or d is above 8192; the few-token kernel is rated up to half low from d = 3072 on, where R_inter's
+// stream sets its pace, and the pair kernel a quarter low at the power cap.  177 of them can run on either: 13 take the slower one,
+// 300 x 6144 35.0 / 29.9, the others by up to 8 % (1 x 128 2.67 / 2.48, 777 x 3072 18.8 / 17.8, 777 x 4096 30.0 / 28.6).  f = filled part
+// of a wave:
 //  * here: 1.8 + 0.0155 per column (2 + 0.025 above 256 columns, 1.6 + 0.0155 up to 128) for launch and epilogue, from 129 to 256
 //    tokens 1.6 + 0.022 (2 + 0.032, 1.4 + 0.022), what they were with warp-level instructions: the few-token kernel contracts K in
 //    parts, which these tiles do in one accumulator, and a line that follows the shorter epilogue gives up precision (codes that differ
-//    from those of 64-bit arithmetic, few tokens / here: 220 x 5504 6 / 51 of 1.2 M).  Then per K step of 64 the operand bytes, 0.17 + 0.0003 per column + 0.03 f (up to 128 columns, where a stage is two of these steps, 0.145 +
-//    0.0003 per column + 0.035 f, but from d = 6272 on, where R_inter's stream sets the pace), or the math, 0.00114 per column;
+//    from those of 64-bit arithmetic, few tokens / here: 220 x 5504 6 / 51 of 1.2 M).  Then per K step of 64 the operand bytes, 0.17 +
+//    0.0003 per column + 0.03 f (up to 128 columns, where a stage is two of these steps, 0.145 + 0.0003 per column + 0.035 f, but from d
+//    = 6272 on, where R_inter's stream sets the pace), or the math, 0.00114 per column;
 //  * few tokens: 3.1 / 4.4 / 5.6 up to 16 / 64 / 128 tokens, plus 0.22 / 0.2 / 0.36 per K step of the longest split; above, 6.4 (6.1 up
-//    to 176 tokens: 160 x 2816 15.2 / 16.05 as layers) at 144 tokens and 0.025 per token more, 0.5 per CTA of a cluster above four, 0.42 per K step (us, few tokens / here: 144
-//    tokens d = 2560 9.7 / 10.4, d = 4096 13.6 / 14.9; 208 d = 2560 12.6 / 10.4, d = 4096 15.0 / 15.0 (the layer with N = 6144
-//    22.7 / 23.2), d = 5120 19.5 / 20.1; 256 d = 4096 16.2 / 15.1, d = 5120 20.9 / 20.0; 128 d = 2048 8.1 / 7.6).  Beside clusters of six
-//    (d = 2048 ... 2816, up to 192 tokens) this is a microsecond more than they take with cold operands, and the line lies between
-//    what cold ones and an R_inter in the L2 ask for (layers with N = d, few tokens / here: 144 x 2432 cold 0.95 of the time, in the
-//    L2 1.11; 152 x 2560 0.93 and 1.09, 176 x 2560 0.97 and 1.11, 176 x 2816 0.97 and 1.06, 112 x 2176 0.95 and 1.04);
-//  * few tokens whose sums are pushed: 2.7 + 0.22 per K step + 0.025 per token, 0.04 above 32 tokens (us, here / few tokens, 1, 16 and 32 tokens: d = 256 2.95 / 2.96, 2.95 /
-//    3.21, 2.95 / 4.49; d = 512 3.97 / 3.08, 3.37 / 3.21, 3.46 / 3.60; d = 768 5.25 / 3.21, 4.24 / 3.37, 4.36 / 3.85);
+//    to 176 tokens: 160 x 2816 15.2 / 16.05 as layers) at 144 tokens and 0.025 per token more, 0.5 per CTA of a cluster above four, 0.42
+//    per K step (us, few tokens / here: 144 tokens d = 2560 9.7 / 10.4, d = 4096 13.6 / 14.9; 208 d = 2560 12.6 / 10.4, d = 4096 15.0 /
+//    15.0 (the layer with N = 6144 22.7 / 23.2), d = 5120 19.5 / 20.1; 256 d = 4096 16.2 / 15.1, d = 5120 20.9 / 20.0; 128 d = 2048 8.1 /
+//    7.6).  Beside clusters of six (d = 2048 ... 2816, up to 192 tokens) this is a microsecond more than they take with cold operands,
+//    and the line lies between what cold ones and an R_inter in the L2 ask for (layers with N = d, few tokens / here: 144 x 2432 cold
+//    0.95 of the time, in the L2 1.11; 152 x 2560 0.93 and 1.09, 176 x 2560 0.97 and 1.11, 176 x 2816 0.97 and 1.06, 112 x 2176 0.95 and
+//    1.04);
+//  * few tokens whose sums are pushed: 2.7 + 0.22 per K step + 0.025 per token, 0.04 above 32 tokens (us, here / few tokens, 1, 16 and 32
+//    tokens: d = 256 2.95 / 2.96, 2.95 / 3.21, 2.95 / 4.49; d = 512 3.97 / 3.08, 3.37 / 3.21, 3.46 / 3.60; d = 768 5.25 / 3.21, 4.24 /
+//    3.37, 4.36 / 3.85);
 //  * above 192 tokens a cluster of three has five units for its first CTA: 0.6 more (216 d = 4864 19.3 / 18.2);
 //  * above d = 6144, where these tiles take up to 3 us less than the figures say: 7.6 up to 192 tokens, 10.5 above, 0.42 per K step
 //    (144 d = 6912 26.9 / 25.4, 150 d = 7040 28.2 / 26.3, 208 d = 7680 33.1 / 30.0);
-//  * pair kernel: 6.8, plus per K step 0.32 for a wave and 0.2 + 0.14 f for the last, partly filled one.
+//  * pair kernel: 6.8, plus per K step 0.32 for a wave and 0.2 + 0.14 f for the last, partly filled one (layers with N = d at 40 sizes
+//    beside the line, 1772 to 4076 tokens, pair kernel / here: 0.99 to 1.6 of the time; 2540 x 2048 36.2 / 30.9, 2028 x 2048 25.3 / 25.05).
 // The other formats follow the same figures, which were not fitted to them; wide_gemm_width says how that was checked.
-// A layer of 2048 tokens and more fills the pair kernel's waves and stays there (one-wave tiles would be wider than
-// 384 columns; 2048 x 4096 measured 51.6 with 480 columns, 46.8 in the pair kernel).
+// From 2048 x 4096 on a layer fills the pair kernel's waves and stays there: one-wave tiles would be wider than 384 columns (2048 x 4096
+// measured 51.6 with 480 columns, 46.8 in the pair kernel).
 static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int few_S, bool push, int max_pairs) {
   const int64_t rows = (M + 255) / 256, steps = d / 64;
   // The line of 65 to 96 tokens, clusters of six, stays where it was, and so does that of an X below 128 KiB (up to 64 tokens; with
@@ -576,7 +569,8 @@ static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int few_S, b
     else if (M <= 64) other = 4.4 + 0.2 * few_steps;
     else if (M <= 128) other = 5.6 + 0.36 * few_steps;
     else if (d > 6144) other = (M <= 192 ? 7.6 : 10.5) + 0.42 * few_steps;
-    else other = (M <= 176 ? 6.1 : 6.4) + 0.025 * (double)(M - 144) + (few_S > 4 ? 0.5 * (few_S - 4) : (few_S == 3 && M > 192 ? 0.6 : 0.0)) + 0.42 * few_steps;
+    else other = (M <= 176 ? 6.1 : 6.4) + 0.025 * (double)(M - 144) + 0.42 * few_steps +
+                 (few_S > 4 ? 0.5 * (few_S - 4) : (few_S == 3 && M > 192 ? 0.6 : 0.0));
   } else {
     const int64_t tiles = rows * ((d + 255) / 256);
     const int64_t full = tiles / max_pairs, rest = tiles % max_pairs;
@@ -597,13 +591,18 @@ static torq_status rotate_wide(DeviceState* st, int fmt, const void* X, const vo
     return TORQ_ERR_LAUNCH;
   if (!tail) tmRt = tmR;
   const int rows = (int)((M + 255) / 256), cols = (int)((d + width - 1) / width);
-  auto launch = [&](auto r32, auto r128, auto r256, auto r384) {
-    launch_tc(width > 256 ? r384 : (width > 128 ? r256 : (width > 32 ? r128 : r32)), 2, 2 * rows * cols, C::THREADS, C::smem_bytes(width), s, tmX, tmR, tmRt,
-              static_cast<const __nv_bfloat16*>(R_intra), codes, scales, (int)M, (int)d, tensor_scale, rows, width, st->err_word);
+  auto launch = [&](auto format) {
+    constexpr int F = decltype(format)::value;
+    launch_tc(width > 256   ? rotate_quantize_wide_kernel<F, 384>
+              : width > 128 ? rotate_quantize_wide_kernel<F, 256>
+              : width > 32  ? rotate_quantize_wide_kernel<F, 128>
+                            : rotate_quantize_wide_kernel<F, 32>,
+              2, 2 * rows * cols, C::THREADS, C::smem_bytes(width), s, tmX, tmR, tmRt, static_cast<const __nv_bfloat16*>(R_intra),
+              codes, scales, (int)M, (int)d, tensor_scale, rows, width, st->err_word);
   };
-  if (fmt == FMT_MXINT4) launch(rotate_quantize_wide_kernel<FMT_MXINT4, 32>, rotate_quantize_wide_kernel<FMT_MXINT4, 128>, rotate_quantize_wide_kernel<FMT_MXINT4, 256>, rotate_quantize_wide_kernel<FMT_MXINT4, 384>);
-  else if (fmt == FMT_NVFP4) launch(rotate_quantize_wide_kernel<FMT_NVFP4, 32>, rotate_quantize_wide_kernel<FMT_NVFP4, 128>, rotate_quantize_wide_kernel<FMT_NVFP4, 256>, rotate_quantize_wide_kernel<FMT_NVFP4, 384>);
-  else launch(rotate_quantize_wide_kernel<FMT_MXFP4, 32>, rotate_quantize_wide_kernel<FMT_MXFP4, 128>, rotate_quantize_wide_kernel<FMT_MXFP4, 256>, rotate_quantize_wide_kernel<FMT_MXFP4, 384>);
+  if (fmt == FMT_MXINT4) launch(std::integral_constant<int, FMT_MXINT4>{});
+  else if (fmt == FMT_NVFP4) launch(std::integral_constant<int, FMT_NVFP4>{});
+  else launch(std::integral_constant<int, FMT_MXFP4>{});
   return launch_status();
 }
 
@@ -621,22 +620,21 @@ static torq_status rotate_fewtok(DeviceState* st, int fmt, const void* X, const 
   const float ts = fmt == FMT_NVFP4 ? tensor_scale : 0.0f;
   const __nv_bfloat16* ri = static_cast<const __nv_bfloat16*>(R_intra);
   // sums pushed, with five, four or three stages; pulled, two CTAs per SM: one set of epilogue warps; one CTA: two sets
-  auto launch = [&](auto push5, auto push4, auto push3, auto one, auto shared, auto two) {
-    const bool share = few.stages == RotFewCfg::SHARED_STAGES, small = few.push || share || ntok <= 64;
-    launch_tc(few.push ? (few.stages == RotFewCfg::PUSH_STAGES ? push5 : (share ? push3 : push4)) : (share ? shared : (small ? one : two)), S,
-              tiles * S, small ? 192 : 320, smem, s, tmX, tmR, ri, codes, scales, (int)M, (int)d, ntok, S, ft0,
+  const bool share = few.stages == RotFewCfg::SHARED_STAGES, small = few.push || share || ntok <= 64;
+  auto launch = [&](auto format) {
+    constexpr int F = decltype(format)::value, P = RotFewCfg::PUSH_STAGES, NS = RotFewCfg::SHARED_STAGES;
+    launch_tc(few.push ? (few.stages == P ? rotate_fewtok_kernel<F, 1, true, P>
+                          : share         ? rotate_fewtok_kernel<F, 1, true, NS>
+                                          : rotate_fewtok_kernel<F, 1, true>)
+              : share  ? rotate_fewtok_kernel<F, 1, false, NS>
+              : small  ? rotate_fewtok_kernel<F, 1>
+                       : rotate_fewtok_kernel<F, 2>,
+              S, tiles * S, small ? 192 : 320, smem, s, tmX, tmR, ri, codes, scales, (int)M, (int)d, ntok, S, ft0,
               fewtok_leave_together(M, tiles, few, st) ? 1 : 0, kAheadTiles / (tiles * S), ts, st->err_word);
   };
-  constexpr int NS = RotFewCfg::SHARED_STAGES;
-  if (fmt == FMT_MXINT4)
-    launch(rotate_fewtok_kernel<FMT_MXINT4, 1, true, RotFewCfg::PUSH_STAGES>, rotate_fewtok_kernel<FMT_MXINT4, 1, true>, rotate_fewtok_kernel<FMT_MXINT4, 1, true, NS>, rotate_fewtok_kernel<FMT_MXINT4, 1>, rotate_fewtok_kernel<FMT_MXINT4, 1, false, NS>,
-           rotate_fewtok_kernel<FMT_MXINT4, 2>);
-  else if (fmt == FMT_NVFP4)
-    launch(rotate_fewtok_kernel<FMT_NVFP4, 1, true, RotFewCfg::PUSH_STAGES>, rotate_fewtok_kernel<FMT_NVFP4, 1, true>, rotate_fewtok_kernel<FMT_NVFP4, 1, true, NS>, rotate_fewtok_kernel<FMT_NVFP4, 1>, rotate_fewtok_kernel<FMT_NVFP4, 1, false, NS>,
-           rotate_fewtok_kernel<FMT_NVFP4, 2>);
-  else
-    launch(rotate_fewtok_kernel<FMT_MXFP4, 1, true, RotFewCfg::PUSH_STAGES>, rotate_fewtok_kernel<FMT_MXFP4, 1, true>, rotate_fewtok_kernel<FMT_MXFP4, 1, true, NS>, rotate_fewtok_kernel<FMT_MXFP4, 1>, rotate_fewtok_kernel<FMT_MXFP4, 1, false, NS>,
-           rotate_fewtok_kernel<FMT_MXFP4, 2>);
+  if (fmt == FMT_MXINT4) launch(std::integral_constant<int, FMT_MXINT4>{});
+  else if (fmt == FMT_NVFP4) launch(std::integral_constant<int, FMT_NVFP4>{});
+  else launch(std::integral_constant<int, FMT_MXFP4>{});
   return launch_status();
 }
 
@@ -679,7 +677,8 @@ static torq_status rotate_quantize_impl(const void* X, const void* R_inter, cons
     if (width > 0) return rotate_wide(st, fmt, X, R_inter, R_intra, M, d, codes, scales, tensor_scale, width, s);
   }
   if (M <= kRotFewMaxTokens && d % 128 == 0 && x_terms == 1 && fmt != FMT_F32OUT)
-    return rotate_fewtok(st, fmt, X, R_inter, R_intra, M, d, 0, (int)(d / 128), fewtok_rotation(M, d, R_intra != nullptr, st), codes, scales, tensor_scale, s);
+    return rotate_fewtok(st, fmt, X, R_inter, R_intra, M, d, 0, (int)(d / 128), fewtok_rotation(M, d, R_intra != nullptr, st), codes,
+                         scales, tensor_scale, s);
   if (!encode_2d(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, (uint64_t)M, (uint64_t)d * x_terms, 128, 64) ||
       !encode_2d(&tmR, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, R_inter, (uint64_t)d, (uint64_t)d, 64, 64))
     return TORQ_ERR_LAUNCH;
@@ -811,8 +810,8 @@ torq_status torq_rotate_quantize_structured_nvfp4(const void* X, const void* R_B
 //    do not know: there they are high by up to a third (200 x 4096, K = 14336 17.3 modelled, 13.1 measured; 300 x 4096, K = 4096 7.8,
 //    6.7) and take 192 columns in one slab where 128 in two would fit the pairs too (512 x 4096, K = 14336; 700 x 3072, K = 4096);
 //  * few tokens (17 to 128, S CTAs per tile): 2.3 + 0.2 per K step of the longest split + per token 0.025 with S = 1 (the
-//    accumulator goes to Y), else 0.012 + 0.035 / S.  With pulled sums; pushed ones (17 to 32 tokens, K > 2048) take less, and even by these
-//    figures the one-wave kernel is 1.11 times and more their time at every size;
+//    accumulator goes to Y), else 0.012 + 0.035 / S.  With pulled sums; pushed ones (17 to 32 tokens, K > 2048) take less, and even by
+//    these figures the one-wave kernel is 1.11 times and more their time at every size;
 //  * pair kernel: one wave 4.1 + 0.9 f + (0.285 + 0.04 f) per K step, more (the last one as narrower tiles) 5.2 + per K step
 //    0.325 for a full wave and 0.21 + 0.14 f for the last.
 // The same figures choose for NVFP4, MXINT4 (twice the steps) and float32 output, which were not fitted.  A sweep of 5250 calls, the
@@ -899,7 +898,9 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
     // Few tokens: 128 output features x all tokens per CTA, K split over a cluster, reduced through
     // distributed shared memory.
     const int64_t steps = (K + FC::BK - 1) / FC::BK;
-    const int S = FC::push((int)M, (int)K) ? push_gemm_cluster(M, tiles, steps, st) : fewtok_gemm_cluster(ntok, tiles, steps, FC::ctas_per_sm((int)M, (int)K), st);
+    const bool push = FC::push((int)M, (int)K);
+    const int ctas = FC::ctas_per_sm((int)M, (int)K);
+    const int S = push ? push_gemm_cluster(M, tiles, steps, st) : fewtok_gemm_cluster(ntok, tiles, steps, ctas, st);
     const int width = M > 16 ? wide_gemm_width(M, N, steps, S, st->gemm_pairs) : 0;
     if (width > 0) return gemm_wide<FMT>(st, Aq, As, Wq, Ws, M, N, K, Y, y_dtype, alpha, width, s);
     if (!encode_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, Wq, (uint64_t)N, krow, 128, 128) ||
@@ -908,10 +909,11 @@ static torq_status gemm_impl(const void* Aq, const void* As, const void* Wq, con
     // sums pushed (FC::push); up to 64 tokens: one set of epilogue warps, two CTAs per SM; more: two sets.  65 to 80 tokens in
     // MXINT4 fit twice on an SM as well, and share it only where that gives them more K splits (us, shared / alone, 72 tokens:
     // N = 768, K = 3072 4.9 / 4.4, N = 1536 6.0 / 5.1, S = 8 either way; N = 6144, K = 4096, S = 4 and 1: 9.1 / 9.9).
-    const bool small = FC::ctas_per_sm((int)M, (int)K) >= 2 && (ntok <= 64 || S > fewtok_gemm_cluster(ntok, tiles, steps, 1, st));
-    launch_tc(FC::push((int)M, (int)K) ? gemm_fewtok_kernel<FMT, 1, true> : (small ? gemm_fewtok_kernel<FMT, 1> : gemm_fewtok_kernel<FMT, 2>),
-              S, tiles * S, small ? 192 : 320, FC::smem_bytes((int)M, (int)K), s, tmB, tmA, static_cast<const uint8_t*>(As),
-              static_cast<const uint8_t*>(Ws), Y, y_dtype == TORQ_BF16 ? 1 : 0, (int)M, (int)N, (int)K, ntok, S, kAheadTiles / (tiles * S), alpha, st->err_word);
+    const bool small = ctas >= 2 && (ntok <= 64 || S > fewtok_gemm_cluster(ntok, tiles, steps, 1, st));
+    launch_tc(push ? gemm_fewtok_kernel<FMT, 1, true> : (small ? gemm_fewtok_kernel<FMT, 1> : gemm_fewtok_kernel<FMT, 2>), S, tiles * S,
+              small ? 192 : 320, FC::smem_bytes((int)M, (int)K), s, tmB, tmA, static_cast<const uint8_t*>(As),
+              static_cast<const uint8_t*>(Ws), Y, y_dtype == TORQ_BF16 ? 1 : 0, (int)M, (int)N, (int)K, ntok, S,
+              kAheadTiles / (tiles * S), alpha, st->err_word);
     return launch_status();
   }
   const int width = wide_gemm_width(M, N, (K + GemmWideCfg<FMT>::BK - 1) / GemmWideCfg<FMT>::BK, 0, st->gemm_pairs);
