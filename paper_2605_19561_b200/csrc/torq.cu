@@ -518,13 +518,14 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 // stream sets its pace, and the pair kernel a quarter low at the power cap.  177 of them can run on either: 13 take the slower one,
 // 300 x 6144 35.0 / 29.9, the others by up to 8 % (1 x 128 2.67 / 2.48, 777 x 3072 18.8 / 17.8, 777 x 4096 30.0 / 28.6).  f = filled part
 // of a wave:
-//  * here: 1.8 + 0.0155 per column (2 + 0.025 above 256 columns, 1.6 + 0.0155 up to 128) for launch and epilogue, from 129 to 256
+//  * here: 1.8 + 0.0155 per column (2 + 0.025 above 256 columns, 1.6 + 0.0155 up to 128) for launch and epilogue, from 177 to 256
 //    tokens 1.6 + 0.022 (2 + 0.032, 1.4 + 0.022), what they were with warp-level instructions: the few-token kernel contracts K in
-//    parts, which these tiles do in one accumulator, and a line that follows the shorter epilogue gives up precision (codes that differ
-//    from those of 64-bit arithmetic, few tokens / here: 220 x 5504 6 / 51 of 1.2 M).  Then per K step of 64 the operand bytes, 0.17 +
+//    parts, which these tiles do in one accumulator, and a line that follows the shorter epilogue gives up precision for its 2 to 10 %
+//    (codes that differ from those of 64-bit arithmetic, few tokens / here: 220 x 5504 6 / 51 of 1.2 M; layers with N = d 180 x 3072
+//    18.5 / 16.7, 245 x 4096 22.85 / 21.6, 204 x 5120 27.2 / 28.15).  Then per K step of 64 the operand bytes, 0.17 +
 //    0.0003 per column + 0.03 f (up to 128 columns, where a stage is two of these steps, 0.145 + 0.0003 per column + 0.035 f, but from d
 //    = 6272 on, where R_inter's stream sets the pace), or the math, 0.00114 per column;
-//  * few tokens: 3.1 / 4.4 / 5.6 up to 16 / 64 / 128 tokens, plus 0.22 / 0.2 / 0.36 per K step of the longest split; above, 6.4 (6.1 up
+//  * few tokens: 3.1 / 4.4 / 5.6 up to 16 / 64 / 128 tokens, plus 0.22 / 0.2 / 0.36 per K step of the longest split; above, 6.4 (5.9 up
 //    to 176 tokens: 160 x 2816 15.2 / 16.05 as layers) at 144 tokens and 0.025 per token more, 0.5 per CTA of a cluster above four, 0.42
 //    per K step (us, few tokens / here: 144 tokens d = 2560 9.7 / 10.4, d = 4096 13.6 / 14.9; 208 d = 2560 12.6 / 10.4, d = 4096 15.0 /
 //    15.0 (the layer with N = 6144 22.7 / 23.2), d = 5120 19.5 / 20.1; 256 d = 4096 16.2 / 15.1, d = 5120 20.9 / 20.0; 128 d = 2048 8.1 /
@@ -536,8 +537,8 @@ torq_status torq_quantize_mxfp4(const void* Z, torq_dtype z_dtype, int64_t M, in
 //    tokens: d = 256 2.95 / 2.96, 2.95 / 3.21, 2.95 / 4.49; d = 512 3.97 / 3.08, 3.37 / 3.21, 3.46 / 3.60; d = 768 5.25 / 3.21, 4.24 /
 //    3.37, 4.36 / 3.85);
 //  * above 192 tokens a cluster of three has five units for its first CTA: 0.6 more (216 d = 4864 19.3 / 18.2);
-//  * above d = 6144, where these tiles take up to 3 us less than the figures say: 7.6 up to 192 tokens, 10.5 above, 0.42 per K step
-//    (144 d = 6912 26.9 / 25.4, 150 d = 7040 28.2 / 26.3, 208 d = 7680 33.1 / 30.0);
+//  * above d = 6144, where these tiles take up to 3 us less than the figures say: 7.0 up to 176 tokens, 7.6 up to 192, 10.5 above, 0.42
+//    per K step (144 d = 6912 26.9 / 25.4, 150 d = 7040 28.2 / 26.3, 208 d = 7680 33.1 / 30.0);
 //  * pair kernel: 6.8, plus per K step 0.32 for a wave and 0.2 + 0.14 f for the last, partly filled one (layers with N = d at 40 sizes
 //    beside the line, 1772 to 4076 tokens, pair kernel / here: 0.99 to 1.6 of the time; 2540 x 2048 36.2 / 30.9, 2028 x 2048 25.3 / 25.05).
 // The other formats follow the same figures, which were not fitted to them; wide_gemm_width says how that was checked.
@@ -550,7 +551,7 @@ static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int few_S, b
   // tokens / here: d = 1024 63 tokens 5.7 / 5.8, 64 tokens 5.7 / 4.5; d = 1152 56 5.6 / 5.7, 60 5.7 / 4.7; d = 1536 40 5.9 / 9.3, 48
   // 6.0 / 5.6).
   const bool two_slabs = d <= 6144 && (M > 96 || (M <= 64 && M * d >= 65536));
-  const bool against_parts = M > 128 && M <= kRotFewMaxTokens;
+  const bool against_parts = M > 176 && M <= kRotFewMaxTokens;
   const double column = against_parts ? 0.022 : 0.0155, column_wide = against_parts ? 0.032 : 0.025, fixed = against_parts ? 1.6 : 1.8;
   double best = 1e30;
   int width = 0;
@@ -568,8 +569,8 @@ static int wide_rotation_width(int64_t M, int64_t d, int few_steps, int few_S, b
     else if (M <= 16) other = 3.1 + 0.22 * few_steps;
     else if (M <= 64) other = 4.4 + 0.2 * few_steps;
     else if (M <= 128) other = 5.6 + 0.36 * few_steps;
-    else if (d > 6144) other = (M <= 192 ? 7.6 : 10.5) + 0.42 * few_steps;
-    else other = (M <= 176 ? 6.1 : 6.4) + 0.025 * (double)(M - 144) + 0.42 * few_steps +
+    else if (d > 6144) other = (M <= 176 ? 7.0 : (M <= 192 ? 7.6 : 10.5)) + 0.42 * few_steps;
+    else other = (M <= 176 ? 5.9 : 6.4) + 0.025 * (double)(M - 144) + 0.42 * few_steps +
                  (few_S > 4 ? 0.5 * (few_S - 4) : (few_S == 3 && M > 192 ? 0.6 : 0.0));
   } else {
     const int64_t tiles = rows * ((d + 255) / 256);

@@ -257,7 +257,7 @@ def test_gemm_takes_two_slabs_per_stage_where_they_are_the_faster(fmt, M, N, K, 
     assert torq.torq_last_device_error() == 0
 
 
-@pytest.mark.parametrize("fmt,M,d", [("mxfp4", 180, 3072), ("mxfp4", 186, 3328), ("mxint4", 205, 3584), ("mxfp4", 225, 3840), ("nvfp4", 245, 4096),
+@pytest.mark.parametrize("fmt,M,d", [("mxfp4", 131, 2304), ("mxfp4", 180, 3072), ("mxfp4", 186, 3328), ("mxint4", 205, 3584), ("mxfp4", 225, 3840), ("nvfp4", 245, 4096),
                                      ("mxfp4", 185, 4608), ("mxfp4", 200, 4992), ("mxfp4", 212, 5120), ("mxfp4", 220, 5504), ("mxfp4", 250, 5760)])
 def test_rotation_of_129_to_256_tokens_keeps_its_sums_in_parts(fmt, M, d):
     """The few-token kernel contracts K in three to five parts, each in an accumulator of its own, and is the nearer to 64 bits for it: the
